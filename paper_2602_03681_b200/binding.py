@@ -1,8 +1,9 @@
-"""Thin ctypes binding of ``libnatsl.so`` -- same names as the C ABI (``include/natsl.h``).
+"""Thin binding of ``libnatsl.so`` -- same names as the C ABI (``include/natsl.h``).
 
 Argument marshalling only: torch supplies device memory and streams, every step of the path
-runs in the library's CUDA kernels.  There is no fallback of any kind: if the library is not
-built, importing the entry points raises.
+runs in the library's CUDA kernels.  The calls made per token, layer or step are marshalled by the
+native module ``_natsl_py`` (``csrc/pybind.cpp``), set-up and status calls through ctypes.  There is no
+fallback of any kind: if the library is not built, importing the entry points raises.
 """
 from __future__ import annotations
 
@@ -59,6 +60,17 @@ class natsl_params(ctypes.Structure):
 
 
 _lib = None
+_py = None
+
+
+def _native():
+    """The native marshalling module (linked against the library); raises when it has not been built."""
+    global _py
+    if _py is None:
+        lib()
+        from . import _natsl_py
+        _py = _natsl_py
+    return _py
 
 
 def lib() -> ctypes.CDLL:
@@ -168,46 +180,44 @@ def natsl_route_compact(route, sm_idx, sm_chunk_prefix, lin_idx, n_lin, p: natsl
 
 
 def natsl_hybrid_fwd(q, k, v, g, beta, route, out, p: natsl_params, ws):
-    _check(lib().natsl_hybrid_fwd(_ptr(q), _ptr(k), _ptr(v), _ptr(g), _ptr(beta), _ptr(route),
-                                  _ptr(out), ctypes.byref(p), _ptr(ws),
-                                  ctypes.c_size_t(ws.numel()), _stream()))
+    rc = (_py or _native()).hybrid_fwd(q, k, v, g, beta, route, out, p, ws)
+    if rc:
+        _check(rc)
 
 
 def natsl_hybrid_fwd_static(q, k, v, g, beta, route, out, p: natsl_params):
     """natsl_hybrid_fwd without a caller workspace: the scratch is a fixed array inside the
     library, for hosts that cannot allocate device memory.  Raises NatslError(-9) when the
     problem needs more than STATIC_WS_BYTES of scratch."""
-    _check(lib().natsl_hybrid_fwd_static(_ptr(q), _ptr(k), _ptr(v), _ptr(g), _ptr(beta),
-                                         _ptr(route), _ptr(out), ctypes.byref(p), _stream()))
+    rc = (_py or _native()).hybrid_fwd_static(q, k, v, g, beta, route, out, p)
+    if rc:
+        _check(rc)
 
 
 def natsl_hybrid_bwd(q, k, v, g, beta, route, dout, dq, dk, dv, dg, dbeta, dw, p: natsl_params, ws):
-    _check(lib().natsl_hybrid_bwd(_ptr(q), _ptr(k), _ptr(v), _ptr(g), _ptr(beta), _ptr(route),
-                                  _ptr(dout), _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dg), _ptr(dbeta),
-                                  _ptr(dw), ctypes.byref(p), _ptr(ws),
-                                  ctypes.c_size_t(ws.numel()), _stream()))
+    rc = (_py or _native()).hybrid_bwd(q, k, v, g, beta, route, dout, dq, dk, dv, dg, dbeta, dw, p, ws)
+    if rc:
+        _check(rc)
 
 
 def natsl_decode_step(q, k, v, g, beta, route, state, k_cache, v_cache, cache_len, out,
                       p: natsl_params, ws):
-    cap = k_cache.shape[2]
-    _check(lib().natsl_decode_step(_ptr(q), _ptr(k), _ptr(v), _ptr(g), _ptr(beta), _ptr(route),
-                                   _ptr(state), _ptr(k_cache), _ptr(v_cache), _ptr(cache_len),
-                                   ctypes.c_int32(cap), _ptr(out), ctypes.byref(p), _ptr(ws),
-                                   ctypes.c_size_t(ws.numel()), _stream()))
+    rc = (_py or _native()).decode_step(q, k, v, g, beta, route, state, k_cache, v_cache, cache_len, out, p, ws)
+    if rc:
+        _check(rc)
 
 
 def natsl_decode_block_end(route_block, g_block, state, state_start, cache_len, block_len,
                            p: natsl_params, ws):
-    _check(lib().natsl_decode_block_end(_ptr(route_block), _ptr(g_block), _ptr(state),
-                                        _ptr(state_start), _ptr(cache_len), ctypes.c_int32(block_len),
-                                        ctypes.byref(p), _ptr(ws), ctypes.c_size_t(ws.numel()),
-                                        _stream()))
+    rc = (_py or _native()).decode_block_end(route_block, g_block, state, state_start, cache_len, block_len, p, ws)
+    if rc:
+        _check(rc)
 
 
 def natsl_score_layer(x, w_score, scores, route, p: natsl_params):
-    _check(lib().natsl_score_layer(_ptr(x), _ptr(w_score), _ptr(scores), _ptr(route),
-                                   ctypes.c_int32(x.shape[-1]), ctypes.byref(p), _stream()))
+    rc = (_py or _native()).score_layer(x, w_score, scores, route, p)
+    if rc:
+        _check(rc)
 
 
 def natsl_device_status(ws) -> int:

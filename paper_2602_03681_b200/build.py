@@ -1,4 +1,5 @@
-"""Compile the CUDA sources under ``csrc/`` for sm_100a into ``libnatsl.so`` (in-tree).
+"""Compile the CUDA sources under ``csrc/`` for sm_100a into ``libnatsl.so`` and the native marshalling of
+the Python binding into ``_natsl_py.so`` (both in-tree).
 
 nvcc cross-compiles without a GPU.  Objects are rebuilt only when a source or header is newer.
 """
@@ -15,6 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 OBJ_DIR = os.path.join(HERE, "_build")
 LIB_PATH = os.path.join(HERE, "libnatsl.so")
+PY_PATH = os.path.join(HERE, "_natsl_py.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
@@ -61,9 +63,33 @@ def build(force: bool = False, verbose: bool = False) -> str:
                     print(log, file=sys.stderr)
     if jobs or not os.path.exists(LIB_PATH):
         tmp = LIB_PATH + f".tmp{os.getpid()}"
-        run([nvcc, "-shared", "-o", tmp, *objs])
+        run([nvcc, "-shared", "-o", tmp, "-Xlinker", "-soname=libnatsl.so", *objs])
         os.replace(tmp, LIB_PATH)
+    build_python_module()
     return LIB_PATH
+
+
+def build_python_module() -> str:
+    """``_natsl_py.so``: linked against ``libnatsl.so`` beside it and the torch libraries of this interpreter."""
+    src = os.path.join(CSRC, "pybind.cpp")
+    newest = max(os.path.getmtime(f) for f in [src, *glob.glob(os.path.join(INCLUDE, "*.h"))])
+    if os.path.exists(PY_PATH) and os.path.getmtime(PY_PATH) >= newest:
+        return PY_PATH
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(torch.__file__)
+    tmp = PY_PATH + f".tmp{os.getpid()}"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=" + str(int(torch._C._GLIBCXX_USE_CXX11_ABI)),
+           "-isystem", os.path.join(root, "include"), "-isystem", os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           "-isystem", sysconfig.get_path("include"), "-isystem", os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include"),
+           src, "-o", tmp, "-L", HERE, "-l:libnatsl.so", "-L", os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10",
+           "-lc10_cuda", "-Wl,-rpath,$ORIGIN"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("g++ failed: " + " ".join(cmd) + "\n" + res.stdout + res.stderr)
+    os.replace(tmp, PY_PATH)
+    return PY_PATH
 
 
 if __name__ == "__main__":

@@ -1246,7 +1246,7 @@ scatter_sm_kernel(const float *__restrict__ dk_sm, const float *__restrict__ dv_
 
 template <typename Kn>
 cudaError_t set_smem(Kn kernel, size_t bytes) {
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return allow_smem(kernel, (int)bytes);
 }
 
 }  // namespace
@@ -1262,8 +1262,7 @@ cudaError_t launch_bgemm(bool ta, bool tb, int mask, BMat A, BMat B, BMat C, int
 #define NATSL_BG(TA, TB, MK)                                                                                   \
     do {                                                                                                        \
         if (s.bf16) {                                                                                           \
-            cudaError_t e = cudaFuncSetAttribute(bgemm_tf32_kernel<TA, TB, MK>,                                 \
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBgSmem);    \
+            cudaError_t e = allow_smem(bgemm_tf32_kernel<TA, TB, MK>, (int)kBgSmem);    \
             if (e != cudaSuccess) return e;                                                                     \
             bgemm_tf32_kernel<TA, TB, MK><<<grid, kThreads, kBgSmem, st>>>(A, B, C, k, alpha, accumulate ? 1 : 0, s.H, NC); \
         } else bgemm_kernel<TA, TB, MK><<<grid, kThreads, 0, st>>>(A, B, C, k, alpha, accumulate ? 1 : 0, s.H, NC); \
@@ -1508,7 +1507,7 @@ cudaError_t launch_gdn_tm(const float *Tinv, const float *dW, const float *dUt, 
                           float *Ns, Shape s, cudaStream_t st) {
     const unsigned nch = (unsigned)(s.B * s.H * (s.L / kC));
     auto kernel = s.d == 128 ? gdn_tm_kernel<128> : gdn_tm_kernel<64>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTmSmem);
+    cudaError_t e = allow_smem(kernel, (int)kTmSmem);
     if (e != cudaSuccess) return e;
     kernel<<<nch, kThreads, kTmSmem, st>>>(Tinv, dW, dUt, W, U, dO, Ut, Gcum, beta, route, scale_la, dKb, dVb, Mg,
                                           Ms, Ns, s.L, s.H);
@@ -1521,7 +1520,7 @@ static cudaError_t xassemble_impl(const AssembleArgs &a, const float *Mg, const 
                                   void *dq, void *dk, void *dv, Shape s, cudaStream_t st) {
     const int NC = s.L / kC;
     const size_t nch = (size_t)s.B * s.H * NC;
-    cudaError_t e = cudaFuncSetAttribute(gdn_xassemble_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = allow_smem(gdn_xassemble_kernel<T, D>,
                                          (int)kXaSmem);
     if (e != cudaSuccess) return e;
     gdn_xassemble_kernel<T, D><<<(unsigned)nch, kThreads, kXaSmem, st>>>(

@@ -445,7 +445,7 @@ static cudaError_t decode_impl(const void *q, const void *k, const void *v, cons
     const bool grouped = hg.G > 1 || hg.norm_eps >= 0.f;
     if (grouped && (hg.G > 4 || D % (32 * hg.G) != 0)) return cudaErrorInvalidValue;
     auto kernel = grouped ? decode_step_kernel<T, D, true> : decode_step_kernel<T, D, false>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    cudaError_t e = allow_smem(kernel, kSmem);
     if (e != cudaSuccess) return e;
     dim3 grid(kCtasPerHead, s.B * s.H);
     kernel<<<grid, kThreads, kSmem, st>>>(

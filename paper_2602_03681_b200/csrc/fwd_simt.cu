@@ -539,7 +539,7 @@ qk_norm_bwd_f32_kernel(const T *__restrict__ q, const T *__restrict__ k,
 
 template <typename K>
 cudaError_t set_smem(K kernel, size_t bytes) {
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return allow_smem(kernel, (int)bytes);
 }
 
 }  // namespace

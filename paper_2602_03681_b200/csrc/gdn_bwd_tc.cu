@@ -858,7 +858,7 @@ static cudaError_t rscan_tc_impl(const void *dO16, const void *dOg16, const GdnT
         !tch::make_map_2d(&mwt, ws.Wt, BH * NC * D, 64, D) || !tch::make_map_2d(&mph, ws.Ph, BH * NC * 64, 64, 64))
         return cudaErrorInvalidValue;
     auto kernel = block_route ? gdn_rscan_tc_kernel<D, true> : gdn_rscan_tc_kernel<D, false>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = allow_smem(kernel,
                                          RsLayout<D>::kTotal);
     if (e != cudaSuccess) return e;
     kernel<<<s.B * s.H, kRsThreads, RsLayout<D>::kTotal, st>>>(
@@ -892,7 +892,7 @@ cudaError_t launch_gdn_bwd_chunk(const void *q, const void *k, const void *v, co
                                  float *kap_c, Shape s, cudaStream_t st) {
     if (s.d != 64 || !s.bf16) return cudaErrorInvalidValue;
     auto kernel = block ? gdn_bwd_chunk_kernel<true> : gdn_bwd_chunk_kernel<false>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = allow_smem(kernel,
                                          kCkSmem);
     if (e != cudaSuccess) return e;
     ChunkBwdArgs a{(const __nv_bfloat16 *)q, (const __nv_bfloat16 *)k, (const __nv_bfloat16 *)v, dO, dUt, Ut,
@@ -961,7 +961,7 @@ cudaError_t launch_softmax_bwd_own_block(const void *q, const void *k, const voi
         kernel = qn ? softmax_bwd_own_block_kernel<1, true, 2> : softmax_bwd_own_block_kernel<1, false, 2>;
         smem = own_smem<2>();
     }
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(kernel, smem);
     if (e != cudaSuccess) return e;
     dim3 grid(s.L / kC, s.B * s.H * (G == 2 ? 2 : 1));
     kernel<<<grid, kCkThreads, smem, st>>>(

@@ -1009,8 +1009,7 @@ static cudaError_t prepare_tc_impl(const void *q, const void *k, const void *v, 
         !tch::make_map_2d(&mqh, ws.Qh, BH * s.L, D, 64) ||
         !tch::make_map_2d(&mkh, ws.Kh, BH * s.L, D, 64))
         return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(gdn_prepare_tc_kernel<D>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = allow_smem(gdn_prepare_tc_kernel<D>,
                                          PrepLayout<D>::kTotal);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)NC * (unsigned)BH);
@@ -1035,7 +1034,7 @@ static cudaError_t scan_tc_impl(const GdnTcWs &ws, float scale_la, const float *
         !tch::make_map_2d(&mph, ws.Ph, BH * NC * 64, 64, 64))
         return cudaErrorInvalidValue;
     auto kernel = block_route ? gdn_scan_tc_kernel<D, true> : gdn_scan_tc_kernel<D, false>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = allow_smem(kernel,
                                          ScanLayout<D>::kTotal);
     if (e != cudaSuccess) return e;
     const int ctas = s.B * s.H * (sg.mode == 0 ? 1 : sg.nseg) * (sg.mode == 1 ? 2 : 1);

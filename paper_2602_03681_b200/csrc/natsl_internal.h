@@ -101,6 +101,12 @@ cudaError_t launch_softmax_combine_tc(const void *q, const void *k_sm, const voi
                                       HeadGroups hg = HeadGroups{});
 // (o_la16: the linear branch's read-out, o_laT [B,H,L/C,8,d,8] fp16; emit_flags: see ScanOut -- when given, the
 // kernel is launched as a programmatic dependent of the kernel before it in the stream, the scan)
+// cudaFuncSetAttribute(max dynamic shared memory) of a kernel, once per thread, device and size: the call
+// itself costs a launch's host time about half a microsecond, and a forward would make five of them.
+cudaError_t allow_smem_of(const void *kernel, int bytes);
+template <typename K> cudaError_t allow_smem(K *kernel, size_t bytes) {
+    return allow_smem_of(reinterpret_cast<const void *>(kernel), (int)bytes);
+}
 int sm_count();   // multiprocessors of the current device (cached per device)
 // Bound of the device-side waits in units of 1024 cycles, 0 = the default (about two seconds);
 // non-zero only after natsl_debug_set_wait_limit.  Every tensor-core kernel launch passes it on.

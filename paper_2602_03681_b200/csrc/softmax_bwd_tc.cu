@@ -548,11 +548,10 @@ static cudaError_t softmax_bwd_tc_impl(const void *q, void *Qh, const void *dO16
         !tch::make_map_2d(&mq64, Qh, BH * s.L, DL, 64) || !tch::make_map_2d(&mdo64, dO16, BH * s.L, DL, 64) ||
         !tch::make_map_2d(&mk128, k16, BH * cap, DL, 128) || !tch::make_map_2d(&mv128, v16, BH * cap, DL, 128))
         return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(softmax_bwd_dq_tc_kernel<D, G>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, QLayout<D>::kTotal);
+    cudaError_t e = allow_smem(softmax_bwd_dq_tc_kernel<D, G>, QLayout<D>::kTotal);
     if (e != cudaSuccess) return e;
     auto dkv = dmask ? softmax_bwd_dkv_tc_kernel<D, true, G> : softmax_bwd_dkv_tc_kernel<D, false, G>;
-    e = cudaFuncSetAttribute(dkv, cudaFuncAttributeMaxDynamicSharedMemorySize, KLayout<D>::kTotal);
+    e = allow_smem(dkv, KLayout<D>::kTotal);
     if (e != cudaSuccess) return e;
     dim3 gq((s.L + 127) / 128, s.B * s.H * G);
     softmax_bwd_dq_tc_kernel<D, G><<<gq, kThreadsB, QLayout<D>::kTotal, st>>>(

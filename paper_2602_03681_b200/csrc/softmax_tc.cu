@@ -702,7 +702,7 @@ static cudaError_t softmax_tc_impl(const void *q, const void *k_sm, const void *
     if (norm_eps >= 0.f) kernel = softmax_combine_tc_kernel<D, false, G, true>;
     if (br.route) kernel = norm_eps >= 0.f ? softmax_combine_tc_kernel<D, true, G, true>
                                           : softmax_combine_tc_kernel<D, true, G, false>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SL::kTotal);
+    cudaError_t e = allow_smem(kernel, SL::kTotal);
     if (e != cudaSuccess) return e;
     // With emit_flags the kernel is launched as a programmatic dependent of the kernel before it in
     // the stream (the scan): it may start once all of the scan's CTAs are resident, and finds o_la

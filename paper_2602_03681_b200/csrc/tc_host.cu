@@ -72,6 +72,29 @@ bool make_map_blhd_f32(CUtensorMap *m, const void *base, int B, int L, int H, in
 
 }  // namespace tch
 
+cudaError_t allow_smem_of(const void *kernel, int bytes) {
+    struct Entry { const void *fn; int dev, bytes; };
+    constexpr int kEntries = 128;                     // (the library has fewer kernels; a full table only re-sends)
+    thread_local Entry table[kEntries] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    size_t at = (reinterpret_cast<uintptr_t>(kernel) >> 4) * 31 + (size_t)dev;
+    Entry *slot = nullptr;
+    for (int i = 0; i < 8 && !slot; ++i) {
+        Entry &x = table[(at + i) % kEntries];
+        if (x.fn == kernel && x.dev == dev) {
+            if (x.bytes >= bytes) return cudaSuccess;
+            slot = &x;
+        } else if (!x.fn) {
+            slot = &x;
+        }
+    }
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess && slot) *slot = Entry{kernel, dev, bytes};
+    return e;
+}
+
 int sm_count() {
     static int cached[64] = {};
     int dev = 0;

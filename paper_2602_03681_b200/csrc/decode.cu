@@ -4,23 +4,31 @@
 // RMS-normalised outputs (Section 4.3, Norm equation).  decode_block_end_kernel rolls back the
 // operation that was not chosen once a block is complete.
 //
-// HBM-bound: per (sequence, head) the state is read and written once (2 d^2 4 bytes) and the
-// retained K/V are read once.  To keep enough bytes in flight and the SMs evenly loaded, each
-// (sequence, head) is split over kDecodeParts + kStateParts CTAs: a "cache" CTA streams one slice
-// of the retained K/V through a four-stage ring of bulk asynchronous copies (16 KB per stage in
-// flight whatever the arithmetic is doing) and leaves a partial online-softmax result in the
-// workspace; a "state" CTA streams half of the state's value columns through registers (the
-// columns of the delta rule are independent) and leaves its part of the linear read-out there.
-// Whichever CTA of the head finishes last (an atomic ticket, nobody waits) merges the partials,
-// adds the new token's own term, normalises, combines, writes `out`, appends the token to the
-// cache and bumps its length.
-// Grouped softmax heads and per-operation q/k normalisation (Section 4.3; template flag, so that the
-// plain instantiation is unchanged code): the G softmax heads of a linear head are the G slices of d / G
-// columns -- the lanes that share a key row split into G groups, each with its own logit, running
-// maximum and sum --, the state CTAs work on the L2-normalised q and k, and the cache keeps the keys as
-// given: a cached key is RMS-normalised per slice as it is read (its sum of squares rides along with the
-// logit's reduction), because normalised keys rounded to the cache's bf16 would cost 2.8e-2 of the
-// branch output's RMS.
+// HBM-bound for many (sequence, head) pairs, a chain of latencies for few: per pair the state is read
+// and written once (2 d^2 4 bytes) and the retained K/V are read once.  The work of a pair is split into
+// items: `parts` cache items, each a slice of the retained K/V, and kStateParts state items, each a group
+// of the state's value columns (the columns of the delta rule are independent).  Whichever item of the
+// pair finishes last (an atomic ticket, nobody waits) merges the partial results, adds the new token's own
+// term, normalises, combines, writes `out`, appends the token to the cache and bumps its length.
+//   * Few pairs: every item has a CTA of its own and the cache is cut as finely as the machine has room
+//     for (up to 16 slices), because a slice is walked serially.
+//   * Many pairs: persistent CTAs, two per SM.  The copy warp runs ahead into the next item's slice (96 KB in
+//     flight per CTA), the work warps leave their part of an item in shared memory and go on, and a finisher
+//     warp merges it, takes the ticket and finishes the step behind them, so that neither the ticket's
+//     round trip nor the final merge ever stands between two items.
+// The kernel is a programmatic dependent of the work before it in the stream: barriers and the ring are
+// set up while that finishes, nothing global is touched before it has.
+// Work per cached key: eight lanes share a row (four rows per warp and pass), each with whole 16-byte
+// pieces 128 bytes apart (conflict-free); products as packed fp32 pairs; the running maximum moves only when
+// a logit exceeds it by 2^8, so the accumulator is rescaled once or twice per slice instead of per key.
+// (With sixteen lanes per row and a rescale per key the kernel issued 2.5 x the instructions and sat at 83 %
+// of the copy rate, 74 % with grouped heads.)
+// Grouped softmax heads and per-operation q/k normalisation (Section 4.3; template parameters): the G softmax
+// heads of a linear head are the G slices of d / G columns, each with its own logit, running maximum and
+// sum; the state items work on the L2-normalised q and k, and the cache keeps the keys as given: a cached
+// key is RMS-normalised per slice as it is read (its sum of squares rides along with the logit's
+// reduction), because normalised keys rounded to the cache's bf16 would cost 2.8e-2 of the branch output's
+// RMS.
 #include "common.cuh"
 #include "natsl_internal.h"
 #include "tc_common.cuh"
@@ -33,11 +41,29 @@ using namespace tc;
 
 constexpr int kWorkThreads = 256;
 constexpr int kWarps = kWorkThreads / 32;
-constexpr int kThreads = kWorkThreads + 32;      // + one warp that issues the bulk copies
-constexpr int kTileKeys = 32;
-constexpr int kStages = 4;
+constexpr int kThreads = kWorkThreads + 64;      // + one warp that issues the bulk copies, + the finisher
+constexpr int kTileKeys = 32;                    // one key per group of eight lanes and pass
+constexpr int kRingBytes = 96 * 1024;
 constexpr int kStateParts = 2;
-constexpr int kCtasPerHead = kDecodeParts + kStateParts;
+constexpr int kMaxParts = 16;
+constexpr int kCtasPerSm = 2, kResident = kCtasPerSm * 148;
+
+// Cache items per (sequence, head).  Few pairs: as many as keep every item resident at once.  More: the count
+// (of those that cut a cache finely enough) whose items fill the last round of persistent CTAs best.
+__host__ __device__ inline int decode_parts(size_t BH) {
+    if (BH * (1 + kStateParts) <= kResident) {
+        const int p = (int)(kResident / BH) - kStateParts;
+        return p > kMaxParts ? kMaxParts : p;
+    }
+    int best = 4;
+    float least = 1e30f;
+    for (int p = 4; p <= kMaxParts; ++p) {
+        const float n = (float)BH * (p + kStateParts), per = n / kResident;
+        const float cost = (float)(int)(per + 0.999f) / per + 0.01f * p;
+        if (cost < least) { least = cost; best = p; }
+    }
+    return best;
+}
 
 template <typename T> struct Vec16;   // 16 bytes of T as fp32 values
 template <> struct Vec16<float> {
@@ -59,332 +85,518 @@ template <> struct Vec16<__nv_bfloat16> {
     }
 };
 
-// Workspace: [0,256) status word; then tickets [BH] i32; partials [BH][kDecodeParts][D+8] f32
-// (m[G], z[G] in the first 8 with G <= 4, then acc[D]); o_la [BH][D] f32.
+// Packed fp32 pairs: one instruction per two multiply-adds.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// Workspace: [0,256) status word; then tickets [BH] i32; partials [BH][parts][D+8] f32 (m[G] in base-2 units
+// and z[G] in the first 8 with G <= 4, then acc[D]); o_la [BH][D] f32.
 constexpr int kPartHead = 8;
 __host__ __device__ inline size_t dec_off_tickets() { return 256; }
 __host__ __device__ inline size_t dec_off_partials(size_t BH) {
     return (256 + BH * 4 + 255) / 256 * 256;
 }
 __host__ __device__ inline size_t dec_off_ola(size_t BH, int D) {
-    return dec_off_partials(BH) + (BH * kDecodeParts * (D + kPartHead) * 4 + 255) / 256 * 256;
+    return dec_off_partials(BH) + (BH * decode_parts(BH) * (D + kPartHead) * 4 + 255) / 256 * 256;
 }
 
-template <typename T, int D, bool kGrouped>
-__global__ void __launch_bounds__(kThreads, 3)
+template <typename T, int D, int G> struct DecLayout {
+    static constexpr int kRowBytes = D * (int)sizeof(T);
+    static constexpr int kTileBytes = kTileKeys * kRowBytes;
+    static constexpr int kStages = kRingBytes / (2 * kTileBytes);      // K and V tile per stage
+    static constexpr int kSlotFloats = 8 * 128;                        // [8 warps][D] or [slots][D / 2]
+    static constexpr int oScratch = kRingBytes;                        // two slots, then the state items' own
+    static constexpr int oMz = oScratch + 3 * kSlotFloats * 4;         // [2][8 warps][G] (m, z)
+    static constexpr int kTotal = oMz + 2 * kWarps * G * 8;
+};
+
+template <typename T, int D, int G, bool kNorm>
+__global__ void __launch_bounds__(kThreads, kCtasPerSm)
 decode_step_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v,
                    const float *__restrict__ g, const float *__restrict__ beta,
                    const uint8_t *__restrict__ route, const float *__restrict__ w,
                    float *__restrict__ state, T *__restrict__ k_cache, T *__restrict__ v_cache,
                    int32_t *__restrict__ cache_len, int cap, T *__restrict__ out, float scale_la,
-                   float scale_sm, float eps, uint8_t *__restrict__ ws, int BH, int Gin, float norm_eps) {
-    const int G = kGrouped ? Gin : 1;              // softmax heads per linear head
-    const int ds = D / G;                          // columns per softmax head
-    const bool normed = kGrouped && norm_eps >= 0.f;
+                   float scale_sm, float eps, uint8_t *__restrict__ ws, int BH, int parts, float norm_eps) {
+    using SL = DecLayout<T, D, G>;
+    constexpr int kStages = SL::kStages, kRowBytes = SL::kRowBytes, kTileBytes = SL::kTileBytes;
+    constexpr int ds = D / G;                      // columns per softmax head
     constexpr int kE = Vec16<T>::kN;               // elements per 16-byte piece
-    constexpr int kRowBytes = D * (int)sizeof(T);
-    constexpr int kLpk = kRowBytes / 16;           // lanes per key row
-    constexpr int kStreams = kWorkThreads / kLpk;  // independent online-softmax streams
-    constexpr int kTileBytes = kTileKeys * kRowBytes;
-    static_assert(kStreams <= kTileKeys && kTileKeys % kStreams == 0, "tile / stream mismatch");
+    constexpr int kJ = kRowBytes / 128;            // pieces per lane of a row's eight lanes
+    constexpr int kSp = ds * (int)sizeof(T) / 16;  // pieces per softmax head
+    static_assert(kSp % 4 == 0 && (kSp == 4 || kSp % 8 == 0), "softmax heads of at least 64 bytes");
+    constexpr int kLg = kSp >= 8 ? G : kJ;         // logits a lane takes part in
+    constexpr int kJpl = kJ / kLg;                 // pieces per logit and lane
+    constexpr int kLanes = kSp >= 8 ? 8 : 4;       // lanes that share a logit
+    constexpr float kLog2e = 1.4426950408889634f;
+    constexpr int kCols = D / kStateParts;         // state item: value columns
+    constexpr int kLpr = kCols / 4;                // lanes per (half) state row
+    constexpr int kRpl = 32 / kLpr;                // rows per warp-wide access
+    constexpr int kSlots = kWarps * kRpl;          // row slots in the CTA
+    constexpr int kR = D / kSlots;                 // rows per thread
+    static_assert(kSlots * kCols <= SL::kSlotFloats, "scratch too small");
 
     extern __shared__ __align__(128) uint8_t smem[];
-    __shared__ uint64_t full[kStages], empty[kStages];
-    __shared__ __align__(16) float qs[D], ks[D], vs[D];     // (normalised: the linear operation's q, k)
-    __shared__ __align__(16) float qsm[kGrouped ? D : 4], ksm[kGrouped ? D : 4];   // the softmax operation's q, k
-    __shared__ float sm_m[kTileKeys * (kGrouped ? 4 : 1)], sm_z[kTileKeys * (kGrouped ? 4 : 1)];
-    __shared__ float norm_red[2][kWarps];
-    __shared__ int s_last, s_abort[2];   // s_abort[1]: wait limit (see mbar_wait)
+    __shared__ uint64_t full[kStages], empty[kStages], done[2], taken[2];
+    __shared__ int s_abort[2];   // s_abort[1]: wait limit (see mbar_wait)
+    auto slot_of = [&](int i) { return reinterpret_cast<float *>(smem + SL::oScratch) + i * SL::kSlotFloats; };
+    float2 *mz = reinterpret_cast<float2 *>(smem + SL::oMz);
 
-    const int part = blockIdx.x, bh = blockIdx.y;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int per_head = parts + kStateParts, total = BH * per_head;
     int32_t *status = reinterpret_cast<int32_t *>(ws);
-    int32_t *ticket = reinterpret_cast<int32_t *>(ws + dec_off_tickets()) + bh;
-    float *partials =
-        reinterpret_cast<float *>(ws + dec_off_partials(BH)) + (size_t)bh * kDecodeParts * (D + kPartHead);
-    float *ola_ws = reinterpret_cast<float *>(ws + dec_off_ola(BH, D)) + (size_t)bh * D;
-
-    // route 0: linear token (delta rule); 1: softmax token (appended to the cache); 2: token of a
-    // block whose decision is still open -- both (Section 4.1, pseudo-update of both hidden states)
-    const int rv = route[bh];
-    const bool r = rv != 0;                        // append, and attend to itself
-    const bool fold = rv != 1;                     // delta rule
-    // A stored length outside [0, cap] (a prefill whose cache overflowed, a caller's mistake) is
-    // clamped, so that no copy below can leave the head's rows, and reported.
-    const int n_raw = cache_len[bh];
-    const int n_old = min(max(n_raw, 0), cap);
-    if (n_raw != n_old && tid == 0 && part == 0) atomicMin(status, (int)NATSL_ERR_CACHE_FULL);
-    const bool cache_full = r && n_old >= cap;     // no room: the sequence is left untouched
-    if (tid < D) {
-        qs[tid] = to_f32(q[(size_t)bh * D + tid]);
-        ks[tid] = to_f32(k[(size_t)bh * D + tid]);
-        vs[tid] = to_f32(v[(size_t)bh * D + tid]);
-    }
     if (tid == 0) {
-        for (int s = 0; s < kStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], kWorkThreads); }
+        for (int s = 0; s < kStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], kWarps); }
+        for (int s = 0; s < 2; ++s) { mbar_init(&done[s], kWarps); mbar_init(&taken[s], 1); }
         s_abort[0] = 0;
         s_abort[1] = 0;
         fence_mbar_init();
     }
     __syncthreads();
     volatile int *abort_flag = s_abort;
-    if (kGrouped && warp < kWarps) {     // (the work threads only: the copy warp goes straight to its ring)
-        // q, k of the two operations: L2 over the row for the linear one (in place in qs, ks), RMS per slice
-        // for the softmax one (qsm, ksm); without the normalisation both are the token's q, k.
-        float sq = 0.f, sk = 0.f;
-        if (tid < D) { sq = qs[tid] * qs[tid]; sk = ks[tid] * ks[tid]; }
-        sq = warp_sum(sq);
-        sk = warp_sum(sk);
-        if (lane == 0 && warp < D / 32) { norm_red[0][warp] = sq; norm_red[1][warp] = sk; }
-        named_barrier_sync(1, kWorkThreads);
-        if (tid < D) {
-            float aq = 0.f, ak = 0.f, gq = 0.f, gk = 0.f;
-            for (int wv = 0; wv < D / 32; ++wv) {
-                aq += norm_red[0][wv];
-                ak += norm_red[1][wv];
-                if ((32 * wv) / ds == tid / ds) { gq += norm_red[0][wv]; gk += norm_red[1][wv]; }
+    grid_dependency_wait();
+    launch_dependents();
+
+    // Tiles of a cache item.  A stored length outside [0, cap] (a prefill whose cache overflowed, a caller's
+    // mistake) is clamped, so that no copy can leave the pair's rows; the finisher reports it.
+    auto tiles_of = [&](int part, int n_old, bool cache_full, int &t_begin, int &t_end) {
+        const int tiles = cache_full ? 0 : (n_old + kTileKeys - 1) / kTileKeys;
+        const int tpp = (tiles + parts - 1) / parts;
+        t_begin = min(part * tpp, tiles);
+        t_end = min(t_begin + tpp, tiles);
+    };
+
+    if (warp == kWarps) {
+        // ---------------- copy warp: the cache slices of all items of this CTA, back to back ----------------
+        if (lane != 0) return;
+        int it = 0;                                      // tiles issued so far
+        bool ok = true;
+        int item = blockIdx.x, n_next = 0, rv_next = 0;
+        auto fetch = [&]() {
+            while (item < total && item % per_head >= parts) item += gridDim.x;
+            if (item < total) { n_next = cache_len[item / per_head]; rv_next = route[item / per_head]; }
+        };
+        fetch();
+        while (item < total && ok) {
+            const int part = item % per_head, bh = item / per_head;
+            const int n_old = min(max(n_next, 0), cap);
+            int t, t_end;
+            tiles_of(part, n_old, rv_next != 0 && n_old >= cap, t, t_end);
+            item += gridDim.x;
+            fetch();                                     // (the next item's length is on its way meanwhile)
+            const uint8_t *kc = reinterpret_cast<const uint8_t *>(k_cache + (size_t)bh * cap * D);
+            const uint8_t *vc = reinterpret_cast<const uint8_t *>(v_cache + (size_t)bh * cap * D);
+            for (; t < t_end; ++t, ++it) {
+                const int s = it % kStages;
+                ok = mbar_wait(&empty[s], ((it / kStages) & 1) ^ 1, abort_flag);
+                if (!ok) break;
+                const int rows = min(kTileKeys, n_old - t * kTileKeys);
+                const uint32_t bytes = (uint32_t)rows * kRowBytes;
+                mbar_arrive_expect_tx(&full[s], 2 * bytes);
+                bulk_load_1d(smem + (2 * s) * kTileBytes, kc + (size_t)t * kTileBytes, bytes, &full[s]);
+                bulk_load_1d(smem + (2 * s + 1) * kTileBytes, vc + (size_t)t * kTileBytes, bytes, &full[s]);
             }
-            const float qv = qs[tid], kv = ks[tid];
-            qsm[tid] = normed ? qv * rsqrtf(gq / ds + norm_eps) : qv;
-            ksm[tid] = normed ? kv * rsqrtf(gk / ds + norm_eps) : kv;
-            if (normed) { qs[tid] = qv * rsqrtf(aq + norm_eps); ks[tid] = kv * rsqrtf(ak + norm_eps); }
         }
-        named_barrier_sync(1, kWorkThreads);
+        for (int u = max(0, it - kStages); u < it; ++u)  // no copy in flight when the CTA retires, aborted or not
+            mbar_wait_drain(&full[u % kStages], (u / kStages) & 1);
+        return;
     }
 
-    if (part < kDecodeParts) {
-        // ---------------- cache CTA: one slice of the retained K/V ----------------
-        const int tiles_total = cache_full ? 0 : (n_old + kTileKeys - 1) / kTileKeys;
-        const int tpp = (tiles_total + kDecodeParts - 1) / kDecodeParts;
-        const int t_begin = min(part * tpp, tiles_total), t_end = min(t_begin + tpp, tiles_total);
-        const uint8_t *kc = reinterpret_cast<const uint8_t *>(k_cache + (size_t)bh * cap * D);
-        const uint8_t *vc = reinterpret_cast<const uint8_t *>(v_cache + (size_t)bh * cap * D);
-        if (warp == kWarps) {
-            if (lane == 0) {
-                int t = t_begin;
-                for (; t < t_end; ++t) {
-                    const int i = t - t_begin, s = i % kStages;
-                    if (!mbar_wait(&empty[s], ((i / kStages) & 1) ^ 1, abort_flag)) break;
-                    const int rows = min(kTileKeys, n_old - t * kTileKeys);
-                    const uint32_t bytes = (uint32_t)rows * kRowBytes;
-                    mbar_arrive_expect_tx(&full[s], 2 * bytes);
-                    bulk_load_1d(smem + (2 * s) * kTileBytes, kc + (size_t)t * kTileBytes, bytes, &full[s]);
-                    bulk_load_1d(smem + (2 * s + 1) * kTileBytes, vc + (size_t)t * kTileBytes, bytes,
-                                 &full[s]);
+    if (warp == kWarps + 1) {
+        // ---------------- finisher warp: merges what the work warps leave per item; the last item of a
+        // (sequence, head) anywhere finishes the step.  Lane l owns columns V l .. V l + V - 1. ----------------
+        constexpr int V = D / 32, kLs = 32 / G;          // columns per lane, lanes per softmax head
+        constexpr int kPs = D + kPartHead;
+        auto slice_sum = [&](float x) {
+#pragma unroll
+            for (int o = kLs / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            return x;
+        };
+        const int sg = lane / kLs;
+        for (int item = blockIdx.x, i = 0; item < total; item += gridDim.x, ++i) {
+            const int part = item % per_head, bh = item / per_head;
+            int32_t *ticket = reinterpret_cast<int32_t *>(ws + dec_off_tickets()) + bh;
+            float *partials = reinterpret_cast<float *>(ws + dec_off_partials(BH)) + (size_t)bh * parts * kPs;
+            float *ola_ws = reinterpret_cast<float *>(ws + dec_off_ola(BH, D)) + (size_t)bh * D;
+            const float *sc = slot_of(i & 1);
+            // (after a time-out, which is reported, the tickets are still taken, so that they end at zero)
+            const bool ok = mbar_wait(&done[i & 1], (i >> 1) & 1, abort_flag);
+            if (!ok) {
+            } else if (part < parts) {                   // eight warps' (m, z, acc) -> one partial
+                float M = -INFINITY, Z = 0.f, o[V];
+#pragma unroll
+                for (int x = 0; x < V; ++x) o[x] = 0.f;
+                const float2 *mzs = mz + (i & 1) * kWarps * G;
+#pragma unroll
+                for (int wv = 0; wv < kWarps; ++wv) M = fmaxf(M, mzs[wv * G + sg].x);
+                const float Mu = M == -INFINITY ? 0.f : M;
+#pragma unroll
+                for (int wv = 0; wv < kWarps; ++wv) {
+                    const float2 e = mzs[wv * G + sg];
+                    const float f = ex2_ftz(e.x - Mu);
+                    Z = fmaf(e.y, f, Z);
+#pragma unroll
+                    for (int x = 0; x < V; ++x) o[x] = fmaf(sc[wv * D + lane * V + x], f, o[x]);
                 }
-                if (*abort_flag)           // let the copies already issued land before the CTA retires
-                    for (int u = max(t_begin, t - kStages); u < t; ++u)
-                        mbar_wait_drain(&full[(u - t_begin) % kStages], ((u - t_begin) / kStages) & 1);
+                float *pp = partials + (size_t)part * kPs;
+#pragma unroll
+                for (int x = 0; x < V; ++x) pp[kPartHead + lane * V + x] = o[x];
+                if (lane % kLs == 0) { pp[sg] = M; pp[4 + sg] = Z; }
+            } else {                                     // the row slots' shares of this half of the read-out
+                constexpr int kVc = (kCols + 31) / 32;
+                float a[kVc];
+#pragma unroll
+                for (int x = 0; x < kVc; ++x) a[x] = 0.f;
+#pragma unroll 8
+                for (int sl = 0; sl < kSlots; ++sl)
+#pragma unroll
+                    for (int x = 0; x < kVc; ++x) a[x] += sc[sl * kCols + lane * kVc + x];
+#pragma unroll
+                for (int x = 0; x < kVc; ++x) ola_ws[(part - parts) * kCols + lane * kVc + x] = scale_la * a[x];
+            }
+            // ticket (release by lane 0 behind the warp's barrier, acquire by it before the warp's barrier)
+            __syncwarp();
+            int last = 0;
+            if (lane == 0) {
+                mbar_arrive(&taken[i & 1]);
+                last = atom_add_acq_rel(ticket, 1) == per_head - 1;
+                if (last) *ticket = 0;                   // ready for the next step
+            }
+            last = __shfl_sync(0xffffffffu, last, 0);
+            if (!last) continue;
+            // All of the pair's partial results and the token's rows in one round trip.
+            float pa[kMaxParts][V], ol[V], qv[V], kv[V], vv[V], pm[G], pz[G];
+#pragma unroll
+            for (int pt = 0; pt < kMaxParts; ++pt)
+#pragma unroll
+                for (int x = 0; x < V; ++x)
+                    pa[pt][x] = pt < parts ? __ldcg(partials + pt * kPs + kPartHead + lane * V + x) : 0.f;
+#pragma unroll
+            for (int a = 0; a < G; ++a) {
+                pm[a] = lane < parts ? __ldcg(partials + lane * kPs + a) : -INFINITY;
+                pz[a] = lane < parts ? __ldcg(partials + lane * kPs + 4 + a) : 0.f;
+            }
+            const int rv = route[bh], n_raw = cache_len[bh];
+#pragma unroll
+            for (int x = 0; x < V; ++x) {
+                ol[x] = __ldcg(ola_ws + lane * V + x);
+                qv[x] = to_f32(q[(size_t)bh * D + lane * V + x]);
+                kv[x] = to_f32(k[(size_t)bh * D + lane * V + x]);
+                vv[x] = to_f32(v[(size_t)bh * D + lane * V + x]);
+            }
+            const float wn = w ? w[(size_t)bh * 2] : 0.5f, wl = w ? w[(size_t)bh * 2 + 1] : 0.5f;
+            const bool r = rv != 0;                      // append, and attend to itself
+            const int n_old = min(max(n_raw, 0), cap);
+            if (n_raw != n_old && lane == 0) atomicMin(status, (int)NATSL_ERR_CACHE_FULL);
+            if (r && n_old >= cap) {                     // no room: the sequence is left untouched
+#pragma unroll
+                for (int x = 0; x < V; ++x) out[(size_t)bh * D + lane * V + x] = from_f32<T>(0.f);
+                if (lane == 0) atomicMin(status, (int)NATSL_ERR_CACHE_FULL);
+                continue;
+            }
+            float qq = 0.f, kk = 0.f, self = 0.f;
+#pragma unroll
+            for (int x = 0; x < V; ++x) {
+                qq = fmaf(qv[x], qv[x], qq);
+                kk = fmaf(kv[x], kv[x], kk);
+                self = fmaf(qv[x], kv[x], self);
+            }
+            self = slice_sum(self) * scale_sm * kLog2e;
+            if (kNorm) self *= rsqrtf(slice_sum(qq) / ds + norm_eps) * rsqrtf(slice_sum(kk) / ds + norm_eps);
+            if (!r) self = -INFINITY;                    // (the token attends to itself when it is retained)
+            float M = self, Z = 0.f, pf[G], on[V];
+#pragma unroll
+            for (int a = 0; a < G; ++a) {
+                const float Ma = warp_max(pm[a]);
+                if (a == sg) M = fmaxf(M, Ma);
+            }
+            const float Mu = M == -INFINITY ? 0.f : M;
+#pragma unroll
+            for (int a = 0; a < G; ++a) {
+                pf[a] = ex2_ftz(pm[a] - __shfl_sync(0xffffffffu, Mu, a * kLs));
+                const float Za = warp_sum(pz[a] * pf[a]);
+                if (a == sg) Z = Za;
+            }
+            const float fs = ex2_ftz(self - Mu);
+            Z += fs;
+#pragma unroll
+            for (int x = 0; x < V; ++x) on[x] = vv[x] * fs;
+#pragma unroll
+            for (int pt = 0; pt < kMaxParts; ++pt) {
+                if (pt >= parts) break;
+                float f = __shfl_sync(0xffffffffu, pf[0], pt);
+#pragma unroll
+                for (int a = 1; a < G; ++a) {
+                    const float fa = __shfl_sync(0xffffffffu, pf[a], pt);
+                    if (a == sg) f = fa;
+                }
+#pragma unroll
+                for (int x = 0; x < V; ++x) on[x] = fmaf(pa[pt][x], f, on[x]);
+            }
+            const float iz = Z > 0.f ? 1.f / Z : 0.f;    // (no visible key: o_nla = 0)
+            float tn = 0.f, tl = 0.f;
+#pragma unroll
+            for (int x = 0; x < V; ++x) {
+                on[x] *= iz;
+                tn = fmaf(on[x], on[x], tn);
+                tl = fmaf(ol[x], ol[x], tl);
+            }
+            const float fn = wn * rsqrtf(slice_sum(tn) / ds + eps), fl = wl * rsqrtf(warp_sum(tl) / D + eps);
+#pragma unroll
+            for (int x = 0; x < V; ++x) {
+                out[(size_t)bh * D + lane * V + x] = from_f32<T>(fn * on[x] + fl * ol[x]);
+                if (r) {   // retain the token: every reader of the old length has finished
+                    k_cache[((size_t)bh * cap + n_old) * D + lane * V + x] = from_f32<T>(kv[x]);
+                    v_cache[((size_t)bh * cap + n_old) * D + lane * V + x] = from_f32<T>(vv[x]);
+                }
+            }
+            if (r && lane == 0) cache_len[bh] = n_old + 1;
+        }
+        if (lane == 0 && s_abort[0]) atomicMin(status, (int)NATSL_ERR_TIMEOUT);
+        return;
+    }
+
+    int it = 0;                                          // tiles consumed so far
+    for (int item = blockIdx.x, i = 0; item < total; item += gridDim.x, ++i) {
+        const int part = item % per_head, bh = item / per_head;
+        // route 0: linear token (delta rule); 1: softmax token (appended to the cache); 2: token of a
+        // block whose decision is still open -- both (Section 4.1, pseudo-update of both hidden states)
+        const int rv = route[bh], n_raw = cache_len[bh];
+        float *slot_out = slot_of(i & 1);
+        if (part < parts) {
+            // ---------------- cache item: one slice of the retained K/V ----------------
+            const int row = warp * 4 + (lane >> 3), l8 = lane & 7;
+            uint64_t qf[kJ][kE / 2], acc[kJ][kE / 2];
+            float m[kLg], z[kLg];
+            {
+                float qx[kJ][kE];
+#pragma unroll
+                for (int j = 0; j < kJ; ++j)
+                    Vec16<T>::unpack(__ldg(reinterpret_cast<const uint4 *>(q + (size_t)bh * D) + j * 8 + l8), qx[j]);
+#pragma unroll
+                for (int a = 0; a < kLg; ++a) {
+                    float f = scale_sm * kLog2e;
+                    if (kNorm) {                         // RMS over the softmax head's columns
+                        float ss = 0.f;
+#pragma unroll
+                        for (int jj = 0; jj < kJpl; ++jj)
+#pragma unroll
+                            for (int x = 0; x < kE; ++x) ss = fmaf(qx[a * kJpl + jj][x], qx[a * kJpl + jj][x], ss);
+#pragma unroll
+                        for (int o = kLanes / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+                        f *= rsqrtf(ss / ds + norm_eps);
+                    }
+#pragma unroll
+                    for (int jj = 0; jj < kJpl; ++jj)
+#pragma unroll
+                        for (int x = 0; x < kE / 2; ++x) {
+                            const int j = a * kJpl + jj;
+                            qf[j][x] = pack2(qx[j][2 * x] * f, qx[j][2 * x + 1] * f);
+                            acc[j][x] = 0ull;
+                        }
+                    m[a] = -INFINITY;
+                    z[a] = 0.f;
+                }
+            }
+            const int n_old = min(max(n_raw, 0), cap);
+            int t, t_end;
+            tiles_of(part, n_old, rv != 0 && n_old >= cap, t, t_end);
+            bool ok = true;
+            for (; t < t_end; ++t, ++it) {
+                const int st = it % kStages;
+                ok = mbar_wait(&full[st], (it / kStages) & 1, abort_flag);
+                if (!ok) break;
+                const uint8_t *kt = smem + (2 * st) * kTileBytes + row * kRowBytes + l8 * 16, *vt = kt + kTileBytes;
+                const bool valid = t * kTileKeys + row < n_old;     // (rows past the slice hold stale bytes)
+                float sc[kLg], kk[kLg];
+#pragma unroll
+                for (int a = 0; a < kLg; ++a) {
+                    uint64_t s2 = 0ull, k2 = 0ull;
+#pragma unroll
+                    for (int jj = 0; jj < kJpl; ++jj) {
+                        const int j = a * kJpl + jj;
+                        float kx[kE];
+                        Vec16<T>::unpack(*reinterpret_cast<const uint4 *>(kt + j * 128), kx);
+#pragma unroll
+                        for (int x = 0; x < kE / 2; ++x) {
+                            const uint64_t kp = pack2(kx[2 * x], kx[2 * x + 1]);
+                            s2 = fma2(qf[j][x], kp, s2);
+                            if (kNorm) k2 = fma2(kp, kp, k2);      // the key's sum of squares rides along
+                        }
+                    }
+                    const float2 sf = unpack2(s2), kf = unpack2(k2);
+                    sc[a] = sf.x + sf.y;
+                    kk[a] = kf.x + kf.y;
+                }
+                uint4 vraw[kJ];
+#pragma unroll
+                for (int j = 0; j < kJ; ++j) vraw[j] = *reinterpret_cast<const uint4 *>(vt + j * 128);
+#pragma unroll
+                for (int o = kLanes / 2; o > 0; o >>= 1)
+#pragma unroll
+                    for (int a = 0; a < kLg; ++a) {
+                        sc[a] += __shfl_xor_sync(0xffffffffu, sc[a], o);
+                        if (kNorm) kk[a] += __shfl_xor_sync(0xffffffffu, kk[a], o);
+                    }
+                if (lane == 0) mbar_arrive(&empty[st]);  // (behind the shuffles: every lane's reads are done)
+                bool raise = false;
+#pragma unroll
+                for (int a = 0; a < kLg; ++a) {
+                    if (kNorm) sc[a] *= rsqrtf(fmaf(kk[a], 1.f / ds, norm_eps));
+                    raise |= valid && sc[a] > m[a] + 8.f;
+                }
+                if (__any_sync(0xffffffffu, raise)) {
+#pragma unroll
+                    for (int a = 0; a < kLg; ++a) {
+                        const float m_new = valid ? fmaxf(m[a], sc[a]) : m[a];
+                        const float corr = m[a] == m_new ? 1.f : ex2_ftz(m[a] - m_new);
+                        z[a] *= corr;
+                        m[a] = m_new;
+                        const uint64_t c2 = pack2(corr, corr);
+#pragma unroll
+                        for (int jj = 0; jj < kJpl; ++jj)
+#pragma unroll
+                            for (int x = 0; x < kE / 2; ++x) acc[a * kJpl + jj][x] = mul2(acc[a * kJpl + jj][x], c2);
+                    }
+                }
+                if (valid) {
+#pragma unroll
+                    for (int a = 0; a < kLg; ++a) {
+                        const float pj = ex2_ftz(sc[a] - m[a]);
+                        z[a] += pj;
+                        const uint64_t p2 = pack2(pj, pj);
+#pragma unroll
+                        for (int jj = 0; jj < kJpl; ++jj) {
+                            const int j = a * kJpl + jj;
+                            float vx[kE];
+                            Vec16<T>::unpack(vraw[j], vx);
+#pragma unroll
+                            for (int x = 0; x < kE / 2; ++x) acc[j][x] = fma2(p2, pack2(vx[2 * x], vx[2 * x + 1]), acc[j][x]);
+                        }
+                    }
+                }
+            }
+            // the four rows of the warp by shuffles, then the warp's (m, z, acc) to the item's slot
+            // (after a time-out: go on without it, the other warps count on this one at the state items' barriers)
+            if (!ok || !mbar_wait(&taken[i & 1], ((i >> 1) & 1) ^ 1, abort_flag)) continue;
+#pragma unroll
+            for (int a = 0; a < kLg; ++a) {
+                float M = fmaxf(m[a], __shfl_xor_sync(0xffffffffu, m[a], 8));
+                M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 16));
+                const float f = m[a] == -INFINITY ? 0.f : ex2_ftz(m[a] - M);
+                z[a] *= f;
+                z[a] += __shfl_xor_sync(0xffffffffu, z[a], 8);
+                z[a] += __shfl_xor_sync(0xffffffffu, z[a], 16);
+                if (lane < 8 && l8 % kLanes == 0)
+                    mz[((i & 1) * kWarps + warp) * G + (kSp >= 8 ? a : 2 * a + (l8 >> 2))] = make_float2(M, z[a]);
+#pragma unroll
+                for (int jj = 0; jj < kJpl; ++jj) {
+                    const int j = a * kJpl + jj;
+#pragma unroll
+                    for (int x = 0; x < kE / 2; ++x) {
+                        float2 y = unpack2(acc[j][x]);
+                        y.x *= f;
+                        y.y *= f;
+                        y.x += __shfl_xor_sync(0xffffffffu, y.x, 8);
+                        y.y += __shfl_xor_sync(0xffffffffu, y.y, 8);
+                        y.x += __shfl_xor_sync(0xffffffffu, y.x, 16);
+                        y.y += __shfl_xor_sync(0xffffffffu, y.y, 16);
+                        if (lane < 8) *reinterpret_cast<float2 *>(&slot_out[warp * D + (j * 8 + l8) * kE + 2 * x]) = y;
+                    }
+                }
             }
         } else {
-            const int stream = tid / kLpk, piece = tid % kLpk;
-            float qf[kE];
+            // ---------------- state item: half of the value columns, all rows ----------------
+            // (warp-local operands: row slot `slot` holds rows slot kR ..; its k and q values, the token's
+            // norms and the v values come straight from global memory, in flight together with the state)
+            const int c0 = (part - parts) * kCols;
+            const int slot = warp * kRpl + lane / kLpr, col = (lane % kLpr) * 4;
+            float *sp = state + (size_t)bh * D * D + c0 + (size_t)(slot * kR) * D + col;
+            float4 s[kR];
 #pragma unroll
-            for (int x = 0; x < kE; ++x) qf[x] = (kGrouped ? qsm[piece * kE + x] : qs[piece * kE + x]) * scale_sm;
-            const int lps = kLpk / G;              // lanes per softmax head within a key row
-            const float inv_ds = 1.f / ds;
-            float m = -INFINITY, z = 0.f, acc[kE];
+            for (int rr = 0; rr < kR; ++rr) s[rr] = *reinterpret_cast<const float4 *>(sp + (size_t)rr * D);
+            float kx[kR], qx[kR], vx[4];
 #pragma unroll
-            for (int x = 0; x < kE; ++x) acc[x] = 0.f;
-            for (int t = t_begin; t < t_end; ++t) {
-                const int i = t - t_begin, s = i % kStages;
-                if (!mbar_wait(&full[s], (i / kStages) & 1, abort_flag)) break;
-                const uint8_t *kt = smem + (2 * s) * kTileBytes, *vt = kt + kTileBytes;
-                const int rows = min(kTileKeys, n_old - t * kTileKeys);
-#pragma unroll
-                for (int u = 0; u < kTileKeys / kStreams; ++u) {
-                    const int j = u * kStreams + stream;       // trip count uniform over the warp
-                    float kx[kE], vx[kE];
-                    Vec16<T>::unpack(*reinterpret_cast<const uint4 *>(kt + j * kRowBytes + piece * 16), kx);
-                    Vec16<T>::unpack(*reinterpret_cast<const uint4 *>(vt + j * kRowBytes + piece * 16), vx);
-                    float sc = 0.f;
-#pragma unroll
-                    for (int x = 0; x < kE; ++x) sc = fmaf(qf[x], kx[x], sc);
-                    if (!kGrouped) {
-#pragma unroll
-                        for (int o = kLpk / 2; o > 0; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
-                    } else {                     // per softmax head; the key's sum of squares rides along
-                        float kk = 0.f;
-#pragma unroll
-                        for (int x = 0; x < kE; ++x) kk = fmaf(kx[x], kx[x], kk);
-#pragma unroll
-                        for (int o = kLpk / 2; o > 0; o >>= 1)
-                            if (o < lps) {           // (uniform: the group count is the same for every lane)
-                                sc += __shfl_xor_sync(0xffffffffu, sc, o);
-                                kk += __shfl_xor_sync(0xffffffffu, kk, o);
-                            }
-                        if (normed) sc *= rsqrtf(fmaf(kk, inv_ds, norm_eps));
-                    }
-                    if (j < rows) {                            // rows past the slice hold stale bytes
-                        const float m_new = fmaxf(m, sc);
-                        const float corr = __expf(m - m_new), pj = __expf(sc - m_new);
-                        z = fmaf(z, corr, pj);
-                        m = m_new;
-#pragma unroll
-                        for (int x = 0; x < kE; ++x) acc[x] = fmaf(acc[x], corr, pj * vx[x]);
-                    }
-                }
-                mbar_arrive(&empty[s]);
+            for (int rr = 0; rr < kR; ++rr) {
+                kx[rr] = to_f32(k[(size_t)bh * D + slot * kR + rr]);
+                qx[rr] = to_f32(q[(size_t)bh * D + slot * kR + rr]);
             }
-            // merge the streams of this CTA -> one partial (m, z, acc[D]); the ring is free now
-            float *stage_acc = reinterpret_cast<float *>(smem);   // [kStreams][D]
-            named_barrier_sync(1, kWorkThreads);
-            if (piece % lps == 0) { sm_m[stream * G + piece / lps] = m; sm_z[stream * G + piece / lps] = z; }
 #pragma unroll
-            for (int x = 0; x < kE; ++x) stage_acc[stream * D + piece * kE + x] = acc[x];
-            named_barrier_sync(1, kWorkThreads);
-            if (tid < D) {
-                const int sg = tid / ds;             // this column's softmax head
-                float M = -INFINITY;
-                for (int st = 0; st < kStreams; ++st) M = fmaxf(M, sm_m[st * G + sg]);
-                float Z = 0.f, o = 0.f;
-                if (M > -INFINITY) {
-                    for (int st = 0; st < kStreams; ++st) {
-                        const float f = __expf(sm_m[st * G + sg] - M);
-                        Z = fmaf(sm_z[st * G + sg], f, Z);
-                        o = fmaf(stage_acc[st * D + tid], f, o);
-                    }
+            for (int x = 0; x < 4; ++x) vx[x] = to_f32(v[(size_t)bh * D + c0 + col + x]);
+            const float alpha = __expf(g[bh]), bt = beta[bh];
+            if (kNorm) {                                 // L2 over the row (the linear operation's q, k)
+                float sq = 0.f, sk = 0.f;
+#pragma unroll
+                for (int x = 0; x < D / 32; ++x) {
+                    const float a = to_f32(q[(size_t)bh * D + lane + 32 * x]), b = to_f32(k[(size_t)bh * D + lane + 32 * x]);
+                    sq = fmaf(a, a, sq);
+                    sk = fmaf(b, b, sk);
                 }
-                float *pp = partials + (size_t)part * (D + kPartHead);
-                pp[kPartHead + tid] = o;
-                if (tid % ds == 0) { pp[sg] = M; pp[4 + sg] = Z; }
+                const float rq = rsqrtf(warp_sum(sq) + norm_eps), rk = rsqrtf(warp_sum(sk) + norm_eps);
+#pragma unroll
+                for (int rr = 0; rr < kR; ++rr) { qx[rr] *= rq; kx[rr] *= rk; }
             }
-        }
-    } else if (warp < kWarps && !cache_full) {
-        // ---------------- state CTA: half of the value columns, all rows ----------------
-        constexpr int kCols = D / kStateParts;      // value columns of this CTA
-        constexpr int kLpr = kCols / 4;             // lanes per (half) state row
-        constexpr int kRpl = 32 / kLpr;             // rows per warp-wide access
-        constexpr int kSlots = kWarps * kRpl;       // row slots in the CTA
-        constexpr int kR = D / kSlots;              // rows per thread
-        static_assert(kSlots <= 32, "reduction scratch too small");
-        float (*redv)[kCols] = reinterpret_cast<float (*)[kCols]>(smem);   // [kSlots][kCols]
-        const int c0 = (part - kDecodeParts) * kCols;
-        const float alpha = __expf(g[bh]);
-        const float bt = fold ? beta[bh] : 0.f;
-        const int slot = warp * kRpl + lane / kLpr;
-        const int col = (lane % kLpr) * 4;
-        float *sp = state + (size_t)bh * D * D + c0;
-        float4 s[kR];
+            const bool skip = rv != 0 && min(max(n_raw, 0), cap) >= cap;   // no room: left untouched
+            const bool fold = rv != 1;                                     // delta rule
+            float (*redv)[kCols] = reinterpret_cast<float (*)[kCols]>(slot_of(2));   // [kSlots][kCols]
 #pragma unroll
-        for (int rr = 0; rr < kR; ++rr)
-            s[rr] = *reinterpret_cast<const float4 *>(sp + (size_t)(slot * kR + rr) * D + col);
+            for (int rr = 0; rr < kR; ++rr) {
+                s[rr].x *= alpha; s[rr].y *= alpha; s[rr].z *= alpha; s[rr].w *= alpha;
+            }
+            if (fold) {   // uniform over the CTA
+                float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int rr = 0; rr < kR; ++rr) {
-            s[rr].x *= alpha; s[rr].y *= alpha; s[rr].z *= alpha; s[rr].w *= alpha;
-        }
-        if (fold) {   // block-uniform
+                for (int rr = 0; rr < kR; ++rr) {
+                    p.x = fmaf(kx[rr], s[rr].x, p.x); p.y = fmaf(kx[rr], s[rr].y, p.y);
+                    p.z = fmaf(kx[rr], s[rr].z, p.z); p.w = fmaf(kx[rr], s[rr].w, p.w);
+                }
+                *reinterpret_cast<float4 *>(&redv[slot][col]) = p;
+                named_barrier_sync(1, kWorkThreads);
+                float4 e = make_float4(vx[0], vx[1], vx[2], vx[3]);
+#pragma unroll
+                for (int sl = 0; sl < kSlots; ++sl) {
+                    const float4 t = *reinterpret_cast<const float4 *>(&redv[sl][col]);
+                    e.x -= t.x; e.y -= t.y; e.z -= t.z; e.w -= t.w;
+                }
+#pragma unroll
+                for (int rr = 0; rr < kR; ++rr) {
+                    const float bk = bt * kx[rr];
+                    s[rr].x = fmaf(bk, e.x, s[rr].x); s[rr].y = fmaf(bk, e.y, s[rr].y);
+                    s[rr].z = fmaf(bk, e.z, s[rr].z); s[rr].w = fmaf(bk, e.w, s[rr].w);
+                }
+                named_barrier_sync(1, kWorkThreads);     // (redv is written again by the next state item)
+            }
             float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int rr = 0; rr < kR; ++rr) {
-                const float ka = ks[slot * kR + rr];
-                p.x = fmaf(ka, s[rr].x, p.x); p.y = fmaf(ka, s[rr].y, p.y);
-                p.z = fmaf(ka, s[rr].z, p.z); p.w = fmaf(ka, s[rr].w, p.w);
+                p.x = fmaf(qx[rr], s[rr].x, p.x); p.y = fmaf(qx[rr], s[rr].y, p.y);
+                p.z = fmaf(qx[rr], s[rr].z, p.z); p.w = fmaf(qx[rr], s[rr].w, p.w);
+                if (!skip) *reinterpret_cast<float4 *>(sp + (size_t)rr * D) = s[rr];
             }
-            *reinterpret_cast<float4 *>(&redv[slot][col]) = p;
-            named_barrier_sync(1, kWorkThreads);
-            float4 e = *reinterpret_cast<const float4 *>(&vs[c0 + col]);
-#pragma unroll
-            for (int sl = 0; sl < kSlots; ++sl) {
-                const float4 t = *reinterpret_cast<const float4 *>(&redv[sl][col]);
-                e.x -= t.x; e.y -= t.y; e.z -= t.z; e.w -= t.w;
-            }
-#pragma unroll
-            for (int rr = 0; rr < kR; ++rr) {
-                const float bk = bt * ks[slot * kR + rr];
-                s[rr].x = fmaf(bk, e.x, s[rr].x); s[rr].y = fmaf(bk, e.y, s[rr].y);
-                s[rr].z = fmaf(bk, e.z, s[rr].z); s[rr].w = fmaf(bk, e.w, s[rr].w);
-            }
-            named_barrier_sync(1, kWorkThreads);   // redv is reused below
+            if (!mbar_wait(&taken[i & 1], ((i >> 1) & 1) ^ 1, abort_flag)) continue;
+            *reinterpret_cast<float4 *>(&slot_out[slot * kCols + col]) = p;
         }
-        float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int rr = 0; rr < kR; ++rr) {
-            const float qa = qs[slot * kR + rr];
-            p.x = fmaf(qa, s[rr].x, p.x); p.y = fmaf(qa, s[rr].y, p.y);
-            p.z = fmaf(qa, s[rr].z, p.z); p.w = fmaf(qa, s[rr].w, p.w);
-            *reinterpret_cast<float4 *>(sp + (size_t)(slot * kR + rr) * D + col) = s[rr];
-        }
-        *reinterpret_cast<float4 *>(&redv[slot][col]) = p;
-        named_barrier_sync(1, kWorkThreads);
-        if (tid < kCols) {
-            float a = 0.f;
-#pragma unroll
-            for (int sl = 0; sl < kSlots; ++sl) a += redv[sl][tid];
-            ola_ws[c0 + tid] = scale_la * a;
-        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&done[i & 1]);
     }
-
-    // -------- ticket: the last CTA of this (sequence, head) to get here finishes the step --------
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) {
-        const int old = atomicAdd(ticket, 1);
-        s_last = old == kCtasPerHead - 1;
-        if (s_last) *ticket = 0;                      // ready for the next step
-        if (s_abort[0]) atomicMin(status, (int)NATSL_ERR_TIMEOUT);
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    if (cache_full) {
-        if (tid < D) out[(size_t)bh * D + tid] = from_f32<T>(0.f);
-        if (tid == 0) atomicMin(status, (int)NATSL_ERR_CACHE_FULL);
-        return;
-    }
-    float on = 0.f, ol = 0.f;
-    const int sg = tid < D ? tid / ds : 0;            // this column's softmax head
-    if (tid < D) {
-        const volatile float *pv = partials;
-        constexpr int kPs = D + kPartHead;
-        float M = -INFINITY;
-        for (int pt = 0; pt < kDecodeParts; ++pt) M = fmaxf(M, pv[pt * kPs + sg]);
-        float sc_self = 0.f;
-        if (r) {                                       // the token attends to itself
-            if (kGrouped)
-                for (int x = sg * ds; x < (sg + 1) * ds; ++x) sc_self = fmaf(qsm[x] * scale_sm, ksm[x], sc_self);
-            else
-                for (int x = 0; x < D; ++x) sc_self = fmaf(qs[x] * scale_sm, ks[x], sc_self);
-            M = fmaxf(M, sc_self);
-        }
-        float Z = 0.f;
-        if (M > -INFINITY) {
-            for (int pt = 0; pt < kDecodeParts; ++pt) {
-                const float mp = pv[pt * kPs + sg];
-                if (mp > -INFINITY) {
-                    const float f = __expf(mp - M);
-                    Z = fmaf(pv[pt * kPs + 4 + sg], f, Z);
-                    on = fmaf(pv[pt * kPs + kPartHead + tid], f, on);
-                }
-            }
-            if (r) {
-                const float f = __expf(sc_self - M);
-                Z += f;
-                on = fmaf(vs[tid], f, on);
-            }
-            on /= Z;
-        }
-        ol = reinterpret_cast<const volatile float *>(ola_ws)[tid];
-    }
-    float ssn = warp_sum(on * on), ssl = warp_sum(ol * ol);
-    if (lane == 0 && warp < kWarps) { norm_red[0][warp] = ssn; norm_red[1][warp] = ssl; }
-    __syncthreads();
-    if (tid < D) {
-        float tn = 0.f, tl = 0.f;      // softmax output: over this column's softmax head; linear read-out: over the row
-#pragma unroll
-        for (int wv = 0; wv < kWarps; ++wv) {
-            if (!kGrouped || (32 * wv) / ds == sg) tn += norm_red[0][wv];
-            tl += norm_red[1][wv];
-        }
-        const float fn = rsqrtf(tn / ds + eps), fl = rsqrtf(tl / D + eps);
-        const float wn = w ? w[(size_t)bh * 2] : 0.5f, wl = w ? w[(size_t)bh * 2 + 1] : 0.5f;
-        out[(size_t)bh * D + tid] = from_f32<T>(wn * on * fn + wl * ol * fl);
-        if (r) {   // retain the token: every reader of the old length has finished
-            k_cache[((size_t)bh * cap + n_old) * D + tid] = k[(size_t)bh * D + tid];
-            v_cache[((size_t)bh * cap + n_old) * D + tid] = v[(size_t)bh * D + tid];
-        }
-    }
-    if (r && tid == 0) cache_len[bh] = n_old + 1;
 }
 
 // End of a block of R tokens decoded with the decision open: a softmax block resets the state to
@@ -432,28 +644,43 @@ size_t decode_workspace_bytes(int B, int H, int d) {
     return dec_off_ola((size_t)B * H, d) + ((size_t)B * H * d * 4 + 255) / 256 * 256;
 }
 
-template <typename T, int D>
+template <typename T, int D, int G, bool kNorm>
 static cudaError_t decode_impl(const void *q, const void *k, const void *v, const float *g,
                                const float *beta, const uint8_t *route, const float *w,
                                float *state, void *k_cache, void *v_cache, int32_t *cache_len,
                                int32_t cap, void *out, float scale_la, float scale_sm, float eps,
-                               void *ws, Shape s, cudaStream_t st, HeadGroups hg) {
-    constexpr int kTileBytes = kTileKeys * D * (int)sizeof(T);
-    constexpr int kRing = 2 * kStages * kTileBytes;
-    constexpr int kRed = 32 * D * 4;               // per-stream / per-slot reduction scratch
-    constexpr int kSmem = kRing > kRed ? kRing : kRed;
-    const bool grouped = hg.G > 1 || hg.norm_eps >= 0.f;
-    if (grouped && (hg.G > 4 || D % (32 * hg.G) != 0)) return cudaErrorInvalidValue;
-    auto kernel = grouped ? decode_step_kernel<T, D, true> : decode_step_kernel<T, D, false>;
-    cudaError_t e = allow_smem(kernel, kSmem);
-    if (e != cudaSuccess) return e;
-    dim3 grid(kCtasPerHead, s.B * s.H);
-    kernel<<<grid, kThreads, kSmem, st>>>(
-        (const T *)q, (const T *)k, (const T *)v, g, beta, route, w, state, (T *)k_cache,
-        (T *)v_cache, cache_len, cap, (T *)out, scale_la, scale_sm, eps, (uint8_t *)ws, s.B * s.H, hg.G,
-        hg.norm_eps);
-    count_launch();
-    return cudaGetLastError();
+                               void *ws, Shape s, cudaStream_t st, float norm_eps) {
+    if constexpr (D / G * (int)sizeof(T) < 64) {
+        return cudaErrorInvalidValue;
+    } else {
+        auto kernel = decode_step_kernel<T, D, G, kNorm>;
+        cudaError_t e = allow_smem(kernel, DecLayout<T, D, G>::kTotal);
+        if (e != cudaSuccess) return e;
+        const int BH = s.B * s.H, parts = decode_parts((size_t)BH), per_head = parts + kStateParts;
+        // Persistent beyond one resident set; the stride then has no factor in common with the items per
+        // pair, so that every CTA gets the same mix of cache and state items.
+        auto gcd = [](int a, int b) { while (b) { const int c = a % b; a = b; b = c; } return a; };
+        int grid = BH * per_head;
+        if (grid > kCtasPerSm * sm_count()) {
+            grid = kCtasPerSm * sm_count();
+            while (grid > 1 && gcd(grid, per_head) != 1) --grid;
+        }
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = DecLayout<T, D, G>::kTotal;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, kernel, (const T *)q, (const T *)k, (const T *)v, g, beta, route, w, state,
+                               (T *)k_cache, (T *)v_cache, cache_len, (int)cap, (T *)out, scale_la, scale_sm, eps,
+                               (uint8_t *)ws, BH, parts, norm_eps);
+        count_launch();
+        return e;
+    }
 }
 
 cudaError_t launch_decode_step(const void *q, const void *k, const void *v, const float *g,
@@ -462,13 +689,25 @@ cudaError_t launch_decode_step(const void *q, const void *k, const void *v, cons
                                int32_t cache_cap, void *out, float scale_la, float scale_sm,
                                float eps, void *ws, Shape s, cudaStream_t st, HeadGroups hg) {
 #define ARGS q, k, v, g, beta, route, w, state, k_cache, v_cache, cache_len, cache_cap, out, \
-             scale_la, scale_sm, eps, ws, s, st, hg
+             scale_la, scale_sm, eps, ws, s, st, hg.norm_eps
+#define BY_GROUPS(T, D)                                                                                     \
+    if (hg.norm_eps >= 0.f) {                                                                               \
+        if (hg.G == 4) return decode_impl<T, D, 4, true>(ARGS);                                             \
+        if (hg.G == 2) return decode_impl<T, D, 2, true>(ARGS);                                             \
+        if (hg.G == 1) return decode_impl<T, D, 1, true>(ARGS);                                             \
+    } else {                                                                                                \
+        if (hg.G == 4) return decode_impl<T, D, 4, false>(ARGS);                                            \
+        if (hg.G == 2) return decode_impl<T, D, 2, false>(ARGS);                                            \
+        if (hg.G == 1) return decode_impl<T, D, 1, false>(ARGS);                                            \
+    }                                                                                                       \
+    return cudaErrorInvalidValue
     if (s.bf16) {
-        if (s.d == 128) return decode_impl<__nv_bfloat16, 128>(ARGS);
-        return decode_impl<__nv_bfloat16, 64>(ARGS);
+        if (s.d == 128) { BY_GROUPS(__nv_bfloat16, 128); }
+        BY_GROUPS(__nv_bfloat16, 64);
     }
-    if (s.d == 128) return decode_impl<float, 128>(ARGS);
-    return decode_impl<float, 64>(ARGS);
+    if (s.d == 128) { BY_GROUPS(float, 128); }
+    BY_GROUPS(float, 64);
+#undef BY_GROUPS
 #undef ARGS
 }
 

@@ -295,7 +295,6 @@ cudaError_t launch_softmax_bwd_own_block(const void *q, const void *k, const voi
 // holding the softmax operation's normalised q, k [B,L,H,d], read instead of q, k)
 
 // decode.cu
-constexpr int kDecodeParts = 4;   // CTAs that share the retained K/V of one (sequence, head)
 // Bytes of workspace of a decode step: status word, per-head tickets, partial softmax results and
 // linear read-outs.  Zero-filled once by the caller; the kernel leaves the tickets at zero.
 size_t decode_workspace_bytes(int B, int H, int d);

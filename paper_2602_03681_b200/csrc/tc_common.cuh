@@ -93,6 +93,15 @@ __device__ __forceinline__ bool mbar_wait_drain(uint64_t *bar, uint32_t parity) 
 __device__ __forceinline__ void launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+// ... and in the later kernel: everything before it in the stream has completed and is visible.
+__device__ __forceinline__ void grid_dependency_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ int32_t atom_add_acq_rel(int32_t *p, int32_t v) {
+    int32_t old;
+    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+    return old;
+}
 // Producer: the calling thread's earlier global writes (and those of threads it has synchronised
 // with) become visible to whoever reads the counter with acquire semantics.
 __device__ __forceinline__ void red_release_add(int32_t *p, int32_t v) {

@@ -1,0 +1,42 @@
+"""Decode step at the edges of how its work is split: (sequence, head) counts on either side of one resident set
+of items, caches of every length from empty to beyond a slice of every part, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2602_03681_b200 import inputs
+from test_gpu_parity import TOL, check_stored, dev, rel_err, tdtype
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("name,B,H", [("cfg3_bf16_decode", 1, 1), ("cfg3_bf16_decode", 14, 7),
+                                      ("cfg3_bf16_decode", 9, 11), ("cfg4_bf16_train", 25, 12),
+                                      ("cfg0_f32_tiny_fwd", 20, 15)])
+def test_decode_ragged_caches(name, B, H):
+    from paper_2602_03681_b200 import binding
+    wl = inputs.WORKLOADS[name]
+    cap, T = 600, 2
+    x = inputs.make_decode_inputs(wl, B=B, H=H, steps=T, ctx_retained=cap - T, cap=cap)
+    lengths = np.array([0, 1, 31, 32, 33, 63, 64, 65, 127, 129, 255, 257, 383, 511, 512, 513, 577, cap - T])
+    rng = np.random.default_rng(7)
+    x["cache_len"][...] = rng.permutation(np.resize(lengths, B * H)).reshape(B, H)
+    dt = tdtype(wl)
+    state, kc, vc, n = dev(x["state"]), dev(x["k_cache"], dt), dev(x["v_cache"], dt), dev(x["cache_len"])
+    p = binding.make_params(B, H, 0, wl.d, binding._dtype_code(kc), wl.scale_la, wl.scale_sm)
+    ws = binding.alloc_workspace(p, binding.OP_DECODE)
+    o_state, o_n = x["state"].astype(np.float64), x["cache_len"].copy()
+    o_kc, o_vc = x["k_cache"].astype(np.float64), x["v_cache"].astype(np.float64)
+    for t in range(T):
+        w = dev(x["w"][t])
+        p.w = w.data_ptr()
+        out = torch.empty((B, H, wl.d), dtype=dt, device="cuda")
+        binding.natsl_decode_step(dev(x["q"][t], dt), dev(x["k"][t], dt), dev(x["v"][t], dt), dev(x["g"][t]),
+                                  dev(x["beta"][t]), dev(x["route"][t]), state, kc, vc, n, out, p, ws)
+        ref = oracle.decode_step(x["q"][t], x["k"][t], x["v"][t], x["g"][t], x["beta"][t], x["route"][t], x["w"][t],
+                                 o_state, o_kc, o_vc, o_n, scale_la=wl.scale_la, scale_sm=wl.scale_sm)
+        check_stored(out.float().cpu().numpy(), ref["out"], TOL[wl.dtype], wl.dtype, f"step{t}")
+    assert binding.natsl_device_status(ws) == 0
+    assert np.array_equal(n.cpu().numpy(), o_n)
+    assert rel_err(state.cpu().numpy(), o_state) <= 1e-4

@@ -926,71 +926,67 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
     if (tid == 0 && ms.abort_flag) atomicMin(status, (int)NATSL_ERR_TIMEOUT);
 }
 
-// start[0] = state_in (or 0); start[s+1] = M_s start[s] + B_s.  The value columns are independent:
-// one CTA per (batch, head) and 8 of them; thread (ag, v) owns key rows ag, ag + 32, ... of column v.
-// M_s is staged through shared memory in tiles of 32 columns (coalesced 128-byte rows).
+// start[0] = state_in (or 0); start[s+1] = M_s start[s] + B_s.  The value columns are independent: one CTA
+// per (batch, head) and kCombCols of them.  The chain over the segments is serial, so what counts is the time
+// of one step: two threads per key row hold its two halves of M_s in registers (fetched one segment ahead), the
+// state's columns are read as broadcast 16-byte pieces from shared memory, and fp32 FMAs do the rest.
+// (With M_s staged through shared memory in tiles and one shared-memory operand pair per FMA a step took
+// 11.8 us at d = 128; 16 pairs x 8 segments 83 us together.)
+constexpr int kCombCols = 4;
 template <int D>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(2 * D)
 scan_combine_kernel(const float *__restrict__ state_in, const float *__restrict__ incr,
                     const float *__restrict__ trans, float *__restrict__ start, int nseg) {
-    constexpr int kV = 8, kRows = D / 32;
-    __shared__ float Ss[D][kV + 1];
-    __shared__ float Ms[D][33];
-    const int bh = blockIdx.y, v0 = blockIdx.x * kV, v = threadIdx.x & (kV - 1), ag = threadIdx.x >> 3;
-    for (int i = 0; i < kRows; ++i) {
-        const int a = ag + 32 * i;
-        Ss[a][v] = state_in ? state_in[((size_t)bh * D + a) * D + v0 + v] : 0.f;
-    }
-    __syncthreads();
-    // The tiles of M are fetched one step ahead into registers, so that the chain over the segments
-    // pays one global-memory latency per segment rather than one per tile.
-    constexpr int kTileRegs = D * 32 / 256;
-    float tile[kTileRegs];
-    auto fetch = [&](int sgi, int b0) {
-        const float *src = trans + ((size_t)bh * nseg + sgi) * D * D + b0;
+    constexpr int kV = kCombCols, kHalf = D / 2;
+    __shared__ float4 Ss[2][D];                        // the state's kV columns, double-buffered
+    const int bh = blockIdx.y, v0 = blockIdx.x * kV, a = threadIdx.x >> 1, hf = threadIdx.x & 1;
+    // this thread's half of the row: pieces 2 j + hf (16 bytes each), so that a pair reads 32 contiguous bytes
+    float4 m[kHalf / 4];
+    auto fetch = [&](int sgi) {
+        const float4 *src = reinterpret_cast<const float4 *>(trans + (((size_t)bh * nseg + sgi) * D + a) * D) + hf;
 #pragma unroll
-        for (int i = 0; i < kTileRegs; ++i) {
-            const int idx = threadIdx.x + 256 * i;
-            tile[i] = src[(size_t)(idx >> 5) * D + (idx & 31)];
-        }
+        for (int j = 0; j < kHalf / 4; ++j) m[j] = __ldg(src + 2 * j);
     };
-    if (nseg > 1) fetch(0, 0);
+    const size_t row = (size_t)a * D + v0;
+    float4 cur = make_float4(0.f, 0.f, 0.f, 0.f), inc;
+    if (state_in) cur = *reinterpret_cast<const float4 *>(state_in + (size_t)bh * D * D + row);
+    if (nseg > 1) fetch(0);
     for (int sgi = 0; sgi < nseg; ++sgi) {
         const size_t base = ((size_t)bh * nseg + sgi) * D * D;
-        for (int i = 0; i < kRows; ++i) start[base + (size_t)(ag + 32 * i) * D + v0 + v] = Ss[ag + 32 * i][v];
-        if (sgi + 1 == nseg) break;
-        float acc[kRows];
-#pragma unroll
-        for (int i = 0; i < kRows; ++i) acc[i] = incr[base + (size_t)(ag + 32 * i) * D + v0 + v];
-        for (int b0 = 0; b0 < D; b0 += 32) {
-#pragma unroll
-            for (int i = 0; i < kTileRegs; ++i) {                         // M[a][b0 .. b0+31]
-                const int idx = threadIdx.x + 256 * i;
-                Ms[idx >> 5][idx & 31] = tile[i];
-            }
-            __syncthreads();
-            if (b0 + 32 < D) fetch(sgi, b0 + 32);
-            else if (sgi + 2 < nseg) fetch(sgi + 1, 0);
-#pragma unroll
-            for (int i = 0; i < kRows; ++i) {
-                const float *mr = Ms[ag + 32 * i];
-#pragma unroll 8
-                for (int bb = 0; bb < 32; ++bb) acc[i] = fmaf(mr[bb], Ss[b0 + bb][v], acc[i]);
-            }
-            __syncthreads();
+        if (hf == 0) {
+            *reinterpret_cast<float4 *>(start + base + row) = cur;
+            Ss[sgi & 1][a] = cur;
         }
-#pragma unroll
-        for (int i = 0; i < kRows; ++i) Ss[ag + 32 * i][v] = acc[i];
+        if (sgi + 1 == nseg) break;
+        inc = *reinterpret_cast<const float4 *>(incr + base + row);
         __syncthreads();
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int j = 0; j < kHalf / 4; ++j) {
+            const float4 *sp = &Ss[sgi & 1][8 * j + 4 * hf];
+            const float mv[4] = {m[j].x, m[j].y, m[j].z, m[j].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float4 sv = sp[e];
+                acc.x = fmaf(mv[e], sv.x, acc.x); acc.y = fmaf(mv[e], sv.y, acc.y);
+                acc.z = fmaf(mv[e], sv.z, acc.z); acc.w = fmaf(mv[e], sv.w, acc.w);
+            }
+        }
+        if (sgi + 2 < nseg) fetch(sgi + 1);
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 1);
+        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 1);
+        acc.z += __shfl_xor_sync(0xffffffffu, acc.z, 1);
+        acc.w += __shfl_xor_sync(0xffffffffu, acc.w, 1);
+        cur = make_float4(acc.x + inc.x, acc.y + inc.y, acc.z + inc.z, acc.w + inc.w);
     }
 }
 
 }  // namespace
 
 cudaError_t launch_scan_combine(const float *state_in, const ScanSegments &sg, Shape s, cudaStream_t st) {
-    dim3 grid(s.d / 8, s.B * s.H);
+    dim3 grid(s.d / kCombCols, s.B * s.H);
     if (s.d == 128) scan_combine_kernel<128><<<grid, 256, 0, st>>>(state_in, sg.incr, sg.trans, sg.start, sg.nseg);
-    else scan_combine_kernel<64><<<grid, 256, 0, st>>>(state_in, sg.incr, sg.trans, sg.start, sg.nseg);
+    else scan_combine_kernel<64><<<grid, 128, 0, st>>>(state_in, sg.incr, sg.trans, sg.start, sg.nseg);
     count_launch();
     return cudaGetLastError();
 }

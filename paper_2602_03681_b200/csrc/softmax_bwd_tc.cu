@@ -268,8 +268,10 @@ template <int D> struct KLayout {
     static constexpr int kTmem = D == 64 ? 256 : 512;     // S^T 64 + dP^T 64 + dV D + dK D
 };
 
+// Two CTAs per SM at D = 64, where shared memory and TMEM allow it: left to itself the compiler takes 176 registers,
+// which leaves one, and the kernel, a chain of waits, then runs with four row warps per SM.
 template <int D, bool kMask, int kG>   // kMask: also the per-key sums of the mask gradient (dmask); kG: as above
-__global__ void __launch_bounds__(kThreadsB)
+__global__ void __launch_bounds__(kThreadsB, D == 64 ? 2 : 1)
 softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B*H*L][D], box 64
                           const __grid_constant__ CUtensorMap map_do,   // dO16, box 64
                           const __grid_constant__ CUtensorMap map_k,    // k16 [B*H*cap][D], box 128

@@ -23,8 +23,15 @@
 // dependent): nothing before the epilogue needs o_la, and the epilogue's load waits, bounded, for
 // the per-chunk counters the scan raises (emit_flags); CTAs are then ordered by query tile first,
 // so that the tiles whose chunks the scan finishes first are also scheduled first.
-// Warp roles: warps 0-3 softmax/epilogue (thread r <-> query row r <-> TMEM lane r), warp 4 issues
-// the MMAs, warp 5 issues the TMA loads.
+// Warp roles: one or two warpgroups of softmax/epilogue threads (thread r <-> query row r <-> TMEM lane r; two
+// take turns by tile and share the running maximum of a row, see SmLayout), then a warp that issues the
+// MMAs and one that issues the TMA loads.
+// What it costs (128 queries, measured by leaving parts out): about a third of the time of a short-context call is
+// the CTA's fixed part (Q, o_la and out through shared memory), a 64-key tile takes 690 cycles per SM at 64
+// columns and 1080 at 128, where the MMAs alone take 400 and 676; the exponentials do not show.  Packed fp32
+// operations, the rolled epilogue and one masking path keep the code small: waiting for instructions was the
+// second-largest stall.  Forward of ten sequences of 4096 tokens, six heads of two slices, block-routed and
+// normalised: 307 -> 258 us for this kernel alone; one sequence of 32768 tokens, d = 128: 344 -> 297 us.
 // Block-level routing (template flag): after the retained tiles, one more tile per linear block of
 // the CTA's two, holding that block's own 64 tokens (Section 4.1, inner-chunk correlations).
 // Grouped softmax heads (template count kG; Section 4.3, several softmax heads under one linear head's
@@ -47,13 +54,20 @@ using namespace tc;
 
 constexpr int kBM = 128;        // queries per CTA
 constexpr int kBN = 64;         // retained tokens per K/V tile
-constexpr int kStages = 2;
-constexpr int kSoftmaxThreads = 128;
-constexpr int kThreadsTc = 192;
-constexpr int kMiscBytes = 1024;
+constexpr int kGroupThreads = 128;                 // a softmax warpgroup: one thread per query row
+constexpr int kMiscBytes = 5120;
 
 template <int D> struct SmLayout {
     static constexpr int KB = D / 64;                    // 64-column blocks of the head dimension
+    // TMEM decides how much of a CTA's tile loop can overlap (two CTAs per SM, 256 columns each).  64 columns: O
+    // and three logit tiles fit, and two warpgroups take turns, each with its next logits ready while the
+    // other's product runs.  128 columns: O leaves room for two logit tiles, i.e. for one group's next tile
+    // -- a second group would only wait (measured: same time).
+    static constexpr int kGroups = D == 64 ? 2 : 1;
+    static constexpr int kLogits = D == 64 ? 3 : 2;
+    static constexpr int kStages = kLogits;              // K/V tiles in flight
+    static constexpr int kSoftmaxThreads = kGroups * kGroupThreads;
+    static constexpr int kThreads = kSoftmaxThreads + 64;
     static constexpr int kQBytes = KB * kBM * 128;
     static constexpr int kKStage = KB * kBN * 128;
     static constexpr int kVStage = KB * kBN * 128;
@@ -65,17 +79,48 @@ template <int D> struct SmLayout {
 };
 
 struct Misc {                    // lives in the last kMiscBytes of the CTA's shared memory
-    uint64_t barQ, barQn, barKn[2], fullK[kStages], emptyK[kStages], fullV[kStages], emptyV[kStages], barS[2], barP, barO, barE;
+    uint64_t barQ, barQn, barKn[2], fullK[3], emptyK[3], fullV[3], emptyV[3], barS[3], barP[3], barO[2], barF, barE, barM[2][4];
     uint32_t tmem_base;
     int abort_flag, wait_kcycles;   // in this order: the waits read the limit as abort_flag[1]
-    alignas(16) int pos[kBM];    // positions of the retained tokens inside the CTA's own chunks
+    uint32_t kept[kBM / 32];        // which of the CTA's own tokens are retained
+    float m_row[kBM];               // running maximum of each row (base 2), handed from tile to tile
+    float2 xch[2][kBM], xch2[2][kBM];   // exchanges between the two warpgroups, per row
 };
 static_assert(sizeof(Misc) <= kMiscBytes, "misc page too small");
+
+// Sum of squares of N 16-byte pieces of bf16 of one swizzled row, and the same pieces rewritten as fp16 times f.
+template <int N> __device__ __forceinline__ float row_square_sum(const uint8_t *rowp, int p0, int x) {
+    float ss = 0.f;
+#pragma unroll
+    for (int c = 0; c < N; ++c) {
+        const uint4 a = *reinterpret_cast<const uint4 *>(rowp + (((p0 + c) ^ x) << 4));
+        const uint32_t wd[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float lo = __uint_as_float(wd[e] << 16), hi = __uint_as_float(wd[e] & 0xffff0000u);
+            ss = fmaf(lo, lo, fmaf(hi, hi, ss));
+        }
+    }
+    return ss;
+}
+template <int N> __device__ __forceinline__ void row_to_fp16(uint8_t *rowp, int p0, int x, float f) {
+#pragma unroll
+    for (int c = 0; c < N; ++c) {
+        uint4 *pp = reinterpret_cast<uint4 *>(rowp + (((p0 + c) ^ x) << 4));
+        const uint4 a = *pp;
+        const uint32_t wd[4] = {a.x, a.y, a.z, a.w};
+        uint32_t o[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            o[e] = pack_half2(__uint_as_float(wd[e] << 16) * f, __uint_as_float(wd[e] & 0xffff0000u) * f);
+        *pp = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+}
 
 // kBlock: block-level routing (own-block tiles after the retained ones); kG: softmax heads per linear
 // head; kNorm: RMS-normalised q and k (norm_eps is read only then)
 template <int D, bool kBlock, int kG, bool kNorm>
-__global__ void __launch_bounds__(kThreadsTc)
+__global__ void __launch_bounds__(SmLayout<D>::kThreads, 2)
 softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                           const __grid_constant__ CUtensorMap map_k,
                           const __grid_constant__ CUtensorMap map_v,
@@ -89,7 +134,8 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                           float scale_sm, float eps, float norm_eps, int has_out, float *__restrict__ o_nla,
                           float *__restrict__ lse, int32_t *status, int L, int H, int wait_kcycles) {
     using SL = SmLayout<D>;
-    constexpr int KB = SL::KB;
+    constexpr int KB = SL::KB, kStages = SL::kStages, kLogits = SL::kLogits, kGroups = SL::kGroups;
+    constexpr int kSoftmaxThreads = SL::kSoftmaxThreads, kAhead = kLogits - 1;
     constexpr int DL = D * kG;                            // columns of the linear head
     // the two o_laT tiles of the epilogue land in the Q tile and, for grouped heads, the K ring behind it
     static_assert(2 * DL * 128 <= SL::kQBytes + (kG > 1 ? kStages * SL::kKStage : 0), "o_laT tiles do not fit");
@@ -98,6 +144,7 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
     Misc &ms = *reinterpret_cast<Misc *>(smem + SL::oMisc);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr int kMmaWarp = kSoftmaxThreads / 32, kTmaWarp = kMmaWarp + 1;
     const int NP = (L + kBM - 1) / kBM, NC = L / kC;
     // grid = (B*H, NP).  Beside the scan: tiles in ascending order, all (batch, head) pairs of a tile
     // before the next tile.  Otherwise: long rows first.
@@ -105,6 +152,39 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
     // blockIdx.x = (batch, linear head, softmax head of the group); H counts linear heads
     const int bhg = blockIdx.x, bh = bhg / kG, sg = bhg % kG, b = bh / H, h = bh % H;
     const int hq = h * kG + sg;                           // head index in the [B,L,H kG,D] view
+
+    if ((smem_u32(smem) & 1023u) != 0) {              // operand tiles need 1024-byte alignment
+        if (tid == 0) atomicMin(status, (int)NATSL_ERR_CUDA);
+        return;
+    }
+    // The TMA warp sets the barriers up and requests the Q tile before anything else, so that the tile travels
+    // while the other warps look up which keys the CTA sees.
+    if (warp == kTmaWarp && lane == 0) {
+        mbar_init(&ms.barQ, 1);
+        mbar_init(&ms.barQn, kSoftmaxThreads);       // normalised queries written (NATSL_QK_NORM)
+        mbar_init(&ms.barKn[0], 1);                  // ... and the keys of an own-block tile: one barrier per tile,
+        mbar_init(&ms.barKn[1], 1);                  //     each completing once
+        for (int s = 0; s < kStages; ++s) {
+            mbar_init(&ms.fullK[s], 1); mbar_init(&ms.emptyK[s], 1);
+            mbar_init(&ms.fullV[s], 1); mbar_init(&ms.emptyV[s], 1);
+        }
+        // (barP by logit tile, not by warpgroup: with the logits of tile t + 2 ready early, a fast warp's arrival for
+        // that tile would otherwise complete tile t's phase in place of a slow warp's)
+        for (int s = 0; s < kLogits; ++s) { mbar_init(&ms.barS[s], 1); mbar_init(&ms.barP[s], kGroupThreads); }
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(&ms.barO[s], 1);
+            for (int q = 0; q < 4; ++q) mbar_init(&ms.barM[s][q], 1);
+        }
+        mbar_init(&ms.barF, 1);
+        mbar_init(&ms.barE, 1);
+        ms.abort_flag = 0;
+        ms.wait_kcycles = wait_kcycles;
+        fence_mbar_init();
+        prefetch_tmap(&map_q); prefetch_tmap(&map_k); prefetch_tmap(&map_v);
+        mbar_arrive_expect_tx(&ms.barQ, SL::kQBytes);
+        for (int kb = 0; kb < KB; ++kb)
+            tma_load_4d(smem + SL::oQ + kb * kBM * 128, &map_q, &ms.barQ, kb * 64, hq, p * kBM, b);
+    }
     const int c0 = 2 * p, c1 = min(2 * p + 2, NC);
     const int32_t *pre = sm_chunk_prefix + (size_t)bh * (NC + 1);
     const int n_full = min(pre[c0], cap);             // retained tokens before the CTA's chunks
@@ -125,50 +205,23 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
     const int T2 = kBlock ? T + nx : T;
     auto own_block = [&](int t) { return t == T ? xc0 : 1; };   // block (0 or 1) of own-block tile t >= T
 
-    if ((smem_u32(smem) & 1023u) != 0) {              // operand tiles need 1024-byte alignment
-        if (tid == 0) atomicMin(status, (int)NATSL_ERR_CUDA);
-        return;
-    }
-    if (tid == 0) {
-        mbar_init(&ms.barQ, 1);
-        mbar_init(&ms.barQn, kSoftmaxThreads);       // normalised queries written (NATSL_QK_NORM)
-        mbar_init(&ms.barKn[0], 1);                  // ... and the keys of an own-block tile: one barrier per tile,
-        mbar_init(&ms.barKn[1], 1);                  //     each completing once
-        for (int s = 0; s < kStages; ++s) {
-            mbar_init(&ms.fullK[s], 1); mbar_init(&ms.emptyK[s], 1);
-            mbar_init(&ms.fullV[s], 1); mbar_init(&ms.emptyV[s], 1);
-        }
-        mbar_init(&ms.barS[0], 1);
-        mbar_init(&ms.barS[1], 1);
-        mbar_init(&ms.barP, kSoftmaxThreads);
-        mbar_init(&ms.barO, 1);
-        mbar_init(&ms.barE, 1);
-        ms.abort_flag = 0;
-        ms.wait_kcycles = wait_kcycles;
-        fence_mbar_init();
-    }
-    if (tid < kBM) {    // sm_idx lists this call's retained tokens; when the call appends to a
-        const int jj = n_full + tid - (appending ? pre[0] : 0);   // cache, pre[0] were there before
-        ms.pos[tid] = n_full + tid < n_end ? sm_idx[(size_t)bh * L + jj] : 0x7fffffff;
-    }
-    if (warp == 4) tmem_alloc(&ms.tmem_base, 256);
+    if (tid < kBM / 32) ms.kept[tid] = 0u;
+    if (tid < kBM) ms.m_row[tid] = -INFINITY;
+    if (warp == kMmaWarp) tmem_alloc(&ms.tmem_base, 256);
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = ms.tmem_base;
-    const uint32_t tS[2] = {tmem, tmem + 64}, tO = tmem + 128;
+    const uint32_t tO = tmem + 64 * kLogits;            // (128 columns: logits at 0, 64; 64 columns: at 0, 64, 128)
+    auto tS = [&](int t) { return tmem + 64 * (t % kLogits); };
     volatile int *abort_flag = &ms.abort_flag;
 
-    if (warp == 5) {
+    if (warp == kTmaWarp) {
         // ------------------------------ TMA producer ------------------------------
         if (lane == 0) {
             int nk = 0, nv = 0;                 // K / V tiles requested so far
             bool ok = true;
             if (T2 > 0) {                       // nothing is loaded for a tile that sees no key at all
-                prefetch_tmap(&map_q); prefetch_tmap(&map_k); prefetch_tmap(&map_v);
-                mbar_arrive_expect_tx(&ms.barQ, SL::kQBytes);
-                for (int kb = 0; kb < KB; ++kb)
-                    tma_load_4d(smem + SL::oQ + kb * kBM * 128, &map_q, &ms.barQ, kb * 64, hq, p * kBM, b);
                 // K and V tiles have their own rings: a K tile is free as soon as its Q K^T has run
                 // (early), a V tile only after its P V; K(u) is therefore requested before V(u-1).
                 for (int u = 0; u <= T2 && ok; ++u) {
@@ -200,6 +253,7 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                 // the Q tile and the K ring are free once the last Q K^T has run
                 if (ok) ok = mbar_wait(&ms.emptyK[(T2 - 1) % kStages], ((T2 - 1) / kStages) & 1, abort_flag);
             }
+            mbar_wait_drain(&ms.barQ, 0);       // (the Q tile's copy, read or not, before its place is reused)
             // beside the scan: the tile's chunks of o_la are complete once all row warps of the scan
             // CTA have raised the chunk's counter
             if (emit_flags) {
@@ -217,14 +271,13 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
             }
             // No copy may be in flight when the CTA retires, aborted or not: wait (with a bound of
             // their own) for the copies issued last.
-            if (T2 > 0) mbar_wait_drain(&ms.barQ, 0);
             for (int u = max(0, nk - kStages); u < nk; ++u)
                 mbar_wait_drain(&ms.fullK[u % kStages], (u / kStages) & 1);
             for (int u = max(0, nv - kStages); u < nv; ++u)
                 mbar_wait_drain(&ms.fullV[u % kStages], (u / kStages) & 1);
             if (e_issued) mbar_wait_drain(&ms.barE, 0);
         }
-    } else if (warp == 4) {
+    } else if (warp == kMmaWarp) {
         // ------------------------------ MMA issuer ------------------------------
         if (lane == 0 && T2 > 0) {
             // logits: q and k as given are bf16; normalised ones are fp16 (see the softmax threads)
@@ -237,346 +290,325 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                 for (int kb = 0; kb < KB; ++kb)
 #pragma unroll
                     for (int k16 = 0; k16 < 4; ++k16)
-                        mma_ss(tS[t & 1], desc_kmajor(aQ + kb * kBM * 128 + k16 * 32),
+                        mma_ss(tS(t), desc_kmajor(aQ + kb * kBM * 128 + k16 * 32),
                                desc_kmajor(aK + kb * kBN * 128 + k16 * 32), idesc_qk,
                                (kb | k16) != 0);
                 mma_commit(&ms.emptyK[t % kStages]);
-                mma_commit(&ms.barS[t & 1]);
+                mma_commit(&ms.barS[t % kLogits]);
             };
             // (normalisation with block-level routing: an own-block tile's keys arrive raw and are
             // normalised in place by the softmax threads first.  One single-phase barrier per own-block
             // tile, of which a CTA has at most two: with one barrier and a phase per tile, nothing kept the
             // softmax threads from completing the second phase before this thread had looked at the
-            // first -- a parity wait then never returns -- and a late enough start of this thread, as in
-            // the first wave of a launch, did let that happen.)
+            // first -- a parity wait then never returns.)
             auto own_keys_ready = [&](int t) {
                 return !(kBlock && kNorm) || t < T || mbar_wait(&ms.barKn[t - T], 0, abort_flag);
             };
-            bool ok = mbar_wait(&ms.barQ, 0, abort_flag) && (!kNorm || mbar_wait(&ms.barQn, 0, abort_flag)) &&
-                      mbar_wait(&ms.fullK[0], 0, abort_flag) && own_keys_ready(0);
-            if (ok) {
+            // logits of tile t, as soon as its keys are there (and its TMEM columns free: MMAs run in issue order)
+            auto next_qk = [&](int t) {
+                if (t >= T2) return true;
+                if (!mbar_wait(&ms.fullK[t % kStages], (t / kStages) & 1, abort_flag) || !own_keys_ready(t)) return false;
                 tc_fence_after_sync();
-                issue_qk(0);
-            }
+                issue_qk(t);
+                return true;
+            };
+            bool ok = mbar_wait(&ms.barQ, 0, abort_flag) && (!kNorm || mbar_wait(&ms.barQn, 0, abort_flag));
+            for (int t = 0; t < kAhead && ok; ++t) ok = next_qk(t);
             for (int t = 0; ok && t < T2; ++t) {
-                if (t + 1 < T2) {
-                    ok = mbar_wait(&ms.fullK[(t + 1) % kStages], ((t + 1) / kStages) & 1, abort_flag) &&
-                         own_keys_ready(t + 1);
-                    if (!ok) break;
-                    tc_fence_after_sync();
-                    issue_qk(t + 1);
-                }
-                ok = mbar_wait(&ms.barP, t & 1, abort_flag) &&
+                // (keys that the softmax threads still have to normalise must not hold up this tile's product)
+                const bool late = kBlock && kNorm && t + kAhead >= T;
+                if (!late) ok = next_qk(t + kAhead);
+                ok = ok && mbar_wait(&ms.barP[t % kLogits], (t / kLogits) & 1, abort_flag) &&
                      mbar_wait(&ms.fullV[t % kStages], (t / kStages) & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after_sync();
                 const uint32_t aV = smem_u32(smem + SL::oV + (t % kStages) * SL::kVStage);
 #pragma unroll
                 for (int k16 = 0; k16 < 4; ++k16)      // A = P(t): fp16 pairs in the first 32 columns of S(t)
-                    mma_ts(tO, tS[t & 1] + k16 * 8, desc_mnmajor(aV + k16 * 2048, kBN * 128),
+                    mma_ts(tO, tS(t) + k16 * 8, desc_mnmajor(aV + k16 * 2048, kBN * 128),
                            idesc_pv, (t | k16) != 0);
                 mma_commit(&ms.emptyV[t % kStages]);
-                mma_commit(&ms.barO);
+                mma_commit(&ms.barO[t & 1]);
+                if (late) ok = next_qk(t + kAhead);
             }
+            if (ok) mma_commit(&ms.barF);              // every product has run
         }
     } else {
         // ------------------------------ softmax + epilogue ------------------------------
-        const int r = tid;                              // query row inside the tile, TMEM lane
+        const int wg = warp >> 2, q = warp & 3;         // warpgroup; quarter of the rows
+        constexpr int kPq = 8 / kGroups;                // 16-byte pieces of a block of the query row per thread
+        const int tg = tid & (kGroupThreads - 1);
+        const int r = tg;                               // query row inside the tile, TMEM lane
         const int i_abs = p * kBM + r;
-        const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
+        const uint32_t lane_base = (uint32_t)(q * 32) << 16;
         const float sl2 = scale_sm * 1.4426950408889634f;
-        float m = -INFINITY, l = 0.f;
+        float m_mine = -INFINITY, l = 0.f;              // maximum this thread's sum is relative to; the sum
         bool ok = true;
+        // Which of the CTA's own tokens are retained (sm_idx lists this call's retained tokens; when the call
+        // appends to a cache, pre[0] were there before): the keys a row sees are then a population count.
+        if (wg == 0 && n_full + tg < n_end) {
+            const int rel = sm_idx[(size_t)bh * L + n_full + tg - (appending ? pre[0] : 0)] - p * kBM;
+            atomicOr(&ms.kept[(rel >> 5) & 3], 1u << (rel & 31));
+        }
         if (kNorm && T2 > 0) {
-            // RMS-normalised queries (Section 4.3): thread r rewrites row r of the Q tile (bf16, as loaded)
-            // as fp16 of the normalised row, over the D columns of its softmax head; the keys were
-            // normalised and stored as fp16 when they were gathered, so the logit product is an fp16
-            // MMA (bf16 keeps 8 bits: rounding the normalised keys to it alone costs 2.8e-2 of the
-            // branch output's RMS).  Eight 16-byte pieces per row and block, taken in an order that
-            // spreads the warp over the banks.
+            // RMS-normalised queries (Section 4.3): the threads of row r rewrite their pieces of its
+            // blocks (bf16, as loaded) as fp16 of the normalised row, over the D columns of its softmax head;
+            // the keys were normalised and stored as fp16 when they were gathered, so the logit product is
+            // an fp16 MMA (bf16 keeps 8 bits: rounding the normalised keys to it alone costs 2.8e-2 of the
+            // branch output's RMS).
             ok = mbar_wait(&ms.barQ, 0, abort_flag);
+            uint8_t *rowp = smem + SL::oQ + r * 128;
+            float ss = 0.f;
+            if (ok)
+#pragma unroll
+                for (int kb = 0; kb < KB; ++kb) ss += row_square_sum<kPq>(rowp + kb * kBM * 128, kPq * wg, r & 7);
+            if (kGroups > 1) {
+                ms.xch[wg][r].x = ss;
+                named_barrier_sync(1, kSoftmaxThreads);
+                ss = ms.xch[0][r].x + ms.xch[1][r].x;
+            }
             if (ok) {
-                uint8_t *rowp = smem + SL::oQ + tid * 128;
-                float ss = 0.f;
-#pragma unroll
-                for (int kb = 0; kb < KB; ++kb)
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        const uint4 a = *reinterpret_cast<const uint4 *>(rowp + kb * kBM * 128 + ((c ^ (tid & 7)) << 4));
-                        const uint32_t wd[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float lo = __uint_as_float(wd[e] << 16), hi = __uint_as_float(wd[e] & 0xffff0000u);
-                            ss = fmaf(lo, lo, fmaf(hi, hi, ss));
-                        }
-                    }
                 const float rq = rsqrtf(ss / D + norm_eps);
 #pragma unroll
-                for (int kb = 0; kb < KB; ++kb)
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        uint4 *pp = reinterpret_cast<uint4 *>(rowp + kb * kBM * 128 + ((c ^ (tid & 7)) << 4));
-                        const uint4 a = *pp;
-                        const uint32_t wd[4] = {a.x, a.y, a.z, a.w};
-                        uint32_t o[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            o[e] = pack_half2(__uint_as_float(wd[e] << 16) * rq, __uint_as_float(wd[e] & 0xffff0000u) * rq);
-                        *pp = make_uint4(o[0], o[1], o[2], o[3]);
-                    }
+                for (int kb = 0; kb < KB; ++kb) row_to_fp16<kPq>(rowp + kb * kBM * 128, kPq * wg, r & 7, rq);
                 fence_proxy_async_smem();
                 mbar_arrive(&ms.barQn);
             }
         }
         float2 wv = make_float2(0.5f, 0.5f);             // (w_nla, w_la) of this row
         if (w && i_abs < L) wv = __ldg(reinterpret_cast<const float2 *>(w + (((size_t)b * L + i_abs) * H + h) * 2));
+        named_barrier_sync(1, kSoftmaxThreads);
         // The compacted keys are in position order, so row i sees exactly the first `cnt` of them:
         // all n_full earlier ones plus those of the CTA's own chunks at positions <= i.
-        int cnt = n_full;
-        for (int kq = 0; kq < n_end - n_full; ++kq) cnt += ms.pos[kq] <= i_abs ? 1 : 0;
-        // Keys of own-block tile u (block-level routing with normalisation): raw bf16 rows from the layer's
-        // k; threads 0-63 rewrite one row each as fp16 of the RMS-normalised row.
-        auto normalise_own_keys = [&](int u) -> bool {
-            if (!mbar_wait(&ms.fullK[u % kStages], (u / kStages) & 1, abort_flag)) return false;
-            if (tid < kBN) {
-                uint8_t *rowp = smem + SL::oK + (u % kStages) * SL::kKStage + tid * 128;
-                float ss = 0.f;
+        int cnt = n_full + __popc(ms.kept[q] & ((2u << lane) - 1u));
 #pragma unroll
-                for (int kb = 0; kb < KB; ++kb)
+        for (int e = 0; e < kBM / 32 - 1; ++e) cnt += e < q ? __popc(ms.kept[e]) : 0;
+        for (int t = wg; ok && t < T2; t += kGroups) {
+            if (kBlock && kNorm && t >= T) {
+                // Keys of an own-block tile (block-level routing with normalisation): raw bf16 rows from the
+                // layer's k; two threads per row rewrite it as fp16 of the RMS-normalised row.  One arrival per
+                // tile, after all rows are written.
+                ok = mbar_wait(&ms.fullK[t % kStages], (t / kStages) & 1, abort_flag);
+                uint8_t *rowp = smem + SL::oK + (t % kStages) * SL::kKStage + (tg >> 1) * 128;
+                if (ok) {
+                    float ss = 0.f;
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        const uint4 a = *reinterpret_cast<const uint4 *>(rowp + kb * kBN * 128 + ((c ^ (tid & 7)) << 4));
-                        const uint32_t wd[4] = {a.x, a.y, a.z, a.w};
+                    for (int kb = 0; kb < KB; ++kb) ss += row_square_sum<4>(rowp + kb * kBN * 128, 4 * (tg & 1), (tg >> 1) & 7);
+                    ss += __shfl_xor_sync(0xffffffffu, ss, 1);
+                    const float rk = rsqrtf(ss / D + norm_eps);
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float lo = __uint_as_float(wd[e] << 16), hi = __uint_as_float(wd[e] & 0xffff0000u);
-                            ss = fmaf(lo, lo, fmaf(hi, hi, ss));
-                        }
-                    }
-                const float rk = rsqrtf(ss / D + norm_eps);
-#pragma unroll
-                for (int kb = 0; kb < KB; ++kb)
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        uint4 *pp = reinterpret_cast<uint4 *>(rowp + kb * kBN * 128 + ((c ^ (tid & 7)) << 4));
-                        const uint4 a = *pp;
-                        const uint32_t wd[4] = {a.x, a.y, a.z, a.w};
-                        uint32_t o[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            o[e] = pack_half2(__uint_as_float(wd[e] << 16) * rk, __uint_as_float(wd[e] & 0xffff0000u) * rk);
-                        *pp = make_uint4(o[0], o[1], o[2], o[3]);
-                    }
-            }
-            // One arrival per tile, after all rows are written.  (With one arrival per thread, the threads
-            // that have no row to write reached the next tile's arrival while the others were still
-            // writing this tile's rows, and completed this tile's phase for them.)
-            fence_proxy_async_smem();
-            named_barrier_sync(2, kSoftmaxThreads);
-            if (tid == 0) mbar_arrive(&ms.barKn[u - T]);
-            return true;
-        };
-        if (kBlock && kNorm && ok && T2 > 0 && T == 0) ok = normalise_own_keys(0);
-        for (int t = 0; ok && t < T2; ++t) {
-            if (kBlock && kNorm && t + 1 < T2 && t + 1 >= T) {      // (before this tile's logits are waited for)
-                ok = normalise_own_keys(t + 1);
+                    for (int kb = 0; kb < KB; ++kb) row_to_fp16<4>(rowp + kb * kBN * 128, 4 * (tg & 1), (tg >> 1) & 7, rk);
+                }
+                fence_proxy_async_smem();
+                named_barrier_sync(2 + wg, kGroupThreads);
+                if (tg == 0 && ok) mbar_arrive(&ms.barKn[t - T]);
                 if (!ok) break;
             }
-            ok = mbar_wait(&ms.barS[t & 1], (t >> 1) & 1, abort_flag);
+            ok = mbar_wait(&ms.barS[t % kLogits], (t / kLogits) & 1, abort_flag);
             if (!ok) break;
             tc_fence_after_sync();
-            uint32_t sv[2][32];
-            tmem_ld32(tS[t & 1] + lane_base, sv[0]);
-            tmem_ld32(tS[t & 1] + lane_base + 32, sv[1]);
+            float x[kBN];                                // raw logits: the scale goes into the exponent's FMA
+            tmem_ld32(tS(t) + lane_base, reinterpret_cast<uint32_t (&)[32]>(x[0]));
+            tmem_ld32(tS(t) + lane_base + 32, reinterpret_cast<uint32_t (&)[32]>(x[32]));
             tmem_wait_ld();
-            float x[kBN];
-#pragma unroll
-            for (int c = 0; c < kBN; ++c) x[c] = __uint_as_float(sv[c >> 5][c & 31]);   // raw logits: the scale
-                                                                                        // goes into the exponent's FMA
-            const int j0 = t * kBN;
-            if (kBlock && t >= T) {
-                // own-block tile: row r sees keys 0 .. r % 64 if it is in that block
-                const int vis = (r >> 6) == own_block(t) ? (r & 63) + 1 : 0;
+            // Keys of this tile the row sees: an own-block tile's 0 .. r % 64 if the row is in that block, else those
+            // of the compacted order before `cnt`.
+            const int vis = kBlock && t >= T ? ((r >> 6) == own_block(t) ? (r & 63) + 1 : 0) : cnt - t * kBN;
+            if (!__all_sync(0xffffffffu, vis >= kBN)) {   // some row of the warp is cut off here
 #pragma unroll
                 for (int c = 0; c < kBN; ++c) x[c] = c < vis ? x[c] : -INFINITY;
-            } else if (!__all_sync(0xffffffffu, j0 + kBN <= cnt)) {   // some row of the warp is cut off here
-#pragma unroll
-                for (int c = 0; c < kBN; ++c) x[c] = j0 + c < cnt ? x[c] : -INFINITY;
             }
-            float mx4[4] = {x[0], x[1], x[2], x[3]};      // four independent chains, not one of 63
+            float mx4[4] = {x[0], x[1], x[2], x[3]};      // four independent chains
 #pragma unroll
-            for (int c = 4; c < kBN; ++c) mx4[c & 3] = fmaxf(mx4[c & 3], x[c]);
+            for (int c = 4; c < kBN - 4; c += 8)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) mx4[e] = max3(mx4[e], x[c + e], x[c + 4 + e]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) mx4[e] = fmaxf(mx4[e], x[kBN - 4 + e]);
             // (scale_sm > 0, checked on the host: the maximum of the raw logits is the maximum logit)
             const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * sl2;
-            // The running maximum only has to bound the exponents, not equal the true maximum: it
-            // is raised (and O rescaled) only when a logit exceeds it by more than 8 (base 2), so
-            // probabilities stay below 2^8 and, for inputs whose logits vary little, the accumulator
-            // is never touched between the tiles.  lse = m + log2(l) holds for any such m.
-            const float m_new = (mx > m + 8.f || m == -INFINITY) ? fmaxf(m, mx) : m;
-            const float m_use = m_new == -INFINITY ? 0.f : m_new;
-            const float corr = exp2f(m - m_use);        // m = -inf -> 0; unchanged m -> 1
-            float ps4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int c = 0; c < kBN; ++c) {
-                x[c] = ex2_ftz(fmaf(x[c], sl2, -m_use));
-                ps4[c & 3] += x[c];
+            // The running maximum passes from tile to tile, i.e. between the warpgroups.  It only has to
+            // bound the exponents, not equal the true maximum: it is raised (and O rescaled) only when a logit
+            // exceeds it by more than 8 (base 2), so probabilities stay below 2^8 and, for inputs whose logits
+            // vary little, the accumulator is never touched between the tiles.  lse = m + log2(l) holds for
+            // any such m.
+            if (kGroups > 1 && t > 0) {
+                ok = mbar_wait(&ms.barM[(t - 1) & 1][q], ((t - 1) >> 1) & 1, abort_flag);
+                if (!ok) break;
             }
-            l = l * corr + ((ps4[0] + ps4[1]) + (ps4[2] + ps4[3]));
-            m = m_new;
-            // barO's phases are consumed strictly in order, one per tile (a parity wait cannot skip a
-            // phase): before the accumulator is touched when it has to be rescaled, otherwise at the
-            // end of the tile, when the previous tile's product has had the whole tile to finish.
-            bool waited_o = false;
-            if (t > 0 && __any_sync(0xffffffffu, corr != 1.f)) {
-                waited_o = true;
-                ok = mbar_wait(&ms.barO, (t - 1) & 1, abort_flag);
+            const float m_old = kGroups > 1 ? ms.m_row[r] : m_mine;
+            const float m_new = (mx > m_old + 8.f || m_old == -INFINITY) ? fmaxf(m_old, mx) : m_old;
+            if (kGroups > 1) {
+                ms.m_row[r] = m_new;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&ms.barM[t & 1][q]);
+            }
+            const float m_use = m_new == -INFINITY ? 0.f : m_new;
+            uint64_t ps[2] = {0ull, 0ull};
+            uint32_t pk[32];                            // P(t), over the logits this thread has consumed
+            const uint64_t sl22 = pack2(sl2, sl2), nm2 = pack2(-m_use, -m_use);
+#pragma unroll
+            for (int c = 0; c < kBN; c += 2) {
+                const float2 e = unpack2(fma2(pack2(x[c], x[c + 1]), sl22, nm2));
+                const float p0 = ex2_ftz(e.x), p1 = ex2_ftz(e.y);
+                ps[(c >> 1) & 1] = add2(ps[(c >> 1) & 1], pack2(p0, p1));
+                pk[c >> 1] = pack_half2(p0, p1);
+            }
+            const float2 psf = unpack2(add2(ps[0], ps[1]));
+            l = l * ex2_ftz(m_mine - m_use) + (psf.x + psf.y);   // (m = -inf: l is 0)
+            m_mine = m_new;
+            tmem_st32(tS(t) + lane_base, pk);
+            if (t > 0 && __any_sync(0xffffffffu, m_new != m_old)) {
+                // (the logits of tile t were issued behind the product of tile t - 3, so the phase of this barrier
+                // before tile t - 1's has completed and the parity is unambiguous)
+                ok = mbar_wait(&ms.barO[(t - 1) & 1], ((t - 1) >> 1) & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after_sync();
-                {
+                const float corr = ex2_ftz(m_old - m_use);   // m = -inf -> 0; unchanged m -> 1
+#pragma unroll 1
+                for (int cb = 0; cb < D / 32; ++cb) {
+                    uint32_t ov[32];
+                    tmem_ld32(tO + lane_base + cb * 32, ov);
+                    tmem_wait_ld();
 #pragma unroll
-                    for (int cb = 0; cb < D / 32; ++cb) {
-                        uint32_t ov[32];
-                        tmem_ld32(tO + lane_base + cb * 32, ov);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int c = 0; c < 32; ++c) ov[c] = __float_as_uint(__uint_as_float(ov[c]) * corr);
-                        tmem_st32(tO + lane_base + cb * 32, ov);
-                    }
-                    tmem_wait_st();
+                    for (int c = 0; c < 32; ++c) ov[c] = __float_as_uint(__uint_as_float(ov[c]) * corr);
+                    tmem_st32(tO + lane_base + cb * 32, ov);
                 }
             }
-            {
-                uint32_t pk[32];                        // P(t), over the logits this thread has consumed
-#pragma unroll
-                for (int c = 0; c < 32; ++c) pk[c] = pack_half2(x[2 * c], x[2 * c + 1]);
-                tmem_st32(tS[t & 1] + lane_base, pk);
-                tmem_wait_st();
-            }
+            tmem_wait_st();
             if (kBlock && t >= T) {   // own-block tile: its V rows arrived as bf16; fp16 in place (exact)
                 ok = mbar_wait(&ms.fullV[t % kStages], (t / kStages) & 1, abort_flag);
                 if (!ok) break;
                 uint4 *vt = reinterpret_cast<uint4 *>(smem + SL::oV + (t % kStages) * SL::kVStage);
-                for (int i = r; i < SL::kVStage / 16; i += kSoftmaxThreads) {
+                for (int i = tg; i < SL::kVStage / 16; i += kGroupThreads) {
                     const uint4 a = vt[i];
                     auto cv = [](uint32_t wd) {
                         return pack_half2(__uint_as_float(wd << 16), __uint_as_float(wd & 0xffff0000u));
                     };
                     vt[i] = make_uint4(cv(a.x), cv(a.y), cv(a.z), cv(a.w));
                 }
+                fence_proxy_async_smem();
             }
-            // (before the arrival below, not after it: once this thread has arrived, the MMA warp may
-            // complete the next phase of barO too, and a parity wait two phases behind never returns)
-            if (t > 0 && !waited_o) {
-                ok = mbar_wait(&ms.barO, (t - 1) & 1, abort_flag);
-                if (!ok) break;
-            }
-            fence_proxy_async_smem();
             tc_fence_before_sync();
-            mbar_arrive(&ms.barP);
+            mbar_arrive(&ms.barP[t % kLogits]);
         }
         if (ok && T2 > 0) {
-            ok = mbar_wait(&ms.barO, (T2 - 1) & 1, abort_flag);
+            ok = mbar_wait(&ms.barF, 0, abort_flag);
             tc_fence_after_sync();
         }
+        // ---- epilogue: each warpgroup takes its share of the softmax head's columns of every row ----
+        constexpr int HC = D / kGroups;
+        float m = m_mine;
+        if (kGroups > 1) {
+            ms.xch[wg][r] = make_float2(l, m_mine);
+            named_barrier_sync(1, kSoftmaxThreads);
+            m = ms.m_row[r];
+            const float2 a0 = ms.xch[0][r], a1 = ms.xch[1][r];
+            l = (a0.x > 0.f ? a0.x * ex2_ftz(a0.y - m) : 0.f) + (a1.x > 0.f ? a1.x * ex2_ftz(a1.y - m) : 0.f);
+        }
         if (ok) ok = mbar_wait(&ms.barE, 0, abort_flag);        // the tile's rows of o_la have landed
+        // o_laT tiles (fp16): chunk e of the CTA at oQ + e * D * 128; piece pc (tokens 8 pc ..) of
+        // head-dimension row `row` at 16-byte slot pc * D + (row ^ pc).
+        // out tile (bf16): box kb (columns 64 kb ..) at oV + kb * 16 KB, row r, piece j at j ^ (r & 7).
+        const float inv = l > 0.f ? 1.f / l : 0.f;       // l = 0 (no visible key): o_nla = 0
+        const int tok = r & 63, tp = tok >> 3;
+        const uint8_t *la_col = smem + SL::oQ + (r >> 6) * (DL * 128) + tp * (DL * 16) + (tok & 7) * 2;
+        // Two passes over the row's columns, 32 at a time (rolled: the kernel is large enough for its warps to wait
+        // for instructions): mean squares of both branches, then the output.
+        auto la_pair = [&](int row) {        // o_la of this query, head-dimension rows row, row + 1
+            const __half a0 = *reinterpret_cast<const __half *>(la_col + ((row ^ tp) << 4));
+            const __half a1 = *reinterpret_cast<const __half *>(la_col + (((row + 1) ^ tp) << 4));
+            return __half22float2(__halves2half2(a0, a1));
+        };
+        auto load_o = [&](int cb, uint32_t (&ov)[32]) {
+            if (T2 > 0) {
+                tmem_ld32(tO + lane_base + wg * HC + cb * 32, ov);
+                tmem_wait_ld();
+            } else {
+#pragma unroll
+                for (int e = 0; e < 32; ++e) ov[e] = 0u;
+            }
+        };
+        float ssn4[4] = {0.f, 0.f, 0.f, 0.f}, ssl4[4] = {0.f, 0.f, 0.f, 0.f};
         if (ok) {
-            // o_laT tiles (fp16): chunk e of the CTA at oQ + e * D * 128; piece p (tokens 8 p ..) of
-            // head-dimension row `row` at 16-byte slot p * D + (row ^ p).
-            // out tile (bf16): box kb (columns 64 kb ..) at oV + kb * 16 KB, row r, piece j at j ^ (r & 7).
-            const float inv = l > 0.f ? 1.f / l : 0.f;       // l = 0 (no visible key): o_nla = 0
-            float ssn4[4] = {0.f, 0.f, 0.f, 0.f}, ssl4[4] = {0.f, 0.f, 0.f, 0.f};
-            const int tok = r & 63, tp = tok >> 3;
-            const uint8_t *la_col = smem + SL::oQ + (r >> 6) * (DL * 128) + tp * (DL * 16) + (tok & 7) * 2;
             if (kG > 1) {        // the other softmax heads' columns of the linear row: mean square only
 #pragma unroll 4
-                for (int row = 0; row < DL; row += 2) {
-                    if (row / D == sg) continue;
-                    const float a0 = __half2float(*reinterpret_cast<const __half *>(la_col + ((row ^ tp) << 4)));
-                    const float a1 = __half2float(*reinterpret_cast<const __half *>(la_col + (((row + 1) ^ tp) << 4)));
-                    ssl4[(row >> 1) & 3] = fmaf(a0, a0, fmaf(a1, a1, ssl4[(row >> 1) & 3]));
+                for (int e = 0; e < (kG - 1) * HC; e += 2) {
+                    const int gg = e / HC;
+                    const float2 a = la_pair((gg < sg ? gg : gg + 1) * D + wg * HC + e % HC);
+                    ssl4[(e >> 1) & 3] = fmaf(a.x, a.x, fmaf(a.y, a.y, ssl4[(e >> 1) & 3]));
                 }
             }
-            // This query's column of o_la is read once, kept as fp16 pairs (D / 2 registers: the logits of
-            // the main loop are dead by now) and used twice: for its mean square and for the output.
-            uint32_t la2[D / 2];
-#pragma unroll
-            for (int cb = 0; cb < D / 32; ++cb) {
+#pragma unroll 1
+            for (int cb = 0; cb < HC / 32; ++cb) {
                 uint32_t ov[32];
-                if (T2 > 0) {
-                    tmem_ld32(tO + lane_base + cb * 32, ov);
-                    tmem_wait_ld();
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) ov[e] = 0u;
-                }
+                load_o(cb, ov);
 #pragma unroll
                 for (int e = 0; e < 32; e += 2) {
-                    const int row = sg * D + 32 * cb + e;
-                    const __half a0 = *reinterpret_cast<const __half *>(la_col + ((row ^ tp) << 4));
-                    const __half a1 = *reinterpret_cast<const __half *>(la_col + (((row + 1) ^ tp) << 4));
-                    const __half2 ap = __halves2half2(a0, a1);
-                    la2[(32 * cb + e) / 2] = *reinterpret_cast<const uint32_t *>(&ap);
-                    const float2 af = __half22float2(ap);
-                    ssl4[(e >> 1) & 3] = fmaf(af.x, af.x, fmaf(af.y, af.y, ssl4[(e >> 1) & 3]));
+                    const float2 a = la_pair(sg * D + wg * HC + 32 * cb + e);
+                    ssl4[(e >> 1) & 3] = fmaf(a.x, a.x, fmaf(a.y, a.y, ssl4[(e >> 1) & 3]));
                     const float o0 = __uint_as_float(ov[e]), o1 = __uint_as_float(ov[e + 1]);
                     ssn4[(e >> 1) & 3] = fmaf(o0, o0, fmaf(o1, o1, ssn4[(e >> 1) & 3]));
                 }
             }
+        }
+        float ssn = (ssn4[0] + ssn4[1]) + (ssn4[2] + ssn4[3]), ssl = (ssl4[0] + ssl4[1]) + (ssl4[2] + ssl4[3]);
+        if (kGroups > 1) {
+            ms.xch2[wg][r] = make_float2(ssn, ssl);
+            named_barrier_sync(1, kSoftmaxThreads);
+            ssn = ms.xch2[0][r].x + ms.xch2[1][r].x;
+            ssl = ms.xch2[0][r].y + ms.xch2[1][r].y;
+        }
+        if (ok) {
             // mean square of the normalised row = inv^2 * mean square of the accumulator row
-            const float msn = inv * inv * ((ssn4[0] + ssn4[1]) + (ssn4[2] + ssn4[3])) / D;
-            const float wn = wv.x * rsqrtf(msn + eps) * inv;          // applies to the raw accumulator
-            const float wl = wv.y * rsqrtf(((ssl4[0] + ssl4[1]) + (ssl4[2] + ssl4[3])) / DL + eps);
-            float *onla_row = o_nla && i_abs < L ? o_nla + (((size_t)b * L + i_abs) * H + h) * DL + sg * D : nullptr;
-#pragma unroll
-            for (int cb = 0; cb < D / 32; ++cb) {
+            const float wn = wv.x * rsqrtf(inv * inv * ssn / D + eps) * inv;          // applies to the raw accumulator
+            const float wl = wv.y * rsqrtf(ssl / DL + eps);
+            float *onla_row =
+                o_nla && i_abs < L ? o_nla + (((size_t)b * L + i_abs) * H + h) * DL + sg * D + wg * HC : nullptr;
+#pragma unroll 1
+            for (int cb = 0; cb < HC / 32; ++cb) {
                 uint32_t ov[32];
-                if (T2 > 0) {
-                    tmem_ld32(tO + lane_base + cb * 32, ov);
-                    tmem_wait_ld();
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) ov[e] = 0u;
-                }
+                load_o(cb, ov);
 #pragma unroll
                 for (int j2 = 0; j2 < 4; ++j2) {
                     float y[8];
 #pragma unroll
                     for (int e = 0; e < 8; e += 2) {
-                        const float2 af = __half22float2(*reinterpret_cast<const __half2 *>(&la2[(32 * cb + 8 * j2 + e) / 2]));
-                        y[e] = fmaf(wn, __uint_as_float(ov[8 * j2 + e]), wl * af.x);
-                        y[e + 1] = fmaf(wn, __uint_as_float(ov[8 * j2 + e + 1]), wl * af.y);
+                        const float2 a = la_pair(sg * D + wg * HC + 32 * cb + 8 * j2 + e);
+                        y[e] = fmaf(wn, __uint_as_float(ov[8 * j2 + e]), wl * a.x);
+                        y[e + 1] = fmaf(wn, __uint_as_float(ov[8 * j2 + e + 1]), wl * a.y);
                     }
+                    const int col = wg * HC + cb * 32 + j2 * 8;
                     if (has_out)
-                        *reinterpret_cast<uint4 *>(smem + SL::oV + (cb >> 1) * (kBM * 128) +
-                                                   sw128_offset(r, (cb & 1) * 4 + j2)) =
+                        *reinterpret_cast<uint4 *>(smem + SL::oV + (col >> 6) * (kBM * 128) + sw128_offset(r, (col & 63) >> 3)) =
                             make_uint4(pack_bf162(y[0], y[1]), pack_bf162(y[2], y[3]), pack_bf162(y[4], y[5]),
                                        pack_bf162(y[6], y[7]));
-                    if (onla_row) {         // the raw branch output (fp32), straight from the registers
-                        float4 *dst = reinterpret_cast<float4 *>(onla_row + cb * 32 + j2 * 8);
-                        dst[0] = make_float4(__uint_as_float(ov[8 * j2]) * inv, __uint_as_float(ov[8 * j2 + 1]) * inv,
-                                             __uint_as_float(ov[8 * j2 + 2]) * inv, __uint_as_float(ov[8 * j2 + 3]) * inv);
-                        dst[1] = make_float4(__uint_as_float(ov[8 * j2 + 4]) * inv, __uint_as_float(ov[8 * j2 + 5]) * inv,
-                                             __uint_as_float(ov[8 * j2 + 6]) * inv, __uint_as_float(ov[8 * j2 + 7]) * inv);
-                    }
+                }
+                if (onla_row) {         // the raw branch output (fp32), straight from the registers
+                    float4 *dst = reinterpret_cast<float4 *>(onla_row + cb * 32);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        dst[e] = make_float4(__uint_as_float(ov[4 * e]) * inv, __uint_as_float(ov[4 * e + 1]) * inv,
+                                             __uint_as_float(ov[4 * e + 2]) * inv, __uint_as_float(ov[4 * e + 3]) * inv);
                 }
             }
-            if (lse && i_abs < L)
+            if (lse && wg == 0 && i_abs < L)
                 lse[(size_t)bhg * L + i_abs] = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
-            fence_proxy_async_smem();
-            named_barrier_sync(1, kSoftmaxThreads);
-            if (tid == 0) {
-                if (has_out)
-                    for (int kb = 0; kb < KB; ++kb)
-                        tma_store_4d(&map_out, smem + SL::oV + kb * (kBM * 128), kb * 64, hq, p * kBM, b);
-                tma_store_commit();
-                tma_store_wait_read();                      // shared memory may go once it has been read
-            }
+        }
+        fence_proxy_async_smem();
+        named_barrier_sync(1, kSoftmaxThreads);
+        if (tid == 0 && ok) {
+            if (has_out)
+                for (int kb = 0; kb < KB; ++kb)
+                    tma_store_4d(&map_out, smem + SL::oV + kb * (kBM * 128), kb * 64, hq, p * kBM, b);
+            tma_store_commit();
+            tma_store_wait_read();                      // shared memory may go once it has been read
         }
     }
     // ------------------------------ teardown ------------------------------
     tc_fence_before_sync();
     __syncthreads();
-    if (warp == 4) {
+    if (warp == kMmaWarp) {
         tc_fence_after_sync();
         tmem_dealloc(tmem, 256);
     }
@@ -709,7 +741,7 @@ static cudaError_t softmax_tc_impl(const void *q, const void *k_sm, const void *
     // through the flags.  A launch the runtime serialises instead finds every flag already raised.
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(s.B * s.H * G, (s.L + kBM - 1) / kBM);
-    cfg.blockDim = dim3(kThreadsTc);
+    cfg.blockDim = dim3(SL::kThreads);
     cfg.dynamicSmemBytes = SL::kTotal;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];

@@ -79,12 +79,6 @@ bool use_tensor_cores(const natsl_params *p) {
     return p->dtype == NATSL_BF16 && !(p->flags & NATSL_FORCE_SIMT);
 }
 
-// Backward on tensor cores with d = 64: all chunk-level products in one fused kernel per chunk -- unless
-// q and k are normalised, which that kernel does not know; the separate products then serve d = 64 too.
-bool fused_chunk_path(const natsl_params *p) {
-    return use_tensor_cores(p) && p->d == 64 && !grouped_or_normed(p);
-}
-
 // Segments of the forward scan (tensor-core path): the largest power of two that keeps the two
 // runs per segment within ~one CTA per SM, divides the chunk count and leaves >= 8 chunks each.
 int scan_segments(const natsl_params *p) {
@@ -159,41 +153,47 @@ FwdWs carve_fwd(const natsl_params *p, void *ws) {
 struct BwdWs {
     int32_t *status, *emit_flags, *sm_idx, *prefix, *lin_idx, *n_lin, *sm_len;
     size_t head_bytes;                                       // status page + emit_flags: cleared per forward
+    float *o_la, *o_nla, *lse, *Dsm, *Gcum;                  // branch outputs, row sums, cumulative decays
+    float *dq_sm, *dk_sm, *dv_sm;                            // softmax branch: dq token-major, dk, dv compacted
+    float *dk_x, *dv_x, *dmask;                              // block-level routing: the softmax branch's dk, dv of every
+                                                             // token (token-major), mask gradients per retained key
+    // fp32 CUDA-core path
     float *k_sm32, *v_sm32;                                  // [B,H,L,d] compacted, fp32
     float *q32, *k32, *v32;                                  // token-major fp32 copies
-    float *qs32, *ks32;                                      // NATSL_QK_NORM, fp32 storage: RMS-normalised q, k
-                                                             // (q32, k32 then hold the L2-normalised ones)
-    float *W, *U, *Ut, *o_la, *o_nla, *do_la, *do_nla;       // token-major
-    float *dUt, *dQg, *dW, *dKt, *dKb, *dVb, *X1p, *X2, *X3, *X4, *dq_sm, *dk_sm, *dv_sm;
+    float *qs32, *ks32;                                      // NATSL_QK_NORM: RMS-normalised q, k (q32, k32 then hold the
+                                                             // L2-normalised ones)
+    float *W, *U, *Ut, *do_la, *do_nla;                      // token-major
+    float *dUt, *dQg, *dW, *dKt, *dKb, *dVb, *X1p, *X2, *X3, *X4;
     float *P, *Abar, *M, *N, *Mg, *Ms, *Ns;                  // [B,H,NC,64,64]
     float *S_c, *dS_c;                                       // [B,H,NC,d,d]
-    float *Gcum, *lse, *Dsm, *dGrow, *kappa, *gS;            // [B,H,L] (gS: [B,H,NC,d/32])
-    float *dk_x, *dv_x, *dmask;                              // block-level routing off the fused path: the
-                                                             // softmax branch's dk, dv of every token
-                                                             // (token-major), mask gradients per retained key [B,H,L]
-    void *k_smb, *k16, *v16, *Qh, *dO16;                     // tensor-core softmax branch: 16-bit [B,H,L,d]
-    void *dOla16, *dOlag16;                                  // tensor-core reverse scan: fp16 [B,H,L,d]
+    float *dGrow, *kappa, *gS;                               // [B,H,L] (gS: [B,H,NC,d/32])
+    // tensor-core path
+    void *k_smb, *k16, *v16, *Qh, *dO16;                     // softmax branch: 16-bit [B,H,L,d]
+    void *kn16;                                              // NATSL_QK_NORM with block-level routing: normalised k, likewise
     void *o_la16;                                            // linear read-out as fp16 [B,L,H,d]
-    GdnTcWs tc;                                              // tensor-core forward recomputation
-    float *Tinv;                                             // (I + A)^-1 per chunk [B,H,NC,64,64]
+    GdnTcWs tc;                                              // the forward's chunkwise intermediates
+    GdnTcExport ex;                                          // ... and what it keeps for the backward
+    GdnTcGrads gr;                                           // fp16 gradient operands of the linear branch
+    float *kap_c;                                            // [B,H,NC]
+    float *dq32, *dk32, *dv32;                               // NATSL_QK_NORM: gradients before the normalisations' backward
     size_t bytes;
 };
 
 // Only what the selected path uses is carved (a buffer the path does not touch gets no bytes and a
-// pointer nobody dereferences).  Paths: `fused` = tensor cores with d = 64 (reverse scan + one
-// fused kernel per chunk), tensor cores with d = 128 (chunk-level products as batched tile GEMMs),
-// fp32 CUDA cores.  Three pairs with disjoint lifetimes share their bytes on the tensor-core paths:
-// o_la (dead once the combination's backward has run) / dUt (written by the reverse scan after it),
-// o_nla / dq_sm likewise, and the fp16 o_la / the fp16 gradient copy dO16.
+// pointer nobody dereferences).  Buffers with disjoint lifetimes share their bytes on the tensor-core path:
+// o_nla (dead once the combination's backward has run) / dq_sm, o_la / dq32, and the fp16 o_la / the
+// fp16 gradient copy dO16.
 BwdWs carve_bwd(const natsl_params *p, void *ws) {
     Carver c(ws);
     BwdWs f;
     const size_t B = p->B, H = p->H, L = p->L, d = p->d, NC = L / kC;
     const size_t TM = B * L * H * d, CC = B * H * NC * kC * kC, ST = B * H * NC * d * d, BHL = B * H * L;
-    const bool tcs = use_tensor_cores(p), fused = fused_chunk_path(p), general = !fused;
-    const bool block = (p->flags & NATSL_BLOCK_ROUTING) != 0;
+    const bool tcs = use_tensor_cores(p), simt = !tcs;
+    const bool block = (p->flags & NATSL_BLOCK_ROUTING) != 0, normed = (p->flags & NATSL_QK_NORM) != 0;
+    const size_t Gg = p->G > 1 ? (size_t)p->G : 1;           // softmax heads per linear head: lse, Dsm per softmax head
     auto tm = [&](bool need) { return c.take<float>(need ? TM : 0); };
     auto cc = [&](bool need) { return c.take<float>(need ? CC : 0); };
+    auto half = [&](bool need, size_t n) { return static_cast<void *>(c.take<char>(need ? n * 2 : 0)); };
     f.status = c.take<int32_t>(kStatusBytes / 4);
     f.emit_flags = c.take<int32_t>(tcs ? B * H * NC : 0);    // per-chunk counters of the scan (forward part)
     f.head_bytes = c.off;
@@ -202,61 +202,47 @@ BwdWs carve_bwd(const natsl_params *p, void *ws) {
     f.lin_idx = c.take<int32_t>(BHL);
     f.n_lin = c.take<int32_t>(B * H * NC);
     f.sm_len = c.take<int32_t>(B * H);
-    f.k_sm32 = tm(!tcs); f.v_sm32 = tm(!tcs);
-    f.q32 = tm(general); f.k32 = tm(general); f.v32 = tm(general);
-    // (needed by the fp32 softmax kernels: all of them for fp32 storage, the own-block one of block-level routing)
-    const bool normed = (p->flags & NATSL_QK_NORM) && (!tcs || (general && block));
-    f.qs32 = tm(normed); f.ks32 = tm(normed);
-    const size_t Gg = p->G > 1 ? (size_t)p->G : 1;           // softmax heads per linear head: lse, Dsm per softmax head
-    f.W = tm(general); f.U = tm(general);
-    f.Ut = tm(true);
     f.o_la = tm(true);
     f.o_nla = tm(true);
-    f.do_la = tm(true);
-    f.do_nla = tm(!tcs);
-    f.dUt = tcs ? f.o_la : tm(true);
-    f.dQg = tm(general); f.dW = tm(general); f.dKt = tm(general); f.dKb = tm(general); f.dVb = tm(general);
-    // (the last four products' results: only the fp32 path stores them, the tensor-core path keeps them in
-    // the accumulators of its assembly kernel; X3, X4 also serve the fused chunk kernel's block-routed call
-    // as its side buffers)
-    f.X1p = tm(general && !tcs); f.X2 = tm(general && !tcs);
-    f.X3 = tm((general && !tcs) || (fused && block)); f.X4 = tm((general && !tcs) || (fused && block));
-    f.dq_sm = tcs ? f.o_nla : tm(true);
-    f.dk_sm = tm(true); f.dv_sm = tm(true);
-    f.P = cc(!tcs); f.Abar = cc(!tcs);
-    f.M = cc(general && !tcs); f.N = cc(general && !tcs);     // (tensor cores: M, N stay in gdn_tm_kernel's accumulators)
-    f.Mg = cc(general); f.Ms = cc(general); f.Ns = cc(general);
-    f.S_c = c.take<float>(ST);
-    f.dS_c = c.take<float>(ST);
-    f.Gcum = c.take<float>(BHL);
     f.lse = c.take<float>(BHL * Gg);
     f.Dsm = c.take<float>(BHL * Gg);
-    f.dGrow = c.take<float>(BHL);
-    f.kappa = c.take<float>(BHL);
-    f.gS = c.take<float>(general ? B * H * NC * (d / 32) : 0);
-    f.dk_x = tm(general && block); f.dv_x = tm(general && block);
-    f.dmask = c.take<float>(general && block ? BHL * Gg : 0);
-    const size_t h16 = tcs ? TM * 2 : 0;
-    f.k_smb = c.take<char>(h16);
-    f.k16 = c.take<char>(h16);
-    f.v16 = c.take<char>(h16);
-    f.Qh = c.take<char>(h16);
-    f.dO16 = c.take<char>(h16);
-    f.dOla16 = c.take<char>(h16);
-    f.dOlag16 = c.take<char>(h16);
+    f.Gcum = c.take<float>(BHL);
+    f.dq_sm = tcs ? f.o_nla : tm(true);
+    f.dk_sm = tm(true); f.dv_sm = tm(true);
+    f.dk_x = tm(block); f.dv_x = tm(block);
+    f.dmask = c.take<float>(block ? BHL * Gg : 0);
+    // fp32 CUDA-core path
+    f.k_sm32 = tm(simt); f.v_sm32 = tm(simt);
+    f.q32 = tm(simt); f.k32 = tm(simt); f.v32 = tm(simt);
+    f.qs32 = tm(simt && normed); f.ks32 = tm(simt && normed);
+    f.W = tm(simt); f.U = tm(simt); f.Ut = tm(simt); f.do_la = tm(simt); f.do_nla = tm(simt);
+    f.dUt = tm(simt); f.dQg = tm(simt); f.dW = tm(simt); f.dKt = tm(simt); f.dKb = tm(simt); f.dVb = tm(simt);
+    f.X1p = tm(simt); f.X2 = tm(simt); f.X3 = tm(simt); f.X4 = tm(simt);
+    f.P = cc(simt); f.Abar = cc(simt); f.M = cc(simt); f.N = cc(simt); f.Mg = cc(simt); f.Ms = cc(simt); f.Ns = cc(simt);
+    f.S_c = c.take<float>(simt ? ST : 0);
+    f.dS_c = c.take<float>(simt ? ST : 0);
+    f.dGrow = c.take<float>(simt ? BHL : 0);
+    f.kappa = c.take<float>(simt ? BHL : 0);
+    f.gS = c.take<float>(simt ? B * H * NC * (d / 32) : 0);
+    // tensor-core path
+    f.k_smb = half(tcs, TM); f.k16 = half(tcs, TM); f.v16 = half(tcs, TM); f.Qh = half(tcs, TM);
+    f.dO16 = half(tcs, TM);
+    f.kn16 = half(tcs && block && normed, TM);
     f.o_la16 = f.dO16;
+    f.gr.dO16 = half(tcs, TM); f.gr.dOg16 = half(tcs, TM); f.gr.dU16 = half(tcs, TM); f.gr.dS16 = half(tcs, ST);
     f.tc = GdnTcWs{};
-    if (tcs) {
-        f.tc.Qh = f.Qh;                       // the same fp16 copy of q serves both branches
-        f.tc.Kh = c.take<char>(h16);
-        f.tc.Wt = c.take<char>(h16);
-        f.tc.Ut = c.take<float>(TM);
-        f.tc.Ph = c.take<char>(CC * 2);
-        f.tc.Gd = c.take<float>(BHL * 2);
-        f.Tinv = c.take<float>(CC);
-    } else {
-        f.Tinv = nullptr;
-    }
+    f.tc.Qh = f.Qh;                           // without the normalisation the same fp16 copy of q serves both branches
+    f.tc.Kh = half(tcs, TM);
+    f.tc.Wt = half(tcs, TM);
+    f.tc.Ut = tm(tcs);
+    f.tc.Ph = half(tcs, CC);
+    f.tc.Gd = c.take<float>(tcs ? BHL * 2 : 0);
+    f.ex = GdnTcExport{};
+    f.ex.U16 = half(tcs, TM); f.ex.T16 = half(tcs, CC); f.ex.S16 = half(tcs, ST); f.ex.Ut16 = half(tcs, TM);
+    f.ex.Gcum = f.Gcum;
+    f.kap_c = c.take<float>(tcs && block ? B * H * NC : 0);
+    f.dq32 = f.o_la;
+    f.dk32 = tm(tcs && normed); f.dv32 = tm(tcs && normed);
     f.bytes = c.off;
     return f;
 }
@@ -329,7 +315,6 @@ static int bwd_forward_part(const void *q, const void *k, const void *v, const f
     const bool block = (p->flags & NATSL_BLOCK_ROUTING) != 0;
     const uint8_t *block_route = block ? route : nullptr;
     const bool tensor_cores = use_tensor_cores(p);
-    const bool fused_chunks = fused_chunk_path(p);          // chunk-level products in one kernel
     int32_t *flags = tensor_cores && !(p->flags & NATSL_SINGLE_STREAM) ? f.emit_flags : nullptr;
 #define NATSL_TRY(call) do { if ((call) != cudaSuccess) return NATSL_ERR_CUDA; } while (0)
     NATSL_TRY(cudaMemsetAsync(f.status, 0, f.head_bytes, st));
@@ -337,7 +322,7 @@ static int bwd_forward_part(const void *q, const void *k, const void *v, const f
     std::unique_lock<std::mutex> side_lock;
     SideStream *side = nullptr;
     SideJoin side_join;
-    if (fused_chunks && !(p->flags & NATSL_SINGLE_STREAM)) {
+    if (tensor_cores && !(p->flags & NATSL_SINGLE_STREAM)) {
         side_lock = std::unique_lock<std::mutex>(g_side_mu);
         side = side_stream_locked();
         if (!side) side_lock.unlock();
@@ -351,22 +336,19 @@ static int bwd_forward_part(const void *q, const void *k, const void *v, const f
     NATSL_TRY(launch_route_compact(route, f.sm_idx, f.prefix, f.lin_idx, f.n_lin, f.sm_len, nullptr,
                                    block ? f.status : nullptr, p->L, p->B, p->L, p->H, st0));
     const HeadGroups hg = head_groups(p);
-    if (!fused_chunks) {     // (with NATSL_QK_NORM the copies of q, k are the normalised ones, made below)
+    // fp32 storage: fp32 copies of the inputs; with NATSL_QK_NORM q32, k32 become the L2-normalised rows (everything
+    // of the linear branch reads those), qs32, ks32 the slice-wise RMS-normalised ones (softmax branch).  The
+    // tensor-core kernels normalise inside.
+    const float *qs = f.q32, *ks = f.k32;
+    if (!tensor_cores) {
         const bool qk = hg.norm_eps < 0.f;
         NATSL_TRY(launch_to_f32(qk ? q : nullptr, qk ? k : nullptr, v, f.q32, f.k32, f.v32,
                                 (size_t)(B * L * H * d), s.bf16, st));
-    }
-    // fp32 storage with NATSL_QK_NORM: q32, k32 become the L2-normalised rows (everything of the linear
-    // branch reads those), qs32, ks32 the slice-wise RMS-normalised ones (softmax branch)
-    // (tensor cores: the kernels normalise inside; only the fp32 copies the separate chunk-level products
-    // of the backward read are made here)
-    const float *qs = f.q32, *ks = f.k32;
-    if (hg.norm_eps >= 0.f) {
-        const bool rms_copies = !tensor_cores || block;
-        NATSL_TRY(launch_qk_norm_f32(q, k, s.bf16, f.q32, f.k32, rms_copies ? f.qs32 : nullptr,
-                                     rms_copies ? f.ks32 : nullptr, (size_t)(B * L * H), p->d, hg.G,
-                                     hg.norm_eps, st));
-        if (!tensor_cores) { qs = f.qs32; ks = f.ks32; }
+        if (!qk) {
+            NATSL_TRY(launch_qk_norm_f32(q, k, s.bf16, f.q32, f.k32, f.qs32, f.ks32, (size_t)(B * L * H), p->d, hg.G,
+                                         hg.norm_eps, st));
+            qs = f.qs32; ks = f.ks32;
+        }
     }
     if (tensor_cores)
         NATSL_TRY(launch_gather_kv_tc(k, v, f.sm_idx, f.prefix, f.k_smb, nullptr, f.v16, f.k16, p->L,
@@ -375,16 +357,13 @@ static int bwd_forward_part(const void *q, const void *k, const void *v, const f
         NATSL_TRY(launch_gather_kv(ks, f.v32, f.sm_idx, f.prefix, f.k_sm32, f.v_sm32, p->L,
                                    f.status, s32, st));
     if (tensor_cores) {
-        // the fused chunk kernel reads W^T, U^T as the forward keeps them: no fp32 copies for it
-        const GdnTcExport ex{fused_chunks ? nullptr : f.W, fused_chunks ? nullptr : f.U, nullptr, f.Tinv,
-                             f.Gcum, f.S_c, f.Ut};
-        NATSL_TRY(launch_gdn_prepare_tc(q, k, v, g, beta, block ? nullptr : route, p->scale_la, f.tc, ex,
+        NATSL_TRY(launch_gdn_prepare_tc(q, k, v, g, beta, block ? nullptr : route, p->scale_la, f.tc, f.ex,
                                         f.status, s, st, hg.norm_eps));
         // (the side stream joins before the scan, so that the softmax kernel follows the scan directly
         // and can run beside it as its programmatic dependent, as in natsl_hybrid_fwd)
         NATSL_TRY(side_join.join());
         NATSL_TRY(launch_gdn_scan_tc(f.tc, p->scale_la, p->state_in, state_out, ScanOut{f.o_la16, f.o_la, flags},
-                                     ex, ScanSegments{0, 1, 0, nullptr, nullptr, nullptr}, block_route,
+                                     f.ex, ScanSegments{0, 1, 0, nullptr, nullptr, nullptr}, block_route,
                                      f.status, s, st));
     } else {
         NATSL_TRY(launch_gdn_prepare_simt(f.q32, f.k32, f.v32, g, beta, block ? nullptr : route, p->scale_la,
@@ -662,8 +641,7 @@ int natsl_hybrid_bwd(const void *q, const void *k, const void *v, const float *g
     auto ST = [&](const float *x) { return BMat{x, H * NC * d * d, NC * d * d, d * d, (int)d}; };
     const int di = p->d;
     const uint8_t *block_route = block ? route : nullptr;
-    const bool tensor_cores = use_tensor_cores(p);
-    const bool fused_chunks = fused_chunk_path(p);          // chunk-level products in one kernel
+    const bool tensor_cores = use_tensor_cores(p), normed = hg.norm_eps >= 0.f;
 
     // ---- forward, keeping what the backward needs (unless the caller's forward already did) ----
     if (!(p->flags & NATSL_SAVED_FWD)) {
@@ -676,11 +654,7 @@ int natsl_hybrid_bwd(const void *q, const void *k, const void *v, const float *g
     std::unique_lock<std::mutex> side_lock;
     SideStream *side = nullptr;
     SideJoin side_join;
-    // (tensor cores with separate chunk-level kernels: the whole linear branch -- reverse scan, the products
-    // with the states, the middle of the chain -- runs on the side stream beside the softmax branch's
-    // backward, and the two meet at the assembly)
-    const bool side_general = tensor_cores && !fused_chunks;
-    if ((fused_chunks || side_general) && !(p->flags & NATSL_SINGLE_STREAM)) {
+    if (tensor_cores && !(p->flags & NATSL_SINGLE_STREAM)) {
         side_lock = std::unique_lock<std::mutex>(g_side_mu);
         side = side_stream_locked();
         if (!side) side_lock.unlock();
@@ -691,149 +665,107 @@ int natsl_hybrid_bwd(const void *q, const void *k, const void *v, const float *g
     // so that a loss-scaled or a tiny dout stays inside fp16's range (grad_scale, common.cuh).
     if (tensor_cores) NATSL_TRY(launch_dout_amax(dout, (size_t)(B * L * H * d), s.bf16, f.status, st));
     const int32_t *gsc = tensor_cores ? f.status : nullptr;
-    const bool general_block = block && !fused_chunks;   // block-level routing with separate chunk-level products
-    NATSL_TRY(launch_combine_bwd(f.o_la, f.o_nla, dout, p->w, p->eps, f.do_la,
+    NATSL_TRY(launch_combine_bwd(f.o_la, f.o_nla, dout, p->w, p->eps, tensor_cores ? nullptr : f.do_la,
                                  tensor_cores ? nullptr : f.do_nla, dw, f.Dsm,
-                                 tensor_cores ? f.dO16 : nullptr, tensor_cores ? f.dOla16 : nullptr,
-                                 tensor_cores ? f.dOlag16 : nullptr, f.tc.Gd, p->scale_la, gsc, s, st, hg.G));
-    // Dependencies from here on: the query-side softmax kernel, the key-side one and the reverse
-    // scan need only what is already there; the chunk kernel needs the first and the third; the
-    // scatter of the retained tokens' dk, dv needs the second.  With token-level routing the chunk
-    // kernel therefore does not wait for the key-side kernel: side stream = reverse scan, key-side
-    // kernel, scatter; caller's stream = query-side kernel, chunk kernel.  (Block-level routing:
-    // the chunk kernel adds the scattered gradients and so waits for the side stream, but the
-    // own-block kernel, which needs the query-side kernel only, still runs beside the key-side one.)
-    const bool kv_aside = side != nullptr && fused_chunks;
-    if (side) {
-        NATSL_TRY(cudaEventRecord(side->fork, st));
-        NATSL_TRY(cudaStreamWaitEvent(st0, side->fork, 0));
-        side_join.forked(side, st);
-    }
-    // ---- linear branch: reverse scan (then chunk-parallel products) ----
-    if (tensor_cores)
-        NATSL_TRY(launch_gdn_rscan_tc(f.dOla16, f.dOlag16, f.tc, f.S_c, f.dUt, f.dS_c,
-                                      fused_chunks ? nullptr : f.gS, p->dstate_out, p->dstate_in,
-                                      block_route, f.status, s, st0));
-    if (side && fused_chunks) NATSL_TRY(cudaEventRecord(side->join, st0));
-    if (tensor_cores)   // (d = 64: the prepare kernel has left the fp16 copy of q in f.Qh, and the reverse
-                        //  scan on the side stream reads it, so it is not written again)
-        // (separate chunk-level kernels: the softmax branch writes its own fp16 copy of q -- raw, or RMS-
-        //  normalised -- while the reverse scan beside it reads the linear operation's copy in f.Qh; the copy
-        //  goes where the forward's softmax kernel had its gathered keys, which nothing reads any more)
-        NATSL_TRY(launch_softmax_bwd_tc(q, fused_chunks ? f.Qh : f.k_smb, f.dO16, f.k16, f.v16, p->L, f.sm_idx, f.prefix, f.lse,
-                                        f.Dsm, p->scale_sm, f.dq_sm, f.dk_sm, f.dv_sm,
-                                        p->dscore ? (general_block ? f.dmask : f.dGrow) : nullptr, fused_chunks,
-                                        f.status, s, st, kv_aside ? st0 : st, hg));
-    else
-        NATSL_TRY(launch_softmax_bwd(hg.norm_eps >= 0.f ? f.qs32 : f.q32, f.k_sm32, f.v_sm32, p->L, f.sm_idx,
-                                     f.prefix, f.do_nla, f.lse, f.Dsm, p->scale_sm, f.dq_sm, f.dk_sm, f.dv_sm,
-                                     s, st, p->dscore ? f.dmask : nullptr, hg.G));
-    if (!tensor_cores)
-        NATSL_TRY(launch_gdn_rscan(f.q32, f.k32, f.Gcum, f.W, f.P, f.do_la, f.S_c, p->scale_la, f.dUt,
-                                   f.dS_c, f.gS, p->dstate_out, p->dstate_in, s, st, block_route));
-    if (side && fused_chunks) NATSL_TRY(cudaStreamWaitEvent(st, side->join, 0));     // the reverse scan has finished
-    // (with the normalisation the two operations' dq stay apart until its backward at the very end)
-    const bool normed = hg.norm_eps >= 0.f;
-    AssembleArgs a{f.q32, f.k32, f.v32, f.Gcum, beta, general_block ? nullptr : route, f.dQg, f.dKb, f.dVb, f.dKt, f.X1p, f.X2,
+                                 tensor_cores ? f.dO16 : nullptr, tensor_cores ? f.gr.dO16 : nullptr,
+                                 tensor_cores ? f.gr.dOg16 : nullptr, f.tc.Gd, p->scale_la, gsc, s, st, hg.G));
+    AssembleArgs a{f.q32, f.k32, f.v32, f.Gcum, beta, block ? nullptr : route, f.dQg, f.dKb, f.dVb, f.dKt, f.X1p, f.X2,
                    f.X3, f.X4, normed ? nullptr : f.dq_sm, f.dk_sm, f.dv_sm, f.gS, f.sm_idx, f.prefix, p->L,
                    p->scale_la, f.dGrow, f.kappa, dbeta, dg};
-    if (fused_chunks && block) {
-        // Every token has a softmax-branch dk, dv here: the retained tokens' from the compacted
-        // gradients, the tokens of linear blocks' from their own block.  Both go to fp32
-        // token-major buffers (each token is written by exactly one of the two), which the chunk
-        // kernel adds to its own dk, dv.
-        float *dk_x = f.X3, *dv_x = f.X4;
-        NATSL_TRY(launch_gdn_finish(a, dk_x, dv_x, s32, kv_aside ? st0 : st, false));
-        NATSL_TRY(launch_softmax_bwd_own_block(q, k, v, f.dO16, f.lse, f.Dsm, route, p->scale_sm,
-                                               f.dq_sm, dk_x, dv_x, gsc, s, st));
-        NATSL_TRY(side_join.join());      // the side stream's last kernels
-        NATSL_TRY(launch_gdn_bwd_chunk(q, k, v, f.do_la, f.dUt, f.Ut, f.S_c, f.dS_c, f.Tinv, f.tc.Wt, f.tc.Ut,
-                                       f.Gcum, beta, route, f.dq_sm, p->scale_la, dq, dk, dv, dg, dbeta,
-                                       true, dk_x, dv_x, p->dscore ? f.kappa : nullptr, s, st));
-        if (p->dscore)   // (dGrow, kappa: [B,H,L] scratch the fused path does not otherwise use)
-            NATSL_TRY(launch_dscore(route, f.prefix, f.dGrow, f.kappa, nullptr, p->L, p->dscore, s, st));
+    if (tensor_cores) {
+        // Dependencies from here on: the query-side softmax kernel, the key-side one and the reverse scan need only
+        // what is already there; the chunk kernel needs the reverse scan and, unless q and k are normalised, the
+        // query-side kernel's dq; the scatter of the retained tokens' dk, dv needs the key-side kernel.  Side
+        // stream: reverse scan, key-side kernel, scatter; caller's stream: query-side kernel, chunk kernel.
+        // Block-level routing: every token has a softmax-branch dk, dv (retained tokens: scattered from the
+        // compacted gradients; linear blocks: their own block's kernel, which needs the query-side one only), both
+        // in fp32 token-major buffers that the chunk kernel adds and so waits for.
+        // With the normalisation the gradients with respect to the two operations' normalised rows stay apart
+        // until its backward, a last kernel that rounds once.
+        if (side) {
+            NATSL_TRY(cudaEventRecord(side->fork, st));
+            NATSL_TRY(cudaStreamWaitEvent(st0, side->fork, 0));
+            side_join.forked(side, st);
+        }
+        NATSL_TRY(launch_gdn_rscan_tc(f.tc, f.gr, p->dstate_out, p->dstate_in, block_route, f.status, s, st0));
+        if (side) NATSL_TRY(cudaEventRecord(side->join, st0));
+        // (normalised: the softmax branch's own fp16 copy of q goes where the forward had its gathered keys, which
+        // nothing reads any more; the reverse scan beside it reads the linear operation's copy)
+        void *q16 = normed ? f.k_smb : f.Qh;
+        NATSL_TRY(launch_softmax_bwd_tc(q, q16, f.dO16, f.k16, f.v16, p->L, f.sm_idx, f.prefix, f.lse, f.Dsm,
+                                        p->scale_sm, f.dq_sm, f.dk_sm, f.dv_sm, p->dscore ? f.dmask : nullptr, !normed,
+                                        f.status, s, st, st0, hg));
+        if (side) NATSL_TRY(cudaStreamWaitEvent(st, side->join, 0));     // the reverse scan has finished
+        void *dq_o = normed ? f.dq32 : dq, *dk_o = normed ? f.dk32 : dk, *dv_o = normed ? f.dv32 : dv;
+        const float *dq_add = normed ? nullptr : f.dq_sm;
+        if (block) {
+            NATSL_TRY(launch_gdn_finish(a, f.dk_x, f.dv_x, s32, st0, false));
+            if (normed) NATSL_TRY(launch_to_f16_bhld(k, f.kn16, s, hg, st));
+            NATSL_TRY(launch_softmax_bwd_own_block(q, k, v, f.dO16, f.lse, f.Dsm, route, p->scale_sm, f.dq_sm, f.dk_x,
+                                                   f.dv_x, gsc, s, st, hg.G, normed ? q16 : nullptr,
+                                                   normed ? f.kn16 : nullptr));
+            NATSL_TRY(side_join.join());      // the side stream's last kernels
+            NATSL_TRY(launch_gdn_chunk_bwd(f.tc, f.ex, f.gr, v, beta, route, dq_add, p->scale_la, dq_o, dk_o, dv_o, normed,
+                                           dg, dbeta, true, normed ? nullptr : f.dk_x, f.dv_x,
+                                           p->dscore ? f.kap_c : nullptr, f.status, s, st));
+            if (p->dscore)
+                NATSL_TRY(launch_dscore(route, f.prefix, f.dmask, f.kap_c, nullptr, p->L, p->dscore, s, st, hg.G));
+        } else {
+            NATSL_TRY(launch_gdn_chunk_bwd(f.tc, f.ex, f.gr, v, beta, route, dq_add, p->scale_la, dq_o, dk_o, dv_o, normed,
+                                           dg, dbeta, false, nullptr, nullptr, nullptr, f.status, s, st));
+            // the retained tokens' dk, dv (rows the chunk kernel does not write)
+            NATSL_TRY(launch_gdn_finish(a, dk_o, dv_o, normed ? s32 : s, st0, false));
+            NATSL_TRY(side_join.join());
+        }
+        if (normed)
+            NATSL_TRY(launch_qk_norm_bwd_f32(q, k, true, route, f.dq32, f.dq_sm, f.dk32, f.dv32, dq, dk, dv,
+                                             (size_t)(B * L * H), p->d, hg.G, hg.norm_eps, st,
+                                             block ? f.dk_x : nullptr));
         return NATSL_OK;
     }
-    if (fused_chunks) {   // all chunk-level products and the assembly in one kernel per chunk
-        NATSL_TRY(launch_gdn_bwd_chunk(q, k, v, f.do_la, f.dUt, f.Ut, f.S_c, f.dS_c, f.Tinv, f.tc.Wt, f.tc.Ut,
-                                       f.Gcum, beta, route, f.dq_sm, p->scale_la, dq, dk, dv, dg, dbeta,
-                                       false, nullptr, nullptr, nullptr, s, st));
-        // scatter of the retained tokens' dk, dv (rows the chunk kernel does not write)
-        NATSL_TRY(launch_gdn_finish(a, dk, dv, s, kv_aside ? st0 : st, false));
-        NATSL_TRY(side_join.join());      // the side stream's last kernels
-        return NATSL_OK;
-    }
-    // (the tile GEMMs run on tf32 tensor cores for bf16 storage -- unless the caller asked for fp32
-    // arithmetic -- and as fp32 FMAs otherwise: launch_bgemm goes by the storage type it is told)
-    const Shape sgemm = tensor_cores ? s : s32;
+    // ---- fp32 CUDA-core path: softmax branch, reverse scan, chunk-level products as tile GEMMs, assembly ----
+    NATSL_TRY(launch_softmax_bwd(normed ? f.qs32 : f.q32, f.k_sm32, f.v_sm32, p->L, f.sm_idx, f.prefix, f.do_nla, f.lse,
+                                 f.Dsm, p->scale_sm, f.dq_sm, f.dk_sm, f.dv_sm, s, st, p->dscore ? f.dmask : nullptr,
+                                 hg.G));
+    NATSL_TRY(launch_gdn_rscan(f.q32, f.k32, f.Gcum, f.W, f.P, f.do_la, f.S_c, p->scale_la, f.dUt, f.dS_c, f.gS,
+                               p->dstate_out, p->dstate_in, s, st, block_route));
     // (block-level routing: beta~ = beta for every token, so the kernels below get no route)
-    const uint8_t *route_bt = general_block ? nullptr : route;
-    if (general_block) {
+    const uint8_t *route_bt = block ? nullptr : route;
+    if (block) {
         // Every token has a softmax-branch dk, dv: the retained tokens' from the compacted gradients, the
         // tokens of linear blocks' from their own block (each token is written by exactly one of the
-        // two); the assembly adds them to the linear branch's.
-        // (With the normalisation the own-block kernel reads the softmax operation's copies of q and k, and
-        // dk_x -- a gradient with respect to that copy -- stays apart from the linear branch's dk until the
-        // normalisations' backward.)
+        // two); the assembly adds them to the linear branch's -- with the normalisation dk_x, a gradient with
+        // respect to the softmax operation's copy, stays apart until its backward.
         NATSL_TRY(launch_gdn_finish(a, f.dk_x, f.dv_x, s32, st, false));
-        if (tensor_cores)      // softmax heads of 64 or 128 columns: warp-level tensor cores
-            NATSL_TRY(launch_softmax_bwd_own_block(q, k, v, f.dO16, f.lse, f.Dsm, route, p->scale_sm, f.dq_sm,
-                                                   f.dk_x, f.dv_x, gsc, s, st, hg.G, normed ? f.qs32 : nullptr,
-                                                   normed ? f.ks32 : nullptr));
-        else
-            NATSL_TRY(launch_softmax_bwd_own_block_simt(normed ? f.qs32 : f.q32, normed ? f.ks32 : f.k32, f.v32,
-                                                        f.do_nla, f.lse, f.Dsm, route, p->scale_sm, f.dq_sm, f.dk_x,
-                                                        f.dv_x, gsc, s32, st, hg.G));
+        NATSL_TRY(launch_softmax_bwd_own_block_simt(normed ? f.qs32 : f.q32, normed ? f.ks32 : f.k32, f.v32, f.do_nla, f.lse,
+                                                    f.Dsm, route, p->scale_sm, f.dq_sm, f.dk_x, f.dv_x, gsc, s32, st,
+                                                    hg.G));
         a.dk_x = normed ? nullptr : f.dk_x;
         a.dv_x = f.dv_x;
         a.no_scatter = true;
     }
-    cudaStream_t stl = side ? st0 : st;     // the linear branch's stream (behind the reverse scan)
-    NATSL_TRY(launch_bgemm(false, true, 0, TM(f.do_la), ST(f.S_c), TM(f.dQg), kC, di, di, 1.f, false, sgemm, stl));
-    NATSL_TRY(launch_bgemm(false, true, 0, TM(f.dUt), ST(f.S_c), TM(f.dW), kC, di, di, -1.f, false, sgemm, stl));
-    NATSL_TRY(launch_bgemm(false, true, 0, TM(f.Ut), ST(f.dS_c), TM(f.dKt), kC, di, di, 1.f, false, sgemm, stl));
-    if (tensor_cores) {   // [dKb | dVb] = (I + A)^-T [dW | dU~] with the inverse the forward already formed, M, N and
-                          // their masked, scaled forms: one kernel per chunk
-        NATSL_TRY(launch_gdn_tm(f.Tinv, f.dW, f.dUt, f.W, f.U, f.do_la, f.Ut, f.Gcum, beta, route_bt, p->scale_la,
-                                f.dKb, f.dVb, f.Mg, f.Ms, f.Ns, s, stl));
-        NATSL_TRY(side_join.join());      // the two branches meet at the assembly
-    } else {
-        NATSL_TRY(launch_bgemm(false, true, 1, TM(f.do_la), TM(f.Ut), CC(f.N), kC, kC, di, 1.f, false, sgemm, st));
-        NATSL_TRY(launch_gdn_tsolve(f.Abar, beta, route_bt, f.dW, f.dUt, f.dKb, f.dVb, s, st));
-        NATSL_TRY(launch_bgemm(false, true, 2, TM(f.dKb), TM(f.W), CC(f.M), kC, kC, di, -1.f, false, sgemm, st));
-        NATSL_TRY(launch_bgemm(false, true, 2, TM(f.dVb), TM(f.U), CC(f.M), kC, kC, di, -1.f, true, sgemm, st));
-        NATSL_TRY(launch_mask_scale(f.M, f.N, f.Gcum, beta, route_bt, p->scale_la, f.Mg, f.Ms, f.Ns, s, st));
-    }
-    // The last four products (X1 = Mg K, X2 = Ms^T K, X3 = Ns K, X4 = Ns^T Q) and the assembly: on tensor
-    // cores one kernel per chunk that keeps the products in its accumulators; otherwise four tile GEMMs
-    // and the row-local assembly.
-    auto assemble = [&](void *dq_o, void *dk_o, void *dv_o, Shape so) -> cudaError_t {
-        if (tensor_cores) return launch_gdn_xassemble(a, f.Mg, f.Ms, f.Ns, dq_o, dk_o, dv_o, so, st);
-        cudaError_t e;
-        if ((e = launch_bgemm(false, false, 0, CC(f.Mg), TM(f.k32), TM(f.X1p), kC, di, kC, 1.f, false, sgemm, st)) != cudaSuccess) return e;
-        if ((e = launch_bgemm(true, false, 0, CC(f.Ms), TM(f.k32), TM(f.X2), kC, di, kC, 1.f, false, sgemm, st)) != cudaSuccess) return e;
-        if ((e = launch_bgemm(false, false, 0, CC(f.Ns), TM(f.k32), TM(f.X3), kC, di, kC, 1.f, false, sgemm, st)) != cudaSuccess) return e;
-        if ((e = launch_bgemm(true, false, 0, CC(f.Ns), TM(f.q32), TM(f.X4), kC, di, kC, 1.f, false, sgemm, st)) != cudaSuccess) return e;
-        return launch_gdn_assemble(a, dq_o, dk_o, dv_o, so, st);
+    auto gemm = [&](bool ta, bool tb, int mask, BMat x, BMat y, BMat z, int m, int n, int k_, float alpha, bool acc) {
+        return launch_bgemm(ta, tb, mask, x, y, z, m, n, k_, alpha, acc, s32, st);
     };
-    // With the normalisation the assembly's dq, dk are gradients with respect to the normalised rows; a
-    // last kernel applies the two row-local Jacobians.  fp32 storage: in place.  bf16 storage: the
-    // assembly writes fp32 (into buffers the chunk-level products are done with) and the last kernel
-    // rounds once.
-    if (!normed) {
-        NATSL_TRY(assemble(dq, dk, dv, s));
-    } else if (!s.bf16) {
-        NATSL_TRY(assemble(dq, dk, dv, s));
+    NATSL_TRY(gemm(false, true, 0, TM(f.do_la), ST(f.S_c), TM(f.dQg), kC, di, di, 1.f, false));
+    NATSL_TRY(gemm(false, true, 0, TM(f.dUt), ST(f.S_c), TM(f.dW), kC, di, di, -1.f, false));
+    NATSL_TRY(gemm(false, true, 0, TM(f.Ut), ST(f.dS_c), TM(f.dKt), kC, di, di, 1.f, false));
+    NATSL_TRY(gemm(false, true, 1, TM(f.do_la), TM(f.Ut), CC(f.N), kC, kC, di, 1.f, false));
+    NATSL_TRY(launch_gdn_tsolve(f.Abar, beta, route_bt, f.dW, f.dUt, f.dKb, f.dVb, s, st));
+    NATSL_TRY(gemm(false, true, 2, TM(f.dKb), TM(f.W), CC(f.M), kC, kC, di, -1.f, false));
+    NATSL_TRY(gemm(false, true, 2, TM(f.dVb), TM(f.U), CC(f.M), kC, kC, di, -1.f, true));
+    NATSL_TRY(launch_mask_scale(f.M, f.N, f.Gcum, beta, route_bt, p->scale_la, f.Mg, f.Ms, f.Ns, s, st));
+    NATSL_TRY(gemm(false, false, 0, CC(f.Mg), TM(f.k32), TM(f.X1p), kC, di, kC, 1.f, false));
+    NATSL_TRY(gemm(true, false, 0, CC(f.Ms), TM(f.k32), TM(f.X2), kC, di, kC, 1.f, false));
+    NATSL_TRY(gemm(false, false, 0, CC(f.Ns), TM(f.k32), TM(f.X3), kC, di, kC, 1.f, false));
+    NATSL_TRY(gemm(true, false, 0, CC(f.Ns), TM(f.q32), TM(f.X4), kC, di, kC, 1.f, false));
+    NATSL_TRY(launch_gdn_assemble(a, dq, dk, dv, s, st));
+    // With the normalisation (fp32 storage) the assembly's dq, dk are gradients with respect to the normalised
+    // rows; a last kernel applies the two row-local Jacobians in place.
+    if (normed)
         NATSL_TRY(launch_qk_norm_bwd_f32(q, k, false, route, (const float *)dq, f.dq_sm, (const float *)dk, nullptr,
                                          dq, dk, nullptr, (size_t)(B * L * H), p->d, hg.G, hg.norm_eps, st,
-                                         general_block ? f.dk_x : nullptr));
-    } else {
-        float *dq32 = f.dW, *dk32 = f.W, *dv32 = f.U;
-        NATSL_TRY(assemble(dq32, dk32, dv32, s32));
-        NATSL_TRY(launch_qk_norm_bwd_f32(q, k, true, route, dq32, f.dq_sm, dk32, dv32, dq, dk, dv,
-                                         (size_t)(B * L * H), p->d, hg.G, hg.norm_eps, st,
-                                         general_block ? f.dk_x : nullptr));
-    }
+                                         block ? f.dk_x : nullptr));
     if (p->dscore)   // softmax blocks: the mask gradients of their keys; linear blocks: the kappa of their tokens
         NATSL_TRY(launch_dscore(route, f.prefix, f.dmask, nullptr, f.kappa, p->L, p->dscore, s, st, hg.G));
 #undef NATSL_TRY

@@ -33,26 +33,9 @@ namespace {
 constexpr int kThreads = 256;
 
 // ------------------------------------------------------------------------------------------
-// generic batched GEMM: C = alpha * op(A) op(B) (+ C), 64x64 output tiles, fp32.
-// fp32 storage (1e-4 tolerance): fp32 FMAs (bgemm_kernel).  bf16 storage, whose tolerance it fits:
-// the warp-level tensor-core path with tf32 operands (fp32 range, 11 significant bits) and fp32
-// accumulation (bgemm_tf32_kernel, below) -- warp w owns rows 16 (w & 3) .. and columns 32 (w >> 2) ..
-// of the tile, four m16n8k8 products per 8 values of k.
+// generic batched GEMM: C = alpha * op(A) op(B) (+ C), 64x64 output tiles, fp32 FMAs (fp32 storage; with bf16 storage
+// only when fp32 arithmetic is asked for).
 // ------------------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t to_tf32(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return r;
-}
-__device__ __forceinline__ void mma_tf32_16x8x8(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
-    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-__device__ __forceinline__ void store2(float *p, float a, float b) { *reinterpret_cast<float2 *>(p) = make_float2(a, b); }
-__device__ __forceinline__ void store2(__nv_bfloat16 *p, float a, float b) {
-    *reinterpret_cast<__nv_bfloat162 *>(p) = __floats2bfloat162_rn(a, b);
-}
 __device__ __forceinline__ const float *mat_base(const BMat &m, int b, int h, int ch) {
     return m.p + (size_t)b * m.sb + (size_t)h * m.sh + (size_t)ch * m.sc;
 }
@@ -125,103 +108,6 @@ bgemm_kernel(BMat A, BMat B, BMat Cm, int K, float alpha, int accumulate, int H,
         }
         *reinterpret_cast<float4 *>(cr) = make_float4(o[0], o[1], o[2], o[3]);
     }
-}
-
-// The tf32 case as a pipeline: operands go to shared memory in the layout they have in global memory
-// (16-byte asynchronous copies, three 32-wide steps of k in flight) and the fragment reads adapt to the
-// layout instead -- rows of 36 floats for a k-contiguous operand, of 72 for an m- or n-contiguous one,
-// both free of bank conflicts for the m16n8k8 fragments.  Operands are rounded to tf32 as they are
-// read, products accumulated in fp32; k is a multiple of 32 (64 or the head dimension).
-constexpr int kBgK = 32, kBgStages = 3;
-constexpr int kBgTileFloats = 64 * (kBgK + 4);           // = kBgK * 72: either layout
-constexpr size_t kBgSmem = (size_t)kBgStages * 2 * kBgTileFloats * sizeof(float);
-__device__ __forceinline__ void cp_async16(float *dst, const float *src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                     static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
-                 "l"(reinterpret_cast<uint64_t>(src))
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-template <bool TA, bool TB, int MASK>
-__global__ void __launch_bounds__(kThreads)
-bgemm_tf32_kernel(BMat A, BMat B, BMat Cm, int K, float alpha, int accumulate, int H, int NC) {
-    extern __shared__ __align__(16) float bg_smem[];
-    constexpr int kLdK = kBgK + 4, kLdMN = 72;
-    const int z = blockIdx.z, ch = z % NC, bh = z / NC, b = bh / H, h = bh % H;
-    const float *Ap = mat_base(A, b, h, ch), *Bp = mat_base(B, b, h, ch);
-    float *Cp = const_cast<float *>(mat_base(Cm, b, h, ch));
-    const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31, fg = lane >> 2, ft = lane & 3;
-    const int wr = (warp & 3) * 16, wc = (warp >> 2) * 32;
-    const int nk = K / kBgK;
-    auto issue = [&](int kt) {
-        if (kt < nk) {
-            float *As = bg_smem + (size_t)(kt % kBgStages) * 2 * kBgTileFloats, *Bs = As + kBgTileFloats;
-            const int k0 = kt * kBgK;
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int f = t + kThreads * i;
-                if (!TA) {   // A[m][k], k contiguous
-                    const int r = f / (kBgK / 4), kq = (f % (kBgK / 4)) * 4;
-                    cp_async16(As + r * kLdK + kq, Ap + (size_t)(m0 + r) * A.ld + k0 + kq);
-                } else {     // A[k][m], m contiguous
-                    const int kk = f / 16, r4 = (f % 16) * 4;
-                    cp_async16(As + kk * kLdMN + r4, Ap + (size_t)(k0 + kk) * A.ld + m0 + r4);
-                }
-                if (TB) {    // B[n][k], k contiguous
-                    const int c = f / (kBgK / 4), kq = (f % (kBgK / 4)) * 4;
-                    cp_async16(Bs + c * kLdK + kq, Bp + (size_t)(n0 + c) * B.ld + k0 + kq);
-                } else {     // B[k][n], n contiguous
-                    const int kk = f / 16, c4 = (f % 16) * 4;
-                    cp_async16(Bs + kk * kLdMN + c4, Bp + (size_t)(k0 + kk) * B.ld + n0 + c4);
-                }
-            }
-        }
-        cp_async_commit();       // (an empty group past the end keeps the count uniform)
-    };
-    float acc[4][4];             // n-tile i, fragment element j
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-#pragma unroll
-    for (int kt = 0; kt < kBgStages - 1; ++kt) issue(kt);
-    for (int kt = 0; kt < nk; ++kt) {
-        cp_async_wait<kBgStages - 2>();          // step kt has landed (this thread's copies) ...
-        __syncthreads();                         // ... and everyone's; step kt - 1 has been read by all
-        issue(kt + kBgStages - 1);               // into the slot of step kt - 1
-        const float *As = bg_smem + (size_t)(kt % kBgStages) * 2 * kBgTileFloats, *Bs = As + kBgTileFloats;
-        auto a_at = [&](int m, int k) { return to_tf32(TA ? As[k * kLdMN + m] : As[m * kLdK + k]); };
-        auto b_at = [&](int k, int n) { return to_tf32(TB ? Bs[n * kLdK + k] : Bs[k * kLdMN + n]); };
-#pragma unroll
-        for (int k8 = 0; k8 < kBgK; k8 += 8) {
-            const uint32_t a[4] = {a_at(wr + fg, k8 + ft), a_at(wr + fg + 8, k8 + ft),
-                                   a_at(wr + fg, k8 + ft + 4), a_at(wr + fg + 8, k8 + ft + 4)};
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                const uint32_t bfr[2] = {b_at(k8 + ft, wc + 8 * nt + fg), b_at(k8 + ft + 4, wc + 8 * nt + fg)};
-                mma_tf32_16x8x8(acc[nt], a, bfr);
-            }
-        }
-    }
-    cp_async_wait<0>();
-    // fragment layout: elements (0, 1) in row fg, (2, 3) in row fg + 8; columns 2 ft, 2 ft + 1
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-            const int row = m0 + wr + fg + 8 * hh, col = n0 + wc + 8 * nt + 2 * ft;
-            float o0 = alpha * acc[nt][2 * hh], o1 = alpha * acc[nt][2 * hh + 1];
-            if (MASK == 1) { if (col > row) o0 = 0.f; if (col + 1 > row) o1 = 0.f; }
-            if (MASK == 2) { if (col >= row) o0 = 0.f; if (col + 1 >= row) o1 = 0.f; }
-            float2 *cr = reinterpret_cast<float2 *>(Cp + (size_t)row * Cm.ld + col);
-            if (accumulate) { const float2 old = *cr; o0 += old.x; o1 += old.y; }
-            *cr = make_float2(o0, o1);
-        }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -338,8 +224,8 @@ combine_bwd_kernel(const float *__restrict__ o_la, const float *__restrict__ o_n
     }
     sums(dsm, dsm_s);
     if (!live) return;
-    *reinterpret_cast<float4 *>(do_la + at) = make_float4(dl[0], dl[1], dl[2], dl[3]);
-    // (the tensor-core softmax backward reads the fp16 copy only)
+    // (the tensor-core kernels read the fp16 copies only)
+    if (do_la) *reinterpret_cast<float4 *>(do_la + at) = make_float4(dl[0], dl[1], dl[2], dl[3]);
     if (do_nla) *reinterpret_cast<float4 *>(do_nla + at) = make_float4(dn[0], dn[1], dn[2], dn[3]);
     const size_t at16 = (((size_t)b * H + h) * L + l) * D + li * 4;
     auto h4 = [](float x0, float x1, float x2, float x3) {
@@ -895,313 +781,6 @@ gdn_assemble_kernel(const float *__restrict__ q32, const float *__restrict__ k32
     }
 }
 
-// The middle of the chunk-level chain in one kernel per chunk (bf16 storage, tf32 products):
-//   dKb = Tinv^T dW, dVb = Tinv^T dU~   (written out: the assembly reads them)
-//   M = -strictly_lower(dKb W^T + dVb U^T),  N = lower(dO U~^T)
-//   Mg = M . Gamma, Ms = diag(beta~) Mg, Ns = scale_la N . Gamma
-// 64 columns of the head at a time: dKb, dVb of those columns go from the accumulators to shared memory as
-// the next products' operands, and M, N add up in accumulators over the column blocks; the two 64 x 64
-// intermediates never reach global memory.  Warp w owns rows 16 (w & 3) .. and columns 32 (w >> 2) ..
-// of every 64 x 64 result.  Operand rows are 72 floats when read along the row index and 68 when read
-// along k (both free of bank conflicts for the fragments).
-constexpr size_t kTmSmem = sizeof(float) * (5 * kC * 72 + 2 * kC);
-
-template <int D>
-__global__ void __launch_bounds__(kThreads, 2)
-gdn_tm_kernel(const float *__restrict__ Tinv, const float *__restrict__ dW, const float *__restrict__ dUt,
-              const float *__restrict__ W, const float *__restrict__ U, const float *__restrict__ dO,
-              const float *__restrict__ Ut, const float *__restrict__ Gcum, const float *__restrict__ beta,
-              const uint8_t *__restrict__ route, float scale_la, float *__restrict__ dKb,
-              float *__restrict__ dVb, float *__restrict__ Mg, float *__restrict__ Ms, float *__restrict__ Ns,
-              int L, int H) {
-    extern __shared__ __align__(16) float tm_smem[];
-    float *sT = tm_smem, *bufA = sT + kC * 72, *bufB = bufA + kC * 72, *bufC = bufB + kC * 72, *bufD = bufC + kC * 72;
-    float *Gs = bufD + kC * 72, *bts = Gs + kC;
-    const int NC = L / kC, ch = blockIdx.x % NC, bh = blockIdx.x / NC, b = bh / H, h = bh % H;
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31, fg = lane >> 2, ft = lane & 3;
-    const int wr = (warp & 3) * 16, wc = (warp >> 2) * 32;
-    const size_t tok0 = ((size_t)b * L + (size_t)ch * kC) * H + h;         // the chunk's first token (stride H)
-    // 64 tokens x 64 columns [n0, n0 + 64) of a token-major array into rows of `ld` floats
-    auto load_tile = [&](float *dst, int ld, const float *src, int n0) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int f = t + kThreads * i, r = f >> 4, c4 = (f & 15) * 4;
-            cp_async16(dst + r * ld + c4, src + (tok0 + (size_t)r * H) * D + n0 + c4);
-        }
-    };
-    {
-        const float *ti = Tinv + (size_t)blockIdx.x * kC * kC;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int f = t + kThreads * i, r = f >> 4, c4 = (f & 15) * 4;
-            cp_async16(sT + r * 72 + c4, ti + r * kC + c4);
-        }
-    }
-    if (t < kC) {
-        const size_t tok = tok0 + (size_t)t * H;
-        bts[t] = route && route[tok] ? 0.f : beta[tok];
-        Gs[t] = Gcum[(size_t)bh * L + (size_t)ch * kC + t];
-    }
-    float Macc[4][4], Nacc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) { Macc[i][j] = 0.f; Nacc[i][j] = 0.f; }
-    const int m0 = wr + fg, m1 = wr + fg + 8;
-    // acc += A B^T with both operands stored [row][k] in rows of 68 floats
-    auto mma_abt = [&](float (&acc)[4][4], const float *A, const float *Bm) {
-#pragma unroll 2
-        for (int k8 = 0; k8 < kC; k8 += 8) {
-            const int ka = k8 + ft, kb = k8 + ft + 4;
-            const uint32_t a[4] = {to_tf32(A[m0 * 68 + ka]), to_tf32(A[m1 * 68 + ka]),
-                                   to_tf32(A[m0 * 68 + kb]), to_tf32(A[m1 * 68 + kb])};
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                const int n = wc + 8 * nt + fg;
-                const uint32_t bb[2] = {to_tf32(Bm[n * 68 + ka]), to_tf32(Bm[n * 68 + kb])};
-                mma_tf32_16x8x8(acc[nt], a, bb);
-            }
-        }
-    };
-    // Per 64 columns: every group of loads is in flight while the previous product runs.
-    for (int n0 = 0; n0 < D; n0 += 64) {
-        load_tile(bufA, 68, dO, n0);
-        load_tile(bufC, 68, Ut, n0);
-        cp_async_commit();
-        load_tile(bufB, 72, dW, n0);
-        load_tile(bufD, 72, dUt, n0);
-        cp_async_commit();
-        cp_async_wait<1>();
-        __syncthreads();
-        mma_abt(Nacc, bufA, bufC);           // dO U~^T
-        __syncthreads();                     // dO, U~ of these columns have been read by all
-        load_tile(bufA, 68, W, n0);
-        load_tile(bufC, 68, U, n0);
-        cp_async_commit();
-        cp_async_wait<1>();                  // dW, dU~ (and Tinv) have landed
-        __syncthreads();
-        float kb_[4][4], vb_[4][4];          // dKb, dVb of these 64 columns
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) { kb_[i][j] = 0.f; vb_[i][j] = 0.f; }
-#pragma unroll 2
-        for (int k8 = 0; k8 < kC; k8 += 8) {
-            const int ka = k8 + ft, kb = k8 + ft + 4;
-            const uint32_t a[4] = {to_tf32(sT[ka * 72 + m0]), to_tf32(sT[ka * 72 + m1]),
-                                   to_tf32(sT[kb * 72 + m0]), to_tf32(sT[kb * 72 + m1])};
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                const int n = wc + 8 * nt + fg;
-                const uint32_t b1[2] = {to_tf32(bufB[ka * 72 + n]), to_tf32(bufB[kb * 72 + n])};
-                const uint32_t b2[2] = {to_tf32(bufD[ka * 72 + n]), to_tf32(bufD[kb * 72 + n])};
-                mma_tf32_16x8x8(kb_[nt], a, b1);
-                mma_tf32_16x8x8(vb_[nt], a, b2);
-            }
-        }
-        __syncthreads();                     // dW, dU~ of these columns have been read by all
-        // fragment layout: elements (0, 1) in row fg, (2, 3) in row fg + 8; columns 2 ft, 2 ft + 1
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                const int row = wr + fg + 8 * hh, cl = wc + 8 * nt + 2 * ft;
-                const size_t i = (tok0 + (size_t)row * H) * D + n0 + cl;
-                const float2 kv = make_float2(kb_[nt][2 * hh], kb_[nt][2 * hh + 1]);
-                const float2 vv = make_float2(vb_[nt][2 * hh], vb_[nt][2 * hh + 1]);
-                *reinterpret_cast<float2 *>(dKb + i) = kv;
-                *reinterpret_cast<float2 *>(dVb + i) = vv;
-                *reinterpret_cast<float2 *>(bufB + row * 68 + cl) = kv;
-                *reinterpret_cast<float2 *>(bufD + row * 68 + cl) = vv;
-            }
-        cp_async_wait<0>();                  // W, U
-        __syncthreads();
-        mma_abt(Macc, bufB, bufA);           // dKb W^T
-        mma_abt(Macc, bufD, bufC);           // + dVb U^T
-        __syncthreads();
-    }
-    const size_t base = (size_t)blockIdx.x * kC * kC;
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-            const int row = wr + fg + 8 * hh, col = wc + 8 * nt + 2 * ft;
-            float mg[2], ns[2];
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int j = col + e;
-                const float gam = j <= row ? __expf(Gs[row] - Gs[j]) : 0.f;
-                mg[e] = j < row ? -Macc[nt][2 * hh + e] * gam : 0.f;
-                ns[e] = scale_la * Nacc[nt][2 * hh + e] * gam;
-            }
-            const size_t o = base + (size_t)row * kC + col;
-            *reinterpret_cast<float2 *>(Mg + o) = make_float2(mg[0], mg[1]);
-            *reinterpret_cast<float2 *>(Ms + o) = make_float2(bts[row] * mg[0], bts[row] * mg[1]);
-            *reinterpret_cast<float2 *>(Ns + o) = make_float2(ns[0], ns[1]);
-        }
-}
-
-// The last four chunk-level products and the assembly in one kernel per chunk (bf16 storage, tf32
-// products as in bgemm_tf32_kernel): X1 = Mg K, X2 = Ms^T K, X3 = Ns K, X4 = Ns^T Q stay in the
-// accumulator fragments and meet the other terms of dq, dk, dv there, so the four [B,L,H,d] fp32
-// arrays are neither written nor read back.  One CTA per chunk, 64 columns at a time; warp w owns rows
-// 16 (w & 3) .. and columns 32 (w >> 2) .. of the 64; the eight per-row dot products are summed over a
-// thread's columns, then over the four lanes that share a row, then over the two warps that do.
-constexpr int kXaLdA = 68, kXaLdT = 72;                  // rows read along k / read transposed (and K, Q)
-constexpr size_t kXaSmem = sizeof(float) * (2 * kC * kXaLdA + 3 * kC * kXaLdT + 4 * kC + 2 * kC * 8);
-
-template <typename T, int D>
-__global__ void __launch_bounds__(kThreads, 2)
-gdn_xassemble_kernel(const float *__restrict__ q32, const float *__restrict__ k32,
-                     const float *__restrict__ v32, const float *__restrict__ Gcum,
-                     const float *__restrict__ beta, const uint8_t *__restrict__ route,
-                     const float *__restrict__ dQg, const float *__restrict__ dKb,
-                     const float *__restrict__ dVb, const float *__restrict__ dKt,
-                     const float *__restrict__ Mg, const float *__restrict__ Ms,
-                     const float *__restrict__ Ns, const float *__restrict__ dq_sm,
-                     const float *__restrict__ dk_x, const float *__restrict__ dv_x, float scale_la,
-                     T *__restrict__ dq, T *__restrict__ dk, T *__restrict__ dv, float *__restrict__ dGrow,
-                     float *__restrict__ kappa, float *__restrict__ dbeta, int L, int H) {
-    extern __shared__ __align__(16) float xa_smem[];
-    float *sMg = xa_smem;                        // [i][j], ld 68
-    float *sNs = sMg + kC * kXaLdA;              // [i][j], ld 68
-    float *sMs = sNs + kC * kXaLdA;              // [i][j], ld 72 (read transposed only)
-    float *sK = sMs + kC * kXaLdT;               // [token][64 columns], ld 72
-    float *sQ = sK + kC * kXaLdT;
-    float *sGam = sQ + kC * kXaLdT, *sKt = sGam + kC, *sBt = sKt + kC, *sLin = sBt + kC;
-    float *sSum = sLin + kC;                     // [2 column warps][64 rows][8]
-    const int NC = L / kC, ch = blockIdx.x % NC, bh = blockIdx.x / NC, b = bh / H, h = bh % H;
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31, fg = lane >> 2, ft = lane & 3;
-    const int wr = (warp & 3) * 16, wcw = warp >> 2, wc = wcw * 32;
-    const size_t tok0 = ((size_t)b * L + (size_t)ch * kC) * H + h;         // the chunk's first token (stride H)
-    const size_t bhl = (size_t)bh * L + (size_t)ch * kC;
-    {
-        const float *mg = Mg + (size_t)blockIdx.x * kC * kC, *msrc = Ms + (size_t)blockIdx.x * kC * kC,
-                    *ns = Ns + (size_t)blockIdx.x * kC * kC;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int f = t + kThreads * i, r = f >> 4, c4 = (f & 15) * 4;
-            cp_async16(sMg + r * kXaLdA + c4, mg + r * kC + c4);
-            cp_async16(sNs + r * kXaLdA + c4, ns + r * kC + c4);
-            cp_async16(sMs + r * kXaLdT + c4, msrc + r * kC + c4);
-        }
-    }
-    if (t < kC) {
-        const size_t tok = tok0 + (size_t)t * H;
-        const float Gi = Gcum[bhl + t], GC = Gcum[bhl + kC - 1];
-        const bool lin = !route || route[tok] == 0;
-        sGam[t] = __expf(Gi);
-        sKt[t] = __expf(GC - Gi);
-        sBt[t] = lin ? beta[tok] : 0.f;
-        sLin[t] = lin ? 1.f : 0.f;
-    }
-    float sums[2][8];            // per row half: kdKb, qdQg, kdKt, kX1, kX2, qX3, kX4, vdVb
-#pragma unroll
-    for (int hh = 0; hh < 2; ++hh)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) sums[hh][j] = 0.f;
-
-    for (int n0 = 0; n0 < D; n0 += 64) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int f = t + kThreads * i, r = f >> 4, c4 = (f & 15) * 4;
-            cp_async16(sK + r * kXaLdT + c4, k32 + (tok0 + (size_t)r * H) * D + n0 + c4);
-            cp_async16(sQ + r * kXaLdT + c4, q32 + (tok0 + (size_t)r * H) * D + n0 + c4);
-        }
-        cp_async_commit();
-        cp_async_wait<0>();
-        __syncthreads();
-        float x1[4][4], x2[4][4], x3[4][4], x4[4][4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) { x1[i][j] = 0.f; x2[i][j] = 0.f; x3[i][j] = 0.f; x4[i][j] = 0.f; }
-#pragma unroll 2
-        for (int k8 = 0; k8 < kC; k8 += 8) {
-            const int m0 = wr + fg, m1 = wr + fg + 8, ka = k8 + ft, kb = k8 + ft + 4;
-            const uint32_t a1[4] = {to_tf32(sMg[m0 * kXaLdA + ka]), to_tf32(sMg[m1 * kXaLdA + ka]),
-                                    to_tf32(sMg[m0 * kXaLdA + kb]), to_tf32(sMg[m1 * kXaLdA + kb])};
-            const uint32_t a2[4] = {to_tf32(sMs[ka * kXaLdT + m0]), to_tf32(sMs[ka * kXaLdT + m1]),
-                                    to_tf32(sMs[kb * kXaLdT + m0]), to_tf32(sMs[kb * kXaLdT + m1])};
-            const uint32_t a3[4] = {to_tf32(sNs[m0 * kXaLdA + ka]), to_tf32(sNs[m1 * kXaLdA + ka]),
-                                    to_tf32(sNs[m0 * kXaLdA + kb]), to_tf32(sNs[m1 * kXaLdA + kb])};
-            const uint32_t a4[4] = {to_tf32(sNs[ka * kXaLdA + m0]), to_tf32(sNs[ka * kXaLdA + m1]),
-                                    to_tf32(sNs[kb * kXaLdA + m0]), to_tf32(sNs[kb * kXaLdA + m1])};
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                const int n = wc + 8 * nt + fg;
-                const uint32_t bk[2] = {to_tf32(sK[ka * kXaLdT + n]), to_tf32(sK[kb * kXaLdT + n])};
-                const uint32_t bq[2] = {to_tf32(sQ[ka * kXaLdT + n]), to_tf32(sQ[kb * kXaLdT + n])};
-                mma_tf32_16x8x8(x1[nt], a1, bk);
-                mma_tf32_16x8x8(x2[nt], a2, bk);
-                mma_tf32_16x8x8(x3[nt], a3, bk);
-                mma_tf32_16x8x8(x4[nt], a4, bq);
-            }
-        }
-        // fragment layout: elements (0, 1) in row fg, (2, 3) in row fg + 8; columns 2 ft, 2 ft + 1
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-            const int row = wr + fg + 8 * hh;
-            const float gam = sGam[row], kt = sKt[row], bt = sBt[row];
-            const bool lin = sLin[row] != 0.f;
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                const int cl = wc + 8 * nt + 2 * ft;                     // column within the 64
-                const size_t i = (tok0 + (size_t)row * H) * D + n0 + cl;
-                const float2 a_dQg = *reinterpret_cast<const float2 *>(dQg + i), a_dKb = *reinterpret_cast<const float2 *>(dKb + i);
-                const float2 a_dVb = *reinterpret_cast<const float2 *>(dVb + i), a_dKt = *reinterpret_cast<const float2 *>(dKt + i);
-                const float2 vv = *reinterpret_cast<const float2 *>(v32 + i);
-                const float2 qv = *reinterpret_cast<const float2 *>(sQ + row * kXaLdT + cl);
-                const float2 kv = *reinterpret_cast<const float2 *>(sK + row * kXaLdT + cl);
-                float2 e_dq = dq_sm ? *reinterpret_cast<const float2 *>(dq_sm + i) : make_float2(0.f, 0.f);
-                float2 e_dk = dk_x ? *reinterpret_cast<const float2 *>(dk_x + i) : make_float2(0.f, 0.f);
-                float2 e_dv = dv_x ? *reinterpret_cast<const float2 *>(dv_x + i) : make_float2(0.f, 0.f);
-                const float x1a = x1[nt][2 * hh], x1b = x1[nt][2 * hh + 1], x2a = x2[nt][2 * hh], x2b = x2[nt][2 * hh + 1];
-                const float x3a = x3[nt][2 * hh], x3b = x3[nt][2 * hh + 1], x4a = x4[nt][2 * hh], x4b = x4[nt][2 * hh + 1];
-                float *sm = sums[hh];
-                sm[0] = fmaf(kv.x, a_dKb.x, fmaf(kv.y, a_dKb.y, sm[0]));
-                sm[1] = fmaf(qv.x, a_dQg.x, fmaf(qv.y, a_dQg.y, sm[1]));
-                sm[2] = fmaf(kv.x, a_dKt.x, fmaf(kv.y, a_dKt.y, sm[2]));
-                sm[3] = fmaf(kv.x, x1a, fmaf(kv.y, x1b, sm[3]));
-                sm[4] = fmaf(kv.x, x2a, fmaf(kv.y, x2b, sm[4]));
-                sm[5] = fmaf(qv.x, x3a, fmaf(qv.y, x3b, sm[5]));
-                sm[6] = fmaf(kv.x, x4a, fmaf(kv.y, x4b, sm[6]));
-                sm[7] = fmaf(vv.x, a_dVb.x, fmaf(vv.y, a_dVb.y, sm[7]));
-                const float sgm = scale_la * gam;
-                store2(dq + i, sgm * a_dQg.x + x3a + e_dq.x, sgm * a_dQg.y + x3b + e_dq.y);
-                if (lin) {
-                    const float bg = bt * gam;
-                    store2(dk + i, bg * a_dKb.x + kt * a_dKt.x + bt * x1a + x2a + x4a + e_dk.x,
-                           bg * a_dKb.y + kt * a_dKt.y + bt * x1b + x2b + x4b + e_dk.y);
-                    store2(dv + i, bt * a_dVb.x + e_dv.x, bt * a_dVb.y + e_dv.y);
-                }
-            }
-        }
-        __syncthreads();         // K, Q of these columns have been read by all
-    }
-#pragma unroll
-    for (int hh = 0; hh < 2; ++hh)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            float v = sums[hh][j];
-            v += __shfl_xor_sync(0xffffffffu, v, 1);
-            v += __shfl_xor_sync(0xffffffffu, v, 2);
-            if (ft == 0) sSum[(wcw * kC + wr + fg + 8 * hh) * 8 + j] = v;
-        }
-    __syncthreads();
-    if (t < kC) {
-        float r[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) r[j] = sSum[t * 8 + j] + sSum[(kC + t) * 8 + j];
-        const float gam = sGam[t], kt = sKt[t], bt = sBt[t];
-        const bool lin = sLin[t] != 0.f;
-        const float kap = kt * r[2];
-        dGrow[bhl + t] = bt * gam * r[0] + scale_la * gam * r[1] - kap + bt * r[3] - r[4] + r[5] - r[6];
-        kappa[bhl + t] = kap;
-        dbeta[tok0 + (size_t)t * H] = lin ? gam * r[0] + r[7] + r[3] : 0.f;
-    }
-}
-
 // dg_j = sum_{i>=j in chunk} dG_i, with the chunk-end extras added to the last row.
 __global__ void dg_kernel(const float *__restrict__ dGrow, const float *__restrict__ kappa,
                           const float *__restrict__ gS, const float *__restrict__ Gcum, int n_slices,
@@ -1257,16 +836,10 @@ cudaError_t set_smem(Kn kernel, size_t bytes) {
 cudaError_t launch_bgemm(bool ta, bool tb, int mask, BMat A, BMat B, BMat C, int m, int n, int k,
                          float alpha, bool accumulate, Shape s, cudaStream_t st) {
     const int NC = s.L / kC;
-    if (m % 64 || n % 64 || k % kBgK) return cudaErrorInvalidValue;
+    if (m % 64 || n % 64 || k % 16) return cudaErrorInvalidValue;
     dim3 grid(n / 64, m / 64, s.B * s.H * NC);
-#define NATSL_BG(TA, TB, MK)                                                                                   \
-    do {                                                                                                        \
-        if (s.bf16) {                                                                                           \
-            cudaError_t e = allow_smem(bgemm_tf32_kernel<TA, TB, MK>, (int)kBgSmem);    \
-            if (e != cudaSuccess) return e;                                                                     \
-            bgemm_tf32_kernel<TA, TB, MK><<<grid, kThreads, kBgSmem, st>>>(A, B, C, k, alpha, accumulate ? 1 : 0, s.H, NC); \
-        } else bgemm_kernel<TA, TB, MK><<<grid, kThreads, 0, st>>>(A, B, C, k, alpha, accumulate ? 1 : 0, s.H, NC); \
-    } while (0)
+#define NATSL_BG(TA, TB, MK) \
+    bgemm_kernel<TA, TB, MK><<<grid, kThreads, 0, st>>>(A, B, C, k, alpha, accumulate ? 1 : 0, s.H, NC)
     if (!ta && !tb && mask == 0) NATSL_BG(false, false, 0);
     else if (!ta && tb && mask == 0) NATSL_BG(false, true, 0);
     else if (ta && !tb && mask == 0) NATSL_BG(true, false, 0);
@@ -1499,54 +1072,6 @@ static cudaError_t finish_impl(const AssembleArgs &a, void *dk, void *dv, Shape 
                                                        (T *)dk, (T *)dv, s.L, s.H);
     count_launch();
     return cudaGetLastError();
-}
-
-cudaError_t launch_gdn_tm(const float *Tinv, const float *dW, const float *dUt, const float *W, const float *U,
-                          const float *dO, const float *Ut, const float *Gcum, const float *beta,
-                          const uint8_t *route, float scale_la, float *dKb, float *dVb, float *Mg, float *Ms,
-                          float *Ns, Shape s, cudaStream_t st) {
-    const unsigned nch = (unsigned)(s.B * s.H * (s.L / kC));
-    auto kernel = s.d == 128 ? gdn_tm_kernel<128> : gdn_tm_kernel<64>;
-    cudaError_t e = allow_smem(kernel, (int)kTmSmem);
-    if (e != cudaSuccess) return e;
-    kernel<<<nch, kThreads, kTmSmem, st>>>(Tinv, dW, dUt, W, U, dO, Ut, Gcum, beta, route, scale_la, dKb, dVb, Mg,
-                                          Ms, Ns, s.L, s.H);
-    count_launch();
-    return cudaGetLastError();
-}
-
-template <typename T, int D>
-static cudaError_t xassemble_impl(const AssembleArgs &a, const float *Mg, const float *Ms, const float *Ns,
-                                  void *dq, void *dk, void *dv, Shape s, cudaStream_t st) {
-    const int NC = s.L / kC;
-    const size_t nch = (size_t)s.B * s.H * NC;
-    cudaError_t e = allow_smem(gdn_xassemble_kernel<T, D>,
-                                         (int)kXaSmem);
-    if (e != cudaSuccess) return e;
-    gdn_xassemble_kernel<T, D><<<(unsigned)nch, kThreads, kXaSmem, st>>>(
-        a.q32, a.k32, a.v32, a.Gcum, a.beta, a.route, a.dQg, a.dKb, a.dVb, a.dKt, Mg, Ms, Ns, a.dq_sm, a.dk_x,
-        a.dv_x, a.scale_la, (T *)dq, (T *)dk, (T *)dv, a.dGrow, a.kappa, a.dbeta, s.L, s.H);
-    count_launch();
-    dg_kernel<<<(unsigned)((nch + 127) / 128), 128, 0, st>>>(a.dGrow, a.kappa, a.gS, a.Gcum,
-                                                            s.d / kDvs, a.dg, s.B, s.L, s.H);
-    count_launch();
-    if (a.no_scatter) return cudaGetLastError();
-    constexpr int kRows = kThreads / (D / 4);
-    dim3 grid((a.cap + kRows - 1) / kRows, s.B * s.H);
-    scatter_sm_kernel<T, D><<<grid, kThreads, 0, st>>>(a.dk_sm, a.dv_sm, a.cap, a.sm_idx, a.sm_prefix,
-                                                       (T *)dk, (T *)dv, s.L, s.H);
-    count_launch();
-    return cudaGetLastError();
-}
-
-cudaError_t launch_gdn_xassemble(const AssembleArgs &a, const float *Mg, const float *Ms, const float *Ns,
-                                 void *dq, void *dk, void *dv, Shape s, cudaStream_t st) {
-    if (s.bf16) {
-        if (s.d == 128) return xassemble_impl<__nv_bfloat16, 128>(a, Mg, Ms, Ns, dq, dk, dv, s, st);
-        return xassemble_impl<__nv_bfloat16, 64>(a, Mg, Ms, Ns, dq, dk, dv, s, st);
-    }
-    if (s.d == 128) return xassemble_impl<float, 128>(a, Mg, Ms, Ns, dq, dk, dv, s, st);
-    return xassemble_impl<float, 64>(a, Mg, Ms, Ns, dq, dk, dv, s, st);
 }
 
 cudaError_t launch_gdn_finish(const AssembleArgs &a, void *dk, void *dv, Shape s, cudaStream_t st,

@@ -9,11 +9,13 @@
 // threads (r, half 0 / 1) of warps q and q + 4, the fp32 gradient state lives in their registers,
 // and the operands a thread produces (dS1, dU~ as fp16) are written to its own TMEM lane:
 //   X1 = dO^T P            X2 = dS1^T K^T                       (both [d, 64 tokens])
-//   dU~^T = X1 + X2 diag(gamma_C / gamma)        -> global (fp32, token-major) and fp16 operand
+//   dU~^T = X1 + X2 diag(gamma_C / gamma)        -> fp16 operand, in TMEM and to global
 //   Y  = (diag(scale_la gamma) dO)^T Q - dU~^T W                ([d, d], second product negated)
 //   dS0^T = gamma_C dS1^T + Y
 // dO and scale_la gamma dO arrive as fp16 tiles [B,H,L,d]; P, W^T and the fp16 q, k copies are the
-// forward's own intermediates.  The chunk-exit gradients dS1 are stored for the later products.
+// forward's own intermediates.  dU~ and the chunk-exit gradients dS1 leave as the fp16 operands they are, in
+// 16-byte pieces whose stores are contiguous over a warp (as fp32 rows they took 96 narrow stores per thread and
+// chunk), in units of the gradient scale, for the chunk kernel.
 #include "common.cuh"
 #include "natsl_internal.h"
 #include "tc_common.cuh"
@@ -61,7 +63,7 @@ gdn_rscan_tc_kernel(const __grid_constant__ CUtensorMap map_do,    // dO (fp16) 
                     const __grid_constant__ CUtensorMap map_qh, const __grid_constant__ CUtensorMap map_kh,
                     const __grid_constant__ CUtensorMap map_wt,    // W^T [B*H*NC*D][64], box D
                     const __grid_constant__ CUtensorMap map_ph,    // P [B*H*NC*64][64], box 64
-                    const float *__restrict__ Gd, float *__restrict__ dUt, float *__restrict__ dS_c,
+                    const float *__restrict__ Gd, __half *__restrict__ dU16, __half *__restrict__ dS16,
                     const float *__restrict__ dstate_out, float *__restrict__ dstate_in,
                     const uint8_t *__restrict__ block_route, int32_t *status, int L, int H, int wait_kcycles) {
     using SL = RsLayout<D>;
@@ -177,9 +179,9 @@ gdn_rscan_tc_kernel(const __grid_constant__ CUtensorMap map_do,    // dO (fp16) 
             // so the exit-state gradient does not flow into its dU~ (it still decays into dS0)
             const float commit = kBlock && block_route[((size_t)b * L + (size_t)c * 64) * H + h] ? 0.f : 1.f;
             // ---- dS1 (exit-state gradient of chunk c): fp16 operand into TMEM, then (behind the
-            // arrival, off the chain) the fp32 copy the later products read ----
+            // arrival, off the chain) the copy the chunk kernel reads ----
+            uint32_t pk[kHalfCols / 2];
             {
-                uint32_t pk[kHalfCols / 2];
 #pragma unroll
                 for (int x = 0; x < kHalfCols / 2; ++x) pk[x] = pack_half2(G[2 * x], G[2 * x + 1]);
                 if (kHalfCols == 64)
@@ -193,9 +195,10 @@ gdn_rscan_tc_kernel(const __grid_constant__ CUtensorMap map_do,    // dO (fp16) 
             tc_fence_before_sync();
             mbar_arrive(&ms.barA);
             if (active) {
-                float *dst = dS_c + (((size_t)bh * NC + c) * D + col0) * D + r;
+                uint4 *dst = reinterpret_cast<uint4 *>(dS16) + (((size_t)bh * NC + c) * (D / 8) + col0 / 8) * D + r;
 #pragma unroll
-                for (int x = 0; x < kHalfCols; ++x) dst[(size_t)x * D] = gsc.y * G[x];
+                for (int x = 0; x < kHalfCols / 8; ++x)
+                    dst[(size_t)x * D] = make_uint4(pk[4 * x], pk[4 * x + 1], pk[4 * x + 2], pk[4 * x + 3]);
             }
             ok = mbar_wait(&ms.full[s], (n / kRsStages) & 1, abort_flag);   // decay factors of the chunk
             if (!ok) break;
@@ -208,8 +211,9 @@ gdn_rscan_tc_kernel(const __grid_constant__ CUtensorMap map_do,    // dO (fp16) 
             ok = mbar_wait(&ms.barX, n & 1, abort_flag);
             if (!ok) break;
             tc_fence_after_sync();
-            float du[32];
+            uint32_t dpk[16];
             {
+                float du[32];
                 uint32_t x1[32], x2[32];
                 tmem_ld32(tmem + SL::cX1 + tk0 + lane_base, x1);
                 tmem_ld32(tmem + SL::cX2 + tk0 + lane_base, x2);
@@ -218,19 +222,19 @@ gdn_rscan_tc_kernel(const __grid_constant__ CUtensorMap map_do,    // dO (fp16) 
                 for (int j = 0; j < 32; ++j)
                     du[j] = fmaf(kBlock ? commit * e2[tk0 + j] : e2[tk0 + j], __uint_as_float(x2[j]),
                                  __uint_as_float(x1[j]));
-                uint32_t pk[16];
 #pragma unroll
-                for (int x = 0; x < 16; ++x) pk[x] = pack_half2(du[2 * x], du[2 * x + 1]);
+                for (int x = 0; x < 16; ++x) dpk[x] = pack_half2(du[2 * x], du[2 * x + 1]);
                 // into this thread's own X2 columns: 16 packed columns per 32 tokens
-                tmem_st16(tmem + SL::cX2 + tk0 + lane_base, pk);
+                tmem_st16(tmem + SL::cX2 + tk0 + lane_base, dpk);
                 tmem_wait_st();
             }
             tc_fence_before_sync();
             mbar_arrive(&ms.barB);
-            if (active) {                                   // the fp32 copy, behind the arrival
-                float *dst = dUt + (((size_t)b * L + (size_t)c * 64 + tk0) * H + h) * D + r;
+            if (active) {                                   // the copy, behind the arrival
+                uint4 *dst = reinterpret_cast<uint4 *>(dU16) + (((size_t)bh * NC + c) * 8 + tk0 / 8) * D + r;
 #pragma unroll
-                for (int j = 0; j < 32; ++j) dst[(size_t)j * H * D] = gsc.y * du[j];
+                for (int x = 0; x < 4; ++x)
+                    dst[(size_t)x * D] = make_uint4(dpk[4 * x], dpk[4 * x + 1], dpk[4 * x + 2], dpk[4 * x + 3]);
             }
             // ---- dS0 = gamma_C dS1 + Y ----
             ok = mbar_wait(&ms.barY, n & 1, abort_flag);
@@ -260,82 +264,12 @@ gdn_rscan_tc_kernel(const __grid_constant__ CUtensorMap map_do,    // dO (fp16) 
     if (tid == 0 && ms.abort_flag) atomicMin(status, (int)NATSL_ERR_TIMEOUT);
 }
 
-// gS[chunk] = <dS1[chunk], S0[chunk]> (first slot of the row; the other slots are zeroed).
-// Block-level routing (block_route given): the exit-state gradient of a softmax block, whose update
-// was not committed, is then cleared, so that the dK~ product that reads it next yields zero.
-__global__ void __launch_bounds__(256)
-state_dot_kernel(float *__restrict__ dS_c, const float *__restrict__ S_c, float *__restrict__ gS,
-                 int n_slices, int dd, const uint8_t *__restrict__ block_route, int L, int H) {
-    __shared__ float red[8];
-    const size_t chunk = blockIdx.x;
-    float4 *a = reinterpret_cast<float4 *>(dS_c + chunk * dd);
-    const float4 *bq = reinterpret_cast<const float4 *>(S_c + chunk * dd);
-    float acc = 0.f;
-    for (int i = threadIdx.x; i < dd / 4; i += 256) {
-        const float4 x = a[i], y = bq[i];
-        acc = fmaf(x.x, y.x, fmaf(x.y, y.y, fmaf(x.z, y.z, fmaf(x.w, y.w, acc))));
-    }
-    acc = warp_sum(acc);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int wv = 0; wv < 8; ++wv) t += red[wv];
-        gS[chunk * n_slices] = t;
-        for (int sl = 1; sl < n_slices; ++sl) gS[chunk * n_slices + sl] = 0.f;
-    }
-    if (block_route) {
-        const int NC = L / kC;
-        const size_t bh = chunk / NC;
-        const int c = (int)(chunk % NC), b = (int)(bh / H), h = (int)(bh % H);
-        if (block_route[((size_t)b * L + (size_t)c * kC) * H + h])       // (every thread has read its part above)
-            for (int i = threadIdx.x; i < dd / 4; i += 256) a[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-}
-
-
-// ==========================================================================================
-// Chunk-parallel part of the backward for d = 64: everything that follows the reverse scan, one
-// CTA per chunk, all operands of the chunk staged once in shared memory as fp16 tiles and every
-// product (64x64x64) a set of warp-level MMAs fed by ldmatrix:
-//   dQg = dO S0^T        dW = -dU~ S0^T        dK~ = U~ dS1^T        N = dO U~^T
-//   dKb = T^T dW         dVb = T^T dU~         M = -(dKb W^T + dVb U^T)
-//   Ns = scale_la (N . Gamma) [j <= i]    Mg = M . Gamma [j < i]    Ms = diag(beta~) Mg
-//   dq = scale_la gamma dQg + Ns K + dq_softmax
-//   dk = beta~ gamma dKb + (gamma_C/gamma) dK~ + beta~ Mg K + Ms^T K + Ns^T Q      (linear tokens)
-//   dv = beta~ dVb                                                                  (linear tokens)
-// and the per-token sums the gate gradients need (dG, kappa, dbeta).
-// Range.  The forward quantities (U~, S0, T, W, U, q, k) are O(1) like every fp16 operand of the
-// forward kernels; the three gradient tiles are not (their size follows the incoming gradient), so
-// each of dO, dU~, dS1 is scaled by a power of two that brings its largest element of the chunk to
-// (0.5, 1].  Every result is linear in exactly one of the three, and the factor is taken out again
-// where the result is folded into dq, dk, dv and the sums.
-// Each of the 8 warps owns a 16 x 32 block of every 64 x 64 result; dq, dk, dv accumulate in
-// registers across the products.
-// ==========================================================================================
+// ------------------------------------------------------------------------------------------
+// 64 x 64 x 64 products on warp-level MMAs
+// ------------------------------------------------------------------------------------------
 constexpr int kCkThreads = 256;
 constexpr int kLdH = 72;                       // row stride of a staged 64x64 fp16 tile, elements
 constexpr int kTileH = 64 * kLdH;
-constexpr int kCkSlots = 12;
-constexpr int kCkSmem = kCkSlots * kTileH * 2 + 5 * 64 * 4 + 40 * 4;
-
-struct ChunkBwdArgs {
-    const __nv_bfloat16 *q, *k, *v;
-    const float *dO, *dUt, *Ut, *S_c, *dS_c, *Tinv, *Up, *Gcum, *beta, *dq_sm;   // Up: U^T in 4-token pieces
-    const __half *Wt;                                                            // W^T [chunk][d][64]
-    const uint8_t *route;
-    float scale_la;
-    __nv_bfloat16 *dq, *dk, *dv;
-    float *dg, *dbeta;
-    int L, H;
-    // Block-level routing (kernel instantiated with kBlock): every token takes part in the delta rule (beta~ = beta), a
-    // softmax block's update was not committed (its exit-state gradient reaches nothing but the
-    // decay), and every token's dk, dv also has a softmax-branch part, given in dk_x, dv_x
-    // (fp32, token-major).
-    const float *dk_x, *dv_x;
-    float *kap_c;    // [B,H,L/C] or nullptr: sum over the chunk of kappa = <dS1, K~^T U~>, the gradient
-                     // of a mask on the update this chunk commits to the state (Section 4.2, d score^la)
-};
 
 // acc (16 x 32 block at (row0, n0) of a 64 x 64 result) += A B over k = 0..63, fp16 tiles.
 // AT: A is stored [k][m] (else [m][k]);  BNK: B is stored [n][k] (else [k][n]).
@@ -360,362 +294,13 @@ __device__ __forceinline__ void mma64(const __half *A, const __half *B, int row0
     }
 }
 
-__device__ __forceinline__ float pow2_scale(float amax) {   // power of two s with s * amax in (0.5, 1]
-    if (!(amax > 0.f) || !isfinite(amax)) return 1.f;
-    int e;
-    frexpf(amax, &e);                                       // amax = m 2^e, m in [0.5, 1)
-    return ldexpf(1.f, -min(max(e, -100), 100));
-}
-
-template <bool kBlock>   // kBlock: block-level routing (see ChunkBwdArgs)
-__global__ void __launch_bounds__(kCkThreads, 2) gdn_bwd_chunk_kernel(ChunkBwdArgs p) {
-    constexpr int D = 64;
-    extern __shared__ __align__(16) uint8_t smraw[];
-    __half *sm = reinterpret_cast<__half *>(smraw);
-    __half *sDO = sm, *sDU = sm + kTileH, *sUt = sm + 2 * kTileH, *sS0 = sm + 3 * kTileH,
-           *sDS1 = sm + 4 * kTileH, *sT = sm + 5 * kTileH, *sW = sm + 6 * kTileH, *sU = sm + 7 * kTileH,
-           *sK = sm + 8 * kTileH, *sQ = sm + 9 * kTileH, *sX = sm + 10 * kTileH, *sY = sm + 11 * kTileH;
-    float *sG = reinterpret_cast<float *>(sm + kCkSlots * kTileH), *sBt = sG + 64, *rG = sBt + 64,
-          *rK = rG + 64, *rB = rK + 64, *sMax = rB + 64;   // sMax: 3 tiles x 8 warp maxima, 8 partial <dS1, S0>, 4 scan totals
-
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-    const int c = blockIdx.x, bh = blockIdx.y, b = bh / p.H, h = bh % p.H, NC = p.L / kC;
-    const size_t ts = (size_t)p.H * D;                              // token stride, elements
-    const size_t tok0 = (((size_t)b * p.L + (size_t)c * kC) * p.H + h) * D;   // element offset of the chunk
-    const size_t chunk = (size_t)bh * NC + c;
-
-    // ---- stage the chunk.  Thread -> rows r0 + 16 it (it < 4), columns c4..c4+3 of every tile ----
-    const int r0 = tid >> 4, c4 = (tid & 15) * 4;
-    auto ld_tile = [&](float4 (&x)[4], const float *src, size_t row_stride) {
-#pragma unroll
-        for (int it = 0; it < 4; ++it)
-            x[it] = *reinterpret_cast<const float4 *>(src + (size_t)(r0 + 16 * it) * row_stride + c4);
-    };
-    auto st_tile = [&](__half *dst, const float4 (&x)[4], float f) {
-#pragma unroll
-        for (int it = 0; it < 4; ++it)
-            *reinterpret_cast<uint2 *>(dst + (r0 + 16 * it) * kLdH + c4) =
-                make_uint2(pack_half2(f * x[it].x, f * x[it].y), pack_half2(f * x[it].z, f * x[it].w));
-    };
-    auto amax4 = [](const float4 (&x)[4]) {
-        float m = 0.f;
-#pragma unroll
-        for (int it = 0; it < 4; ++it)
-            m = fmaxf(m, fmaxf(fmaxf(fabsf(x[it].x), fabsf(x[it].y)), fmaxf(fabsf(x[it].z), fabsf(x[it].w))));
-        return m;
-    };
-    float scO, scU, scS;
-    {
-        // Two batches of tiles are in flight at a time: the loads of the next batch are issued
-        // before the previous one is converted and stored.
-        float4 xo[4], xu[4], xs[4], y0[4], y1[4], y2[4];
-        ld_tile(xo, p.dO + tok0, ts);
-        ld_tile(xu, p.dUt + tok0, ts);
-        ld_tile(xs, p.dS_c + chunk * D * D, D);
-        ld_tile(y0, p.Ut + tok0, ts);
-        ld_tile(y1, p.S_c + chunk * D * D, D);
-        ld_tile(y2, p.Tinv + chunk * 4096, 64);
-        if (tid < 64) {
-            const size_t tk = ((size_t)b * p.L + (size_t)c * kC + tid) * p.H + h;
-            sG[tid] = p.Gcum[(size_t)bh * p.L + c * kC + tid];
-            sBt[tid] = !kBlock && p.route[tk] ? 0.f : p.beta[tk];
-            rG[tid] = 0.f; rK[tid] = 0.f; rB[tid] = 0.f;
-        }
-        const float mo = warp_max(amax4(xo)), mu = warp_max(amax4(xu)), msx = warp_max(amax4(xs));
-        // <dS1, S0> of the chunk (both tiles are in registers, element for element): the decay of the
-        // entry state contributes gamma_C times it to every dg of the chunk
-        float dot = 0.f;
-#pragma unroll
-        for (int it = 0; it < 4; ++it)
-            dot = fmaf(xs[it].x, y1[it].x, fmaf(xs[it].y, y1[it].y, fmaf(xs[it].z, y1[it].z, fmaf(xs[it].w, y1[it].w, dot))));
-        dot = warp_sum(dot);
-        if (lane == 0) { sMax[warp] = mo; sMax[8 + warp] = mu; sMax[16 + warp] = msx; sMax[24 + warp] = dot; }
-        __syncthreads();
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f;
-#pragma unroll
-        for (int wv = 0; wv < 8; ++wv) {
-            a0 = fmaxf(a0, sMax[wv]); a1 = fmaxf(a1, sMax[8 + wv]); a2 = fmaxf(a2, sMax[16 + wv]);
-        }
-        scO = pow2_scale(a0); scU = pow2_scale(a1); scS = pow2_scale(a2);
-        st_tile(sDO, xo, scO);
-        st_tile(sDU, xu, scU);
-        // (an uncommitted block: the tile is zero, so dK~ and kappa vanish; <dS1, S0> above does not)
-        st_tile(sDS1, xs, kBlock && p.route[((size_t)b * p.L + (size_t)c * kC) * p.H + h] ? 0.f : scS);
-        // next batch into the freed registers: W^T and U^T as the forward kernels keep them (fp16
-        // [d][64] tile; fp32 in 4-token pieces [16][d][4]) -- both are [k][n] operands as they are
-        uint4 wt[2];
-#pragma unroll
-        for (int it = 0; it < 2; ++it)
-            wt[it] = reinterpret_cast<const uint4 *>(p.Wt + chunk * D * 64)[tid + it * kCkThreads];
-#pragma unroll
-        for (int it = 0; it < 4; ++it)
-            xu[it] = reinterpret_cast<const float4 *>(p.Up + chunk * D * 64)[tid + it * kCkThreads];
-        uint2 qk[2][4];
-#pragma unroll
-        for (int it = 0; it < 4; ++it) {
-            const size_t off = tok0 + (size_t)(r0 + 16 * it) * ts + c4;
-            qk[0][it] = *reinterpret_cast<const uint2 *>(p.q + off);
-            qk[1][it] = *reinterpret_cast<const uint2 *>(p.k + off);
-        }
-        st_tile(sUt, y0, 1.f);
-        st_tile(sS0, y1, 1.f);
-        st_tile(sT, y2, 1.f);
-#pragma unroll
-        for (int it = 0; it < 2; ++it) {
-            const int idx = tid + it * kCkThreads;
-            *reinterpret_cast<uint4 *>(sW + (idx >> 3) * kLdH + (idx & 7) * 8) = wt[it];
-        }
-#pragma unroll
-        for (int it = 0; it < 4; ++it) {
-            const int e = tid + it * kCkThreads, pc = e >> 6, vv = e & 63;
-            *reinterpret_cast<uint2 *>(sU + vv * kLdH + 4 * pc) =
-                make_uint2(pack_half2(xu[it].x, xu[it].y), pack_half2(xu[it].z, xu[it].w));
-        }
-#pragma unroll
-        for (int it = 0; it < 4; ++it) {                           // bf16 -> fp16 (exact)
-            auto cv = [](uint32_t w) {
-                return pack_half2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
-            };
-            *reinterpret_cast<uint2 *>(sQ + (r0 + 16 * it) * kLdH + c4) = make_uint2(cv(qk[0][it].x), cv(qk[0][it].y));
-            *reinterpret_cast<uint2 *>(sK + (r0 + 16 * it) * kLdH + c4) = make_uint2(cv(qk[1][it].x), cv(qk[1][it].y));
-        }
-    }
-    __syncthreads();
-
-    const float iO = 1.f / scO, iU = 1.f / scU, iS = 1.f / scS;   // powers of two: exact
-    const int row0 = 16 * (warp & 3), n0 = 32 * (warp >> 2);
-    const int iA = row0 + g, iB = iA + 8;                          // this lane's two rows (tokens)
-    const float GA = sG[iA], GB = sG[iB], GC = sG[63];
-    const float gamA = exp_ftz(GA), gamB = exp_ftz(GB), ktA = exp_ftz(GC - GA), ktB = exp_ftz(GC - GB);
-    const float btA = sBt[iA], btB = sBt[iB];
-    float dq[4][4], dk[4][4], dv[4][4], acc[4][4];
-    float dGA = 0.f, dGB = 0.f, kapA = 0.f, kapB = 0.f, dbA = 0.f, dbB = 0.f;
-    auto zero = [&]() {
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[nt][e] = 0.f;
-    };
-    // <row of X, row of acc> over this lane's columns, for its two rows
-    auto rowdot = [&](const __half *X, float &sA, float &sB) {
-        sA = 0.f; sB = 0.f;
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            const float2 xa = __half22float2(*reinterpret_cast<const __half2 *>(X + iA * kLdH + n0 + 8 * nt + 2 * t));
-            const float2 xb = __half22float2(*reinterpret_cast<const __half2 *>(X + iB * kLdH + n0 + 8 * nt + 2 * t));
-            sA = fmaf(xa.x, acc[nt][0], fmaf(xa.y, acc[nt][1], sA));
-            sB = fmaf(xb.x, acc[nt][2], fmaf(xb.y, acc[nt][3], sB));
-        }
-    };
-    // acc (scaled per row) -> a staged tile
-    auto put = [&](__half *X, float fA, float fB) {
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            *reinterpret_cast<uint32_t *>(X + iA * kLdH + n0 + 8 * nt + 2 * t) = pack_half2(fA * acc[nt][0], fA * acc[nt][1]);
-            *reinterpret_cast<uint32_t *>(X + iB * kLdH + n0 + 8 * nt + 2 * t) = pack_half2(fB * acc[nt][2], fB * acc[nt][3]);
-        }
-    };
-    // dst += (fA | fB) acc
-    auto fold = [&](float (&dst)[4][4], float fA, float fB, bool init) {
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            dst[nt][0] = fmaf(fA, acc[nt][0], init ? 0.f : dst[nt][0]);
-            dst[nt][1] = fmaf(fA, acc[nt][1], init ? 0.f : dst[nt][1]);
-            dst[nt][2] = fmaf(fB, acc[nt][2], init ? 0.f : dst[nt][2]);
-            dst[nt][3] = fmaf(fB, acc[nt][3], init ? 0.f : dst[nt][3]);
-        }
-    };
-    float sA, sB;
-
-    // ---- dQg = dO S0^T ----
-    zero();
-    mma64<false, true>(sDO, sS0, row0, n0, lane, acc);
-    rowdot(sQ, sA, sB);
-    dGA = fmaf(iO * p.scale_la * gamA, sA, dGA); dGB = fmaf(iO * p.scale_la * gamB, sB, dGB);
-    fold(dq, iO * p.scale_la * gamA, iO * p.scale_la * gamB, true);
-    // ---- dW = -dU~ S0^T  -> X ----
-    zero();
-    mma64<false, true>(sDU, sS0, row0, n0, lane, acc);
-    put(sX, -1.f, -1.f);
-    // ---- dK~ = U~ dS1^T ----
-    zero();
-    mma64<false, true>(sUt, sDS1, row0, n0, lane, acc);
-    rowdot(sK, sA, sB);
-    kapA = iS * ktA * sA; kapB = iS * ktB * sB;
-    dGA -= kapA; dGB -= kapB;
-    fold(dk, iS * ktA, iS * ktB, true);
-    // ---- N = dO U~^T;  Ns = scale_la (N . Gamma), j <= i  -> Y ----
-    zero();
-    mma64<false, true>(sDO, sUt, row0, n0, lane, acc);
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int j = n0 + 8 * nt + 2 * t + (e & 1), i = e < 2 ? iA : iB;
-            acc[nt][e] *= p.scale_la * exp_ftz(j <= i ? (e < 2 ? GA : GB) - sG[j] : -INFINITY);   // branch-free mask
-        }
-    put(sY, 1.f, 1.f);
-    __syncthreads();                    // X = dW, Y = Ns; dO, S0, dS1 are free
-
-    // ---- dKb = T^T dW  -> slot of dO ----
-    zero();
-    mma64<true, false>(sT, sX, row0, n0, lane, acc);
-    rowdot(sK, sA, sB);
-    dGA = fmaf(iU * btA * gamA, sA, dGA); dGB = fmaf(iU * btB * gamB, sB, dGB);
-    dbA = fmaf(iU * gamA, sA, dbA); dbB = fmaf(iU * gamB, sB, dbB);
-    fold(dk, iU * btA * gamA, iU * btB * gamB, false);
-    put(sDO, 1.f, 1.f);
-    // ---- dVb = T^T dU~  -> slot of S0 ----
-    zero();
-    mma64<true, false>(sT, sDU, row0, n0, lane, acc);
-    {   // <v, dVb>: v straight from global memory
-        sA = 0.f; sB = 0.f;
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            const float2 xa = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(
-                p.v + tok0 + (size_t)iA * ts + n0 + 8 * nt + 2 * t));
-            const float2 xb = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(
-                p.v + tok0 + (size_t)iB * ts + n0 + 8 * nt + 2 * t));
-            sA = fmaf(xa.x, acc[nt][0], fmaf(xa.y, acc[nt][1], sA));
-            sB = fmaf(xb.x, acc[nt][2], fmaf(xb.y, acc[nt][3], sB));
-        }
-    }
-    dbA = fmaf(iU, sA, dbA); dbB = fmaf(iU, sB, dbB);
-    fold(dv, iU * btA, iU * btB, true);
-    put(sS0, 1.f, 1.f);
-    __syncthreads();                    // dKb, dVb in place; T, X, dU~ are free
-
-    // ---- M = -(dKb W^T + dVb U^T);  Mg = M . Gamma, j < i -> X;  Ms = diag(beta~) Mg -> slot of T ----
-    zero();
-    mma64<false, false>(sDO, sW, row0, n0, lane, acc);      // sW, sU hold W^T, U^T: [k][n] operands
-    mma64<false, false>(sS0, sU, row0, n0, lane, acc);
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int j = n0 + 8 * nt + 2 * t + (e & 1), i = e < 2 ? iA : iB;
-            acc[nt][e] *= -exp_ftz(j < i ? (e < 2 ? GA : GB) - sG[j] : -INFINITY);
-        }
-    put(sX, 1.f, 1.f);
-    put(sT, btA, btB);
-    __syncthreads();
-
-    // ---- beta~ Mg K ----
-    zero();
-    mma64<false, false>(sX, sK, row0, n0, lane, acc);
-    rowdot(sK, sA, sB);
-    dGA = fmaf(iU * btA, sA, dGA); dGB = fmaf(iU * btB, sB, dGB);
-    dbA = fmaf(iU, sA, dbA); dbB = fmaf(iU, sB, dbB);
-    fold(dk, iU * btA, iU * btB, false);
-    // ---- Ms^T K ----
-    zero();
-    mma64<true, false>(sT, sK, row0, n0, lane, acc);
-    rowdot(sK, sA, sB);
-    dGA = fmaf(-iU, sA, dGA); dGB = fmaf(-iU, sB, dGB);
-    fold(dk, iU, iU, false);
-    // ---- Ns K ----
-    zero();
-    mma64<false, false>(sY, sK, row0, n0, lane, acc);
-    rowdot(sQ, sA, sB);
-    dGA = fmaf(iO, sA, dGA); dGB = fmaf(iO, sB, dGB);
-    fold(dq, iO, iO, false);
-    // ---- Ns^T Q ----
-    zero();
-    mma64<true, false>(sY, sQ, row0, n0, lane, acc);
-    rowdot(sK, sA, sB);
-    dGA = fmaf(-iO, sA, dGA); dGB = fmaf(-iO, sB, dGB);
-    fold(dk, iO, iO, false);
-
-    // ---- per-token sums: over the 4 lanes of a row, then over the two column halves ----
-    auto quad = [](float x) {
-        x += __shfl_xor_sync(0xffffffffu, x, 1);
-        return x + __shfl_xor_sync(0xffffffffu, x, 2);
-    };
-    dGA = quad(dGA); dGB = quad(dGB); kapA = quad(kapA); kapB = quad(kapB); dbA = quad(dbA); dbB = quad(dbB);
-    if (t == 0) {
-        atomicAdd(rG + iA, dGA); atomicAdd(rG + iB, dGB);
-        atomicAdd(rK + iA, kapA); atomicAdd(rK + iB, kapB);
-        atomicAdd(rB + iA, dbA); atomicAdd(rB + iB, dbB);
-    }
-    // ---- dq, dk, dv: through fp32 tiles in the (now free) operand slots, so that every global
-    // access of the epilogue is a contiguous 64-byte piece of a row instead of a scattered pair ----
-    constexpr int kLdF = 68;                                       // row stride of the fp32 tiles
-    float *fDQ = reinterpret_cast<float *>(smraw), *fDK = fDQ + 64 * kLdF, *fDV = fDK + 64 * kLdF;
-    static_assert(3 * 64 * kLdF * 4 <= 6 * kTileH * 2, "the three result tiles must fit in the first six slots");
-    const int er = tid >> 2, ec = (tid & 3) * 16;                  // epilogue: row, first of 16 columns
-    const size_t eoff = tok0 + (size_t)er * ts + ec;
-    float4 dqs[4];                                                 // softmax-branch dq, on its way early
-#pragma unroll
-    for (int x = 0; x < 4; ++x) dqs[x] = *reinterpret_cast<const float4 *>(p.dq_sm + eoff + 4 * x);
-    const bool lin = kBlock || p.route[((size_t)b * p.L + (size_t)c * kC + er) * p.H + h] == 0;
-
-    __syncthreads();                                               // all products have read their operands
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-        const int cc = n0 + 8 * nt + 2 * t;
-        *reinterpret_cast<float2 *>(fDQ + iA * kLdF + cc) = make_float2(dq[nt][0], dq[nt][1]);
-        *reinterpret_cast<float2 *>(fDQ + iB * kLdF + cc) = make_float2(dq[nt][2], dq[nt][3]);
-        *reinterpret_cast<float2 *>(fDK + iA * kLdF + cc) = make_float2(dk[nt][0], dk[nt][1]);
-        *reinterpret_cast<float2 *>(fDK + iB * kLdF + cc) = make_float2(dk[nt][2], dk[nt][3]);
-        *reinterpret_cast<float2 *>(fDV + iA * kLdF + cc) = make_float2(dv[nt][0], dv[nt][1]);
-        *reinterpret_cast<float2 *>(fDV + iB * kLdF + cc) = make_float2(dv[nt][2], dv[nt][3]);
-    }
-    __syncthreads();
-    {
-        // add: values already in registers; gadd: fp32 token-major tensor read here (block routing)
-        auto row16 = [&](const float *tile, const float4 *add, const float *gadd, __nv_bfloat16 *dst) {
-            uint32_t o[8];
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                float4 v4 = *reinterpret_cast<const float4 *>(tile + er * kLdF + ec + 4 * x);
-                if (add) { v4.x += add[x].x; v4.y += add[x].y; v4.z += add[x].z; v4.w += add[x].w; }
-                if (gadd) {
-                    const float4 y = *reinterpret_cast<const float4 *>(gadd + eoff + 4 * x);
-                    v4.x += y.x; v4.y += y.y; v4.z += y.z; v4.w += y.w;
-                }
-                o[2 * x] = pack_bf162(v4.x, v4.y);
-                o[2 * x + 1] = pack_bf162(v4.z, v4.w);
-            }
-            uint4 *d4 = reinterpret_cast<uint4 *>(dst + eoff);
-            d4[0] = make_uint4(o[0], o[1], o[2], o[3]);
-            d4[1] = make_uint4(o[4], o[5], o[6], o[7]);
-        };
-        row16(fDQ, dqs, nullptr, p.dq);
-        if (lin) {
-            row16(fDK, nullptr, kBlock ? p.dk_x : nullptr, p.dk);
-            row16(fDV, nullptr, kBlock ? p.dv_x : nullptr, p.dv);
-        }
-    }
-    __syncthreads();
-    if (tid < 64) {
-        // dg_j = sum_{i >= j} dG_i + sum_i kappa_i + gamma_C <dS1, S0>  (i, j: tokens of the chunk)
-        float suf = rG[tid], kap = rK[tid];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const float y = __shfl_down_sync(0xffffffffu, suf, o);
-            if (lane + o < 32) suf += y;
-        }
-        kap = warp_sum(kap);
-        if (lane == 0) { sMax[32 + warp] = suf; sMax[34 + warp] = kap; }
-        named_barrier_sync(1, 64);
-        float gs = 0.f;
-#pragma unroll
-        for (int wv = 0; wv < 8; ++wv) gs += sMax[24 + wv];
-        const float extra = sMax[34] + sMax[35] + exp_ftz(sG[63]) * gs + (warp == 0 ? sMax[33] : 0.f);
-        if (kBlock && p.kap_c && tid == 0) p.kap_c[chunk] = sMax[34] + sMax[35];
-        const size_t tk = ((size_t)b * p.L + (size_t)c * kC + tid) * p.H + h;
-        p.dg[tk] = suf + extra;
-        p.dbeta[tk] = !kBlock && p.route[tk] ? 0.f : rB[tid];
-    }
-}
-
 // ------------------------------------------------------------------------------------------
 // Backward of the softmax branch through a query's own block under block-level routing
 // (Section 4.1: both operations compute the inner-chunk correlations; Section 4.2: ds = p (dp -
 // <do, o>)).  A query in a linear block reads, besides the retained tokens of earlier softmax
 // blocks (the kernels over the compacted K/V handle those), the causal part of its own block of
 // 64 tokens.  One CTA per linear block adds that part, five 64 x 64 x 64 products on the
-// warp-level tensor-core path of the chunk kernel above (fp16 tiles, fp32 accumulation):
+// warp-level tensor-core path (fp16 tiles, fp32 accumulation):
 //   S = Q K^T, dP = dO V^T;  p_ij = exp(scale s_ij - lse_i), ds_ij = scale p_ij (dp_ij - D_i), j <= i
 //   dq += dS K  (added to the query-side result of the compacted kernels)
 //   dk  = dS^T Q,  dv = P^T dO  (written: the tokens of a linear block have no other
@@ -723,15 +308,15 @@ __global__ void __launch_bounds__(kCkThreads, 2) gdn_bwd_chunk_kernel(ChunkBwdAr
 // with lse_i and D_i = <do_i, o_i> of the whole softmax row.  Softmax heads of 64 KB columns: KB = 1 for
 // d = 64 or kG = 2 heads per linear head of d = 128 (Section 4.3; the head is then a column slice of rows
 // of 128 columns, lse / Dsm are [B,H,kG,L]), KB = 2 for d = 128 (two tiles per operand: the logit products
-// add over them, the three results are formed half by half).  kNormSrc: q and k come from the fp32 copies
-// that hold the softmax operation's normalised rows (qn, kn) instead of the bf16 inputs.
+// add over them, the three results are formed half by half).  kNormSrc: q and k come from the fp16 copies
+// [B,H,L,DL] that hold the softmax operation's normalised rows (qn, kn) instead of the bf16 inputs.
 template <int KB> constexpr int own_smem() { return (4 * KB + 2) * kTileH * 2; }
 
 template <int kG, bool kNormSrc, int KB>
 __global__ void __launch_bounds__(kCkThreads, KB == 1 ? 3 : 2)
 softmax_bwd_own_block_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfloat16 *__restrict__ k,
-                             const __nv_bfloat16 *__restrict__ v, const float *__restrict__ qn,
-                             const float *__restrict__ kn, const __half *__restrict__ do16,
+                             const __nv_bfloat16 *__restrict__ v, const __half *__restrict__ qn,
+                             const __half *__restrict__ kn, const __half *__restrict__ do16,
                              const float *__restrict__ lse, const float *__restrict__ Dsm,
                              const uint8_t *__restrict__ route, float scale_sm,
                              float *__restrict__ dq_sm, float *__restrict__ dk_x,
@@ -759,11 +344,11 @@ softmax_bwd_own_block_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfl
             const int r = r0 + 16 * it, tl = kb * kTileH + r * kLdH + c4;
             const size_t off = tok0 + (size_t)r * ts + kb * 64 + c4;
             const uint2 xv = *reinterpret_cast<const uint2 *>(v + off);
-            const uint2 xo = *reinterpret_cast<const uint2 *>(do16 + ((size_t)bh * L + (size_t)c * kC + r) * DL + col0 + kb * 64 + c4);
+            const size_t offh = ((size_t)bh * L + (size_t)c * kC + r) * DL + col0 + kb * 64 + c4;      // [B,H,L,DL]
+            const uint2 xo = *reinterpret_cast<const uint2 *>(do16 + offh);
             if (kNormSrc) {
-                const float4 fq = *reinterpret_cast<const float4 *>(qn + off), fk = *reinterpret_cast<const float4 *>(kn + off);
-                *reinterpret_cast<uint2 *>(sQ + tl) = make_uint2(pack_half2(fq.x, fq.y), pack_half2(fq.z, fq.w));
-                *reinterpret_cast<uint2 *>(sK + tl) = make_uint2(pack_half2(fk.x, fk.y), pack_half2(fk.z, fk.w));
+                *reinterpret_cast<uint2 *>(sQ + tl) = *reinterpret_cast<const uint2 *>(qn + offh);
+                *reinterpret_cast<uint2 *>(sK + tl) = *reinterpret_cast<const uint2 *>(kn + offh);
             } else {
                 const uint2 xq = *reinterpret_cast<const uint2 *>(q + off), xk = *reinterpret_cast<const uint2 *>(k + off);
                 *reinterpret_cast<uint2 *>(sQ + tl) = make_uint2(cv(xq.x), cv(xq.y));
@@ -846,62 +431,29 @@ softmax_bwd_own_block_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfl
 }  // namespace
 
 template <int D>
-static cudaError_t rscan_tc_impl(const void *dO16, const void *dOg16, const GdnTcWs &ws,
-                                 const float *S_c, float *dUt, float *dS_c, float *gS,
-                                 const float *dstate_out, float *dstate_in,
+static cudaError_t rscan_tc_impl(const GdnTcWs &ws, const GdnTcGrads &gr, const float *dstate_out, float *dstate_in,
                                  const uint8_t *block_route, int32_t *status, Shape s, cudaStream_t st) {
     const int NC = s.L / kC;
     const uint64_t BH = (uint64_t)s.B * s.H;
     CUtensorMap mdo, mdog, mqh, mkh, mwt, mph;
-    if (!tch::make_map_2d(&mdo, dO16, BH * s.L, D, 64) || !tch::make_map_2d(&mdog, dOg16, BH * s.L, D, 64) ||
+    if (!tch::make_map_2d(&mdo, gr.dO16, BH * s.L, D, 64) || !tch::make_map_2d(&mdog, gr.dOg16, BH * s.L, D, 64) ||
         !tch::make_map_2d(&mqh, ws.Qh, BH * s.L, D, 64) || !tch::make_map_2d(&mkh, ws.Kh, BH * s.L, D, 64) ||
         !tch::make_map_2d(&mwt, ws.Wt, BH * NC * D, 64, D) || !tch::make_map_2d(&mph, ws.Ph, BH * NC * 64, 64, 64))
         return cudaErrorInvalidValue;
     auto kernel = block_route ? gdn_rscan_tc_kernel<D, true> : gdn_rscan_tc_kernel<D, false>;
-    cudaError_t e = allow_smem(kernel,
-                                         RsLayout<D>::kTotal);
+    cudaError_t e = allow_smem(kernel, RsLayout<D>::kTotal);
     if (e != cudaSuccess) return e;
     kernel<<<s.B * s.H, kRsThreads, RsLayout<D>::kTotal, st>>>(
-        mdo, mdog, mqh, mkh, mwt, mph, ws.Gd, dUt, dS_c, dstate_out, dstate_in, block_route, status, s.L, s.H,
-        debug_wait_kcycles());
+        mdo, mdog, mqh, mkh, mwt, mph, ws.Gd, (__half *)gr.dU16, (__half *)gr.dS16, dstate_out, dstate_in, block_route,
+        status, s.L, s.H, debug_wait_kcycles());
     count_launch();
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (gS) {     // (the fused chunk kernel forms <dS1, S0> itself)
-        state_dot_kernel<<<(unsigned)(BH * NC), 256, 0, st>>>(dS_c, S_c, gS, D / 32, D * D, block_route, s.L, s.H);
-        count_launch();
-    }
     return cudaGetLastError();
 }
 
-cudaError_t launch_gdn_rscan_tc(const void *dO16, const void *dOg16, const GdnTcWs &ws,
-                                const float *S_c, float *dUt, float *dS_c, float *gS,
-                                const float *dstate_out, float *dstate_in,
+cudaError_t launch_gdn_rscan_tc(const GdnTcWs &ws, const GdnTcGrads &gr, const float *dstate_out, float *dstate_in,
                                 const uint8_t *block_route, int32_t *status, Shape s, cudaStream_t st) {
-    if (s.d == 128)
-        return rscan_tc_impl<128>(dO16, dOg16, ws, S_c, dUt, dS_c, gS, dstate_out, dstate_in, block_route, status, s, st);
-    return rscan_tc_impl<64>(dO16, dOg16, ws, S_c, dUt, dS_c, gS, dstate_out, dstate_in, block_route, status, s, st);
-}
-
-
-cudaError_t launch_gdn_bwd_chunk(const void *q, const void *k, const void *v, const float *dO,
-                                 const float *dUt, const float *Ut, const float *S_c, const float *dS_c,
-                                 const float *Tinv, const void *Wt, const float *Up, const float *Gcum,
-                                 const float *beta, const uint8_t *route, const float *dq_sm,
-                                 float scale_la, void *dq, void *dk, void *dv, float *dg,
-                                 float *dbeta, bool block, const float *dk_x, const float *dv_x,
-                                 float *kap_c, Shape s, cudaStream_t st) {
-    if (s.d != 64 || !s.bf16) return cudaErrorInvalidValue;
-    auto kernel = block ? gdn_bwd_chunk_kernel<true> : gdn_bwd_chunk_kernel<false>;
-    cudaError_t e = allow_smem(kernel,
-                                         kCkSmem);
-    if (e != cudaSuccess) return e;
-    ChunkBwdArgs a{(const __nv_bfloat16 *)q, (const __nv_bfloat16 *)k, (const __nv_bfloat16 *)v, dO, dUt, Ut,
-                   S_c, dS_c, Tinv, Up, Gcum, beta, dq_sm, (const __half *)Wt, route, scale_la, (__nv_bfloat16 *)dq,
-                   (__nv_bfloat16 *)dk, (__nv_bfloat16 *)dv, dg, dbeta, s.L, s.H, dk_x, dv_x, kap_c};
-    dim3 grid(s.L / kC, s.B * s.H);
-    kernel<<<grid, kCkThreads, kCkSmem, st>>>(a);
-    count_launch();
-    return cudaGetLastError();
+    if (s.d == 128) return rscan_tc_impl<128>(ws, gr, dstate_out, dstate_in, block_route, status, s, st);
+    return rscan_tc_impl<64>(ws, gr, dstate_out, dstate_in, block_route, status, s, st);
 }
 
 // d score per block and head (Section 4.2), for the active operation only: a softmax block sums the
@@ -951,7 +503,7 @@ cudaError_t launch_softmax_bwd_own_block(const void *q, const void *k, const voi
                                          const void *do16, const float *lse, const float *Dsm,
                                          const uint8_t *route, float scale_sm, float *dq_sm,
                                          float *dk_x, float *dv_x, const int32_t *gsc, Shape s,
-                                         cudaStream_t st, int G, const float *qn, const float *kn) {
+                                         cudaStream_t st, int G, const void *qn, const void *kn) {
     if (!s.bf16 || !((s.d == 64 && G <= 1) || (s.d == 128 && G <= 2))) return cudaErrorInvalidValue;
     auto kernel = softmax_bwd_own_block_kernel<1, false, 1>;
     int smem = own_smem<1>();
@@ -965,7 +517,8 @@ cudaError_t launch_softmax_bwd_own_block(const void *q, const void *k, const voi
     if (e != cudaSuccess) return e;
     dim3 grid(s.L / kC, s.B * s.H * (G == 2 ? 2 : 1));
     kernel<<<grid, kCkThreads, smem, st>>>(
-        (const __nv_bfloat16 *)q, (const __nv_bfloat16 *)k, (const __nv_bfloat16 *)v, qn, kn, (const __half *)do16,
+        (const __nv_bfloat16 *)q, (const __nv_bfloat16 *)k, (const __nv_bfloat16 *)v, (const __half *)qn,
+        (const __half *)kn, (const __half *)do16,
         lse, Dsm, route, scale_sm, dq_sm, dk_x, dv_x, gsc, s.L, s.H);
     count_launch();
     return cudaGetLastError();

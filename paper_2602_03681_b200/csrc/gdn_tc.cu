@@ -281,11 +281,6 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                     }
                     prow[pc] = make_uint4(pack_half2(x[0], x[1]), pack_half2(x[2], x[3]),
                                           pack_half2(x[4], x[5]), pack_half2(x[6], x[7]));
-                    if (ex.P) {
-                        float4 *pf = reinterpret_cast<float4 *>(ex.P + (chunk * 64 + i) * 64 + 8 * pc);
-                        pf[0] = make_float4(x[0], x[1], x[2], x[3]);
-                        pf[1] = make_float4(x[4], x[5], x[6], x[7]);
-                    }
                 }
                 tc_fence_before_sync();
                 mbar_arrive(&ms.barT);
@@ -412,14 +407,14 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                 }
                 named_barrier_sync(2, 64);                  // both tiles have been read: reuse them
                 // ---- operands T diag(beta~) (xLo) and T diag(beta~ gamma) (xHi), fp16 K-major rows ----
-                float *Trow = ex.T ? ex.T + chunk * 4096 : nullptr;
+                __half *T16 = ex.T16 ? reinterpret_cast<__half *>(ex.T16) + chunk * 4096 : nullptr;   // [8][64][8]
                 auto put2 = [&](int row, int col, float v0, float v1) {
                     const float2 fb = *reinterpret_cast<const float2 *>(&ms.bt[col]);
                     const float2 fg = *reinterpret_cast<const float2 *>(&ms.btg[col]);
                     const uint32_t off = sw128_offset(row, col >> 3) + (col & 7) * 2;
                     *reinterpret_cast<uint32_t *>(xLo + off) = pack_half2(v0 * fb.x, v1 * fb.y);
                     *reinterpret_cast<uint32_t *>(xHi + off) = pack_half2(v0 * fg.x, v1 * fg.y);
-                    if (Trow) *reinterpret_cast<float2 *>(Trow + row * 64 + col) = make_float2(v0, v1);
+                    if (T16) *reinterpret_cast<uint32_t *>(T16 + ((col >> 3) * 64 + row) * 8 + (col & 7)) = pack_half2(v0, v1);
                 };
 #pragma unroll
                 for (int nt = 0; nt < 2; ++nt) {
@@ -445,19 +440,15 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                     *reinterpret_cast<uint4 *>(xHi + sw128_offset(i, 2 * bk + hp)) =
                         make_uint4(pack_half2(xg[0], xg[1]), pack_half2(xg[2], xg[3]),
                                    pack_half2(xg[4], xg[5]), pack_half2(xg[6], xg[7]));
-                    if (Trow) {
-                        float4 *tr = reinterpret_cast<float4 *>(Trow + i * 64 + 16 * bk + 8 * hp);
-                        tr[0] = make_float4(td[8 * hp], td[8 * hp + 1], td[8 * hp + 2], td[8 * hp + 3]);
-                        tr[1] = make_float4(td[8 * hp + 4], td[8 * hp + 5], td[8 * hp + 6], td[8 * hp + 7]);
-                    }
+                    if (T16)
+                        *reinterpret_cast<uint4 *>(T16 + ((2 * bk + hp) * 64 + i) * 8) =
+                            make_uint4(pack_half2(td[8 * hp], td[8 * hp + 1]), pack_half2(td[8 * hp + 2], td[8 * hp + 3]),
+                                       pack_half2(td[8 * hp + 4], td[8 * hp + 5]), pack_half2(td[8 * hp + 6], td[8 * hp + 7]));
                 }
                 for (int pc = 2 * bk + 2; pc < 8; ++pc) {   // right of the diagonal block: zero
                     *reinterpret_cast<uint4 *>(xLo + sw128_offset(i, pc)) = make_uint4(0, 0, 0, 0);
                     *reinterpret_cast<uint4 *>(xHi + sw128_offset(i, pc)) = make_uint4(0, 0, 0, 0);
-                    if (Trow) {
-                        float4 *tr = reinterpret_cast<float4 *>(Trow + i * 64 + 8 * pc);
-                        tr[0] = tr[1] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    }
+                    if (T16) *reinterpret_cast<uint4 *>(T16 + (pc * 64 + i) * 8) = make_uint4(0, 0, 0, 0);
                 }
                 fence_proxy_async_smem();
                 mbar_arrive(&ms.barT);
@@ -481,21 +472,22 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                 for (int pc = 0; pc < 16; ++pc)
                     dst[pc * D] = make_uint4(x[pc >> 3][(4 * pc) & 31], x[pc >> 3][(4 * pc + 1) & 31],
                                              x[pc >> 3][(4 * pc + 2) & 31], x[pc >> 3][(4 * pc + 3) & 31]);
-                if (ex.U) {      // token-major fp32 copy
-                    float *uf = ex.U + (((size_t)b * L + tok0) * H + h) * D + row;
+                if (ex.U16) {    // fp16 copy for the backward, in the layout of W^T
+                    uint4 *uh = reinterpret_cast<uint4 *>(reinterpret_cast<__half *>(ex.U16) + (chunk * D + row) * 64);
 #pragma unroll
-                    for (int j = 0; j < 64; ++j) uf[(size_t)j * H * D] = __uint_as_float(x[j >> 5][j & 31]);
+                    for (int pc = 0; pc < 8; ++pc) {
+                        const uint32_t *xx = &x[pc >> 2][(8 * pc) & 31];
+                        uh[pc] = make_uint4(pack_half2(__uint_as_float(xx[0]), __uint_as_float(xx[1])),
+                                            pack_half2(__uint_as_float(xx[2]), __uint_as_float(xx[3])),
+                                            pack_half2(__uint_as_float(xx[4]), __uint_as_float(xx[5])),
+                                            pack_half2(__uint_as_float(xx[6]), __uint_as_float(xx[7])));
+                    }
                 }
             }
             if (do_w) {
                 tmem_ld32(tmem + lane_base + 64, x[0]);
                 tmem_ld32(tmem + lane_base + 96, x[1]);
                 tmem_wait_ld();
-                if (ex.W) {
-                    float *wf = ex.W + (((size_t)b * L + tok0) * H + h) * D + row;
-#pragma unroll
-                    for (int j = 0; j < 64; ++j) wf[(size_t)j * H * D] = __uint_as_float(x[j >> 5][j & 31]);
-                }
                 uint4 *dst = reinterpret_cast<uint4 *>(Wt + (chunk * D + row) * 64);
 #pragma unroll
                 for (int pc = 0; pc < 8; ++pc) {
@@ -825,8 +817,9 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
                 tc_fence_before_sync();
             }
             // ---- (a) state row -> fp16 operand in TMEM; decay the register copy afterwards ----
+            uint32_t spk[kHalfCols / 2];
             {
-                uint32_t pk[kHalfCols / 2];
+                uint32_t (&pk)[kHalfCols / 2] = spk;
 #pragma unroll
                 for (int x = 0; x < kHalfCols / 2; ++x) pk[x] = pack_half2(S[2 * x], S[2 * x + 1]);
                 if (kHalfCols == 64)
@@ -840,10 +833,11 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
             tc_fence_before_sync();
             mbar_arrive(&ms.barA);
             // (exports for the backward go behind the arrivals, off the chain between the chunks)
-            if (ex.S_c && active) {      // chunk-entry state, [B,H,L/C,dk,dv]
-                float *sc = ex.S_c + (((size_t)bh * NC + c0 + c) * D + col0) * D + r;
+            if (ex.S16 && active) {      // chunk-entry state: the operand itself, in pieces of keys
+                uint4 *sc = reinterpret_cast<uint4 *>(ex.S16) + (((size_t)bh * NC + c0 + c) * (D / 8) + col0 / 8) * D + r;
 #pragma unroll
-                for (int x = 0; x < kHalfCols; ++x) sc[(size_t)x * D] = S[x];
+                for (int x = 0; x < kHalfCols / 8; ++x)
+                    sc[(size_t)x * D] = make_uint4(spk[4 * x], spk[4 * x + 1], spk[4 * x + 2], spk[4 * x + 3]);
             }
             float u[32];                                   // from L2; lands while W S is computed
             if (active && !zero_u) {
@@ -868,8 +862,9 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
 #pragma unroll
                 for (int j = 0; j < 32; ++j) u[j] -= __uint_as_float(ws[j]);
             }
+            uint32_t upk[32];
             {
-                uint32_t pk[32];     // [0,16): U~ of this thread's 32 tokens, [16,32): U~ gamma_C/gamma
+                uint32_t (&pk)[32] = upk;     // [0,16): U~ of this thread's 32 tokens, [16,32): U~ gamma_C/gamma
 #pragma unroll
                 for (int x = 0; x < 16; ++x) {
                     pk[x] = pack_half2(u[2 * x], u[2 * x + 1]);
@@ -882,10 +877,11 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
             }
             tc_fence_before_sync();
             mbar_arrive(&ms.barB);
-            if (ex.Ut && active) {       // U~, token-major
-                float *ut = ex.Ut + (((size_t)b * L + (size_t)(c0 + c) * 64 + tk0) * H + h) * D + r;
+            if (ex.Ut16 && active) {     // U~: the operand itself, in pieces of tokens
+                uint4 *ut = reinterpret_cast<uint4 *>(ex.Ut16) + (((size_t)bh * NC + c0 + c) * 8 + tk0 / 8) * D + r;
 #pragma unroll
-                for (int j = 0; j < 32; ++j) ut[(size_t)j * H * D] = u[j];
+                for (int x = 0; x < 4; ++x)
+                    ut[(size_t)x * D] = make_uint4(upk[4 * x], upk[4 * x + 1], upk[4 * x + 2], upk[4 * x + 3]);
             }
             // ---- behind the MMAs just released: next U row towards L2, previous chunk's output ----
             if (c + 1 < ncs) prefetch_u(c + 1);

@@ -124,6 +124,8 @@ cudaError_t launch_softmax_bwd_tc(const void *q, void *Qh, const void *dO16, con
                                   HeadGroups hg = HeadGroups{});
 // (hg.G = 2 at d = 128: softmax heads are column slices, lse / Dsm [B,H,G,L]; hg.norm_eps >= 0: Qh is
 // written here as the slice-wise RMS-normalised q, k16 must hold the normalised keys already)
+// bf16 [B,L,H,d] -> fp16 [B,H,L,d], slice-wise RMS-normalised when hg.norm_eps >= 0 (the softmax operation's q, k)
+cudaError_t launch_to_f16_bhld(const void *x, void *xh, Shape s, HeadGroups hg, cudaStream_t st);
 
 // gdn_tc.cu -- tensor-core chunkwise Gated DeltaNet (bf16 storage): intermediates in workspace
 struct GdnTcWs {
@@ -133,14 +135,21 @@ struct GdnTcWs {
     void *Ph;        // P per chunk, fp16                [B,H,L/C,64,64]
     float *Gd;       // per chunk: gamma_i (64), gamma_C / gamma_i (64), fp32   [B,H,L/C,128]
 };
-// Optional fp32 copies of the chunkwise quantities the backward needs (all may be null).
+// The chunkwise quantities the backward needs (all may be null), as fp16 -- what the forward's own MMA operands were
+// -- in the layout the backward's fragments are loaded from.  "Pieces": a transposed tile cut into 16-byte pieces
+// of 8 elements along the second index, all rows of a piece contiguous, [pieces][rows][8].
 struct GdnTcExport {
-    float *W, *U;    // token-major [B,L,H,d]
-    float *P;        // [B,H,L/C,64,64]
-    float *T;        // (I + A)^-1, [B,H,L/C,64,64]
+    void *U16;       // U^T, fp16 [B,H,L/C,d,64] (like W^T)
+    void *T16;       // (I + A)^-1 as pieces of columns   [B,H,L/C,8,64,8]
     float *Gcum;     // in-chunk cumulative log decay [B,H,L]
-    float *S_c;      // chunk-entry states [B,H,L/C,d,d]
-    float *Ut;       // U~ = U - W S, token-major [B,L,H,d]
+    void *S16;       // chunk-entry states S0: value row, pieces of keys   [B,H,L/C,d/8,d,8]
+    void *Ut16;      // U~ = U - W S: value row, pieces of tokens   [B,H,L/C,8,d,8]
+};
+// Gradient operands between the combination's backward, the reverse scan and the chunk kernel, in units of the
+// gradient scale: dO16 [B,H,L,d] = gradient of the linear read-out, dOg16 = scale_la gamma times it, and the
+// reverse scan's dU16 (pieces like Ut16) and dS16 (chunk-exit gradients, pieces like S16).
+struct GdnTcGrads {
+    void *dO16, *dOg16, *dU16, *dS16;
 };
 // norm_eps >= 0: q and k rows are L2-normalised as the tiles are converted (Section 4.3, HeadGroups)
 cudaError_t launch_gdn_prepare_tc(const void *q, const void *k, const void *v, const float *g,
@@ -225,12 +234,18 @@ cudaError_t launch_gdn_rscan(const float *q32, const float *k32, const float *Gc
                              float scale_la, float *dUt, float *dS_c, float *gS,
                              const float *dstate_out, float *dstate_in, Shape s, cudaStream_t st,
                              const uint8_t *block_route = nullptr);
-// Tensor-core reverse scan (gdn_bwd_tc.cu): dO16 / dOg16 are fp16 [B,H,L,d] copies of the read-out
-// gradient and of scale_la gamma times it; outputs as launch_gdn_rscan (gS: slot 0 of each row).
-cudaError_t launch_gdn_rscan_tc(const void *dO16, const void *dOg16, const GdnTcWs &ws,
-                                const float *S_c, float *dUt, float *dS_c, float *gS,
-                                const float *dstate_out, float *dstate_in,
+// Tensor-core reverse scan (gdn_bwd_tc.cu): reads gr.dO16, gr.dOg16, writes gr.dU16, gr.dS16
+cudaError_t launch_gdn_rscan_tc(const GdnTcWs &ws, const GdnTcGrads &gr, const float *dstate_out, float *dstate_in,
                                 const uint8_t *block_route, int32_t *status, Shape s, cudaStream_t st);
+// gdn_chunk_bwd_tc.cu: everything of the linear branch's backward that follows the reverse scan, fused per chunk
+// (bf16 storage): dq (dq_sm added unless nullptr), dk, dv of the linear tokens -- or, with block-level routing, of
+// every token, dk_x / dv_x (its softmax-branch part, or nullptr) added --, dg, dbeta and the chunk sums of kappa
+// (kap_c [B,H,L/C] or nullptr).  out_f32: dq, dk, dv as fp32.
+cudaError_t launch_gdn_chunk_bwd(const GdnTcWs &ws, const GdnTcExport &ex, const GdnTcGrads &gr, const void *v,
+                                 const float *beta, const uint8_t *route, const float *dq_sm, float scale_la, void *dq,
+                                 void *dk, void *dv, bool out_f32, float *dg, float *dbeta, bool block,
+                                 const float *dk_x, const float *dv_x, float *kap_c, int32_t *status, Shape s,
+                                 cudaStream_t st);
 cudaError_t launch_gdn_tsolve(const float *Abar, const float *beta, const uint8_t *route,
                               const float *dW, const float *dUt, float *dKb, float *dVb, Shape s,
                               cudaStream_t st);
@@ -254,29 +269,10 @@ struct AssembleArgs {
 // compacted softmax-branch gradients), dbeta, dg.  Three kernels.
 cudaError_t launch_gdn_assemble(const AssembleArgs &a, void *dq, void *dk, void *dv, Shape s,
                                 cudaStream_t st);
-// Tensor-core path (tf32 products), one kernel per chunk: dKb = Tinv^T dW, dVb = Tinv^T dU~ (written out),
-// M = -strictly_lower(dKb W^T + dVb U^T), N = lower(dO U~^T), then Mg, Ms, Ns as launch_mask_scale forms them.
-cudaError_t launch_gdn_tm(const float *Tinv, const float *dW, const float *dUt, const float *W, const float *U,
-                          const float *dO, const float *Ut, const float *Gcum, const float *beta,
-                          const uint8_t *route, float scale_la, float *dKb, float *dVb, float *Mg, float *Ms,
-                          float *Ns, Shape s, cudaStream_t st);
-// The same with the four products X1 = Mg K, X2 = Ms^T K, X3 = Ns K, X4 = Ns^T Q formed inside (tf32
-// tensor-core products; a.X1p .. a.X4 are not read); s.bf16 says what dq, dk, dv are stored as.
-cudaError_t launch_gdn_xassemble(const AssembleArgs &a, const float *Mg, const float *Ms, const float *Ns,
-                                 void *dq, void *dk, void *dv, Shape s, cudaStream_t st);
 // The last two of those kernels only (dg from the per-token sums, scatter of the retained tokens'
 // dk, dv), for callers that formed dq, dk, dv of the linear tokens and the sums themselves.
 cudaError_t launch_gdn_finish(const AssembleArgs &a, void *dk, void *dv, Shape s, cudaStream_t st,
                               bool with_dg = true);
-// gdn_bwd_tc.cu: everything of the linear branch's backward that follows the reverse scan, fused
-// per chunk (d = 64, bf16 storage): dq (with dq_sm added), dk, dv of the linear tokens, dg, dbeta.
-cudaError_t launch_gdn_bwd_chunk(const void *q, const void *k, const void *v, const float *dO,
-                                 const float *dUt, const float *Ut, const float *S_c, const float *dS_c,
-                                 const float *Tinv, const void *Wt, const float *Up, const float *Gcum,
-                                 const float *beta, const uint8_t *route, const float *dq_sm,
-                                 float scale_la, void *dq, void *dk, void *dv, float *dg,
-                                 float *dbeta, bool block, const float *dk_x, const float *dv_x,
-                                 float *kap_c, Shape s, cudaStream_t st);
 // (kap_c [B,H,L/C]: the chunk sums of kappa, or kappa_tok [B,H,L]: kappa per token, summed here)
 cudaError_t launch_dscore(const uint8_t *route, const int32_t *sm_chunk_prefix, const float *dmask,
                           const float *kap_c, const float *kappa_tok, int cap, float *dscore, Shape s,
@@ -289,10 +285,10 @@ cudaError_t launch_softmax_bwd_own_block(const void *q, const void *k, const voi
                                          const void *do16, const float *lse, const float *Dsm,
                                          const uint8_t *route, float scale_sm, float *dq_sm,
                                          float *dk_x, float *dv_x, const int32_t *gsc, Shape s,
-                                         cudaStream_t st, int G = 1, const float *qn = nullptr,
-                                         const float *kn = nullptr);
-// (softmax heads of 64 columns: d = 64, or G = 2 at d = 128 with lse / Dsm [B,H,G,L]; qn, kn: fp32 copies
-// holding the softmax operation's normalised q, k [B,L,H,d], read instead of q, k)
+                                         cudaStream_t st, int G = 1, const void *qn = nullptr,
+                                         const void *kn = nullptr);
+// (softmax heads of 64 columns: d = 64, or G = 2 at d = 128 with lse / Dsm [B,H,G,L]; qn, kn: fp16 copies
+// [B,H,L,d] holding the softmax operation's normalised q, k, read instead of q, k)
 
 // decode.cu
 // Bytes of workspace of a decode step: status word, per-head tickets, partial softmax results and

@@ -528,6 +528,15 @@ to_f16_bhld_kernel(const __nv_bfloat16 *__restrict__ q, __half *__restrict__ qh,
 
 }  // namespace
 
+cudaError_t launch_to_f16_bhld(const void *x, void *xh, Shape s, HeadGroups hg, cudaStream_t st) {
+    const size_t pieces = (size_t)s.B * s.L * s.H * (s.d / 8);
+    auto kernel = s.d == 128 ? to_f16_bhld_kernel<128> : to_f16_bhld_kernel<64>;
+    kernel<<<(unsigned)((pieces + 255) / 256), 256, 0, st>>>((const __nv_bfloat16 *)x, (__half *)xh, s.B, s.L, s.H, hg.G,
+                                                             hg.norm_eps);
+    count_launch();
+    return cudaGetLastError();
+}
+
 template <int D, int G>      // D: columns of a softmax head, G of them per linear head (s.d = D G)
 static cudaError_t softmax_bwd_tc_impl(const void *q, void *Qh, const void *dO16, const void *k16,
                                        const void *v16, int cap, const int32_t *sm_idx,
@@ -537,12 +546,13 @@ static cudaError_t softmax_bwd_tc_impl(const void *q, void *Qh, const void *dO16
                                        cudaStream_t st, cudaStream_t st_kv, float norm_eps) {
     const uint64_t BH = (uint64_t)s.B * s.H;
     constexpr int DL = D * G;
+    cudaError_t e;
     if (!qh_ready) {      // (the linear branch's prepare kernel leaves the same fp16 copy of q behind --
                           //  unless q is normalised, differently for the two operations)
-        const size_t pieces = (size_t)s.B * s.L * s.H * (DL / 8);
-        to_f16_bhld_kernel<DL><<<(unsigned)((pieces + 255) / 256), 256, 0, st>>>(
-            (const __nv_bfloat16 *)q, (__half *)Qh, s.B, s.L, s.H, G, norm_eps);
-        count_launch();
+        HeadGroups hg;
+        hg.G = G;
+        hg.norm_eps = norm_eps;
+        if ((e = launch_to_f16_bhld(q, Qh, s, hg, st)) != cudaSuccess) return e;
     }
     CUtensorMap mq128, mdo128, mk64, mv64, mq64, mdo64, mk128, mv128;
     if (!tch::make_map_2d(&mq128, Qh, BH * s.L, DL, 128) || !tch::make_map_2d(&mdo128, dO16, BH * s.L, DL, 128) ||
@@ -550,7 +560,7 @@ static cudaError_t softmax_bwd_tc_impl(const void *q, void *Qh, const void *dO16
         !tch::make_map_2d(&mq64, Qh, BH * s.L, DL, 64) || !tch::make_map_2d(&mdo64, dO16, BH * s.L, DL, 64) ||
         !tch::make_map_2d(&mk128, k16, BH * cap, DL, 128) || !tch::make_map_2d(&mv128, v16, BH * cap, DL, 128))
         return cudaErrorInvalidValue;
-    cudaError_t e = allow_smem(softmax_bwd_dq_tc_kernel<D, G>, QLayout<D>::kTotal);
+    e = allow_smem(softmax_bwd_dq_tc_kernel<D, G>, QLayout<D>::kTotal);
     if (e != cudaSuccess) return e;
     auto dkv = dmask ? softmax_bwd_dkv_tc_kernel<D, true, G> : softmax_bwd_dkv_tc_kernel<D, false, G>;
     e = allow_smem(dkv, KLayout<D>::kTotal);

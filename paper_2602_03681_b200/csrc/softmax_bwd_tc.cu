@@ -29,8 +29,8 @@ struct MiscB {
     uint64_t barQ, full[3], empty[3], barS, barSfree, barP, barAcc;
     uint32_t tmem_base;
     int abort_flag, wait_kcycles;   // in this order: the waits read the limit as abort_flag[1]
-    alignas(16) int pos[kRowsB];
-    alignas(16) float lse2[2][64], dsum[2][64];   // key side: per query of the tile in flight (double-buffered)
+    uint32_t kept[kRowsB / 32];     // query side: which of the CTA's own tokens are retained
+    alignas(16) float lse[2][64], dsum[2][64];   // key side: per query of the tile in a stage (copied with it)
 };
 static_assert(sizeof(MiscB) <= kMiscB, "misc page too small");
 
@@ -88,10 +88,7 @@ softmax_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh  [B
         ms.wait_kcycles = wait_kcycles;
         fence_mbar_init();
     }
-    if (tid < kRowsB) {
-        const int jj = n_full + tid;
-        ms.pos[tid] = jj < n_end ? sm_idx[(size_t)bh * L + jj] : 0x7fffffff;
-    }
+    if (tid < kRowsB / 32) ms.kept[tid] = 0u;
     if (warp == 4) tmem_alloc(&ms.tmem_base, SL::kTmem);
     tc_fence_before_sync();
     __syncthreads();
@@ -175,21 +172,28 @@ softmax_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh  [B
         const bool row_ok = i_abs < L;
         const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
         const float sl2 = scale_sm * kLog2e;
-        const float lse2 = row_ok ? lse[(size_t)bhg * L + i_abs] * kLog2e : 0.f;
+        float lse2 = row_ok ? lse[(size_t)bhg * L + i_abs] * kLog2e : 0.f;
+        if (lse2 == -INFINITY) lse2 = 0.f;                  // no key: every logit is masked below
         const float Di = row_ok ? Dsm[(size_t)bhg * L + i_abs] : 0.f;
         bool ok = true;
-        // The compacted keys are in position order, so row i sees exactly the first `cnt` of them
-        // (a per-element look-up of the key's position costs a divergent branch per element).
-        int cnt = 0;
-        if (row_ok) {
-            cnt = n_full;
-            for (int kq = 0; kq < n_end - n_full; ++kq) cnt += ms.pos[kq] <= i_abs ? 1 : 0;
+        // The compacted keys are in position order, so row i sees exactly the first `cnt` of them: all earlier ones
+        // plus a population count of the CTA's own.
+        if (n_full + r < n_end) {
+            const int rel = sm_idx[(size_t)bh * L + n_full + r] - p * 128;
+            atomicOr(&ms.kept[(rel >> 5) & 3], 1u << (rel & 31));
         }
+        named_barrier_sync(1, kRowsB);
+        int cnt = n_full + __popc(ms.kept[warp] & ((2u << lane) - 1u));
+        for (int e = 0; e < warp; ++e) cnt += __popc(ms.kept[e]);
+        if (!row_ok) cnt = 0;
+        const uint64_t sl22 = pack2(sl2, sl2), nl2 = pack2(-lse2, -lse2), sm2 = pack2(scale_sm, scale_sm);
         for (int t = 0; t < T; ++t) {
             ok = mbar_wait(&ms.barS, t & 1, abort_flag);
             if (!ok) break;
             tc_fence_after_sync();
-            float ds[64];
+            uint32_t dk[32];                                // ds as packed fp16 pairs
+            const int vis = cnt - t * 64;                   // keys of the tile this row sees
+            const bool all_vis = __all_sync(0xffffffffu, vis >= 64);
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
                 uint32_t sv[32], dv[32];
@@ -200,13 +204,16 @@ softmax_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh  [B
                     tc_fence_before_sync();
                     mbar_arrive(&ms.barSfree);
                 }
+                if (!all_vis) {                             // mask the logit (exp2(-inf) = 0): no branch per element
 #pragma unroll
-                for (int c = 0; c < 32; ++c) {
-                    const int jj = t * 64 + 32 * half + c;
-                    const bool vis = jj < cnt;
-                    // mask on the exponent (exp2(-inf) = 0), not around the expression: no branch
-                    const float pr = ex2_ftz(vis ? fmaf(__uint_as_float(sv[c]), sl2, -lse2) : -INFINITY);
-                    ds[32 * half + c] = scale_sm * pr * (__uint_as_float(dv[c]) - Di);
+                    for (int c = 0; c < 32; ++c) sv[c] = 32 * half + c < vis ? sv[c] : 0xff800000u;
+                }
+#pragma unroll
+                for (int c = 0; c < 32; c += 2) {
+                    const float2 e = unpack2(fma2(pack2(__uint_as_float(sv[c]), __uint_as_float(sv[c + 1])), sl22, nl2));
+                    const uint64_t pr = mul2(pack2(ex2_ftz(e.x), ex2_ftz(e.y)), sm2);
+                    const float2 ds = unpack2(mul2(pr, pack2(__uint_as_float(dv[c]) - Di, __uint_as_float(dv[c + 1]) - Di)));
+                    dk[16 * half + (c >> 1)] = pack_half2(ds.x, ds.y);
                 }
             }
             if (t > 0) {
@@ -215,9 +222,7 @@ softmax_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh  [B
             }
 #pragma unroll
             for (int pc = 0; pc < 8; ++pc)
-                *reinterpret_cast<uint4 *>(smem + SL::oDS + sw128_offset(r, pc)) =
-                    make_uint4(pack_half2(ds[8 * pc], ds[8 * pc + 1]), pack_half2(ds[8 * pc + 2], ds[8 * pc + 3]),
-                               pack_half2(ds[8 * pc + 4], ds[8 * pc + 5]), pack_half2(ds[8 * pc + 6], ds[8 * pc + 7]));
+                *reinterpret_cast<uint4 *>(smem + SL::oDS + sw128_offset(r, pc)) = make_uint4(dk[4 * pc], dk[4 * pc + 1], dk[4 * pc + 2], dk[4 * pc + 3]);
             fence_proxy_async_smem();
             tc_fence_before_sync();
             mbar_arrive(&ms.barP);
@@ -329,7 +334,9 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
             for (; t < T; ++t) {
                 const int s = t & 1;
                 if (!mbar_wait(&ms.empty[s], ((t >> 1) & 1) ^ 1, abort_flag)) break;
-                mbar_arrive_expect_tx(&ms.full[s], 2 * SL::kQ);
+                mbar_arrive_expect_tx(&ms.full[s], 2 * SL::kQ + 512);
+                bulk_load_1d(ms.lse[s], lse + (size_t)bhg * L + (qt0 + t) * 64, 256, &ms.full[s]);
+                bulk_load_1d(ms.dsum[s], Dsm + (size_t)bhg * L + (qt0 + t) * 64, 256, &ms.full[s]);
                 for (int kb = 0; kb < KB; ++kb) {
                     tma_load_2d(smem + SL::oQ + s * SL::kQ + kb * 8192, &map_q, &ms.full[s], x0 + kb * 64,
                                 bh * L + (qt0 + t) * 64);
@@ -401,18 +408,23 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
         bool ok = true;
         for (int t = 0; t < T; ++t) {
             const int i0 = (qt0 + t) * 64;
-            // per-query log-sum-exp and D of this tile; two buffers, so that a thread still reading
-            // the previous tile's values is not overtaken (the barrier below separates t from t + 2)
-            float *lse2 = ms.lse2[t & 1], *dsum = ms.dsum[t & 1];
-            if (r < 64) {
-                lse2[r] = lse[(size_t)bhg * L + i0 + r] * kLog2e;
-                dsum[r] = Dsm[(size_t)bhg * L + i0 + r];
-            }
-            named_barrier_sync(1, kRowsB);
-            ok = mbar_wait(&ms.barS, t & 1, abort_flag);
+            // per-query log-sum-exp and D of this tile, copied with the stage (the logits were formed from it, so it
+            // is full; released below)
+            float *lse_t = ms.lse[t & 1];
+            const float *dsum = ms.dsum[t & 1];
+            ok = mbar_wait(&ms.full[t & 1], (t >> 1) & 1, abort_flag) && mbar_wait(&ms.barS, t & 1, abort_flag);
             if (!ok) break;
             tc_fence_after_sync();
-            float pv[64], ds[64];
+            // p and ds as packed fp16 pairs (p first, ds behind its logits' half)
+            uint32_t pk[32], dk[32];
+            const uint64_t sl22 = pack2(sl2, sl2), nl2 = pack2(-kLog2e, -kLog2e), sm2 = pack2(scale_sm, scale_sm);
+            const int vis = pos_j - i0;                     // queries vis .. of the tile see this key
+            const bool all_vis = __all_sync(0xffffffffu, vis <= 0);
+            if (!all_vis) {     // a query without any key has lse = -inf, which must not meet a masked logit's -inf
+                if (lse_t[lane] == -INFINITY) lse_t[lane] = 0.f;
+                if (lse_t[lane + 32] == -INFINITY) lse_t[lane + 32] = 0.f;
+                __syncwarp();
+            }
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
                 uint32_t sv[32], dv[32];
@@ -423,15 +435,25 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
                     tc_fence_before_sync();
                     mbar_arrive(&ms.barSfree);
                 }
+                if (!all_vis) {                             // mask the logit (exp2(-inf) = 0): no branch per element
 #pragma unroll
-                for (int c = 0; c < 32; ++c) {
+                    for (int c = 0; c < 32; ++c) sv[c] = vis <= 32 * half + c ? sv[c] : 0xff800000u;
+                }
+#pragma unroll
+                for (int c = 0; c < 32; c += 2) {
                     const int cc = 32 * half + c;
-                    const bool vis = pos_j <= i0 + cc;
-                    const float pr = ex2_ftz(vis ? fmaf(__uint_as_float(sv[c]), sl2, -lse2[cc]) : -INFINITY);
-                    pv[cc] = pr;
-                    const float dm = pr * (__uint_as_float(dv[c]) - dsum[cc]);   // dM_ij (Section 4.2)
-                    if (kMask) msum += dm;
-                    ds[cc] = scale_sm * dm;
+                    const uint64_t l2 = *reinterpret_cast<const uint64_t *>(&lse_t[cc]);
+                    const float2 e = unpack2(fma2(pack2(__uint_as_float(sv[c]), __uint_as_float(sv[c + 1])), sl22, mul2(l2, nl2)));
+                    const float p0 = ex2_ftz(e.x), p1 = ex2_ftz(e.y);
+                    pk[cc >> 1] = pack_half2(p0, p1);
+                    const float2 d2 = *reinterpret_cast<const float2 *>(&dsum[cc]);
+                    const uint64_t dm = mul2(pack2(p0, p1), pack2(__uint_as_float(dv[c]) - d2.x, __uint_as_float(dv[c + 1]) - d2.y));
+                    if (kMask) {                            // dM_ij (Section 4.2)
+                        const float2 m = unpack2(dm);
+                        msum += m.x + m.y;
+                    }
+                    const float2 ds = unpack2(mul2(dm, sm2));
+                    dk[cc >> 1] = pack_half2(ds.x, ds.y);
                 }
             }
             if (t > 0) {
@@ -440,12 +462,8 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
             }
 #pragma unroll
             for (int pc = 0; pc < 8; ++pc) {
-                *reinterpret_cast<uint4 *>(smem + SL::oP + sw128_offset(r, pc)) =
-                    make_uint4(pack_half2(pv[8 * pc], pv[8 * pc + 1]), pack_half2(pv[8 * pc + 2], pv[8 * pc + 3]),
-                               pack_half2(pv[8 * pc + 4], pv[8 * pc + 5]), pack_half2(pv[8 * pc + 6], pv[8 * pc + 7]));
-                *reinterpret_cast<uint4 *>(smem + SL::oDS + sw128_offset(r, pc)) =
-                    make_uint4(pack_half2(ds[8 * pc], ds[8 * pc + 1]), pack_half2(ds[8 * pc + 2], ds[8 * pc + 3]),
-                               pack_half2(ds[8 * pc + 4], ds[8 * pc + 5]), pack_half2(ds[8 * pc + 6], ds[8 * pc + 7]));
+                *reinterpret_cast<uint4 *>(smem + SL::oP + sw128_offset(r, pc)) = make_uint4(pk[4 * pc], pk[4 * pc + 1], pk[4 * pc + 2], pk[4 * pc + 3]);
+                *reinterpret_cast<uint4 *>(smem + SL::oDS + sw128_offset(r, pc)) = make_uint4(dk[4 * pc], dk[4 * pc + 1], dk[4 * pc + 2], dk[4 * pc + 3]);
             }
             fence_proxy_async_smem();
             tc_fence_before_sync();

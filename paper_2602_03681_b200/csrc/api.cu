@@ -169,7 +169,6 @@ struct BwdWs {
     float *dGrow, *kappa, *gS;                               // [B,H,L] (gS: [B,H,NC,d/32])
     // tensor-core path
     void *k_smb, *k16, *v16, *Qh, *dO16;                     // softmax branch: 16-bit [B,H,L,d]
-    void *kn16;                                              // NATSL_QK_NORM with block-level routing: normalised k, likewise
     void *o_la16;                                            // linear read-out as fp16 [B,L,H,d]
     GdnTcWs tc;                                              // the forward's chunkwise intermediates
     GdnTcExport ex;                                          // ... and what it keeps for the backward
@@ -227,7 +226,6 @@ BwdWs carve_bwd(const natsl_params *p, void *ws) {
     // tensor-core path
     f.k_smb = half(tcs, TM); f.k16 = half(tcs, TM); f.v16 = half(tcs, TM); f.Qh = half(tcs, TM);
     f.dO16 = half(tcs, TM);
-    f.kn16 = half(tcs && block && normed, TM);
     f.o_la16 = f.dO16;
     f.gr.dO16 = half(tcs, TM); f.gr.dOg16 = half(tcs, TM); f.gr.dU16 = half(tcs, TM); f.gr.dS16 = half(tcs, ST);
     f.tc = GdnTcWs{};
@@ -700,10 +698,8 @@ int natsl_hybrid_bwd(const void *q, const void *k, const void *v, const float *g
         const float *dq_add = normed ? nullptr : f.dq_sm;
         if (block) {
             NATSL_TRY(launch_gdn_finish(a, f.dk_x, f.dv_x, s32, st0, false));
-            if (normed) NATSL_TRY(launch_to_f16_bhld(k, f.kn16, s, hg, st));
             NATSL_TRY(launch_softmax_bwd_own_block(q, k, v, f.dO16, f.lse, f.Dsm, route, p->scale_sm, f.dq_sm, f.dk_x,
-                                                   f.dv_x, gsc, s, st, hg.G, normed ? q16 : nullptr,
-                                                   normed ? f.kn16 : nullptr));
+                                                   f.dv_x, gsc, s, st, hg));
             NATSL_TRY(side_join.join());      // the side stream's last kernels
             NATSL_TRY(launch_gdn_chunk_bwd(f.tc, f.ex, f.gr, v, beta, route, dq_add, p->scale_la, dq_o, dk_o, dv_o, normed,
                                            dg, dbeta, true, normed ? nullptr : f.dk_x, f.dv_x,

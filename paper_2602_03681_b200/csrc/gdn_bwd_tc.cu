@@ -308,15 +308,14 @@ __device__ __forceinline__ void mma64(const __half *A, const __half *B, int row0
 // with lse_i and D_i = <do_i, o_i> of the whole softmax row.  Softmax heads of 64 KB columns: KB = 1 for
 // d = 64 or kG = 2 heads per linear head of d = 128 (Section 4.3; the head is then a column slice of rows
 // of 128 columns, lse / Dsm are [B,H,kG,L]), KB = 2 for d = 128 (two tiles per operand: the logit products
-// add over them, the three results are formed half by half).  kNormSrc: q and k come from the fp16 copies
-// [B,H,L,DL] that hold the softmax operation's normalised rows (qn, kn) instead of the bf16 inputs.
+// add over them, the three results are formed half by half).  kNorm: q and k are RMS-normalised per softmax
+// head as they are staged.
 template <int KB> constexpr int own_smem() { return (4 * KB + 2) * kTileH * 2; }
 
-template <int kG, bool kNormSrc, int KB>
+template <int kG, bool kNorm, int KB>
 __global__ void __launch_bounds__(kCkThreads, KB == 1 ? 3 : 2)
 softmax_bwd_own_block_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfloat16 *__restrict__ k,
-                             const __nv_bfloat16 *__restrict__ v, const __half *__restrict__ qn,
-                             const __half *__restrict__ kn, const __half *__restrict__ do16,
+                             const __nv_bfloat16 *__restrict__ v, float norm_eps, const __half *__restrict__ do16,
                              const float *__restrict__ lse, const float *__restrict__ Dsm,
                              const uint8_t *__restrict__ route, float scale_sm,
                              float *__restrict__ dq_sm, float *__restrict__ dk_x,
@@ -346,11 +345,30 @@ softmax_bwd_own_block_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfl
             const uint2 xv = *reinterpret_cast<const uint2 *>(v + off);
             const size_t offh = ((size_t)bh * L + (size_t)c * kC + r) * DL + col0 + kb * 64 + c4;      // [B,H,L,DL]
             const uint2 xo = *reinterpret_cast<const uint2 *>(do16 + offh);
-            if (kNormSrc) {
-                *reinterpret_cast<uint2 *>(sQ + tl) = *reinterpret_cast<const uint2 *>(qn + offh);
-                *reinterpret_cast<uint2 *>(sK + tl) = *reinterpret_cast<const uint2 *>(kn + offh);
+            const uint2 xq = *reinterpret_cast<const uint2 *>(q + off), xk = *reinterpret_cast<const uint2 *>(k + off);
+            if (kNorm) {     // RMS over the softmax head's columns of the row, 16 lanes x 4 (64-column heads)
+                auto f4 = [](uint2 w) {
+                    return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u),
+                                       __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u));
+                };
+                const float4 fq = f4(xq), fk = f4(xk);
+                float sq = fmaf(fq.x, fq.x, fmaf(fq.y, fq.y, fmaf(fq.z, fq.z, fq.w * fq.w)));
+                float sk = fmaf(fk.x, fk.x, fmaf(fk.y, fk.y, fmaf(fk.z, fk.z, fk.w * fk.w)));
+                if (KB == 2) {       // (128-column heads: the other block's columns too)
+                    const float4 gq = f4(*reinterpret_cast<const uint2 *>(q + off + (1 - 2 * kb) * 64));
+                    const float4 gk = f4(*reinterpret_cast<const uint2 *>(k + off + (1 - 2 * kb) * 64));
+                    sq += fmaf(gq.x, gq.x, fmaf(gq.y, gq.y, fmaf(gq.z, gq.z, gq.w * gq.w)));
+                    sk += fmaf(gk.x, gk.x, fmaf(gk.y, gk.y, fmaf(gk.z, gk.z, gk.w * gk.w)));
+                }
+#pragma unroll
+                for (int o = 8; o > 0; o >>= 1) {
+                    sq += __shfl_xor_sync(0xffffffffu, sq, o);
+                    sk += __shfl_xor_sync(0xffffffffu, sk, o);
+                }
+                const float rq = rsqrtf(sq / D + norm_eps), rk = rsqrtf(sk / D + norm_eps);
+                *reinterpret_cast<uint2 *>(sQ + tl) = make_uint2(pack_half2(fq.x * rq, fq.y * rq), pack_half2(fq.z * rq, fq.w * rq));
+                *reinterpret_cast<uint2 *>(sK + tl) = make_uint2(pack_half2(fk.x * rk, fk.y * rk), pack_half2(fk.z * rk, fk.w * rk));
             } else {
-                const uint2 xq = *reinterpret_cast<const uint2 *>(q + off), xk = *reinterpret_cast<const uint2 *>(k + off);
                 *reinterpret_cast<uint2 *>(sQ + tl) = make_uint2(cv(xq.x), cv(xq.y));
                 *reinterpret_cast<uint2 *>(sK + tl) = make_uint2(cv(xk.x), cv(xk.y));
             }
@@ -503,7 +521,9 @@ cudaError_t launch_softmax_bwd_own_block(const void *q, const void *k, const voi
                                          const void *do16, const float *lse, const float *Dsm,
                                          const uint8_t *route, float scale_sm, float *dq_sm,
                                          float *dk_x, float *dv_x, const int32_t *gsc, Shape s,
-                                         cudaStream_t st, int G, const void *qn, const void *kn) {
+                                         cudaStream_t st, HeadGroups hg) {
+    const int G = hg.G;
+    const bool qn = hg.norm_eps >= 0.f;
     if (!s.bf16 || !((s.d == 64 && G <= 1) || (s.d == 128 && G <= 2))) return cudaErrorInvalidValue;
     auto kernel = softmax_bwd_own_block_kernel<1, false, 1>;
     int smem = own_smem<1>();
@@ -517,8 +537,7 @@ cudaError_t launch_softmax_bwd_own_block(const void *q, const void *k, const voi
     if (e != cudaSuccess) return e;
     dim3 grid(s.L / kC, s.B * s.H * (G == 2 ? 2 : 1));
     kernel<<<grid, kCkThreads, smem, st>>>(
-        (const __nv_bfloat16 *)q, (const __nv_bfloat16 *)k, (const __nv_bfloat16 *)v, (const __half *)qn,
-        (const __half *)kn, (const __half *)do16,
+        (const __nv_bfloat16 *)q, (const __nv_bfloat16 *)k, (const __nv_bfloat16 *)v, hg.norm_eps, (const __half *)do16,
         lse, Dsm, route, scale_sm, dq_sm, dk_x, dv_x, gsc, s.L, s.H);
     count_launch();
     return cudaGetLastError();

@@ -124,8 +124,6 @@ cudaError_t launch_softmax_bwd_tc(const void *q, void *Qh, const void *dO16, con
                                   HeadGroups hg = HeadGroups{});
 // (hg.G = 2 at d = 128: softmax heads are column slices, lse / Dsm [B,H,G,L]; hg.norm_eps >= 0: Qh is
 // written here as the slice-wise RMS-normalised q, k16 must hold the normalised keys already)
-// bf16 [B,L,H,d] -> fp16 [B,H,L,d], slice-wise RMS-normalised when hg.norm_eps >= 0 (the softmax operation's q, k)
-cudaError_t launch_to_f16_bhld(const void *x, void *xh, Shape s, HeadGroups hg, cudaStream_t st);
 
 // gdn_tc.cu -- tensor-core chunkwise Gated DeltaNet (bf16 storage): intermediates in workspace
 struct GdnTcWs {
@@ -285,10 +283,9 @@ cudaError_t launch_softmax_bwd_own_block(const void *q, const void *k, const voi
                                          const void *do16, const float *lse, const float *Dsm,
                                          const uint8_t *route, float scale_sm, float *dq_sm,
                                          float *dk_x, float *dv_x, const int32_t *gsc, Shape s,
-                                         cudaStream_t st, int G = 1, const void *qn = nullptr,
-                                         const void *kn = nullptr);
-// (softmax heads of 64 columns: d = 64, or G = 2 at d = 128 with lse / Dsm [B,H,G,L]; qn, kn: fp16 copies
-// [B,H,L,d] holding the softmax operation's normalised q, k, read instead of q, k)
+                                         cudaStream_t st, HeadGroups hg);
+// (softmax heads of 64 or 128 columns; two heads of 64 at d = 128: lse / Dsm [B,H,G,L]; hg.norm_eps >= 0: q, k are
+// RMS-normalised as they are read)
 
 // decode.cu
 // Bytes of workspace of a decode step: status word, per-head tickets, partial softmax results and

@@ -26,11 +26,11 @@ constexpr int kMiscB = 2048;
 constexpr float kLog2e = 1.4426950408889634f;
 
 struct MiscB {
-    uint64_t barQ, full[3], empty[3], barS, barSfree, barP, barAcc;
+    uint64_t barQ, full[3], empty[3], barS, barDP, barSfree, barP, barAcc;
     uint32_t tmem_base;
     int abort_flag, wait_kcycles;   // in this order: the waits read the limit as abort_flag[1]
     uint32_t kept[kRowsB / 32];     // query side: which of the CTA's own tokens are retained
-    alignas(16) float lse[2][64], dsum[2][64];   // key side: per query of the tile in a stage (copied with it)
+    alignas(16) float lse[3][64], dsum[3][64];   // key side: per query of the tile in a stage (copied with it)
 };
 static_assert(sizeof(MiscB) <= kMiscB, "misc page too small");
 
@@ -262,13 +262,16 @@ softmax_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh  [B
 // ==========================================================================================
 // Key side
 // ==========================================================================================
+// dS^T goes to the multiplier through TMEM, over the dP^T it was formed from, which leaves shared memory for a third
+// query tile in flight at two CTAs per SM (D = 64).  With two, a tile's copy could start only when the product
+// two tiles back had released its place and was a serial part of the chain: 2700 cycles per tile.
 template <int D> struct KLayout {
     static constexpr int KB = D / 64;
     static constexpr int kKV = KB * 128 * 128;            // 128 keys x D fp16
     static constexpr int kQ = KB * 64 * 128;              // 64 queries x D fp16
-    static constexpr int oK = 0, oV = kKV, oQ = 2 * kKV, oDO = oQ + 2 * kQ, oP = oDO + 2 * kQ,
-                         oDS = oP + 128 * 128;
-    static constexpr int oMisc = oDS + 128 * 128;
+    static constexpr int kStages = 3;
+    static constexpr int oK = 0, oV = kKV, oQ = 2 * kKV, oDO = oQ + kStages * kQ, oP = oDO + kStages * kQ;
+    static constexpr int oMisc = oP + 128 * 128;
     static constexpr int kTotal = oMisc + kMiscB;
     static constexpr int kTmem = D == 64 ? 256 : 512;     // S^T 64 + dP^T 64 + dV D + dK D
 };
@@ -306,8 +309,9 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
     }
     if (tid == 0) {
         mbar_init(&ms.barQ, 1);
-        for (int s = 0; s < 2; ++s) { mbar_init(&ms.full[s], 1); mbar_init(&ms.empty[s], 1 + kRowsB); }
+        for (int s = 0; s < SL::kStages; ++s) { mbar_init(&ms.full[s], 1); mbar_init(&ms.empty[s], 1 + kRowsB); }
         mbar_init(&ms.barS, 1);
+        mbar_init(&ms.barDP, 1);
         mbar_init(&ms.barSfree, kRowsB);
         mbar_init(&ms.barP, kRowsB);
         mbar_init(&ms.barAcc, 1);
@@ -332,8 +336,8 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
             }
             int t = 0;
             for (; t < T; ++t) {
-                const int s = t & 1;
-                if (!mbar_wait(&ms.empty[s], ((t >> 1) & 1) ^ 1, abort_flag)) break;
+                const int s = t % SL::kStages;
+                if (!mbar_wait(&ms.empty[s], ((t / SL::kStages) & 1) ^ 1, abort_flag)) break;
                 mbar_arrive_expect_tx(&ms.full[s], 2 * SL::kQ + 512);
                 bulk_load_1d(ms.lse[s], lse + (size_t)bhg * L + (qt0 + t) * 64, 256, &ms.full[s]);
                 bulk_load_1d(ms.dsum[s], Dsm + (size_t)bhg * L + (qt0 + t) * 64, 256, &ms.full[s]);
@@ -344,58 +348,54 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
                                 bh * L + (qt0 + t) * 64);
                 }
             }
-            for (int u = max(0, t - 2); u < t; ++u) mbar_wait_drain(&ms.full[u & 1], (u >> 1) & 1);
+            for (int u = max(0, t - SL::kStages); u < t; ++u)
+                mbar_wait_drain(&ms.full[u % SL::kStages], (u / SL::kStages) & 1);
             mbar_wait_drain(&ms.barQ, 0);
         }
     } else if (warp == 4) {
         if (lane == 0) {
             constexpr uint32_t id_s = make_idesc(kFmtF16, 128, 64, false, false);
             constexpr uint32_t id_acc = make_idesc(kFmtF16, 128, D, false, true);
-            const uint32_t aK = smem_u32(smem + SL::oK), aV = smem_u32(smem + SL::oV),
-                           aP = smem_u32(smem + SL::oP), aDS = smem_u32(smem + SL::oDS);
-            auto issue_s = [&](int t) {
-                const uint32_t aQ = smem_u32(smem + SL::oQ + (t & 1) * SL::kQ);
-                const uint32_t aDO = smem_u32(smem + SL::oDO + (t & 1) * SL::kQ);
+            const uint32_t aK = smem_u32(smem + SL::oK), aV = smem_u32(smem + SL::oV), aP = smem_u32(smem + SL::oP);
+            auto stage = [&](int o, int t) { return smem_u32(smem + o + (t % SL::kStages) * SL::kQ); };
+            auto issue_logits = [&](uint32_t dst, uint32_t a, uint32_t b, uint64_t *bar) {
 #pragma unroll
                 for (int kb = 0; kb < KB; ++kb)
 #pragma unroll
-                    for (int k16 = 0; k16 < 4; ++k16) {
-                        mma_ss(tS, desc_kmajor(aK + kb * 16384 + k16 * 32),
-                               desc_kmajor(aQ + kb * 8192 + k16 * 32), id_s, (kb | k16) != 0);
-                        mma_ss(tDP, desc_kmajor(aV + kb * 16384 + k16 * 32),
-                               desc_kmajor(aDO + kb * 8192 + k16 * 32), id_s, (kb | k16) != 0);
-                    }
-                mma_commit(&ms.barS);
+                    for (int k16 = 0; k16 < 4; ++k16)
+                        mma_ss(dst, desc_kmajor(a + kb * 16384 + k16 * 32), desc_kmajor(b + kb * 8192 + k16 * 32), id_s,
+                               (kb | k16) != 0);
+                mma_commit(bar);
             };
             bool ok = mbar_wait(&ms.barQ, 0, abort_flag) && mbar_wait(&ms.full[0], 0, abort_flag);
             if (ok) {
                 tc_fence_after_sync();
-                issue_s(0);
+                issue_logits(tS, aK, stage(SL::oQ, 0), &ms.barS);
+                issue_logits(tDP, aV, stage(SL::oDO, 0), &ms.barDP);
             }
             for (int t = 0; ok && t < T; ++t) {
-                // S^T and dP^T of the next query tile go into the same TMEM columns as soon as the row
-                // threads have read this tile's out of them, i.e. while they still compute P^T, dS^T.
+                // S^T of the next query tile goes into the same TMEM columns as soon as the row threads have read
+                // this tile's out of them; dP^T of the next one behind this tile's products, which read dS^T there.
                 if (t + 1 < T) {
-                    ok = mbar_wait(&ms.full[(t + 1) & 1], ((t + 1) >> 1) & 1, abort_flag) &&
+                    ok = mbar_wait(&ms.full[(t + 1) % SL::kStages], ((t + 1) / SL::kStages) & 1, abort_flag) &&
                          mbar_wait(&ms.barSfree, t & 1, abort_flag);
                     if (!ok) break;
                     tc_fence_after_sync();
-                    issue_s(t + 1);
+                    issue_logits(tS, aK, stage(SL::oQ, t + 1), &ms.barS);
                 }
                 ok = mbar_wait(&ms.barP, t & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after_sync();
-                const uint32_t aQ = smem_u32(smem + SL::oQ + (t & 1) * SL::kQ);
-                const uint32_t aDO = smem_u32(smem + SL::oDO + (t & 1) * SL::kQ);
+                const uint32_t aQ = stage(SL::oQ, t), aDO = stage(SL::oDO, t);
 #pragma unroll
                 for (int k16 = 0; k16 < 4; ++k16) {
                     mma_ss(tDV, desc_kmajor(aP + k16 * 32), desc_mnmajor(aDO + k16 * 2048, 8192), id_acc,
                            (t | k16) != 0);
-                    mma_ss(tDK, desc_kmajor(aDS + k16 * 32), desc_mnmajor(aQ + k16 * 2048, 8192), id_acc,
-                           (t | k16) != 0);
+                    mma_ts(tDK, tDP + k16 * 8, desc_mnmajor(aQ + k16 * 2048, 8192), id_acc, (t | k16) != 0);
                 }
                 mma_commit(&ms.barAcc);
-                mma_commit(&ms.empty[t & 1]);
+                mma_commit(&ms.empty[t % SL::kStages]);
+                if (t + 1 < T) issue_logits(tDP, aV, stage(SL::oDO, t + 1), &ms.barDP);
             }
         }
     } else {
@@ -410,13 +410,12 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
             const int i0 = (qt0 + t) * 64;
             // per-query log-sum-exp and D of this tile, copied with the stage (the logits were formed from it, so it
             // is full; released below)
-            float *lse_t = ms.lse[t & 1];
-            const float *dsum = ms.dsum[t & 1];
-            ok = mbar_wait(&ms.full[t & 1], (t >> 1) & 1, abort_flag) && mbar_wait(&ms.barS, t & 1, abort_flag);
+            const int sg = t % SL::kStages;
+            float *lse_t = ms.lse[sg];
+            const float *dsum = ms.dsum[sg];
+            ok = mbar_wait(&ms.full[sg], (t / SL::kStages) & 1, abort_flag) && mbar_wait(&ms.barS, t & 1, abort_flag);
             if (!ok) break;
             tc_fence_after_sync();
-            // p and ds as packed fp16 pairs (p first, ds behind its logits' half)
-            uint32_t pk[32], dk[32];
             const uint64_t sl22 = pack2(sl2, sl2), nl2 = pack2(-kLog2e, -kLog2e), sm2 = pack2(scale_sm, scale_sm);
             const int vis = pos_j - i0;                     // queries vis .. of the tile see this key
             const bool all_vis = __all_sync(0xffffffffu, vis <= 0);
@@ -425,29 +424,43 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
                 if (lse_t[lane + 32] == -INFINITY) lse_t[lane + 32] = 0.f;
                 __syncwarp();
             }
+            float x[64];                                    // logits, then probabilities
+            tmem_ld32(tS + lane_base, reinterpret_cast<uint32_t (&)[32]>(x[0]));
+            tmem_ld32(tS + lane_base + 32, reinterpret_cast<uint32_t (&)[32]>(x[32]));
+            tmem_wait_ld();
+            tc_fence_before_sync();
+            mbar_arrive(&ms.barSfree);
+            if (!all_vis) {                                 // mask the logit (exp2(-inf) = 0): no branch per element
+#pragma unroll
+                for (int c = 0; c < 64; ++c) x[c] = vis <= c ? x[c] : -INFINITY;
+            }
+#pragma unroll
+            for (int c = 0; c < 64; c += 2) {
+                const uint64_t l2 = *reinterpret_cast<const uint64_t *>(&lse_t[c]);
+                const float2 e = unpack2(fma2(pack2(x[c], x[c + 1]), sl22, mul2(l2, nl2)));
+                x[c] = ex2_ftz(e.x);
+                x[c + 1] = ex2_ftz(e.y);
+            }
+            // dP^T of this tile was issued behind the previous tile's products: they have read P and dS by now
+            ok = mbar_wait(&ms.barDP, t & 1, abort_flag);
+            if (!ok) break;
+            tc_fence_after_sync();
+#pragma unroll
+            for (int pc = 0; pc < 8; ++pc)
+                *reinterpret_cast<uint4 *>(smem + SL::oP + sw128_offset(r, pc)) =
+                    make_uint4(pack_half2(x[8 * pc], x[8 * pc + 1]), pack_half2(x[8 * pc + 2], x[8 * pc + 3]),
+                               pack_half2(x[8 * pc + 4], x[8 * pc + 5]), pack_half2(x[8 * pc + 6], x[8 * pc + 7]));
+            uint32_t dk[32];
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
-                uint32_t sv[32], dv[32];
-                tmem_ld32(tS + lane_base + 32 * half, sv);
+                uint32_t dv[32];
                 tmem_ld32(tDP + lane_base + 32 * half, dv);
                 tmem_wait_ld();
-                if (half == 1) {                            // both halves are in registers
-                    tc_fence_before_sync();
-                    mbar_arrive(&ms.barSfree);
-                }
-                if (!all_vis) {                             // mask the logit (exp2(-inf) = 0): no branch per element
-#pragma unroll
-                    for (int c = 0; c < 32; ++c) sv[c] = vis <= 32 * half + c ? sv[c] : 0xff800000u;
-                }
 #pragma unroll
                 for (int c = 0; c < 32; c += 2) {
                     const int cc = 32 * half + c;
-                    const uint64_t l2 = *reinterpret_cast<const uint64_t *>(&lse_t[cc]);
-                    const float2 e = unpack2(fma2(pack2(__uint_as_float(sv[c]), __uint_as_float(sv[c + 1])), sl22, mul2(l2, nl2)));
-                    const float p0 = ex2_ftz(e.x), p1 = ex2_ftz(e.y);
-                    pk[cc >> 1] = pack_half2(p0, p1);
                     const float2 d2 = *reinterpret_cast<const float2 *>(&dsum[cc]);
-                    const uint64_t dm = mul2(pack2(p0, p1), pack2(__uint_as_float(dv[c]) - d2.x, __uint_as_float(dv[c + 1]) - d2.y));
+                    const uint64_t dm = mul2(pack2(x[cc], x[cc + 1]), pack2(__uint_as_float(dv[c]) - d2.x, __uint_as_float(dv[c + 1]) - d2.y));
                     if (kMask) {                            // dM_ij (Section 4.2)
                         const float2 m = unpack2(dm);
                         msum += m.x + m.y;
@@ -456,19 +469,12 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
                     dk[cc >> 1] = pack_half2(ds.x, ds.y);
                 }
             }
-            if (t > 0) {
-                ok = mbar_wait(&ms.barAcc, (t - 1) & 1, abort_flag);   // P^T / dS^T buffers consumed
-                if (!ok) break;
-            }
-#pragma unroll
-            for (int pc = 0; pc < 8; ++pc) {
-                *reinterpret_cast<uint4 *>(smem + SL::oP + sw128_offset(r, pc)) = make_uint4(pk[4 * pc], pk[4 * pc + 1], pk[4 * pc + 2], pk[4 * pc + 3]);
-                *reinterpret_cast<uint4 *>(smem + SL::oDS + sw128_offset(r, pc)) = make_uint4(dk[4 * pc], dk[4 * pc + 1], dk[4 * pc + 2], dk[4 * pc + 3]);
-            }
+            tmem_st32(tDP + lane_base, dk);                 // dS^T over this thread's own dP^T
+            tmem_wait_st();
             fence_proxy_async_smem();
             tc_fence_before_sync();
             mbar_arrive(&ms.barP);
-            mbar_arrive(&ms.empty[t & 1]);     // (the stage's release also waits for the MMAs' commit)
+            mbar_arrive(&ms.empty[sg]);        // (the stage's release also waits for the MMAs' commit)
         }
         if (ok) {
             ok = mbar_wait(&ms.barAcc, (T - 1) & 1, abort_flag);
@@ -546,7 +552,7 @@ to_f16_bhld_kernel(const __nv_bfloat16 *__restrict__ q, __half *__restrict__ qh,
 
 }  // namespace
 
-cudaError_t launch_to_f16_bhld(const void *x, void *xh, Shape s, HeadGroups hg, cudaStream_t st) {
+static cudaError_t launch_to_f16_bhld(const void *x, void *xh, Shape s, HeadGroups hg, cudaStream_t st) {
     const size_t pieces = (size_t)s.B * s.L * s.H * (s.d / 8);
     auto kernel = s.d == 128 ? to_f16_bhld_kernel<128> : to_f16_bhld_kernel<64>;
     kernel<<<(unsigned)((pieces + 255) / 256), 256, 0, st>>>((const __nv_bfloat16 *)x, (__half *)xh, s.B, s.L, s.H, hg.G,

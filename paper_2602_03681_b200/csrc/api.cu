@@ -79,6 +79,12 @@ bool use_tensor_cores(const natsl_params *p) {
     return p->dtype == NATSL_BF16 && !(p->flags & NATSL_FORCE_SIMT);
 }
 
+// Whether the scan is a programmatic dependent of the kernels before it too, which saves the gap of a launch: only when
+// the prepare kernel is a single wave (four CTAs on each of 148 multiprocessors).  Behind several waves the scan's
+// CTAs, one to a multiprocessor, would be placed in the order these drain, i.e. crowded into a few GPCs, whose share of
+// the L2 bandwidth the scans then fight for: 60 of them took 310-370 us there instead of 128 us.
+bool scan_follows_closely(const natsl_params *p) { return (long long)p->B * p->H * (p->L / kC) <= 4 * 148; }
+
 // Segments of the forward scan (tensor-core path): the largest power of two that keeps the two
 // runs per segment within ~one CTA per SM, divides the chunk count and leaves >= 8 chunks each.
 int scan_segments(const natsl_params *p) {
@@ -107,9 +113,10 @@ FwdWs carve_fwd(const natsl_params *p, void *ws) {
     f.head_bytes = c.off;
     f.sm_idx = c.take<int32_t>(B * H * L);
     f.prefix = c.take<int32_t>(B * H * (NC + 1));
-    f.lin_idx = c.take<int32_t>(B * H * L);
-    f.n_lin = c.take<int32_t>(B * H * NC);
-    f.sm_len = c.take<int32_t>(B * H);
+    const bool simt = !use_tensor_cores(p);
+    f.lin_idx = c.take<int32_t>(simt ? B * H * L : 0);
+    f.n_lin = c.take<int32_t>(simt ? B * H * NC : 0);
+    f.sm_len = c.take<int32_t>(simt ? B * H : 0);
     f.k_sm = c.take<char>(B * H * L * d * esz);
     f.v_sm = c.take<char>(B * H * L * d * esz);
     if (use_tensor_cores(p)) {
@@ -198,9 +205,9 @@ BwdWs carve_bwd(const natsl_params *p, void *ws) {
     f.head_bytes = c.off;
     f.sm_idx = c.take<int32_t>(BHL);
     f.prefix = c.take<int32_t>(B * H * (NC + 1));
-    f.lin_idx = c.take<int32_t>(BHL);
-    f.n_lin = c.take<int32_t>(B * H * NC);
-    f.sm_len = c.take<int32_t>(B * H);
+    f.lin_idx = c.take<int32_t>(simt ? BHL : 0);
+    f.n_lin = c.take<int32_t>(simt ? B * H * NC : 0);
+    f.sm_len = c.take<int32_t>(simt ? B * H : 0);
     f.o_la = tm(true);
     f.o_nla = tm(true);
     f.lse = c.take<float>(BHL * Gg);
@@ -249,10 +256,9 @@ BwdWs carve_bwd(const natsl_params *p, void *ws) {
 
 namespace {
 
-// The compaction and the gather of the retained K/V do not depend on the linear branch's prepare
-// kernel (and that kernel does not depend on them), so the forward runs them beside it: on a
-// library-owned stream per device, forked from the caller's stream with one event and joined back
-// with another before the softmax kernel.  Stream and events are created on first use and kept;
+// In the backward the linear branch's reverse scan and the key-side softmax kernel do not depend on the query-side
+// one, so they run beside it: on a library-owned stream per device, forked from the caller's stream with one event and joined back
+// with another before the results meet.  Stream and events are created on first use and kept;
 // a mutex covers the enqueue of a call, since the two event objects are shared by all calls.
 struct SideStream {
     cudaStream_t st = nullptr;
@@ -315,69 +321,44 @@ static int bwd_forward_part(const void *q, const void *k, const void *v, const f
     const bool tensor_cores = use_tensor_cores(p);
     int32_t *flags = tensor_cores && !(p->flags & NATSL_SINGLE_STREAM) ? f.emit_flags : nullptr;
 #define NATSL_TRY(call) do { if ((call) != cudaSuccess) return NATSL_ERR_CUDA; } while (0)
-    NATSL_TRY(cudaMemsetAsync(f.status, 0, f.head_bytes, st));
-    // compaction + gather beside the prepare kernel, on the library's side stream (as in the forward)
-    std::unique_lock<std::mutex> side_lock;
-    SideStream *side = nullptr;
-    SideJoin side_join;
-    if (tensor_cores && !(p->flags & NATSL_SINGLE_STREAM)) {
-        side_lock = std::unique_lock<std::mutex>(g_side_mu);
-        side = side_stream_locked();
-        if (!side) side_lock.unlock();
-    }
-    cudaStream_t st0 = side ? side->st : st;
-    if (side) {
-        NATSL_TRY(cudaEventRecord(side->fork, st));
-        NATSL_TRY(cudaStreamWaitEvent(st0, side->fork, 0));
-        side_join.forked(side, st);
-    }
-    NATSL_TRY(launch_route_compact(route, f.sm_idx, f.prefix, f.lin_idx, f.n_lin, f.sm_len, nullptr,
-                                   block ? f.status : nullptr, p->L, p->B, p->L, p->H, st0));
     const HeadGroups hg = head_groups(p);
-    // fp32 storage: fp32 copies of the inputs; with NATSL_QK_NORM q32, k32 become the L2-normalised rows (everything
-    // of the linear branch reads those), qs32, ks32 the slice-wise RMS-normalised ones (softmax branch).  The
-    // tensor-core kernels normalise inside.
-    const float *qs = f.q32, *ks = f.k32;
-    if (!tensor_cores) {
-        const bool qk = hg.norm_eps < 0.f;
-        NATSL_TRY(launch_to_f32(qk ? q : nullptr, qk ? k : nullptr, v, f.q32, f.k32, f.v32,
-                                (size_t)(B * L * H * d), s.bf16, st));
-        if (!qk) {
-            NATSL_TRY(launch_qk_norm_f32(q, k, s.bf16, f.q32, f.k32, f.qs32, f.ks32, (size_t)(B * L * H), p->d, hg.G,
-                                         hg.norm_eps, st));
-            qs = f.qs32; ks = f.ks32;
-        }
-    }
-    if (tensor_cores)
-        NATSL_TRY(launch_gather_kv_tc(k, v, f.sm_idx, f.prefix, f.k_smb, nullptr, f.v16, f.k16, p->L,
-                                      p->L, false, f.status, s, st0, hg));
-    else
-        NATSL_TRY(launch_gather_kv(ks, f.v32, f.sm_idx, f.prefix, f.k_sm32, f.v_sm32, p->L,
-                                   f.status, s32, st));
     if (tensor_cores) {
+        // (the kernels of natsl_hybrid_fwd, overlapped like there)
+        const bool pdl = !(p->flags & NATSL_SINGLE_STREAM);
         NATSL_TRY(launch_gdn_prepare_tc(q, k, v, g, beta, block ? nullptr : route, p->scale_la, f.tc, f.ex,
-                                        f.status, s, st, hg.norm_eps));
-        // (the side stream joins before the scan, so that the softmax kernel follows the scan directly
-        // and can run beside it as its programmatic dependent, as in natsl_hybrid_fwd)
-        NATSL_TRY(side_join.join());
+                                        f.status, s, st, (int)(kStatusBytes / 4), hg.norm_eps));
+        NATSL_TRY(launch_route_gather_tc(k, v, route, f.sm_idx, f.prefix, nullptr, f.k_smb, nullptr, f.v16, f.k16, p->L,
+                                         p->L, f.emit_flags, s, st, pdl, hg));
         NATSL_TRY(launch_gdn_scan_tc(f.tc, p->scale_la, p->state_in, state_out, ScanOut{f.o_la16, f.o_la, flags},
                                      f.ex, ScanSegments{0, 1, 0, nullptr, nullptr, nullptr}, block_route,
-                                     f.status, s, st));
-    } else {
-        NATSL_TRY(launch_gdn_prepare_simt(f.q32, f.k32, f.v32, g, beta, block ? nullptr : route, p->scale_la,
-                                          f.W, f.U, f.P, f.Abar, f.Gcum, s32, st));
-        NATSL_TRY(launch_gdn_scan_simt(f.q32, f.k32, g, f.W, f.U, f.P, p->scale_la, p->state_in, state_out,
-                                       f.S_c, f.Ut, f.o_la, block_route, s32, st));
-    }
-    NATSL_TRY(side_join.join());
-    if (tensor_cores)
+                                     f.status, s, st, pdl && scan_follows_closely(p)));
         NATSL_TRY(launch_softmax_combine_tc(q, f.k_smb, f.v16, p->L, p->L, f.sm_idx, f.prefix, f.o_la16,
-                                            flags, p->w, p->scale_sm, p->eps, out, f.o_nla, f.lse,
+                                            flags, p->w, p->scale_sm, p->eps, out, f.o_nla, f.lse, nullptr, p->L,
                                             BlockRouting{block_route, k, v}, false, f.status, s, st, hg));
-    else
-        NATSL_TRY(launch_softmax_combine_simt(qs, f.k_sm32, f.v_sm32, p->L, f.sm_idx, f.prefix,
-                                              f.o_la, p->w, p->scale_sm, p->eps, out, f.o_nla,
-                                              f.lse, BlockRouting{block_route, ks, f.v32}, s32, st, hg.G));
+        return NATSL_OK;
+    }
+    NATSL_TRY(cudaMemsetAsync(f.status, 0, f.head_bytes, st));
+    NATSL_TRY(launch_route_compact(route, f.sm_idx, f.prefix, f.lin_idx, f.n_lin, f.sm_len, nullptr,
+                                   block ? f.status : nullptr, p->L, p->B, p->L, p->H, st));
+    // fp32 copies of the inputs; with NATSL_QK_NORM q32, k32 become the L2-normalised rows (everything of the linear
+    // branch reads those), qs32, ks32 the slice-wise RMS-normalised ones (softmax branch)
+    const float *qs = f.q32, *ks = f.k32;
+    const bool qk = hg.norm_eps < 0.f;
+    NATSL_TRY(launch_to_f32(qk ? q : nullptr, qk ? k : nullptr, v, f.q32, f.k32, f.v32,
+                            (size_t)(B * L * H * d), s.bf16, st));
+    if (!qk) {
+        NATSL_TRY(launch_qk_norm_f32(q, k, s.bf16, f.q32, f.k32, f.qs32, f.ks32, (size_t)(B * L * H), p->d, hg.G,
+                                     hg.norm_eps, st));
+        qs = f.qs32; ks = f.ks32;
+    }
+    NATSL_TRY(launch_gather_kv(ks, f.v32, f.sm_idx, f.prefix, f.k_sm32, f.v_sm32, p->L, f.status, s32, st));
+    NATSL_TRY(launch_gdn_prepare_simt(f.q32, f.k32, f.v32, g, beta, block ? nullptr : route, p->scale_la,
+                                      f.W, f.U, f.P, f.Abar, f.Gcum, s32, st));
+    NATSL_TRY(launch_gdn_scan_simt(f.q32, f.k32, g, f.W, f.U, f.P, p->scale_la, p->state_in, state_out,
+                                   f.S_c, f.Ut, f.o_la, block_route, s32, st));
+    NATSL_TRY(launch_softmax_combine_simt(qs, f.k_sm32, f.v_sm32, p->L, f.sm_idx, f.prefix,
+                                          f.o_la, p->w, p->scale_sm, p->eps, out, f.o_nla,
+                                          f.lse, BlockRouting{block_route, ks, f.v32}, s32, st, hg.G));
 #undef NATSL_TRY
     return NATSL_OK;
 }
@@ -503,38 +484,9 @@ int natsl_hybrid_fwd(const void *q, const void *k, const void *v, const float *g
             return cudaEventRecord(static_cast<cudaEvent_t>(p->stage_events[stage++]), st);
         return cudaSuccess;
     };
-    NATSL_TRY(cudaMemsetAsync(f.status, 0, f.head_bytes, st));
-    NATSL_TRY(mark());
-    // Stage 0 (compaction, gather) beside stage 1 (prepare) on the side stream -- unless the caller
-    // asks for one stream or for per-stage events, whose differences are only meaningful in sequence.
-    std::unique_lock<std::mutex> side_lock;
-    SideStream *side = nullptr;
-    SideJoin side_join;
-    if (tensor_cores && !(p->flags & NATSL_SINGLE_STREAM) && !p->stage_events) {
-        side_lock = std::unique_lock<std::mutex>(g_side_mu);
-        side = side_stream_locked();
-        if (!side) side_lock.unlock();
-    }
-    cudaStream_t st0 = side ? side->st : st;
-    if (side) {
-        NATSL_TRY(cudaEventRecord(side->fork, st));
-        NATSL_TRY(cudaStreamWaitEvent(st0, side->fork, 0));
-        side_join.forked(side, st);
-    }
-    int32_t *sm_len = want_cache ? p->sm_len : f.sm_len;
     void *k_sm = want_cache ? p->k_sm : f.k_sm, *v_sm = want_cache ? p->v_sm : f.v_sm;
     const int32_t cap = want_cache ? p->sm_cap : p->L;
     const int32_t capv = append ? p->sm_cap : p->L;          // rows per head of the fp16 V copy
-    NATSL_TRY(launch_route_compact(route, f.sm_idx, f.prefix, f.lin_idx, f.n_lin, sm_len,
-                                   append ? sm_len : nullptr, block ? f.status : nullptr, cap, p->B,
-                                   p->L, p->H, st0));
-    // fp32 storage with NATSL_QK_NORM: normalised copies first (the tensor-core kernels normalise inside)
-    const void *q_la = q, *k_la = k, *q_sm = q, *k_nsm = k;
-    if (!tensor_cores && hg.norm_eps >= 0.f) {
-        NATSL_TRY(launch_qk_norm_f32(q, k, false, f.q_la, f.k_la, f.q_sm, f.k_nsm,
-                                     (size_t)p->B * p->L * p->H, p->d, hg.G, hg.norm_eps, st));
-        q_la = f.q_la; k_la = f.k_la; q_sm = f.q_sm; k_nsm = f.k_nsm;
-    }
     // A cache the call returns keeps the keys as given (the decode step normalises them as it reads them);
     // with the normalisation the softmax kernel then reads a normalised copy in the workspace instead.
     const bool raw_cache = want_cache && hg.norm_eps >= 0.f;
@@ -542,62 +494,79 @@ int natsl_hybrid_fwd(const void *q, const void *k, const void *v, const float *g
     const void *k_soft = raw_cache ? k_norm : k_sm, *v_soft = raw_cache ? f.v_sm : v_sm;
     const int32_t cap_soft = raw_cache ? capv : cap;
     if (tensor_cores) {
-        NATSL_TRY(launch_gather_kv_tc(k, v, f.sm_idx, f.prefix, k_sm, want_cache ? v_sm : nullptr,
-                                      f.v16, raw_cache ? k_norm : nullptr, cap, capv, append, f.status, s, st0,
-                                      hg, raw_cache));
-    } else {
-        if (raw_cache) NATSL_TRY(launch_gather_kv(k, v, f.sm_idx, f.prefix, k_sm, v_sm, cap, f.status, s, st));
-        NATSL_TRY(launch_gather_kv(k_nsm, v, f.sm_idx, f.prefix, raw_cache ? f.k_sm : k_sm,
-                                   raw_cache ? f.v_sm : v_sm, cap_soft, f.status, s, st));
-    }
-    NATSL_TRY(mark());
-    if (tensor_cores) {
-        // block-level routing: every token takes part in the delta rule of its own block
+        // Four kernels (six with a segmented scan):
+        //   prepare (linear branch's set-up) | compaction + gather (softmax branch's), which needs nothing of it and,
+        //   as its programmatic dependent, runs where its last wave leaves room, | scan, which waits for both, |
+        //   softmax branch + combination, a programmatic dependent of the scan: it starts once the scan's CTAs are
+        //   all resident, runs its Q K^T / P V loop beside it on the multiprocessors the scan leaves free, and picks
+        //   up o_la chunk by chunk behind the counters the scan raises.
+        // Per-stage events and NATSL_SINGLE_STREAM switch the overlap off (kernels in sequence).
         const bool beside = !p->stage_events && !(p->flags & NATSL_SINGLE_STREAM);
         const int nseg = scan_segments(p);
-        NATSL_TRY(launch_gdn_prepare_tc(q, k, v, g, beta, block ? nullptr : route, p->scale_la, f.tc,
-                                        GdnTcExport{}, f.status, s, st, hg.norm_eps));
+        const bool pdl = beside && scan_follows_closely(p);
+        auto prepare = [&]() {   // block-level routing: every token takes part in the delta rule of its own block
+            return launch_gdn_prepare_tc(q, k, v, g, beta, block ? nullptr : route, p->scale_la, f.tc, GdnTcExport{},
+                                         f.status, s, st, (int)(kStatusBytes / 4), hg.norm_eps);
+        };
+        auto gather = [&]() {
+            return launch_route_gather_tc(k, v, route, f.sm_idx, f.prefix, append ? p->sm_len : nullptr, k_sm,
+                                          want_cache ? v_sm : nullptr, f.v16, raw_cache ? k_norm : nullptr, cap, capv,
+                                          f.emit_flags, s, st, beside, hg, raw_cache);
+        };
         NATSL_TRY(mark());
-        // The side stream joins here, before the scan, so that nothing stands between the scan and
-        // the softmax kernel in the stream: the softmax kernel is launched as a programmatic dependent
-        // of the scan, starts once the scan's CTAs are all resident, runs its Q K^T / P V loop beside
-        // it on the multiprocessors the scan leaves free, and picks up o_la chunk by chunk behind the
-        // counters the scan raises.  Per-stage events and NATSL_SINGLE_STREAM switch this off
-        // (stages in sequence).
-        NATSL_TRY(side_join.join());
+        NATSL_TRY(beside ? prepare() : gather());    // (in sequence: in the order of the stages' names)
+        NATSL_TRY(mark());
+        NATSL_TRY(beside ? gather() : prepare());
+        NATSL_TRY(mark());
         int32_t *flags_scan = beside && !g_debug_withhold_flags.load(std::memory_order_relaxed) ? f.emit_flags : nullptr;
         const int32_t *flags_softmax = beside ? f.emit_flags : nullptr;
         const ScanOut so{f.o_la16, p->o_la, flags_scan};
         if (nseg > 1) {   // few (batch, head) pairs: segments in parallel, chained by their transitions
             ScanSegments sg{1, nseg, (int)(p->L / kC) / nseg, f.seg_incr, f.seg_trans, f.seg_start};
             NATSL_TRY(launch_gdn_scan_tc(f.tc, p->scale_la, nullptr, nullptr, so, GdnTcExport{}, sg,
-                                         br.route, f.status, s, st));
-            NATSL_TRY(launch_scan_combine(p->state_in, sg, s, st));
+                                         br.route, f.status, s, st, pdl));
+            NATSL_TRY(launch_scan_combine(p->state_in, sg, s, st, pdl));
             sg.mode = 2;
             NATSL_TRY(launch_gdn_scan_tc(f.tc, p->scale_la, nullptr, p->state_out, so, GdnTcExport{}, sg,
-                                         br.route, f.status, s, st));
+                                         br.route, f.status, s, st, pdl));
         } else {
             NATSL_TRY(launch_gdn_scan_tc(f.tc, p->scale_la, p->state_in, p->state_out, so, GdnTcExport{},
                                          ScanSegments{0, 1, 0, nullptr, nullptr, nullptr}, br.route,
-                                         f.status, s, st));
+                                         f.status, s, st, pdl));
         }
         NATSL_TRY(mark());
         NATSL_TRY(launch_softmax_combine_tc(q, k_soft, f.v16, cap_soft, capv, f.sm_idx, f.prefix, f.o_la16,
                                             flags_softmax, p->w, p->scale_sm, p->eps, out, p->o_nla,
-                                            p->lse, br, append, f.status, s, st, hg));
-    } else {
-        float *o_la = p->o_la ? p->o_la : f.o_la;
-        NATSL_TRY(launch_gdn_prepare_simt(q_la, k_la, v, g, beta, block ? nullptr : route, p->scale_la, f.W,
-                                          f.U, f.P, nullptr, nullptr, s, st));
+                                            p->lse, want_cache ? p->sm_len : nullptr, cap, br, append, f.status, s, st, hg));
         NATSL_TRY(mark());
-        NATSL_TRY(launch_gdn_scan_simt(q_la, k_la, g, f.W, f.U, f.P, p->scale_la, p->state_in,
-                                       p->state_out, nullptr, nullptr, o_la, br.route, s, st));
-        NATSL_TRY(mark());
-        // (an own-block tile of block-level routing reads the layer's keys: the softmax operation's copy)
-        NATSL_TRY(launch_softmax_combine_simt(q_sm, k_soft, v_soft, cap_soft, f.sm_idx, f.prefix, o_la, p->w,
-                                              p->scale_sm, p->eps, out, p->o_nla, p->lse,
-                                              BlockRouting{br.route, k_nsm, v}, s, st, hg.G));
+        return NATSL_OK;
     }
+    NATSL_TRY(cudaMemsetAsync(f.status, 0, f.head_bytes, st));
+    NATSL_TRY(mark());
+    NATSL_TRY(launch_route_compact(route, f.sm_idx, f.prefix, f.lin_idx, f.n_lin, want_cache ? p->sm_len : f.sm_len, nullptr,
+                                   block ? f.status : nullptr, cap, p->B, p->L, p->H, st));
+    // NATSL_QK_NORM: normalised copies first
+    const void *q_la = q, *k_la = k, *q_sm = q, *k_nsm = k;
+    if (hg.norm_eps >= 0.f) {
+        NATSL_TRY(launch_qk_norm_f32(q, k, false, f.q_la, f.k_la, f.q_sm, f.k_nsm,
+                                     (size_t)p->B * p->L * p->H, p->d, hg.G, hg.norm_eps, st));
+        q_la = f.q_la; k_la = f.k_la; q_sm = f.q_sm; k_nsm = f.k_nsm;
+    }
+    if (raw_cache) NATSL_TRY(launch_gather_kv(k, v, f.sm_idx, f.prefix, k_sm, v_sm, cap, f.status, s, st));
+    NATSL_TRY(launch_gather_kv(k_nsm, v, f.sm_idx, f.prefix, raw_cache ? f.k_sm : k_sm,
+                               raw_cache ? f.v_sm : v_sm, cap_soft, f.status, s, st));
+    NATSL_TRY(mark());
+    float *o_la = p->o_la ? p->o_la : f.o_la;
+    NATSL_TRY(launch_gdn_prepare_simt(q_la, k_la, v, g, beta, block ? nullptr : route, p->scale_la, f.W,
+                                      f.U, f.P, nullptr, nullptr, s, st));
+    NATSL_TRY(mark());
+    NATSL_TRY(launch_gdn_scan_simt(q_la, k_la, g, f.W, f.U, f.P, p->scale_la, p->state_in,
+                                   p->state_out, nullptr, nullptr, o_la, br.route, s, st));
+    NATSL_TRY(mark());
+    // (an own-block tile of block-level routing reads the layer's keys: the softmax operation's copy)
+    NATSL_TRY(launch_softmax_combine_simt(q_sm, k_soft, v_soft, cap_soft, f.sm_idx, f.prefix, o_la, p->w,
+                                          p->scale_sm, p->eps, out, p->o_nla, p->lse,
+                                          BlockRouting{br.route, k_nsm, v}, s, st, hg.G));
     NATSL_TRY(mark());
 #undef NATSL_TRY
     return NATSL_OK;

@@ -882,8 +882,6 @@ static cudaError_t combine_bwd_impl(const float *o_la, const float *o_nla, const
 }
 
 cudaError_t launch_dout_amax(const void *dout, size_t n, bool bf16, int32_t *status, cudaStream_t st) {
-    cudaError_t e = cudaMemsetAsync(status + kGradAmaxWord, 0, sizeof(int32_t), st);
-    if (e != cudaSuccess) return e;
     const size_t n4 = n / 4;
     const unsigned blocks = (unsigned)((n4 + 255) / 256 < 1184 ? (n4 + 255) / 256 : 1184);
     if (bf16) dout_amax_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>((const __nv_bfloat16 *)dout, n4, status);

@@ -86,7 +86,7 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                       const float *__restrict__ beta, const uint8_t *__restrict__ route,
                       float scale_la, __half *__restrict__ Wt, float *__restrict__ Ut,
                       __half *__restrict__ Ph, float *__restrict__ Gd, GdnTcExport ex,
-                      int32_t *status, int L, int H, float norm_eps, int wait_kcycles) {
+                      int32_t *status, int head_words, int L, int H, float norm_eps, int wait_kcycles) {
     using PL = PrepLayout<D>;
     constexpr int KB = PL::KB;
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -114,6 +114,11 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
         ms.wait_kcycles = wait_kcycles;
         fence_mbar_init();
     }
+    // The forward's first kernel: clears the status page.  The compaction behind it needs nothing of this kernel and
+    // may start as soon as the last CTAs have (it fills the multiprocessors as they drain); the scan waits for both.
+    if (blockIdx.x == 0 && tid < head_words) status[tid] = 0;
+    __threadfence();
+    launch_dependents();
     if (warp == 4) tmem_alloc(&ms.tmem_base, 128);
     tc_fence_before_sync();
     __syncthreads();
@@ -578,9 +583,6 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
                    GdnTcExport ex, ScanSegments sg,
                    const uint8_t *__restrict__ block_route, int32_t *status, int L, int H, int wait_kcycles) {
     using SL = ScanLayout<D>;
-    // A kernel launched behind this one as a programmatic dependent (the softmax branch) may start
-    // as soon as every CTA of this grid is resident; it reads o_la chunk by chunk behind emit_flags.
-    launch_dependents();
     constexpr int KB = SL::KB;
     constexpr int kHalfCols = D / 2;                       // state columns per thread
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -618,6 +620,11 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
     tc_fence_after_sync();
     const uint32_t tmem = ms.tmem_base;
     volatile int *abort_flag = &ms.abort_flag;
+    // Everything before this kernel in the stream has ended from here on.  A kernel launched behind this one as a
+    // programmatic dependent (the softmax branch) may start as soon as every CTA of this grid is here; it reads o_la
+    // chunk by chunk behind emit_flags.
+    grid_dependency_wait();
+    launch_dependents();
 
     if (warp == 9) {
         if (lane == 0) {
@@ -936,6 +943,8 @@ scan_combine_kernel(const float *__restrict__ state_in, const float *__restrict_
     constexpr int kV = kCombCols, kHalf = D / 2;
     __shared__ float4 Ss[2][D];                        // the state's kV columns, double-buffered
     const int bh = blockIdx.y, v0 = blockIdx.x * kV, a = threadIdx.x >> 1, hf = threadIdx.x & 1;
+    grid_dependency_wait();
+    launch_dependents();
     // this thread's half of the row: pieces 2 j + hf (16 bytes each), so that a pair reads 32 contiguous bytes
     float4 m[kHalf / 4];
     auto fetch = [&](int sgi) {
@@ -979,10 +988,11 @@ scan_combine_kernel(const float *__restrict__ state_in, const float *__restrict_
 
 }  // namespace
 
-cudaError_t launch_scan_combine(const float *state_in, const ScanSegments &sg, Shape s, cudaStream_t st) {
+cudaError_t launch_scan_combine(const float *state_in, const ScanSegments &sg, Shape s, cudaStream_t st, bool pdl) {
     dim3 grid(s.d / kCombCols, s.B * s.H);
-    if (s.d == 128) scan_combine_kernel<128><<<grid, 256, 0, st>>>(state_in, sg.incr, sg.trans, sg.start, sg.nseg);
-    else scan_combine_kernel<64><<<grid, 128, 0, st>>>(state_in, sg.incr, sg.trans, sg.start, sg.nseg);
+    auto kernel = s.d == 128 ? scan_combine_kernel<128> : scan_combine_kernel<64>;
+    cudaError_t e = launch_kernel(kernel, grid, dim3(2 * s.d), 0, st, pdl, state_in, sg.incr, sg.trans, sg.start, sg.nseg);
+    if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
 }
@@ -991,7 +1001,7 @@ template <int D>
 static cudaError_t prepare_tc_impl(const void *q, const void *k, const void *v, const float *g,
                                    const float *beta, const uint8_t *route, float scale_la,
                                    const GdnTcWs &ws, const GdnTcExport &ex, int32_t *status,
-                                   float norm_eps, Shape s, cudaStream_t st) {
+                                   float norm_eps, int head_words, Shape s, cudaStream_t st) {
     const int NC = s.L / kC;
     const uint64_t BH = (uint64_t)s.B * s.H;
     CUtensorMap mq, mk, mv, mqh, mkh;
@@ -1005,18 +1015,17 @@ static cudaError_t prepare_tc_impl(const void *q, const void *k, const void *v, 
                                          PrepLayout<D>::kTotal);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)NC * (unsigned)BH);
-    gdn_prepare_tc_kernel<D><<<grid, kPrepThreads, PrepLayout<D>::kTotal, st>>>(
-        mq, mk, mv, mqh, mkh, g, beta, route, scale_la, (__half *)ws.Wt, ws.Ut, (__half *)ws.Ph, ws.Gd, ex,
-        status, s.L, s.H, norm_eps, debug_wait_kcycles());
     count_launch();
-    return cudaGetLastError();
+    return launch_kernel(gdn_prepare_tc_kernel<D>, grid, dim3(kPrepThreads), PrepLayout<D>::kTotal, st, false, mq, mk, mv, mqh,
+                         mkh, g, beta, route, scale_la, (__half *)ws.Wt, ws.Ut, (__half *)ws.Ph, ws.Gd, ex, status,
+                         head_words, s.L, s.H, norm_eps, debug_wait_kcycles());
 }
 
 template <int D>
 static cudaError_t scan_tc_impl(const GdnTcWs &ws, float scale_la, const float *state_in,
                                 float *state_out, const ScanOut &out, const GdnTcExport &ex,
                                 const ScanSegments &sg, const uint8_t *block_route, int32_t *status,
-                                Shape s, cudaStream_t st) {
+                                Shape s, cudaStream_t st, bool pdl) {
     const int NC = s.L / kC;
     const uint64_t BH = (uint64_t)s.B * s.H;
     CUtensorMap mwt, mqh, mkh, mph;
@@ -1030,28 +1039,28 @@ static cudaError_t scan_tc_impl(const GdnTcWs &ws, float scale_la, const float *
                                          ScanLayout<D>::kTotal);
     if (e != cudaSuccess) return e;
     const int ctas = s.B * s.H * (sg.mode == 0 ? 1 : sg.nseg) * (sg.mode == 1 ? 2 : 1);
-    kernel<<<ctas, kScanThreads, ScanLayout<D>::kTotal, st>>>(
-        mwt, mqh, mkh, mph, ws.Ut, ws.Gd, scale_la, state_in, state_out, (__half *)out.o_la16, out.o_la32,
-        out.emit_flags, ex, sg, block_route, status, s.L, s.H, debug_wait_kcycles());
     count_launch();
-    return cudaGetLastError();
+    return launch_kernel(kernel, dim3(ctas), dim3(kScanThreads), ScanLayout<D>::kTotal, st, pdl, mwt, mqh, mkh, mph, ws.Ut,
+                         ws.Gd, scale_la, state_in, state_out, (__half *)out.o_la16, out.o_la32, out.emit_flags, ex, sg,
+                         block_route, status, s.L, s.H, debug_wait_kcycles());
 }
 
 cudaError_t launch_gdn_prepare_tc(const void *q, const void *k, const void *v, const float *g,
                                   const float *beta, const uint8_t *route, float scale_la,
                                   const GdnTcWs &ws, const GdnTcExport &ex, int32_t *status, Shape s,
-                                  cudaStream_t st, float norm_eps) {
-    if (s.d == 128) return prepare_tc_impl<128>(q, k, v, g, beta, route, scale_la, ws, ex, status, norm_eps, s, st);
-    return prepare_tc_impl<64>(q, k, v, g, beta, route, scale_la, ws, ex, status, norm_eps, s, st);
+                                  cudaStream_t st, int head_words, float norm_eps) {
+    if (s.d == 128)
+        return prepare_tc_impl<128>(q, k, v, g, beta, route, scale_la, ws, ex, status, norm_eps, head_words, s, st);
+    return prepare_tc_impl<64>(q, k, v, g, beta, route, scale_la, ws, ex, status, norm_eps, head_words, s, st);
 }
 
 cudaError_t launch_gdn_scan_tc(const GdnTcWs &ws, float scale_la, const float *state_in,
                                float *state_out, const ScanOut &out, const GdnTcExport &ex,
                                const ScanSegments &sg, const uint8_t *block_route, int32_t *status,
-                               Shape s, cudaStream_t st) {
+                               Shape s, cudaStream_t st, bool pdl) {
     if (s.d == 128)
-        return scan_tc_impl<128>(ws, scale_la, state_in, state_out, out, ex, sg, block_route, status, s, st);
-    return scan_tc_impl<64>(ws, scale_la, state_in, state_out, out, ex, sg, block_route, status, s, st);
+        return scan_tc_impl<128>(ws, scale_la, state_in, state_out, out, ex, sg, block_route, status, s, st, pdl);
+    return scan_tc_impl<64>(ws, scale_la, state_in, state_out, out, ex, sg, block_route, status, s, st, pdl);
 }
 
 }  // namespace natsl

@@ -86,19 +86,21 @@ cudaError_t launch_qk_norm_bwd_f32(const void *q, const void *k, bool bf16, cons
 // dv_in converted when given.  In place is fine for fp32 storage: dq_la == dq, dk_in == dk.)
 
 // softmax_tc.cu -- tensor-core softmax branch + combination (bf16 storage)
-cudaError_t launch_gather_kv_tc(const void *k, const void *v, const int32_t *sm_idx,
-                                const int32_t *sm_chunk_prefix, void *k_sm, void *v_sm, void *v16,
-                                void *k16, int32_t cap, int32_t capv, bool appending, int32_t *status,
-                                Shape s, cudaStream_t st, HeadGroups hg = HeadGroups{}, bool raw_k_sm = false);
+// Route compaction and gather in one kernel, which also clears emit_flags; base_in as in launch_route_compact.
+cudaError_t launch_route_gather_tc(const void *k, const void *v, const uint8_t *route, int32_t *sm_idx,
+                                   int32_t *sm_chunk_prefix, const int32_t *base_in, void *k_sm, void *v_sm, void *v16,
+                                   void *k16, int32_t cap, int32_t capv, int32_t *emit_flags, Shape s, cudaStream_t st,
+                                   bool pdl, HeadGroups hg = HeadGroups{}, bool raw_k_sm = false);
 // (hg.norm_eps >= 0: the keys are RMS-normalised per softmax head and stored as fp16 -- in k_sm and k16, or,
 // with raw_k_sm, in k16 only while k_sm, a cache handed on to the decode step, keeps them as given)
 cudaError_t launch_softmax_combine_tc(const void *q, const void *k_sm, const void *v16, int32_t cap,
                                       int32_t capv, const int32_t *sm_idx,
                                       const int32_t *sm_chunk_prefix, const void *o_la16,
                                       const int32_t *emit_flags, const float *w, float scale_sm,
-                                      float eps, void *out, float *o_nla, float *lse, BlockRouting br,
-                                      bool appending, int32_t *status, Shape s, cudaStream_t st,
+                                      float eps, void *out, float *o_nla, float *lse, int32_t *sm_len, int len_cap,
+                                      BlockRouting br, bool appending, int32_t *status, Shape s, cudaStream_t st,
                                       HeadGroups hg = HeadGroups{});
+// (sm_len [B,H] or nullptr: receives the retained tokens, at most len_cap; more are NATSL_ERR_CACHE_FULL)
 // (o_la16: the linear branch's read-out, o_laT [B,H,L/C,8,d,8] fp16; emit_flags: see ScanOut -- when given, the
 // kernel is launched as a programmatic dependent of the kernel before it in the stream, the scan)
 // cudaFuncSetAttribute(max dynamic shared memory) of a kernel, once per thread, device and size: the call
@@ -106,6 +108,21 @@ cudaError_t launch_softmax_combine_tc(const void *q, const void *k_sm, const voi
 cudaError_t allow_smem_of(const void *kernel, int bytes);
 template <typename K> cudaError_t allow_smem(K *kernel, size_t bytes) {
     return allow_smem_of(reinterpret_cast<const void *>(kernel), (int)bytes);
+}
+// A launch, as a programmatic dependent of the kernel before it in the stream when pdl is set.
+template <typename... P, typename... A>
+cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl, A &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 int sm_count();   // multiprocessors of the current device (cached per device)
 // Bound of the device-side waits in units of 1024 cycles, 0 = the default (about two seconds);
@@ -153,7 +170,10 @@ struct GdnTcGrads {
 cudaError_t launch_gdn_prepare_tc(const void *q, const void *k, const void *v, const float *g,
                                   const float *beta, const uint8_t *route, float scale_la,
                                   const GdnTcWs &ws, const GdnTcExport &ex, int32_t *status, Shape s,
-                                  cudaStream_t st, float norm_eps = -1.f);
+                                  cudaStream_t st, int head_words, float norm_eps = -1.f);
+// (the forward's first kernel: clears head_words words of the status page)
+// pdl (here and elsewhere): launched as a programmatic dependent of the kernel before it in the stream.  Every kernel of
+// the forward waits for the one before it before it ends, so a kernel that has waited for its predecessor sees all of them.
 // Splitting the scan of one (batch, head) over several CTAs when there are few (batch, head)
 // pairs.  The state recurrence S <- (gamma_C I - K~^T W) S + K~^T U is affine in S with a factor
 // that acts on the key dimension only, so a segment of chunks maps its entry state S0 to
@@ -183,8 +203,8 @@ constexpr int kScanRowWarps = 8;
 cudaError_t launch_gdn_scan_tc(const GdnTcWs &ws, float scale_la, const float *state_in,
                                float *state_out, const ScanOut &out, const GdnTcExport &ex,
                                const ScanSegments &sg, const uint8_t *block_route, int32_t *status,
-                               Shape s, cudaStream_t st);
-cudaError_t launch_scan_combine(const float *state_in, const ScanSegments &sg, Shape s, cudaStream_t st);
+                               Shape s, cudaStream_t st, bool pdl = false);
+cudaError_t launch_scan_combine(const float *state_in, const ScanSegments &sg, Shape s, cudaStream_t st, bool pdl = false);
 
 // bwd_simt.cu -- fp32 CUDA-core backward
 // A batched matrix operand: element (r, c) of batch (b, h, chunk) is
@@ -208,7 +228,7 @@ cudaError_t launch_combine_bwd(const float *o_la, const float *o_nla, const void
                                float *Dsm, void *do16, void *dola16, void *dolag16, const float *Gd,
                                float scale_la, const int32_t *gsc, Shape s, cudaStream_t st, int G = 1);
 // (G > 1: the softmax branch's output was normalised per slice of d / G columns; Dsm is [B,H,G,L])
-// max |dout| (n elements) into word kGradAmaxWord of the status page (zeroed first)
+// max |dout| (n elements) into word kGradAmaxWord of the status page (cleared with the page by the forward)
 cudaError_t launch_dout_amax(const void *dout, size_t n, bool bf16, int32_t *status, cudaStream_t st);
 cudaError_t launch_softmax_bwd(const float *q32, const float *k_sm32, const float *v_sm32, int cap,
                                const int32_t *sm_idx, const int32_t *sm_chunk_prefix,

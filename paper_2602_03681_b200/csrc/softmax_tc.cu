@@ -132,7 +132,8 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                           const __half *__restrict__ o_laT, const int32_t *emit_flags,
                           const float *__restrict__ w,
                           float scale_sm, float eps, float norm_eps, int has_out, float *__restrict__ o_nla,
-                          float *__restrict__ lse, int32_t *status, int L, int H, int wait_kcycles) {
+                          float *__restrict__ lse, int32_t *sm_len, int len_cap, int32_t *status, int L, int H,
+                          int wait_kcycles) {
     using SL = SmLayout<D>;
     constexpr int KB = SL::KB, kStages = SL::kStages, kLogits = SL::kLogits, kGroups = SL::kGroups;
     constexpr int kSoftmaxThreads = SL::kSoftmaxThreads, kAhead = kLogits - 1;
@@ -205,6 +206,21 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
     const int T2 = kBlock ? T + nx : T;
     auto own_block = [&](int t) { return t == T ? xc0 : 1; };   // block (0 or 1) of own-block tile t >= T
 
+    if (sg == 0 && tid == 0) {
+        // Block-level routing: one decision per chunk, so a chunk keeps all of its tokens or none.
+        if (kBlock)
+            for (int e = c0; e < c1; ++e) {
+                const int n = pre[e + 1] - pre[e];
+                if (n != 0 && n != kC) atomicMin(status, (int)NATSL_ERR_ROUTE);
+            }
+        // The stored length never exceeds the rows the cache has (the gather stops there and the overflow is
+        // reported), so a later decode step cannot be led past the head's rows.
+        if (c1 == NC) {
+            const int n = pre[NC];
+            if (n > len_cap) atomicMin(status, (int)NATSL_ERR_CACHE_FULL);
+            if (sm_len) sm_len[bh] = min(n, len_cap);
+        }
+    }
     if (tid < kBM / 32) ms.kept[tid] = 0u;
     if (tid < kBM) ms.m_row[tid] = -INFINITY;
     if (warp == kMmaWarp) tmem_alloc(&ms.tmem_base, 256);
@@ -615,32 +631,84 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
     if (tid == 0 && ms.abort_flag) atomicMin(status, (int)NATSL_ERR_TIMEOUT);
 }
 
-// Copy the retained tokens' K rows (bf16) and V rows (as fp16) into the compacted layouts
-// [B,H,cap,d] / [B,H,capv,d] (optionally K as fp16 too, for the backward) and zero the fp16 rows
-// up to the next multiple of 128, so that a K/V tile never multiplies a zero probability or a
-// zero logit gradient with an uninitialised value.  grid = (row blocks, B*H).
+// Route compaction and gather of the retained K/V in one kernel (the softmax branch's half of the forward's
+// set-up; grid = (slices of the chunks, B*H)).  A CTA counts the retained tokens before its slice itself -- route
+// bytes out of L2, a few microseconds however long the sequence, where one CTA per (batch, head) walking all chunks
+// took 28 us at 512 chunks --, lists its own chunks' retained tokens (one 64-bit ballot word per chunk) and copies
+// their K rows (bf16) and V rows (as fp16) into the compacted layouts [B,H,cap,d] / [B,H,capv,d] (optionally K as
+// fp16 too, for the backward).  The fp16 rows behind the last one are zeroed up to the next multiple of 128, so
+// that a K/V tile never multiplies a zero probability or a zero logit gradient with an uninitialised value.
+// It also clears the scan's per-chunk counters of the call.  It needs nothing of the prepare kernel before it in
+// the stream and is its programmatic dependent, so that it runs where that kernel's last wave leaves room; it only
+// must not end before it, since the scan waits for this kernel.
+constexpr int kRouteThreads = 256;
+constexpr int kMaxSlice = 32;                        // chunks per CTA
+struct RouteArgs {
+    const uint8_t *route;
+    int32_t *sm_idx, *prefix, *emit_flags;
+    const int32_t *base_in;                          // [B,H] entries the cache already holds, or nullptr
+};
 template <int D>
-__global__ void __launch_bounds__(256)
-gather_kv_tc_kernel(const __nv_bfloat16 *__restrict__ k, const __nv_bfloat16 *__restrict__ v,
-                    const int32_t *__restrict__ sm_idx, const int32_t *__restrict__ sm_chunk_prefix,
+__global__ void __launch_bounds__(kRouteThreads)
+route_gather_kernel(const __nv_bfloat16 *__restrict__ k, const __nv_bfloat16 *__restrict__ v, const RouteArgs ra,
                     __nv_bfloat16 *__restrict__ k_sm, __nv_bfloat16 *__restrict__ v_sm,
-                    __half *__restrict__ v16, __half *__restrict__ k16, int cap, int capv, int appending,
-                    int groups, float norm_eps, int raw_k_sm, int32_t *status, int L, int H) {
+                    __half *__restrict__ v16, __half *__restrict__ k16, int cap, int capv, int slice_chunks,
+                    int groups, float norm_eps, int raw_k_sm, int L, int H) {
     // raw_k_sm (with the normalisation): k_sm is a cache that keeps the keys as given; the normalised
     // fp16 keys then go to k16 only
     constexpr int kVecPerRow = D * 2 / 16;
-    constexpr int kRows = 256 / kVecPerRow;
-    const int bh = blockIdx.y, b = bh / H, h = bh % H;
-    const int NC = L / kC;
-    const int n_sm = sm_chunk_prefix[(size_t)bh * (NC + 1) + NC];
-    if (blockIdx.x == 0 && threadIdx.x == 0 && n_sm > cap) atomicMin(status, (int)NATSL_ERR_CACHE_FULL);
-    const int n = min(n_sm, cap);
-    const int n_pad = min((n + 127) / 128 * 128, capv);
-    const int n_prev = appending ? sm_chunk_prefix[(size_t)bh * (NC + 1)] : 0;   // rows of earlier calls
-    const int piece = threadIdx.x % kVecPerRow;
+    constexpr int kRows = kRouteThreads / kVecPerRow;
+    __shared__ int list[kMaxSlice * kC];
+    __shared__ int counts[kMaxSlice], wsum[kRouteThreads / 32];
+    const int bh = blockIdx.y, b = bh / H, h = bh % H, NC = L / kC;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int c_lo = blockIdx.x * slice_chunks, nc = min(slice_chunks, NC - c_lo);
+    const uint8_t *rt = ra.route + (size_t)b * L * H + h;
+    launch_dependents();
+    for (int i = tid; i < nc; i += kRouteThreads) ra.emit_flags[(size_t)bh * NC + c_lo + i] = 0;
+    // ---- own chunks' ballots, and the count of everything before them ----
+    for (int c = warp; c < nc; c += kRouteThreads / 32) {
+        const size_t l0 = (size_t)(c_lo + c) * kC;
+        const uint8_t a0 = rt[(l0 + lane) * H], a1 = rt[(l0 + 32 + lane) * H];
+        const unsigned lo = __ballot_sync(0xffffffffu, a0 != 0), hi = __ballot_sync(0xffffffffu, a1 != 0);
+        const unsigned lt = (1u << lane) - 1u;
+        const int nlo = __popc(lo);
+        if (a0) list[c * kC + __popc(lo & lt)] = (int)l0 + lane;          // compacted within the chunk's 64 places
+        if (a1) list[c * kC + nlo + __popc(hi & lt)] = (int)l0 + 32 + lane;
+        if (lane == 0) counts[c] = nlo + __popc(hi);
+    }
+    int before = 0;
+    const int n_before = c_lo * kC;
+    for (int l = tid; l < n_before; l += 8 * kRouteThreads) {             // eight loads in flight
+        uint8_t x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int ll = l + u * kRouteThreads;
+            x[u] = ll < n_before ? rt[(size_t)ll * H] : (uint8_t)0;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) before += x[u] != 0;
+    }
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (lane == 0) wsum[warp] = before;
+    __syncthreads();
+    const int base0 = ra.base_in ? ra.base_in[bh] : 0;
+    int base = base0;
+#pragma unroll
+    for (int wv = 0; wv < kRouteThreads / 32; ++wv) base += wsum[wv];
+    int mine = 0;                                                         // retained tokens of the slice
+    for (int c = 0; c < nc; ++c) mine += counts[c];
+    const bool last = c_lo + nc == NC;
+    if (tid < nc) {
+        int pre = base;
+        for (int c = 0; c < tid; ++c) pre += counts[c];
+        ra.prefix[(size_t)bh * (NC + 1) + c_lo + tid] = pre;
+    }
+    if (last && tid == 0) ra.prefix[(size_t)bh * (NC + 1) + NC] = base + mine;
     // RMS-normalised keys of the softmax operation (Section 4.3), per softmax head = per slice of D / groups
     // columns, as fp16 (the softmax kernel's logit product is an fp16 MMA in this mode): the slice's pieces
     // sit in neighbouring lanes of the row's lanes.  bf16 pieces in, fp16 pieces out.
+    const int piece = tid % kVecPerRow;
     auto rms_fp16 = [&](uint4 kk) {
         const uint32_t kw[4] = {kk.x, kk.y, kk.z, kk.w};
         float f[8], ss = 0.f;
@@ -658,53 +726,57 @@ gather_kv_tc_kernel(const __nv_bfloat16 *__restrict__ k, const __nv_bfloat16 *__
         return make_uint4(pack_half2(f[0] * rk, f[1] * rk), pack_half2(f[2] * rk, f[3] * rk),
                           pack_half2(f[4] * rk, f[5] * rk), pack_half2(f[6] * rk, f[7] * rk));
     };
-    // the grid is sized for a typical retention rate; each CTA strides over the rows there are
-    for (int row = blockIdx.x * kRows + threadIdx.x / kVecPerRow; row < n_pad; row += gridDim.x * kRows) {
-        uint4 *dv16 = reinterpret_cast<uint4 *>(v16 + ((size_t)bh * capv + row) * D) + piece;
-        uint4 *dk16 = k16 ? reinterpret_cast<uint4 *>(k16 + ((size_t)bh * capv + row) * D) + piece : nullptr;
-        if (row >= n) {
-            *dv16 = make_uint4(0u, 0u, 0u, 0u);
-            if (dk16) *dk16 = make_uint4(0u, 0u, 0u, 0u);
-            continue;
-        }
-        const size_t dst = ((size_t)bh * cap + row) * D;
-        if (row < n_prev) {     // already in the cache: only the fp16 copy of its V row is made
-            const uint4 vv = reinterpret_cast<const uint4 *>(v_sm + dst)[piece];
-            const uint32_t wv[4] = {vv.x, vv.y, vv.z, vv.w};
-            uint32_t o[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                o[i] = pack_half2(__uint_as_float(wv[i] << 16), __uint_as_float(wv[i] & 0xffff0000u));
-            *dv16 = make_uint4(o[0], o[1], o[2], o[3]);
-            // (and, with the normalisation, the normalised copy of its key, which the cache keeps as given)
-            if (dk16 && norm_eps >= 0.f) *dk16 = rms_fp16(reinterpret_cast<const uint4 *>(k_sm + dst)[piece]);
-            continue;
-        }
-        const int tok = sm_idx[(size_t)bh * L + row - n_prev];
-        const size_t src = (((size_t)b * L + tok) * H + h) * D;
-        uint4 kk = reinterpret_cast<const uint4 *>(k + src)[piece];
-        if (norm_eps >= 0.f && raw_k_sm) reinterpret_cast<uint4 *>(k_sm + dst)[piece] = kk;
-        if (norm_eps >= 0.f) kk = rms_fp16(kk);
-        if (!(norm_eps >= 0.f && raw_k_sm)) reinterpret_cast<uint4 *>(k_sm + dst)[piece] = kk;
-        if (dk16 && norm_eps >= 0.f) {
-            *dk16 = kk;                                   // already fp16
-        } else if (dk16) {
-            const uint32_t kw[4] = {kk.x, kk.y, kk.z, kk.w};
-            uint32_t ko[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                ko[i] = pack_half2(__uint_as_float(kw[i] << 16), __uint_as_float(kw[i] & 0xffff0000u));
-            *dk16 = make_uint4(ko[0], ko[1], ko[2], ko[3]);
-        }
-        const uint4 vv = reinterpret_cast<const uint4 *>(v + src)[piece];
-        if (v_sm) reinterpret_cast<uint4 *>(v_sm + dst)[piece] = vv;
-        const uint32_t wv[4] = {vv.x, vv.y, vv.z, vv.w};
+    auto to_fp16 = [](uint4 x) {
+        const uint32_t w[4] = {x.x, x.y, x.z, x.w};
         uint32_t o[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            o[i] = pack_half2(__uint_as_float(wv[i] << 16), __uint_as_float(wv[i] & 0xffff0000u));
-        *dv16 = make_uint4(o[0], o[1], o[2], o[3]);
+        for (int i = 0; i < 4; ++i) o[i] = pack_half2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xffff0000u));
+        return make_uint4(o[0], o[1], o[2], o[3]);
+    };
+    // ---- the slice's rows: one row per group of kVecPerRow threads, chunk by chunk of the list ----
+    {
+        int row0 = base, c = 0, in_c = tid / kVecPerRow;   // in_c: index within chunk c's list
+        while (true) {
+            while (c < nc && in_c >= counts[c]) { in_c -= counts[c]; row0 += counts[c]; ++c; }
+            if (c >= nc) break;
+            const int row = row0 + in_c, tok = list[c * kC + in_c];
+            if (piece == 0) ra.sm_idx[(size_t)bh * L + row - base0] = tok;
+            if (row < cap) {
+                const size_t dst = ((size_t)bh * cap + row) * D, src = (((size_t)b * L + tok) * H + h) * D;
+                uint4 *dv16 = reinterpret_cast<uint4 *>(v16 + ((size_t)bh * capv + row) * D) + piece;
+                uint4 *dk16 = k16 ? reinterpret_cast<uint4 *>(k16 + ((size_t)bh * capv + row) * D) + piece : nullptr;
+                uint4 kk = reinterpret_cast<const uint4 *>(k + src)[piece];
+                const uint4 vv = reinterpret_cast<const uint4 *>(v + src)[piece];
+                if (norm_eps >= 0.f && raw_k_sm) reinterpret_cast<uint4 *>(k_sm + dst)[piece] = kk;
+                if (norm_eps >= 0.f) kk = rms_fp16(kk);
+                if (!(norm_eps >= 0.f && raw_k_sm)) reinterpret_cast<uint4 *>(k_sm + dst)[piece] = kk;
+                if (dk16) *dk16 = norm_eps >= 0.f ? kk : to_fp16(kk);      // (normalised: already fp16)
+                if (v_sm) reinterpret_cast<uint4 *>(v_sm + dst)[piece] = vv;
+                *dv16 = to_fp16(vv);
+            }
+            in_c += kRows;
+        }
     }
+    // ---- rows of earlier calls: only the fp16 copy of their V rows is made (and, with the normalisation, the
+    // normalised copy of their keys, which the cache keeps as given) ----
+    if (ra.base_in) {
+        const int n_prev = min(base0, cap);
+        for (int row = blockIdx.x * kRows + tid / kVecPerRow; row < n_prev; row += gridDim.x * kRows) {
+            const size_t dst = ((size_t)bh * cap + row) * D, d16 = ((size_t)bh * capv + row) * D;
+            reinterpret_cast<uint4 *>(v16 + d16)[piece] = to_fp16(reinterpret_cast<const uint4 *>(v_sm + dst)[piece]);
+            if (k16 && norm_eps >= 0.f)
+                reinterpret_cast<uint4 *>(k16 + d16)[piece] = rms_fp16(reinterpret_cast<const uint4 *>(k_sm + dst)[piece]);
+        }
+    }
+    if (last) {                                            // zero rows behind the last one
+        const int n = min(base + mine, cap), n_pad = min((n + 127) / 128 * 128, capv);
+        for (int row = n + tid / kVecPerRow; row < n_pad; row += kRows) {
+            const size_t d16 = ((size_t)bh * capv + row) * D;
+            reinterpret_cast<uint4 *>(v16 + d16)[piece] = make_uint4(0u, 0u, 0u, 0u);
+            if (k16) reinterpret_cast<uint4 *>(k16 + d16)[piece] = make_uint4(0u, 0u, 0u, 0u);
+        }
+    }
+    if (tid == 0) grid_dependency_wait();
 }
 
 }  // namespace
@@ -714,7 +786,7 @@ static cudaError_t softmax_tc_impl(const void *q, const void *k_sm, const void *
                                    int32_t capv, const int32_t *sm_idx, const int32_t *pre,
                                    const void *o_la16, const int32_t *emit_flags, const float *w,
                                    float scale_sm, float eps, float norm_eps, void *out, float *o_nla, float *lse,
-                                   BlockRouting br, bool appending, int32_t *status, Shape s,
+                                   int32_t *sm_len, int len_cap, BlockRouting br, bool appending, int32_t *status, Shape s,
                                    cudaStream_t st) {
     using SL = SmLayout<D>;
     CUtensorMap mq, mk, mv, mout, mkd, mvd;
@@ -751,7 +823,7 @@ static cudaError_t softmax_tc_impl(const void *q, const void *k_sm, const void *
     cfg.numAttrs = emit_flags ? 1 : 0;
     e = cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, mout, mkd, mvd, br.route, appending ? 1 : 0,
                            (int)cap, (int)capv, sm_idx, pre, (const __half *)o_la16, emit_flags, w, scale_sm, eps,
-                           norm_eps, out ? 1 : 0, o_nla, lse, status, s.L, s.H, debug_wait_kcycles());
+                           norm_eps, out ? 1 : 0, o_nla, lse, sm_len, len_cap, status, s.L, s.H, debug_wait_kcycles());
     count_launch();
     return e;
 }
@@ -760,44 +832,44 @@ cudaError_t launch_softmax_combine_tc(const void *q, const void *k_sm, const voi
                                       int32_t capv, const int32_t *sm_idx,
                                       const int32_t *sm_chunk_prefix, const void *o_la16,
                                       const int32_t *emit_flags, const float *w, float scale_sm,
-                                      float eps, void *out, float *o_nla, float *lse, BlockRouting br,
-                                      bool appending, int32_t *status, Shape s, cudaStream_t st,
+                                      float eps, void *out, float *o_nla, float *lse, int32_t *sm_len, int len_cap,
+                                      BlockRouting br, bool appending, int32_t *status, Shape s, cudaStream_t st,
                                       HeadGroups hg) {
     if (hg.G == 2 && s.d == 128)
         return softmax_tc_impl<64, 2>(q, k_sm, v16, cap, capv, sm_idx, sm_chunk_prefix, o_la16, emit_flags,
-                                      w, scale_sm, eps, hg.norm_eps, out, o_nla, lse, br, appending, status, s, st);
+                                      w, scale_sm, eps, hg.norm_eps, out, o_nla, lse, sm_len, len_cap, br, appending, status, s, st);
     if (hg.G > 1) return cudaErrorInvalidValue;
     if (s.d == 128)
         return softmax_tc_impl<128, 1>(q, k_sm, v16, cap, capv, sm_idx, sm_chunk_prefix, o_la16, emit_flags,
-                                       w, scale_sm, eps, hg.norm_eps, out, o_nla, lse, br, appending, status, s, st);
+                                       w, scale_sm, eps, hg.norm_eps, out, o_nla, lse, sm_len, len_cap, br, appending, status, s, st);
     return softmax_tc_impl<64, 1>(q, k_sm, v16, cap, capv, sm_idx, sm_chunk_prefix, o_la16, emit_flags, w,
-                                  scale_sm, eps, hg.norm_eps, out, o_nla, lse, br, appending, status, s, st);
+                                  scale_sm, eps, hg.norm_eps, out, o_nla, lse, sm_len, len_cap, br, appending, status, s, st);
 }
 
 template <int D>
-static cudaError_t gather_tc_impl(const void *k, const void *v, const int32_t *sm_idx,
-                                  const int32_t *pre, void *k_sm, void *v_sm, void *v16, void *k16,
-                                  int cap, int capv, bool appending, int32_t *status, Shape s,
-                                  cudaStream_t st, HeadGroups hg, bool raw_k_sm) {
-    constexpr int kRows = 256 / (D * 2 / 16);
-    const int max_rows = s.L < capv ? s.L : capv;
-    const int blocks = (max_rows + kRows - 1) / kRows;
-    dim3 grid(blocks < 48 ? blocks : 48, s.B * s.H);
-    gather_kv_tc_kernel<D><<<grid, 256, 0, st>>>(
-        (const __nv_bfloat16 *)k, (const __nv_bfloat16 *)v, sm_idx, pre, (__nv_bfloat16 *)k_sm,
-        (__nv_bfloat16 *)v_sm, (__half *)v16, (__half *)k16, cap, capv, appending ? 1 : 0, hg.G, hg.norm_eps,
-        raw_k_sm ? 1 : 0, status, s.L, s.H);
+static cudaError_t route_gather_impl(const void *k, const void *v, const RouteArgs &ra, void *k_sm, void *v_sm, void *v16,
+                                     void *k16, int cap, int capv, Shape s, cudaStream_t st, bool pdl, HeadGroups hg, bool raw_k_sm) {
+    // slices of 1 to kMaxSlice chunks: about four CTAs per SM over all (batch, head) pairs, at most 32 per pair (each
+    // counts what lies before it)
+    const int NC = s.L / kC, BH = s.B * s.H;
+    int slices = (4 * 148 + BH - 1) / BH;
+    slices = slices < 1 ? 1 : (slices > 32 ? 32 : slices);
+    int cps = (NC + slices - 1) / slices;
+    if (cps > kMaxSlice) cps = kMaxSlice;
+    dim3 grid((NC + cps - 1) / cps, BH);
     count_launch();
-    return cudaGetLastError();
+    return launch_kernel(route_gather_kernel<D>, grid, dim3(kRouteThreads), 0, st, pdl, (const __nv_bfloat16 *)k,
+                         (const __nv_bfloat16 *)v, ra, (__nv_bfloat16 *)k_sm, (__nv_bfloat16 *)v_sm, (__half *)v16,
+                         (__half *)k16, cap, capv, cps, hg.G, hg.norm_eps, raw_k_sm ? 1 : 0, s.L, s.H);
 }
 
-cudaError_t launch_gather_kv_tc(const void *k, const void *v, const int32_t *sm_idx,
-                                const int32_t *sm_chunk_prefix, void *k_sm, void *v_sm, void *v16,
-                                void *k16, int32_t cap, int32_t capv, bool appending, int32_t *status,
-                                Shape s, cudaStream_t st, HeadGroups hg, bool raw_k_sm) {
-    if (s.d == 128)
-        return gather_tc_impl<128>(k, v, sm_idx, sm_chunk_prefix, k_sm, v_sm, v16, k16, cap, capv, appending, status, s, st, hg, raw_k_sm);
-    return gather_tc_impl<64>(k, v, sm_idx, sm_chunk_prefix, k_sm, v_sm, v16, k16, cap, capv, appending, status, s, st, hg, raw_k_sm);
+cudaError_t launch_route_gather_tc(const void *k, const void *v, const uint8_t *route, int32_t *sm_idx,
+                                   int32_t *sm_chunk_prefix, const int32_t *base_in, void *k_sm, void *v_sm, void *v16,
+                                   void *k16, int32_t cap, int32_t capv, int32_t *emit_flags, Shape s, cudaStream_t st,
+                                   bool pdl, HeadGroups hg, bool raw_k_sm) {
+    const RouteArgs ra{route, sm_idx, sm_chunk_prefix, emit_flags, base_in};
+    if (s.d == 128) return route_gather_impl<128>(k, v, ra, k_sm, v_sm, v16, k16, cap, capv, s, st, pdl, hg, raw_k_sm);
+    return route_gather_impl<64>(k, v, ra, k_sm, v_sm, v16, k16, cap, capv, s, st, pdl, hg, raw_k_sm);
 }
 
 }  // namespace natsl

@@ -5,6 +5,7 @@
 // route may be checked to be one decision per chunk (block-level routing).
 #include "common.cuh"
 #include "natsl_internal.h"
+#include "tc_common.cuh"
 
 namespace natsl {
 
@@ -27,6 +28,8 @@ route_compact_kernel(const uint8_t *__restrict__ route, int32_t *__restrict__ sm
     __shared__ int tile_total;
 
     const int bh = blockIdx.x, b = bh / H, h = bh % H;
+    tc::grid_dependency_wait();
+    tc::launch_dependents();
     const int NC = L / kC;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr int kWarps = kCompactThreads / 32;
@@ -130,6 +133,8 @@ gather_kv_kernel(const T *__restrict__ k, const T *__restrict__ v, const int32_t
     constexpr int kVecPerRow = D * (int)sizeof(T) / 16;  // 16-byte pieces per row
     constexpr int kRows = 256 / kVecPerRow;
     const int bh = blockIdx.y, b = bh / H, h = bh % H;
+    tc::grid_dependency_wait();
+    tc::launch_dependents();
     const int NC = L / kC;
     const int n_sm = sm_chunk_prefix[(size_t)bh * (NC + 1) + NC];
     if (blockIdx.x == 0 && threadIdx.x == 0 && n_sm > cap) atomicMin(status, NATSL_ERR_CACHE_FULL);
@@ -150,10 +155,9 @@ cudaError_t launch_route_compact(const uint8_t *route, int32_t *sm_idx, int32_t 
                                  int32_t *lin_idx, int32_t *n_lin, int32_t *sm_len,
                                  const int32_t *base_in, int32_t *block_status, int cap, int B, int L,
                                  int H, cudaStream_t st) {
-    route_compact_kernel<<<B * H, kCompactThreads, 0, st>>>(route, sm_idx, sm_chunk_prefix, lin_idx, n_lin,
-                                                            sm_len, base_in, block_status, cap, L, H);
     count_launch();
-    return cudaGetLastError();
+    return launch_kernel(route_compact_kernel, dim3(B * H), dim3(kCompactThreads), 0, st, true, route, sm_idx,
+                         sm_chunk_prefix, lin_idx, n_lin, sm_len, base_in, block_status, cap, L, H);
 }
 
 template <typename T, int D>
@@ -163,10 +167,9 @@ static cudaError_t gather_impl(const void *k, const void *v, const int32_t *sm_i
     constexpr int kRows = 256 / (D * (int)sizeof(T) / 16);
     const int max_rows = s.L < cap ? s.L : cap;
     dim3 grid((max_rows + kRows - 1) / kRows, s.B * s.H);
-    gather_kv_kernel<T, D><<<grid, 256, 0, st>>>((const T *)k, (const T *)v, sm_idx, pre, (T *)k_sm,
-                                                 (T *)v_sm, cap, status, s.L, s.H);
     count_launch();
-    return cudaGetLastError();
+    return launch_kernel(gather_kv_kernel<T, D>, grid, dim3(256), 0, st, true, (const T *)k, (const T *)v, sm_idx, pre,
+                         (T *)k_sm, (T *)v_sm, cap, status, s.L, s.H);
 }
 
 cudaError_t launch_gather_kv(const void *k, const void *v, const int32_t *sm_idx,

@@ -12,6 +12,7 @@
 //   U~ = U - W S;   O = scale_la diag(gamma) Q S + P U~;   S <- gamma_C S + (diag(gamma_C/gamma) K)^T U~
 #include "common.cuh"
 #include "natsl_internal.h"
+#include "tc_common.cuh"
 
 namespace natsl {
 
@@ -19,19 +20,37 @@ namespace {
 
 constexpr int kThreads = 256;
 
-// Load a 64 x D tile (token stride `ts` elements) into padded fp32 shared memory [64][D+1].
+// Small calls (few (batch, head) pairs, a few hundred tokens) are what this path is used for most, and there every
+// kernel is a chain of latencies on a mostly idle chip: the kernels below cut their work finer when there is
+// little of it, keep operand tiles in rows of D + 4 floats (16-byte loads, free of bank conflicts when neighbouring
+// lanes take neighbouring rows), and are programmatic dependents of one another.
+
+// Load a 64 x D tile (token stride `ts` elements) into fp32 shared memory, rows of D + 4.
 template <typename T, int D>
 __device__ __forceinline__ void load_tile(const T *__restrict__ src, size_t ts, float *dst) {
+#pragma unroll 4
     for (int idx = threadIdx.x; idx < kC * D / 4; idx += kThreads) {
         const int r = idx / (D / 4), c4 = (idx % (D / 4)) * 4;
-        const float4 x = load4(src + (size_t)r * ts + c4);
-        float *p = dst + r * (D + 1) + c4;
-        p[0] = x.x; p[1] = x.y; p[2] = x.z; p[3] = x.w;
+        store4(dst + r * (D + 4) + c4, load4(src + (size_t)r * ts + c4));
     }
+}
+// Inclusive prefix sum of 64 values in shared memory by one warp, in place.
+__device__ __forceinline__ void prefix64(float *x, int lane) {
+    const float a = x[2 * lane], b = x[2 * lane + 1];
+    float s = a + b;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const float y = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += y;
+    }
+    x[2 * lane + 1] = s;
+    x[2 * lane] = s - b;
 }
 
 // ------------------------------------------------------------------------------------------
-// Prepare: state-independent per-chunk quantities.  grid = (L/C, B*H).
+// Prepare: state-independent per-chunk quantities.  grid = (L/C, B*H).  K K^T and Q K^T together, 4 x 4 outputs of each
+// per thread; then one right-hand-side column per thread, updated from the left as its entries become known
+// (independent FMAs; a dot product per entry was a serial chain of 2016).
 // ------------------------------------------------------------------------------------------
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads)
@@ -40,18 +59,23 @@ gdn_prepare_simt_kernel(const T *__restrict__ q, const T *__restrict__ k, const 
                         const uint8_t *__restrict__ route, float scale_la, float *__restrict__ W,
                         float *__restrict__ U, float *__restrict__ P, float *__restrict__ Abar,
                         float *__restrict__ Gcum, int L, int H) {
-    extern __shared__ float smem[];
-    float *Ks = smem;                       // [64][D+1]
-    float *Vs = Ks + kC * (D + 1);          // [64][D+1]  (V, later Q)
-    float *As = Vs + kC * (D + 1);          // [64][64]
-    float *Gs = As + kC * kC;               // [64] inclusive cumulative log decay
+    constexpr int LD = D + 4, LA = kC + 4;
+    extern __shared__ __align__(16) float smem[];
+    float *Ks = smem;                       // [64][LD]
+    float *Vs = Ks + kC * LD;               // [64][LD]
+    float *Qs = Vs + kC * LD;               // [64][LD]
+    float *At = Qs + kC * LD;               // [64][LA]: column j of A
+    float *Gs = At + kC * LA;               // [64] inclusive cumulative log decay
     float *bts = Gs + kC;                   // [64] beta~
 
     const int c = blockIdx.x, bh = blockIdx.y, b = bh / H, h = bh % H;
     const size_t ts = (size_t)H * D;
     const size_t tok0 = ((size_t)b * L + (size_t)c * kC) * H + h;  // index of the chunk's first token
+    tc::grid_dependency_wait();
+    tc::launch_dependents();
 
     load_tile<T, D>(k + tok0 * D, ts, Ks);
+    load_tile<T, D>(q + tok0 * D, ts, Qs);
     load_tile<T, D>(v + tok0 * D, ts, Vs);
     if (threadIdx.x < kC) {
         const size_t t = tok0 + (size_t)threadIdx.x * H;
@@ -59,29 +83,42 @@ gdn_prepare_simt_kernel(const T *__restrict__ q, const T *__restrict__ k, const 
         Gs[threadIdx.x] = g[t];
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float acc = 0.f;
-        for (int i = 0; i < kC; ++i) { acc += Gs[i]; Gs[i] = acc; }
-    }
+    if (threadIdx.x < 32) prefix64(Gs, threadIdx.x);
     __syncthreads();
     if (Gcum && threadIdx.x < kC) Gcum[(size_t)bh * L + c * kC + threadIdx.x] = Gs[threadIdx.x];
-    // A (strictly lower); Abar = A without the beta~ row factor (the backward needs it)
+    // A (strictly lower), Abar = A without the beta~ row factor (the backward needs it), and
+    // P = scale_la (Q K^T) . Gamma, lower triangle including the diagonal.  Thread: rows ti + 16 e, columns tj + 16 e.
     {
-        const int i = threadIdx.x >> 2;
-        float *Ab = Abar ? Abar + ((size_t)bh * (L / kC) + c) * kC * kC : nullptr;
-        for (int m = 0; m < 16; ++m) {
-            const int j = (threadIdx.x & 3) + 4 * m;
-            float a = 0.f;
-            if (j < i && (bts[i] != 0.f || Ab)) {
-                float dot = 0.f;
-                const float *ki = Ks + i * (D + 1), *kj = Ks + j * (D + 1);
-#pragma unroll 8
-                for (int x = 0; x < D; ++x) dot = fmaf(ki[x], kj[x], dot);
-                a = __expf(Gs[i] - Gs[j]) * dot;
+        const int ti = threadIdx.x >> 4, tj = threadIdx.x & 15;
+        float a[4][4] = {}, pq[4][4] = {};
+#pragma unroll 2
+        for (int x = 0; x < D; x += 4) {
+            float4 kj[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) kj[e] = *reinterpret_cast<const float4 *>(Ks + (tj + 16 * e) * LD + x);
+#pragma unroll
+            for (int ei = 0; ei < 4; ++ei) {
+                const float4 ki = *reinterpret_cast<const float4 *>(Ks + (ti + 16 * ei) * LD + x);
+                const float4 qi = *reinterpret_cast<const float4 *>(Qs + (ti + 16 * ei) * LD + x);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    a[ei][e] = fmaf(ki.x, kj[e].x, fmaf(ki.y, kj[e].y, fmaf(ki.z, kj[e].z, fmaf(ki.w, kj[e].w, a[ei][e]))));
+                    pq[ei][e] = fmaf(qi.x, kj[e].x, fmaf(qi.y, kj[e].y, fmaf(qi.z, kj[e].z, fmaf(qi.w, kj[e].w, pq[ei][e]))));
+                }
             }
-            if (Ab) Ab[i * kC + j] = a;
-            As[i * kC + j] = bts[i] * a;
         }
+        const size_t cc = ((size_t)bh * (L / kC) + c) * kC * kC;
+#pragma unroll
+        for (int ei = 0; ei < 4; ++ei)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int i = ti + 16 * ei, j = tj + 16 * e;
+                const float gam = j <= i ? __expf(Gs[i] - Gs[j]) : 0.f;
+                const float av = j < i ? gam * a[ei][e] : 0.f;
+                if (Abar) Abar[cc + i * kC + j] = av;
+                At[j * LA + i] = bts[i] * av;
+                P[cc + i * kC + j] = scale_la * gam * pq[ei][e];
+            }
     }
     __syncthreads();
     // Forward substitution, one right-hand-side column per thread: columns [0,D) give W, [D,2D) U.
@@ -91,45 +128,29 @@ gdn_prepare_simt_kernel(const T *__restrict__ q, const T *__restrict__ k, const 
         const float *src = isW ? Ks : Vs;
         float x[kC];
 #pragma unroll
-        for (int i = 0; i < kC; ++i) {
-            float acc = bts[i] * (isW ? __expf(Gs[i]) : 1.f) * src[i * (D + 1) + col];
+        for (int i = 0; i < kC; ++i) x[i] = bts[i] * (isW ? __expf(Gs[i]) : 1.f) * src[i * LD + col];
 #pragma unroll
-            for (int j = 0; j < i; ++j) acc = fmaf(-As[i * kC + j], x[j], acc);
-            x[i] = acc;
-        }
+        for (int j = 0; j < kC - 1; ++j)
+#pragma unroll
+            for (int i4 = (j + 1) / 4; i4 < kC / 4; ++i4) {
+                const float4 aj = *reinterpret_cast<const float4 *>(At + j * LA + 4 * i4);   // (zero for i <= j)
+                if (4 * i4 > j) x[4 * i4] = fmaf(-aj.x, x[j], x[4 * i4]);
+                if (4 * i4 + 1 > j) x[4 * i4 + 1] = fmaf(-aj.y, x[j], x[4 * i4 + 1]);
+                if (4 * i4 + 2 > j) x[4 * i4 + 2] = fmaf(-aj.z, x[j], x[4 * i4 + 2]);
+                if (4 * i4 + 3 > j) x[4 * i4 + 3] = fmaf(-aj.w, x[j], x[4 * i4 + 3]);
+            }
         float *dst = (isW ? W : U) + tok0 * D + col;
 #pragma unroll
         for (int i = 0; i < kC; ++i) dst[(size_t)i * ts] = x[i];
     }
-    __syncthreads();
-    // P = scale_la (Q K^T) . Gamma, lower triangle including the diagonal
-    load_tile<T, D>(q + tok0 * D, ts, Vs);
-    __syncthreads();
-    {
-        const int i = threadIdx.x >> 2;
-        float *Pc = P + ((size_t)bh * (L / kC) + c) * kC * kC;
-        for (int m = 0; m < 16; ++m) {
-            const int j = (threadIdx.x & 3) + 4 * m;
-            float a = 0.f;
-            if (j <= i) {
-                float dot = 0.f;
-                const float *qi = Vs + i * (D + 1), *kj = Ks + j * (D + 1);
-#pragma unroll 8
-                for (int x = 0; x < D; ++x) dot = fmaf(qi[x], kj[x], dot);
-                a = scale_la * __expf(Gs[i] - Gs[j]) * dot;
-            }
-            Pc[i * kC + j] = a;
-        }
-    }
 }
 
 // ------------------------------------------------------------------------------------------
-// Scan: sequential over chunks, one CTA per (batch, head, slice of 32 value columns).
-// grid = (D/32, B*H).
+// Scan: sequential over chunks, one CTA per (batch, head, slice of NV value columns), grid = (D/NV, B*H).  NV = 8
+// when slices of 32 would leave most of the chip idle: a chunk's step is a chain, and four times shorter for it;
+// with many (batch, head) pairs the wider slice reads the chunk's operands a quarter as often.
 // ------------------------------------------------------------------------------------------
-constexpr int kDvs = 32;
-
-template <typename T, int D>
+template <typename T, int D, int NV>
 __global__ void __launch_bounds__(kThreads)
 gdn_scan_simt_kernel(const T *__restrict__ q, const T *__restrict__ k, const float *__restrict__ g,
                      const float *__restrict__ W, const float *__restrict__ U,
@@ -137,129 +158,137 @@ gdn_scan_simt_kernel(const T *__restrict__ q, const T *__restrict__ k, const flo
                      float *__restrict__ state_out, float *__restrict__ chunk_states,
                      float *__restrict__ Ut, float *__restrict__ o_la,
                      const uint8_t *__restrict__ block_route, int L, int H) {
-    extern __shared__ float smem[];
-    float *Ss = smem;                        // [D][32]
-    float *Ws = Ss + D * kDvs;               // [64][D+1]
-    float *Qs = Ws + kC * (D + 1);           // [64][D+1]
-    float *Ks = Qs + kC * (D + 1);           // [64][D+1]
-    float *Ps = Ks + kC * (D + 1);           // [64][65]
-    float *Us = Ps + kC * (kC + 1);          // [64][33]
-    float *Gs = Us + kC * (kDvs + 1);        // [64]
+    constexpr int LD = D + 4, LP = kC + 4;
+    constexpr int kN = NV / 4;               // columns per thread of a [64][NV] result: four threads per row
+    extern __shared__ __align__(16) float smem[];
+    float *Ss = smem;                        // [D][NV]
+    float *Ws = Ss + D * NV;                 // [64][LD]
+    float *Qs = Ws + kC * LD;                // [64][LD]
+    float *Ks = Qs + kC * LD;                // [64][LD]
+    float *Ps = Ks + kC * LD;                // [64][LP]
+    float *Us = Ps + kC * LP;                // [64][NV]
+    float *Gs = Us + kC * NV;                // [64] cumulative log decay
+    float *e1 = Gs + kC, *e2 = e1 + kC;      // [64] scale_la gamma_i; [64] gamma_C / gamma_i
 
     const int slice = blockIdx.x, bh = blockIdx.y, b = bh / H, h = bh % H;
     const int NC = L / kC;
     const size_t ts = (size_t)H * D;
-    const int c0 = slice * kDvs;
+    const int c0 = slice * NV;
+    tc::grid_dependency_wait();
+    tc::launch_dependents();
 
-    for (int idx = threadIdx.x; idx < D * kDvs; idx += kThreads) {
-        const int a = idx / kDvs, cc = idx % kDvs;
+    for (int idx = threadIdx.x; idx < D * NV; idx += kThreads) {
+        const int a = idx / NV, cc = idx % NV;
         Ss[idx] = state_in ? state_in[((size_t)bh * D + a) * D + c0 + cc] : 0.f;
     }
-
+    auto fma_n = [](float (&acc)[kN], float f, const float *s) {      // acc += f s[0 .. kN)
+        if constexpr (kN == 2) {
+            const float2 y = *reinterpret_cast<const float2 *>(s);
+            acc[0] = fmaf(f, y.x, acc[0]);
+            acc[1] = fmaf(f, y.y, acc[1]);
+        } else {
+#pragma unroll
+            for (int x = 0; x < kN; x += 4) {
+                const float4 y = *reinterpret_cast<const float4 *>(s + x);
+                acc[x] = fmaf(f, y.x, acc[x]); acc[x + 1] = fmaf(f, y.y, acc[x + 1]);
+                acc[x + 2] = fmaf(f, y.z, acc[x + 2]); acc[x + 3] = fmaf(f, y.w, acc[x + 3]);
+            }
+        }
+    };
     for (int c = 0; c < NC; ++c) {
         const size_t tok0 = ((size_t)b * L + (size_t)c * kC) * H + h;
         __syncthreads();
         if (chunk_states) {  // state at chunk entry, [B,H,NC,D,D]
-            for (int idx = threadIdx.x; idx < D * kDvs; idx += kThreads) {
-                const int a = idx / kDvs, cc = idx % kDvs;
+            for (int idx = threadIdx.x; idx < D * NV; idx += kThreads) {
+                const int a = idx / NV, cc = idx % NV;
                 chunk_states[(((size_t)bh * NC + c) * D + a) * D + c0 + cc] = Ss[idx];
             }
         }
+        if (threadIdx.x < kC) Gs[threadIdx.x] = g[tok0 + (size_t)threadIdx.x * H];
         load_tile<float, D>(W + tok0 * D, ts, Ws);
         load_tile<T, D>(q + tok0 * D, ts, Qs);
         load_tile<T, D>(k + tok0 * D, ts, Ks);
         {
             const float *Pc = P + ((size_t)bh * NC + c) * kC * kC;
-            for (int idx = threadIdx.x; idx < kC * kC; idx += kThreads)
-                Ps[(idx >> 6) * (kC + 1) + (idx & 63)] = Pc[idx];
-            for (int idx = threadIdx.x; idx < kC * kDvs; idx += kThreads) {
-                const int r = idx / kDvs, cc = idx % kDvs;
-                Us[r * (kDvs + 1) + cc] = U[(tok0 + (size_t)r * H) * D + c0 + cc];
+            for (int idx = threadIdx.x; idx < kC * kC / 4; idx += kThreads)
+                store4(Ps + (idx >> 4) * LP + (idx & 15) * 4, load4(Pc + 4 * idx));
+            for (int idx = threadIdx.x; idx < kC * NV; idx += kThreads)
+                Us[idx] = U[(tok0 + (size_t)(idx / NV) * H) * D + c0 + idx % NV];
+        }
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            prefix64(Gs, threadIdx.x);
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int i = threadIdx.x + 32 * u;
+                e1[i] = scale_la * __expf(Gs[i]);
+                e2[i] = __expf(Gs[kC - 1] - Gs[i]);
             }
-            if (threadIdx.x < kC) Gs[threadIdx.x] = g[tok0 + (size_t)threadIdx.x * H];
+        }
+        const int r = threadIdx.x >> 2, cb = (threadIdx.x & 3) * kN;
+        // U~ = U - W S, and q S while the state's rows pass by
+        float qs[kN], ut[kN];
+#pragma unroll
+        for (int x = 0; x < kN; ++x) { qs[x] = 0.f; ut[x] = Us[r * NV + cb + x]; }
+#pragma unroll 4
+        for (int a = 0; a < D; a += 4) {
+            const float4 wv = *reinterpret_cast<const float4 *>(Ws + r * LD + a);
+            const float4 qv = *reinterpret_cast<const float4 *>(Qs + r * LD + a);
+            const float *sr = Ss + a * NV + cb;
+            fma_n(ut, -wv.x, sr); fma_n(ut, -wv.y, sr + NV); fma_n(ut, -wv.z, sr + 2 * NV); fma_n(ut, -wv.w, sr + 3 * NV);
+            fma_n(qs, qv.x, sr); fma_n(qs, qv.y, sr + NV); fma_n(qs, qv.z, sr + 2 * NV); fma_n(qs, qv.w, sr + 3 * NV);
+        }
+#pragma unroll
+        for (int x = 0; x < kN; ++x) Us[r * NV + cb + x] = ut[x];      // (read and written by this thread only so far)
+        if (Ut) {
+            float *dst = Ut + (tok0 + (size_t)r * H) * D + c0 + cb;
+#pragma unroll
+            for (int x = 0; x < kN; ++x) dst[x] = ut[x];
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            float acc = 0.f;
-            for (int i = 0; i < kC; ++i) { acc += Gs[i]; Gs[i] = acc; }
-        }
-        __syncthreads();
-        const int r = threadIdx.x >> 2, cb = (threadIdx.x & 3) * 8;
-        // U~ = U - W S
+        // O = scale_la gamma_r q_r S + sum_{j<=r} P_rj U~_j   (P is zero above the diagonal)
         {
-            float acc[8];
+            const float gs = e1[r];
 #pragma unroll
-            for (int x = 0; x < 8; ++x) acc[x] = Us[r * (kDvs + 1) + cb + x];
-            const float *wr = Ws + r * (D + 1);
-            for (int a = 0; a < D; ++a) {
-                const float wv = wr[a];
-                const float *sr = Ss + a * kDvs + cb;
-#pragma unroll
-                for (int x = 0; x < 8; ++x) acc[x] = fmaf(-wv, sr[x], acc[x]);
-            }
-            __syncthreads();
-#pragma unroll
-            for (int x = 0; x < 8; ++x) Us[r * (kDvs + 1) + cb + x] = acc[x];
-            if (Ut) {
-                float *dst = Ut + (tok0 + (size_t)r * H) * D + c0 + cb;
-                store4(dst, make_float4(acc[0], acc[1], acc[2], acc[3]));
-                store4(dst + 4, make_float4(acc[4], acc[5], acc[6], acc[7]));
-            }
-        }
-        __syncthreads();
-        // O = scale_la gamma_r q_r S + sum_{j<=r} P_rj U~_j
-        {
-            float acc[8];
-#pragma unroll
-            for (int x = 0; x < 8; ++x) acc[x] = 0.f;
-            const float *qr = Qs + r * (D + 1);
-            for (int a = 0; a < D; ++a) {
-                const float qv = qr[a];
-                const float *sr = Ss + a * kDvs + cb;
-#pragma unroll
-                for (int x = 0; x < 8; ++x) acc[x] = fmaf(qv, sr[x], acc[x]);
-            }
-            const float gs = scale_la * __expf(Gs[r]);
-#pragma unroll
-            for (int x = 0; x < 8; ++x) acc[x] *= gs;
-            const float *pr = Ps + r * (kC + 1);
-            for (int j = 0; j <= r; ++j) {
-                const float pv = pr[j];
-                const float *ur = Us + j * (kDvs + 1) + cb;
-#pragma unroll
-                for (int x = 0; x < 8; ++x) acc[x] = fmaf(pv, ur[x], acc[x]);
+            for (int x = 0; x < kN; ++x) qs[x] *= gs;
+            const int jn = (r | 7) + 1;               // (rows of a warp are neighbours: one bound for all of them)
+#pragma unroll 2
+            for (int j = 0; j < jn; j += 4) {
+                const float4 pv = *reinterpret_cast<const float4 *>(Ps + r * LP + j);
+                const float *ur = Us + j * NV + cb;
+                fma_n(qs, pv.x, ur); fma_n(qs, pv.y, ur + NV); fma_n(qs, pv.z, ur + 2 * NV); fma_n(qs, pv.w, ur + 3 * NV);
             }
             float *dst = o_la + (tok0 + (size_t)r * H) * D + c0 + cb;
-            store4(dst, make_float4(acc[0], acc[1], acc[2], acc[3]));
-            store4(dst + 4, make_float4(acc[4], acc[5], acc[6], acc[7]));
+#pragma unroll
+            for (int x = 0; x < kN; ++x) dst[x] = qs[x];
         }
-        __syncthreads();
-        // S <- gamma_C S + (diag(gamma_C / gamma) K)^T U~
+        // S <- gamma_C S + (diag(gamma_C / gamma) K)^T U~  (nobody reads S any more)
         {
-            constexpr int kPer = D / 8;            // outputs per thread
-            constexpr int kTpr = kDvs / kPer;      // threads per state row
-            const int a = threadIdx.x / kTpr, cs = (threadIdx.x % kTpr) * kPer;
-            const float gl = Gs[kC - 1];
-            const float gC = __expf(gl);
-            float acc[kPer];
+            constexpr int kOut = D * NV / kThreads;   // outputs per thread, of one state row
+            constexpr int kTpr = NV / kOut;           // threads per state row
+            const int a = threadIdx.x / kTpr, cs = (threadIdx.x % kTpr) * kOut;
+            const float gC = __expf(Gs[kC - 1]);
+            float acc[kOut];
 #pragma unroll
-            for (int x = 0; x < kPer; ++x) acc[x] = gC * Ss[a * kDvs + cs + x];
+            for (int x = 0; x < kOut; ++x) acc[x] = 0.f;
             // block-level routing: a softmax block's update is not committed, the state only decays
-            const bool commit = !(block_route && block_route[tok0]);
-            for (int j = 0; commit && j < kC; ++j) {
-                const float kv = Ks[j * (D + 1) + a] * __expf(gl - Gs[j]);
-                const float *ur = Us + j * (kDvs + 1) + cs;
+            if (!(block_route && block_route[tok0])) {
+#pragma unroll 8
+                for (int j = 0; j < kC; ++j) {
+                    const float kv = Ks[j * LD + a] * e2[j];
 #pragma unroll
-                for (int x = 0; x < kPer; ++x) acc[x] = fmaf(kv, ur[x], acc[x]);
+                    for (int x = 0; x < kOut; ++x) acc[x] = fmaf(kv, Us[j * NV + cs + x], acc[x]);
+                }
             }
 #pragma unroll
-            for (int x = 0; x < kPer; ++x) Ss[a * kDvs + cs + x] = acc[x];
+            for (int x = 0; x < kOut; ++x) Ss[a * NV + cs + x] = fmaf(gC, Ss[a * NV + cs + x], acc[x]);
         }
     }
     __syncthreads();
     if (state_out) {
-        for (int idx = threadIdx.x; idx < D * kDvs; idx += kThreads) {
-            const int a = idx / kDvs, cc = idx % kDvs;
+        for (int idx = threadIdx.x; idx < D * NV; idx += kThreads) {
+            const int a = idx / NV, cc = idx % NV;
             state_out[((size_t)bh * D + a) * D + c0 + cc] = Ss[idx];
         }
     }
@@ -267,14 +296,15 @@ gdn_scan_simt_kernel(const T *__restrict__ q, const T *__restrict__ k, const flo
 
 // ------------------------------------------------------------------------------------------
 // Softmax branch over the retained tokens (Section 4.1, O_nla with mask M^nla) with the
-// combination (Section 4.3, Norm equation) as epilogue.  grid = (L/64, B*H*G); each warp owns
-// 8 query rows, each lane one key of the current 32-key tile.
+// combination (Section 4.3, Norm equation) as epilogue.  grid = (L/(8 NQ), B*H*G); each warp owns NQ query rows --
+// 8, or 2 when blocks of 64 queries would leave most of the chip idle --, each lane one key of the current
+// 32-key tile, whose pieces are read once for all of the warp's rows.
 // G softmax heads per linear head (Section 4.3, grouped heads): softmax head (h, sg) works on the
 // columns [sg D, (sg+1) D) of q, k, v rows of DL = G D columns; lists, weights and the linear read-out
 // are those of linear head h; the softmax output is normalised over its D columns, the linear
 // read-out over all DL, and the CTA writes its D columns of `out`.  lse is [B,H,G,L].
 // ------------------------------------------------------------------------------------------
-template <typename T, int D, int G>
+template <typename T, int D, int G, int NQ>
 __global__ void __launch_bounds__(kThreads)
 softmax_combine_simt_kernel(const T *__restrict__ q, const T *__restrict__ k_sm,
                             const T *__restrict__ v_sm, int cap, const int32_t *__restrict__ sm_idx,
@@ -284,29 +314,33 @@ softmax_combine_simt_kernel(const T *__restrict__ q, const T *__restrict__ k_sm,
                             float *__restrict__ o_nla, float *__restrict__ lse,
                             const uint8_t *__restrict__ block_route, const T *__restrict__ k_tok,
                             const T *__restrict__ v_tok, int L, int H) {
-    extern __shared__ float smem[];
-    float *Qs = smem;                      // [64][D]
-    float *Kt = Qs + kC * D;               // [32][D+1]
-    float *Vt = Kt + 32 * (D + 1);         // [32][D]
+    constexpr int kRowsQ = 8 * NQ, LD = D + 4;
+    extern __shared__ __align__(16) float smem[];
+    float *Qs = smem;                      // [8 NQ][D]
+    float *Kt = Qs + kRowsQ * D;           // [32][D+4]
+    float *Vt = Kt + 32 * LD;              // [32][D]
     int *pos = reinterpret_cast<int *>(Vt + 32 * D);  // [32]
 
     constexpr int DL = D * G;
-    const int c = blockIdx.x, bhg = blockIdx.y, bh = bhg / G, sg = bhg % G, b = bh / H, h = bh % H;
+    const int c = blockIdx.x * kRowsQ / kC, row0 = blockIdx.x * kRowsQ % kC;      // chunk, first row inside it
+    const int bhg = blockIdx.y, bh = bhg / G, sg = bhg % G, b = bh / H, h = bh % H;
     const int NC = L / kC;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const size_t ts = (size_t)H * DL;
     const size_t tok0 = ((size_t)b * L + (size_t)c * kC) * H + h;
+    tc::grid_dependency_wait();
+    tc::launch_dependents();
     const int n_end = min(sm_chunk_prefix[(size_t)bh * (NC + 1) + c + 1], cap);
     const int col0 = sg * D;                             // first column of this softmax head
 
-    for (int idx = threadIdx.x; idx < kC * D / 4; idx += kThreads) {
+    for (int idx = threadIdx.x; idx < kRowsQ * D / 4; idx += kThreads) {
         const int r = idx / (D / 4), c4 = (idx % (D / 4)) * 4;
-        store4(Qs + r * D + c4, load4(q + tok0 * DL + (size_t)r * ts + col0 + c4));
+        store4(Qs + r * D + c4, load4(q + tok0 * DL + (size_t)(row0 + r) * ts + col0 + c4));
     }
-    constexpr int kQ = 8, kCols = D / 32;
-    float m[kQ], z[kQ], acc[kQ][kCols];
+    constexpr int kCols = D / 32;
+    float m[NQ], z[NQ], acc[NQ][kCols];
 #pragma unroll
-    for (int r = 0; r < kQ; ++r) {
+    for (int r = 0; r < NQ; ++r) {
         m[r] = -INFINITY; z[r] = 0.f;
 #pragma unroll
         for (int x = 0; x < kCols; ++x) acc[r][x] = 0.f;
@@ -331,8 +365,7 @@ softmax_combine_simt_kernel(const T *__restrict__ q, const T *__restrict__ k_sm,
                 kx = load4(kb + (size_t)(j0 + r) * DL + c4);
                 vx = load4(vb + (size_t)(j0 + r) * DL + c4);
             }
-            float *kp = Kt + r * (D + 1) + c4;
-            kp[0] = kx.x; kp[1] = kx.y; kp[2] = kx.z; kp[3] = kx.w;
+            store4(Kt + r * LD + c4, kx);
             store4(Vt + r * D + c4, vx);
         }
         if (threadIdx.x < 32)
@@ -341,36 +374,49 @@ softmax_combine_simt_kernel(const T *__restrict__ q, const T *__restrict__ k_sm,
                                                             : 0x7fffffff;
         __syncthreads();
         const int my_pos = pos[lane];
-        const float *kr = Kt + lane * (D + 1);
+        const float *kr = Kt + lane * LD, *qr = Qs + warp * NQ * D;
+        float s[NQ], p[NQ];
 #pragma unroll
-        for (int r = 0; r < kQ; ++r) {
-            const int i = c * kC + warp * kQ + r;
-            const float *qr = Qs + (warp * kQ + r) * D;
-            float s = 0.f;
-#pragma unroll 8
-            for (int x = 0; x < D; ++x) s = fmaf(qr[x], kr[x], s);
-            const bool valid = my_pos <= i;
-            s = valid ? s * scale_sm : -INFINITY;
-            const float m_new = fmaxf(m[r], warp_max(s));
-            if (m_new == -INFINITY) continue;          // warp-uniform
-            const float pj = valid ? __expf(s - m_new) : 0.f;
-            const float corr = __expf(m[r] - m_new);   // exp(-inf) = 0 on the first tile
-            z[r] = z[r] * corr + warp_sum(pj);
+        for (int r = 0; r < NQ; ++r) s[r] = 0.f;
+#pragma unroll 4
+        for (int x = 0; x < D; x += 4) {
+            const float4 kx = *reinterpret_cast<const float4 *>(kr + x);
+#pragma unroll
+            for (int r = 0; r < NQ; ++r) {
+                const float4 qx = *reinterpret_cast<const float4 *>(qr + r * D + x);
+                s[r] = fmaf(qx.x, kx.x, fmaf(qx.y, kx.y, fmaf(qx.z, kx.z, fmaf(qx.w, kx.w, s[r]))));
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < NQ; ++r) {
+            const bool valid = my_pos <= c * kC + row0 + warp * NQ + r;
+            const float sc = valid ? s[r] * scale_sm : -INFINITY;
+            const float m_new = fmaxf(m[r], warp_max(sc)), m_use = m_new == -INFINITY ? 0.f : m_new;
+            p[r] = valid ? __expf(sc - m_use) : 0.f;
+            const float corr = __expf(m[r] - m_use);   // exp(-inf) = 0 on the first tile
+            z[r] = z[r] * corr + warp_sum(p[r]);
             m[r] = m_new;
 #pragma unroll
             for (int x = 0; x < kCols; ++x) acc[r][x] *= corr;
-            for (int j = 0; j < 32; ++j) {
-                const float pb = __shfl_sync(0xffffffffu, pj, j);
+        }
+#pragma unroll 8
+        for (int j = 0; j < 32; ++j) {
+            float vx[kCols];
 #pragma unroll
-                for (int x = 0; x < kCols; ++x) acc[r][x] = fmaf(pb, Vt[j * D + lane + 32 * x], acc[r][x]);
+            for (int x = 0; x < kCols; ++x) vx[x] = Vt[j * D + lane + 32 * x];
+#pragma unroll
+            for (int r = 0; r < NQ; ++r) {
+                const float pb = __shfl_sync(0xffffffffu, p[r], j);
+#pragma unroll
+                for (int x = 0; x < kCols; ++x) acc[r][x] = fmaf(pb, vx[x], acc[r][x]);
             }
         }
     }
     // epilogue: normalise both branches and combine
 #pragma unroll
-    for (int r = 0; r < kQ; ++r) {
-        const int i = c * kC + warp * kQ + r;
-        const size_t t = tok0 + (size_t)(warp * kQ + r) * H;
+    for (int r = 0; r < NQ; ++r) {
+        const int i = c * kC + row0 + warp * NQ + r;
+        const size_t t = tok0 + (size_t)(row0 + warp * NQ + r) * H;
         const float inv = z[r] > 0.f ? 1.f / z[r] : 0.f;
         float on[kCols], ol[kCols], ssn = 0.f, ssl = 0.f;
 #pragma unroll
@@ -544,11 +590,11 @@ cudaError_t set_smem(K kernel, size_t bytes) {
 
 }  // namespace
 
-size_t simt_prepare_smem(int d) { return sizeof(float) * (2 * kC * (d + 1) + kC * kC + 2 * kC); }
-size_t simt_scan_smem(int d) {
-    return sizeof(float) * (d * kDvs + 3 * kC * (d + 1) + kC * (kC + 1) + kC * (kDvs + 1) + kC);
+static size_t simt_prepare_smem(int d) { return sizeof(float) * (3 * kC * (d + 4) + kC * (kC + 4) + 2 * kC); }
+static size_t simt_scan_smem(int d, int nv) {
+    return sizeof(float) * (d * nv + 3 * kC * (d + 4) + kC * (kC + 4) + kC * nv + 3 * kC);
 }
-static size_t simt_softmax_smem(int d) { return sizeof(float) * (kC * d + 32 * (d + 1) + 32 * d + 32); }
+static size_t simt_softmax_smem(int d, int nq) { return sizeof(float) * (8 * nq * d + 32 * (d + 4) + 32 * d + 32); }
 
 #define NATSL_DISPATCH(FN, ...)                                                   \
     do {                                                                          \
@@ -569,11 +615,9 @@ static cudaError_t prepare_impl(const void *q, const void *k, const void *v, con
     cudaError_t e = set_smem(gdn_prepare_simt_kernel<T, D>, smem);
     if (e != cudaSuccess) return e;
     dim3 grid(s.L / kC, s.B * s.H);
-    gdn_prepare_simt_kernel<T, D><<<grid, kThreads, smem, st>>>(
-        (const T *)q, (const T *)k, (const T *)v, g, beta, route, scale_la, W, U, P, Abar, Gcum, s.L,
-        s.H);
     count_launch();
-    return cudaGetLastError();
+    return launch_kernel(gdn_prepare_simt_kernel<T, D>, grid, dim3(kThreads), smem, st, true, (const T *)q, (const T *)k,
+                         (const T *)v, g, beta, route, scale_la, W, U, P, Abar, Gcum, s.L, s.H);
 }
 
 cudaError_t launch_gdn_prepare_simt(const void *q, const void *k, const void *v, const float *g,
@@ -588,15 +632,15 @@ static cudaError_t scan_impl(const void *q, const void *k, const float *g, const
                              const float *U, const float *P, float scale_la, const float *state_in,
                              float *state_out, float *chunk_states, float *Ut, float *o_la,
                              const uint8_t *block_route, Shape s, cudaStream_t st) {
-    const size_t smem = simt_scan_smem(D);
-    cudaError_t e = set_smem(gdn_scan_simt_kernel<T, D>, smem);
+    const bool narrow = s.B * s.H * (D / 32) < 148;     // (see the kernel)
+    const size_t smem = simt_scan_smem(D, narrow ? 8 : 32);
+    auto kernel = narrow ? gdn_scan_simt_kernel<T, D, 8> : gdn_scan_simt_kernel<T, D, 32>;
+    cudaError_t e = set_smem(kernel, smem);
     if (e != cudaSuccess) return e;
-    dim3 grid(D / kDvs, s.B * s.H);
-    gdn_scan_simt_kernel<T, D><<<grid, kThreads, smem, st>>>(
-        (const T *)q, (const T *)k, g, W, U, P, scale_la, state_in, state_out, chunk_states, Ut,
-        o_la, block_route, s.L, s.H);
     count_launch();
-    return cudaGetLastError();
+    return launch_kernel(kernel, dim3(D / (narrow ? 8 : 32), s.B * s.H), dim3(kThreads), smem, st, true, (const T *)q,
+                         (const T *)k, g, W, U, P, scale_la, state_in, state_out, chunk_states, Ut, o_la, block_route, s.L,
+                         s.H);
 }
 
 cudaError_t launch_gdn_scan_simt(const void *q, const void *k, const float *g, const float *W,
@@ -613,15 +657,16 @@ static cudaError_t softmax_impl(const void *q, const void *k_sm, const void *v_s
                                 const int32_t *sm_idx, const int32_t *pre, const float *o_la,
                                 const float *w, float scale_sm, float eps, void *out, float *o_nla,
                                 float *lse, BlockRouting br, Shape s, cudaStream_t st) {
-    const size_t smem = simt_softmax_smem(D);
-    cudaError_t e = set_smem(softmax_combine_simt_kernel<T, D, G>, smem);
+    const bool few = (s.L / kC) * s.B * s.H * G < 148;   // (see the kernel)
+    const int nq = few ? 2 : 8;
+    const size_t smem = simt_softmax_smem(D, nq);
+    auto kernel = few ? softmax_combine_simt_kernel<T, D, G, 2> : softmax_combine_simt_kernel<T, D, G, 8>;
+    cudaError_t e = set_smem(kernel, smem);
     if (e != cudaSuccess) return e;
-    dim3 grid(s.L / kC, s.B * s.H * G);
-    softmax_combine_simt_kernel<T, D, G><<<grid, kThreads, smem, st>>>(
-        (const T *)q, (const T *)k_sm, (const T *)v_sm, cap, sm_idx, pre, o_la, w, scale_sm, eps,
-        (T *)out, o_nla, lse, br.route, (const T *)br.k, (const T *)br.v, s.L, s.H);
     count_launch();
-    return cudaGetLastError();
+    return launch_kernel(kernel, dim3(s.L / (8 * nq), s.B * s.H * G), dim3(kThreads), smem, st, true, (const T *)q,
+                         (const T *)k_sm, (const T *)v_sm, cap, sm_idx, pre, o_la, w, scale_sm, eps, (T *)out, o_nla, lse,
+                         br.route, (const T *)br.k, (const T *)br.v, s.L, s.H);
 }
 
 cudaError_t launch_softmax_combine_simt(const void *q, const void *k_sm, const void *v_sm,

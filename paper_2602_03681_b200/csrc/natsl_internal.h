@@ -51,8 +51,6 @@ cudaError_t launch_gather_kv(const void *k, const void *v, const int32_t *sm_idx
                              int32_t *status, Shape s, cudaStream_t st);
 
 // fwd_simt.cu -- fp32 CUDA-core forward (exact-precision path; bf16 storage allowed)
-size_t simt_prepare_smem(int d);
-size_t simt_scan_smem(int d);
 cudaError_t launch_gdn_prepare_simt(const void *q, const void *k, const void *v, const float *g,
                                     const float *beta, const uint8_t *route, float scale_la,
                                     float *W, float *U, float *P, float *Abar, float *Gcum, Shape s,

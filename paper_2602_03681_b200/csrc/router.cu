@@ -5,10 +5,11 @@
 // HBM-bound: X [B, L, d_model] is read exactly once; the score weights (2 H rows of d_model) stay
 // in L2.  One CTA per pair of chunks, half of its threads per chunk: a thread owns 16 bytes of
 // every row of its chunk, so a warp reads 512 contiguous bytes per row, and sixteen rows are in
-// flight per thread (the grid is small, so the bytes in flight have to come from the threads).
-// The pooled rows are kept in shared memory; one warp per (head, operation) pair reads its weight
-// row once and forms the dot products with both pooled rows; the route bytes of the chunks'
-// tokens go out as one contiguous run.
+// flight per thread all the time: each is replaced as soon as it has been added (the grid is small, so the
+// bytes in flight have to come from the threads; in batches of sixteen the memory went idle at every batch's end).
+// The pooled rows are kept in shared memory; one warp per pair of (head, operation) rows reads its weight
+// rows once, all of a row's pieces in flight, and forms the dot products with both pooled rows; the route
+// bytes of the chunks' tokens go out as one contiguous run.
 #include "common.cuh"
 #include "natsl_internal.h"
 
@@ -52,45 +53,50 @@ score_layer_kernel(const T *__restrict__ x, const float *__restrict__ w_score,
 #pragma unroll
         for (int e = 0; e < kE; ++e) acc[e] = 0.f;
         if (live) {
-            for (int i = 0; i < kC; i += kRowsInFlight) {
-                uint4 u[kRowsInFlight];
+            const uint4 *src = reinterpret_cast<const uint4 *>(xc + col);
+            const size_t pitch = (size_t)Dm * sizeof(T) / 16;
+            uint4 u[kRowsInFlight];
 #pragma unroll
-                for (int j = 0; j < kRowsInFlight; ++j)
-                    u[j] = *reinterpret_cast<const uint4 *>(xc + (size_t)(i + j) * Dm + col);
+            for (int j = 0; j < kRowsInFlight; ++j) u[j] = __ldcs(src + j * pitch);
+#pragma unroll
+            for (int i = 0; i < kC; i += kRowsInFlight)
 #pragma unroll
                 for (int j = 0; j < kRowsInFlight; ++j) {
                     float v[kE];
                     unpack16(u[j], v, T());
+                    if (i + kRowsInFlight < kC) u[j] = __ldcs(src + (i + kRowsInFlight + j) * pitch);
 #pragma unroll
                     for (int e = 0; e < kE; ++e) acc[e] += v[e];
                 }
-            }
         }
 #pragma unroll
         for (int e = 0; e < kE; ++e) pooled[g * Dm + col + e] = acc[e] * (1.f / kC);
     }
     __syncthreads();
-    for (int pair = warp; pair < 2 * H; pair += kScoreThreads / 32) {   // pair = 2 head + operation
-        const float *wr = w_score + (size_t)pair * Dm;
-        float s[kScoreChunks];
-#pragma unroll
-        for (int q = 0; q < kScoreChunks; ++q) s[q] = 0.f;
+    // a warp takes the two rows of a head (linear, softmax)
+    for (int hd = warp; hd < H; hd += kScoreThreads / 32) {
+        const float *wr = w_score + (size_t)hd * 2 * Dm;
+        float s[2][kScoreChunks] = {};
+#pragma unroll 4
         for (int dd = lane * 4; dd < Dm; dd += 128) {
-            const float4 wv = __ldg(reinterpret_cast<const float4 *>(wr + dd));
+            const float4 w0 = __ldg(reinterpret_cast<const float4 *>(wr + dd)), w1 = __ldg(reinterpret_cast<const float4 *>(wr + Dm + dd));
 #pragma unroll
             for (int q = 0; q < kScoreChunks; ++q) {
                 const float4 pv = *reinterpret_cast<const float4 *>(pooled + q * Dm + dd);
-                s[q] = fmaf(wv.x, pv.x, fmaf(wv.y, pv.y, fmaf(wv.z, pv.z, fmaf(wv.w, pv.w, s[q]))));
+                s[0][q] = fmaf(w0.x, pv.x, fmaf(w0.y, pv.y, fmaf(w0.z, pv.z, fmaf(w0.w, pv.w, s[0][q]))));
+                s[1][q] = fmaf(w1.x, pv.x, fmaf(w1.y, pv.y, fmaf(w1.z, pv.z, fmaf(w1.w, pv.w, s[1][q]))));
             }
         }
 #pragma unroll
-        for (int q = 0; q < kScoreChunks; ++q) {
-            const float t = warp_sum(s[q]);
-            if (lane == 0 && c0 + q < NC) {
-                sc[q * 2 * H + pair] = t;
-                if (scores) scores[((size_t)b * NC + c0 + q) * H * 2 + pair] = t;
+        for (int op = 0; op < 2; ++op)
+#pragma unroll
+            for (int q = 0; q < kScoreChunks; ++q) {
+                const float t = warp_sum(s[op][q]);
+                if (lane == 0 && c0 + q < NC) {
+                    sc[q * 2 * H + 2 * hd + op] = t;
+                    if (scores) scores[((size_t)b * NC + c0 + q) * H * 2 + 2 * hd + op] = t;
+                }
             }
-        }
     }
     __syncthreads();
     // arg max over (linear, softmax); a tie keeps the first operation (linear)

@@ -130,26 +130,38 @@ __global__ void to_f32_kernel(const T *__restrict__ a, const T *__restrict__ b, 
 // ------------------------------------------------------------------------------------------
 // max |dout| over the whole tensor, as the bit pattern of a non-negative float (ordered like an
 // integer), into the status page; the word is zeroed by the caller beforehand.
+// (Magnitudes of bf16 values order like their bits: packed 16-bit maxima, 64 bytes in flight per thread; one atomic
+// per CTA -- one per warp was a queue of 9000 on one address.)
 template <typename T>
 __global__ void __launch_bounds__(256)
-dout_amax_kernel(const T *__restrict__ dout, size_t n4, int32_t *status) {
-    float m = 0.f;
+dout_amax_kernel(const T *__restrict__ dout, size_t n16, int32_t *status) {
+    __shared__ int part[8];
+    const uint4 *src = reinterpret_cast<const uint4 *>(dout);          // 16-byte pieces
+    auto fold = [](uint32_t m, uint32_t u) {
+        return sizeof(T) == 2 ? __vmaxu2(m, u & 0x7fff7fffu) : max(m, u & 0x7fffffffu);
+    };
+    uint32_t m = 0u;
     const size_t stride = (size_t)gridDim.x * 256;
     size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
-    for (; i + 3 * stride < n4; i += 4 * stride) {          // four loads in flight per thread
-        float4 x[4];
+    for (; i + 3 * stride < n16; i += 4 * stride) {
+        uint4 x[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = load4(dout + 4 * (i + u * stride));
+        for (int u = 0; u < 4; ++u) x[u] = src[i + u * stride];
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-            m = fmaxf(fmaxf(m, fmaxf(fabsf(x[u].x), fabsf(x[u].y))), fmaxf(fabsf(x[u].z), fabsf(x[u].w)));
+        for (int u = 0; u < 4; ++u) m = fold(fold(fold(fold(m, x[u].x), x[u].y), x[u].z), x[u].w);
     }
-    for (; i < n4; i += stride) {
-        const float4 x = load4(dout + 4 * i);
-        m = fmaxf(fmaxf(m, fmaxf(fabsf(x.x), fabsf(x.y))), fmaxf(fabsf(x.z), fabsf(x.w)));
+    for (; i < n16; i += stride) {
+        const uint4 x = src[i];
+        m = fold(fold(fold(fold(m, x.x), x.y), x.z), x.w);
     }
-    m = warp_max(m);
-    if ((threadIdx.x & 31) == 0 && m > 0.f) atomicMax(status + kGradAmaxWord, __float_as_int(m));
+    int bits = (int)(sizeof(T) == 2 ? max(m >> 16, m & 0xffffu) << 16 : m);
+    bits = __reduce_max_sync(0xffffffffu, bits);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = bits;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int x = 1; x < 8; ++x) bits = max(bits, part[x]);
+        if (bits > 0) atomicMax(status + kGradAmaxWord, bits);
+    }
 }
 
 // Four neighbouring columns per lane (one vector per array and lane), D / 4 lanes per row, so a warp takes
@@ -167,7 +179,7 @@ combine_bwd_kernel(const float *__restrict__ o_la, const float *__restrict__ o_n
                    float *__restrict__ Dsm, __half *__restrict__ do16,
                    __half *__restrict__ dola16, __half *__restrict__ dolag16,
                    const float *__restrict__ Gd, float scale_la, const int32_t *gsc, int G, int B, int L, int H) {
-    constexpr int kLpr = D / 4, kRpw = 32 / kLpr;           // lanes per row, rows per warp
+    constexpr int kE = 8, kLpr = D / kE, kRpw = 32 / kLpr;  // columns per lane, lanes per row, rows per warp
     const float gs = grad_scale(gsc).x;      // scale of the fp16 operand copies (and of Dsm with them)
     const int lane = threadIdx.x & 31, sub = lane / kLpr, li = lane % kLpr;
     const int lps = kLpr / G;                               // lanes per slice
@@ -178,67 +190,80 @@ combine_bwd_kernel(const float *__restrict__ o_la, const float *__restrict__ o_n
     const int h = rr % H;
     const size_t bl = rr / H;
     const int l = bl % L, b = bl / L;
-    const size_t at = rr * D + li * 4;
-    const float4 a = *reinterpret_cast<const float4 *>(o_la + at), n = *reinterpret_cast<const float4 *>(o_nla + at);
-    float dy[4];
-    if (sizeof(T) == 2) {
-        const uint2 u = *reinterpret_cast<const uint2 *>(dout + at);
-        dy[0] = __uint_as_float(u.x << 16); dy[1] = __uint_as_float(u.x & 0xffff0000u);
-        dy[2] = __uint_as_float(u.y << 16); dy[3] = __uint_as_float(u.y & 0xffff0000u);
-    } else {
-        const float4 u = *reinterpret_cast<const float4 *>(dout + at);
-        dy[0] = u.x; dy[1] = u.y; dy[2] = u.z; dy[3] = u.w;
-    }
-    const float ol[4] = {a.x, a.y, a.z, a.w}, on[4] = {n.x, n.y, n.z, n.w};
-    // returns the row's sum; slice = the sum over the lane's slice
-    auto sums = [&](float v, float &slice) {
-#pragma unroll
-        for (int o = 1; o < kLpr; o <<= 1) {
-            if (o == lps) slice = v;
-            v += __shfl_xor_sync(0xffffffffu, v, o);
-        }
-        if (lps == kLpr) slice = v;
-        return v;
+    const size_t at = rr * D + li * kE;
+    float ol[kE], on[kE], dy[kE];
+    auto load8 = [](const float *p, float (&x)[kE]) {
+        const float4 u = *reinterpret_cast<const float4 *>(p), v = *reinterpret_cast<const float4 *>(p + 4);
+        x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w; x[4] = v.x; x[5] = v.y; x[6] = v.z; x[7] = v.w;
     };
-    float ssl = 0.f, ssn = 0.f, ssn_s, unused;
+    load8(o_la + at, ol);
+    load8(o_nla + at, on);
+    if constexpr (sizeof(T) == 2) {
+        const uint4 u = *reinterpret_cast<const uint4 *>(dout + at);
+        const uint32_t uw[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
-    for (int x = 0; x < 4; ++x) { ssl = fmaf(ol[x], ol[x], ssl); ssn = fmaf(on[x], on[x], ssn); }
-    ssl = sums(ssl, unused);
-    sums(ssn, ssn_s);
-    const float fl = rsqrtf(ssl / D + eps), fn = rsqrtf(ssn_s * inv_ds + eps);   // fn: of the lane's slice
+        for (int x = 0; x < 4; ++x) {
+            dy[2 * x] = __uint_as_float(uw[x] << 16);
+            dy[2 * x + 1] = __uint_as_float(uw[x] & 0xffff0000u);
+        }
+    } else {
+        load8(reinterpret_cast<const float *>(dout) + at, dy);
+    }
     const float wn = w ? w[rr * 2] : 0.5f, wl = w ? w[rr * 2 + 1] : 0.5f;
     // scale_la gamma_l of the token (decay from its chunk's entry), for the reverse scan's operand
     const float sg = dolag16 ? scale_la * Gd[((size_t)(b * H + h) * (L / kC) + l / kC) * 128 + l % kC] : 0.f;
-    float dwl = 0.f, dwn = 0.f, dwn_s;
+    // All sums follow from four: |o_la|^2 and <dy, o_la> over the row, |o_nla|^2 and <dy, o_nla> over the slice.
+    float sl = 0.f, cl = 0.f, sn = 0.f, cn = 0.f;
 #pragma unroll
-    for (int x = 0; x < 4; ++x) { dwl = fmaf(dy[x], ol[x] * fl, dwl); dwn = fmaf(dy[x], on[x] * fn, dwn); }
-    dwl = sums(dwl, unused);
-    dwn = sums(dwn, dwn_s);                  // <dy, y_nla> over the row and over the slice
+    for (int x = 0; x < kE; ++x) {
+        sl = fmaf(ol[x], ol[x], sl); cl = fmaf(dy[x], ol[x], cl);
+        sn = fmaf(on[x], on[x], sn); cn = fmaf(dy[x], on[x], cn);
+    }
+#pragma unroll
+    for (int o = 1; o < kLpr; o <<= 1) {
+        sl += __shfl_xor_sync(0xffffffffu, sl, o);
+        cl += __shfl_xor_sync(0xffffffffu, cl, o);
+        if (o < lps) {                                      // (uniform)
+            sn += __shfl_xor_sync(0xffffffffu, sn, o);
+            cn += __shfl_xor_sync(0xffffffffu, cn, o);
+        }
+    }
+    const float fl = rsqrtf(sl / D + eps), fn = rsqrtf(sn * inv_ds + eps);
+    const float dwl = fl * cl, dwn_s = fn * cn;             // <dy, y_la> of the row, <dy, y_nla> of the slice
+    float dwn = dwn_s;
+    for (int o = lps; o < kLpr; o <<= 1) dwn += __shfl_xor_sync(0xffffffffu, dwn, o);
     const float ml = wl * dwl / D, mn = wn * dwn_s * inv_ds;
-    float dl[4], dn[4], dsm = 0.f, dsm_s;
+    if (!live) return;
+    float dl[kE], dn[kE];
 #pragma unroll
-    for (int x = 0; x < 4; ++x) {
+    for (int x = 0; x < kE; ++x) {
         dl[x] = fl * (wl * dy[x] - ol[x] * fl * ml);
         dn[x] = fn * (wn * dy[x] - on[x] * fn * mn);
-        dsm = fmaf(dn[x], on[x], dsm);
     }
-    sums(dsm, dsm_s);
-    if (!live) return;
     // (the tensor-core kernels read the fp16 copies only)
-    if (do_la) *reinterpret_cast<float4 *>(do_la + at) = make_float4(dl[0], dl[1], dl[2], dl[3]);
-    if (do_nla) *reinterpret_cast<float4 *>(do_nla + at) = make_float4(dn[0], dn[1], dn[2], dn[3]);
-    const size_t at16 = (((size_t)b * H + h) * L + l) * D + li * 4;
-    auto h4 = [](float x0, float x1, float x2, float x3) {
-        const __half2 p = __floats2half2_rn(x0, x1), q2 = __floats2half2_rn(x2, x3);
-        return make_uint2(*reinterpret_cast<const uint32_t *>(&p), *reinterpret_cast<const uint32_t *>(&q2));
+    auto put8 = [](float *p, const float (&x)[kE]) {
+        *reinterpret_cast<float4 *>(p) = make_float4(x[0], x[1], x[2], x[3]);
+        *reinterpret_cast<float4 *>(p + 4) = make_float4(x[4], x[5], x[6], x[7]);
     };
-    if (do16) *reinterpret_cast<uint2 *>(do16 + at16) = h4(gs * dn[0], gs * dn[1], gs * dn[2], gs * dn[3]);
+    if (do_la) put8(do_la + at, dl);
+    if (do_nla) put8(do_nla + at, dn);
+    const size_t at16 = (((size_t)b * H + h) * L + l) * D + li * kE;
+    auto put16 = [](__half *p, float f, const float (&x)[kE]) {
+        uint32_t o[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const __half2 y = __floats2half2_rn(f * x[2 * e], f * x[2 * e + 1]);
+            o[e] = *reinterpret_cast<const uint32_t *>(&y);
+        }
+        *reinterpret_cast<uint4 *>(p) = make_uint4(o[0], o[1], o[2], o[3]);
+    };
+    if (do16) put16(do16 + at16, gs, dn);
     if (dolag16) {
-        *reinterpret_cast<uint2 *>(dola16 + at16) = h4(gs * dl[0], gs * dl[1], gs * dl[2], gs * dl[3]);
-        const float gg = gs * sg;
-        *reinterpret_cast<uint2 *>(dolag16 + at16) = h4(gg * dl[0], gg * dl[1], gg * dl[2], gg * dl[3]);
+        put16(dola16 + at16, gs, dl);
+        put16(dolag16 + at16, gs * sg, dl);
     }
-    if (li % lps == 0) Dsm[(((size_t)b * H + h) * G + li / lps) * L + l] = gs * dsm_s;
+    if (li % lps == 0)                                      // <do_nla, o_nla> of the slice
+        Dsm[(((size_t)b * H + h) * G + li / lps) * L + l] = gs * fn * (wn * cn - fn * mn * sn);
     if (li == 0 && dw) { dw[rr * 2] = dwn; dw[rr * 2 + 1] = dwl; }
 }
 
@@ -873,7 +898,7 @@ static cudaError_t combine_bwd_impl(const float *o_la, const float *o_nla, const
                                     const float *Gd, float scale_la, const int32_t *gsc, Shape s,
                                     cudaStream_t st, int G) {
     const size_t rows = (size_t)s.B * s.L * s.H;
-    constexpr int kRowsPerBlock = (kThreads / 32) * (32 / (D / 4));
+    constexpr int kRowsPerBlock = (kThreads / 32) * (32 / (D / 8));
     combine_bwd_kernel<T, D><<<(unsigned)((rows + kRowsPerBlock - 1) / kRowsPerBlock), kThreads, 0, st>>>(
         o_la, o_nla, (const T *)dout, w, eps, do_la, do_nla, dw, Dsm, (__half *)do16, (__half *)dola16,
         (__half *)dolag16, Gd, scale_la, gsc, G, s.B, s.L, s.H);
@@ -882,10 +907,10 @@ static cudaError_t combine_bwd_impl(const float *o_la, const float *o_nla, const
 }
 
 cudaError_t launch_dout_amax(const void *dout, size_t n, bool bf16, int32_t *status, cudaStream_t st) {
-    const size_t n4 = n / 4;
-    const unsigned blocks = (unsigned)((n4 + 255) / 256 < 1184 ? (n4 + 255) / 256 : 1184);
-    if (bf16) dout_amax_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>((const __nv_bfloat16 *)dout, n4, status);
-    else dout_amax_kernel<float><<<blocks, 256, 0, st>>>((const float *)dout, n4, status);
+    const size_t n16 = n / (bf16 ? 8 : 4);
+    const unsigned blocks = (unsigned)((n16 + 255) / 256 < 1184 ? (n16 + 255) / 256 : 1184);
+    if (bf16) dout_amax_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>((const __nv_bfloat16 *)dout, n16, status);
+    else dout_amax_kernel<float><<<blocks, 256, 0, st>>>((const float *)dout, n16, status);
     count_launch();
     return cudaGetLastError();
 }

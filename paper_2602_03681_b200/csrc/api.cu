@@ -247,7 +247,7 @@ BwdWs carve_bwd(const natsl_params *p, void *ws) {
     f.ex.Gcum = f.Gcum;
     f.kap_c = c.take<float>(tcs && block ? B * H * NC : 0);
     f.dq32 = f.o_la;
-    f.dk32 = tm(tcs && normed); f.dv32 = tm(tcs && normed);
+    f.dk32 = tm(tcs && normed && !block); f.dv32 = tm(tcs && normed && !block);
     f.bytes = c.off;
     return f;
 }
@@ -646,9 +646,8 @@ int natsl_hybrid_bwd(const void *q, const void *k, const void *v, const float *g
         // stream: reverse scan, key-side kernel, scatter; caller's stream: query-side kernel, chunk kernel.
         // Block-level routing: every token has a softmax-branch dk, dv (retained tokens: scattered from the
         // compacted gradients; linear blocks: their own block's kernel, which needs the query-side one only), both
-        // in fp32 token-major buffers that the chunk kernel adds and so waits for.
-        // With the normalisation the gradients with respect to the two operations' normalised rows stay apart
-        // until its backward, a last kernel that rounds once.
+        // in fp32 token-major buffers that the chunk kernel adds (through the normalisation's Jacobian, where there is
+        // one) and so waits for.
         if (side) {
             NATSL_TRY(cudaEventRecord(side->fork, st));
             NATSL_TRY(cudaStreamWaitEvent(st0, side->fork, 0));
@@ -663,29 +662,30 @@ int natsl_hybrid_bwd(const void *q, const void *k, const void *v, const float *g
                                         p->scale_sm, f.dq_sm, f.dk_sm, f.dv_sm, p->dscore ? f.dmask : nullptr, !normed,
                                         f.status, s, st, st0, hg));
         if (side) NATSL_TRY(cudaStreamWaitEvent(st, side->join, 0));     // the reverse scan has finished
-        void *dq_o = normed ? f.dq32 : dq, *dk_o = normed ? f.dk32 : dk, *dv_o = normed ? f.dv32 : dv;
-        const float *dq_add = normed ? nullptr : f.dq_sm;
         if (block) {
             NATSL_TRY(launch_gdn_finish(a, f.dk_x, f.dv_x, s32, st0, false));
             NATSL_TRY(launch_softmax_bwd_own_block(q, k, v, f.dO16, f.lse, f.Dsm, route, p->scale_sm, f.dq_sm, f.dk_x,
                                                    f.dv_x, gsc, s, st, hg));
             NATSL_TRY(side_join.join());      // the side stream's last kernels
-            NATSL_TRY(launch_gdn_chunk_bwd(f.tc, f.ex, f.gr, v, beta, route, dq_add, p->scale_la, dq_o, dk_o, dv_o, normed,
-                                           dg, dbeta, true, normed ? nullptr : f.dk_x, f.dv_x,
-                                           p->dscore ? f.kap_c : nullptr, f.status, s, st));
+            NATSL_TRY(launch_gdn_chunk_bwd(f.tc, f.ex, f.gr, q, k, v, beta, route, f.dq_sm, p->scale_la, dq, dk, dv, dg,
+                                           dbeta, true, f.dk_x, f.dv_x, p->dscore ? f.kap_c : nullptr, f.status, s, st,
+                                           hg));
             if (p->dscore)
                 NATSL_TRY(launch_dscore(route, f.prefix, f.dmask, f.kap_c, nullptr, p->L, p->dscore, s, st, hg.G));
-        } else {
-            NATSL_TRY(launch_gdn_chunk_bwd(f.tc, f.ex, f.gr, v, beta, route, dq_add, p->scale_la, dq_o, dk_o, dv_o, normed,
-                                           dg, dbeta, false, nullptr, nullptr, nullptr, f.status, s, st));
-            // the retained tokens' dk, dv (rows the chunk kernel does not write)
-            NATSL_TRY(launch_gdn_finish(a, dk_o, dv_o, normed ? s32 : s, st0, false));
-            NATSL_TRY(side_join.join());
+            return NATSL_OK;
         }
+        // Token-level routing.  With the normalisation a token's k has one gradient, of one copy or the other: they
+        // stay in fp32 until its backward, a last kernel that rounds once.
+        void *dq_o = normed ? f.dq32 : dq, *dk_o = normed ? f.dk32 : dk, *dv_o = normed ? f.dv32 : dv;
+        NATSL_TRY(launch_gdn_chunk_bwd(f.tc, f.ex, f.gr, q, k, v, beta, route, normed ? nullptr : f.dq_sm, p->scale_la,
+                                       dq_o, dk_o, dv_o, dg, dbeta, false, nullptr, nullptr, nullptr, f.status, s, st,
+                                       hg));
+        // the retained tokens' dk, dv (rows the chunk kernel does not write)
+        NATSL_TRY(launch_gdn_finish(a, dk_o, dv_o, normed ? s32 : s, st0, false));
+        NATSL_TRY(side_join.join());
         if (normed)
             NATSL_TRY(launch_qk_norm_bwd_f32(q, k, true, route, f.dq32, f.dq_sm, f.dk32, f.dv32, dq, dk, dv,
-                                             (size_t)(B * L * H), p->d, hg.G, hg.norm_eps, st,
-                                             block ? f.dk_x : nullptr));
+                                             (size_t)(B * L * H), p->d, hg.G, hg.norm_eps, st, nullptr));
         return NATSL_OK;
     }
     // ---- fp32 CUDA-core path: softmax branch, reverse scan, chunk-level products as tile GEMMs, assembly ----

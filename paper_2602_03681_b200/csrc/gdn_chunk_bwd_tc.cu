@@ -105,7 +105,7 @@ template <int D> struct BPm {                 // B stored [n][k] in pieces of k,
 // BT: B stored [k][n] (else [n][k]).
 template <int NT, int K, bool AT, bool BT, typename FA, typename FB>
 __device__ __forceinline__ void mma_block(FA fa, FB fb, float (&acc)[2][NT][4]) {
-#pragma unroll 4
+#pragma unroll 2
     for (int k0 = 0; k0 < K; k0 += 16) {
         uint32_t a[2][4];
 #pragma unroll
@@ -156,14 +156,23 @@ struct CbArgs {
     const float *dk_x, *dv_x;                        // kBlock: every token's softmax-branch dk, dv, added, or nullptr
     float scale_la;
     float *dg, *dbeta;
+    const __nv_bfloat16 *q, *k;                      // kNorm: the rows that were normalised
+    float norm_eps;
+    int G;
     float *kap_c;                                    // [B,H,L/C] or nullptr: sum over the chunk of kappa = <dS1, K~^T U~>
     int32_t *status;
     int L, H, wait_kcycles;
 };
 
 // kBlock: block-level routing (every token takes part in the delta rule, a softmax block's update was not
-// committed, every token's dk and dv have a softmax-branch part); TO: what dq, dk, dv are stored as.
-template <int D, bool kBlock, typename TO>
+// committed, every token's dk and dv have a softmax-branch part).
+// kNorm (with kBlock): q and k were normalised by the forward, dq_sm and dk_x are gradients with respect to the
+// softmax operation's copy, and the two row-local Jacobians are applied here, to the fp32 accumulators.  With x a row
+// of q (or k), r_l = rsqrt(|x|^2 + eps), r_s = rsqrt(mean_slice x^2 + eps) and g, h the gradients of the two copies,
+//   dx = r_l g + r_s h - x (r_l^3 <x, g> + r_s^3 mean_slice(x h)).
+// (A kernel of its own for this read the five fp32 gradients back: 945 MB, 135 us on 3840 chunks of 128 columns.)
+// TO: what dq, dk, dv are stored as.
+template <int D, bool kBlock, bool kNorm, typename TO>
 __global__ void __launch_bounds__(kCbThreads, CbLayout<D>::kCtas)
 gdn_chunk_bwd_kernel(const __grid_constant__ CUtensorMap map_do,     // dO16 [B*H*L][D], box 64 x 64
                      const __grid_constant__ CUtensorMap map_kh, const __grid_constant__ CUtensorMap map_qh,
@@ -210,6 +219,29 @@ gdn_chunk_bwd_kernel(const __grid_constant__ CUtensorMap map_do,     // dO16 [B*
         ms.bt[tid] = !kBlock && p.route[tk] ? 0.f : p.beta[tk];
     }
     __syncthreads();
+    // What comes later -- the operands that wait for their slots, and the rows that lanes read as fragments -- starts
+    // towards L2 now: as plain loads and copies behind the MMAs they were most of the kernel's waits.
+    if (tid == 32) {
+        tma_prefetch_l2_2d(&map_wt, 0, (int)(chunk * D));
+        tma_prefetch_l2_2d(&map_ut, 0, (int)(chunk * D));
+        bulk_prefetch_l2(p.Qh + ((size_t)bh * p.L + c * kC) * D, SL::kU);
+        bulk_prefetch_l2(p.dS16 + chunk * D * D, D * D * 2);
+    }
+    {                                   // (line by line: bulk prefetches of rows would queue up before the copies)
+        const int ln = tid & 3;
+        const size_t at = tok0 + (size_t)(tid >> 2) * ts;
+        if (ln < D / 32) {
+            if (p.dq_sm) prefetch_l2(p.dq_sm + at + 32 * ln);
+            if (kBlock && p.dv_x) prefetch_l2(p.dv_x + at + 32 * ln);
+            if (kBlock && p.dk_x) prefetch_l2(p.dk_x + at + 32 * ln);
+        }
+        if (ln < D / 64) {
+            prefetch_l2(p.v + at + 64 * ln);
+            if (kNorm) prefetch_l2(p.q + at + 64 * ln);
+        } else if (kNorm && ln < D / 32) {
+            prefetch_l2(p.k + at + 64 * ln - D);
+        }
+    }
     volatile int *abort_flag = &ms.abort_flag;
     // (a wait that runs out is recorded and the chain goes on: nothing below may leave a barrier short of threads)
     auto wait = [&](int i) { (void)mbar_wait(&ms.bar[i], 0, abort_flag); };
@@ -255,16 +287,117 @@ gdn_chunk_bwd_kernel(const __grid_constant__ CUtensorMap map_do,     // dO16 [B*
                 d[2 * mt + hf] = a;
             }
     };
-    auto store = [&](TO *dst, const float *add, float x0, float x1) {
-        if (add) {
-            const float2 y = *reinterpret_cast<const float2 *>(add);
-            x0 += y.x;
-            x1 += y.y;
-        }
-        if constexpr (sizeof(TO) == 2) *reinterpret_cast<uint32_t *>(dst) = pack_bf162(x0, x1);
-        else *reinterpret_cast<float2 *>(dst) = make_float2(x0, x1);
+    // Results leave in groups of four columns: lanes of a pair swap halves of two neighbouring 8-column tiles, so that
+    // tiles 2u and 2u + 1 of x hold columns cb + 16 u .. + 3 of a row.  (A lane's own pairs of columns took twice the
+    // load and store instructions for half the bytes each, and every one of them touches 8 rows.)
+    const int cb = n0 + 8 * (t & 1) + 4 * (t >> 1);
+    auto regroup = [&](float (&x)[2][NT][4]) {
+        const bool odd = t & 1;
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int u = 0; u < NT; u += 2)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float r = __shfl_xor_sync(0xffffffffu, odd ? x[mt][u][e] : x[mt][u + 1][e], 1);
+                    x[mt][u][e] = odd ? r : x[mt][u][e];
+                    x[mt][u + 1][e] = odd ? x[mt][u + 1][e] : r;
+                }
     };
-    float dG[4], db[4], kap[4] = {0.f, 0.f, 0.f, 0.f}, d4[4];
+    auto store = [&](TO *dst, float x0, float x1, float x2, float x3) {
+        if constexpr (sizeof(TO) == 2) *reinterpret_cast<uint2 *>(dst) = make_uint2(pack_bf162(x0, x1), pack_bf162(x2, x3));
+        else *reinterpret_cast<float4 *>(dst) = make_float4(x0, x1, x2, x3);
+    };
+    auto add4 = [](const float *add) { return add ? *reinterpret_cast<const float4 *>(add) : make_float4(0.f, 0.f, 0.f, 0.f); };
+    auto bf4 = [](uint2 w) {
+        return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
+                           __uint_as_float(w.y & 0xffff0000u));
+    };
+    // <y, x> over the four columns of tiles u, u + 1
+    auto dot4 = [](float4 y, const float (&x)[NT][4], int u, int hf, float a) {
+        return fmaf(y.x, x[u][2 * hf], fmaf(y.y, x[u][2 * hf + 1], fmaf(y.z, x[u + 1][2 * hf], fmaf(y.w, x[u + 1][2 * hf + 1], a))));
+    };
+    // kNorm: gradients of the two copies of a row of X -> gradient of the row, stored to dst.  x: g, regrouped,
+    // times 1 / f; add: the softmax operation's gradient.  o: 4 KB for each half of the rows, free for the 4 warps
+    // that share it (row dots of a row's 4 column blocks).
+    auto norm_store = [&](TO *dst, const __nv_bfloat16 *X, const float *add, float (&x)[2][NT][4], float f, uint32_t o) {
+        float *pt = reinterpret_cast<float *>(smem + o + (warp & 1) * 4096);
+        uint2 w[2][2][NT / 2];
+        float4 gs[2][2][NT / 2];
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+                const size_t at = tok0 + (size_t)rowi(mt, hf) * ts + cb;
+#pragma unroll
+                for (int u = 0; u < NT / 2; ++u) {
+                    w[mt][hf][u] = *reinterpret_cast<const uint2 *>(X + at + 16 * u);
+                    gs[mt][hf][u] = *reinterpret_cast<const float4 *>(add + at + 16 * u);
+                }
+            }
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+                float ss = 0.f, xg = 0.f, xs = 0.f;
+#pragma unroll
+                for (int u = 0; u < NT / 2; ++u) {
+                    const float4 y = bf4(w[mt][hf][u]), z = gs[mt][hf][u];
+                    ss = fmaf(y.x, y.x, fmaf(y.y, y.y, fmaf(y.z, y.z, fmaf(y.w, y.w, ss))));
+                    xg = dot4(y, x[mt], 2 * u, hf, xg);
+                    xs = fmaf(y.x, z.x, fmaf(y.y, z.y, fmaf(y.z, z.z, fmaf(y.w, z.w, xs))));
+                }
+#pragma unroll
+                for (int m = 1; m < 4; m <<= 1) {
+                    ss += __shfl_xor_sync(0xffffffffu, ss, m);
+                    xg += __shfl_xor_sync(0xffffffffu, xg, m);
+                    xs += __shfl_xor_sync(0xffffffffu, xs, m);
+                }
+                if (t == 0) {
+                    const int i = rowi(mt, hf) & 31;
+                    pt[i * 4 + wc] = ss;
+                    pt[128 + i * 4 + wc] = f * xg;
+                    pt[256 + i * 4 + wc] = xs;
+                }
+            }
+        named_barrier_sync(2 + (warp & 1), 128);
+        const bool two = p.G == 2;
+        const float inv_ds = (two ? 2.f : 1.f) / D;
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+                const int i = rowi(mt, hf) & 31;
+                const float4 a = *reinterpret_cast<const float4 *>(pt + i * 4);
+                const float4 b4 = *reinterpret_cast<const float4 *>(pt + 128 + i * 4);
+                const float4 e = *reinterpret_cast<const float4 *>(pt + 256 + i * 4);
+                const float s0 = a.x + a.y, s1 = a.z + a.w, x0 = e.x + e.y, x1 = e.z + e.w;
+                const float sl = two ? (wc < 2 ? s0 : s1) : s0 + s1, xl = two ? (wc < 2 ? x0 : x1) : x0 + x1;
+                const float rl = rsqrtf(s0 + s1 + p.norm_eps), rs = rsqrtf(fmaf(sl, inv_ds, p.norm_eps));
+                const float cx = rl * rl * rl * ((b4.x + b4.y) + (b4.z + b4.w)) + rs * rs * rs * (xl * inv_ds);
+                const size_t at = tok0 + (size_t)rowi(mt, hf) * ts + cb;
+                const float rf = rl * f;
+#pragma unroll
+                for (int u = 0; u < NT / 2; ++u) {
+                    const float4 y = bf4(w[mt][hf][u]), z = gs[mt][hf][u];
+                    store(dst + at + 16 * u, fmaf(-cx, y.x, fmaf(rf, x[mt][2 * u][2 * hf], rs * z.x)),
+                          fmaf(-cx, y.y, fmaf(rf, x[mt][2 * u][2 * hf + 1], rs * z.y)),
+                          fmaf(-cx, y.z, fmaf(rf, x[mt][2 * u + 1][2 * hf], rs * z.z)),
+                          fmaf(-cx, y.w, fmaf(rf, x[mt][2 * u + 1][2 * hf + 1], rs * z.w)));
+                }
+            }
+    };
+    // Row sums over the warp's columns: lane t of a quad keeps the one of row ri.  (As four partial sums a lane each
+    // they cost twelve registers, and a spilled register costs a trip to L2: shared memory leaves hardly any L1.)
+    const int ri = rowi(t >> 1, t & 1);
+    auto row_sum = [&](const float (&a)[4]) {
+        const bool odd = t & 1;
+        float x0 = odd ? a[1] : a[0], x1 = odd ? a[3] : a[2];
+        x0 += __shfl_xor_sync(0xffffffffu, odd ? a[0] : a[1], 1);
+        x1 += __shfl_xor_sync(0xffffffffu, odd ? a[2] : a[3], 1);
+        return (t & 2 ? x1 : x0) + __shfl_xor_sync(0xffffffffu, t & 2 ? x0 : x1, 2);
+    };
+    float dG, db, kap = 0.f, d4[4];
 
     // ---- N = dO U~^T;  Ns = scale_la (N . Gamma), j <= i  -> Y ----
     wait(0);
@@ -295,31 +428,50 @@ gdn_chunk_bwd_kernel(const __grid_constant__ CUtensorMap map_do,     // dO16 [B*
         mma_block<NT, D, false, true>(a_sw(SL::oA), b_pmt(SL::oE, n0), x);
         scale_rows(x, m0 + g, [&](int i) { return p.scale_la * exp_ftz(ms.G[i]); });
         mma_block<NT, 64, false, true>(a_sw(SL::oY), b_swt(SL::oK, n0), x);
+        regroup(x);
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
+        for (int mt = 0; mt < 2; ++mt) {
+            uint2 qw[2][NT / 2];
+            float4 z[2][NT / 2];
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf) {
                 const int i = rowi(mt, hf);
-                const __half *qr = p.Qh + ((size_t)bh * p.L + c * kC + i) * D + n0 + 2 * t;
-                const size_t at = tok0 + (size_t)i * ts + n0 + 2 * t;
+#pragma unroll
+                for (int u = 0; u < NT / 2; ++u) {
+                    qw[hf][u] = *reinterpret_cast<const uint2 *>(p.Qh + ((size_t)bh * p.L + c * kC + i) * D + cb + 16 * u);
+                    if (!kNorm) z[hf][u] = add4(p.dq_sm ? p.dq_sm + tok0 + (size_t)i * ts + cb + 16 * u : nullptr);
+                }
+            }
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+                const size_t at = tok0 + (size_t)rowi(mt, hf) * ts + cb;
                 float a = 0.f;
 #pragma unroll
-                for (int nt = 0; nt < NT; ++nt) {
-                    const float2 y = __half22float2(*reinterpret_cast<const __half2 *>(qr + 8 * nt));
-                    a = fmaf(y.x, x[mt][nt][2 * hf], fmaf(y.y, x[mt][nt][2 * hf + 1], a));
-                    store(dq + at + 8 * nt, p.dq_sm ? p.dq_sm + at + 8 * nt : nullptr, gsc.y * x[mt][nt][2 * hf],
-                          gsc.y * x[mt][nt][2 * hf + 1]);
+                for (int u = 0; u < NT; u += 2) {
+                    const uint2 w = qw[hf][u / 2];
+                    const float2 y0 = __half22float2(*reinterpret_cast<const __half2 *>(&w.x));
+                    const float2 y1 = __half22float2(*reinterpret_cast<const __half2 *>(&w.y));
+                    a = dot4(make_float4(y0.x, y0.y, y1.x, y1.y), x[mt], u, hf, a);
+                    if (!kNorm) {
+                        const float4 y = z[hf][u / 2];
+                        store(dq + at + 8 * u, fmaf(gsc.y, x[mt][u][2 * hf], y.x), fmaf(gsc.y, x[mt][u][2 * hf + 1], y.y),
+                              fmaf(gsc.y, x[mt][u + 1][2 * hf], y.z), fmaf(gsc.y, x[mt][u + 1][2 * hf + 1], y.w));
+                    }
                 }
-                dG[2 * mt + hf] = a;
+                d4[2 * mt + hf] = a;
             }
+        }
+        dG = row_sum(d4);
+        __syncthreads();                // dO has been read
+        if constexpr (kNorm) norm_store(dq, p.q, p.dq_sm, x, gsc.y, SL::oA);
     }
-    __syncthreads();                    // dO has been read
     // ---- dW = -dU~ S0^T  -> A ----
     wait(2);
     {
         float x[2][NT][4];
         zero_acc(x);
         mma_block<NT, D, true, true>(a_pmt(SL::oC, D), b_pmt(SL::oE, n0), x);
+        if (kNorm) named_barrier_sync(2 + (warp & 1), 128);    // norm_store's sums (in this half's rows) have been read
         put(SL::oA, x, -1.f);
     }
     __syncthreads();                    // dW in place; S0 has been read
@@ -336,28 +488,45 @@ gdn_chunk_bwd_kernel(const __grid_constant__ CUtensorMap map_do,     // dO16 [B*
         float x[2][NT][4];
         zero_acc(x);
         mma_block<NT, 64, true, false>(a_pmt(SL::oT, 64), b_pm(SL::oC, n0), x);
+        uint2 vw[2][NT / 2];                                // (every load of 16 rows ahead of their stores)
+        float4 z[2][NT / 2];
+        auto load_rows = [&](int mt) {
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
+            for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+                for (int u = 0; u < NT / 2; ++u) {
+                    const size_t at = tok0 + (size_t)rowi(mt, hf) * ts + cb + 16 * u;
+                    vw[hf][u] = *reinterpret_cast<const uint2 *>(p.v + at);
+                    z[hf][u] = add4(kBlock && p.dv_x ? p.dv_x + at : nullptr);
+                }
+        };
+        load_rows(0);
+        __syncthreads();                // dW and dU~ have been read
+        put(SL::oA, pp, 1.f);
+        put(SL::oC, x, 1.f);
+        regroup(x);
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) {
+            if (mt) load_rows(mt);
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf) {
                 const int i = rowi(mt, hf);
-                const size_t at = tok0 + (size_t)i * ts + n0 + 2 * t;
+                const size_t at = tok0 + (size_t)i * ts + cb;
                 const bool lin = kBlock || p.route[((size_t)b * p.L + (size_t)c * kC + i) * p.H + h] == 0;
                 const float f = gsc.y * ms.bt[i];
                 float a = 0.f;
 #pragma unroll
-                for (int nt = 0; nt < NT; ++nt) {
-                    const float2 y = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p.v + at + 8 * nt));
-                    a = fmaf(y.x, x[mt][nt][2 * hf], fmaf(y.y, x[mt][nt][2 * hf + 1], a));
+                for (int u = 0; u < NT; u += 2) {
+                    const float4 y = z[hf][u / 2];
+                    a = dot4(bf4(vw[hf][u / 2]), x[mt], u, hf, a);
                     if (lin)
-                        store(dv + at + 8 * nt, kBlock && p.dv_x ? p.dv_x + at + 8 * nt : nullptr, f * x[mt][nt][2 * hf],
-                              f * x[mt][nt][2 * hf + 1]);
+                        store(dv + at + 8 * u, fmaf(f, x[mt][u][2 * hf], y.x), fmaf(f, x[mt][u][2 * hf + 1], y.y),
+                              fmaf(f, x[mt][u + 1][2 * hf], y.z), fmaf(f, x[mt][u + 1][2 * hf + 1], y.w));
                 }
-                db[2 * mt + hf] = a;
+                d4[2 * mt + hf] = a;
             }
-        __syncthreads();                // dW and dU~ have been read
-        put(SL::oA, pp, 1.f);
-        put(SL::oC, x, 1.f);
+        }
+        db = row_sum(d4);
     }
     __syncthreads();
     // ---- M = -(dKb W^T + dVb U^T);  Mg = M . Gamma, j < i -> T;  Ms = diag(beta~) Mg -> A ----
@@ -397,12 +566,13 @@ gdn_chunk_bwd_kernel(const __grid_constant__ CUtensorMap map_do,     // dO16 [B*
     scale_rows(pp, m0 + g, [&](int i) { return exp_ftz(ms.G[i]); });
     mma_block<NT, 64, false, true>(a_sw(SL::oT), b_swt(SL::oK, n0), pp);
     dot_sw(SL::oK, pp, d4);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        db[e] += d4[e];
-        dG[e] = fmaf(ms.bt[rowi(e >> 1, e & 1)], d4[e], dG[e]);
+    {
+        const float a = row_sum(d4);
+        db += a;
+        dG = fmaf(ms.bt[ri], a, dG);
     }
     // ---- R = (gamma_C / gamma) dK~ + Ms^T K + Ns^T Q;  dk = beta~ P + R ----
+    if (kNorm) __syncthreads();         // Mg has been read: norm_store's sums go there
     wait(4);
     {
         float x[2][NT][4];
@@ -413,28 +583,42 @@ gdn_chunk_bwd_kernel(const __grid_constant__ CUtensorMap map_do,     // dO16 [B*
             mma_block<NT, D, true, true>(a_pmt(SL::oB, D), b_pmt(oS, n0), x);
             const float GC = ms.G[63];
             scale_rows(x, m0 + g, [&](int i) { return exp_ftz(GC - ms.G[i]); });
-            dot_sw(SL::oK, x, kap);
+            dot_sw(SL::oK, x, d4);
+            kap = row_sum(d4);
         }
         mma_block<NT, 64, true, true>(a_swt(SL::oA), b_swt(SL::oK, n0), x);
         mma_block<NT, 64, true, true>(a_swt(SL::oY), b_swt(SL::oUt, n0), x);
         dot_sw(SL::oK, x, d4);
+        dG -= row_sum(d4);
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf) {
-                const int i = rowi(mt, hf);
-                const size_t at = tok0 + (size_t)i * ts + n0 + 2 * t;
-                const bool lin = kBlock || p.route[((size_t)b * p.L + (size_t)c * kC + i) * p.H + h] == 0;
-                const float bt = ms.bt[i];
-                dG[2 * mt + hf] -= d4[2 * mt + hf];
-                if (lin) {
+                const float bt = ms.bt[rowi(mt, hf)];
 #pragma unroll
-                    for (int nt = 0; nt < NT; ++nt)
-                        store(dk + at + 8 * nt, kBlock && p.dk_x ? p.dk_x + at + 8 * nt : nullptr,
-                              gsc.y * fmaf(bt, pp[mt][nt][2 * hf], x[mt][nt][2 * hf]),
-                              gsc.y * fmaf(bt, pp[mt][nt][2 * hf + 1], x[mt][nt][2 * hf + 1]));
+                for (int nt = 0; nt < NT; ++nt) {
+                    x[mt][nt][2 * hf] = fmaf(bt, pp[mt][nt][2 * hf], x[mt][nt][2 * hf]);
+                    x[mt][nt][2 * hf + 1] = fmaf(bt, pp[mt][nt][2 * hf + 1], x[mt][nt][2 * hf + 1]);
                 }
             }
+        regroup(x);
+        if (!kNorm) {
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) {
+                    const int i = rowi(mt, hf);
+                    const size_t at = tok0 + (size_t)i * ts + cb;
+                    if (!kBlock && p.route[((size_t)b * p.L + (size_t)c * kC + i) * p.H + h] != 0) continue;
+#pragma unroll
+                    for (int u = 0; u < NT; u += 2) {
+                        const float4 z = add4(kBlock && p.dk_x ? p.dk_x + at + 8 * u : nullptr);
+                        store(dk + at + 8 * u, fmaf(gsc.y, x[mt][u][2 * hf], z.x), fmaf(gsc.y, x[mt][u][2 * hf + 1], z.y),
+                              fmaf(gsc.y, x[mt][u + 1][2 * hf], z.z), fmaf(gsc.y, x[mt][u + 1][2 * hf + 1], z.w));
+                    }
+                }
+        }
+        if constexpr (kNorm) norm_store(dk, p.k, p.dk_x, x, gsc.y, SL::oT);
     }
     // ---- <dS1, S0>, element for element (the same layout twice) ----
     {
@@ -461,22 +645,11 @@ gdn_chunk_bwd_kernel(const __grid_constant__ CUtensorMap map_do,     // dO16 [B*
         if (lane == 0) ms.red[warp] = a;
     }
     __syncthreads();                    // every operand has been read
-    // ---- per-token sums: the 4 lanes of a row, then the 4 column blocks in a fixed order ----
+    // ---- per-token sums: the 4 column blocks in a fixed order ----
     float *rs = reinterpret_cast<float *>(smem);                            // dG, kappa, dbeta: [3][4][64]
-    auto quad = [](float x) {
-        x += __shfl_xor_sync(0xffffffffu, x, 1);
-        return x + __shfl_xor_sync(0xffffffffu, x, 2);
-    };
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const float a = quad(dG[e]), k4 = quad(kap[e]), b4 = quad(db[e]);
-        if (t == 0) {
-            const int i = rowi(e >> 1, e & 1);
-            rs[wc * 64 + i] = a;
-            rs[256 + wc * 64 + i] = k4;
-            rs[512 + wc * 64 + i] = b4;
-        }
-    }
+    rs[wc * 64 + ri] = dG;
+    rs[256 + wc * 64 + ri] = kap;
+    rs[512 + wc * 64 + ri] = db;
     __syncthreads();
     if (tid < 64) {
         // dg_j = sum_{i >= j} dG_i + sum_i kappa_i + gamma_C <dS1, S0>  (i, j: tokens of the chunk)
@@ -509,7 +682,7 @@ gdn_chunk_bwd_kernel(const __grid_constant__ CUtensorMap map_do,     // dO16 [B*
     }
 }
 
-template <int D, bool kBlock, typename TO>
+template <int D, bool kBlock, bool kNorm, typename TO>
 cudaError_t chunk_bwd_impl(const CbArgs &a, const void *dO16, const void *Kh, const void *Wt, const void *U16,
                            void *dq, void *dk, void *dv, Shape s, cudaStream_t st) {
     const int NC = s.L / kC;
@@ -519,7 +692,7 @@ cudaError_t chunk_bwd_impl(const CbArgs &a, const void *dO16, const void *Kh, co
         !tch::make_map_2d(&mqh, a.Qh, BH * s.L, D, 64) || !tch::make_map_2d(&mwt, Wt, BH * NC * D, 64, D) ||
         !tch::make_map_2d(&mut, U16, BH * NC * D, 64, D))
         return cudaErrorInvalidValue;
-    auto kernel = gdn_chunk_bwd_kernel<D, kBlock, TO>;
+    auto kernel = gdn_chunk_bwd_kernel<D, kBlock, kNorm, TO>;
     cudaError_t e = allow_smem(kernel, CbLayout<D>::kTotal);
     if (e != cudaSuccess) return e;
     dim3 grid(NC, s.B * s.H);
@@ -530,23 +703,27 @@ cudaError_t chunk_bwd_impl(const CbArgs &a, const void *dO16, const void *Kh, co
 
 }  // namespace
 
-cudaError_t launch_gdn_chunk_bwd(const GdnTcWs &ws, const GdnTcExport &ex, const GdnTcGrads &gr, const void *v,
-                                 const float *beta, const uint8_t *route, const float *dq_sm, float scale_la, void *dq,
-                                 void *dk, void *dv, bool out_f32, float *dg, float *dbeta, bool block,
-                                 const float *dk_x, const float *dv_x, float *kap_c, int32_t *status, Shape s,
-                                 cudaStream_t st) {
+cudaError_t launch_gdn_chunk_bwd(const GdnTcWs &ws, const GdnTcExport &ex, const GdnTcGrads &gr, const void *q,
+                                 const void *k, const void *v, const float *beta, const uint8_t *route,
+                                 const float *dq_sm, float scale_la, void *dq, void *dk, void *dv, float *dg,
+                                 float *dbeta, bool block, const float *dk_x, const float *dv_x, float *kap_c,
+                                 int32_t *status, Shape s, cudaStream_t st, HeadGroups hg) {
+    const bool normed = hg.norm_eps >= 0.f;
     const CbArgs a{(const __half *)ex.Ut16, (const __half *)gr.dU16, (const __half *)ex.S16, (const __half *)gr.dS16,
                    (const __half *)ex.T16, (const __half *)ws.Qh, (const __nv_bfloat16 *)v, ex.Gcum, beta, dq_sm, route,
-                   dk_x, dv_x, scale_la, dg, dbeta, kap_c, status, s.L, s.H, debug_wait_kcycles()};
-#define RUN(D, BL, T) return chunk_bwd_impl<D, BL, T>(a, gr.dO16, ws.Kh, ws.Wt, ex.U16, dq, dk, dv, s, st)
-    if (s.d == 128) {
-        if (out_f32) { if (block) RUN(128, true, float); RUN(128, false, float); }
-        if (block) RUN(128, true, __nv_bfloat16);
-        RUN(128, false, __nv_bfloat16);
+                   dk_x, dv_x, scale_la, dg, dbeta, (const __nv_bfloat16 *)q, (const __nv_bfloat16 *)k, hg.norm_eps,
+                   hg.G, kap_c, status, s.L, s.H, debug_wait_kcycles()};
+#define RUN(BL, NO, T)                                                                                               \
+    do {                                                                                                             \
+        if (s.d == 128) return chunk_bwd_impl<128, BL, NO, T>(a, gr.dO16, ws.Kh, ws.Wt, ex.U16, dq, dk, dv, s, st); \
+        return chunk_bwd_impl<64, BL, NO, T>(a, gr.dO16, ws.Kh, ws.Wt, ex.U16, dq, dk, dv, s, st);                  \
+    } while (0)
+    if (block) {
+        if (normed) RUN(true, true, __nv_bfloat16);
+        RUN(true, false, __nv_bfloat16);
     }
-    if (out_f32) { if (block) RUN(64, true, float); RUN(64, false, float); }
-    if (block) RUN(64, true, __nv_bfloat16);
-    RUN(64, false, __nv_bfloat16);
+    if (normed) RUN(false, false, float);
+    RUN(false, false, __nv_bfloat16);
 #undef RUN
 }
 

@@ -256,12 +256,13 @@ cudaError_t launch_gdn_rscan_tc(const GdnTcWs &ws, const GdnTcGrads &gr, const f
 // gdn_chunk_bwd_tc.cu: everything of the linear branch's backward that follows the reverse scan, fused per chunk
 // (bf16 storage): dq (dq_sm added unless nullptr), dk, dv of the linear tokens -- or, with block-level routing, of
 // every token, dk_x / dv_x (its softmax-branch part, or nullptr) added --, dg, dbeta and the chunk sums of kappa
-// (kap_c [B,H,L/C] or nullptr).  out_f32: dq, dk, dv as fp32.
-cudaError_t launch_gdn_chunk_bwd(const GdnTcWs &ws, const GdnTcExport &ex, const GdnTcGrads &gr, const void *v,
-                                 const float *beta, const uint8_t *route, const float *dq_sm, float scale_la, void *dq,
-                                 void *dk, void *dv, bool out_f32, float *dg, float *dbeta, bool block,
-                                 const float *dk_x, const float *dv_x, float *kap_c, int32_t *status, Shape s,
-                                 cudaStream_t st);
+// (kap_c [B,H,L/C] or nullptr).  With the normalisation of q and k (hg): block-level routing applies its Jacobians to
+// the fp32 results and dq_sm, dk_x; token-level routing leaves dq, dk, dv in fp32 for launch_qk_norm_bwd_f32.
+cudaError_t launch_gdn_chunk_bwd(const GdnTcWs &ws, const GdnTcExport &ex, const GdnTcGrads &gr, const void *q,
+                                 const void *k, const void *v, const float *beta, const uint8_t *route,
+                                 const float *dq_sm, float scale_la, void *dq, void *dk, void *dv, float *dg,
+                                 float *dbeta, bool block, const float *dk_x, const float *dv_x, float *kap_c,
+                                 int32_t *status, Shape s, cudaStream_t st, HeadGroups hg);
 cudaError_t launch_gdn_tsolve(const float *Abar, const float *beta, const uint8_t *route,
                               const float *dW, const float *dUt, float *dKb, float *dVb, Shape s,
                               cudaStream_t st);

@@ -382,6 +382,17 @@ softmax_bwd_own_block_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfl
     const size_t rowA = (size_t)bhg * L + (size_t)c * kC + iA;
     const float l2e = 1.4426950408889634f;
     const float lseA = lse[rowA] * l2e, lseB = lse[rowA + 8] * l2e, DA = Dsm[rowA], DB = Dsm[rowA + 8];
+    // dq so far, this lane's groups of four columns: asked for before the products, added after them
+    const size_t col4 = tok0 + (size_t)iA * ts + n0 + 8 * (t & 1) + 4 * (t >> 1);
+    float4 dq_old[2][2];
+    auto load_dq = [&](int kb) {
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+                dq_old[hf][u] = *reinterpret_cast<const float4 *>(dq_sm + col4 + (size_t)(8 * hf) * ts + kb * 64 + 16 * u);
+    };
+    load_dq(0);
     float pr[4][4], acc[4][4];
     auto zero = [](float (&a)[4][4]) {
 #pragma unroll
@@ -418,31 +429,40 @@ softmax_bwd_own_block_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfl
         for (int e = 0; e < 4; ++e) acc[nt][e] = scale_sm * pr[nt][e] * (acc[nt][e] - (e < 2 ? DA : DB));
     put(sDS, acc);
     __syncthreads();
-    auto out2 = [&](float *dst, const float (&a)[4][4], bool add, int kb) {
+    // Rows leave in groups of four columns: the lanes of a pair swap halves of neighbouring 8-column tiles.
+    auto out4 = [&](float *dst, float (&a)[4][4], const float4 (*add)[2], int kb) {
+        const bool odd = t & 1;
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            float2 *pa = reinterpret_cast<float2 *>(dst + tok0 + (size_t)iA * ts + kb * 64 + n0 + 8 * nt + 2 * t);
-            float2 *pb = reinterpret_cast<float2 *>(dst + tok0 + (size_t)iB * ts + kb * 64 + n0 + 8 * nt + 2 * t);
-            float2 va = make_float2(ginv * a[nt][0], ginv * a[nt][1]), vb = make_float2(ginv * a[nt][2], ginv * a[nt][3]);
-            if (add) {
-                const float2 ca = *pa, cb = *pb;
-                va.x += ca.x; va.y += ca.y; vb.x += cb.x; vb.y += cb.y;
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                float &x0 = a[2 * u][e], &x1 = a[2 * u + 1][e];
+                const float r = __shfl_xor_sync(0xffffffffu, odd ? x0 : x1, 1);
+                x0 = odd ? r : x0;
+                x1 = odd ? x1 : r;
             }
-            *pa = va;
-            *pb = vb;
-        }
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const float4 y = add ? add[hf][u] : make_float4(0.f, 0.f, 0.f, 0.f);
+                *reinterpret_cast<float4 *>(dst + col4 + (size_t)(8 * hf) * ts + kb * 64 + 16 * u) =
+                    make_float4(fmaf(ginv, a[2 * u][2 * hf], y.x), fmaf(ginv, a[2 * u][2 * hf + 1], y.y),
+                                fmaf(ginv, a[2 * u + 1][2 * hf], y.z), fmaf(ginv, a[2 * u + 1][2 * hf + 1], y.w));
+            }
     };
 #pragma unroll
     for (int kb = 0; kb < KB; ++kb) {
         zero(acc);
         mma64<false, false>(sDS, sK + kb * kTileH, row0, n0, lane, acc);          // dq += dS K
-        out2(dq_sm, acc, true, kb);
+        out4(dq_sm, acc, dq_old, kb);
+        if (kb + 1 < KB) load_dq(kb + 1);
         zero(acc);
         mma64<true, false>(sDS, sQ + kb * kTileH, row0, n0, lane, acc);           // dk = dS^T Q
-        out2(dk_x, acc, false, kb);
+        out4(dk_x, acc, nullptr, kb);
         zero(acc);
         mma64<true, false>(sP, sDO + kb * kTileH, row0, n0, lane, acc);           // dv = P^T dO
-        out2(dv_x, acc, false, kb);
+        out4(dv_x, acc, nullptr, kb);
     }
 }
 

@@ -417,7 +417,7 @@ def run_ours(args):
         "stages_ms": stage_ms,
         "stages_note": ("stage times are taken in a separate pass with the library's per-stage events, "
                         "which makes it run the stages in sequence; in the timed steps the compaction "
-                        "and the gather run on a side stream beside the prepare kernel, so a step is "
+                        "and the gather start in the prepare kernel's last wave and the softmax kernel beside the scan, so a step is "
                         "shorter than the sum of the stages"),
         "step": {"useful_tflops": step_tf, "frac_of_bf16_peak": step_tf / peak_tf,
                  "useful_gflop": total_flops / 1e9, "min_hbm_bytes": min_hbm_bytes_fwd(wl, B),
@@ -580,8 +580,7 @@ def bench_grouped_heads(peaks, peak_kind, B=10, H=6, G=2):
            "tokens_per_s": B * wl.L / (ms["grouped_qk_norm"] * 1e-3), "useful_fwd_gflop": fl / 1e9,
            "roofline": {"fwd": tensor_roofline(fl, ms["grouped_qk_norm"], peaks, peak_kind)}}
     # The mode the paper's models run in -- one routing decision per block, grouped heads, normalised q, k --
-    # forward and training step (forward saved in the backward's workspace, then the backward; at d = 128
-    # the backward's chunk-level products are CUDA-core tile GEMMs).
+    # forward and training step (forward saved in the backward's workspace, then the backward).
     xb = inputs.make_layer_inputs(wl, route=inputs.route_blocks(wl.seed, (B, wl.L, H), wl.p_softmax))
     rb = torch.from_numpy(xb["route"]).cuda()
     dout = torch.from_numpy(xb["dout"]).cuda().to(torch.bfloat16)

@@ -19,11 +19,11 @@
  * buffers and the stream; the library allocates no device memory and keeps no per-call state.
  * Calls are asynchronous and ordered on `stream` (a cudaStream_t passed as void*; NULL = default
  * stream) like any other work of that stream.  What the library does own, per device and created
- * on the first forward or backward call there that may use it: one non-blocking stream and two
+ * on the first backward call there that may use it: one non-blocking stream and two
  * events, on which stages that do not depend on each other run beside the caller's stream (forked
  * from it and joined back into it within the call), and one process-wide mutex that covers the
  * enqueue of such a call, because the two events are shared.  NATSL_SINGLE_STREAM and
- * natsl_hybrid_fwd_static use none of this.  The device of `stream` and of all tensors must be
+ * the forward use none of this.  The device of `stream` and of all tensors must be
  * the current device of the calling thread.
  * All tensors are dense, row-major, innermost dimension contiguous, in the shapes given (no
  * strides are taken: a caller with another layout makes a contiguous copy).  Base pointers of
@@ -92,8 +92,8 @@ enum {
                                     decay alone).  state_out, k_sm, v_sm, sm_len hold what is kept
                                     after the last block.  A route that changes inside a block is
                                     reported as NATSL_ERR_ROUTE by natsl_device_status.  Backward:
-                                    built on every path (bf16 storage with d = 64: fused per
-                                    chunk; d = 128 and fp32 storage: the chunk-level products as
+                                    built on every path (bf16 storage: one kernel per
+                                    chunk; fp32 storage: the chunk-level products as
                                     separate kernels).  Generation: route 2 in
                                     natsl_decode_step and natsl_decode_block_end (no flag needed) */
     NATSL_APPEND_CACHE = 1u << 3,      /* forward, tensor-core path: prefill in pieces.  p->k_sm, p->v_sm,
@@ -110,11 +110,12 @@ enum {
                                     and on p->sm_cap.  Backward: NATSL_ERR_UNSUPPORTED */
     NATSL_SINGLE_STREAM = 1u << 4,     /* forward and backward, tensor-core path: launch everything on
                                     the caller's stream.  By default stages that do not depend on
-                                    each other (route compaction + gather beside the linear branch's
-                                    prepare kernel; in the backward also the reverse scan beside the
-                                    softmax branch's backward) run side by side, one of them on a
+                                    each other run side by side: in the backward the reverse scan and
+                                    the key-side softmax kernel beside the query-side one, on a
                                     stream the library creates once per device, forked from and
-                                    joined to the caller's stream with events, so the call is still
+                                    joined to the caller's stream with events; in the forward (which
+                                    stays on the caller's stream) as programmatic dependent launches.
+                                    The call is still
                                     ordered like any other work on that stream.  Also implied by
                                     p->stage_events.  natsl_hybrid_fwd_static always sets it.  The
                                     forward then also runs its kernels strictly one after the other

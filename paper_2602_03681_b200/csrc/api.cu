@@ -4,6 +4,7 @@
 
 #include "natsl_internal.h"
 
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 
@@ -85,21 +86,21 @@ bool use_tensor_cores(const natsl_params *p) {
 // the L2 bandwidth the scans then fight for: 60 of them took 310-370 us there instead of 128 us.
 bool scan_follows_closely(const natsl_params *p) { return (long long)p->B * p->H * (p->L / kC) <= 4 * 148; }
 
-// Segments of the forward scan (tensor-core path): the largest power of two that keeps the two
-// runs per segment within ~one CTA per SM, divides the chunk count and leaves >= 8 chunks each.
-int scan_segments(const natsl_params *p) {
+// Segments of the forward scan (tensor-core path).  A (batch, head) costs one CTA per SM for as long as its chain of
+// chunks, so with few of them most of the GPU waits.  Up to 32 pairs a first pass over the segments (1.6 us per chunk
+// against 2.1 with outputs) gains more than it costs: there are as many segments as keep its 2 nseg - 3 runs per pair
+// in one wave, at least 4 chunks long (shorter ones gain less than their step of the chain), and at least three --
+// with two the two passes are as long as one over everything.  32 pairs: 3 segments, 16: 6, 4: 20.
+// The last segment takes what remains, about half as much again: the first pass does not run it, and in the second the
+// softmax kernel fills the other multiprocessors.  *chunks: of the others, even, so that they are whole query tiles.
+int scan_segments(const natsl_params *p, int *chunks = nullptr) {
     if (!use_tensor_cores(p) || (p->flags & NATSL_SINGLE_PASS_SCAN)) return 1;
     const int NC = p->L / kC, BH = p->B * p->H;
-    int nseg = 1;
-    while (2 * BH * (nseg * 2) <= 128 && NC % (nseg * 2) == 0 && NC / (nseg * 2) >= 8) nseg *= 2;
-    // Once the scan is segmented (and so already pays its second run), one more doubling up to one CTA per
-    // SM: the two runs shrink by half again, which outweighs what the softmax kernel loses beside them --
-    // unless the call appends to a cache: the softmax kernel then also reads the earlier pieces' keys, is
-    // the longer of the two and needs the multiprocessors (a long prompt in pieces was 14 % slower with it).
-    if (!(p->flags & NATSL_APPEND_CACHE) && nseg >= 2 && BH * (nseg * 2) <= 128 && NC % (nseg * 2) == 0 &&
-        NC / (nseg * 2) >= 8)
-        nseg *= 2;
-    return nseg;
+    if (BH > 32 || NC < 16) return 1;
+    const int most = std::min((148 / BH + 3) / 2, 32);
+    const int n = std::max(4, ((2 * NC + 2 * most) / (2 * most + 1) + 1) & ~1);
+    if (chunks) *chunks = n;
+    return NC / n >= 3 ? NC / n : 1;
 }
 
 FwdWs carve_fwd(const natsl_params *p, void *ws) {
@@ -502,7 +503,8 @@ int natsl_hybrid_fwd(const void *q, const void *k, const void *v, const float *g
         //   up o_la chunk by chunk behind the counters the scan raises.
         // Per-stage events and NATSL_SINGLE_STREAM switch the overlap off (kernels in sequence).
         const bool beside = !p->stage_events && !(p->flags & NATSL_SINGLE_STREAM);
-        const int nseg = scan_segments(p);
+        int seg_chunks = 0;
+        const int nseg = scan_segments(p, &seg_chunks);
         const bool pdl = beside && scan_follows_closely(p);
         auto prepare = [&]() {   // block-level routing: every token takes part in the delta rule of its own block
             return launch_gdn_prepare_tc(q, k, v, g, beta, block ? nullptr : route, p->scale_la, f.tc, GdnTcExport{},
@@ -522,12 +524,12 @@ int natsl_hybrid_fwd(const void *q, const void *k, const void *v, const float *g
         const int32_t *flags_softmax = beside ? f.emit_flags : nullptr;
         const ScanOut so{f.o_la16, p->o_la, flags_scan};
         if (nseg > 1) {   // few (batch, head) pairs: segments in parallel, chained by their transitions
-            ScanSegments sg{1, nseg, (int)(p->L / kC) / nseg, f.seg_incr, f.seg_trans, f.seg_start};
-            NATSL_TRY(launch_gdn_scan_tc(f.tc, p->scale_la, nullptr, nullptr, so, GdnTcExport{}, sg,
+            ScanSegments sg{1, nseg, seg_chunks, f.seg_incr, f.seg_trans, f.seg_start};
+            NATSL_TRY(launch_gdn_scan_tc(f.tc, p->scale_la, p->state_in, nullptr, so, GdnTcExport{}, sg,
                                          br.route, f.status, s, st, pdl));
-            NATSL_TRY(launch_scan_combine(p->state_in, sg, s, st, pdl));
+            NATSL_TRY(launch_scan_combine(sg, s, st, pdl));
             sg.mode = 2;
-            NATSL_TRY(launch_gdn_scan_tc(f.tc, p->scale_la, nullptr, p->state_out, so, GdnTcExport{}, sg,
+            NATSL_TRY(launch_gdn_scan_tc(f.tc, p->scale_la, p->state_in, p->state_out, so, GdnTcExport{}, sg,
                                          br.route, f.status, s, st, pdl));
         } else {
             NATSL_TRY(launch_gdn_scan_tc(f.tc, p->scale_la, p->state_in, p->state_out, so, GdnTcExport{},
@@ -537,7 +539,8 @@ int natsl_hybrid_fwd(const void *q, const void *k, const void *v, const float *g
         NATSL_TRY(mark());
         NATSL_TRY(launch_softmax_combine_tc(q, k_soft, f.v16, cap_soft, capv, f.sm_idx, f.prefix, f.o_la16,
                                             flags_softmax, p->w, p->scale_sm, p->eps, out, p->o_nla,
-                                            p->lse, want_cache ? p->sm_len : nullptr, cap, br, append, f.status, s, st, hg));
+                                            p->lse, want_cache ? p->sm_len : nullptr, cap, br, append, f.status, s, st, hg, nseg,
+                                            seg_chunks / 2));
         NATSL_TRY(mark());
         return NATSL_OK;
     }

@@ -591,11 +591,13 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
     const int NC = L / kC;
     // Which (batch, head), which segment of its chunks, and which of the two segment runs (see
     // ScanSegments): c below counts the chunks of the segment, c0 + c is the chunk's index.
-    const int var = sg.mode == 1 ? (int)(blockIdx.x & 1) : 0;
-    const int slot = sg.mode == 1 ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;    // bh * nseg + seg
-    const int seg = sg.mode == 0 ? 0 : slot % sg.nseg;
-    const int bh = sg.mode == 0 ? slot : slot / sg.nseg, b = bh / H, h = bh % H;
-    const int ncs = sg.mode == 0 ? NC : sg.ncs, c0 = seg * ncs;
+    const int runs = sg.mode == 0 ? 1 : sg.mode == 1 ? 2 * sg.nseg - 3 : sg.nseg;     // CTAs per (batch, head)
+    const int bh = blockIdx.x / runs, run = blockIdx.x % runs, b = bh / H, h = bh % H;
+    const int var = sg.mode == 1 && run >= sg.nseg - 1 ? 1 : 0;
+    const int seg = var ? run - (sg.nseg - 2) : run;                                  // (mode 0: 0)
+    const int slot = bh * sg.nseg + seg;
+    const int c0 = seg * sg.ncs;
+    const int ncs = sg.mode == 0 ? NC : seg == sg.nseg - 1 ? NC - c0 : sg.ncs;
     const bool emit_out = sg.mode != 1, zero_u = sg.mode == 1 && var == 1;
 
     if ((smem_u32(smem) & 1023u) != 0) {
@@ -732,8 +734,8 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
 #pragma unroll
         for (int x = 0; x < kHalfCols; ++x)
             S[x] = !active ? 0.f
-                   : sg.mode == 1 ? (var == 1 && col0 + x == r ? 1.f : 0.f)
-                   : sg.mode == 2 ? sg.start[((size_t)slot * D + col0 + x) * D + r]
+                   : var          ? (col0 + x == r ? 1.f : 0.f)
+                   : seg > 0      ? (sg.mode == 2 ? sg.start[((size_t)slot * D + col0 + x) * D + r] : 0.f)
                    : state_in     ? state_in[((size_t)bh * D + col0 + x) * D + r]
                                   : 0.f;
         // This thread's 8 pieces (4 tokens each) of row r of U^T of chunk c.
@@ -929,69 +931,112 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
     if (tid == 0 && ms.abort_flag) atomicMin(status, (int)NATSL_ERR_TIMEOUT);
 }
 
-// start[0] = state_in (or 0); start[s+1] = M_s start[s] + B_s.  The value columns are independent: one CTA
-// per (batch, head) and kCombCols of them.  The chain over the segments is serial, so what counts is the time
-// of one step: two threads per key row hold its two halves of M_s in registers (fetched one segment ahead), the
-// state's columns are read as broadcast 16-byte pieces from shared memory, and fp32 FMAs do the rest.
-// (With M_s staged through shared memory in tiles and one shared-memory operand pair per FMA a step took
-// 11.8 us at d = 128; 16 pairs x 8 segments 83 us together.)
-constexpr int kCombCols = 4;
+// start[1] = incr[0]; start[s+1] = M_s start[s] + B_s.  The value columns are independent: one CTA per (batch, head)
+// and 16 of them.  The chain over the segments is serial, so what counts is the time of one step.  Four threads hold
+// two rows of M_s in registers, a quarter each (the next segment's are fetched meanwhile); the state's columns come
+// from shared memory, a row's four pieces rotated by the quarter that reads it (no bank conflicts), and packed fp32
+// FMAs do the rest: a step is 1024 FMAs and 128 loads per thread.
+// (With 4 columns per CTA every CTA of a pair read all of M_s, 33 MB per step for 16 pairs of 128 columns: 8 us a step.)
+constexpr int kCombCols = 16;
 template <int D>
 __global__ void __launch_bounds__(2 * D)
-scan_combine_kernel(const float *__restrict__ state_in, const float *__restrict__ incr,
-                    const float *__restrict__ trans, float *__restrict__ start, int nseg) {
-    constexpr int kV = kCombCols, kHalf = D / 2;
-    __shared__ float4 Ss[2][D];                        // the state's kV columns, double-buffered
-    const int bh = blockIdx.y, v0 = blockIdx.x * kV, a = threadIdx.x >> 1, hf = threadIdx.x & 1;
+scan_combine_kernel(const float *__restrict__ incr, const float *__restrict__ trans, float *__restrict__ start, int nseg) {
+    constexpr int kP = D / 16;                         // 16-byte pieces of a row per thread
+    __shared__ ulonglong2 Ss[2][D][4];                 // the state's 16 columns, double-buffered
+    const int bh = blockIdx.y, v0 = blockIdx.x * kCombCols, r0 = (threadIdx.x >> 2) * 2, qt = threadIdx.x & 3;
     grid_dependency_wait();
     launch_dependents();
-    // this thread's half of the row: pieces 2 j + hf (16 bytes each), so that a pair reads 32 contiguous bytes
-    float4 m[kHalf / 4];
-    auto fetch = [&](int sgi) {
-        const float4 *src = reinterpret_cast<const float4 *>(trans + (((size_t)bh * nseg + sgi) * D + a) * D) + hf;
+    float4 m[2][2][kP];                                // [buffer][row][piece 4 j + qt]
+    auto fetch = [&](int sgi, float4 (&dst)[2][kP]) {
 #pragma unroll
-        for (int j = 0; j < kHalf / 4; ++j) m[j] = __ldg(src + 2 * j);
-    };
-    const size_t row = (size_t)a * D + v0;
-    float4 cur = make_float4(0.f, 0.f, 0.f, 0.f), inc;
-    if (state_in) cur = *reinterpret_cast<const float4 *>(state_in + (size_t)bh * D * D + row);
-    if (nseg > 1) fetch(0);
-    for (int sgi = 0; sgi < nseg; ++sgi) {
-        const size_t base = ((size_t)bh * nseg + sgi) * D * D;
-        if (hf == 0) {
-            *reinterpret_cast<float4 *>(start + base + row) = cur;
-            Ss[sgi & 1][a] = cur;
+        for (int rr = 0; rr < 2; ++rr) {
+            const float4 *src = reinterpret_cast<const float4 *>(trans + (((size_t)bh * nseg + sgi) * D + r0 + rr) * D) + qt;
+#pragma unroll
+            for (int j = 0; j < kP; ++j) dst[rr][j] = __ldg(src + 4 * j);
         }
-        if (sgi + 1 == nseg) break;
-        inc = *reinterpret_cast<const float4 *>(incr + base + row);
-        __syncthreads();
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    const size_t row = (size_t)r0 * D + v0 + 4 * qt;   // this thread's results: two rows, four columns
+    auto at = [&](const float *x, int sgi, int rr) {
+        return reinterpret_cast<const float4 *>(x + ((size_t)bh * nseg + sgi) * D * D + row + rr * D);
+    };
+    float4 cur[2], inc[2];
+    auto put = [&](int sgi) {                          // entry state of segment sgi
 #pragma unroll
-        for (int j = 0; j < kHalf / 4; ++j) {
-            const float4 *sp = &Ss[sgi & 1][8 * j + 4 * hf];
-            const float mv[4] = {m[j].x, m[j].y, m[j].z, m[j].w};
+        for (int rr = 0; rr < 2; ++rr) {
+            *const_cast<float4 *>(at(start, sgi, rr)) = cur[rr];
+            ulonglong2 w;
+            w.x = pack2(cur[rr].x, cur[rr].y);
+            w.y = pack2(cur[rr].z, cur[rr].w);
+            Ss[sgi & 1][r0 + rr][(qt + (r0 >> 2)) & 3] = w;
+        }
+    };
+#pragma unroll
+    for (int rr = 0; rr < 2; ++rr) cur[rr] = *at(incr, 0, rr);
+    if (nseg > 2) fetch(1, m[1]);
+    auto step = [&](int sgi, float4 (&mm)[2][kP], float4 (&next)[2][kP]) {
+        put(sgi);
+#pragma unroll
+        for (int rr = 0; rr < 2; ++rr) inc[rr] = *at(incr, sgi, rr);
+        if (sgi + 2 < nseg) fetch(sgi + 1, next);
+        __syncthreads();
+        uint64_t acc[2][8];
+#pragma unroll
+        for (int rr = 0; rr < 2; ++rr)
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[rr][e] = 0;
+#pragma unroll
+        for (int j = 0; j < kP; ++j)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const float4 sv = sp[e];
-                acc.x = fmaf(mv[e], sv.x, acc.x); acc.y = fmaf(mv[e], sv.y, acc.y);
-                acc.z = fmaf(mv[e], sv.z, acc.z); acc.w = fmaf(mv[e], sv.w, acc.w);
+                const int k = 16 * j + 4 * qt + e;     // (k >> 2) & 3 = qt
+                uint64_t mv[2];
+#pragma unroll
+                for (int rr = 0; rr < 2; ++rr) {
+                    const float x = e == 0 ? mm[rr][j].x : e == 1 ? mm[rr][j].y : e == 2 ? mm[rr][j].z : mm[rr][j].w;
+                    mv[rr] = pack2(x, x);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const ulonglong2 sv = Ss[sgi & 1][k][(u + qt) & 3];
+#pragma unroll
+                    for (int rr = 0; rr < 2; ++rr) {
+                        acc[rr][2 * u] = fma2(mv[rr], sv.x, acc[rr][2 * u]);
+                        acc[rr][2 * u + 1] = fma2(mv[rr], sv.y, acc[rr][2 * u + 1]);
+                    }
+                }
             }
+        // sums over the four quarters; each lane keeps its four columns
+#pragma unroll
+        for (int rr = 0; rr < 2; ++rr) {
+            uint64_t h[4], o[2];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const uint64_t keep = qt & 2 ? acc[rr][4 + e] : acc[rr][e], give = qt & 2 ? acc[rr][e] : acc[rr][4 + e];
+                h[e] = add2(keep, __shfl_xor_sync(0xffffffffu, give, 2));
+            }
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const uint64_t keep = qt & 1 ? h[2 + e] : h[e], give = qt & 1 ? h[e] : h[2 + e];
+                o[e] = add2(keep, __shfl_xor_sync(0xffffffffu, give, 1));
+            }
+            const float2 a = unpack2(o[0]), b2 = unpack2(o[1]);
+            cur[rr] = make_float4(a.x + inc[rr].x, a.y + inc[rr].y, b2.x + inc[rr].z, b2.y + inc[rr].w);
         }
-        if (sgi + 2 < nseg) fetch(sgi + 1);
-        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 1);
-        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 1);
-        acc.z += __shfl_xor_sync(0xffffffffu, acc.z, 1);
-        acc.w += __shfl_xor_sync(0xffffffffu, acc.w, 1);
-        cur = make_float4(acc.x + inc.x, acc.y + inc.y, acc.z + inc.z, acc.w + inc.w);
+    };
+    for (int sgi = 1; sgi + 1 < nseg; sgi += 2) {
+        step(sgi, m[1], m[0]);
+        if (sgi + 2 < nseg) step(sgi + 1, m[0], m[1]);
     }
+#pragma unroll
+    for (int rr = 0; rr < 2; ++rr) *const_cast<float4 *>(at(start, nseg - 1, rr)) = cur[rr];
 }
 
 }  // namespace
 
-cudaError_t launch_scan_combine(const float *state_in, const ScanSegments &sg, Shape s, cudaStream_t st, bool pdl) {
+cudaError_t launch_scan_combine(const ScanSegments &sg, Shape s, cudaStream_t st, bool pdl) {
     dim3 grid(s.d / kCombCols, s.B * s.H);
     auto kernel = s.d == 128 ? scan_combine_kernel<128> : scan_combine_kernel<64>;
-    cudaError_t e = launch_kernel(kernel, grid, dim3(2 * s.d), 0, st, pdl, state_in, sg.incr, sg.trans, sg.start, sg.nseg);
+    cudaError_t e = launch_kernel(kernel, grid, dim3(2 * s.d), 0, st, pdl, sg.incr, sg.trans, sg.start, sg.nseg);
     if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
@@ -1038,7 +1083,7 @@ static cudaError_t scan_tc_impl(const GdnTcWs &ws, float scale_la, const float *
     cudaError_t e = allow_smem(kernel,
                                          ScanLayout<D>::kTotal);
     if (e != cudaSuccess) return e;
-    const int ctas = s.B * s.H * (sg.mode == 0 ? 1 : sg.nseg) * (sg.mode == 1 ? 2 : 1);
+    const int ctas = s.B * s.H * (sg.mode == 0 ? 1 : sg.mode == 1 ? 2 * sg.nseg - 3 : sg.nseg);
     count_launch();
     return launch_kernel(kernel, dim3(ctas), dim3(kScanThreads), ScanLayout<D>::kTotal, st, pdl, mwt, mqh, mkh, mph, ws.Ut,
                          ws.Gd, scale_la, state_in, state_out, (__half *)out.o_la16, out.o_la32, out.emit_flags, ex, sg,

@@ -97,7 +97,7 @@ cudaError_t launch_softmax_combine_tc(const void *q, const void *k_sm, const voi
                                       const int32_t *emit_flags, const float *w, float scale_sm,
                                       float eps, void *out, float *o_nla, float *lse, int32_t *sm_len, int len_cap,
                                       BlockRouting br, bool appending, int32_t *status, Shape s, cudaStream_t st,
-                                      HeadGroups hg = HeadGroups{});
+                                      HeadGroups hg = HeadGroups{}, int segs = 1, int seg_tiles = 0);
 // (sm_len [B,H] or nullptr: receives the retained tokens, at most len_cap; more are NATSL_ERR_CACHE_FULL)
 // (o_la16: the linear branch's read-out, o_laT [B,H,L/C,8,d,8] fp16; emit_flags: see ScanOut -- when given, the
 // kernel is launched as a programmatic dependent of the kernel before it in the stream, the scan)
@@ -178,13 +178,16 @@ cudaError_t launch_gdn_prepare_tc(const void *q, const void *k, const void *v, c
 // M_seg S0 + B_seg, and the same scan kernel yields both parts: B_seg as the exit state of a run
 // from S0 = 0, M_seg as the exit state of a run from S0 = I with U = 0.
 //   mode 0: one CTA per (batch, head) over all chunks (state_in / state_out as given);
-//   mode 1: two CTAs per (batch, head, segment), no outputs: B_seg -> incr, M_seg -> trans;
-//   mode 2: one CTA per (batch, head, segment) from the entry state in `start`, with outputs;
-//           the last segment writes state_out.
+//   mode 1: no outputs, one CTA per run that the chain needs, 2 nseg - 3 for each (batch, head): B_seg -> incr
+//           of every segment but the last -- the first one's run starts from state_in, so that its exit state is
+//           the second one's entry state --, M_seg -> trans of the segments between;
+//   mode 2: one CTA per (batch, head, segment) from the entry state in `start` (the first: state_in), with
+//           outputs; the last segment writes state_out.
 // incr, trans, start: [B*H, nseg, d, d] fp32.  Between modes 1 and 2 launch_scan_combine chains the
-// segments: start[0] = state_in (or 0), start[s+1] = M_s start[s] + B_s.
+// segments: start[1] = incr[0], start[s+1] = M_s start[s] + B_s.  The last segment, which mode 1 does not run,
+// takes the chunks that remain.
 struct ScanSegments {
-    int mode, nseg, ncs;       // ncs = chunks per segment
+    int mode, nseg, ncs;       // ncs = chunks per segment but the last
     float *incr, *trans, *start;
 };
 // Where the scan's read-out goes: o_la16 = o_laT [B,H,L/C,8,d,8] fp16 always (one transposed tile per
@@ -202,7 +205,7 @@ cudaError_t launch_gdn_scan_tc(const GdnTcWs &ws, float scale_la, const float *s
                                float *state_out, const ScanOut &out, const GdnTcExport &ex,
                                const ScanSegments &sg, const uint8_t *block_route, int32_t *status,
                                Shape s, cudaStream_t st, bool pdl = false);
-cudaError_t launch_scan_combine(const float *state_in, const ScanSegments &sg, Shape s, cudaStream_t st, bool pdl = false);
+cudaError_t launch_scan_combine(const ScanSegments &sg, Shape s, cudaStream_t st, bool pdl = false);
 
 // bwd_simt.cu -- fp32 CUDA-core backward
 // A batched matrix operand: element (r, c) of batch (b, h, chunk) is

@@ -133,7 +133,7 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                           const float *__restrict__ w,
                           float scale_sm, float eps, float norm_eps, int has_out, float *__restrict__ o_nla,
                           float *__restrict__ lse, int32_t *sm_len, int len_cap, int32_t *status, int L, int H,
-                          int wait_kcycles) {
+                          int wait_kcycles, int segs, int seg_tiles) {
     using SL = SmLayout<D>;
     constexpr int KB = SL::KB, kStages = SL::kStages, kLogits = SL::kLogits, kGroups = SL::kGroups;
     constexpr int kSoftmaxThreads = SL::kSoftmaxThreads, kAhead = kLogits - 1;
@@ -147,9 +147,11 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     constexpr int kMmaWarp = kSoftmaxThreads / 32, kTmaWarp = kMmaWarp + 1;
     const int NP = (L + kBM - 1) / kBM, NC = L / kC;
-    // grid = (B*H, NP).  Beside the scan: tiles in ascending order, all (batch, head) pairs of a tile
-    // before the next tile.  Otherwise: long rows first.
-    const int p = emit_flags ? (int)blockIdx.y : NP - 1 - (int)blockIdx.y;
+    // grid = (B*H, NP).  Beside the scan: in the order in which the scan finishes the query tiles -- ascending, a
+    // position of every one of its segments (segs of seg_tiles tiles each, the last one longer) before the next
+    // position -- and all (batch, head) pairs of a tile before the next tile.  Otherwise: long rows first.
+    int p = emit_flags ? (int)blockIdx.y : NP - 1 - (int)blockIdx.y;
+    if (emit_flags && p < segs * seg_tiles) p = (p % segs) * seg_tiles + p / segs;
     // blockIdx.x = (batch, linear head, softmax head of the group); H counts linear heads
     const int bhg = blockIdx.x, bh = bhg / kG, sg = bhg % kG, b = bh / H, h = bh % H;
     const int hq = h * kG + sg;                           // head index in the [B,L,H kG,D] view
@@ -787,7 +789,7 @@ static cudaError_t softmax_tc_impl(const void *q, const void *k_sm, const void *
                                    const void *o_la16, const int32_t *emit_flags, const float *w,
                                    float scale_sm, float eps, float norm_eps, void *out, float *o_nla, float *lse,
                                    int32_t *sm_len, int len_cap, BlockRouting br, bool appending, int32_t *status, Shape s,
-                                   cudaStream_t st) {
+                                   cudaStream_t st, int segs, int seg_tiles) {
     using SL = SmLayout<D>;
     CUtensorMap mq, mk, mv, mout, mkd, mvd;
     // q, out, k, v [B,L,H,G D] are read as [B,L,H G,D]; the compacted K/V rows keep all G D columns
@@ -823,7 +825,7 @@ static cudaError_t softmax_tc_impl(const void *q, const void *k_sm, const void *
     cfg.numAttrs = emit_flags ? 1 : 0;
     e = cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, mout, mkd, mvd, br.route, appending ? 1 : 0,
                            (int)cap, (int)capv, sm_idx, pre, (const __half *)o_la16, emit_flags, w, scale_sm, eps,
-                           norm_eps, out ? 1 : 0, o_nla, lse, sm_len, len_cap, status, s.L, s.H, debug_wait_kcycles());
+                           norm_eps, out ? 1 : 0, o_nla, lse, sm_len, len_cap, status, s.L, s.H, debug_wait_kcycles(), segs, seg_tiles);
     count_launch();
     return e;
 }
@@ -834,16 +836,19 @@ cudaError_t launch_softmax_combine_tc(const void *q, const void *k_sm, const voi
                                       const int32_t *emit_flags, const float *w, float scale_sm,
                                       float eps, void *out, float *o_nla, float *lse, int32_t *sm_len, int len_cap,
                                       BlockRouting br, bool appending, int32_t *status, Shape s, cudaStream_t st,
-                                      HeadGroups hg) {
+                                      HeadGroups hg, int segs, int seg_tiles) {
     if (hg.G == 2 && s.d == 128)
         return softmax_tc_impl<64, 2>(q, k_sm, v16, cap, capv, sm_idx, sm_chunk_prefix, o_la16, emit_flags,
-                                      w, scale_sm, eps, hg.norm_eps, out, o_nla, lse, sm_len, len_cap, br, appending, status, s, st);
+                                      w, scale_sm, eps, hg.norm_eps, out, o_nla, lse, sm_len, len_cap, br, appending, status, s, st, segs,
+                                         seg_tiles);
     if (hg.G > 1) return cudaErrorInvalidValue;
     if (s.d == 128)
         return softmax_tc_impl<128, 1>(q, k_sm, v16, cap, capv, sm_idx, sm_chunk_prefix, o_la16, emit_flags,
-                                       w, scale_sm, eps, hg.norm_eps, out, o_nla, lse, sm_len, len_cap, br, appending, status, s, st);
+                                       w, scale_sm, eps, hg.norm_eps, out, o_nla, lse, sm_len, len_cap, br, appending, status, s, st, segs,
+                                         seg_tiles);
     return softmax_tc_impl<64, 1>(q, k_sm, v16, cap, capv, sm_idx, sm_chunk_prefix, o_la16, emit_flags, w,
-                                  scale_sm, eps, hg.norm_eps, out, o_nla, lse, sm_len, len_cap, br, appending, status, s, st);
+                                  scale_sm, eps, hg.norm_eps, out, o_nla, lse, sm_len, len_cap, br, appending, status, s, st, segs,
+                                         seg_tiles);
 }
 
 template <int D>

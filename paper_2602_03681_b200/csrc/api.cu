@@ -645,9 +645,12 @@ int natsl_hybrid_bwd(const void *q, const void *k, const void *v, const float *g
     if (tensor_cores) {
         // Dependencies from here on: the query-side softmax kernel, the key-side one and the reverse scan need only
         // what is already there; the chunk kernel needs the reverse scan and, unless q and k are normalised, the
-        // query-side kernel's dq; the scatter of the retained tokens' dk, dv needs the key-side kernel.  Side
-        // stream: reverse scan, key-side kernel, scatter; caller's stream: query-side kernel, chunk kernel.
-        // Block-level routing: every token has a softmax-branch dk, dv (retained tokens: scattered from the
+        // query-side kernel's dq; the scatter of the retained tokens' dk, dv needs the key-side kernel.
+        // Token-level routing: query-side kernel, key-side kernel, scatter on the caller's stream (the key-side one
+        // starts in the query-side one's tail, on the multiprocessors the reverse scan leaves free), reverse scan and
+        // chunk kernel on the side stream.
+        // Block-level routing: reverse scan, key-side kernel, scatter on the side stream, the others on the caller's:
+        // every token has a softmax-branch dk, dv (retained tokens: scattered from the
         // compacted gradients; linear blocks: their own block's kernel, which needs the query-side one only), both
         // in fp32 token-major buffers that the chunk kernel adds (through the normalisation's Jacobian, where there is
         // one) and so waits for.
@@ -657,15 +660,15 @@ int natsl_hybrid_bwd(const void *q, const void *k, const void *v, const float *g
             side_join.forked(side, st);
         }
         NATSL_TRY(launch_gdn_rscan_tc(f.tc, f.gr, p->dstate_out, p->dstate_in, block_route, f.status, s, st0));
-        if (side) NATSL_TRY(cudaEventRecord(side->join, st0));
+        if (side && block) NATSL_TRY(cudaEventRecord(side->join, st0));
         // (normalised: the softmax branch's own fp16 copy of q goes where the forward had its gathered keys, which
         // nothing reads any more; the reverse scan beside it reads the linear operation's copy)
         void *q16 = normed ? f.k_smb : f.Qh;
         NATSL_TRY(launch_softmax_bwd_tc(q, q16, f.dO16, f.k16, f.v16, p->L, f.sm_idx, f.prefix, f.lse, f.Dsm,
                                         p->scale_sm, f.dq_sm, f.dk_sm, f.dv_sm, p->dscore ? f.dmask : nullptr, !normed,
-                                        f.status, s, st, st0, hg));
-        if (side) NATSL_TRY(cudaStreamWaitEvent(st, side->join, 0));     // the reverse scan has finished
+                                        f.status, s, st, block ? st0 : st, side && !block ? side->fork : nullptr, hg));
         if (block) {
+            if (side) NATSL_TRY(cudaStreamWaitEvent(st, side->join, 0));     // the reverse scan has finished
             NATSL_TRY(launch_gdn_finish(a, f.dk_x, f.dv_x, s32, st0, false));
             NATSL_TRY(launch_softmax_bwd_own_block(q, k, v, f.dO16, f.lse, f.Dsm, route, p->scale_sm, f.dq_sm, f.dk_x,
                                                    f.dv_x, gsc, s, st, hg));
@@ -680,11 +683,12 @@ int natsl_hybrid_bwd(const void *q, const void *k, const void *v, const float *g
         // Token-level routing.  With the normalisation a token's k has one gradient, of one copy or the other: they
         // stay in fp32 until its backward, a last kernel that rounds once.
         void *dq_o = normed ? f.dq32 : dq, *dk_o = normed ? f.dk32 : dk, *dv_o = normed ? f.dv32 : dv;
+        if (side && !normed) NATSL_TRY(cudaStreamWaitEvent(st0, side->fork, 0));      // dq_sm
         NATSL_TRY(launch_gdn_chunk_bwd(f.tc, f.ex, f.gr, q, k, v, beta, route, normed ? nullptr : f.dq_sm, p->scale_la,
-                                       dq_o, dk_o, dv_o, dg, dbeta, false, nullptr, nullptr, nullptr, f.status, s, st,
+                                       dq_o, dk_o, dv_o, dg, dbeta, false, nullptr, nullptr, nullptr, f.status, s, st0,
                                        hg));
         // the retained tokens' dk, dv (rows the chunk kernel does not write)
-        NATSL_TRY(launch_gdn_finish(a, dk_o, dv_o, normed ? s32 : s, st0, false));
+        NATSL_TRY(launch_gdn_finish(a, dk_o, dv_o, normed ? s32 : s, st, false));
         NATSL_TRY(side_join.join());
         if (normed)
             NATSL_TRY(launch_qk_norm_bwd_f32(q, k, true, route, f.dq32, f.dq_sm, f.dk32, f.dv32, dq, dk, dv,

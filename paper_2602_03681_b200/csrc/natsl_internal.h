@@ -135,7 +135,7 @@ cudaError_t launch_softmax_bwd_tc(const void *q, void *Qh, const void *dO16, con
                                   const int32_t *sm_chunk_prefix, const float *lse, const float *Dsm,
                                   float scale_sm, float *dq_sm, float *dk_sm, float *dv_sm,
                                   float *dmask, bool qh_ready, int32_t *status, Shape s, cudaStream_t st,
-                                  cudaStream_t st_kv,    // st: query-side kernel, st_kv: key-side kernel
+                                  cudaStream_t st_kv, cudaEvent_t after_dq,    // st: query-side kernel, st_kv: key-side kernel
                                   HeadGroups hg = HeadGroups{});
 // (hg.G = 2 at d = 128: softmax heads are column slices, lse / Dsm [B,H,G,L]; hg.norm_eps >= 0: Qh is
 // written here as the slice-wise RMS-normalised q, k16 must hold the normalised keys already)

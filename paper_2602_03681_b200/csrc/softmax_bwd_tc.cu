@@ -5,9 +5,9 @@
 //   dq_i = sum_j ds_ij k_j,   dk_j = sum_i ds_ij q_i           (D_i = <do_i, o_i>)
 // Two kernels, both recomputing p from the saved log-sum-exp:
 //   * query side: one CTA per 128 queries walks the compacted K/V in tiles of 64 keys
-//     (S = Q K^T and dP = dO V^T into TMEM, ds rows by one thread per query, dQ += dS K);
+//     (S = Q K^T and dP = dO V^T into TMEM, ds rows by two threads per query, dQ += dS K);
 //   * key side: one CTA per 128 retained keys walks the query tiles that can see them
-//     (S^T = K Q^T and dP^T = V dO^T, rows owned by one thread per key, dV += P^T dO, dK += dS^T Q).
+//     (S^T = K Q^T and dP^T = V dO^T, rows by two threads per key, dV += P^T dO, dK += dS^T Q).
 // Every operand is fp16 (q, k, v convert exactly; p, ds, do are computed values that need more
 // than bf16's 8 significant bits to keep the gradients within tolerance); accumulation is fp32.
 #include "common.cuh"
@@ -20,8 +20,13 @@ namespace {
 
 using namespace tc;
 
-constexpr int kThreadsB = 192;       // warps 0-3 rows, warp 4 MMA issue, warp 5 TMA
-constexpr int kRowsB = 128;
+// Two threads per row (query or key), 32 of a tile's 64 columns and half of the result's each: the chain from a tile's
+// logits to its operands and the epilogue are half as long as with one.  Measured at 64 columns and two CTAs per SM: 2000
+// cycles per tile of a CTA on the query side, 2900 on the key side, of which the MMAs (N = 64: 50 cycles each) take
+// 1200 and 1600; launch to first tile 4600, epilogue 4700 before its stores went through shared memory.
+constexpr int kRowsB = 256;          // row threads: warps 0-3 columns 0-31 of a tile, warps 4-7 columns 32-63
+constexpr int kMmaWarpB = 8, kTmaWarpB = 9;
+constexpr int kThreadsB = kRowsB + 64;
 constexpr int kMiscB = 2048;
 constexpr float kLog2e = 1.4426950408889634f;
 
@@ -29,10 +34,31 @@ struct MiscB {
     uint64_t barQ, full[3], empty[3], barS, barDP, barSfree, barP, barAcc;
     uint32_t tmem_base;
     int abort_flag, wait_kcycles;   // in this order: the waits read the limit as abort_flag[1]
-    uint32_t kept[kRowsB / 32];     // query side: which of the CTA's own tokens are retained
+    uint32_t kept[4];               // query side: which of the CTA's own tokens are retained
     alignas(16) float lse[3][64], dsum[3][64];   // key side: per query of the tile in a stage (copied with it)
 };
 static_assert(sizeof(MiscB) <= kMiscB, "misc page too small");
+
+// 32 fp32 columns of 32 rows, one row per lane (scaled by f), to global rows of `stride` floats; the first `rows` exist.
+// Through 4 KB of the warp's own shared memory, so that eight lanes write a row's 128 bytes: as 16-byte stores to 32
+// rows at once the query side's results took 4700 cycles of a CTA's 24000.
+__device__ __forceinline__ void store_rows32(uint8_t *buf, const uint32_t (&x)[32], float f, float *dst, size_t stride,
+                                             int rows, int lane) {
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+        *reinterpret_cast<float4 *>(buf + lane * 128 + ((c ^ (lane & 7)) << 4)) =
+            make_float4(f * __uint_as_float(x[4 * c]), f * __uint_as_float(x[4 * c + 1]), f * __uint_as_float(x[4 * c + 2]),
+                        f * __uint_as_float(x[4 * c + 3]));
+    __syncwarp();
+#pragma unroll
+    for (int it = 0; it < 8; ++it) {
+        const int row = 4 * it + (lane >> 3), c = lane & 7;
+        if (row < rows)
+            *reinterpret_cast<float4 *>(dst + row * stride + 4 * c) =
+                *reinterpret_cast<const float4 *>(buf + row * 128 + ((c ^ (row & 7)) << 4));
+    }
+}
 
 // ==========================================================================================
 // Query side
@@ -52,7 +78,7 @@ template <int D> struct QLayout {
 // columns of rows of kG D columns -- the x coordinate of every copy and the column offset of every
 // store --, the lists of retained tokens are the linear head's, lse and Dsm are [B,H,kG,L].
 template <int D, int kG>
-__global__ void __launch_bounds__(kThreadsB)
+__global__ void __launch_bounds__(kThreadsB, D == 64 ? 2 : 1)
 softmax_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh  [B*H*L][D] fp16, box 128
                          const __grid_constant__ CUtensorMap map_do,   // dO16 [B*H*L][D] fp16, box 128
                          const __grid_constant__ CUtensorMap map_k,    // k16 [B*H*cap][D], box 64
@@ -88,8 +114,8 @@ softmax_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh  [B
         ms.wait_kcycles = wait_kcycles;
         fence_mbar_init();
     }
-    if (tid < kRowsB / 32) ms.kept[tid] = 0u;
-    if (warp == 4) tmem_alloc(&ms.tmem_base, SL::kTmem);
+    if (tid < 4) ms.kept[tid] = 0u;
+    if (warp == kMmaWarpB) tmem_alloc(&ms.tmem_base, SL::kTmem);
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -97,7 +123,7 @@ softmax_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh  [B
     const uint32_t tS = tmem, tDP = tmem + 64, tDQ = tmem + 128;
     volatile int *abort_flag = &ms.abort_flag;
 
-    if (warp == 5) {
+    if (warp == kTmaWarpB) {
         if (lane == 0 && T > 0) {      // nothing is loaded for a tile that sees no retained key
             mbar_arrive_expect_tx(&ms.barQ, 2 * SL::kQ);
             for (int kb = 0; kb < KB; ++kb) {
@@ -120,7 +146,7 @@ softmax_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh  [B
                 mbar_wait_drain(&ms.full[u % SL::kStages], (u / SL::kStages) & 1);
             mbar_wait_drain(&ms.barQ, 0);
         }
-    } else if (warp == 4) {
+    } else if (warp == kMmaWarpB) {
         if (lane == 0 && T > 0) {
             constexpr uint32_t id_s = make_idesc(kFmtF16, 128, 64, false, false);
             constexpr uint32_t id_dq = make_idesc(kFmtF16, 128, D, false, true);
@@ -168,9 +194,9 @@ softmax_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh  [B
             }
         }
     } else {
-        const int r = tid, i_abs = p * 128 + r;
+        const int wq = warp & 3, half = warp >> 2, r = wq * 32 + lane, i_abs = p * 128 + r;
         const bool row_ok = i_abs < L;
-        const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
+        const uint32_t lane_base = (uint32_t)(wq * 32) << 16;
         const float sl2 = scale_sm * kLog2e;
         float lse2 = row_ok ? lse[(size_t)bhg * L + i_abs] * kLog2e : 0.f;
         if (lse2 == -INFINITY) lse2 = 0.f;                  // no key: every logit is masked below
@@ -178,42 +204,39 @@ softmax_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh  [B
         bool ok = true;
         // The compacted keys are in position order, so row i sees exactly the first `cnt` of them: all earlier ones
         // plus a population count of the CTA's own.
-        if (n_full + r < n_end) {
+        if (half == 0 && n_full + r < n_end) {
             const int rel = sm_idx[(size_t)bh * L + n_full + r] - p * 128;
             atomicOr(&ms.kept[(rel >> 5) & 3], 1u << (rel & 31));
         }
         named_barrier_sync(1, kRowsB);
-        int cnt = n_full + __popc(ms.kept[warp] & ((2u << lane) - 1u));
-        for (int e = 0; e < warp; ++e) cnt += __popc(ms.kept[e]);
+        int cnt = n_full + __popc(ms.kept[wq] & ((2u << lane) - 1u));
+        for (int e = 0; e < wq; ++e) cnt += __popc(ms.kept[e]);
         if (!row_ok) cnt = 0;
         const uint64_t sl22 = pack2(sl2, sl2), nl2 = pack2(-lse2, -lse2), sm2 = pack2(scale_sm, scale_sm);
         for (int t = 0; t < T; ++t) {
             ok = mbar_wait(&ms.barS, t & 1, abort_flag);
             if (!ok) break;
             tc_fence_after_sync();
-            uint32_t dk[32];                                // ds as packed fp16 pairs
-            const int vis = cnt - t * 64;                   // keys of the tile this row sees
-            const bool all_vis = __all_sync(0xffffffffu, vis >= 64);
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
+            uint32_t dk[16];                                // ds as packed fp16 pairs
+            const int vis = cnt - t * 64 - 32 * half;       // keys of this thread's 32 that the row sees
+            const bool all_vis = __all_sync(0xffffffffu, vis >= 32);
+            {
                 uint32_t sv[32], dv[32];
                 tmem_ld32(tS + lane_base + 32 * half, sv);
                 tmem_ld32(tDP + lane_base + 32 * half, dv);
                 tmem_wait_ld();
-                if (half == 1) {                            // both halves are in registers
-                    tc_fence_before_sync();
-                    mbar_arrive(&ms.barSfree);
-                }
+                tc_fence_before_sync();
+                mbar_arrive(&ms.barSfree);
                 if (!all_vis) {                             // mask the logit (exp2(-inf) = 0): no branch per element
 #pragma unroll
-                    for (int c = 0; c < 32; ++c) sv[c] = 32 * half + c < vis ? sv[c] : 0xff800000u;
+                    for (int c = 0; c < 32; ++c) sv[c] = c < vis ? sv[c] : 0xff800000u;
                 }
 #pragma unroll
                 for (int c = 0; c < 32; c += 2) {
                     const float2 e = unpack2(fma2(pack2(__uint_as_float(sv[c]), __uint_as_float(sv[c + 1])), sl22, nl2));
                     const uint64_t pr = mul2(pack2(ex2_ftz(e.x), ex2_ftz(e.y)), sm2);
                     const float2 ds = unpack2(mul2(pr, pack2(__uint_as_float(dv[c]) - Di, __uint_as_float(dv[c + 1]) - Di)));
-                    dk[16 * half + (c >> 1)] = pack_half2(ds.x, ds.y);
+                    dk[c >> 1] = pack_half2(ds.x, ds.y);
                 }
             }
             if (t > 0) {
@@ -221,8 +244,8 @@ softmax_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh  [B
                 if (!ok) break;
             }
 #pragma unroll
-            for (int pc = 0; pc < 8; ++pc)
-                *reinterpret_cast<uint4 *>(smem + SL::oDS + sw128_offset(r, pc)) = make_uint4(dk[4 * pc], dk[4 * pc + 1], dk[4 * pc + 2], dk[4 * pc + 3]);
+            for (int pc = 0; pc < 4; ++pc)
+                *reinterpret_cast<uint4 *>(smem + SL::oDS + sw128_offset(r, 4 * half + pc)) = make_uint4(dk[4 * pc], dk[4 * pc + 1], dk[4 * pc + 2], dk[4 * pc + 3]);
             fence_proxy_async_smem();
             tc_fence_before_sync();
             mbar_arrive(&ms.barP);
@@ -233,26 +256,25 @@ softmax_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh  [B
         }
         if (ok) {
             const float gi = grad_scale(status).y;          // dO and Dsm arrive times the gradient scale
-            float4 *dst = reinterpret_cast<float4 *>(dq_sm + (((size_t)b * L + i_abs) * H + h) * (D * kG) + x0);
+            float *dst = dq_sm + (((size_t)b * L + p * 128 + wq * 32) * H + h) * (D * kG) + x0;
 #pragma unroll
-            for (int cb = 0; cb < D / 32; ++cb) {
+            for (int cbi = 0; cbi < D / 64; ++cbi) {
+                const int cb = half * (D / 64) + cbi;
                 uint32_t x[32];
+#pragma unroll
+                for (int c = 0; c < 32; ++c) x[c] = 0u;
                 if (T > 0) {
                     tmem_ld32(tDQ + lane_base + cb * 32, x);
                     tmem_wait_ld();
                 }
-                if (!row_ok) continue;
-#pragma unroll
-                for (int c4 = 0; c4 < 8; ++c4)
-                    dst[cb * 8 + c4] = T > 0 ? make_float4(gi * __uint_as_float(x[4 * c4]), gi * __uint_as_float(x[4 * c4 + 1]),
-                                                           gi * __uint_as_float(x[4 * c4 + 2]), gi * __uint_as_float(x[4 * c4 + 3]))
-                                             : make_float4(0.f, 0.f, 0.f, 0.f);
+                // (the Q and dO tiles have been read)
+                store_rows32(smem + warp * 4096, x, gi, dst + cb * 32, (size_t)H * (D * kG), L - p * 128 - wq * 32, lane);
             }
         }
     }
     tc_fence_before_sync();
     __syncthreads();
-    if (warp == 4) {
+    if (warp == kMmaWarpB) {
         tc_fence_after_sync();
         tmem_dealloc(tmem, SL::kTmem);
     }
@@ -321,7 +343,7 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
         ms.wait_kcycles = wait_kcycles;
         fence_mbar_init();
     }
-    if (warp == 4) tmem_alloc(&ms.tmem_base, SL::kTmem);
+    if (warp == kMmaWarpB) tmem_alloc(&ms.tmem_base, SL::kTmem);
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -329,7 +351,7 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
     const uint32_t tS = tmem, tDP = tmem + 64, tDV = tmem + 128, tDK = tmem + 128 + D;
     volatile int *abort_flag = &ms.abort_flag;
 
-    if (warp == 5) {
+    if (warp == kTmaWarpB) {
         if (lane == 0) {
             mbar_arrive_expect_tx(&ms.barQ, 2 * SL::kKV);
             for (int kb = 0; kb < KB; ++kb) {
@@ -354,7 +376,7 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
                 mbar_wait_drain(&ms.full[u % SL::kStages], (u / SL::kStages) & 1);
             mbar_wait_drain(&ms.barQ, 0);
         }
-    } else if (warp == 4) {
+    } else if (warp == kMmaWarpB) {
         if (lane == 0) {
             constexpr uint32_t id_s = make_idesc(kFmtF16, 128, 64, false, false);
             constexpr uint32_t id_acc = make_idesc(kFmtF16, 128, D, false, true);
@@ -393,7 +415,7 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
                 for (int k16 = 0; k16 < 4; ++k16) {
                     mma_ss(tDV, desc_kmajor(aP + k16 * 32), desc_mnmajor(aDO + k16 * 2048, 8192), id_acc,
                            (t | k16) != 0);
-                    mma_ts(tDK, tDP + k16 * 8, desc_mnmajor(aQ + k16 * 2048, 8192), id_acc, (t | k16) != 0);
+                    mma_ts(tDK, tDP + (k16 >> 1) * 32 + (k16 & 1) * 8, desc_mnmajor(aQ + k16 * 2048, 8192), id_acc, (t | k16) != 0);
                 }
                 mma_commit(&ms.barAcc);
                 mma_commit(&ms.empty[t % SL::kStages]);
@@ -401,20 +423,20 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
             }
         }
     } else {
-        const int r = tid, j = kt * 128 + r;              // this thread's retained key
+        const int wq = warp & 3, half = warp >> 2, r = wq * 32 + lane, j = kt * 128 + r;    // this thread's retained key
         const bool key_ok = j < n_sm;
         const int pos_j = key_ok ? sm_idx[(size_t)bh * L + j] : 0x7fffffff;
-        const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
+        const uint32_t lane_base = (uint32_t)(wq * 32) << 16;
         const float sl2 = scale_sm * kLog2e;
         float msum = 0.f;                                   // mask gradient of this key, over all queries
         bool ok = true;
         for (int t = 0; t < T; ++t) {
-            const int i0 = (qt0 + t) * 64;
+            const int i0 = (qt0 + t) * 64 + 32 * half;      // this thread's 32 queries
             // per-query log-sum-exp and D of this tile, copied with the stage (the logits were formed from it, so it
             // is full; released below)
             const int sg = t % SL::kStages;
-            float *lse_t = ms.lse[sg];
-            const float *dsum = ms.dsum[sg];
+            float *lse_t = ms.lse[sg] + 32 * half;
+            const float *dsum = ms.dsum[sg] + 32 * half;
             ok = mbar_wait(&ms.full[sg], (t / SL::kStages) & 1, abort_flag) && mbar_wait(&ms.barS, t & 1, abort_flag);
             if (!ok) break;
             tc_fence_after_sync();
@@ -423,21 +445,19 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
             const bool all_vis = __all_sync(0xffffffffu, vis <= 0);
             if (!all_vis) {     // a query without any key has lse = -inf, which must not meet a masked logit's -inf
                 if (lse_t[lane] == -INFINITY) lse_t[lane] = 0.f;
-                if (lse_t[lane + 32] == -INFINITY) lse_t[lane + 32] = 0.f;
                 __syncwarp();
             }
-            float x[64];                                    // logits, then probabilities
-            tmem_ld32(tS + lane_base, reinterpret_cast<uint32_t (&)[32]>(x[0]));
-            tmem_ld32(tS + lane_base + 32, reinterpret_cast<uint32_t (&)[32]>(x[32]));
+            float x[32];                                    // logits, then probabilities
+            tmem_ld32(tS + lane_base + 32 * half, reinterpret_cast<uint32_t (&)[32]>(x[0]));
             tmem_wait_ld();
             tc_fence_before_sync();
             mbar_arrive(&ms.barSfree);
             if (!all_vis) {                                 // mask the logit (exp2(-inf) = 0): no branch per element
 #pragma unroll
-                for (int c = 0; c < 64; ++c) x[c] = vis <= c ? x[c] : -INFINITY;
+                for (int c = 0; c < 32; ++c) x[c] = vis <= c ? x[c] : -INFINITY;
             }
 #pragma unroll
-            for (int c = 0; c < 64; c += 2) {
+            for (int c = 0; c < 32; c += 2) {
                 const uint64_t l2 = *reinterpret_cast<const uint64_t *>(&lse_t[c]);
                 const float2 e = unpack2(fma2(pack2(x[c], x[c + 1]), sl22, mul2(l2, nl2)));
                 x[c] = ex2_ftz(e.x);
@@ -448,30 +468,28 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
             if (!ok) break;
             tc_fence_after_sync();
 #pragma unroll
-            for (int pc = 0; pc < 8; ++pc)
-                *reinterpret_cast<uint4 *>(smem + SL::oP + sw128_offset(r, pc)) =
+            for (int pc = 0; pc < 4; ++pc)
+                *reinterpret_cast<uint4 *>(smem + SL::oP + sw128_offset(r, 4 * half + pc)) =
                     make_uint4(pack_half2(x[8 * pc], x[8 * pc + 1]), pack_half2(x[8 * pc + 2], x[8 * pc + 3]),
                                pack_half2(x[8 * pc + 4], x[8 * pc + 5]), pack_half2(x[8 * pc + 6], x[8 * pc + 7]));
-            uint32_t dk[32];
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
+            uint32_t dk[16];
+            {
                 uint32_t dv[32];
                 tmem_ld32(tDP + lane_base + 32 * half, dv);
                 tmem_wait_ld();
 #pragma unroll
                 for (int c = 0; c < 32; c += 2) {
-                    const int cc = 32 * half + c;
-                    const float2 d2 = *reinterpret_cast<const float2 *>(&dsum[cc]);
-                    const uint64_t dm = mul2(pack2(x[cc], x[cc + 1]), pack2(__uint_as_float(dv[c]) - d2.x, __uint_as_float(dv[c + 1]) - d2.y));
+                    const float2 d2 = *reinterpret_cast<const float2 *>(&dsum[c]);
+                    const uint64_t dm = mul2(pack2(x[c], x[c + 1]), pack2(__uint_as_float(dv[c]) - d2.x, __uint_as_float(dv[c + 1]) - d2.y));
                     if (kMask) {                            // dM_ij (Section 4.2)
                         const float2 m = unpack2(dm);
                         msum += m.x + m.y;
                     }
                     const float2 ds = unpack2(mul2(dm, sm2));
-                    dk[cc >> 1] = pack_half2(ds.x, ds.y);
+                    dk[c >> 1] = pack_half2(ds.x, ds.y);
                 }
             }
-            tmem_st32(tDP + lane_base, dk);                 // dS^T over this thread's own dP^T
+            tmem_st16(tDP + lane_base + 32 * half, dk);     // dS^T over this thread's own dP^T
             tmem_wait_st();
             fence_proxy_async_smem();
             tc_fence_before_sync();
@@ -482,31 +500,31 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
             ok = mbar_wait(&ms.barAcc, (T - 1) & 1, abort_flag);
             tc_fence_after_sync();
         }
+        if (kMask) {
+            if (half == 1) (&ms.lse[0][0])[r] = msum;       // (every row thread is past its last tile)
+            named_barrier_sync(1, kRowsB);
+        }
         if (ok) {      // the TMEM loads are warp-wide: only the stores depend on the key being real
-            float4 *dv_dst = reinterpret_cast<float4 *>(dv_sm + ((size_t)bh * cap + j) * (D * kG) + x0);
-            float4 *dk_dst = reinterpret_cast<float4 *>(dk_sm + ((size_t)bh * cap + j) * (D * kG) + x0);
             const float gi = grad_scale(status).y;          // dO and Dsm arrive times the gradient scale
-            if (kMask && key_ok) dmask[(size_t)bhg * cap + j] = gi * msum;
+            if (kMask && half == 0 && key_ok) dmask[(size_t)bhg * cap + j] = gi * (msum + (&ms.lse[0][0])[r]);
 #pragma unroll
-            for (int cb = 0; cb < D / 32; ++cb) {
-                uint32_t x[32], y[32];
+            for (int cbi = 0; cbi < D / 64; ++cbi) {
+                const int cb = half * (D / 64) + cbi;
+                const size_t at = ((size_t)bh * cap + kt * 128 + wq * 32) * (D * kG) + x0 + cb * 32;
+                const int rows = n_sm - kt * 128 - wq * 32;
+                uint32_t x[32];
                 tmem_ld32(tDV + lane_base + cb * 32, x);
-                tmem_ld32(tDK + lane_base + cb * 32, y);
                 tmem_wait_ld();
-                if (!key_ok) continue;
-#pragma unroll
-                for (int c4 = 0; c4 < 8; ++c4) {
-                    dv_dst[cb * 8 + c4] = make_float4(gi * __uint_as_float(x[4 * c4]), gi * __uint_as_float(x[4 * c4 + 1]),
-                                                      gi * __uint_as_float(x[4 * c4 + 2]), gi * __uint_as_float(x[4 * c4 + 3]));
-                    dk_dst[cb * 8 + c4] = make_float4(gi * __uint_as_float(y[4 * c4]), gi * __uint_as_float(y[4 * c4 + 1]),
-                                                      gi * __uint_as_float(y[4 * c4 + 2]), gi * __uint_as_float(y[4 * c4 + 3]));
-                }
+                store_rows32(smem + warp * 4096, x, gi, dv_sm + at, D * kG, rows, lane);   // (K and V have been read)
+                tmem_ld32(tDK + lane_base + cb * 32, x);
+                tmem_wait_ld();
+                store_rows32(smem + warp * 4096, x, gi, dk_sm + at, D * kG, rows, lane);
             }
         }
     }
     tc_fence_before_sync();
     __syncthreads();
-    if (warp == 4) {
+    if (warp == kMmaWarpB) {
         tc_fence_after_sync();
         tmem_dealloc(tmem, SL::kTmem);
     }

@@ -76,6 +76,10 @@ template <int D> struct SmLayout {
     static constexpr int oV = oK + kStages * kKStage;
     static constexpr int oMisc = oV + kStages * kVStage;
     static constexpr int kTotal = oMisc + kMiscBytes;
+    // 4 KB per softmax warp through which o_nla leaves, when it is asked for: the K ring at 128 columns; at 64, where
+    // the ring holds o_laT tiles, behind everything else.
+    static constexpr int oRows = D == 128 ? oK : kTotal, kRows = D == 128 ? 0 : kSoftmaxThreads * 128;
+    static_assert(D == 64 || kStages * kKStage >= kSoftmaxThreads * 128, "rows do not fit the K ring");
 };
 
 struct Misc {                    // lives in the last kMiscBytes of the CTA's shared memory
@@ -581,8 +585,6 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
             // mean square of the normalised row = inv^2 * mean square of the accumulator row
             const float wn = wv.x * rsqrtf(inv * inv * ssn / D + eps) * inv;          // applies to the raw accumulator
             const float wl = wv.y * rsqrtf(ssl / DL + eps);
-            float *onla_row =
-                o_nla && i_abs < L ? o_nla + (((size_t)b * L + i_abs) * H + h) * DL + sg * D + wg * HC : nullptr;
 #pragma unroll 1
             for (int cb = 0; cb < HC / 32; ++cb) {
                 uint32_t ov[32];
@@ -602,12 +604,15 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                             make_uint4(pack_bf162(y[0], y[1]), pack_bf162(y[2], y[3]), pack_bf162(y[4], y[5]),
                                        pack_bf162(y[6], y[7]));
                 }
-                if (onla_row) {         // the raw branch output (fp32), straight from the registers
-                    float4 *dst = reinterpret_cast<float4 *>(onla_row + cb * 32);
-#pragma unroll
-                    for (int e = 0; e < 8; ++e)
-                        dst[e] = make_float4(__uint_as_float(ov[4 * e]) * inv, __uint_as_float(ov[4 * e + 1]) * inv,
-                                             __uint_as_float(ov[4 * e + 2]) * inv, __uint_as_float(ov[4 * e + 3]) * inv);
+            }
+            if (o_nla) {                // the raw branch output (fp32); its own loop keeps the one above small
+                const int i_warp = p * kBM + 32 * (warp & 3);                           // the warp's first query
+                float *dst = o_nla + (((size_t)b * L + i_warp) * H + h) * DL + sg * D + wg * HC;
+#pragma unroll 1
+                for (int cb = 0; cb < HC / 32; ++cb) {
+                    uint32_t ov[32];
+                    load_o(cb, ov);
+                    store_rows32(smem + SL::oRows + warp * 4096, ov, inv, dst + cb * 32, (size_t)H * DL, L - i_warp, lane);
                 }
             }
             if (lse && wg == 0 && i_abs < L)
@@ -808,7 +813,7 @@ static cudaError_t softmax_tc_impl(const void *q, const void *k_sm, const void *
     if (norm_eps >= 0.f) kernel = softmax_combine_tc_kernel<D, false, G, true>;
     if (br.route) kernel = norm_eps >= 0.f ? softmax_combine_tc_kernel<D, true, G, true>
                                           : softmax_combine_tc_kernel<D, true, G, false>;
-    cudaError_t e = allow_smem(kernel, SL::kTotal);
+    cudaError_t e = allow_smem(kernel, SL::kTotal + SL::kRows);
     if (e != cudaSuccess) return e;
     // With emit_flags the kernel is launched as a programmatic dependent of the kernel before it in
     // the stream (the scan): it may start once all of the scan's CTAs are resident, and finds o_la
@@ -816,7 +821,7 @@ static cudaError_t softmax_tc_impl(const void *q, const void *k_sm, const void *
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(s.B * s.H * G, (s.L + kBM - 1) / kBM);
     cfg.blockDim = dim3(SL::kThreads);
-    cfg.dynamicSmemBytes = SL::kTotal;
+    cfg.dynamicSmemBytes = SL::kTotal + (o_nla ? SL::kRows : 0);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -448,6 +448,27 @@ __device__ __forceinline__ uint32_t pack_bf162(float lo, float hi) {
     return *reinterpret_cast<uint32_t *>(&h);
 }
 
+// 32 fp32 columns of 32 rows, one row per lane (scaled by f), to global rows of `stride` floats; the first `rows` exist.
+// Through 4 KB of the warp's own shared memory, so that eight lanes write a row's 128 bytes: as 16-byte stores to 32
+// rows at once the results of the softmax backward's query side took 4700 cycles of a CTA's 24000.
+__device__ __forceinline__ void store_rows32(uint8_t *buf, const uint32_t (&x)[32], float f, float *dst, size_t stride,
+                                             int rows, int lane) {
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+        *reinterpret_cast<float4 *>(buf + lane * 128 + ((c ^ (lane & 7)) << 4)) =
+            make_float4(f * __uint_as_float(x[4 * c]), f * __uint_as_float(x[4 * c + 1]), f * __uint_as_float(x[4 * c + 2]),
+                        f * __uint_as_float(x[4 * c + 3]));
+    __syncwarp();
+#pragma unroll
+    for (int it = 0; it < 8; ++it) {
+        const int row = 4 * it + (lane >> 3), c = lane & 7;
+        if (row < rows)
+            *reinterpret_cast<float4 *>(dst + row * stride + 4 * c) =
+                *reinterpret_cast<const float4 *>(buf + row * 128 + ((c ^ (row & 7)) << 4));
+    }
+}
+
 }  // namespace tc
 
 // Host side: encoders of the TMA tensor maps (tc_host.cu).  All maps use a box whose inner extent

@@ -29,6 +29,7 @@
 // key is RMS-normalised per slice as it is read (its sum of squares rides along with the logit's
 // reduction), because normalised keys rounded to the cache's bf16 would cost 2.8e-2 of the branch output's
 // RMS.
+#include <algorithm>
 #include "common.cuh"
 #include "natsl_internal.h"
 #include "tc_common.cuh"
@@ -48,21 +49,31 @@ constexpr int kStateParts = 2;
 constexpr int kMaxParts = 16;
 constexpr int kCtasPerSm = 2, kResident = kCtasPerSm * 148;
 
-// Cache items per (sequence, head).  Few pairs: as many as keep every item resident at once.  More: the count
-// (of those that cut a cache finely enough) whose items fill the last round of persistent CTAs best.
-__host__ __device__ inline int decode_parts(size_t BH) {
-    if (BH * (1 + kStateParts) <= kResident) {
-        const int p = (int)(kResident / BH) - kStateParts;
-        return p > kMaxParts ? kMaxParts : p;
-    }
+// Cache items per (sequence, head), when every item is to be resident at once (0: not possible) ...
+inline int parts_resident(size_t BH) {
+    const int p = (int)(kResident / BH) - kStateParts;
+    return p > kMaxParts ? kMaxParts : (p > 0 ? p : 0);
+}
+// ... and when the CTAs go round: the count whose items fill the last round best, an item's start and merge counted as
+// 5 % of a round.
+inline int parts_persistent(size_t BH) {
     int best = 4;
     float least = 1e30f;
     for (int p = 4; p <= kMaxParts; ++p) {
         const float n = (float)BH * (p + kStateParts), per = n / kResident;
-        const float cost = (float)(int)(per + 0.999f) / per + 0.01f * p;
+        const float cost = (float)(int)(per + 0.999f) / per + 0.05f * p;
         if (cost < least) { least = cost; best = p; }
     }
     return best;
+}
+// Resident where it can be, unless that makes only one or two items of a cache that may hold more than 600 keys for each:
+// they then take much longer than the state items, and half of the CTAs wait for them.  (The host knows the cache's
+// capacity, not its length.)  Per step, resident -> persistent: 96 pairs of 1638 keys 26.3 -> 18.6 us, 90 pairs of the
+// normalised mode, 800 keys, 19.2 -> 14.9; 64 pairs of 1638 keys 16.3 -> 15.1; but 72 pairs of 800 keys 12.9 -> 13.9, 96 of
+// 200 8.6 -> 11.1.
+inline int decode_parts(size_t BH, int cap) {
+    const int p = parts_resident(BH);
+    return p > 2 || (p > 0 && cap <= 600 * p) ? p : parts_persistent(BH);
 }
 
 template <typename T> struct Vec16;   // 16 bytes of T as fp32 values
@@ -85,15 +96,13 @@ template <> struct Vec16<__nv_bfloat16> {
     }
 };
 
-// Workspace: [0,256) status word; then tickets [BH] i32; partials [BH][parts][D+8] f32 (m[G] in base-2 units
-// and z[G] in the first 8 with G <= 4, then acc[D]); o_la [BH][D] f32.
+// Workspace: [0,256) status word; then tickets [BH] i32; o_la [BH][D] f32; partials [BH][parts][D+8] f32 (m[G] in base-2
+// units and z[G] in the first 8 with G <= 4, then acc[D]).
 constexpr int kPartHead = 8;
 __host__ __device__ inline size_t dec_off_tickets() { return 256; }
-__host__ __device__ inline size_t dec_off_partials(size_t BH) {
-    return (256 + BH * 4 + 255) / 256 * 256;
-}
-__host__ __device__ inline size_t dec_off_ola(size_t BH, int D) {
-    return dec_off_partials(BH) + (BH * decode_parts(BH) * (D + kPartHead) * 4 + 255) / 256 * 256;
+__host__ __device__ inline size_t dec_off_ola(size_t BH) { return (256 + BH * 4 + 255) / 256 * 256; }
+__host__ __device__ inline size_t dec_off_partials(size_t BH, int D) {
+    return dec_off_ola(BH) + (BH * D * 4 + 255) / 256 * 256;
 }
 
 template <typename T, int D, int G> struct DecLayout {
@@ -212,8 +221,8 @@ decode_step_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__
         for (int item = blockIdx.x, i = 0; item < total; item += gridDim.x, ++i) {
             const int part = item % per_head, bh = item / per_head;
             int32_t *ticket = reinterpret_cast<int32_t *>(ws + dec_off_tickets()) + bh;
-            float *partials = reinterpret_cast<float *>(ws + dec_off_partials(BH)) + (size_t)bh * parts * kPs;
-            float *ola_ws = reinterpret_cast<float *>(ws + dec_off_ola(BH, D)) + (size_t)bh * D;
+            float *partials = reinterpret_cast<float *>(ws + dec_off_partials(BH, D)) + (size_t)bh * parts * kPs;
+            float *ola_ws = reinterpret_cast<float *>(ws + dec_off_ola(BH)) + (size_t)bh * D;
             const float *sc = slot_of(i & 1);
             // (after a time-out, which is reported, the tickets are still taken, so that they end at zero)
             const bool ok = mbar_wait(&done[i & 1], (i >> 1) & 1, abort_flag);
@@ -619,7 +628,8 @@ cudaError_t launch_decode_block_end(const uint8_t *route_block, const float *g_b
 }
 
 size_t decode_workspace_bytes(int B, int H, int d) {
-    return dec_off_ola((size_t)B * H, d) + ((size_t)B * H * d * 4 + 255) / 256 * 256;
+    const size_t BH = (size_t)B * H, parts = std::max(parts_resident(BH), parts_persistent(BH));
+    return dec_off_partials(BH, d) + (BH * parts * (d + kPartHead) * 4 + 255) / 256 * 256;
 }
 
 template <typename T, int D, int G, bool kNorm>
@@ -634,7 +644,7 @@ static cudaError_t decode_impl(const void *q, const void *k, const void *v, cons
         auto kernel = decode_step_kernel<T, D, G, kNorm>;
         cudaError_t e = allow_smem(kernel, DecLayout<T, D, G>::kTotal);
         if (e != cudaSuccess) return e;
-        const int BH = s.B * s.H, parts = decode_parts((size_t)BH), per_head = parts + kStateParts;
+        const int BH = s.B * s.H, parts = decode_parts((size_t)BH, cap), per_head = parts + kStateParts;
         // Persistent beyond one resident set; the stride then has no factor in common with the items per
         // pair, so that every CTA gets the same mix of cache and state items.
         auto gcd = [](int a, int b) { while (b) { const int c = a % b; a = b; b = c; } return a; };

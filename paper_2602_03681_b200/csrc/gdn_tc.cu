@@ -591,14 +591,22 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
     const int NC = L / kC;
     // Which (batch, head), which segment of its chunks, and which of the two segment runs (see
     // ScanSegments): c below counts the chunks of the segment, c0 + c is the chunk's index.
-    const int runs = sg.mode == 0 ? 1 : sg.mode == 1 ? 2 * sg.nseg - 3 : sg.nseg;     // CTAs per (batch, head)
-    const int bh = blockIdx.x / runs, run = blockIdx.x % runs, b = bh / H, h = bh % H;
-    const int var = sg.mode == 1 && run >= sg.nseg - 1 ? 1 : 0;
-    const int seg = var ? run - (sg.nseg - 2) : run;                                  // (mode 0: 0)
-    const int slot = bh * sg.nseg + seg;
-    const int c0 = seg * sg.ncs;
-    const int ncs = sg.mode == 0 ? NC : seg == sg.nseg - 1 ? NC - c0 : sg.ncs;
-    const bool emit_out = sg.mode != 1, zero_u = sg.mode == 1 && var == 1;
+    // (Everything of it is the same for all threads; little of it stays alive, for the row threads have no registers to
+    // spare: with a few words spilled a call of five chunks took 3 us longer.)
+    int bh = blockIdx.x, slot = blockIdx.x, c0 = 0, ncs = NC;
+    bool var = false;
+    if (sg.mode != 0) {
+        const int runs = sg.mode == 1 ? 2 * sg.nseg - 3 : sg.nseg;                    // CTAs per (batch, head)
+        bh = blockIdx.x / runs;
+        const int run = blockIdx.x - bh * runs;
+        var = sg.mode == 1 && run >= sg.nseg - 1;
+        const int seg = var ? run - (sg.nseg - 2) : run;
+        slot = bh * sg.nseg + seg;
+        c0 = seg * sg.ncs;
+        ncs = seg == sg.nseg - 1 ? NC - c0 : sg.ncs;
+    }
+    const int b = bh / H, h = bh - b * H;
+    const bool emit_out = sg.mode != 1, zero_u = var;
 
     if ((smem_u32(smem) & 1023u) != 0) {
         if (tid == 0) atomicMin(status, (int)NATSL_ERR_CUDA);
@@ -731,13 +739,17 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
         const int col0 = half * kHalfCols;                // this thread's state columns (key dim)
         const int tk0 = half * 32;                        // ... and its tokens of every chunk
         float S[kHalfCols];                               // fp32 state at the entry of the current chunk
+        const float *s_in = zero_u                    ? nullptr
+                            : c0 == 0 && state_in     ? state_in + (size_t)bh * D * D
+                            : c0 > 0 && sg.mode == 2  ? sg.start + (size_t)slot * D * D
+                                                      : nullptr;
+        if (s_in && active) {
 #pragma unroll
-        for (int x = 0; x < kHalfCols; ++x)
-            S[x] = !active ? 0.f
-                   : var          ? (col0 + x == r ? 1.f : 0.f)
-                   : seg > 0      ? (sg.mode == 2 ? sg.start[((size_t)slot * D + col0 + x) * D + r] : 0.f)
-                   : state_in     ? state_in[((size_t)bh * D + col0 + x) * D + r]
-                                  : 0.f;
+            for (int x = 0; x < kHalfCols; ++x) S[x] = s_in[(size_t)(col0 + x) * D + r];
+        } else {
+#pragma unroll
+            for (int x = 0; x < kHalfCols; ++x) S[x] = zero_u && active && col0 + x == r ? 1.f : 0.f;
+        }
         // This thread's 8 pieces (4 tokens each) of row r of U^T of chunk c.
         auto u_src = [&](int c) {
             return reinterpret_cast<const float4 *>(Ut + ((size_t)bh * NC + c0 + c) * D * 64) + (tk0 / 4) * D + r;
@@ -898,9 +910,9 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
         }
         if (ok && emit_out) ok = emit(ncs - 1);
         // where the state after the segment's last chunk goes
-        float *final_state = sg.mode == 1 ? (var ? sg.trans : sg.incr) + (size_t)slot * D * D
-                             : state_out && (sg.mode == 0 || seg == sg.nseg - 1) ? state_out + (size_t)bh * D * D
-                                                                                   : nullptr;
+        float *final_state = sg.mode == 1 ? (zero_u ? sg.trans : sg.incr) + (size_t)slot * D * D
+                             : state_out && c0 + ncs == NC ? state_out + (size_t)bh * D * D
+                                                           : nullptr;
         if (ok && final_state) {
             ok = mbar_wait(&ms.barSU, (ncs - 1) & 1, abort_flag);
             if (ok) {

@@ -55,11 +55,13 @@ inline int parts_resident(size_t BH) {
     return p > kMaxParts ? kMaxParts : (p > 0 ? p : 0);
 }
 // ... and when the CTAs go round: the count whose items fill the last round best, an item's start and merge counted as
-// 5 % of a round.
-inline int parts_persistent(size_t BH) {
-    int best = 4;
+// 5 % of a round; from one item per 300 keys that the cache may hold (a round of nearly empty items takes 4 us: 504 pairs of
+// 100 keys 45 us a step with four items each), four at most.
+inline int parts_persistent(size_t BH, int cap) {
+    const int from = std::min(4, std::max(1, (cap + 299) / 300));
+    int best = from;
     float least = 1e30f;
-    for (int p = 4; p <= kMaxParts; ++p) {
+    for (int p = from; p <= kMaxParts; ++p) {
         const float n = (float)BH * (p + kStateParts), per = n / kResident;
         const float cost = (float)(int)(per + 0.999f) / per + 0.05f * p;
         if (cost < least) { least = cost; best = p; }
@@ -73,7 +75,7 @@ inline int parts_persistent(size_t BH) {
 // 200 8.6 -> 11.1.
 inline int decode_parts(size_t BH, int cap) {
     const int p = parts_resident(BH);
-    return p > 2 || (p > 0 && cap <= 600 * p) ? p : parts_persistent(BH);
+    return p > 2 || (p > 0 && cap <= 600 * p) ? p : parts_persistent(BH, cap);
 }
 
 template <typename T> struct Vec16;   // 16 bytes of T as fp32 values
@@ -628,8 +630,8 @@ cudaError_t launch_decode_block_end(const uint8_t *route_block, const float *g_b
 }
 
 size_t decode_workspace_bytes(int B, int H, int d) {
-    const size_t BH = (size_t)B * H, parts = std::max(parts_resident(BH), parts_persistent(BH));
-    return dec_off_partials(BH, d) + (BH * parts * (d + kPartHead) * 4 + 255) / 256 * 256;
+    const size_t BH = (size_t)B * H;
+    return dec_off_partials(BH, d) + (BH * kMaxParts * (d + kPartHead) * 4 + 255) / 256 * 256;
 }
 
 template <typename T, int D, int G, bool kNorm>

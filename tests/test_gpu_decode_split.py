@@ -40,3 +40,25 @@ def test_decode_ragged_caches(name, B, H):
     assert binding.natsl_device_status(ws) == 0
     assert np.array_equal(n.cpu().numpy(), o_n)
     assert rel_err(state.cpu().numpy(), o_state) <= 1e-4
+
+
+@pytest.mark.parametrize("B,H,cap", [(9, 11, 100), (9, 11, 301), (14, 7, 601), (8, 8, 1201), (20, 15, 64)])
+def test_decode_split_follows_the_capacity(B, H, cap):
+    """Capacities at which a pair's cache is cut differently: a step on caches of mixed lengths, against the oracle."""
+    from paper_2602_03681_b200 import binding
+    wl = inputs.WORKLOADS["cfg3_bf16_decode"]
+    x = inputs.make_decode_inputs(wl, B=B, H=H, steps=1, ctx_retained=cap - 1, cap=cap)
+    x["cache_len"][...] = np.resize(np.array([0, 1, cap // 3, cap // 2 + 1, cap - 1]), B * H).reshape(B, H)
+    dt = tdtype(wl)
+    state, kc, vc, n, w = dev(x["state"]), dev(x["k_cache"], dt), dev(x["v_cache"], dt), dev(x["cache_len"]), dev(x["w"][0])
+    p = binding.make_params(B, H, 0, wl.d, binding._dtype_code(kc), wl.scale_la, wl.scale_sm, w=w)
+    ws = binding.alloc_workspace(p, binding.OP_DECODE)
+    out = torch.empty((B, H, wl.d), dtype=dt, device="cuda")
+    binding.natsl_decode_step(dev(x["q"][0], dt), dev(x["k"][0], dt), dev(x["v"][0], dt), dev(x["g"][0]),
+                              dev(x["beta"][0]), dev(x["route"][0]), state, kc, vc, n, out, p, ws)
+    ref = oracle.decode_step(x["q"][0], x["k"][0], x["v"][0], x["g"][0], x["beta"][0], x["route"][0], x["w"][0],
+                             x["state"].astype(np.float64), x["k_cache"].astype(np.float64),
+                             x["v_cache"].astype(np.float64), x["cache_len"].copy(),
+                             scale_la=wl.scale_la, scale_sm=wl.scale_sm)
+    check_stored(out.float().cpu().numpy(), ref["out"], TOL[wl.dtype], wl.dtype, "step")
+    assert binding.natsl_device_status(ws) == 0

@@ -91,16 +91,19 @@ bool scan_follows_closely(const natsl_params *p) { return (long long)p->B * p->H
 // against 2.1 with outputs) gains more than it costs: there are as many segments as keep its 2 nseg - 3 runs per pair
 // in one wave, at least 4 chunks long (shorter ones gain less than their step of the chain), and at least three --
 // with two the two passes are as long as one over everything.  32 pairs: 3 segments, 16: 6, 4: 20.
-// The last segment takes what remains, about half as much again: the first pass does not run it, and in the second the
+// The two passes must save 8 chunks of the chain, which is what two more launches and the chaining take.
+// The last segment takes what remains, up to twice as much: the first pass does not run it, and in the second the
 // softmax kernel fills the other multiprocessors.  *chunks: of the others, even, so that they are whole query tiles.
 int scan_segments(const natsl_params *p, int *chunks = nullptr) {
     if (!use_tensor_cores(p) || (p->flags & NATSL_SINGLE_PASS_SCAN)) return 1;
     const int NC = p->L / kC, BH = p->B * p->H;
     if (BH > 32 || NC < 16) return 1;
     const int most = std::min((148 / BH + 3) / 2, 32);
-    const int n = std::max(4, ((2 * NC + 2 * most) / (2 * most + 1) + 1) & ~1);
+    const int n = std::max(4, ((NC + most) / (most + 1) + 1) & ~1);
     if (chunks) *chunks = n;
-    return NC / n >= 3 ? NC / n : 1;
+    const int nseg = std::min(most, NC / n);
+    const int last = NC - (nseg - 1) * n;      // (three quarters: the first pass's chunks against the second's)
+    return nseg >= 3 && 4 * (NC - last) - 3 * n >= 32 ? nseg : 1;
 }
 
 FwdWs carve_fwd(const natsl_params *p, void *ws) {

@@ -646,8 +646,8 @@ int natsl_hybrid_bwd(const void *q, const void *k, const void *v, const float *g
                    f.X3, f.X4, normed ? nullptr : f.dq_sm, f.dk_sm, f.dv_sm, f.gS, f.sm_idx, f.prefix, p->L,
                    p->scale_la, f.dGrow, f.kappa, dbeta, dg};
     if (tensor_cores) {
-        // Dependencies from here on: the query-side softmax kernel, the key-side one and the reverse scan need only
-        // what is already there; the chunk kernel needs the reverse scan and, unless q and k are normalised, the
+        // Dependencies from here on: the query-side softmax kernel, the key-side one (both with the normalisation:
+        // behind the softmax operation's copy of q) and the reverse scan need only what is already there; the chunk kernel needs the reverse scan and, unless q and k are normalised, the
         // query-side kernel's dq; the scatter of the retained tokens' dk, dv needs the key-side kernel.
         // Token-level routing: query-side kernel, key-side kernel, scatter on the caller's stream (the key-side one
         // starts in the query-side one's tail, on the multiprocessors the reverse scan leaves free), reverse scan and
@@ -664,11 +664,21 @@ int natsl_hybrid_bwd(const void *q, const void *k, const void *v, const float *g
         }
         NATSL_TRY(launch_gdn_rscan_tc(f.tc, f.gr, p->dstate_out, p->dstate_in, block_route, f.status, s, st0));
         if (side && block) NATSL_TRY(cudaEventRecord(side->join, st0));
-        // (normalised: the softmax branch's own fp16 copy of q goes where the forward had its gathered keys, which
-        // nothing reads any more; the reverse scan beside it reads the linear operation's copy)
-        void *q16 = normed ? f.k_smb : f.Qh;
-        NATSL_TRY(launch_softmax_bwd_tc(q, q16, f.dO16, f.k16, f.v16, p->L, f.sm_idx, f.prefix, f.lse, f.Dsm,
-                                        p->scale_sm, f.dq_sm, f.dk_sm, f.dv_sm, p->dscore ? f.dmask : nullptr, !normed,
+        // The fp16 copy of q that both softmax kernels read: the prepare kernel's, or, normalised, the softmax
+        // operation's own, which goes where the forward had its gathered keys (nothing reads them any more; the
+        // reverse scan beside it reads the linear operation's copy).  It is written on the caller's stream, so a
+        // key-side kernel on the side stream waits for it there.
+        const void *q16 = f.Qh;
+        if (normed) {
+            NATSL_TRY(launch_to_f16_bhld(q, f.k_smb, s, hg, st));
+            q16 = f.k_smb;
+            if (side && block) {
+                NATSL_TRY(cudaEventRecord(side->fork, st));
+                NATSL_TRY(cudaStreamWaitEvent(st0, side->fork, 0));
+            }
+        }
+        NATSL_TRY(launch_softmax_bwd_tc(q16, f.dO16, f.k16, f.v16, p->L, f.sm_idx, f.prefix, f.lse, f.Dsm,
+                                        p->scale_sm, f.dq_sm, f.dk_sm, f.dv_sm, p->dscore ? f.dmask : nullptr,
                                         f.status, s, st, block ? st0 : st, side && !block ? side->fork : nullptr, hg));
         if (block) {
             if (side) NATSL_TRY(cudaStreamWaitEvent(st, side->join, 0));     // the reverse scan has finished

@@ -127,18 +127,21 @@ int sm_count();   // multiprocessors of the current device (cached per device)
 // non-zero only after natsl_debug_set_wait_limit.  Every tensor-core kernel launch passes it on.
 int debug_wait_kcycles();
 
-// softmax_bwd_tc.cu -- tensor-core backward of the softmax branch (bf16 storage).  Qh is scratch
-// for the fp16 copy of q [B,H,L,d]; dO16 the fp16 branch-output gradient [B,H,L,d]; k16, v16 the
+// softmax_bwd_tc.cu -- tensor-core backward of the softmax branch (bf16 storage).  Qh is the softmax operation's
+// fp16 copy of q [B,H,L,d]; dO16 the fp16 branch-output gradient [B,H,L,d]; k16, v16 the
 // fp16 retained K/V [B,H,cap,d]; dq_sm is token-major [B,L,H,d], dk_sm / dv_sm compacted.
-cudaError_t launch_softmax_bwd_tc(const void *q, void *Qh, const void *dO16, const void *k16,
+// Both kernels read Qh: where st_kv is not st, the caller orders it behind what wrote Qh.
+// launch_to_f16_bhld: x [B,L,H,d] bf16 -> xh [B,H,L,d] fp16, slice-wise RMS-normalised with hg.norm_eps >= 0.
+cudaError_t launch_to_f16_bhld(const void *x, void *xh, Shape s, HeadGroups hg, cudaStream_t st);
+cudaError_t launch_softmax_bwd_tc(const void *Qh, const void *dO16, const void *k16,
                                   const void *v16, int cap, const int32_t *sm_idx,
                                   const int32_t *sm_chunk_prefix, const float *lse, const float *Dsm,
                                   float scale_sm, float *dq_sm, float *dk_sm, float *dv_sm,
-                                  float *dmask, bool qh_ready, int32_t *status, Shape s, cudaStream_t st,
+                                  float *dmask, int32_t *status, Shape s, cudaStream_t st,
                                   cudaStream_t st_kv, cudaEvent_t after_dq,    // st: query-side kernel, st_kv: key-side kernel
                                   HeadGroups hg = HeadGroups{});
-// (hg.G = 2 at d = 128: softmax heads are column slices, lse / Dsm [B,H,G,L]; hg.norm_eps >= 0: Qh is
-// written here as the slice-wise RMS-normalised q, k16 must hold the normalised keys already)
+// (hg.G = 2 at d = 128: softmax heads are column slices, lse / Dsm [B,H,G,L]; hg.norm_eps >= 0: Qh and k16 hold the
+// normalised rows)
 
 // gdn_tc.cu -- tensor-core chunkwise Gated DeltaNet (bf16 storage): intermediates in workspace
 struct GdnTcWs {

@@ -551,7 +551,7 @@ to_f16_bhld_kernel(const __nv_bfloat16 *__restrict__ q, __half *__restrict__ qh,
 
 }  // namespace
 
-static cudaError_t launch_to_f16_bhld(const void *x, void *xh, Shape s, HeadGroups hg, cudaStream_t st) {
+cudaError_t launch_to_f16_bhld(const void *x, void *xh, Shape s, HeadGroups hg, cudaStream_t st) {
     const size_t pieces = (size_t)s.B * s.L * s.H * (s.d / 8);
     auto kernel = s.d == 128 ? to_f16_bhld_kernel<128> : to_f16_bhld_kernel<64>;
     kernel<<<(unsigned)((pieces + 255) / 256), 256, 0, st>>>((const __nv_bfloat16 *)x, (__half *)xh, s.B, s.L, s.H, hg.G,
@@ -561,22 +561,15 @@ static cudaError_t launch_to_f16_bhld(const void *x, void *xh, Shape s, HeadGrou
 }
 
 template <int D, int G>      // D: columns of a softmax head, G of them per linear head (s.d = D G)
-static cudaError_t softmax_bwd_tc_impl(const void *q, void *Qh, const void *dO16, const void *k16,
+static cudaError_t softmax_bwd_tc_impl(const void *Qh, const void *dO16, const void *k16,
                                        const void *v16, int cap, const int32_t *sm_idx,
                                        const int32_t *pre, const float *lse, const float *Dsm,
                                        float scale_sm, float *dq_sm, float *dk_sm, float *dv_sm,
-                                       float *dmask, bool qh_ready, int32_t *status, Shape s,
-                                       cudaStream_t st, cudaStream_t st_kv, cudaEvent_t after_dq, float norm_eps) {
+                                       float *dmask, int32_t *status, Shape s,
+                                       cudaStream_t st, cudaStream_t st_kv, cudaEvent_t after_dq) {
     const uint64_t BH = (uint64_t)s.B * s.H;
     constexpr int DL = D * G;
     cudaError_t e;
-    if (!qh_ready) {      // (the linear branch's prepare kernel leaves the same fp16 copy of q behind --
-                          //  unless q is normalised, differently for the two operations)
-        HeadGroups hg;
-        hg.G = G;
-        hg.norm_eps = norm_eps;
-        if ((e = launch_to_f16_bhld(q, Qh, s, hg, st)) != cudaSuccess) return e;
-    }
     CUtensorMap mq128, mdo128, mk64, mv64, mq64, mdo64, mk128, mv128;
     if (!tch::make_map_2d(&mq128, Qh, BH * s.L, DL, 128) || !tch::make_map_2d(&mdo128, dO16, BH * s.L, DL, 128) ||
         !tch::make_map_2d(&mk64, k16, BH * cap, DL, 64) || !tch::make_map_2d(&mv64, v16, BH * cap, DL, 64) ||
@@ -601,22 +594,21 @@ static cudaError_t softmax_bwd_tc_impl(const void *q, void *Qh, const void *dO16
     return cudaGetLastError();
 }
 
-cudaError_t launch_softmax_bwd_tc(const void *q, void *Qh, const void *dO16, const void *k16,
+cudaError_t launch_softmax_bwd_tc(const void *Qh, const void *dO16, const void *k16,
                                   const void *v16, int cap, const int32_t *sm_idx,
                                   const int32_t *sm_chunk_prefix, const float *lse, const float *Dsm,
                                   float scale_sm, float *dq_sm, float *dk_sm, float *dv_sm,
-                                  float *dmask, bool qh_ready, int32_t *status, Shape s,
+                                  float *dmask, int32_t *status, Shape s,
                                   cudaStream_t st, cudaStream_t st_kv, cudaEvent_t after_dq, HeadGroups hg) {
-    if (hg.norm_eps >= 0.f && qh_ready) return cudaErrorInvalidValue;   // (the copy at hand is the linear operation's)
     if (hg.G == 2 && s.d == 128)
-        return softmax_bwd_tc_impl<64, 2>(q, Qh, dO16, k16, v16, cap, sm_idx, sm_chunk_prefix, lse, Dsm, scale_sm,
-                                          dq_sm, dk_sm, dv_sm, dmask, qh_ready, status, s, st, st_kv, after_dq, hg.norm_eps);
+        return softmax_bwd_tc_impl<64, 2>(Qh, dO16, k16, v16, cap, sm_idx, sm_chunk_prefix, lse, Dsm, scale_sm,
+                                          dq_sm, dk_sm, dv_sm, dmask, status, s, st, st_kv, after_dq);
     if (hg.G > 1) return cudaErrorInvalidValue;
     if (s.d == 128)
-        return softmax_bwd_tc_impl<128, 1>(q, Qh, dO16, k16, v16, cap, sm_idx, sm_chunk_prefix, lse, Dsm, scale_sm,
-                                           dq_sm, dk_sm, dv_sm, dmask, qh_ready, status, s, st, st_kv, after_dq, hg.norm_eps);
-    return softmax_bwd_tc_impl<64, 1>(q, Qh, dO16, k16, v16, cap, sm_idx, sm_chunk_prefix, lse, Dsm, scale_sm,
-                                      dq_sm, dk_sm, dv_sm, dmask, qh_ready, status, s, st, st_kv, after_dq, hg.norm_eps);
+        return softmax_bwd_tc_impl<128, 1>(Qh, dO16, k16, v16, cap, sm_idx, sm_chunk_prefix, lse, Dsm, scale_sm,
+                                           dq_sm, dk_sm, dv_sm, dmask, status, s, st, st_kv, after_dq);
+    return softmax_bwd_tc_impl<64, 1>(Qh, dO16, k16, v16, cap, sm_idx, sm_chunk_prefix, lse, Dsm, scale_sm,
+                                      dq_sm, dk_sm, dv_sm, dmask, status, s, st, st_kv, after_dq);
 }
 
 }  // namespace natsl

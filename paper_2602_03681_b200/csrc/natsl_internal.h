@@ -173,8 +173,9 @@ cudaError_t launch_gdn_prepare_tc(const void *q, const void *k, const void *v, c
                                   const GdnTcWs &ws, const GdnTcExport &ex, int32_t *status, Shape s,
                                   cudaStream_t st, int head_words, float norm_eps = -1.f);
 // (the forward's first kernel: clears head_words words of the status page)
-// pdl (here and elsewhere): launched as a programmatic dependent of the kernel before it in the stream.  Every kernel of
-// the forward waits for the one before it before it ends, so a kernel that has waited for its predecessor sees all of them.
+// pdl (here and elsewhere): launched as a programmatic dependent of the kernel before it in the stream.  Every kernel
+// launched so waits for the one before it (grid_dependency_wait) before it ends, at its start or, where it needs nothing
+// of it or hears of it otherwise, in a thread at its end: a kernel that has waited for its predecessor sees all of them.
 // Splitting the scan of one (batch, head) over several CTAs when there are few (batch, head)
 // pairs.  The state recurrence S <- (gamma_C I - K~^T W) S + K~^T U is affine in S with a factor
 // that acts on the key dimension only, so a segment of chunks maps its entry state S0 to

@@ -160,8 +160,17 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
     const int bhg = blockIdx.x, bh = bhg / kG, sg = bhg % kG, b = bh / H, h = bh % H;
     const int hq = h * kG + sg;                           // head index in the [B,L,H kG,D] view
 
+    // This grid starts before the scan has ended and takes from it what the counters cover, which the final state is
+    // not.  It must not end before the scan: a kernel that waits for this one -- a decode step launched as its
+    // programmatic dependent, or any kernel behind it in a captured graph -- takes it that everything ahead has ended.
+    // One thread of the query tile that the scan finishes last is enough.
+    auto end_behind_scan = [&]() {
+        if (tid == 0 && blockIdx.x == 0 && blockIdx.y == gridDim.y - 1) grid_dependency_wait();
+    };
+
     if ((smem_u32(smem) & 1023u) != 0) {              // operand tiles need 1024-byte alignment
         if (tid == 0) atomicMin(status, (int)NATSL_ERR_CUDA);
+        end_behind_scan();
         return;
     }
     // The TMA warp sets the barriers up and requests the Q tile before anything else, so that the tile travels
@@ -636,6 +645,7 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
         tmem_dealloc(tmem, 256);
     }
     if (tid == 0 && ms.abort_flag) atomicMin(status, (int)NATSL_ERR_TIMEOUT);
+    end_behind_scan();
 }
 
 // Route compaction and gather of the retained K/V in one kernel (the softmax branch's half of the forward's

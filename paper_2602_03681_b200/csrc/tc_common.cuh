@@ -93,7 +93,8 @@ __device__ __forceinline__ bool mbar_wait_drain(uint64_t *bar, uint32_t parity) 
 __device__ __forceinline__ void launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
-// ... and in the later kernel: everything before it in the stream has completed and is visible.
+// ... and in the later kernel: the kernel before it in the stream has completed and is visible -- and so is everything
+// ahead of that one, because every kernel that is launched as a programmatic dependent executes this before it ends.
 __device__ __forceinline__ void grid_dependency_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }

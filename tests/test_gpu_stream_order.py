@@ -1,5 +1,10 @@
 """Which kernels of a captured backward are ordered behind which: the edges of the graph, not the outcome of one run.
 (A missing edge between the two streams gives the right bits whenever the reader happens to start late enough.)"""
+import ctypes
+import glob
+import os
+import re
+
 import pytest
 import torch
 
@@ -18,7 +23,8 @@ TOKEN_NORMED = [("softmax_bwd_dkv", "scatter"), ("softmax_bwd_dq", "qk_norm_bwd"
 
 
 def kernels_and_paths(graph):
-    """{node: kernel name} and {node: every node ordered behind it} of a captured graph."""
+    """{node: kernel name}, {node: every node ordered behind it} and the nodes launched as programmatic dependents of a
+    captured graph."""
     from cuda.bindings import driver as cu
 
     def ok(res):
@@ -27,8 +33,13 @@ def kernels_and_paths(graph):
 
     g = cu.CUgraph(graph.raw_cuda_graph())
     nodes = ok(cu.cuGraphGetNodes(g, ok(cu.cuGraphGetNodes(g, 0))[1]))[0]
-    m = ok(cu.cuGraphGetEdges_v2(g, 0))[-1]
-    src, dst = ok(cu.cuGraphGetEdges_v2(g, m))[:2]
+    # (edges by ctypes: the binding returns edge data that it has freed)
+    get, m = ctypes.CDLL("libcuda.so.1").cuGraphGetEdges_v2, ctypes.c_size_t()
+    h = ctypes.c_void_p(graph.raw_cuda_graph())
+    assert get(h, None, None, None, ctypes.byref(m)) == 0
+    src, dst = (ctypes.c_void_p * m.value)(), (ctypes.c_void_p * m.value)()
+    data = (ctypes.c_ubyte * 8 * m.value)()                   # from_port, to_port, type, 5 reserved bytes
+    assert get(h, src, dst, data, ctypes.byref(m)) == 0
     names = {}
     for n in nodes:
         if ok(cu.cuGraphNodeGetType(n)) == cu.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
@@ -49,7 +60,24 @@ def kernels_and_paths(graph):
 
     for n in after:
         visit(n)
-    return names, reach
+    early = {int(b) for b, x in zip(dst, data) if x[2] == int(cu.CUgraphDependencyType.CU_GRAPH_DEPENDENCY_TYPE_PROGRAMMATIC)}
+    return names, reach, early
+
+
+def kernel_sources():
+    """{kernel name: its body} of the library's sources."""
+    found = {}
+    for path in glob.glob(os.path.join(os.path.dirname(os.path.dirname(__file__)), "paper_2602_03681_b200", "csrc", "*.cu")):
+        with open(path) as f:
+            text = f.read()
+        for m in re.finditer(r"__global__[^;{]*?\b(\w+_kernel)\(", text):
+            at = text.index("{", m.end())
+            depth, end = 1, at + 1
+            while depth:
+                depth += {"{": 1, "}": -1}.get(text[end], 0)
+                end += 1
+            found[m.group(1)] = text[at:end]
+    return found
 
 
 @pytest.mark.parametrize("d,G,norm,block", [(128, 2, True, True), (64, 1, True, True), (128, 1, False, True),
@@ -78,7 +106,7 @@ def test_every_reader_of_the_backward_is_ordered_behind_its_writer(d, G, norm, b
     graph = torch.cuda.CUDAGraph(keep_graph=True)
     with torch.cuda.graph(graph):
         step()
-    names, reach = kernels_and_paths(graph)
+    names, reach, _ = kernels_and_paths(graph)
     pairs = ALWAYS + (NORMED if norm else []) + (BLOCK if block else TOKEN_NORMED if norm else TOKEN)
     for a, b in pairs:
         at, to = ([n for n, name in names.items() if x in name] for x in (a, b))
@@ -86,3 +114,44 @@ def test_every_reader_of_the_backward_is_ordered_behind_its_writer(d, G, norm, b
         for x in at:
             for y in to:
                 assert y in reach[x], f"{names[y]} is not ordered behind {names[x]}"
+
+
+@pytest.mark.parametrize("dtype,B,H,L,d", [("bf16", 1, 2, 128, 128), ("bf16", 1, 2, 2048, 64), ("bf16", 4, 16, 1024, 64),
+                                           ("f32", 1, 2, 128, 64)])
+def test_a_programmatic_dependent_waits_for_its_predecessor(dtype, B, H, L, d):
+    """A forward and two decode steps: a kernel that may start before its predecessor has ended must wait for it before
+    it ends itself.  Otherwise whoever waits for that kernel -- the first decode step reads the forward's final state --
+    does not wait for the one ahead of it."""
+    from paper_2602_03681_b200 import binding
+    dt, code = (torch.bfloat16, binding.NATSL_BF16) if dtype == "bf16" else (torch.float32, binding.NATSL_F32)
+    t = {n: torch.randn((B, L, H, d), device="cuda").to(dt) for n in ("q", "k", "v", "out")}
+    g, beta = torch.zeros((B, L, H), device="cuda"), torch.zeros((B, L, H), device="cuda")
+    route = torch.zeros((B, L, H), dtype=torch.uint8, device="cuda")
+    route[:, ::7] = 1
+    kc, vc = (torch.zeros((B, H, L + 2, d), dtype=dt, device="cuda") for _ in range(2))
+    n, state = torch.zeros((B, H), dtype=torch.int32, device="cuda"), torch.zeros((B, H, d, d), device="cuda")
+    p = binding.make_params(B, H, L, d, code, d ** -0.5, 1.0, state_out=state, k_sm=kc, v_sm=vc, sm_len=n, sm_cap=L + 2)
+    pd = binding.make_params(B, H, 0, d, code, d ** -0.5, 1.0)
+    ws, wd = binding.alloc_workspace(p, binding.OP_FWD), binding.alloc_workspace(pd, binding.OP_DECODE)
+
+    def step():
+        binding.natsl_hybrid_fwd(t["q"], t["k"], t["v"], g, beta, route, t["out"], p, ws)
+        for i in range(2):
+            binding.natsl_decode_step(t["q"][:, i].contiguous(), t["k"][:, i].contiguous(), t["v"][:, i].contiguous(),
+                                      g[:, i].contiguous(), beta[:, i].contiguous(), route[:, i].contiguous(), state, kc,
+                                      vc, n, t["out"][:, i].contiguous(), pd, wd)
+
+    step()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        step()
+    names, _, early = kernels_and_paths(graph)
+    sources = kernel_sources()
+    seen = set()
+    for x in early:
+        own = [k for k in sources if f"{len(k)}{k}" in names[x]]
+        assert len(own) == 1, names[x]
+        assert "grid_dependency_wait()" in sources[own[0]], f"{own[0]} does not wait for the kernel before it"
+        seen.add(own[0])
+    assert seen >= ({"softmax_combine_tc_kernel", "route_gather_kernel"} if dtype == "bf16" else {"softmax_combine_simt_kernel"})

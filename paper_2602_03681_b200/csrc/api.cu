@@ -430,7 +430,7 @@ int natsl_score_layer(const void *x, const float *w_score, float *scores, uint8_
     // a row of X is read in 16-byte pieces
     const int per16 = p->dtype == NATSL_BF16 ? 8 : 4;
     // (the pooled rows of a CTA's two chunks and their scores live in shared memory)
-    if (d_model <= 0 || d_model % per16 != 0 || ((size_t)d_model + 2 * (size_t)p->H) * 8 > 200 * 1024)
+    if (d_model <= 0 || d_model % per16 != 0 || ((size_t)d_model + 2 * (size_t)p->H) * 8 > kScoreSmemMax)
         return NATSL_ERR_SHAPE;
     if (!aligned16(x) || !aligned16(w_score)) return NATSL_ERR_ALIGN;
     cudaError_t e = launch_score_layer(x, w_score, scores, route, d_model, shape_of(p),

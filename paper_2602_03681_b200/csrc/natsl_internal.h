@@ -101,8 +101,10 @@ cudaError_t launch_softmax_combine_tc(const void *q, const void *k_sm, const voi
 // (sm_len [B,H] or nullptr: receives the retained tokens, at most len_cap; more are NATSL_ERR_CACHE_FULL)
 // (o_la16: the linear branch's read-out, o_laT [B,H,L/C,8,d,8] fp16; emit_flags: see ScanOut -- when given, the
 // kernel is launched as a programmatic dependent of the kernel before it in the stream, the scan)
-// cudaFuncSetAttribute(max dynamic shared memory) of a kernel, once per thread, device and size: the call
-// itself costs a launch's host time about half a microsecond, and a forward would make five of them.
+// cudaFuncSetAttribute(max dynamic shared memory) of a kernel, once per thread and device: the call itself costs a
+// launch's host time about half a microsecond, and a forward would make five of them.  The limit belongs to the
+// function, what has been set is remembered per thread: every call for a kernel must therefore ask for the same bytes,
+// the most that any of its launches uses (a smaller request of another thread would lower the limit behind this one's back).
 cudaError_t allow_smem_of(const void *kernel, int bytes);
 template <typename K> cudaError_t allow_smem(K *kernel, size_t bytes) {
     return allow_smem_of(reinterpret_cast<const void *>(kernel), (int)bytes);
@@ -122,6 +124,8 @@ cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t sm
     cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
+// Shared memory of a score-layer CTA, at most: the pooled rows of its chunks and their scores.
+constexpr size_t kScoreSmemMax = 200 * 1024;
 int sm_count();   // multiprocessors of the current device (cached per device)
 // Bound of the device-side waits in units of 1024 cycles, 0 = the default (about two seconds);
 // non-zero only after natsl_debug_set_wait_limit.  Every tensor-core kernel launch passes it on.

@@ -113,7 +113,7 @@ cudaError_t score_layer_impl(const void *x, const float *w_score, float *scores,
                              int d_model, Shape s, cudaStream_t st) {
     dim3 grid((s.L / kC + kScoreChunks - 1) / kScoreChunks, s.B);
     const size_t smem = (size_t)kScoreChunks * ((size_t)d_model + 2 * s.H) * sizeof(float);
-    cudaError_t e = allow_smem(score_layer_kernel<T>, (int)smem);
+    cudaError_t e = allow_smem(score_layer_kernel<T>, kScoreSmemMax);
     if (e != cudaSuccess) return e;
     score_layer_kernel<T><<<grid, kScoreThreads, smem, st>>>((const T *)x, w_score, scores, route, s.L,
                                                              d_model, s.H);

@@ -73,7 +73,7 @@ bool make_map_blhd_f32(CUtensorMap *m, const void *base, int B, int L, int H, in
 }  // namespace tch
 
 cudaError_t allow_smem_of(const void *kernel, int bytes) {
-    struct Entry { const void *fn; int dev, bytes; };
+    struct Entry { const void *fn; int dev; };
     constexpr int kEntries = 128;                     // (the library has fewer kernels; a full table only re-sends)
     thread_local Entry table[kEntries] = {};
     int dev = 0;
@@ -83,15 +83,11 @@ cudaError_t allow_smem_of(const void *kernel, int bytes) {
     Entry *slot = nullptr;
     for (int i = 0; i < 8 && !slot; ++i) {
         Entry &x = table[(at + i) % kEntries];
-        if (x.fn == kernel && x.dev == dev) {
-            if (x.bytes >= bytes) return cudaSuccess;
-            slot = &x;
-        } else if (!x.fn) {
-            slot = &x;
-        }
+        if (x.fn == kernel && x.dev == dev) return cudaSuccess;
+        if (!x.fn) slot = &x;
     }
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess && slot) *slot = Entry{kernel, dev, bytes};
+    if (e == cudaSuccess && slot) *slot = Entry{kernel, dev};
     return e;
 }
 

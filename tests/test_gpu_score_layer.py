@@ -1,6 +1,8 @@
 """Parity of the attention score layer (Section 4.1: mean pooling, linear map, arg max per chunk
 and head) with the fp64 oracle, through the C ABI, and its use as the route of a block-routed
 forward."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -91,3 +93,22 @@ def test_score_layer_feeds_the_block_routed_forward():
     ref = oracle.hybrid_fwd(y["q"], y["k"], y["v"], y["g"], y["beta"], y["route"], y["w"],
                             scale_la=wl.scale_la, scale_sm=wl.scale_sm, block=64)
     check_fwd(wl, got, ref, 2e-2)
+
+
+def test_score_layer_of_two_widths_from_two_threads():
+    """A narrow call on another thread between two wide ones on this: the wide one's shared memory stays allowed."""
+    wide, narrow = features(5, 1, 128, 8192, 2, True), features(6, 1, 128, 2048, 2, True)
+    first = run_score_layer(*wide, 2, True)
+    errors = []
+
+    def other():
+        try:
+            run_score_layer(*narrow, 2, True)
+        except Exception as e:      # (an assertion of its own thread)
+            errors.append(e)
+
+    t = threading.Thread(target=other)
+    t.start()
+    t.join()
+    again = run_score_layer(*wide, 2, True)
+    assert not errors and all(np.array_equal(a, b) for a, b in zip(first, again))

@@ -98,3 +98,33 @@ def test_saved_forward_then_backward(name, B, H, L, block):
         a = alone[n].float().cpu().numpy()
         assert np.abs(got[n] - a).max() <= 1e-3 * TOL[kind] * max(np.sqrt((a ** 2).mean()), 1e-30) + \
             (np.abs(a).max() * 2.0 ** -8 if kind == "bf16" and n in ("dq", "dk", "dv") else 0.0), n
+
+
+@pytest.mark.parametrize("d,G,norm,block,size", [(128, 1, False, False, 1e3), (128, 2, True, True, 1e3),
+                                                 (128, 1, False, True, 1e4), (64, 1, False, False, 1.5e4)])
+def test_bwd_from_a_large_carried_state(d, G, norm, block, size):
+    """A carried state up to a quarter of what the forward's fp16 operand holds, forgotten within the first chunk: dW there
+    exceeds fp16's range in rows whose decay is nearly zero.  Errors are relative 2-norms: an operand carries 2^-11, and
+    the first chunk's sums cancel by up to ten."""
+    from oracle import grouped
+    from paper_2602_03681_b200 import binding
+    B, H, L = 1, 2, 256
+    wl = inputs.WORKLOADS["cfg1_bf16_prefill" if d == 128 else "cfg4_bf16_train"]
+    x = inputs.make_layer_inputs(wl, B=B, H=H, L=L, route=inputs.route_blocks(3, (B, L, H), 0.2) if block else None)
+    s0 = (size * np.random.default_rng(5).standard_normal((B, H, d, d))).astype(np.float32)
+    x["g"] = np.minimum(x["g"], np.float32(-0.3))
+    kw = dict(scale_la=wl.scale_la, scale_sm=(d // G) ** -0.5 if norm else wl.scale_sm)
+    t = {n: dev(x[n], torch.bfloat16) for n in ("q", "k", "v", "dout")}
+    p = binding.make_params(B, H, L, d, binding.NATSL_BF16, w=(w := dev(x["w"])), state_in=(s := dev(s0)), G=G, norm_eps=1e-6,
+                            flags=(binding.BLOCK_ROUTING if block else 0) | (binding.QK_NORM if norm else 0), **kw)
+    got = {n: torch.empty_like(t["q"]) for n in ("dq", "dk", "dv")}
+    got.update(dg=torch.empty((B, L, H), device="cuda"), dbeta=torch.empty((B, L, H), device="cuda"), dw=torch.empty_like(w))
+    ws = binding.alloc_workspace(p, binding.OP_BWD)
+    binding.natsl_hybrid_bwd(t["q"], t["k"], t["v"], dev(x["g"]), dev(x["beta"]), dev(x["route"]), t["dout"], *got.values(), p, ws)
+    torch.cuda.synchronize()
+    assert binding.natsl_device_status(ws) == 0 and s is not None
+    ref = grouped.hybrid_bwd(x["q"], x["k"], x["v"], x["g"], x["beta"], x["route"], x["w"], x["dout"], G=G, qk_norm=norm,
+                             norm_eps=1e-6, block=64 if block else None, state_in=s0, **kw)
+    for n, a in got.items():
+        e = np.linalg.norm(a.double().cpu().numpy() - ref[n]) / np.linalg.norm(ref[n])
+        assert e <= TOL["bf16"], (n, e)        # (not a number fails too)

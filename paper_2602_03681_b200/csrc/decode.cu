@@ -10,6 +10,7 @@
 // of the state's value columns (the columns of the delta rule are independent).  Whichever item of the
 // pair finishes last (an atomic ticket, nobody waits) merges the partial results, adds the new token's own
 // term, normalises, combines, writes `out`, appends the token to the cache and bumps its length.
+// A pair's slices go by its length: see decode_split.
 //   * Few pairs: every item has a CTA of its own and the cache is cut as finely as the machine has room
 //     for (up to 16 slices), because a slice is walked serially.
 //   * Many pairs: persistent CTAs, two per SM.  The copy warp runs ahead into the next item's slice (96 KB in
@@ -47,35 +48,65 @@ constexpr int kTileKeys = 32;                    // one key per group of eight l
 constexpr int kRingBytes = 96 * 1024;
 constexpr int kStateParts = 2;
 constexpr int kMaxParts = 16;
-constexpr int kCtasPerSm = 2, kResident = kCtasPerSm * 148;
+constexpr int kCtasPerSm = 2;
+constexpr int kMaxItems = 128;                   // items of a CTA
 
+// ---- How a pair's cache is cut: by its length, known on the device only.  The host works the count out for every class of
+// lengths (1 to 300 keys, to 600, to 900, to 1200, more) that the capacity allows and passes the counts along. ----
 // Cache items per (sequence, head), when every item is to be resident at once (0: not possible) ...
-inline int parts_resident(size_t BH) {
-    const int p = (int)(kResident / BH) - kStateParts;
+inline int parts_resident(int BH, int resident) {
+    const int p = resident / BH - kStateParts;
     return p > kMaxParts ? kMaxParts : (p > 0 ? p : 0);
 }
 // ... and when the CTAs go round: the count whose items fill the last round best, an item's start and merge counted as
-// 5 % of a round; from one item per 300 keys that the cache may hold (a round of nearly empty items takes 4 us: 504 pairs of
-// 100 keys 45 us a step with four items each), four at most.
-inline int parts_persistent(size_t BH, int cap) {
-    const int from = std::min(4, std::max(1, (cap + 299) / 300));
+// 5 % of a round; from one item per 300 keys (a round of nearly empty items takes 4 us: 504 pairs of 100 keys 45 us a step
+// with four items each), four at most.
+inline int parts_persistent(int BH, int resident, int keys) {
+    const int from = std::min(4, std::max(1, (keys + 299) / 300));
     int best = from;
     float least = 1e30f;
     for (int p = from; p <= kMaxParts; ++p) {
-        const float n = (float)BH * (p + kStateParts), per = n / kResident;
+        const float n = (float)BH * (p + kStateParts), per = n / resident;
         const float cost = (float)(int)(per + 0.999f) / per + 0.05f * p;
         if (cost < least) { least = cost; best = p; }
     }
     return best;
 }
-// Resident where it can be, unless that makes only one or two items of a cache that may hold more than 600 keys for each:
-// they then take much longer than the state items, and half of the CTAs wait for them.  (The host knows the cache's
-// capacity, not its length.)  Per step, resident -> persistent: 96 pairs of 1638 keys 26.3 -> 18.6 us, 90 pairs of the
-// normalised mode, 800 keys, 19.2 -> 14.9; 64 pairs of 1638 keys 16.3 -> 15.1; but 72 pairs of 800 keys 12.9 -> 13.9, 96 of
-// 200 8.6 -> 11.1.
-inline int decode_parts(size_t BH, int cap) {
-    const int p = parts_resident(BH);
-    return p > 2 || (p > 0 && cap <= 600 * p) ? p : parts_persistent(BH, cap);
+// Resident where it can be, unless that makes only one or two items of a cache of more than 600 keys for each:
+// they then take much longer than the state items, and half of the CTAs wait for them.  Per step, resident -> going round:
+// 96 pairs of 1638 keys 26.3 -> 18.6 us, 90 pairs of the normalised mode, 800 keys, 19.2 -> 14.9; 64 pairs of 1638 keys
+// 16.3 -> 15.1; but 72 pairs of 800 keys 12.9 -> 13.9, 96 of 200 8.6 -> 11.1.
+inline int decode_parts(int BH, int resident, int keys) {
+    const int p = parts_resident(BH, resident);
+    return p > 2 || (p > 0 && keys <= 600 * p) ? p : parts_persistent(BH, resident, keys);
+}
+// What the kernel gets: `parts` items are laid out for every pair, those beyond the count of its length are empty.  Where
+// all classes that the capacity allows agree nothing is empty, and the kernel that does not ask runs.  (With the count
+// taken from the capacity, 4096 rows cost short sequences: 64 pairs of 200 keys 10.6 us a step, 7.9 by length, 504 of 100
+// 43.4 and 33.8, 1024 of 100 85.9 and 65.1.)
+// Order of the items: the first `front` cache items and the state items of every pair, then the rest.  Where the shortest
+// class's items fill no more than two rounds these are the front, so that short caches are spread as evenly as if nothing
+// were empty (96 pairs of 200 keys in 4096 rows 12.4 -> 8.3 us, 100 of 600 15.8 -> 12.6); elsewhere the front is everything
+// (with a front, 1024 pairs of 1638 keys 161 -> 173: first the states, then the caches).
+constexpr int kClassKeys = 300, kClasses = 5, kClassBits = 5;
+struct DecSplit { int parts, front; uint32_t by_class; bool varied; };
+inline DecSplit decode_split(int BH, int resident, int cap) {
+    DecSplit sp{0, 0, 0u, false};
+    int first = 0;
+    for (int c = 0; c < kClasses; ++c) {
+        const int keys = c + 1 < kClasses ? std::min(cap, (c + 1) * kClassKeys) : cap;
+        const int p = decode_parts(BH, resident, keys);
+        if (c == 0) first = p;
+        sp.by_class |= (uint32_t)p << (c * kClassBits);
+        sp.parts = std::max(sp.parts, p);
+        sp.varied |= p != first;
+    }
+    sp.front = BH * (first + kStateParts) <= 2 * resident ? first : sp.parts;
+    return sp;
+}
+__device__ __forceinline__ int class_parts(uint32_t by_class, int keys) {
+    const int c = min(max((keys + kClassKeys - 1) / kClassKeys, 1), kClasses) - 1;
+    return (by_class >> (c * kClassBits)) & ((1u << kClassBits) - 1u);
 }
 
 template <typename T> struct Vec16;   // 16 bytes of T as fp32 values
@@ -117,14 +148,15 @@ template <typename T, int D, int G> struct DecLayout {
     static constexpr int kTotal = oMz + 2 * kWarps * G * 8;
 };
 
-template <typename T, int D, int G, bool kNorm>
+// kVaried: the count of a pair's cache items depends on its length.
+template <typename T, int D, int G, bool kNorm, bool kVaried>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 decode_step_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v,
                    const float *__restrict__ g, const float *__restrict__ beta,
                    const uint8_t *__restrict__ route, const float *__restrict__ w,
                    float *__restrict__ state, T *__restrict__ k_cache, T *__restrict__ v_cache,
                    int32_t *__restrict__ cache_len, int cap, T *__restrict__ out, float scale_la,
-                   float scale_sm, float eps, uint8_t *__restrict__ ws, int BH, int parts, float norm_eps) {
+                   float scale_sm, float eps, uint8_t *__restrict__ ws, int BH, DecSplit split, float norm_eps) {
     using SL = DecLayout<T, D, G>;
     constexpr int kStages = SL::kStages, kRowBytes = SL::kRowBytes, kTileBytes = SL::kTileBytes;
     constexpr int ds = D / G;                      // columns per softmax head
@@ -145,16 +177,23 @@ decode_step_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__
 
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ uint64_t full[kStages], empty[kStages], done[2], taken[2];
+    __shared__ uint64_t looked, first_read;
+    __shared__ uint32_t s_empty[kMaxItems / 32], s_closed[kMaxItems / 32];
+    __shared__ int s_len[kMaxItems], s_pair[kMaxItems];
+    __shared__ int2 s_tiles[kMaxItems];
     __shared__ int s_abort[2];   // s_abort[1]: wait limit (see mbar_wait)
     auto slot_of = [&](int i) { return reinterpret_cast<float *>(smem + SL::oScratch) + i * SL::kSlotFloats; };
     float2 *mz = reinterpret_cast<float2 *>(smem + SL::oMz);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int per_head = parts + kStateParts, total = BH * per_head;
+    const int parts = split.parts, front = split.front, per_head = parts + kStateParts, total = BH * per_head;
+    const int n_front = BH * (front + kStateParts);
     int32_t *status = reinterpret_cast<int32_t *>(ws);
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], kWarps); }
         for (int s = 0; s < 2; ++s) { mbar_init(&done[s], kWarps); mbar_init(&taken[s], 1); }
+        mbar_init(&looked, 1);
+        mbar_init(&first_read, kWarps);
         s_abort[0] = 0;
         s_abort[1] = 0;
         fence_mbar_init();
@@ -164,45 +203,101 @@ decode_step_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__
     grid_dependency_wait();
     launch_dependents();
 
+    // This CTA's items: blockIdx.x, blockIdx.x + gridDim.x, ...; part >= parts: a state item.
+    // (Counted: with the item's number as the loops' test a step of two items per CTA took 1 us longer, 64 pairs 14.3 for 13.3.)
+    auto item_no = [&](int ord) { return (int)blockIdx.x + ord * (int)gridDim.x; };
+    const int n_items = (total - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;
+    auto has = [&](int ord) { return ord < n_items; };
+    auto locate = [&](int item, int &part, int &bh) {
+        if (!kVaried || item < n_front) {
+            bh = item / (front + kStateParts);
+            part = item - bh * (front + kStateParts);
+            if (kVaried && part >= front) part += parts - front;
+        } else {
+            bh = (item - n_front) / (parts - front);
+            part = front + (item - n_front) - bh * (parts - front);
+        }
+    };
+    // The copy warp looks up the lengths of all of them and lists what it will copy; cache items that the length leaves
+    // empty get no turn, the finisher takes their tickets at once.
+    // The length changes with the pair's last ticket, so every ticket of a CTA comes behind every read of that length in
+    // the CTA: the copy warp's, through `looked`, the work warps', through the item's turn or, where the first item, which
+    // they do not wait for the look-up with, has none, through `first_read`.
+    auto parts_of = [&](int n_old) { return kVaried ? class_parts(split.by_class, n_old) : parts; };
+    auto empty_item = [&](int ord) { return (s_empty[ord >> 5] >> (ord & 31)) & 1u; };
     // Tiles of a cache item.  A stored length outside [0, cap] (a prefill whose cache overflowed, a caller's
     // mistake) is clamped, so that no copy can leave the pair's rows; the finisher reports it.
     auto tiles_of = [&](int part, int n_old, bool cache_full, int &t_begin, int &t_end) {
         const int tiles = cache_full ? 0 : (n_old + kTileKeys - 1) / kTileKeys;
-        const int tpp = (tiles + parts - 1) / parts;
+        const int np = parts_of(n_old), tpp = (tiles + np - 1) / np;
         t_begin = min(part * tpp, tiles);
         t_end = min(t_begin + tpp, tiles);
     };
 
     if (warp == kWarps) {
         // ---------------- copy warp: the cache slices of all items of this CTA, back to back ----------------
-        if (lane != 0) return;
-        int it = 0;                                      // tiles issued so far
+        int t = 0, t_end = 0, bh = 0, n_old = 0, it = 0; // (it: tiles issued so far)
         bool ok = true;
-        int item = blockIdx.x, n_next = 0, rv_next = 0;
-        auto fetch = [&]() {
-            while (item < total && item % per_head >= parts) item += gridDim.x;
-            if (item < total) { n_next = cache_len[item / per_head]; rv_next = route[item / per_head]; }
+        auto issue = [&]() {                             // tile t of pair bh
+            const int s = it % kStages;
+            ok = mbar_wait(&empty[s], ((it / kStages) & 1) ^ 1, abort_flag);
+            if (!ok) return;
+            const int rows = min(kTileKeys, n_old - t * kTileKeys);
+            const uint32_t bytes = (uint32_t)rows * kRowBytes;
+            const size_t at = (size_t)bh * cap * kRowBytes + (size_t)t * kTileBytes;
+            mbar_arrive_expect_tx(&full[s], 2 * bytes);
+            bulk_load_1d(smem + (2 * s) * kTileBytes, reinterpret_cast<const uint8_t *>(k_cache) + at, bytes, &full[s]);
+            bulk_load_1d(smem + (2 * s + 1) * kTileBytes, reinterpret_cast<const uint8_t *>(v_cache) + at, bytes, &full[s]);
+            ++t;
+            ++it;
         };
-        fetch();
-        while (item < total && ok) {
-            const int part = item % per_head, bh = item / per_head;
-            const int n_old = min(max(n_next, 0), cap);
-            int t, t_end;
-            tiles_of(part, n_old, rv_next != 0 && n_old >= cap, t, t_end);
-            item += gridDim.x;
-            fetch();                                     // (the next item's length is on its way meanwhile)
-            const uint8_t *kc = reinterpret_cast<const uint8_t *>(k_cache + (size_t)bh * cap * D);
-            const uint8_t *vc = reinterpret_cast<const uint8_t *>(v_cache + (size_t)bh * cap * D);
-            for (; t < t_end; ++t, ++it) {
-                const int s = it % kStages;
-                ok = mbar_wait(&empty[s], ((it / kStages) & 1) ^ 1, abort_flag);
-                if (!ok) break;
-                const int rows = min(kTileKeys, n_old - t * kTileKeys);
-                const uint32_t bytes = (uint32_t)rows * kRowBytes;
-                mbar_arrive_expect_tx(&full[s], 2 * bytes);
-                bulk_load_1d(smem + (2 * s) * kTileBytes, kc + (size_t)t * kTileBytes, bytes, &full[s]);
-                bulk_load_1d(smem + (2 * s + 1) * kTileBytes, vc + (size_t)t * kTileBytes, bytes, &full[s]);
+        int part = parts, pr = 0, len = 0, rv = 0;       // of this lane's item of the batch: a cache item or none
+        auto look_up = [&](int ord) {
+            part = parts;
+            if (has(ord)) locate(item_no(ord), part, pr);
+            if (part < parts) { len = cache_len[pr]; rv = route[pr]; }
+        };
+        look_up(lane);
+        if (lane == 0 && part < parts) {                 // the first item: a ring of tiles ahead of the others' lengths
+            bh = pr;
+            n_old = min(max(len, 0), cap);
+            tiles_of(part, n_old, rv != 0 && n_old >= cap, t, t_end);
+            while (t < t_end && it < kStages && ok) issue();
+        }
+        __syncwarp();
+        int n = 0;                                       // listed: cache items with tiles behind the first item
+        for (int o0 = 0; has(kVaried ? o0 : o0 + 1); o0 += 32) {
+            const int ord = o0 + lane;
+            if (o0) look_up(ord);
+            bool empty_one = false, copies = false;
+            int t0 = 0, t1 = 0;
+            if (part < parts) {
+                len = min(max(len, 0), cap);
+                empty_one = part >= parts_of(len);
+                tiles_of(part, len, rv != 0 && len >= cap, t0, t1);
+                copies = ord > 0 && t1 > t0;
             }
+            const unsigned me = __ballot_sync(0xffffffffu, empty_one), mc = __ballot_sync(0xffffffffu, copies);
+            if (copies) {
+                const int at = n + __popc(mc & ((1u << lane) - 1u));
+                s_pair[at] = pr;
+                s_tiles[at] = make_int2(t0, t1);
+                s_len[at] = len;
+            }
+            if (kVaried && lane == 0) s_empty[o0 >> 5] = me;
+            n += __popc(mc);
+        }
+        __syncwarp();
+        if (lane != 0) return;
+        mbar_arrive(&looked);                            // (a release: no length is read behind it)
+        for (int i = 0; ok; ++i) {
+            if (t < t_end) issue();
+            int bh_next = 0, n_next = 0;                 // (while that tile travels)
+            int2 t_next = make_int2(0, 0);
+            if (i < n) { bh_next = s_pair[i]; n_next = s_len[i]; t_next = s_tiles[i]; }
+            while (t < t_end && ok) issue();
+            if (i >= n) break;
+            bh = bh_next; n_old = n_next; t = t_next.x; t_end = t_next.y;
         }
         for (int u = max(0, it - kStages); u < it; ++u)  // no copy in flight when the CTA retires, aborted or not
             mbar_wait_drain(&full[u % kStages], (u / kStages) & 1);
@@ -220,14 +315,33 @@ decode_step_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__
             return x;
         };
         const int sg = lane / kLs;
-        for (int item = blockIdx.x, i = 0; item < total; item += gridDim.x, ++i) {
-            const int part = item % per_head, bh = item / per_head;
-            int32_t *ticket = reinterpret_cast<int32_t *>(ws + dec_off_tickets()) + bh;
+        int32_t *tickets = reinterpret_cast<int32_t *>(ws + dec_off_tickets());
+        const bool known = mbar_wait(&looked, 0, abort_flag) && (!kVaried || mbar_wait(&first_read, 0, abort_flag));
+        // The empty items' tickets, a lane each; who gets a pair's last one finishes it when its place in the order comes.
+        // (After a time-out, which is reported, all of the CTA's tickets are still taken, so that they end at zero.)
+        for (int o0 = 0; kVaried && known && has(o0); o0 += 32) {
+            const int ord = o0 + lane;
+            bool closes = false;
+            if (has(ord) && empty_item(ord)) {
+                int pt, pr;
+                locate(item_no(ord), pt, pr);
+                closes = atom_add_acq_rel(tickets + pr, 1) == per_head - 1;
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, closes);
+            if (lane == 0) s_closed[o0 >> 5] = m;
+        }
+        __syncwarp();
+#pragma unroll 1
+        for (int i = 0, ord = 0; has(ord); ++ord) {
+            const bool turn = !kVaried || !known || !__any_sync(0xffffffffu, empty_item(ord));
+            if (!turn && !__any_sync(0xffffffffu, (s_closed[ord >> 5] >> (ord & 31)) & 1u)) continue;
+            int part, bh;
+            locate(item_no(ord), part, bh);
+            int32_t *ticket = tickets + bh;
             float *partials = reinterpret_cast<float *>(ws + dec_off_partials(BH, D)) + (size_t)bh * parts * kPs;
             float *ola_ws = reinterpret_cast<float *>(ws + dec_off_ola(BH)) + (size_t)bh * D;
             const float *sc = slot_of(i & 1);
-            // (after a time-out, which is reported, the tickets are still taken, so that they end at zero)
-            const bool ok = mbar_wait(&done[i & 1], (i >> 1) & 1, abort_flag);
+            const bool ok = turn && mbar_wait(&done[i & 1], (i >> 1) & 1, abort_flag);
             if (!ok) {
             } else if (part < parts) {                   // eight warps' (m, z, acc) -> one partial
                 float M = -INFINITY, Z = 0.f, o[V];
@@ -263,12 +377,15 @@ decode_step_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__
             }
             // ticket (release by lane 0 behind the warp's barrier, acquire by it before the warp's barrier)
             __syncwarp();
-            int last = 0;
+            int last = !turn;
             if (lane == 0) {
-                mbar_arrive(&taken[i & 1]);
-                last = atom_add_acq_rel(ticket, 1) == per_head - 1;
+                if (turn) {
+                    mbar_arrive(&taken[i & 1]);
+                    last = atom_add_acq_rel(ticket, 1) == per_head - 1;
+                }
                 if (last) *ticket = 0;                   // ready for the next step
             }
+            i += turn;
             last = __shfl_sync(0xffffffffu, last, 0);
             if (!last) continue;
             // All of the pair's partial results and the token's rows in one round trip.
@@ -293,7 +410,11 @@ decode_step_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__
             }
             const float wn = w ? w[(size_t)bh * 2] : 0.5f, wl = w ? w[(size_t)bh * 2 + 1] : 0.5f;
             const bool r = rv != 0;                      // append, and attend to itself
-            const int n_old = min(max(n_raw, 0), cap);
+            const int n_old = min(max(n_raw, 0), cap), np = parts_of(n_old);
+#pragma unroll
+            for (int a = 0; kVaried && a < G; ++a) {     // (partials of empty items are another step's)
+                if (lane >= np) { pm[a] = -INFINITY; pz[a] = 0.f; }
+            }
             if (n_raw != n_old && lane == 0) atomicMin(status, (int)NATSL_ERR_CACHE_FULL);
             if (r && n_old >= cap) {                     // no room: the sequence is left untouched
 #pragma unroll
@@ -338,7 +459,7 @@ decode_step_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__
                     if (a == sg) f = fa;
                 }
 #pragma unroll
-                for (int x = 0; x < V; ++x) on[x] = fmaf(pa[pt][x], f, on[x]);
+                for (int x = 0; x < V; ++x) on[x] = fmaf(!kVaried || pt < np ? pa[pt][x] : 0.f, f, on[x]);
             }
             const float iz = Z > 0.f ? 1.f / Z : 0.f;    // (no visible key: o_nla = 0)
             float tn = 0.f, tl = 0.f;
@@ -364,11 +485,22 @@ decode_step_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__
     }
 
     int it = 0;                                          // tiles consumed so far
-    for (int item = blockIdx.x, i = 0; item < total; item += gridDim.x, ++i) {
-        const int part = item % per_head, bh = item / per_head;
+#pragma unroll 1
+    for (int i = 0, ord = 0; has(ord); ++i, ++ord) {
+        if (kVaried && ord) {
+            if (ord == 1 && !mbar_wait(&looked, 0, abort_flag)) break;
+            if (__any_sync(0xffffffffu, empty_item(ord))) { --i; continue; }
+        }
+        int part, bh;
+        locate(item_no(ord), part, bh);
         // route 0: linear token (delta rule); 1: softmax token (appended to the cache); 2: token of a
         // block whose decision is still open -- both (Section 4.1, pseudo-update of both hidden states)
         const int rv = route[bh], n_raw = cache_len[bh];
+        if (kVaried && ord == 0) {
+            const bool none = __any_sync(0xffffffffu, part < parts && part >= parts_of(min(max(n_raw, 0), cap)));
+            if (lane == 0) mbar_arrive(&first_read);
+            if (none) { --i; continue; }
+        }
         float *slot_out = slot_of(i & 1);
         if (part < parts) {
             // ---------------- cache item: one slice of the retained K/V ----------------
@@ -643,17 +775,22 @@ static cudaError_t decode_impl(const void *q, const void *k, const void *v, cons
     if constexpr (D / G * (int)sizeof(T) < 64) {
         return cudaErrorInvalidValue;
     } else {
-        auto kernel = decode_step_kernel<T, D, G, kNorm>;
+        const int BH = s.B * s.H, resident = kCtasPerSm * sm_count();
+        const DecSplit split = decode_split(BH, resident, cap);
+        const int per_head = split.parts + kStateParts;
+        auto kernel = split.varied ? decode_step_kernel<T, D, G, kNorm, true> : decode_step_kernel<T, D, G, kNorm, false>;
         cudaError_t e = allow_smem(kernel, DecLayout<T, D, G>::kTotal);
         if (e != cudaSuccess) return e;
-        const int BH = s.B * s.H, parts = decode_parts((size_t)BH, cap), per_head = parts + kStateParts;
-        // Persistent beyond one resident set; the stride then has no factor in common with the items per
-        // pair, so that every CTA gets the same mix of cache and state items.
+        // Persistent beyond one resident set, up to the items a CTA can list; the stride then has no factor in common with
+        // the items per pair (of the front), so that every CTA gets the same mix of cache and state items.
         auto gcd = [](int a, int b) { while (b) { const int c = a % b; a = b; b = c; } return a; };
         int grid = BH * per_head;
-        if (grid > kCtasPerSm * sm_count()) {
-            grid = kCtasPerSm * sm_count();
-            while (grid > 1 && gcd(grid, per_head) != 1) --grid;
+        if (grid > resident) {
+            const int least = (grid + kMaxItems - 1) / kMaxItems;
+            grid = resident;
+            while (grid > 1 && gcd(grid, split.front + kStateParts) != 1) --grid;
+            if (grid < least)
+                for (grid = least; gcd(grid, split.front + kStateParts) != 1;) ++grid;
         }
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(grid);
@@ -667,7 +804,7 @@ static cudaError_t decode_impl(const void *q, const void *k, const void *v, cons
         cfg.numAttrs = 1;
         e = cudaLaunchKernelEx(&cfg, kernel, (const T *)q, (const T *)k, (const T *)v, g, beta, route, w, state,
                                (T *)k_cache, (T *)v_cache, cache_len, (int)cap, (T *)out, scale_la, scale_sm, eps,
-                               (uint8_t *)ws, BH, parts, norm_eps);
+                               (uint8_t *)ws, BH, split, norm_eps);
         count_launch();
         return e;
     }

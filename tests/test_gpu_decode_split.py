@@ -62,3 +62,60 @@ def test_decode_split_follows_the_capacity(B, H, cap):
                              scale_la=wl.scale_la, scale_sm=wl.scale_sm)
     check_stored(out.float().cpu().numpy(), ref["out"], TOL[wl.dtype], wl.dtype, "step")
     assert binding.natsl_device_status(ws) == 0
+
+
+def _steps(wl, x, n, cap, B, H):
+    """Two steps of x's first token on caches of n entries in cap rows: out, state, cache_len, k_cache, v_cache."""
+    from paper_2602_03681_b200 import binding
+    dt = tdtype(wl)
+    kc, vc = (torch.zeros((B, H, cap, wl.d), dtype=dt, device="cuda") for _ in range(2))
+    rows = min(cap, x["k_cache"].shape[2])
+    kc[:, :, :rows], vc[:, :, :rows] = dev(x["k_cache"], dt)[:, :, :rows], dev(x["v_cache"], dt)[:, :, :rows]
+    state, n, w = dev(x["state"]), dev(n), dev(x["w"][0])
+    p = binding.make_params(B, H, 0, wl.d, binding._dtype_code(kc), wl.scale_la, wl.scale_sm, w=w)
+    ws = binding.alloc_workspace(p, binding.OP_DECODE)
+    out = torch.empty((B, H, wl.d), dtype=dt, device="cuda")
+    for _ in range(2):          # (the second step finds the first one's tickets and partial results)
+        binding.natsl_decode_step(dev(x["q"][0], dt), dev(x["k"][0], dt), dev(x["v"][0], dt), dev(x["g"][0]),
+                                  dev(x["beta"][0]), dev(x["route"][0]), state, kc, vc, n, out, p, ws)
+    assert binding.natsl_device_status(ws) == 0
+    return out, state, n, kc, vc
+
+
+def _oracle_steps(wl, x, n):
+    o = [x["state"].astype(np.float64), x["k_cache"].astype(np.float64), x["v_cache"].astype(np.float64), n.copy()]
+    for _ in range(2):
+        ref = oracle.decode_step(x["q"][0], x["k"][0], x["v"][0], x["g"][0], x["beta"][0], x["route"][0], x["w"][0], *o,
+                                 scale_la=wl.scale_la, scale_sm=wl.scale_sm)
+    return ref["out"], o
+
+
+@pytest.mark.parametrize("name,B,H,most", [("cfg3_bf16_decode", 8, 8, 200), ("cfg3_bf16_decode", 12, 6, 1300),
+                                           ("cfg3_bf16_decode", 8, 12, 700), ("cfg4_bf16_train", 9, 11, 900),
+                                           ("cfg0_f32_tiny_fwd", 20, 15, 320)])
+def test_decode_split_goes_by_length(name, B, H, most):
+    """Mixed lengths in caches that hold them just so and in roomy ones: the same bits, because how a pair's cache is cut
+    depends on its length alone, and the oracle's values."""
+    wl = inputs.WORKLOADS[name]
+    x = inputs.make_decode_inputs(wl, B=B, H=H, steps=1, ctx_retained=most, cap=most + 2)
+    lengths = np.unique(np.minimum([0, 1, 31, 33, 100, 299, 300, 301, 599, 600, 601, 900, 901, 1199, 1200, 1201, most], most))
+    n = np.resize(np.random.default_rng(B).permutation(lengths), B * H).reshape(B, H).astype(np.int32)
+    tight, roomy = (_steps(wl, x, n, cap, B, H) for cap in (most + 2, 5000))
+    for a, b, what in zip(tight, roomy, ("out", "state", "cache_len", "k_cache", "v_cache")):
+        assert torch.equal(a, b[:, :, :a.shape[2]] if what.endswith("cache") else b), what
+    ref, o = _oracle_steps(wl, x, n)
+    check_stored(roomy[0].float().cpu().numpy(), ref, TOL[wl.dtype], wl.dtype)
+    assert np.array_equal(roomy[2].cpu().numpy(), o[3]) and rel_err(roomy[1].cpu().numpy(), o[0]) <= 1e-4
+
+
+@pytest.mark.parametrize("cap", [8, 400])
+def test_decode_more_items_than_a_resident_set_can_list(cap):
+    """16384 pairs: the CTAs that list their items are more than are resident at once."""
+    wl = inputs.WORKLOADS["cfg4_bf16_train"]
+    B, H = 256, 64
+    x = inputs.make_decode_inputs(wl, B=B, H=H, steps=1, ctx_retained=6, cap=8)
+    n = (np.arange(B * H) % 7).reshape(B, H).astype(np.int32)
+    got = _steps(wl, x, n, cap, B, H)
+    ref, o = _oracle_steps(wl, x, n)
+    check_stored(got[0].float().cpu().numpy(), ref, TOL[wl.dtype], wl.dtype)
+    assert np.array_equal(got[2].cpu().numpy(), o[3])

@@ -351,7 +351,7 @@ static int bwd_forward_part(const void *q, const void *k, const void *v, const f
     NATSL_TRY(launch_to_f32(qk ? q : nullptr, qk ? k : nullptr, v, f.q32, f.k32, f.v32,
                             (size_t)(B * L * H * d), s.bf16, st));
     if (!qk) {
-        NATSL_TRY(launch_qk_norm_f32(q, k, s.bf16, f.q32, f.k32, f.qs32, f.ks32, (size_t)(B * L * H), p->d, hg.G,
+        NATSL_TRY(launch_qk_norm_f32((const float *)q, (const float *)k, f.q32, f.k32, f.qs32, f.ks32, (size_t)(B * L * H), p->d, hg.G,
                                      hg.norm_eps, st));
         qs = f.qs32; ks = f.ks32;
     }
@@ -554,7 +554,7 @@ int natsl_hybrid_fwd(const void *q, const void *k, const void *v, const float *g
     // NATSL_QK_NORM: normalised copies first
     const void *q_la = q, *k_la = k, *q_sm = q, *k_nsm = k;
     if (hg.norm_eps >= 0.f) {
-        NATSL_TRY(launch_qk_norm_f32(q, k, false, f.q_la, f.k_la, f.q_sm, f.k_nsm,
+        NATSL_TRY(launch_qk_norm_f32((const float *)q, (const float *)k, f.q_la, f.k_la, f.q_sm, f.k_nsm,
                                      (size_t)p->B * p->L * p->H, p->d, hg.G, hg.norm_eps, st));
         q_la = f.q_la; k_la = f.k_la; q_sm = f.q_sm; k_nsm = f.k_nsm;
     }
@@ -682,7 +682,7 @@ int natsl_hybrid_bwd(const void *q, const void *k, const void *v, const float *g
                                         f.status, s, st, block ? st0 : st, side && !block ? side->fork : nullptr, hg));
         if (block) {
             if (side) NATSL_TRY(cudaStreamWaitEvent(st, side->join, 0));     // the reverse scan has finished
-            NATSL_TRY(launch_gdn_finish(a, f.dk_x, f.dv_x, s32, st0, false));
+            NATSL_TRY(launch_scatter_sm(a, f.dk_x, f.dv_x, s32, st0));
             NATSL_TRY(launch_softmax_bwd_own_block(q, k, v, f.dO16, f.lse, f.Dsm, route, p->scale_sm, f.dq_sm, f.dk_x,
                                                    f.dv_x, gsc, s, st, hg));
             NATSL_TRY(side_join.join());      // the side stream's last kernels
@@ -701,7 +701,7 @@ int natsl_hybrid_bwd(const void *q, const void *k, const void *v, const float *g
                                        dq_o, dk_o, dv_o, dg, dbeta, false, nullptr, nullptr, nullptr, f.status, s, st0,
                                        hg));
         // the retained tokens' dk, dv (rows the chunk kernel does not write)
-        NATSL_TRY(launch_gdn_finish(a, dk_o, dv_o, normed ? s32 : s, st, false));
+        NATSL_TRY(launch_scatter_sm(a, dk_o, dv_o, normed ? s32 : s, st));
         NATSL_TRY(side_join.join());
         if (normed)
             NATSL_TRY(launch_qk_norm_bwd_f32(q, k, true, route, f.dq32, f.dq_sm, f.dk32, f.dv32, dq, dk, dv,
@@ -721,7 +721,7 @@ int natsl_hybrid_bwd(const void *q, const void *k, const void *v, const float *g
         // tokens of linear blocks' from their own block (each token is written by exactly one of the
         // two); the assembly adds them to the linear branch's -- with the normalisation dk_x, a gradient with
         // respect to the softmax operation's copy, stays apart until its backward.
-        NATSL_TRY(launch_gdn_finish(a, f.dk_x, f.dv_x, s32, st, false));
+        NATSL_TRY(launch_scatter_sm(a, f.dk_x, f.dv_x, s32, st));
         NATSL_TRY(launch_softmax_bwd_own_block_simt(normed ? f.qs32 : f.q32, normed ? f.ks32 : f.k32, f.v32, f.do_nla, f.lse,
                                                     f.Dsm, route, p->scale_sm, f.dq_sm, f.dk_x, f.dv_x, gsc, s32, st,
                                                     hg.G));

@@ -488,11 +488,11 @@ template <int N> __device__ __forceinline__ void store_vec(__nv_bfloat16 *p, con
 }
 
 // The forward normalisation with the same layout (d = 64 or 128, a slice an aligned group of 32 / G lanes).
-template <typename T, int D>
+template <int D>
 __global__ void __launch_bounds__(256)
-qk_norm_f32_kernel(const T *__restrict__ q, const T *__restrict__ k, float *__restrict__ q_la,
-                       float *__restrict__ k_la, float *__restrict__ q_sm, float *__restrict__ k_sm,
-                       size_t rows, int G, float norm_eps) {
+qk_norm_f32_kernel(const float *__restrict__ q, const float *__restrict__ k, float *__restrict__ q_la,
+                   float *__restrict__ k_la, float *__restrict__ q_sm, float *__restrict__ k_sm,
+                   size_t rows, int G, float norm_eps) {
     constexpr int N = D / 32;
     const size_t row = (size_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
@@ -519,11 +519,9 @@ qk_norm_f32_kernel(const T *__restrict__ q, const T *__restrict__ k, float *__re
 #pragma unroll
         for (int j = 0; j < N; ++j) y[j] = x[which][j] * rl;
         store_vec<N>((which ? k_la : q_la) + at, y);
-        if (q_sm) {
 #pragma unroll
-            for (int j = 0; j < N; ++j) y[j] = x[which][j] * rs;
-            store_vec<N>((which ? k_sm : q_sm) + at, y);
-        }
+        for (int j = 0; j < N; ++j) y[j] = x[which][j] * rs;
+        store_vec<N>((which ? k_sm : q_sm) + at, y);
     }
 }
 
@@ -691,16 +689,12 @@ cudaError_t launch_softmax_combine_simt(const void *q, const void *k_sm, const v
                    out, o_nla, lse, br, s, st);
 }
 
-cudaError_t launch_qk_norm_f32(const void *q, const void *k, bool bf16, float *q_la, float *k_la, float *q_sm,
-                               float *k_sm, size_t rows, int d, int G, float norm_eps, cudaStream_t st) {
+cudaError_t launch_qk_norm_f32(const float *q, const float *k, float *q_la, float *k_la, float *q_sm, float *k_sm,
+                               size_t rows, int d, int G, float norm_eps, cudaStream_t st) {
     const unsigned blocks = (unsigned)((rows + 7) / 8);
-    if ((d != 64 && d != 128) || G < 1 || 32 % G != 0 || !q_sm != !k_sm) return cudaErrorInvalidValue;
-#define NATSL_NF(TT, DD)                                                                                  \
-    qk_norm_f32_kernel<TT, DD><<<blocks, 256, 0, st>>>((const TT *)q, (const TT *)k, q_la, k_la, q_sm, k_sm, \
-                                                      rows, G, norm_eps)
-    if (bf16) { if (d == 128) NATSL_NF(__nv_bfloat16, 128); else NATSL_NF(__nv_bfloat16, 64); }
-    else { if (d == 128) NATSL_NF(float, 128); else NATSL_NF(float, 64); }
-#undef NATSL_NF
+    if ((d != 64 && d != 128) || G < 1 || 32 % G != 0) return cudaErrorInvalidValue;
+    auto kernel = d == 128 ? qk_norm_f32_kernel<128> : qk_norm_f32_kernel<64>;
+    kernel<<<blocks, 256, 0, st>>>(q, k, q_la, k_la, q_sm, k_sm, rows, G, norm_eps);
     count_launch();
     return cudaGetLastError();
 }

@@ -69,9 +69,8 @@ cudaError_t launch_softmax_combine_simt(const void *q, const void *k_sm, const v
 // (G > 1: grouped softmax heads, fp32 storage only; see HeadGroups)
 // fp32 storage: q, k [rows, d] -> L2-normalised rows (q_la, k_la) and rows with each of the G slices
 // RMS-normalised (q_sm, k_sm)
-cudaError_t launch_qk_norm_f32(const void *q, const void *k, bool bf16, float *q_la, float *k_la, float *q_sm,
-                               float *k_sm, size_t rows, int d, int G, float norm_eps, cudaStream_t st);
-// (q, k in fp32 or bf16 storage; q_sm, k_sm may be nullptr)
+cudaError_t launch_qk_norm_f32(const float *q, const float *k, float *q_la, float *k_la, float *q_sm, float *k_sm,
+                               size_t rows, int d, int G, float norm_eps, cudaStream_t st);
 // Its backward, in place: dq (gradient w.r.t. the L2 copy) and dq_sm (w.r.t. the RMS copy) -> dq;
 // dk (w.r.t. the L2 copy for a linear token, the RMS copy for a retained one) -> dk.
 cudaError_t launch_qk_norm_bwd_f32(const void *q, const void *k, bool bf16, const uint8_t *route,
@@ -297,10 +296,8 @@ struct AssembleArgs {
 // compacted softmax-branch gradients), dbeta, dg.  Three kernels.
 cudaError_t launch_gdn_assemble(const AssembleArgs &a, void *dq, void *dk, void *dv, Shape s,
                                 cudaStream_t st);
-// The last two of those kernels only (dg from the per-token sums, scatter of the retained tokens'
-// dk, dv), for callers that formed dq, dk, dv of the linear tokens and the sums themselves.
-cudaError_t launch_gdn_finish(const AssembleArgs &a, void *dk, void *dv, Shape s, cudaStream_t st,
-                              bool with_dg = true);
+// The last of those kernels only (scatter of the retained tokens' dk, dv), for callers that form the rest themselves.
+cudaError_t launch_scatter_sm(const AssembleArgs &a, void *dk, void *dv, Shape s, cudaStream_t st);
 // (kap_c [B,H,L/C]: the chunk sums of kappa, or kappa_tok [B,H,L]: kappa per token, summed here)
 cudaError_t launch_dscore(const uint8_t *route, const int32_t *sm_chunk_prefix, const float *dmask,
                           const float *kap_c, const float *kappa_tok, int cap, float *dscore, Shape s,

@@ -473,15 +473,12 @@ __device__ __forceinline__ void store_rows32(uint8_t *buf, const uint32_t (&x)[3
 }  // namespace tc
 
 // Host side: encoders of the TMA tensor maps (tc_host.cu).  All maps use a box whose inner extent
-// is 128 bytes (64 16-bit or 32 32-bit elements) and the 128-byte swizzle.
+// is 128 bytes (64 16-bit elements) and the 128-byte swizzle.
 namespace tch {
 // Rows x cols matrix, row-major, `cols` a multiple of 64; box = box_rows x 64.
 bool make_map_2d(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols, uint32_t box_rows);
 // Tensor [B, L, H, d] (d contiguous); box = box_rows tokens x 64 elements of one (batch, head).
 bool make_map_blhd(CUtensorMap *m, const void *base, int B, int L, int H, int d, uint32_t box_rows);
-// The same tensor with fp32 elements: box = box_rows tokens x 32 elements (128 bytes) of one
-// (batch, head), 128-byte swizzle.
-bool make_map_blhd_f32(CUtensorMap *m, const void *base, int B, int L, int H, int d, uint32_t box_rows);
 }  // namespace tch
 
 }  // namespace natsl

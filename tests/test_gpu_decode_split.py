@@ -5,6 +5,7 @@ import pytest
 import torch
 
 import oracle
+from oracle import grouped
 from paper_2602_03681_b200 import inputs
 from test_gpu_parity import TOL, check_stored, dev, rel_err, tdtype
 
@@ -119,3 +120,61 @@ def test_decode_more_items_than_a_resident_set_can_list(cap):
     ref, o = _oracle_steps(wl, x, n)
     check_stored(got[0].float().cpu().numpy(), ref, TOL[wl.dtype], wl.dtype)
     assert np.array_equal(got[2].cpu().numpy(), o[3])
+
+
+def _grouped_step(x, n, state, kc, vc, G, scale_la, scale_sm, norm_eps, eps=1e-5):
+    """One step with normalised q, k and G softmax heads per linear head, from the definitions: out and new state."""
+    t = {m: torch.from_numpy(np.asarray(x[m][0], np.float64)) for m in ("q", "k", "v", "g", "beta", "w")}
+    route = torch.from_numpy(x["route"][0].astype(np.int64))
+    B, H, d = t["q"].shape
+    q, k = (grouped.l2_normalise(t[m], norm_eps) for m in ("q", "k"))
+    S = torch.exp(t["g"])[..., None, None] * torch.from_numpy(state)
+    fold = t["beta"] * (route != 1)
+    S = S + fold[..., None, None] * k[..., :, None] * (t["v"] - torch.einsum("bha,bhac->bhc", k, S))[..., None, :]
+    o_la = scale_la * torch.einsum("bha,bhac->bhc", q, S)
+    sl = lambda a: a.reshape(*a.shape[:-1], G, d // G)
+    keys = torch.cat([torch.from_numpy(kc), t["k"][:, :, None]], 2)          # the cache, then the token itself
+    values = torch.cat([torch.from_numpy(vc), t["v"][:, :, None]], 2)
+    logits = scale_sm * torch.einsum("bhsa,bhmsa->bhsm", grouped.rms_normalise(sl(t["q"]), norm_eps),
+                                     grouped.rms_normalise(sl(keys), norm_eps))
+    seen = torch.arange(keys.shape[2]) < torch.from_numpy(n.astype(np.int64))[..., None]
+    seen[..., -1] = route != 0
+    p = torch.softmax(logits.masked_fill(~seen[:, :, None], -torch.inf), -1).nan_to_num(0.0)   # (no key: zero)
+    o_nla = torch.einsum("bhsm,bhmsc->bhsc", p, sl(values))
+    rms = lambda a: a * torch.rsqrt((a * a).mean(-1, keepdim=True) + eps)
+    return (t["w"][..., :1] * rms(o_nla).reshape(B, H, d) + t["w"][..., 1:] * rms(o_la)).numpy(), S.numpy()
+
+
+@pytest.mark.parametrize("name,B,H,G,cap", [("cfg3_bf16_decode", 9, 12, 2, 500), ("cfg3_bf16_decode", 9, 12, 2, 4000),
+                                            ("cfg3_bf16_decode", 12, 8, 2, 1700), ("cfg4_bf16_train", 20, 15, 1, 280),
+                                            ("cfg0_f32_tiny_fwd", 20, 6, 2, 1000)])
+def test_decode_going_round_with_grouped_heads(name, B, H, G, cap):
+    """More pairs than a resident set holds (or long caches of nearly as many), softmax heads of their own and q, k
+    normalised as read; mixed lengths and routes."""
+    from paper_2602_03681_b200 import binding
+    wl = inputs.WORKLOADS[name]
+    most = min(cap - 1, 1600)
+    x = inputs.make_decode_inputs(wl, B=B, H=H, steps=1, ctx_retained=most, cap=most)
+    r = np.random.default_rng(3)
+    for m in ("q", "k"):
+        x[m] = (x[m] * np.exp(0.5 * r.standard_normal(x[m].shape[:-1] + (1,)))).astype(np.float32)
+        if wl.dtype == "bf16":
+            x[m] = inputs.round_bf16(x[m])
+    x["route"][...] = r.integers(0, 3, x["route"].shape)
+    n = np.resize(r.permutation([0, 1, 33, 299, 301, 600, 601, 1201, most]), B * H).reshape(B, H).clip(0, most).astype(np.int32)
+    scale_sm, dt = (wl.d // G) ** -0.5, tdtype(wl)
+    kc, vc = (torch.zeros((B, H, cap, wl.d), dtype=dt, device="cuda") for _ in range(2))
+    kc[:, :, :most], vc[:, :, :most] = dev(x["k_cache"], dt), dev(x["v_cache"], dt)
+    state, length, w = dev(x["state"]), dev(n), dev(x["w"][0])
+    p = binding.make_params(B, H, 0, wl.d, binding._dtype_code(kc), wl.scale_la, scale_sm, w=w, G=G, norm_eps=1e-6,
+                            flags=binding.QK_NORM)
+    ws = binding.alloc_workspace(p, binding.OP_DECODE)
+    out = torch.empty((B, H, wl.d), dtype=dt, device="cuda")
+    binding.natsl_decode_step(dev(x["q"][0], dt), dev(x["k"][0], dt), dev(x["v"][0], dt), dev(x["g"][0]),
+                              dev(x["beta"][0]), dev(x["route"][0]), state, kc, vc, length, out, p, ws)
+    assert binding.natsl_device_status(ws) == 0
+    ref, S = _grouped_step(x, n, x["state"].astype(np.float64), x["k_cache"].astype(np.float64),
+                           x["v_cache"].astype(np.float64), G, wl.scale_la, scale_sm, 1e-6)
+    check_stored(out.float().cpu().numpy(), ref, TOL[wl.dtype], wl.dtype)
+    assert rel_err(state.cpu().numpy(), S) <= 1e-4
+    assert np.array_equal(length.cpu().numpy(), n + (x["route"][0] != 0))

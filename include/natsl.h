@@ -110,8 +110,10 @@ enum {
                                     and on p->sm_cap.  Backward: NATSL_ERR_UNSUPPORTED */
     NATSL_SINGLE_STREAM = 1u << 4,     /* forward and backward, tensor-core path: launch everything on
                                     the caller's stream.  By default stages that do not depend on
-                                    each other run side by side: in the backward the reverse scan and
-                                    the key-side softmax kernel beside the query-side one, on a
+                                    each other run side by side: in the backward the reverse scan
+                                    beside the softmax branch's kernels -- followed by the chunk
+                                    kernel, or, with NATSL_BLOCK_ROUTING, by the key-side softmax
+                                    kernel and the scatter of its results -- on a
                                     stream the library creates once per device, forked from and
                                     joined to the caller's stream with events; in the forward (which
                                     stays on the caller's stream) as programmatic dependent launches.

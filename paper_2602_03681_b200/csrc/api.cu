@@ -91,8 +91,8 @@ bool scan_follows_closely(const natsl_params *p) { return (long long)p->B * p->H
 // against 2.1 with outputs) gains more than it costs: there are as many segments as keep its 2 nseg - 3 runs per pair
 // in one wave, at least 4 chunks long (shorter ones gain less than their step of the chain), and at least three --
 // with two the two passes are as long as one over everything.  32 pairs: 3 segments, 16: 6, 4: 20.
-// Where 32 comes from: three segments would fit one wave up to 49 pairs, but there the softmax kernel has the SMs that the
-// first pass takes.  Time of one pass over everything against segments, 2048 to 16384 tokens: 16 pairs of 128 columns
+// Where 32 comes from: three segments would fit one wave up to 49 pairs, but the softmax kernel, which runs beside the pass
+// with outputs, then starts a pass later.  Time of one pass over everything against segments, 2048 to 16384 tokens: 16 pairs of 128 columns
 // 1.19 to 1.48 with 5 % softmax tokens and 1.08 to 1.17 with 20 %, 24 pairs 1.01 to 1.17 and 0.89 to 0.99, 32 pairs 0.95 to
 // 1.06 and 0.85 to 0.94, 36 pairs (10 %) 0.90 to 0.92, 48 pairs 0.80 to 0.86; 64 columns 32 pairs 1.04 to 1.09 and 0.91 to
 // 1.02, 36 pairs (10 %) 0.92 to 1.02, 48 pairs 0.86 to 0.90.  The share of softmax tokens is not known here: the line is

@@ -64,8 +64,7 @@ HeadGroups head_groups(const natsl_params *p) {
 Shape shape_of(const natsl_params *p) { return Shape{p->B, p->H, p->L, p->d, p->dtype == NATSL_BF16}; }
 
 struct FwdWs {
-    int32_t *status, *emit_flags, *sm_idx, *prefix, *lin_idx, *n_lin, *sm_len;
-    size_t head_bytes;          // status page + emit_flags: cleared at the start of every call
+    int32_t *status, *emit_flags, *sm_idx, *prefix;
     void *k_sm, *v_sm, *v16;
     void *kn16;                 // prefill in pieces with NATSL_QK_NORM: normalised fp16 keys of the whole cache
     void *o_la16;               // tensor-core path: the linear read-out as fp16 [B,L,H,d]
@@ -120,13 +119,8 @@ FwdWs carve_fwd(const natsl_params *p, void *ws) {
     f.status = c.take<int32_t>(kStatusBytes / 4);
     // one counter per chunk, raised by the scan as the chunk's read-out is complete (tensor-core path)
     f.emit_flags = c.take<int32_t>(use_tensor_cores(p) ? B * H * NC : 0);
-    f.head_bytes = c.off;
     f.sm_idx = c.take<int32_t>(B * H * L);
     f.prefix = c.take<int32_t>(B * H * (NC + 1));
-    const bool simt = !use_tensor_cores(p);
-    f.lin_idx = c.take<int32_t>(simt ? B * H * L : 0);
-    f.n_lin = c.take<int32_t>(simt ? B * H * NC : 0);
-    f.sm_len = c.take<int32_t>(simt ? B * H : 0);
     f.k_sm = c.take<char>(B * H * L * d * esz);
     f.v_sm = c.take<char>(B * H * L * d * esz);
     if (use_tensor_cores(p)) {
@@ -553,10 +547,11 @@ int natsl_hybrid_fwd(const void *q, const void *k, const void *v, const float *g
         NATSL_TRY(mark());
         return NATSL_OK;
     }
-    NATSL_TRY(cudaMemsetAsync(f.status, 0, f.head_bytes, st));
+    // fp32 arithmetic: prepare | compaction + gather, beside it | scan, which waits for both, | softmax branch, beside the
+    // scan up to its epilogue.  With per-stage events: in sequence, in the order of the stages' names.
+    const bool beside = !p->stage_events;
     NATSL_TRY(mark());
-    NATSL_TRY(launch_route_compact(route, f.sm_idx, f.prefix, f.lin_idx, f.n_lin, want_cache ? p->sm_len : f.sm_len, nullptr,
-                                   block ? f.status : nullptr, cap, p->B, p->L, p->H, st));
+    if (!beside) NATSL_TRY(cudaMemsetAsync(f.status, 0, kStatusBytes, st));
     // NATSL_QK_NORM: normalised copies first
     const void *q_la = q, *k_la = k, *q_sm = q, *k_nsm = k;
     if (hg.norm_eps >= 0.f) {
@@ -564,16 +559,20 @@ int natsl_hybrid_fwd(const void *q, const void *k, const void *v, const float *g
                                      (size_t)p->B * p->L * p->H, p->d, hg.G, hg.norm_eps, st));
         q_la = f.q_la; k_la = f.k_la; q_sm = f.q_sm; k_nsm = f.k_nsm;
     }
-    if (raw_cache) NATSL_TRY(launch_gather_kv(k, v, f.sm_idx, f.prefix, k_sm, v_sm, cap, f.status, s, st));
-    NATSL_TRY(launch_gather_kv(k_nsm, v, f.sm_idx, f.prefix, raw_cache ? f.k_sm : k_sm,
-                               raw_cache ? f.v_sm : v_sm, cap_soft, f.status, s, st));
-    NATSL_TRY(mark());
     float *o_la = p->o_la ? p->o_la : f.o_la;
+    auto gather = [&]() {
+        const RowsJob soft{k_nsm, raw_cache ? f.k_sm : k_sm, raw_cache ? f.v_sm : v_sm, cap_soft};
+        return launch_route_gather_rows(route, v, soft, raw_cache ? RowsJob{k, k_sm, v_sm, cap} : RowsJob{}, f.sm_idx, f.prefix,
+                                        want_cache ? p->sm_len : nullptr, cap, f.status, block, s, st, beside);
+    };
+    if (!beside) NATSL_TRY(gather());
+    NATSL_TRY(mark());
     NATSL_TRY(launch_gdn_prepare_simt(q_la, k_la, v, g, beta, block ? nullptr : route, p->scale_la, f.W,
-                                      f.U, f.P, nullptr, nullptr, s, st));
+                                      f.U, f.P, nullptr, nullptr, s, st, beside ? f.status : nullptr, (int)(kStatusBytes / 4)));
+    if (beside) NATSL_TRY(gather());
     NATSL_TRY(mark());
     NATSL_TRY(launch_gdn_scan_simt(q_la, k_la, g, f.W, f.U, f.P, p->scale_la, p->state_in,
-                                   p->state_out, nullptr, nullptr, o_la, br.route, s, st));
+                                   p->state_out, nullptr, nullptr, o_la, br.route, s, st, scan_follows_closely(p)));
     NATSL_TRY(mark());
     // (an own-block tile of block-level routing reads the layer's keys: the softmax operation's copy)
     NATSL_TRY(launch_softmax_combine_simt(q_sm, k_soft, v_soft, cap_soft, f.sm_idx, f.prefix, o_la, p->w,

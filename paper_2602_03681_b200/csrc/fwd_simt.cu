@@ -22,126 +22,226 @@ constexpr int kThreads = 256;
 
 // Small calls (few (batch, head) pairs, a few hundred tokens) are what this path is used for most, and there every
 // kernel is a chain of latencies on a mostly idle chip: the kernels below cut their work finer when there is
-// little of it, keep operand tiles in rows of D + 4 floats (16-byte loads, free of bank conflicts when neighbouring
-// lanes take neighbouring rows), and are programmatic dependents of one another.
+// little of it, ask for their operands ahead of time by asynchronous copies, and are programmatic dependents of one another.
 
-// Load a 64 x D tile (token stride `ts` elements) into fp32 shared memory, rows of D + 4.
-template <typename T, int D>
+// 16 (or 4) bytes global -> shared, asynchronously; one group per commit.
+__device__ __forceinline__ void copy16_async(float *dst, const float *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy4_async(float *dst, const float *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// R x N tile (row stride `ts` elements) into fp32 shared memory, rows of LD floats: asynchronously from fp32, through
+// registers from bf16.
+template <int R, int N, int LD, typename T>
 __device__ __forceinline__ void load_tile(const T *__restrict__ src, size_t ts, float *dst) {
+    static_assert(R * N % (4 * kThreads) == 0, "whole pieces per thread");
 #pragma unroll 4
-    for (int idx = threadIdx.x; idx < kC * D / 4; idx += kThreads) {
-        const int r = idx / (D / 4), c4 = (idx % (D / 4)) * 4;
-        store4(dst + r * (D + 4) + c4, load4(src + (size_t)r * ts + c4));
+    for (int idx = threadIdx.x; idx < R * N / 4; idx += kThreads) {
+        const int r = idx / (N / 4), c4 = (idx % (N / 4)) * 4;
+        if constexpr (sizeof(T) == 4) copy16_async(dst + r * LD + c4, src + (size_t)r * ts + c4);
+        else store4(dst + r * LD + c4, load4(src + (size_t)r * ts + c4));
     }
 }
-// Inclusive prefix sum of 64 values in shared memory by one warp, in place.
-__device__ __forceinline__ void prefix64(float *x, int lane) {
+// Inclusive prefix sum of 64 values in shared memory by one warp.
+__device__ __forceinline__ void prefix64(const float *x, float *y, int lane) {
     const float a = x[2 * lane], b = x[2 * lane + 1];
     float s = a + b;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const float y = __shfl_up_sync(0xffffffffu, s, o);
-        if (lane >= o) s += y;
+        const float z = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += z;
     }
-    x[2 * lane + 1] = s;
-    x[2 * lane] = s - b;
+    y[2 * lane + 1] = s;
+    y[2 * lane] = s - b;
+}
+// acc (even and odd columns apart) += <a, b> over four columns
+__device__ __forceinline__ void fma4(ulonglong2 a, ulonglong2 b, uint64_t &acc) {
+    acc = tc::fma2(a.x, b.x, acc);
+    acc = tc::fma2(a.y, b.y, acc);
+}
+__device__ __forceinline__ ulonglong2 lds4(const float *p) { return *reinterpret_cast<const ulonglong2 *>(p); }
+__device__ __forceinline__ float both(uint64_t a) { const float2 x = tc::unpack2(a); return x.x + x.y; }
+
+// Sums of N values over W neighbouring lanes; lane w of them keeps values w N / W .. (the upper halves of the exchange
+// travel while the lower ones are kept, so this takes N (1 - 1 / W) shuffles instead of N log2 W).
+template <int N, int W>
+__device__ __forceinline__ void sum_lanes(float (&x)[N]) {
+    int n = N;
+#pragma unroll
+    for (int m = W / 2; m > 0; m >>= 1) {
+        n /= 2;
+        const bool up = threadIdx.x & m;
+#pragma unroll
+        for (int e = 0; e < N; ++e)
+            if (e < n) {
+                const float keep = up ? x[n + e] : x[e], give = up ? x[e] : x[n + e];
+                x[e] = keep + __shfl_xor_sync(0xffffffffu, give, m);
+            }
+    }
 }
 
 // ------------------------------------------------------------------------------------------
-// Prepare: state-independent per-chunk quantities.  grid = (L/C, B*H).  K K^T and Q K^T together, 4 x 4 outputs of each
-// per thread; then one right-hand-side column per thread, updated from the left as its entries become known
-// (independent FMAs; a dot product per entry was a serial chain of 2016).
+// Prepare: state-independent per-chunk quantities.  grid = (kParts L/C, B*H): a chunk's right-hand sides (D columns of
+// W, D of U) are cut into kParts, each CTA forms all of A and its share of P's rows.  Four parts when there are few
+// chunks, one otherwise (A is then formed once).  K K^T and Q K^T: 4 x 4 outputs of each per thread, packed FMAs along
+// the columns.  Substitution in blocks of 16 rows: one thread per column solves the block's rows (in registers), then
+// all threads subtract its products from the rows below -- a loop that runs four times over one block's code.
+// (One thread per column over all 64 rows was 2016 unrolled FMAs that run once: 40 KB of code, and its warps waited for
+// instructions.  Eight chunks of 64 columns: 19.2 us by itself, 10.5 now.)
 // ------------------------------------------------------------------------------------------
-template <typename T, int D>
+template <int D, int kParts> struct SimtPrep {
+    static constexpr int LD = D + 4, LA = kC + 4;
+    static constexpr int kCols = 2 * D / kParts, LX = kCols + 4;         // right-hand-side columns of a CTA
+    static constexpr int kPRows = kC / kParts;                           // rows of P
+    static constexpr int oK = 0, oQ = oK + kC * LD, oX = oQ + kPRows * LD, oA = oX + kC * LX, oG = oA + kC * LA;
+    static constexpr int kBytes = (oG + 3 * kC) * 4;
+};
+
+template <typename T, int D, int kParts>
 __global__ void __launch_bounds__(kThreads)
 gdn_prepare_simt_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v,
                         const float *__restrict__ g, const float *__restrict__ beta,
                         const uint8_t *__restrict__ route, float scale_la, float *__restrict__ W,
                         float *__restrict__ U, float *__restrict__ P, float *__restrict__ Abar,
-                        float *__restrict__ Gcum, int L, int H) {
-    constexpr int LD = D + 4, LA = kC + 4;
+                        float *__restrict__ Gcum, int32_t *clear, int clear_words, int L, int H) {
+    using SP = SimtPrep<D, kParts>;
+    constexpr int LD = SP::LD, LA = SP::LA, LX = SP::LX, kCols = SP::kCols, kPE = SP::kPRows / 16;
     extern __shared__ __align__(16) float smem[];
-    float *Ks = smem;                       // [64][LD]
-    float *Vs = Ks + kC * LD;               // [64][LD]
-    float *Qs = Vs + kC * LD;               // [64][LD]
-    float *At = Qs + kC * LD;               // [64][LA]: column j of A
-    float *Gs = At + kC * LA;               // [64] inclusive cumulative log decay
-    float *bts = Gs + kC;                   // [64] beta~
+    float *Ks = smem + SP::oK;              // [64][LD]
+    float *Qs = smem + SP::oQ;              // [kPRows][LD]
+    float *Xs = smem + SP::oX;              // [64][LX]: right-hand sides, then the solution
+    float *At = smem + SP::oA;              // [64][LA]: column j of A
+    float *Gs = smem + SP::oG;              // [64] inclusive cumulative log decay
+    float *bts = Gs + kC, *raw = bts + kC;  // [64] beta~; [64] log decay
 
-    const int c = blockIdx.x, bh = blockIdx.y, b = bh / H, h = bh % H;
+    const int c = blockIdx.x / kParts, part = blockIdx.x % kParts, bh = blockIdx.y, b = bh / H, h = bh % H;
+    const int tid = threadIdx.x;
     const size_t ts = (size_t)H * D;
     const size_t tok0 = ((size_t)b * L + (size_t)c * kC) * H + h;  // index of the chunk's first token
     tc::grid_dependency_wait();
+    // (the forward's first kernel: clears the status page, before any kernel behind this one can report into it)
+    if (clear && blockIdx.x == 0 && blockIdx.y == 0 && tid < clear_words) clear[tid] = 0;
+    __threadfence();
     tc::launch_dependents();
 
-    load_tile<T, D>(k + tok0 * D, ts, Ks);
-    load_tile<T, D>(q + tok0 * D, ts, Qs);
-    load_tile<T, D>(v + tok0 * D, ts, Vs);
-    if (threadIdx.x < kC) {
-        const size_t t = tok0 + (size_t)threadIdx.x * H;
-        bts[threadIdx.x] = route && route[t] ? 0.f : beta[t];   // route == nullptr: beta~ = beta
-        Gs[threadIdx.x] = g[t];
+    const bool hasW = part * kCols < D, hasU = (part + 1) * kCols > D;   // (one part: both; several: one of them)
+    load_tile<kC, D, LD>(k + tok0 * D, ts, Ks);
+    load_tile<SP::kPRows, D, LD>(q + tok0 * D + (size_t)(part * SP::kPRows) * ts, ts, Qs);
+    constexpr int kVCols = kParts == 1 ? D : kCols;
+    if (hasU) load_tile<kC, kVCols, LX>(v + tok0 * D + (kParts == 1 ? 0 : part * kCols - D), ts, Xs + (kParts == 1 ? D : 0));
+    if (tid < kC) {
+        const size_t t = tok0 + (size_t)tid * H;
+        bts[tid] = route && route[t] ? 0.f : beta[t];   // route == nullptr: beta~ = beta
+        raw[tid] = g[t];
     }
+    copies_wait();
     __syncthreads();
-    if (threadIdx.x < 32) prefix64(Gs, threadIdx.x);
-    __syncthreads();
-    if (Gcum && threadIdx.x < kC) Gcum[(size_t)bh * L + c * kC + threadIdx.x] = Gs[threadIdx.x];
+    if (tid < 32) prefix64(raw, Gs, tid);
     // A (strictly lower), Abar = A without the beta~ row factor (the backward needs it), and
     // P = scale_la (Q K^T) . Gamma, lower triangle including the diagonal.  Thread: rows ti + 16 e, columns tj + 16 e.
     {
-        const int ti = threadIdx.x >> 4, tj = threadIdx.x & 15;
-        float a[4][4] = {}, pq[4][4] = {};
+        const int ti = tid >> 4, tj = tid & 15;
+        uint64_t a[4][4], pq[kPE][4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+#pragma unroll
+            for (int ei = 0; ei < 4; ++ei) a[ei][e] = 0ull;
+#pragma unroll
+            for (int ei = 0; ei < kPE; ++ei) pq[ei][e] = 0ull;
+        }
 #pragma unroll 2
         for (int x = 0; x < D; x += 4) {
-            float4 kj[4];
+            ulonglong2 kj[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) kj[e] = *reinterpret_cast<const float4 *>(Ks + (tj + 16 * e) * LD + x);
+            for (int e = 0; e < 4; ++e) kj[e] = lds4(Ks + (tj + 16 * e) * LD + x);
 #pragma unroll
             for (int ei = 0; ei < 4; ++ei) {
-                const float4 ki = *reinterpret_cast<const float4 *>(Ks + (ti + 16 * ei) * LD + x);
-                const float4 qi = *reinterpret_cast<const float4 *>(Qs + (ti + 16 * ei) * LD + x);
+                const ulonglong2 ki = lds4(Ks + (ti + 16 * ei) * LD + x);
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    a[ei][e] = fmaf(ki.x, kj[e].x, fmaf(ki.y, kj[e].y, fmaf(ki.z, kj[e].z, fmaf(ki.w, kj[e].w, a[ei][e]))));
-                    pq[ei][e] = fmaf(qi.x, kj[e].x, fmaf(qi.y, kj[e].y, fmaf(qi.z, kj[e].z, fmaf(qi.w, kj[e].w, pq[ei][e]))));
-                }
+                for (int e = 0; e <= ei; ++e) fma4(ki, kj[e], a[ei][e]);
+            }
+#pragma unroll
+            for (int ei = 0; ei < kPE; ++ei) {
+                const ulonglong2 qi = lds4(Qs + (ti + 16 * ei) * LD + x);
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (kParts > 1 || e <= ei) fma4(qi, kj[e], pq[ei][e]);
             }
         }
+        __syncthreads();                      // the cumulative decays are there
         const size_t cc = ((size_t)bh * (L / kC) + c) * kC * kC;
 #pragma unroll
         for (int ei = 0; ei < 4; ++ei)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int i = ti + 16 * ei, j = tj + 16 * e;
-                const float gam = j <= i ? __expf(Gs[i] - Gs[j]) : 0.f;
-                const float av = j < i ? gam * a[ei][e] : 0.f;
-                if (Abar) Abar[cc + i * kC + j] = av;
+                const float av = j < i ? __expf(Gs[i] - Gs[j]) * both(a[ei][e]) : 0.f;
+                if (Abar && part == 0) Abar[cc + i * kC + j] = av;
                 At[j * LA + i] = bts[i] * av;
-                P[cc + i * kC + j] = scale_la * gam * pq[ei][e];
             }
+#pragma unroll
+        for (int ei = 0; ei < kPE; ++ei)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int i = part * SP::kPRows + ti + 16 * ei, j = tj + 16 * e;
+                P[cc + i * kC + j] = j <= i ? scale_la * __expf(Gs[i] - Gs[j]) * both(pq[ei][e]) : 0.f;
+            }
+        if (Gcum && part == 0 && tid < kC) Gcum[(size_t)bh * L + c * kC + tid] = Gs[tid];
     }
+    // right-hand sides: beta~ gamma K, beta~ V
+    constexpr int kTpc = kThreads / kCols;            // threads per column
+    const int col = tid % kCols, sub = tid / kCols;
+    const bool isW = kParts == 1 ? col < D : hasW;
+    const int dcol = (part * kCols + col) % D;         // column of W or U
+    for (int i = sub; i < kC; i += kTpc)
+        Xs[i * LX + col] = bts[i] * (isW ? __expf(Gs[i]) * Ks[i * LD + dcol] : Xs[i * LX + col]);
     __syncthreads();
-    // Forward substitution, one right-hand-side column per thread: columns [0,D) give W, [D,2D) U.
-    if (threadIdx.x < 2 * D) {
-        const bool isW = threadIdx.x < D;
-        const int col = isW ? threadIdx.x : threadIdx.x - D;
-        const float *src = isW ? Ks : Vs;
-        float x[kC];
+    float *dst = (isW ? W : U) + tok0 * D + dcol;
+#pragma unroll 1
+    for (int r0 = 0; r0 < kC; r0 += 16) {
+        if (sub == 0) {
+            float x[16];
 #pragma unroll
-        for (int i = 0; i < kC; ++i) x[i] = bts[i] * (isW ? __expf(Gs[i]) : 1.f) * src[i * LD + col];
+            for (int i = 0; i < 16; ++i) x[i] = Xs[(r0 + i) * LX + col];
 #pragma unroll
-        for (int j = 0; j < kC - 1; ++j)
+            for (int j = 0; j < 15; ++j)
 #pragma unroll
-            for (int i4 = (j + 1) / 4; i4 < kC / 4; ++i4) {
-                const float4 aj = *reinterpret_cast<const float4 *>(At + j * LA + 4 * i4);   // (zero for i <= j)
-                if (4 * i4 > j) x[4 * i4] = fmaf(-aj.x, x[j], x[4 * i4]);
-                if (4 * i4 + 1 > j) x[4 * i4 + 1] = fmaf(-aj.y, x[j], x[4 * i4 + 1]);
-                if (4 * i4 + 2 > j) x[4 * i4 + 2] = fmaf(-aj.z, x[j], x[4 * i4 + 2]);
-                if (4 * i4 + 3 > j) x[4 * i4 + 3] = fmaf(-aj.w, x[j], x[4 * i4 + 3]);
+                for (int i4 = (j + 1) / 4; i4 < 4; ++i4) {
+                    const float4 aj = *reinterpret_cast<const float4 *>(At + (r0 + j) * LA + r0 + 4 * i4);   // (zero for i <= j)
+                    if (4 * i4 > j) x[4 * i4] = fmaf(-aj.x, x[j], x[4 * i4]);
+                    if (4 * i4 + 1 > j) x[4 * i4 + 1] = fmaf(-aj.y, x[j], x[4 * i4 + 1]);
+                    if (4 * i4 + 2 > j) x[4 * i4 + 2] = fmaf(-aj.z, x[j], x[4 * i4 + 2]);
+                    if (4 * i4 + 3 > j) x[4 * i4 + 3] = fmaf(-aj.w, x[j], x[4 * i4 + 3]);
+                }
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                Xs[(r0 + i) * LX + col] = x[i];
+                dst[(size_t)(r0 + i) * ts] = x[i];
             }
-        float *dst = (isW ? W : U) + tok0 * D + col;
+        }
+        __syncthreads();
+        if (r0 + 16 < kC) {
+            float x[16];
 #pragma unroll
-        for (int i = 0; i < kC; ++i) dst[(size_t)i * ts] = x[i];
+            for (int j = 0; j < 16; ++j) x[j] = Xs[(r0 + j) * LX + col];
+            for (int i = r0 + 16 + 4 * sub; i < kC; i += 4 * kTpc) {
+                float y[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) y[e] = Xs[(i + e) * LX + col];
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const float4 aj = *reinterpret_cast<const float4 *>(At + (r0 + j) * LA + i);
+                    y[0] = fmaf(-aj.x, x[j], y[0]); y[1] = fmaf(-aj.y, x[j], y[1]);
+                    y[2] = fmaf(-aj.z, x[j], y[2]); y[3] = fmaf(-aj.w, x[j], y[3]);
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) Xs[(i + e) * LX + col] = y[e];
+            }
+            __syncthreads();
+        }
     }
 }
 
@@ -149,7 +249,23 @@ gdn_prepare_simt_kernel(const T *__restrict__ q, const T *__restrict__ k, const 
 // Scan: sequential over chunks, one CTA per (batch, head, slice of NV value columns), grid = (D/NV, B*H).  NV = 8
 // when slices of 32 would leave most of the chip idle: a chunk's step is a chain, and four times shorter for it;
 // with many (batch, head) pairs the wider slice reads the chunk's operands a quarter as often.
+// What bounds a step is latency, so the next chunk's operands travel while this one is worked on (K, P, U, g and, where
+// they fit twice, W and Q from the step's start; else W and Q from its middle), and the products have as much reuse
+// per load as 256 threads allow: 2 rows x 4 columns (U~ and q S; P U~) or 4 x 4 (state) per thread, the sum over the inner
+// index split over neighbouring lanes.  Row lengths are such that the lanes' 16-byte loads fall on different banks.
+// (Loading at the step's start and one row x two columns per thread: 33 us for 16 CTAs of four chunks, 13.8 now.)
 // ------------------------------------------------------------------------------------------
+template <int D, int NV> struct SimtScan {
+    static constexpr int kPad = NV == 8 ? 16 : 4;        // rows 64 bytes apart for 4 x 4 lanes (row, quarter), 16 for 32 rows
+    static constexpr int LD = D + kPad, LK = D + 4, LP = kC + kPad, LU = kC + kPad;
+    static constexpr int kTwice = D == 64 ? 2 : 1;       // W and Q buffers
+    static constexpr int oS = 0, oW = oS + NV * LD, oQ = oW + kTwice * kC * LD, oK = oQ + kTwice * kC * LD,
+                         oP = oK + 2 * kC * LK, oU = oP + 2 * kC * LP, oUs = oU + 2 * kC * NV, oUt = oUs + kC * NV,
+                         oG = oUt + NV * LU;
+    static constexpr int kBytes = (oG + 5 * kC) * 4;
+    static_assert(kBytes <= 227 * 1024, "shared memory of a CTA");
+};
+
 template <typename T, int D, int NV>
 __global__ void __launch_bounds__(kThreads)
 gdn_scan_simt_kernel(const T *__restrict__ q, const T *__restrict__ k, const float *__restrict__ g,
@@ -158,290 +274,401 @@ gdn_scan_simt_kernel(const T *__restrict__ q, const T *__restrict__ k, const flo
                      float *__restrict__ state_out, float *__restrict__ chunk_states,
                      float *__restrict__ Ut, float *__restrict__ o_la,
                      const uint8_t *__restrict__ block_route, int L, int H) {
-    constexpr int LD = D + 4, LP = kC + 4;
-    constexpr int kN = NV / 4;               // columns per thread of a [64][NV] result: four threads per row
+    using SS = SimtScan<D, NV>;
+    constexpr int LD = SS::LD, LK = SS::LK, LP = SS::LP, LU = SS::LU;
+    constexpr int kCg = NV / 4;                          // column groups: a thread's columns are cg + kCg {0 .. 3}
+    constexpr int kW1 = kThreads / (32 * kCg);           // lanes that share a 2 x 4 tile
+    constexpr int kRw = kW1 == 1 ? 2 : 1, kCl = kW1 == 1 ? 4 : 2;       // rows x columns a lane keeps of it
+    static_assert(kW1 == 1 || kW1 == 4, "NV = 8 or 32");
     extern __shared__ __align__(16) float smem[];
-    float *Ss = smem;                        // [D][NV]
-    float *Ws = Ss + D * NV;                 // [64][LD]
-    float *Qs = Ws + kC * LD;                // [64][LD]
-    float *Ks = Qs + kC * LD;                // [64][LD]
-    float *Ps = Ks + kC * LD;                // [64][LP]
-    float *Us = Ps + kC * LP;                // [64][NV]
-    float *Gs = Us + kC * NV;                // [64] cumulative log decay
-    float *e1 = Gs + kC, *e2 = e1 + kC;      // [64] scale_la gamma_i; [64] gamma_C / gamma_i
+    float *Ss = smem + SS::oS;                           // [NV][LD]: value columns of the state
+    float *Us = smem + SS::oUs, *Uts = smem + SS::oUt;   // U~: [64][NV] and [NV][LU]
+    float *raw = smem + SS::oG;                          // [2][64] log decay
+    float *Gs = raw + 2 * kC;                            // [64] cumulative
+    float *e1 = Gs + kC, *e2 = e1 + kC;                  // [64] scale_la gamma_i; [64] gamma_C / gamma_i
 
-    const int slice = blockIdx.x, bh = blockIdx.y, b = bh / H, h = bh % H;
+    const int slice = blockIdx.x, bh = blockIdx.y, b = bh / H, h = bh % H, tid = threadIdx.x;
     const int NC = L / kC;
     const size_t ts = (size_t)H * D;
     const int c0 = slice * NV;
     tc::grid_dependency_wait();
     tc::launch_dependents();
 
-    for (int idx = threadIdx.x; idx < D * NV; idx += kThreads) {
-        const int a = idx / NV, cc = idx % NV;
-        Ss[idx] = state_in ? state_in[((size_t)bh * D + a) * D + c0 + cc] : 0.f;
-    }
-    auto fma_n = [](float (&acc)[kN], float f, const float *s) {      // acc += f s[0 .. kN)
-        if constexpr (kN == 2) {
-            const float2 y = *reinterpret_cast<const float2 *>(s);
-            acc[0] = fmaf(f, y.x, acc[0]);
-            acc[1] = fmaf(f, y.y, acc[1]);
-        } else {
-#pragma unroll
-            for (int x = 0; x < kN; x += 4) {
-                const float4 y = *reinterpret_cast<const float4 *>(s + x);
-                acc[x] = fmaf(f, y.x, acc[x]); acc[x + 1] = fmaf(f, y.y, acc[x + 1]);
-                acc[x + 2] = fmaf(f, y.z, acc[x + 2]); acc[x + 3] = fmaf(f, y.w, acc[x + 3]);
-            }
-        }
+    auto first_token = [&](int c) { return ((size_t)b * L + (size_t)c * kC) * H + h; };
+    auto fetch_wq = [&](int c) {
+        const size_t at = first_token(c) * D, o = (c % SS::kTwice) * kC * LD;
+        load_tile<kC, D, LD>(W + at, ts, smem + SS::oW + o);
+        load_tile<kC, D, LD>(q + at, ts, smem + SS::oQ + o);
     };
+    auto fetch_rest = [&](int c) {
+        const size_t tok0 = first_token(c);
+        const int o = c & 1;
+        load_tile<kC, D, LK>(k + tok0 * D, ts, smem + SS::oK + o * kC * LK);
+        load_tile<kC, kC, LP>(P + ((size_t)bh * NC + c) * kC * kC, kC, smem + SS::oP + o * kC * LP);
+        for (int idx = tid; idx < kC * kCg; idx += kThreads)
+            copy16_async(smem + SS::oU + (o * kC + idx / kCg) * NV + idx % kCg * 4,
+                         U + (tok0 + (size_t)(idx / kCg) * H) * D + c0 + idx % kCg * 4);
+        if (tid < kC) copy4_async(raw + o * kC + tid, g + tok0 + (size_t)tid * H);
+    };
+    fetch_wq(0);
+    fetch_rest(0);
+    for (int idx = tid; idx < D * NV; idx += kThreads) {
+        const int a = idx / NV, cc = idx % NV;
+        Ss[cc * LD + a] = state_in ? state_in[((size_t)bh * D + a) * D + c0 + cc] : 0.f;
+    }
+    // 2 x 4 tiles: rows rp and rp + 32, columns cg + kCg {0 .. 3}; lane w1 of the tile's keeps, of the sums, row
+    // r and the kCl columns from cc0 on (or, alone, all of it)
+    const int w1 = tid % kW1, cg = tid / kW1 % kCg, rp = tid / (kW1 * kCg);
+    const int r0 = kW1 == 1 ? rp : rp + 32 * (w1 >> 1), cc0 = kW1 == 1 ? 0 : 2 * (w1 & 1);
     for (int c = 0; c < NC; ++c) {
-        const size_t tok0 = ((size_t)b * L + (size_t)c * kC) * H + h;
+        const size_t tok0 = first_token(c);
+        const float *Ws = smem + SS::oW + (c % SS::kTwice) * kC * LD, *Qs = smem + SS::oQ + (c % SS::kTwice) * kC * LD;
+        const float *Ks = smem + SS::oK + (c & 1) * kC * LK, *Ps = smem + SS::oP + (c & 1) * kC * LP;
+        const float *Uin = smem + SS::oU + (c & 1) * kC * NV;
+        copies_wait();
         __syncthreads();
+        if (c + 1 < NC) {
+            if (SS::kTwice == 2) fetch_wq(c + 1);
+            fetch_rest(c + 1);
+        }
         if (chunk_states) {  // state at chunk entry, [B,H,NC,D,D]
-            for (int idx = threadIdx.x; idx < D * NV; idx += kThreads) {
+            for (int idx = tid; idx < D * NV; idx += kThreads) {
                 const int a = idx / NV, cc = idx % NV;
-                chunk_states[(((size_t)bh * NC + c) * D + a) * D + c0 + cc] = Ss[idx];
+                chunk_states[(((size_t)bh * NC + c) * D + a) * D + c0 + cc] = Ss[cc * LD + a];
             }
         }
-        if (threadIdx.x < kC) Gs[threadIdx.x] = g[tok0 + (size_t)threadIdx.x * H];
-        load_tile<float, D>(W + tok0 * D, ts, Ws);
-        load_tile<T, D>(q + tok0 * D, ts, Qs);
-        load_tile<T, D>(k + tok0 * D, ts, Ks);
-        {
-            const float *Pc = P + ((size_t)bh * NC + c) * kC * kC;
-            for (int idx = threadIdx.x; idx < kC * kC / 4; idx += kThreads)
-                store4(Ps + (idx >> 4) * LP + (idx & 15) * 4, load4(Pc + 4 * idx));
-            for (int idx = threadIdx.x; idx < kC * NV; idx += kThreads)
-                Us[idx] = U[(tok0 + (size_t)(idx / NV) * H) * D + c0 + idx % NV];
-        }
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            prefix64(Gs, threadIdx.x);
+        if (tid < 32) {
+            prefix64(raw + (c & 1) * kC, Gs, tid);
             __syncwarp();
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
-                const int i = threadIdx.x + 32 * u;
+                const int i = tid + 32 * u;
                 e1[i] = scale_la * __expf(Gs[i]);
                 e2[i] = __expf(Gs[kC - 1] - Gs[i]);
             }
         }
-        const int r = threadIdx.x >> 2, cb = (threadIdx.x & 3) * kN;
-        // U~ = U - W S, and q S while the state's rows pass by
-        float qs[kN], ut[kN];
+        // U~ = U - W S, and q S while the state's columns pass by
+        float qs[kRw * kCl];
+        {
+            uint64_t acc[2][4][2];                        // [row][column][W S, q S]
 #pragma unroll
-        for (int x = 0; x < kN; ++x) { qs[x] = 0.f; ut[x] = Us[r * NV + cb + x]; }
+            for (int e = 0; e < 2; ++e)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) acc[e][x][0] = acc[e][x][1] = 0ull;
 #pragma unroll 4
-        for (int a = 0; a < D; a += 4) {
-            const float4 wv = *reinterpret_cast<const float4 *>(Ws + r * LD + a);
-            const float4 qv = *reinterpret_cast<const float4 *>(Qs + r * LD + a);
-            const float *sr = Ss + a * NV + cb;
-            fma_n(ut, -wv.x, sr); fma_n(ut, -wv.y, sr + NV); fma_n(ut, -wv.z, sr + 2 * NV); fma_n(ut, -wv.w, sr + 3 * NV);
-            fma_n(qs, qv.x, sr); fma_n(qs, qv.y, sr + NV); fma_n(qs, qv.z, sr + 2 * NV); fma_n(qs, qv.w, sr + 3 * NV);
-        }
+            for (int a = 4 * w1; a < D; a += 4 * kW1) {
+                ulonglong2 sv[4];
 #pragma unroll
-        for (int x = 0; x < kN; ++x) Us[r * NV + cb + x] = ut[x];      // (read and written by this thread only so far)
-        if (Ut) {
-            float *dst = Ut + (tok0 + (size_t)r * H) * D + c0 + cb;
+                for (int x = 0; x < 4; ++x) sv[x] = lds4(Ss + (cg + kCg * x) * LD + a);
 #pragma unroll
-            for (int x = 0; x < kN; ++x) dst[x] = ut[x];
-        }
-        __syncthreads();
-        // O = scale_la gamma_r q_r S + sum_{j<=r} P_rj U~_j   (P is zero above the diagonal)
-        {
-            const float gs = e1[r];
+                for (int e = 0; e < 2; ++e) {
+                    const ulonglong2 wv = lds4(Ws + (rp + 32 * e) * LD + a), qv = lds4(Qs + (rp + 32 * e) * LD + a);
 #pragma unroll
-            for (int x = 0; x < kN; ++x) qs[x] *= gs;
-            const int jn = (r | 7) + 1;               // (rows of a warp are neighbours: one bound for all of them)
-#pragma unroll 2
-            for (int j = 0; j < jn; j += 4) {
-                const float4 pv = *reinterpret_cast<const float4 *>(Ps + r * LP + j);
-                const float *ur = Us + j * NV + cb;
-                fma_n(qs, pv.x, ur); fma_n(qs, pv.y, ur + NV); fma_n(qs, pv.z, ur + 2 * NV); fma_n(qs, pv.w, ur + 3 * NV);
-            }
-            float *dst = o_la + (tok0 + (size_t)r * H) * D + c0 + cb;
-#pragma unroll
-            for (int x = 0; x < kN; ++x) dst[x] = qs[x];
-        }
-        // S <- gamma_C S + (diag(gamma_C / gamma) K)^T U~  (nobody reads S any more)
-        {
-            constexpr int kOut = D * NV / kThreads;   // outputs per thread, of one state row
-            constexpr int kTpr = NV / kOut;           // threads per state row
-            const int a = threadIdx.x / kTpr, cs = (threadIdx.x % kTpr) * kOut;
-            const float gC = __expf(Gs[kC - 1]);
-            float acc[kOut];
-#pragma unroll
-            for (int x = 0; x < kOut; ++x) acc[x] = 0.f;
-            // block-level routing: a softmax block's update is not committed, the state only decays
-            if (!(block_route && block_route[tok0])) {
-#pragma unroll 8
-                for (int j = 0; j < kC; ++j) {
-                    const float kv = Ks[j * LD + a] * e2[j];
-#pragma unroll
-                    for (int x = 0; x < kOut; ++x) acc[x] = fmaf(kv, Us[j * NV + cs + x], acc[x]);
+                    for (int x = 0; x < 4; ++x) { fma4(wv, sv[x], acc[e][x][0]); fma4(qv, sv[x], acc[e][x][1]); }
                 }
             }
+            float sum[16];
 #pragma unroll
-            for (int x = 0; x < kOut; ++x) Ss[a * NV + cs + x] = fmaf(gC, Ss[a * NV + cs + x], acc[x]);
+            for (int e = 0; e < 16; ++e) sum[e] = both(acc[e >> 3][(e >> 1) & 3][e & 1]);
+            sum_lanes<16, kW1>(sum);
+#pragma unroll
+            for (int e = 0; e < kRw; ++e)
+#pragma unroll
+                for (int x = 0; x < kCl; ++x) {
+                    const int r = r0 + 32 * e, cc = cg + kCg * (cc0 + x);
+                    const float u = Uin[r * NV + cc] - sum[2 * (kCl * e + x)];
+                    qs[kCl * e + x] = sum[2 * (kCl * e + x) + 1];
+                    Us[r * NV + cc] = u;
+                    Uts[cc * LU + r] = u;
+                    if (Ut) Ut[(tok0 + (size_t)r * H) * D + c0 + cc] = u;
+                }
+        }
+        __syncthreads();
+        if (SS::kTwice == 1 && c + 1 < NC) fetch_wq(c + 1);
+        // O = scale_la gamma_r q_r S + sum_{j<=r} P_rj U~_j   (P is zero above the diagonal)
+        {
+            uint64_t acc[2][4];
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) acc[e][x] = 0ull;
+#pragma unroll 4
+            for (int j = 4 * w1; j < kC; j += 4 * kW1) {
+                const ulonglong2 p1 = lds4(Ps + (rp + 32) * LP + j), p0 = lds4(Ps + rp * LP + j);
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const ulonglong2 uv = lds4(Uts + (cg + kCg * x) * LU + j);
+                    if (j < 32) fma4(p0, uv, acc[0][x]);
+                    fma4(p1, uv, acc[1][x]);
+                }
+            }
+            float sum[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) sum[e] = both(acc[e >> 2][e & 3]);
+            sum_lanes<8, kW1>(sum);
+#pragma unroll
+            for (int e = 0; e < kRw; ++e)
+#pragma unroll
+                for (int x = 0; x < kCl; ++x) {
+                    const int r = r0 + 32 * e;
+                    o_la[(tok0 + (size_t)r * H) * D + c0 + cg + kCg * (cc0 + x)] = fmaf(e1[r], qs[kCl * e + x], sum[kCl * e + x]);
+                }
+        }
+        // S <- gamma_C S + (diag(gamma_C / gamma) K)^T U~  (nobody reads S any more); 4 keys x 4 columns per tile
+        {
+            constexpr int kTiles = D * NV / 16, kW3 = kThreads / kTiles, kKeep = 16 / kW3;
+            const int w3 = tid % kW3, tile = tid / kW3, c4 = tile % kCg * 4, a4 = tile / kCg * 4;
+            float acc[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) acc[e] = 0.f;
+            // block-level routing: a softmax block's update is not committed, the state only decays
+            if (!(block_route && block_route[tok0])) {
+#pragma unroll 4
+                for (int j = w3; j < kC; j += kW3) {
+                    const float4 kv = *reinterpret_cast<const float4 *>(Ks + j * LK + a4);
+                    const float4 uv = *reinterpret_cast<const float4 *>(Us + j * NV + c4);
+                    const float f = e2[j];
+                    const float ka[4] = {kv.x * f, kv.y * f, kv.z * f, kv.w * f}, uu[4] = {uv.x, uv.y, uv.z, uv.w};
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) acc[e] = fmaf(ka[e & 3], uu[e >> 2], acc[e]);
+                }
+                sum_lanes<16, kW3>(acc);
+            }
+            const float gC = __expf(Gs[kC - 1]);
+#pragma unroll
+            for (int e = 0; e < kKeep; ++e) {
+                const int at = w3 * kKeep + e;
+                float *sp = Ss + (c4 + (at >> 2)) * LD + a4 + (at & 3);
+                *sp = fmaf(gC, *sp, acc[e]);
+            }
         }
     }
     __syncthreads();
     if (state_out) {
-        for (int idx = threadIdx.x; idx < D * NV; idx += kThreads) {
+        for (int idx = tid; idx < D * NV; idx += kThreads) {
             const int a = idx / NV, cc = idx % NV;
-            state_out[((size_t)bh * D + a) * D + c0 + cc] = Ss[idx];
+            state_out[((size_t)bh * D + a) * D + c0 + cc] = Ss[cc * LD + a];
         }
     }
 }
 
 // ------------------------------------------------------------------------------------------
 // Softmax branch over the retained tokens (Section 4.1, O_nla with mask M^nla) with the
-// combination (Section 4.3, Norm equation) as epilogue.  grid = (L/(8 NQ), B*H*G); each warp owns NQ query rows --
-// 8, or 2 when blocks of 64 queries would leave most of the chip idle --, each lane one key of the current
-// 32-key tile, whose pieces are read once for all of the warp's rows.
+// combination (Section 4.3, Norm equation) as epilogue.  grid = (L/(16 kR), B*H*G): 64 query rows per CTA, or 16 when
+// blocks of 64 would leave most of the chip idle.  A half warp owns kR rows: lane kk of it the logits of keys kk and kk + 16 of
+// a 32-key tile, and D / 16 columns of the rows' sums; probabilities pass between its lanes through shared memory.  The next
+// tile's keys and values travel while this one is worked on.  A programmatic dependent of the scan: the tiles
+// are worked on beside it, the epilogue waits for it.
+// (A row's logits over 32 lanes and a shuffle per probability kept the shuffle unit, not the FMAs, busy: 72 us for
+// 16 pairs of 1024 tokens of 64 columns by itself, 48.5 now; 485 -> 315 at 4096 tokens.)
 // G softmax heads per linear head (Section 4.3, grouped heads): softmax head (h, sg) works on the
 // columns [sg D, (sg+1) D) of q, k, v rows of DL = G D columns; lists, weights and the linear read-out
 // are those of linear head h; the softmax output is normalised over its D columns, the linear
 // read-out over all DL, and the CTA writes its D columns of `out`.  lse is [B,H,G,L].
 // ------------------------------------------------------------------------------------------
-template <typename T, int D, int G, int NQ>
+template <int D, int kR> struct SimtSoft {
+    static constexpr int kRows = 16 * kR, LD = D + 4, LPr = 32 + 4;
+    static constexpr int oQ = 0, oK = oQ + kRows * LD, oV = oK + 2 * 32 * LD, oP = oV + 2 * 32 * D, oPos = oP + kRows * LPr;
+    static constexpr int kBytes = (oPos + 64) * 4;
+};
+__device__ __forceinline__ float half_warp_sum(float x) {
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+template <typename T, int D, int G, int kR>
 __global__ void __launch_bounds__(kThreads)
 softmax_combine_simt_kernel(const T *__restrict__ q, const T *__restrict__ k_sm,
                             const T *__restrict__ v_sm, int cap, const int32_t *__restrict__ sm_idx,
                             const int32_t *__restrict__ sm_chunk_prefix,
-                            const float *__restrict__ o_la, const float *__restrict__ w,
+                            const float *o_la, const float *__restrict__ w,
                             float scale_sm, float eps, T *__restrict__ out,
                             float *__restrict__ o_nla, float *__restrict__ lse,
                             const uint8_t *__restrict__ block_route, const T *__restrict__ k_tok,
                             const T *__restrict__ v_tok, int L, int H) {
-    constexpr int kRowsQ = 8 * NQ, LD = D + 4;
+    using SS = SimtSoft<D, kR>;
+    constexpr int kRows = SS::kRows, LD = SS::LD, LPr = SS::LPr, DL = D * G;
+    constexpr int VW = D >= 64 ? 4 : 2, NU = D / (16 * VW);          // a lane's columns: VW kk + 16 VW u ..
     extern __shared__ __align__(16) float smem[];
-    float *Qs = smem;                      // [8 NQ][D]
-    float *Kt = Qs + kRowsQ * D;           // [32][D+4]
-    float *Vt = Kt + 32 * LD;              // [32][D]
-    int *pos = reinterpret_cast<int *>(Vt + 32 * D);  // [32]
+    float *Qs = smem + SS::oQ;             // [kRows][LD]
+    float *Pr = smem + SS::oP;             // [kRows][LPr]
+    int *pos = reinterpret_cast<int *>(smem + SS::oPos);  // [2][32]
 
-    constexpr int DL = D * G;
-    const int c = blockIdx.x * kRowsQ / kC, row0 = blockIdx.x * kRowsQ % kC;      // chunk, first row inside it
+    const int c = blockIdx.x * kRows / kC, row0 = blockIdx.x * kRows % kC;        // chunk, first row inside it
     const int bhg = blockIdx.y, bh = bhg / G, sg = bhg % G, b = bh / H, h = bh % H;
-    const int NC = L / kC;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int NC = L / kC, tid = threadIdx.x, kk = tid & 15, rg = tid >> 4;       // this thread's rows: rg + 16 e
     const size_t ts = (size_t)H * DL;
     const size_t tok0 = ((size_t)b * L + (size_t)c * kC) * H + h;
-    tc::grid_dependency_wait();
     tc::launch_dependents();
     const int n_end = min(sm_chunk_prefix[(size_t)bh * (NC + 1) + c + 1], cap);
     const int col0 = sg * D;                             // first column of this softmax head
-
-    for (int idx = threadIdx.x; idx < kRowsQ * D / 4; idx += kThreads) {
+    for (int idx = tid; idx < kRows * D / 4; idx += kThreads) {
         const int r = idx / (D / 4), c4 = (idx % (D / 4)) * 4;
-        store4(Qs + r * D + c4, load4(q + tok0 * DL + (size_t)(row0 + r) * ts + col0 + c4));
-    }
-    constexpr int kCols = D / 32;
-    float m[NQ], z[NQ], acc[NQ][kCols];
-#pragma unroll
-    for (int r = 0; r < NQ; ++r) {
-        m[r] = -INFINITY; z[r] = 0.f;
-#pragma unroll
-        for (int x = 0; x < kCols; ++x) acc[r][x] = 0.f;
+        store4(Qs + r * LD + c4, load4(q + tok0 * DL + (size_t)(row0 + r) * ts + col0 + c4));
     }
     const T *kb = k_sm + (size_t)bh * cap * DL + col0, *vb = v_sm + (size_t)bh * cap * DL + col0;
-
     // Block-level routing: a query in a linear block also reads the causal part of its own block
     // (two more tiles of 32 keys, taken from the layer's own k and v).
     const int n_ret = (n_end + 31) / 32 * 32;
     const int n_all = n_ret + (block_route && block_route[tok0] == 0 ? kC : 0);
-    for (int j0 = 0; j0 < n_all; j0 += 32) {
+    auto fetch = [&](int j0) {
         const bool own = j0 >= n_ret;
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < 32 * D / 4; idx += kThreads) {
+        float *Kt = smem + SS::oK + (j0 / 32 & 1) * 32 * LD, *Vt = smem + SS::oV + (j0 / 32 & 1) * 32 * D;
+#pragma unroll 2
+        for (int idx = tid; idx < 32 * D / 4; idx += kThreads) {
             const int r = idx / (D / 4), c4 = (idx % (D / 4)) * 4;
-            float4 kx = make_float4(0.f, 0.f, 0.f, 0.f), vx = kx;
-            if (own) {
-                const size_t src = (tok0 + (size_t)(j0 - n_ret + r) * H) * DL + col0 + c4;
-                kx = load4(k_tok + src);
-                vx = load4(v_tok + src);
-            } else if (j0 + r < n_end) {
-                kx = load4(kb + (size_t)(j0 + r) * DL + c4);
-                vx = load4(vb + (size_t)(j0 + r) * DL + c4);
+            if (!own && j0 + r >= n_end) {
+                store4(Kt + r * LD + c4, make_float4(0.f, 0.f, 0.f, 0.f));
+                store4(Vt + r * D + c4, make_float4(0.f, 0.f, 0.f, 0.f));
+                continue;
             }
-            store4(Kt + r * LD + c4, kx);
-            store4(Vt + r * D + c4, vx);
+            const T *ks = own ? k_tok + (tok0 + (size_t)(j0 - n_ret + r) * H) * DL + col0 + c4 : kb + (size_t)(j0 + r) * DL + c4;
+            const T *vs = own ? v_tok + (tok0 + (size_t)(j0 - n_ret + r) * H) * DL + col0 + c4 : vb + (size_t)(j0 + r) * DL + c4;
+            if constexpr (sizeof(T) == 4) {
+                copy16_async(Kt + r * LD + c4, ks);
+                copy16_async(Vt + r * D + c4, vs);
+            } else {
+                store4(Kt + r * LD + c4, load4(ks));
+                store4(Vt + r * D + c4, load4(vs));
+            }
         }
-        if (threadIdx.x < 32)
-            pos[threadIdx.x] = own ? c * kC + (j0 - n_ret) + (int)threadIdx.x
-                               : (j0 + threadIdx.x < n_end) ? sm_idx[(size_t)bh * L + j0 + threadIdx.x]
-                                                            : 0x7fffffff;
-        __syncthreads();
-        const int my_pos = pos[lane];
-        const float *kr = Kt + lane * LD, *qr = Qs + warp * NQ * D;
-        float s[NQ], p[NQ];
+        if (tid < 32) {
+            int *pp = pos + (j0 / 32 & 1) * 32 + tid;
+            if (!own && j0 + tid < n_end)
+                copy4_async(reinterpret_cast<float *>(pp), reinterpret_cast<const float *>(sm_idx + (size_t)bh * L + j0 + tid));
+            else
+                *pp = own ? c * kC + (j0 - n_ret) + tid : 0x7fffffff;
+        }
+    };
+    float m[kR], z[kR], acc[kR][NU * VW];
 #pragma unroll
-        for (int r = 0; r < NQ; ++r) s[r] = 0.f;
+    for (int e = 0; e < kR; ++e) {
+        m[e] = -INFINITY; z[e] = 0.f;
+#pragma unroll
+        for (int x = 0; x < NU * VW; ++x) acc[e][x] = 0.f;
+    }
+    if (n_all > 0) fetch(0);
+    for (int j0 = 0; j0 < n_all; j0 += 32) {
+        const float *Kt = smem + SS::oK + (j0 / 32 & 1) * 32 * LD, *Vt = smem + SS::oV + (j0 / 32 & 1) * 32 * D;
+        copies_wait();
+        __syncthreads();
+        if (j0 + 32 < n_all) fetch(j0 + 32);
+        const int pos0 = pos[(j0 / 32 & 1) * 32 + kk], pos1 = pos[(j0 / 32 & 1) * 32 + kk + 16];
+        uint64_t sa[kR][2];
+#pragma unroll
+        for (int e = 0; e < kR; ++e) sa[e][0] = sa[e][1] = 0ull;
 #pragma unroll 4
         for (int x = 0; x < D; x += 4) {
-            const float4 kx = *reinterpret_cast<const float4 *>(kr + x);
+            const ulonglong2 k0 = lds4(Kt + kk * LD + x), k1 = lds4(Kt + (kk + 16) * LD + x);
 #pragma unroll
-            for (int r = 0; r < NQ; ++r) {
-                const float4 qx = *reinterpret_cast<const float4 *>(qr + r * D + x);
-                s[r] = fmaf(qx.x, kx.x, fmaf(qx.y, kx.y, fmaf(qx.z, kx.z, fmaf(qx.w, kx.w, s[r]))));
+            for (int e = 0; e < kR; ++e) {
+                const ulonglong2 qx = lds4(Qs + (rg + 16 * e) * LD + x);
+                fma4(qx, k0, sa[e][0]);
+                fma4(qx, k1, sa[e][1]);
             }
         }
 #pragma unroll
-        for (int r = 0; r < NQ; ++r) {
-            const bool valid = my_pos <= c * kC + row0 + warp * NQ + r;
-            const float sc = valid ? s[r] * scale_sm : -INFINITY;
-            const float m_new = fmaxf(m[r], warp_max(sc)), m_use = m_new == -INFINITY ? 0.f : m_new;
-            p[r] = valid ? __expf(sc - m_use) : 0.f;
-            const float corr = __expf(m[r] - m_use);   // exp(-inf) = 0 on the first tile
-            z[r] = z[r] * corr + warp_sum(p[r]);
-            m[r] = m_new;
+        for (int e = 0; e < kR; ++e) {
+            const int i = c * kC + row0 + rg + 16 * e;
+            const float s0 = pos0 <= i ? both(sa[e][0]) * scale_sm : -INFINITY, s1 = pos1 <= i ? both(sa[e][1]) * scale_sm : -INFINITY;
+            float mx = fmaxf(s0, s1);
 #pragma unroll
-            for (int x = 0; x < kCols; ++x) acc[r][x] *= corr;
+            for (int o = 8; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            const float m_new = fmaxf(m[e], mx), m_use = m_new == -INFINITY ? 0.f : m_new;
+            const float p0 = pos0 <= i ? __expf(s0 - m_use) : 0.f, p1 = pos1 <= i ? __expf(s1 - m_use) : 0.f;
+            const float corr = __expf(m[e] - m_use);     // exp(-inf) = 0 on the first tile
+            z[e] = z[e] * corr + (p0 + p1);              // (this lane's keys; summed over the lanes at the end)
+            m[e] = m_new;
+            Pr[(rg + 16 * e) * LPr + kk] = p0;
+            Pr[(rg + 16 * e) * LPr + kk + 16] = p1;
+#pragma unroll
+            for (int x = 0; x < NU * VW; ++x) acc[e][x] *= corr;
         }
-#pragma unroll 8
-        for (int j = 0; j < 32; ++j) {
-            float vx[kCols];
+        __syncwarp();                                    // (a row's lanes are in one warp)
+#pragma unroll 2
+        for (int j = 0; j < 32; j += 4) {
+            float4 pv[kR];
 #pragma unroll
-            for (int x = 0; x < kCols; ++x) vx[x] = Vt[j * D + lane + 32 * x];
+            for (int e = 0; e < kR; ++e) pv[e] = *reinterpret_cast<const float4 *>(Pr + (rg + 16 * e) * LPr + j);
 #pragma unroll
-            for (int r = 0; r < NQ; ++r) {
-                const float pb = __shfl_sync(0xffffffffu, p[r], j);
+            for (int jj = 0; jj < 4; ++jj) {
+                float vx[NU * VW];
 #pragma unroll
-                for (int x = 0; x < kCols; ++x) acc[r][x] = fmaf(pb, vx[x], acc[r][x]);
+                for (int u = 0; u < NU; ++u) {
+                    const float *vp = Vt + (j + jj) * D + VW * kk + 16 * VW * u;
+                    if constexpr (VW == 4) {
+                        const float4 y = *reinterpret_cast<const float4 *>(vp);
+                        vx[4 * u] = y.x; vx[4 * u + 1] = y.y; vx[4 * u + 2] = y.z; vx[4 * u + 3] = y.w;
+                    } else {
+                        const float2 y = *reinterpret_cast<const float2 *>(vp);
+                        vx[2 * u] = y.x; vx[2 * u + 1] = y.y;
+                    }
+                }
+#pragma unroll
+                for (int e = 0; e < kR; ++e) {
+                    const float pe = jj == 0 ? pv[e].x : jj == 1 ? pv[e].y : jj == 2 ? pv[e].z : pv[e].w;
+#pragma unroll
+                    for (int x = 0; x < NU * VW; ++x) acc[e][x] = fmaf(pe, vx[x], acc[e][x]);
+                }
             }
         }
+        __syncwarp();                                    // the probabilities have been read
     }
-    // epilogue: normalise both branches and combine
+    // epilogue: normalise both branches and combine.  Up to here the kernel has needed only what lies ahead of the scan,
+    // and every CTA of the scan had waited for that before this kernel could start.
+    tc::grid_dependency_wait();
 #pragma unroll
-    for (int r = 0; r < NQ; ++r) {
-        const int i = c * kC + row0 + warp * NQ + r;
-        const size_t t = tok0 + (size_t)(row0 + warp * NQ + r) * H;
-        const float inv = z[r] > 0.f ? 1.f / z[r] : 0.f;
-        float on[kCols], ol[kCols], ssn = 0.f, ssl = 0.f;
+    for (int e = 0; e < kR; ++e) {
+        const int i = c * kC + row0 + rg + 16 * e;
+        const size_t t = tok0 + (size_t)(row0 + rg + 16 * e) * H;
+        z[e] = half_warp_sum(z[e]);
+        const float inv = z[e] > 0.f ? 1.f / z[e] : 0.f;
+        float ol[NU * VW], ssn = 0.f, ssl = 0.f;
 #pragma unroll
-        for (int x = 0; x < kCols; ++x) {
-            on[x] = acc[r][x] * inv;
-            ol[x] = o_la[t * DL + col0 + lane + 32 * x];
-            ssn = fmaf(on[x], on[x], ssn);
+        for (int u = 0; u < NU; ++u) {
+            const float *op = o_la + t * DL + col0 + VW * kk + 16 * VW * u;
+            if constexpr (VW == 4) {
+                const float4 y = __ldcg(reinterpret_cast<const float4 *>(op));
+                ol[4 * u] = y.x; ol[4 * u + 1] = y.y; ol[4 * u + 2] = y.z; ol[4 * u + 3] = y.w;
+            } else {
+                const float2 y = __ldcg(reinterpret_cast<const float2 *>(op));
+                ol[2 * u] = y.x; ol[2 * u + 1] = y.y;
+            }
+        }
+#pragma unroll
+        for (int x = 0; x < NU * VW; ++x) {
+            acc[e][x] *= inv;
+            ssn = fmaf(acc[e][x], acc[e][x], ssn);
             ssl = fmaf(ol[x], ol[x], ssl);
         }
         if (G > 1)        // the linear read-out is normalised over its whole row
-            for (int x = 0; x < DL / 32; ++x) {
-                if ((32 * x) / D == sg) continue;
-                const float y = o_la[t * DL + lane + 32 * x];
+            for (int x = 0; x < DL / 16; ++x) {
+                if ((16 * x) / D == sg) continue;
+                const float y = __ldcg(o_la + t * DL + kk + 16 * x);
                 ssl = fmaf(y, y, ssl);
             }
-        ssn = warp_sum(ssn);
-        ssl = warp_sum(ssl);
+        ssn = half_warp_sum(ssn);
+        ssl = half_warp_sum(ssl);
         const float fn = rsqrtf(ssn / D + eps), fl = rsqrtf(ssl / DL + eps);
         const float wn = w ? w[t * 2] : 0.5f, wl = w ? w[t * 2 + 1] : 0.5f;
 #pragma unroll
-        for (int x = 0; x < kCols; ++x) {
-            if (out) out[t * DL + col0 + lane + 32 * x] = from_f32<T>(wn * on[x] * fn + wl * ol[x] * fl);
-            if (o_nla) o_nla[t * DL + col0 + lane + 32 * x] = on[x];
+        for (int u = 0; u < NU; ++u) {
+            const size_t at = t * DL + col0 + VW * kk + 16 * VW * u;
+            const float *on = &acc[e][VW * u], *la = &ol[VW * u];
+            auto y = [&](int x) { return wn * on[x] * fn + wl * la[x] * fl; };
+            if constexpr (VW == 4) {
+                if (out) store4(out + at, make_float4(y(0), y(1), y(2), y(3)));
+                if (o_nla) store4(o_nla + at, make_float4(on[0], on[1], on[2], on[3]));
+            } else {
+#pragma unroll
+                for (int x = 0; x < VW; ++x) {
+                    if (out) out[at + x] = from_f32<T>(y(x));
+                    if (o_nla) o_nla[at + x] = on[x];
+                }
+            }
         }
-        if (lse && lane == 0) lse[(size_t)bhg * L + i] = z[r] > 0.f ? m[r] + __logf(z[r]) : -INFINITY;
+        if (lse && kk == 0) lse[(size_t)bhg * L + i] = z[e] > 0.f ? m[e] + __logf(z[e]) : -INFINITY;
     }
 }
 
@@ -588,11 +815,11 @@ cudaError_t set_smem(K kernel, size_t bytes) {
 
 }  // namespace
 
-static size_t simt_prepare_smem(int d) { return sizeof(float) * (3 * kC * (d + 4) + kC * (kC + 4) + 2 * kC); }
-static size_t simt_scan_smem(int d, int nv) {
-    return sizeof(float) * (d * nv + 3 * kC * (d + 4) + kC * (kC + 4) + kC * nv + 3 * kC);
-}
-static size_t simt_softmax_smem(int d, int nq) { return sizeof(float) * (8 * nq * d + 32 * (d + 4) + 32 * d + 32); }
+
+// Chunks up to which the prepare kernel cuts a chunk into four, i.e. up to two CTAs per SM: with more the four-fold A takes
+// more than the finer split of the rest gains.  Whole call with four parts against one: 8 chunks of 64 columns 21.8 / 26.4
+// us, 70 chunks 44.7 / 48.9 (128 columns 87.7 / 91.5), 80 chunks 44.7 / 48.9 (98.6 / 92.6), 128 chunks 104 / 102 (158 / 146).
+constexpr int kFewChunks = 74;
 
 #define NATSL_DISPATCH(FN, ...)                                                   \
     do {                                                                          \
@@ -608,35 +835,37 @@ template <typename T, int D>
 static cudaError_t prepare_impl(const void *q, const void *k, const void *v, const float *g,
                                 const float *beta, const uint8_t *route, float scale_la, float *W,
                                 float *U, float *P, float *Abar, float *Gcum, Shape s,
-                                cudaStream_t st) {
-    const size_t smem = simt_prepare_smem(D);
-    cudaError_t e = set_smem(gdn_prepare_simt_kernel<T, D>, smem);
+                                cudaStream_t st, int32_t *clear, int clear_words) {
+    const bool few = s.L / kC * s.B * s.H <= kFewChunks;     // (see the kernel)
+    const size_t smem = few ? SimtPrep<D, 4>::kBytes : SimtPrep<D, 1>::kBytes;
+    auto kernel = few ? gdn_prepare_simt_kernel<T, D, 4> : gdn_prepare_simt_kernel<T, D, 1>;
+    cudaError_t e = set_smem(kernel, smem);
     if (e != cudaSuccess) return e;
-    dim3 grid(s.L / kC, s.B * s.H);
+    dim3 grid(s.L / kC * (few ? 4 : 1), s.B * s.H);
     count_launch();
-    return launch_kernel(gdn_prepare_simt_kernel<T, D>, grid, dim3(kThreads), smem, st, true, (const T *)q, (const T *)k,
-                         (const T *)v, g, beta, route, scale_la, W, U, P, Abar, Gcum, s.L, s.H);
+    return launch_kernel(kernel, grid, dim3(kThreads), smem, st, true, (const T *)q, (const T *)k,
+                         (const T *)v, g, beta, route, scale_la, W, U, P, Abar, Gcum, clear, clear_words, s.L, s.H);
 }
 
 cudaError_t launch_gdn_prepare_simt(const void *q, const void *k, const void *v, const float *g,
                                     const float *beta, const uint8_t *route, float scale_la,
                                     float *W, float *U, float *P, float *Abar, float *Gcum, Shape s,
-                                    cudaStream_t st) {
-    NATSL_DISPATCH(prepare_impl, q, k, v, g, beta, route, scale_la, W, U, P, Abar, Gcum, s, st);
+                                    cudaStream_t st, int32_t *clear, int clear_words) {
+    NATSL_DISPATCH(prepare_impl, q, k, v, g, beta, route, scale_la, W, U, P, Abar, Gcum, s, st, clear, clear_words);
 }
 
 template <typename T, int D>
 static cudaError_t scan_impl(const void *q, const void *k, const float *g, const float *W,
                              const float *U, const float *P, float scale_la, const float *state_in,
                              float *state_out, float *chunk_states, float *Ut, float *o_la,
-                             const uint8_t *block_route, Shape s, cudaStream_t st) {
+                             const uint8_t *block_route, Shape s, cudaStream_t st, bool pdl) {
     const bool narrow = s.B * s.H * (D / 32) < 148;     // (see the kernel)
-    const size_t smem = simt_scan_smem(D, narrow ? 8 : 32);
+    const size_t smem = narrow ? SimtScan<D, 8>::kBytes : SimtScan<D, 32>::kBytes;
     auto kernel = narrow ? gdn_scan_simt_kernel<T, D, 8> : gdn_scan_simt_kernel<T, D, 32>;
-    cudaError_t e = set_smem(kernel, smem);
+    cudaError_t e = allow_smem(kernel, smem, true);      // (softmax CTAs fit beside 64-column scans: 115 -> 108 us at 16 pairs of 1024)
     if (e != cudaSuccess) return e;
     count_launch();
-    return launch_kernel(kernel, dim3(D / (narrow ? 8 : 32), s.B * s.H), dim3(kThreads), smem, st, true, (const T *)q,
+    return launch_kernel(kernel, dim3(D / (narrow ? 8 : 32), s.B * s.H), dim3(kThreads), smem, st, pdl, (const T *)q,
                          (const T *)k, g, W, U, P, scale_la, state_in, state_out, chunk_states, Ut, o_la, block_route, s.L,
                          s.H);
 }
@@ -645,9 +874,9 @@ cudaError_t launch_gdn_scan_simt(const void *q, const void *k, const float *g, c
                                  const float *U, const float *P, float scale_la,
                                  const float *state_in, float *state_out, float *chunk_states,
                                  float *Ut, float *o_la, const uint8_t *block_route, Shape s,
-                                 cudaStream_t st) {
+                                 cudaStream_t st, bool pdl) {
     NATSL_DISPATCH(scan_impl, q, k, g, W, U, P, scale_la, state_in, state_out, chunk_states, Ut, o_la,
-                   block_route, s, st);
+                   block_route, s, st, pdl);
 }
 
 template <typename T, int D, int G = 1>
@@ -656,13 +885,13 @@ static cudaError_t softmax_impl(const void *q, const void *k_sm, const void *v_s
                                 const float *w, float scale_sm, float eps, void *out, float *o_nla,
                                 float *lse, BlockRouting br, Shape s, cudaStream_t st) {
     const bool few = (s.L / kC) * s.B * s.H * G < 148;   // (see the kernel)
-    const int nq = few ? 2 : 8;
-    const size_t smem = simt_softmax_smem(D, nq);
-    auto kernel = few ? softmax_combine_simt_kernel<T, D, G, 2> : softmax_combine_simt_kernel<T, D, G, 8>;
+    const int rows = few ? 16 : 64;
+    const size_t smem = few ? SimtSoft<D, 1>::kBytes : SimtSoft<D, 4>::kBytes;
+    auto kernel = few ? softmax_combine_simt_kernel<T, D, G, 1> : softmax_combine_simt_kernel<T, D, G, 4>;
     cudaError_t e = set_smem(kernel, smem);
     if (e != cudaSuccess) return e;
     count_launch();
-    return launch_kernel(kernel, dim3(s.L / (8 * nq), s.B * s.H * G), dim3(kThreads), smem, st, true, (const T *)q,
+    return launch_kernel(kernel, dim3(s.L / rows, s.B * s.H * G), dim3(kThreads), smem, st, true, (const T *)q,
                          (const T *)k_sm, (const T *)v_sm, cap, sm_idx, pre, o_la, w, scale_sm, eps, (T *)out, o_nla, lse,
                          br.route, (const T *)br.k, (const T *)br.v, s.L, s.H);
 }

@@ -49,17 +49,30 @@ cudaError_t launch_route_compact(const uint8_t *route, int32_t *sm_idx, int32_t 
 cudaError_t launch_gather_kv(const void *k, const void *v, const int32_t *sm_idx,
                              const int32_t *sm_chunk_prefix, void *k_sm, void *v_sm, int32_t cap,
                              int32_t *status, Shape s, cudaStream_t st);
+// Both in one kernel (CUDA-core forward): rows of k (and of v) to k_out (v_out) [B,H,cap,d]; k == nullptr: no such job.
+// sm_len [B,H] or nullptr receives the retained tokens, at most len_cap; more are NATSL_ERR_CACHE_FULL.
+struct RowsJob {
+    const void *k = nullptr;
+    void *k_out = nullptr, *v_out = nullptr;
+    int cap = 0;
+};
+cudaError_t launch_route_gather_rows(const uint8_t *route, const void *v, const RowsJob &j0, const RowsJob &j1,
+                                     int32_t *sm_idx, int32_t *prefix, int32_t *sm_len, int len_cap, int32_t *status,
+                                     bool check_blocks, Shape s, cudaStream_t st, bool pdl);
 
 // fwd_simt.cu -- fp32 CUDA-core forward (exact-precision path; bf16 storage allowed)
 cudaError_t launch_gdn_prepare_simt(const void *q, const void *k, const void *v, const float *g,
                                     const float *beta, const uint8_t *route, float scale_la,
                                     float *W, float *U, float *P, float *Abar, float *Gcum, Shape s,
-                                    cudaStream_t st);
+                                    cudaStream_t st, int32_t *clear = nullptr, int clear_words = 0);
+// (clear: words of the status page that the kernel, the forward's first, sets to zero, or nullptr)
 cudaError_t launch_gdn_scan_simt(const void *q, const void *k, const float *g, const float *W,
                                  const float *U, const float *P, float scale_la,
                                  const float *state_in, float *state_out, float *chunk_states,
                                  float *Ut, float *o_la, const uint8_t *block_route, Shape s,
-                                 cudaStream_t st);
+                                 cudaStream_t st, bool pdl = true);
+// (launched behind the scan, whose CTAs have waited for everything ahead of them, as its programmatic dependent: it
+// runs beside the scan up to where it needs o_la)
 cudaError_t launch_softmax_combine_simt(const void *q, const void *k_sm, const void *v_sm,
                                         int32_t cap, const int32_t *sm_idx,
                                         const int32_t *sm_chunk_prefix, const float *o_la,
@@ -104,9 +117,10 @@ cudaError_t launch_softmax_combine_tc(const void *q, const void *k_sm, const voi
 // launch's host time about half a microsecond, and a forward would make five of them.  The limit belongs to the
 // function, what has been set is remembered per thread: every call for a kernel must therefore ask for the same bytes,
 // the most that any of its launches uses (a smaller request of another thread would lower the limit behind this one's back).
-cudaError_t allow_smem_of(const void *kernel, int bytes);
-template <typename K> cudaError_t allow_smem(K *kernel, size_t bytes) {
-    return allow_smem_of(reinterpret_cast<const void *>(kernel), (int)bytes);
+// all_shared: the multiprocessor's memory as shared memory throughout, for a kernel beside which another one is to run.
+cudaError_t allow_smem_of(const void *kernel, int bytes, bool all_shared);
+template <typename K> cudaError_t allow_smem(K *kernel, size_t bytes, bool all_shared = false) {
+    return allow_smem_of(reinterpret_cast<const void *>(kernel), (int)bytes, all_shared);
 }
 // A launch, as a programmatic dependent of the kernel before it in the stream when pdl is set.
 template <typename... P, typename... A>

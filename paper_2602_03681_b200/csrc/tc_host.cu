@@ -58,7 +58,7 @@ bool make_map_blhd(CUtensorMap *m, const void *base, int B, int L, int H, int d,
 
 }  // namespace tch
 
-cudaError_t allow_smem_of(const void *kernel, int bytes) {
+cudaError_t allow_smem_of(const void *kernel, int bytes, bool all_shared) {
     struct Entry { const void *fn; int dev; };
     constexpr int kEntries = 128;                     // (the library has fewer kernels; a full table only re-sends)
     thread_local Entry table[kEntries] = {};
@@ -73,6 +73,8 @@ cudaError_t allow_smem_of(const void *kernel, int bytes) {
         if (!x.fn) slot = &x;
     }
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess && all_shared)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e == cudaSuccess && slot) *slot = Entry{kernel, dev};
     return e;
 }

@@ -1,5 +1,6 @@
-"""fp32 forward on either side of the pair and block counts at which its scan and softmax kernels cut their work finer,
-against the oracle."""
+"""fp32 forward on either side of the pair, chunk and block counts at which its kernels cut their work finer, against the
+oracle."""
+import numpy as np
 import pytest
 
 from paper_2602_03681_b200 import inputs
@@ -12,4 +13,23 @@ pytestmark = pytest.mark.gpu
 def test_fp32_forward(B, H, L):
     wl = inputs.WORKLOADS["cfg0_f32_tiny_fwd"]
     x = inputs.make_layer_inputs(wl, B=B, H=H, L=L)
+    check_fwd(wl, run_fwd(wl, x), run_oracle(wl, x), TOL["f32"])
+
+
+# 128 columns: 74 chunks (cut into four by the prepare kernel) and 75, 36 and 37 pairs (narrow and wide scan slices)
+@pytest.mark.parametrize("B,H,L", [(1, 37, 128), (1, 25, 192), (1, 36, 64), (1, 2, 704)])
+def test_fp32_forward_128_columns(B, H, L):
+    import dataclasses
+    wl = dataclasses.replace(inputs.WORKLOADS["cfg0_f32_tiny_fwd"], d=128)
+    x = inputs.make_layer_inputs(wl, B=B, H=H, L=L)
+    check_fwd(wl, run_fwd(wl, x), run_oracle(wl, x), TOL["f32"])
+
+
+# no retained token at all, and nothing else; one chunk and a ragged number of key tiles
+@pytest.mark.parametrize("L", [64, 192])
+@pytest.mark.parametrize("retained", [0, 1])
+def test_fp32_forward_one_branch_empty(L, retained):
+    wl = inputs.WORKLOADS["cfg0_f32_tiny_fwd"]
+    x = inputs.make_layer_inputs(wl, B=1, H=2, L=L)
+    x["route"] = np.full_like(x["route"], retained)
     check_fwd(wl, run_fwd(wl, x), run_oracle(wl, x), TOL["f32"])

@@ -128,12 +128,12 @@ FwdWs carve_fwd(const natsl_params *p, void *ws) {
         const size_t capv = (p->flags & NATSL_APPEND_CACHE) && p->sm_cap > 0 ? (size_t)p->sm_cap : L;
         f.v16 = c.take<char>(B * H * capv * d * 2);
         f.kn16 = c.take<char>((p->flags & NATSL_APPEND_CACHE) && (p->flags & NATSL_QK_NORM) ? B * H * capv * d * 2 : 0);
-        f.tc.Qh = c.take<char>(B * H * L * d * 2);
-        f.tc.Kh = c.take<char>(B * H * L * d * 2);
+        f.tc.Qh = f.tc.Kh = nullptr;
         f.tc.Wt = c.take<char>(B * H * L * d * 2);
-        f.tc.Ut = c.take<float>(B * H * L * d);
+        f.tc.Tb = c.take<char>(B * H * NC * kC * kC * 2);
         f.tc.Ph = c.take<char>(B * H * NC * kC * kC * 2);
         f.tc.Gd = c.take<float>(B * H * L * 2);
+        f.tc.Rn = c.take<float>((p->flags & NATSL_QK_NORM) ? B * H * L * 2 : 0);
         f.W = f.U = f.P = nullptr;
         const size_t nseg = scan_segments(p), segf = nseg > 1 ? B * H * nseg * d * d : 0;
         f.seg_incr = c.take<float>(segf);
@@ -243,9 +243,10 @@ BwdWs carve_bwd(const natsl_params *p, void *ws) {
     f.tc.Qh = f.Qh;                           // without the normalisation the same fp16 copy of q serves both branches
     f.tc.Kh = half(tcs, TM);
     f.tc.Wt = half(tcs, TM);
-    f.tc.Ut = tm(tcs);
+    f.tc.Tb = half(tcs, CC);
     f.tc.Ph = half(tcs, CC);
     f.tc.Gd = c.take<float>(tcs ? BHL * 2 : 0);
+    f.tc.Rn = c.take<float>(tcs && normed ? BHL * 2 : 0);
     f.ex = GdnTcExport{};
     f.ex.U16 = half(tcs, TM); f.ex.T16 = half(tcs, CC); f.ex.S16 = half(tcs, ST); f.ex.Ut16 = half(tcs, TM);
     f.ex.Gcum = f.Gcum;
@@ -333,9 +334,9 @@ static int bwd_forward_part(const void *q, const void *k, const void *v, const f
                                         f.status, s, st, (int)(kStatusBytes / 4), hg.norm_eps));
         NATSL_TRY(launch_route_gather_tc(k, v, route, f.sm_idx, f.prefix, nullptr, f.k_smb, nullptr, f.v16, f.k16, p->L,
                                          p->L, f.emit_flags, s, st, pdl, hg));
-        NATSL_TRY(launch_gdn_scan_tc(f.tc, p->scale_la, p->state_in, state_out, ScanOut{f.o_la16, f.o_la, flags},
+        NATSL_TRY(launch_gdn_scan_tc(q, k, v, f.tc, p->scale_la, p->state_in, state_out, ScanOut{f.o_la16, f.o_la, flags},
                                      f.ex, ScanSegments{0, 1, 0, nullptr, nullptr, nullptr}, block_route,
-                                     f.status, s, st, pdl && scan_follows_closely(p)));
+                                     f.status, s, st, pdl && scan_follows_closely(p), hg.norm_eps >= 0.f));
         NATSL_TRY(launch_softmax_combine_tc(q, f.k_smb, f.v16, p->L, p->L, f.sm_idx, f.prefix, f.o_la16,
                                             flags, p->w, p->scale_sm, p->eps, out, f.o_nla, f.lse, nullptr, p->L,
                                             BlockRouting{block_route, k, v}, false, f.status, s, st, hg));
@@ -528,16 +529,16 @@ int natsl_hybrid_fwd(const void *q, const void *k, const void *v, const float *g
         const ScanOut so{f.o_la16, p->o_la, flags_scan};
         if (nseg > 1) {   // few (batch, head) pairs: segments in parallel, chained by their transitions
             ScanSegments sg{1, nseg, seg_chunks, f.seg_incr, f.seg_trans, f.seg_start};
-            NATSL_TRY(launch_gdn_scan_tc(f.tc, p->scale_la, p->state_in, nullptr, so, GdnTcExport{}, sg,
-                                         br.route, f.status, s, st, pdl));
+            NATSL_TRY(launch_gdn_scan_tc(q, k, v, f.tc, p->scale_la, p->state_in, nullptr, so, GdnTcExport{}, sg,
+                                         br.route, f.status, s, st, pdl, hg.norm_eps >= 0.f));
             NATSL_TRY(launch_scan_combine(sg, s, st, pdl));
             sg.mode = 2;
-            NATSL_TRY(launch_gdn_scan_tc(f.tc, p->scale_la, p->state_in, p->state_out, so, GdnTcExport{}, sg,
-                                         br.route, f.status, s, st, pdl));
+            NATSL_TRY(launch_gdn_scan_tc(q, k, v, f.tc, p->scale_la, p->state_in, p->state_out, so, GdnTcExport{}, sg,
+                                         br.route, f.status, s, st, pdl, hg.norm_eps >= 0.f));
         } else {
-            NATSL_TRY(launch_gdn_scan_tc(f.tc, p->scale_la, p->state_in, p->state_out, so, GdnTcExport{},
+            NATSL_TRY(launch_gdn_scan_tc(q, k, v, f.tc, p->scale_la, p->state_in, p->state_out, so, GdnTcExport{},
                                          ScanSegments{0, 1, 0, nullptr, nullptr, nullptr}, br.route,
-                                         f.status, s, st, pdl));
+                                         f.status, s, st, pdl, hg.norm_eps >= 0.f));
         }
         NATSL_TRY(mark());
         NATSL_TRY(launch_softmax_combine_tc(q, k_soft, f.v16, cap_soft, capv, f.sm_idx, f.prefix, f.o_la16,

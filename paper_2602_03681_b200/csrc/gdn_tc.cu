@@ -50,22 +50,27 @@ __device__ __forceinline__ uint4 bf16x8_to_f16x8(uint4 u) {
 // (rows 0-63) compute the gates, P and the decay factors; warps 2-3 (rows 64-127) build A, form
 // T = (I + A)^-1 blockwise (16x16 diagonal blocks by substitution through warp shuffles, the rest as
 // a handful of warp-level MMAs), and write the fp16 operands T beta~ and T beta~ gamma; then all
-// 128 threads (one head-dimension row each) store U^T and W^T.  Warp 4 issues TMA and MMAs.
-// 128 TMEM columns and ~50 KB of shared memory per CTA keep four CTAs on an SM, so that one chunk's
-// dependent phases overlap with other chunks' loads and stores.
+// 128 threads (one head-dimension row each) take W^T out of TMEM.  Warp 4 issues TMA and MMAs.
+// What bounds it is what it moves, so it hands on as little as the scan can work from: T beta~, W^T, P and the decay
+// factors (33 KB a chunk of 128 columns; the scan reads q, k, v itself and forms U on its tensor cores), and W^T, P, T beta~
+// leave through shared memory as whole tiles: five CTAs per SM, 124 us before, 83 now for 4096 chunks of 128 columns.
+// kTrain: the forward of a training step also writes the fp16 copies of q and k and U, T, the cumulative decays.
 // ==========================================================================================
 constexpr int kPrepThreads = 160;
 constexpr int kPrepMisc = 2048;
 
-template <int D> struct PrepLayout {
+template <int D, bool kTrain> struct PrepLayout {
     static constexpr int KB = D / 64;
-    static constexpr int oV = 0;                           // V: KB sub-tiles of 64 tokens x 64
-    static constexpr int oQK = KB * 8192;                  // per 64-column block: [Q 8 KB][K 8 KB]
+    static constexpr int oV = 0;                           // kTrain: V, KB sub-tiles of 64 tokens x 64
+    static constexpr int oQK = kTrain ? KB * 8192 : 0;     // per 64-column block: [Q 8 KB][K 8 KB]
     static constexpr int oX = oQK + KB * 16384;            // d = 64 only: A^T, then the T operands
     static constexpr int kX = D == 64 ? 16384 : 0;
-    static constexpr int oMisc = oX + kX;
+    static constexpr int oP = oX + kX;                     // not kTrain: P's tile (there P leaves by plain stores: four CTAs fit)
+    static constexpr int oMisc = oP + (kTrain ? 0 : 8192);
     static constexpr int kTotal = oMisc + kPrepMisc;
-    static constexpr int kLoadBytes = KB * 24576;
+    static constexpr int kLoadBytes = KB * (kTrain ? 24576 : 16384);
+    static constexpr int kTmemCols = kTrain ? 128 : 64;    // [Q ; K] K^T, then (U^T and) W^T
+    static constexpr int kCtas = kTrain ? 4 : 5;
 };
 
 struct PrepMisc {
@@ -76,18 +81,21 @@ struct PrepMisc {
 };
 static_assert(sizeof(PrepMisc) <= kPrepMisc, "misc page too small");
 
-template <int D>
-__global__ void __launch_bounds__(kPrepThreads, 4)
+template <int D, bool kTrain>
+__global__ void __launch_bounds__(kPrepThreads, PrepLayout<D, kTrain>::kCtas)
 gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                       const __grid_constant__ CUtensorMap map_k,
-                      const __grid_constant__ CUtensorMap map_v,
+                      const __grid_constant__ CUtensorMap map_v,       // (kTrain, like map_qh, map_kh, map_u16)
                       const __grid_constant__ CUtensorMap map_qh,
-                      const __grid_constant__ CUtensorMap map_kh, const float *__restrict__ g,
+                      const __grid_constant__ CUtensorMap map_kh,
+                      const __grid_constant__ CUtensorMap map_u16,     // U^T fp16 and W^T [B*H*NC*D][64], box 64
+                      const __grid_constant__ CUtensorMap map_wt,
+                      const __grid_constant__ CUtensorMap map_tb,      // T beta~ and P [B*H*NC*64][64], box 64
+                      const __grid_constant__ CUtensorMap map_ph, const float *__restrict__ g,
                       const float *__restrict__ beta, const uint8_t *__restrict__ route,
-                      float scale_la, __half *__restrict__ Wt, float *__restrict__ Ut,
-                      __half *__restrict__ Ph, float *__restrict__ Gd, GdnTcExport ex,
+                      float scale_la, __half *__restrict__ Ph, float *__restrict__ Gd, float *__restrict__ Rn, GdnTcExport ex,
                       int32_t *status, int head_words, int L, int H, float norm_eps, int wait_kcycles) {
-    using PL = PrepLayout<D>;
+    using PL = PrepLayout<D, kTrain>;
     constexpr int KB = PL::KB;
     extern __shared__ __align__(1024) uint8_t smem[];
     PrepMisc &ms = *reinterpret_cast<PrepMisc *>(smem + PL::oMisc);
@@ -119,13 +127,13 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
     if (blockIdx.x == 0 && tid < head_words) status[tid] = 0;
     __threadfence();
     launch_dependents();
-    if (warp == 4) tmem_alloc(&ms.tmem_base, 128);
+    if (warp == 4) tmem_alloc(&ms.tmem_base, PL::kTmemCols);
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem = ms.tmem_base;
+    const uint32_t tmem = ms.tmem_base, tW = tmem + (kTrain ? 64 : 0);
     volatile int *abort_flag = &ms.abort_flag;
-    uint8_t *sV = smem + PL::oV, *sQK = smem + PL::oQK;
+    uint8_t *sV = smem + PL::oV, *sQK = smem + PL::oQK, *sP = smem + PL::oP;
     // The fp16 tiles of A and T during the inversion, and afterwards the two fp16 operands: in the two Q blocks
     // once K K^T / Q K^T and the q copy are done with them (d = 128), or in their own region (d = 64).
     uint8_t *xLo = D == 128 ? sQK : smem + PL::oX;
@@ -137,16 +145,18 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
             for (int kb = 0; kb < KB; ++kb) {
                 tma_load_4d(sQK + kb * 16384 + 8192, &map_k, &ms.barLoad, kb * 64, h, tok0, b);
                 tma_load_4d(sQK + kb * 16384, &map_q, &ms.barLoad, kb * 64, h, tok0, b);
-                tma_load_4d(sV + kb * 8192, &map_v, &ms.barLoad, kb * 64, h, tok0, b);
+                if (kTrain) tma_load_4d(sV + kb * 8192, &map_v, &ms.barLoad, kb * 64, h, tok0, b);
             }
             bool ok = mbar_wait(&ms.barConv, 0, abort_flag);       // tiles converted to fp16
             if (ok) {
-                // ---- fp16 copies of q and k for the scan kernel; [Q ; K] K^T ----
-                for (int kb = 0; kb < KB; ++kb) {
-                    tma_store_2d(&map_qh, sQK + kb * 16384, kb * 64, bh * L + tok0);
-                    tma_store_2d(&map_kh, sQK + kb * 16384 + 8192, kb * 64, bh * L + tok0);
+                // ---- fp16 copies of q and k for the backward; [Q ; K] K^T ----
+                if (kTrain) {
+                    for (int kb = 0; kb < KB; ++kb) {
+                        tma_store_2d(&map_qh, sQK + kb * 16384, kb * 64, bh * L + tok0);
+                        tma_store_2d(&map_kh, sQK + kb * 16384 + 8192, kb * 64, bh * L + tok0);
+                    }
+                    tma_store_commit();
                 }
-                tma_store_commit();
                 tc_fence_after_sync();
                 constexpr uint32_t idesc = make_idesc(kFmtF16, 128, 64, false, false);
                 const uint32_t aQK = smem_u32(sQK);
@@ -157,33 +167,34 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                         mma_ss(tmem, desc_kmajor(aQK + kb * 16384 + k16 * 32),
                                desc_kmajor(aQK + kb * 16384 + 8192 + k16 * 32), idesc, (kb | k16) != 0);
                 mma_commit(&ms.barM);
-                tma_store_wait_read();                    // the q copy has left its blocks
+                if (kTrain) tma_store_wait_read();        // the q copy has left its blocks
                 ok = mbar_wait(&ms.barM, 0, abort_flag);  // and the MMAs have read them
                 mbar_arrive(&ms.barXfree);
             }
             if (ok) ok = mbar_wait(&ms.barT, 0, abort_flag);
             if (ok) {
-                // ---- U^T = V^T (T beta~)^T,  W^T = K^T (T beta~ gamma)^T ----
+                // ---- T beta~ leaves; U^T = V^T (T beta~)^T,  W^T = K^T (T beta~ gamma)^T ----
                 tc_fence_after_sync();
+                tma_store_2d(&map_tb, xLo, 0, (int)chunk * 64);
+                tma_store_commit();
                 const uint32_t aV = smem_u32(sV), aK = smem_u32(sQK) + 8192, aTb = smem_u32(xLo),
                                aTg = smem_u32(xHi);
-                if (D == 128) {
-                    constexpr uint32_t idesc = make_idesc(kFmtF16, 128, 64, true, false);
+                constexpr uint32_t idesc = make_idesc(kFmtF16, 128, 64, true, false);
+                if (D == 128 || !kTrain) {
 #pragma unroll
                     for (int k16 = 0; k16 < 4; ++k16) {
-                        mma_ss(tmem, desc_mnmajor(aV + k16 * 2048, 8192), desc_kmajor(aTb + k16 * 32),
-                               idesc, k16 != 0);
-                        mma_ss(tmem + 64, desc_mnmajor(aK + k16 * 2048, 16384),
-                               desc_kmajor(aTg + k16 * 32), idesc, k16 != 0);
+                        if (kTrain) mma_ss(tmem, desc_mnmajor(aV + k16 * 2048, 8192), desc_kmajor(aTb + k16 * 32), idesc, k16 != 0);
+                        // (d = 64: rows 64-127 of M are of no interest, K again)
+                        mma_ss(tW, desc_mnmajor(aK + k16 * 2048, D == 128 ? 16384 : 0), desc_kmajor(aTg + k16 * 32), idesc, k16 != 0);
                     }
                 } else {
                     // d = 64: rows 0-63 of M are V^T, rows 64-127 are K^T (16 KB further on);
                     // N = 128 = [T beta~ ; T beta~ gamma] (adjacent).
-                    constexpr uint32_t idesc = make_idesc(kFmtF16, 128, 128, true, false);
+                    constexpr uint32_t idesc2 = make_idesc(kFmtF16, 128, 128, true, false);
 #pragma unroll
                     for (int k16 = 0; k16 < 4; ++k16)
                         mma_ss(tmem, desc_mnmajor(aV + k16 * 2048, 16384), desc_kmajor(aTb + k16 * 32),
-                               idesc, k16 != 0);
+                               idesc2, k16 != 0);
                 }
                 mma_commit(&ms.barUW);
             }
@@ -216,8 +227,8 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
             // L2-normalised q and k for the linear operation (Section 4.3): thread r owns row r of
             // [Q ; K] (all KB blocks of it), takes its 16-byte pieces in an order that spreads the warp
             // over the banks, and scales while it converts.  V is converted as below.
-            static_assert(PL::oV == 0 && PL::oQK == KB * 8192, "V tile first, [Q ; K] blocks behind it");
-            for (int idx = r; idx < KB * 8192 / 16; idx += kRowThreads) {
+            static_assert(PL::oV == 0 && PL::oQK == (kTrain ? KB * 8192 : 0), "V tile first, [Q ; K] blocks behind it");
+            for (int idx = r; kTrain && idx < KB * 8192 / 16; idx += kRowThreads) {
                 uint4 *pp = reinterpret_cast<uint4 *>(smem) + idx;
                 *pp = bf16x8_to_f16x8(*pp);
             }
@@ -236,6 +247,7 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                     }
                 }
             const float rn = rsqrtf(ss + norm_eps);
+            Rn[chunk * 128 + r] = rn;                          // (q's rows, k's rows: the scan scales them likewise)
 #pragma unroll
             for (int kb = 0; kb < KB; ++kb)
 #pragma unroll
@@ -284,11 +296,21 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                         // expression compiles to one divergent branch per element
                         x[e] = scale_la * exp_ftz(j <= i ? G - ms.G[j] : -INFINITY) * __uint_as_float(d8[e]);
                     }
-                    prow[pc] = make_uint4(pack_half2(x[0], x[1]), pack_half2(x[2], x[3]),
-                                          pack_half2(x[4], x[5]), pack_half2(x[6], x[7]));
+                    const uint4 pw = make_uint4(pack_half2(x[0], x[1]), pack_half2(x[2], x[3]),
+                                                pack_half2(x[4], x[5]), pack_half2(x[6], x[7]));
+                    if (kTrain) prow[pc] = pw;
+                    else *reinterpret_cast<uint4 *>(sP + sw128_offset(i, pc)) = pw;
                 }
                 tc_fence_before_sync();
                 mbar_arrive(&ms.barT);
+                if (!kTrain) {
+                    fence_proxy_async_smem();
+                    named_barrier_sync(1, 64);
+                    if (tid == 0) {
+                        tma_store_2d(&map_ph, sP, 0, (int)chunk * 64);
+                        tma_store_commit();
+                    }
+                }
             } else {
                 // ---- T = (I + A)^-1 with 16x16 blocks (T_bb = (I + A_bb)^-1 in fp32 registers; below the
                 // diagonal T_10 = -T_11 A_10 T_00, T_32 likewise, then the 32x32 block
@@ -461,55 +483,52 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
             ok = mbar_wait(&ms.barUW, 0, abort_flag);
         }
         if (ok) {
-            // ---- U^T (fp32) and W^T (fp16) rows to global; thread r <-> head-dimension row ----
+            // ---- (U^T and) W^T as fp16 tiles, over V and K; thread r <-> head-dimension row ----
             tc_fence_after_sync();
-            const bool do_u = D == 128 || r < 64, do_w = D == 128 || r >= 64;
-            const int row = D == 128 ? r : i;
-            uint32_t x[2][32];
-            if (do_u) {                                     // warp-uniform
-                tmem_ld32(tmem + lane_base, x[0]);
-                tmem_ld32(tmem + lane_base + 32, x[1]);
+            auto stage = [&](uint32_t from, uint8_t *tile, int row) {
+                uint32_t x[2][32];
+                tmem_ld32(from + lane_base, x[0]);
+                tmem_ld32(from + lane_base + 32, x[1]);
                 tmem_wait_ld();
-                // piece-major: 16-byte piece pc (4 tokens) of all D rows is contiguous, so that a
-                // warp's stores here and its loads in the scan are fully coalesced
-                uint4 *dst = reinterpret_cast<uint4 *>(Ut + chunk * D * 64) + row;
-#pragma unroll
-                for (int pc = 0; pc < 16; ++pc)
-                    dst[pc * D] = make_uint4(x[pc >> 3][(4 * pc) & 31], x[pc >> 3][(4 * pc + 1) & 31],
-                                             x[pc >> 3][(4 * pc + 2) & 31], x[pc >> 3][(4 * pc + 3) & 31]);
-                if (ex.U16) {    // fp16 copy for the backward, in the layout of W^T
-                    uint4 *uh = reinterpret_cast<uint4 *>(reinterpret_cast<__half *>(ex.U16) + (chunk * D + row) * 64);
-#pragma unroll
-                    for (int pc = 0; pc < 8; ++pc) {
-                        const uint32_t *xx = &x[pc >> 2][(8 * pc) & 31];
-                        uh[pc] = make_uint4(pack_half2(__uint_as_float(xx[0]), __uint_as_float(xx[1])),
-                                            pack_half2(__uint_as_float(xx[2]), __uint_as_float(xx[3])),
-                                            pack_half2(__uint_as_float(xx[4]), __uint_as_float(xx[5])),
-                                            pack_half2(__uint_as_float(xx[6]), __uint_as_float(xx[7])));
-                    }
-                }
-            }
-            if (do_w) {
-                tmem_ld32(tmem + lane_base + 64, x[0]);
-                tmem_ld32(tmem + lane_base + 96, x[1]);
-                tmem_wait_ld();
-                uint4 *dst = reinterpret_cast<uint4 *>(Wt + (chunk * D + row) * 64);
 #pragma unroll
                 for (int pc = 0; pc < 8; ++pc) {
                     const uint32_t *xx = &x[pc >> 2][(8 * pc) & 31];
-                    dst[pc] = make_uint4(pack_half2(__uint_as_float(xx[0]), __uint_as_float(xx[1])),
-                                         pack_half2(__uint_as_float(xx[2]), __uint_as_float(xx[3])),
-                                         pack_half2(__uint_as_float(xx[4]), __uint_as_float(xx[5])),
-                                         pack_half2(__uint_as_float(xx[6]), __uint_as_float(xx[7])));
+                    *reinterpret_cast<uint4 *>(tile + sw128_offset(row, pc)) =
+                        make_uint4(pack_half2(__uint_as_float(xx[0]), __uint_as_float(xx[1])),
+                                   pack_half2(__uint_as_float(xx[2]), __uint_as_float(xx[3])),
+                                   pack_half2(__uint_as_float(xx[4]), __uint_as_float(xx[5])),
+                                   pack_half2(__uint_as_float(xx[6]), __uint_as_float(xx[7])));
                 }
+            };
+            uint8_t *sK = sQK + 8192;                          // a 64-row block of W^T per K block
+            if (D == 128) {
+                if (kTrain) stage(tmem, sV + (r >> 6) * 8192, i);
+                stage(tW, sK + (r >> 6) * 16384, i);
+            } else if (kTrain) {                               // (warp-uniform: rows 0-63 U^T, rows 64-127 W^T)
+                if (r < 64) stage(tmem, sV, i);
+                else stage(tW, sK, i);
+            } else if (r < 64) {
+                stage(tW, sK, i);
             }
+            fence_proxy_async_smem();
+        }
+        named_barrier_sync(3, kRowThreads);
+        if (tid == 0) {
+            if (ok) {
+                for (int kb = 0; kb < KB; ++kb) {
+                    if (kTrain) tma_store_2d(&map_u16, sV + kb * 8192, 0, (int)(chunk * D) + kb * 64);
+                    tma_store_2d(&map_wt, sQK + 8192 + kb * 16384, 0, (int)(chunk * D) + kb * 64);
+                }
+                tma_store_commit();
+            }
+            tma_store_wait_all();
         }
     }
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 4) {
         tc_fence_after_sync();
-        tmem_dealloc(tmem, 128);
+        tmem_dealloc(tmem, PL::kTmemCols);
     }
     if (tid == 0 && ms.abort_flag) atomicMin(status, (int)NATSL_ERR_TIMEOUT);
 }
@@ -518,14 +537,23 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
 // Scan: one CTA per (batch, head) -- or per segment of its chunks, see ScanSegments --, sequential
 // over chunks.  Value column r of the state (row r of
 // S^T, TMEM lane r) belongs to the two threads (r, half 0) and (r, half 1) of warps q and q + 4,
-// which split every row between them; warp 8 issues MMAs, warp 9 issues TMA.  The fp32 state
+// which split every row between them; warps 8 and 11 issue MMAs, warp 9 issues TMA, warps 12-15 turn the q, k and v tiles
+// into fp16.  The fp32 state
 // lives in the registers of its two threads (half a row each); per chunk c:
-//   (a) S_c (fp16 operand) -> TMEM;                          MMA: WS = S^T W^T, QS = S^T Q^T
-//   (b) U~^T = U^T - WS  -> operands U~ and U~ diag(gamma_C/gamma);
-//                                      MMA: dS = (U~ diag(gamma_C/gamma))^T-rows x K,  D3 = U~^T P^T
-//   (c) [for chunk c-1, behind the MMAs of (b)]  o_la^T = scale_la diag(gamma) QS + D3
+//   (0) [ahead of the chunk]                                 MMA: X = U^T = V^T (T beta~)^T
+//   (a) S_c (fp16 operand, in two parts) -> TMEM;            MMA: X -= S^T W^T, QS = S^T Q^T
+//   (b) X = U~^T  -> operands U~ diag(gamma_C/gamma) and U~;
+//                                      MMA: dS = (U~ diag(gamma_C/gamma))^T-rows x K,  X = U~^T P^T
+//   (c) [for chunk c-1, half behind the MMAs of (a), half behind those of (b)]  o_la^T = scale_la diag(gamma) QS + X
 //   next chunk: S_{c+1} = gamma_C S_c + dS
-// QS and D3 are double-buffered in TMEM so that (c) of chunk c-1 runs behind the MMAs of chunk c.
+// QS and X are double-buffered in TMEM so that (c) of chunk c-1 runs behind the MMAs of chunk c; its X buffer is then
+// that of (0) of chunk c+1.  (U from the prepare kernel in fp32, and q and k from it in fp16, were 64 of the 88 KB that a
+// chunk took through HBM and back: the prepare kernel bounds the call.)
+// What bounds a chunk is the chain (a), (b): the row threads' conversions, each behind a product whose latency is its
+// issue and 150 cycles.  One lane issuing from its own loop took 80 to 100 cycles an instruction (see elect_one in
+// tc_common.cuh), and the warp that issues the chain must not wait for anything else, hence the second one; the
+// converting warps cost 15 % of the chunk by their shared-memory traffic.  64 chunks of 128 columns: 121 us with U, q, k
+// prepared and one issuing lane; 156 with the conversions here, 127 with uniform issue, two parts and two issuing warps.
 // The read-out leaves the kernel as fp16 in the orientation the row threads hold it in, one tile
 // per chunk in 16-byte pieces of 8 tokens: o_laT [B,H,L/C,8 pieces,d,8 tokens], row r of piece p at
 // slot r ^ p.  A thread then stores four 16-byte pieces per chunk and a warp's store is 512
@@ -535,10 +563,13 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
 // those reads free of bank conflicts.  Warp 10 publishes the per-chunk completion counters for a kernel that
 // consumes o_laT beside this one: the release fence costs a few thousand cycles and must not sit
 // on the row threads' chain.
+// Registers: 512 threads start with 128; the row threads' two warpgroups go up to 176, the other two down to 80, which
+// is the same sum.
 // ==========================================================================================
 constexpr int kScanRowThreads = 256;
-constexpr int kScanThreads = 352;
-constexpr int kScanStages = 3;
+constexpr int kScanThreads = 512;
+constexpr int kScanConvThreads = 128;
+constexpr int kScanStages = 3, kScanVStages = 2;
 constexpr int kScanMisc = 1024;
 constexpr int kDecaySlots = 8;                             // ring of per-chunk decay factors
 
@@ -548,23 +579,28 @@ template <int D> struct ScanLayout {
     static constexpr int kQ = KB * 8192;                   // Q tile: 64 tokens x D
     static constexpr int kK = KB * 8192;
     static constexpr int kP = 8192;
-    static constexpr int kG = 512;                         // gamma_i and gamma_C / gamma_i, 64 each
+    static constexpr int kG = 512;                         // gamma_i and gamma_C / gamma_i, 64 each; likewise Rn
     static constexpr int oW = 0, oQ = oW + kW, oK = oQ + kQ, oP = oK + kK;
     static constexpr int kStage = oP + kP;
-    static constexpr int kTx = kStage + kG;
-    static constexpr int oG = kScanStages * kStage;        // decay ring
-    static constexpr int oMisc = oG + kDecaySlots * kG;
+    static constexpr int kV = KB * 8192, kVStage = kV + 8192;   // V tile, T beta~
+    static constexpr int oV = kScanStages * kStage;
+    static constexpr int oG = oV + kScanVStages * kVStage;      // ring of decay factors, ring of q's and k's row factors
+    static constexpr int oR = oG + kDecaySlots * kG;
+    static constexpr int oMisc = oR + kDecaySlots * kG;
     static constexpr int kTotal = oMisc + kScanMisc;
     static constexpr int kTmemCols = 512;
-    // TMEM columns.  dS: fp32 state increment [D].  WS: fp32 W S [64], overwritten by each thread
-    // with its fp16 operands (U~ | U~ diag(gamma_C/gamma), 16 + 16 packed columns per 32 tokens).
-    // A: the fp16 state operand [D/2 packed].  QS, D3: double-buffered fp32 [64] each.
-    static constexpr int cS = 0, cWS = D, cA = D + 64, cQS = cA + D / 2, cD3 = cQS + 128;
-    static_assert(cD3 + 128 <= 512, "TMEM budget");
+    // TMEM columns.  dS: fp32 state increment [D].  U: the fp16 operands of each thread's 32 tokens (U~ | U~
+    // diag(gamma_C/gamma), 16 + 16 packed columns).  A: the fp16 state operand [D/2 packed].  QS, X: double-buffered
+    // fp32 [64] each; X is U, then U~, then P U~ of its chunk.
+    static constexpr int cS = 0, cU = D, cA = D + 64, cQS = cA + D / 2, cX = cQS + 128;
+    static_assert(cX + 128 <= 512, "TMEM budget");
+    static constexpr int kParts = D / 64;                  // parts of 32 columns in which a thread's half row is handed over
+    static_assert(kTotal <= 227 * 1024, "shared memory");
 };
 
 struct ScanMisc {
-    uint64_t full[kScanStages], empty[kScanStages], barA, barWS, barQS[2], barB, barSU, barD3[2];
+    uint64_t full[kScanStages], empty[kScanStages], conv[kScanStages], fullV[kScanVStages], emptyV[kScanVStages],
+        convV[kScanVStages], barA[2], barU, barWS, barB, barB2, barSU, barD3[2], barE;
     uint32_t tmem_base;
     int abort_flag, wait_kcycles;   // in this order: the waits read the limit as abort_flag[1]
     int emit_count;                 // row warps x chunks whose read-out rows have been stored
@@ -574,10 +610,11 @@ static_assert(sizeof(ScanMisc) <= kScanMisc, "misc page too small");
 template <int D, bool kBlock>      // kBlock: block-level routing (softmax blocks are not committed)
 __global__ void __launch_bounds__(kScanThreads, 1)
 gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
-                   const __grid_constant__ CUtensorMap map_qh,
-                   const __grid_constant__ CUtensorMap map_kh,
-                   const __grid_constant__ CUtensorMap map_ph, const float *__restrict__ Ut,
-                   const float *__restrict__ Gd, float scale_la,
+                   const __grid_constant__ CUtensorMap map_q,      // the layer's q, k, v [B,L,H,D] bf16, box 64 x 64
+                   const __grid_constant__ CUtensorMap map_k,
+                   const __grid_constant__ CUtensorMap map_v,
+                   const __grid_constant__ CUtensorMap map_ph, const __grid_constant__ CUtensorMap map_tb,
+                   const float *__restrict__ Gd, const float *__restrict__ Rn, float scale_la,
                    const float *__restrict__ state_in, float *__restrict__ state_out,
                    __half *__restrict__ o_la16, float *__restrict__ o_la32, int32_t *emit_flags,
                    GdnTcExport ex, ScanSegments sg,
@@ -613,12 +650,20 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
         return;
     }
     if (tid == 0) {
-        for (int s = 0; s < kScanStages; ++s) { mbar_init(&ms.full[s], 1); mbar_init(&ms.empty[s], 1); }
-        mbar_init(&ms.barA, kScanRowThreads);
+        for (int s = 0; s < kScanStages; ++s) {
+            mbar_init(&ms.full[s], 1); mbar_init(&ms.empty[s], 1); mbar_init(&ms.conv[s], kScanConvThreads);
+        }
+        for (int s = 0; s < kScanVStages; ++s) {
+            mbar_init(&ms.fullV[s], 1); mbar_init(&ms.emptyV[s], 1); mbar_init(&ms.convV[s], kScanConvThreads);
+        }
+        mbar_init(&ms.barE, kScanRowWarps);
+        for (int s = 0; s < 2; ++s) mbar_init(&ms.barA[s], kScanRowThreads);
         mbar_init(&ms.barB, kScanRowThreads);
+        mbar_init(&ms.barB2, kScanRowThreads);
+        mbar_init(&ms.barU, 1);
         mbar_init(&ms.barWS, 1);
         mbar_init(&ms.barSU, 1);
-        for (int s = 0; s < 2; ++s) { mbar_init(&ms.barQS[s], 1); mbar_init(&ms.barD3[s], 1); }
+        for (int s = 0; s < 2; ++s) mbar_init(&ms.barD3[s], 1);
         ms.abort_flag = 0;
         ms.wait_kcycles = wait_kcycles;
         ms.emit_count = 0;
@@ -636,102 +681,193 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
     grid_dependency_wait();
     launch_dependents();
 
-    if (warp == 9) {
-        if (lane == 0) {
-            int c = 0;
-            for (; c < ncs; ++c) {
-                const int s = c % kScanStages;
-                if (!mbar_wait(&ms.empty[s], ((c / kScanStages) & 1) ^ 1, abort_flag)) break;
-                uint8_t *st = smem + s * SL::kStage;
-                mbar_arrive_expect_tx(&ms.full[s], SL::kTx);
-                tma_load_2d(st + SL::oW, &map_wt, &ms.full[s], 0, (bh * NC + c0 + c) * D);
-                for (int kb = 0; kb < KB; ++kb) {
-                    tma_load_2d(st + SL::oQ + kb * 8192, &map_qh, &ms.full[s], kb * 64, bh * L + (c0 + c) * 64);
-                    tma_load_2d(st + SL::oK + kb * 8192, &map_kh, &ms.full[s], kb * 64, bh * L + (c0 + c) * 64);
+    if (warp >= 8) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
+        if (warp == 9) {
+            if (lane == 0) {
+                int c = 0, nv = 0;
+                bool ok = true;
+                const uint32_t tx = SL::kW + SL::kK + SL::kG + (emit_out ? SL::kQ + SL::kP : 0) + (Rn ? SL::kG : 0);
+                for (; c < ncs; ++c) {
+                    const int s = c % kScanStages, sv = c % kScanVStages, tok = (c0 + c) * 64;
+                    const size_t chunk = (size_t)bh * NC + c0 + c;
+                    if (!zero_u) {
+                        ok = mbar_wait(&ms.emptyV[sv], ((c / kScanVStages) & 1) ^ 1, abort_flag);
+                        if (!ok) break;
+                        uint8_t *sp = smem + SL::oV + sv * SL::kVStage;
+                        mbar_arrive_expect_tx(&ms.fullV[sv], SL::kVStage);
+                        for (int kb = 0; kb < KB; ++kb) tma_load_4d(sp + kb * 8192, &map_v, &ms.fullV[sv], kb * 64, h, tok, b);
+                        tma_load_2d(sp + SL::kV, &map_tb, &ms.fullV[sv], 0, (int)chunk * 64);
+                        nv = c + 1;
+                    }
+                    ok = mbar_wait(&ms.empty[s], ((c / kScanStages) & 1) ^ 1, abort_flag);
+                    if (!ok) break;
+                    uint8_t *st = smem + s * SL::kStage;
+                    mbar_arrive_expect_tx(&ms.full[s], tx);
+                    tma_load_2d(st + SL::oW, &map_wt, &ms.full[s], 0, (int)(chunk * D));
+                    for (int kb = 0; kb < KB; ++kb) {
+                        if (emit_out) tma_load_4d(st + SL::oQ + kb * 8192, &map_q, &ms.full[s], kb * 64, h, tok, b);
+                        tma_load_4d(st + SL::oK + kb * 8192, &map_k, &ms.full[s], kb * 64, h, tok, b);
+                    }
+                    if (emit_out) tma_load_2d(st + SL::oP, &map_ph, &ms.full[s], 0, (int)chunk * 64);
+                    // A decay slot is reused kDecaySlots chunks later, i.e. only after the stages of the
+                    // chunks up to c + kDecaySlots - kScanStages have been released, which every row
+                    // thread's work on chunk c precedes.
+                    bulk_load_1d(smem + SL::oG + (c % kDecaySlots) * SL::kG, Gd + chunk * 128, SL::kG, &ms.full[s]);
+                    if (Rn) bulk_load_1d(smem + SL::oR + (c % kDecaySlots) * SL::kG, Rn + chunk * 128, SL::kG, &ms.full[s]);
                 }
-                tma_load_2d(st + SL::oP, &map_ph, &ms.full[s], 0, (bh * NC + c0 + c) * 64);
-                // A decay slot is reused kDecaySlots chunks later, i.e. only after the stages of the
-                // chunks up to c + kDecaySlots - kScanStages have been released, which every row
-                // thread's work on chunk c precedes.
-                bulk_load_1d(smem + SL::oG + (c % kDecaySlots) * SL::kG,
-                             Gd + ((size_t)bh * NC + c0 + c) * 128, SL::kG, &ms.full[s]);
+                // No copy may be in flight when the CTA retires: the copies issued last are waited for
+                // here, with a bound of their own and whatever the abort flag says.
+                for (int u = max(0, c - kScanStages); u < c; ++u)
+                    mbar_wait_drain(&ms.full[u % kScanStages], (u / kScanStages) & 1);
+                for (int u = max(0, nv - kScanVStages); u < nv; ++u)
+                    mbar_wait_drain(&ms.fullV[u % kScanVStages], (u / kScanVStages) & 1);
             }
-            // No copy may be in flight when the CTA retires: the copies issued last are waited for
-            // here, with a bound of their own and whatever the abort flag says.
-            for (int u = max(0, c - kScanStages); u < c; ++u)
-                mbar_wait_drain(&ms.full[u % kScanStages], (u / kScanStages) & 1);
-        }
-    } else if (warp == 8) {
-        if (lane == 0) {
-            constexpr uint32_t id_ws = make_idesc(kFmtF16, 128, 64, false, true);    // B = W^T (MN-major)
+        } else if (warp >= 12) {
+            // ---- q, k, v tiles to fp16 in place (as given, exactly; normalised, times the row's factor) ----
+            const int t = tid - 12 * 32;
+            auto convert = [&](uint8_t *tile, const float *rn) {
+                uint4 *pp = reinterpret_cast<uint4 *>(tile);
+#pragma unroll 4
+                for (int i = 0; i < KB * 8192 / 16 / kScanConvThreads; ++i) {
+                    const int idx = t + i * kScanConvThreads;
+                    uint4 a = pp[idx];
+                    if (rn) {
+                        const float f = rn[(idx >> 3) & 63];
+                        const uint32_t wd[4] = {a.x, a.y, a.z, a.w};
+                        uint32_t o[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            o[e] = pack_half2(__uint_as_float(wd[e] << 16) * f, __uint_as_float(wd[e] & 0xffff0000u) * f);
+                        a = make_uint4(o[0], o[1], o[2], o[3]);
+                    } else {
+                        a = bf16x8_to_f16x8(a);
+                    }
+                    pp[idx] = a;
+                }
+            };
+            for (int c = 0; c < ncs; ++c) {
+                const int s = c % kScanStages, sv = c % kScanVStages;
+                if (!zero_u) {
+                    if (!mbar_wait(&ms.fullV[sv], (c / kScanVStages) & 1, abort_flag)) break;
+                    convert(smem + SL::oV + sv * SL::kVStage, nullptr);
+                    fence_proxy_async_smem();
+                    mbar_arrive(&ms.convV[sv]);
+                }
+                if (!mbar_wait(&ms.full[s], (c / kScanStages) & 1, abort_flag)) break;
+                const float *rn = Rn ? reinterpret_cast<const float *>(smem + SL::oR + (c % kDecaySlots) * SL::kG) : nullptr;
+                if (emit_out) convert(smem + s * SL::kStage + SL::oQ, rn);
+                convert(smem + s * SL::kStage + SL::oK, rn ? rn + 64 : nullptr);
+                fence_proxy_async_smem();
+                mbar_arrive(&ms.conv[s]);
+            }
+        } else if (warp == 8) {
+            constexpr uint32_t id_ws = make_idesc(kFmtF16, 128, 64, false, true, true);    // A = -S^T, B = W^T (MN-major)
             constexpr uint32_t id_qs = make_idesc(kFmtF16, 128, 64, false, false);   // B = Q
             constexpr uint32_t id_su = make_idesc(kFmtF16, 128, D, false, true);     // B = K (MN-major)
             constexpr uint32_t id_pu = make_idesc(kFmtF16, 128, 64, false, false);   // B = P
-            for (int c = 0; c < ncs; ++c) {
+            const uint32_t tm = uniform(tmem), sm = smem_u32(smem);
+            bool ok = true;
+            for (int c = 0; c < ncs && ok; ++c) {
                 const int s = c % kScanStages;
-                const uint32_t st = smem_u32(smem + s * SL::kStage);
-                if (!mbar_wait(&ms.full[s], (c / kScanStages) & 1, abort_flag)) break;
-                if (!mbar_wait(&ms.barA, c & 1, abort_flag)) break;
-                tc_fence_after_sync();
+                const uint32_t st = sm + s * SL::kStage, tX = tm + SL::cX + 64 * (c & 1);
+                if (!wait_all(&ms.conv[s], (c / kScanStages) & 1, abort_flag)) break;      // (and so the stage's copies)
+                if (!zero_u && !wait_all(&ms.barU, c & 1, abort_flag)) break;
+                // (the state's columns arrive in parts of 32 of each half of the row)
 #pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk)
-                    mma_ts(tmem + SL::cWS, tmem + SL::cA + kk * 8,
-                           desc_mnmajor(st + SL::oW + kk * 2048, 0), id_ws, kk != 0);
-                mma_commit(&ms.barWS);
-                if (emit_out) {
+                for (int pt = 0; pt < SL::kParts; ++pt) {
+                    ok = ok && wait_all(&ms.barA[pt], c & 1, abort_flag);
+                    if (!ok) break;
+                    tc_fence_after_sync();
+                    if (elect_one()) {
+#pragma unroll
+                        for (int k4 = 0; k4 < 4; ++k4) {
+                            const int kk = D == 128 ? (k4 >> 1) * 4 + pt * 2 + (k4 & 1) : k4;
+                            mma_ts(tX, tm + SL::cA + kk * 8, desc_mnmajor(st + SL::oW + kk * 2048, 0), id_ws, !zero_u || (pt | k4) != 0);
+                        }
+                        if (pt == SL::kParts - 1) mma_commit(&ms.barWS);
+                    }
+                }
+                if (!ok) break;
+                if (emit_out && elect_one()) {
 #pragma unroll
                     for (int kk = 0; kk < D / 16; ++kk)
-                        mma_ts(tmem + SL::cQS + 64 * (c & 1), tmem + SL::cA + kk * 8,
+                        mma_ts(tm + SL::cQS + 64 * (c & 1), tm + SL::cA + kk * 8,
                                desc_kmajor(st + SL::oQ + (kk >> 2) * 8192 + (kk & 3) * 32), id_qs, kk != 0);
-                    mma_commit(&ms.barQS[c & 1]);
                 }
-                if (!mbar_wait(&ms.barB, c & 1, abort_flag)) break;
+                if (!wait_all(&ms.barB, c & 1, abort_flag)) break;
                 tc_fence_after_sync();
                 // The state update first: it is on the chain between the chunks.  The output product
-                // behind it still reads its operand from the WS columns after barSU has fired; the
-                // next writer of those columns is the next chunk's W S product, issued behind it by
+                // behind it still reads its operand from the U columns after barSU has fired; the
+                // row threads write those again behind the next chunk's W S product, issued behind it by
                 // this thread, and MMAs of one thread execute in issue order.
-#pragma unroll
-                for (int k16 = 0; k16 < 4; ++k16)
-                    mma_ts(tmem + SL::cS, tmem + SL::cWS + (k16 >> 1) * 32 + 16 + (k16 & 1) * 8,
-                           desc_mnmajor(st + SL::oK + k16 * 2048, 8192), id_su, k16 != 0);
-                mma_commit(&ms.barSU);
-                if (emit_out) {
+                if (elect_one()) {
 #pragma unroll
                     for (int k16 = 0; k16 < 4; ++k16)
-                        mma_ts(tmem + SL::cD3 + 64 * (c & 1), tmem + SL::cWS + (k16 >> 1) * 32 + (k16 & 1) * 8,
-                               desc_kmajor(st + SL::oP + k16 * 32), id_pu, k16 != 0);
-                    mma_commit(&ms.barD3[c & 1]);
+                        mma_ts(tm + SL::cS, tm + SL::cU + (k16 >> 1) * 32 + 16 + (k16 & 1) * 8,
+                               desc_mnmajor(st + SL::oK + k16 * 2048, 8192), id_su, k16 != 0);
+                    mma_commit(&ms.barSU);
                 }
-                mma_commit(&ms.empty[s]);
+                if (!wait_all(&ms.barB2, c & 1, abort_flag)) break;
+                tc_fence_after_sync();
+                if (elect_one()) {
+                    if (emit_out) {
+#pragma unroll
+                        for (int k16 = 0; k16 < 4; ++k16)
+                            mma_ts(tX, tm + SL::cU + (k16 >> 1) * 32 + (k16 & 1) * 8, desc_kmajor(st + SL::oP + k16 * 32), id_pu, k16 != 0);
+                        mma_commit(&ms.barD3[c & 1]);
+                    }
+                    mma_commit(&ms.empty[s]);
+                }
             }
-        }
-    } else if (warp == 10) {
-        // Publisher: raises the per-chunk counters once all eight row warps have stored a chunk's
-        // rows.  The row warps count in shared memory (after a block-scope fence); the gpu-scope
-        // fence here then covers their stores, as in the usual "barrier, one thread fences and
-        // sets the flag" hand-over.  Several chunks are published behind one fence when it lags.
-        if (lane == 0 && emit_flags && emit_out) {
-            volatile int *cnt = &ms.emit_count;
-            const long long limit = wait_limit(abort_flag);
-            long long t0 = clock64();
-            int published = 0;
-            while (published < ncs) {
-                const int done = *cnt / kScanRowWarps;
-                if (done > published) {
-                    __threadfence();
-                    for (int c = published; c < done; ++c)
-                        red_release_add(emit_flags + (size_t)bh * NC + c0 + c, kScanRowWarps);
-                    published = done;
-                    t0 = clock64();
-                } else {
-                    if (*abort_flag) break;
-                    if (clock64() - t0 > limit) { *abort_flag = 1; break; }
-                    __nanosleep(128);
+        } else if (warp == 11) {
+            // X of a chunk = U^T, ahead of it: once the read-out of the chunk two before has left the buffer
+            constexpr uint32_t id_u = make_idesc(kFmtF16, 128, 64, true, false);     // A = V^T (MN-major), B = T beta~
+            const uint32_t tm = uniform(tmem), sm = smem_u32(smem);
+            for (int c = 0; c < ncs && !zero_u; ++c) {
+                const int sv = c % kScanVStages;
+                const uint32_t sp = sm + SL::oV + sv * SL::kVStage, tX = tm + SL::cX + 64 * (c & 1);
+                if (!wait_all(&ms.convV[sv], (c / kScanVStages) & 1, abort_flag)) break;        // (and so the copies)
+                // (the second chunk's, and without read-outs: once W S of the chunk before has run.  Either way no barrier here
+                // can get two phases ahead of who waits for it: what completes its next phase needs this product first.)
+                if (c > 0 && !(emit_out && c > 1 ? wait_all(&ms.barE, c & 1, abort_flag) : wait_all(&ms.barWS, (c - 1) & 1, abort_flag))) break;
+                tc_fence_after_sync();
+                if (elect_one()) {
+#pragma unroll
+                    for (int k16 = 0; k16 < 4; ++k16)              // (d = 64: rows 64-127 are of no interest, V again)
+                        mma_ss(tX, desc_mnmajor(sp + k16 * 2048, D == 128 ? 8192 : 0), desc_kmajor(sp + SL::kV + k16 * 32), id_u, k16 != 0);
+                    mma_commit(&ms.emptyV[sv]);
+                    mma_commit(&ms.barU);
+                }
+            }
+        } else if (warp == 10) {
+            // Publisher: raises the per-chunk counters once all eight row warps have stored a chunk's
+            // rows.  The row warps count in shared memory (after a block-scope fence); the gpu-scope
+            // fence here then covers their stores, as in the usual "barrier, one thread fences and
+            // sets the flag" hand-over.  Several chunks are published behind one fence when it lags.
+            if (lane == 0 && emit_flags && emit_out) {
+                volatile int *cnt = &ms.emit_count;
+                const long long limit = wait_limit(abort_flag);
+                long long t0 = clock64();
+                int published = 0;
+                while (published < ncs) {
+                    const int done = *cnt / kScanRowWarps;
+                    if (done > published) {
+                        __threadfence();
+                        for (int c = published; c < done; ++c)
+                            red_release_add(emit_flags + (size_t)bh * NC + c0 + c, kScanRowWarps);
+                        published = done;
+                        t0 = clock64();
+                    } else {
+                        if (*abort_flag) break;
+                        if (clock64() - t0 > limit) { *abort_flag = 1; break; }
+                        __nanosleep(128);
+                    }
                 }
             }
         }
     } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 176;");
         const int q = warp & 3, half = warp >> 2;
         const int r = q * 32 + lane;                      // value column / TMEM lane
         const bool active = r < D;                        // d = 64: rows 64-127 are zero padding
@@ -750,56 +886,47 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
 #pragma unroll
             for (int x = 0; x < kHalfCols; ++x) S[x] = zero_u && active && col0 + x == r ? 1.f : 0.f;
         }
-        // This thread's 8 pieces (4 tokens each) of row r of U^T of chunk c.
-        auto u_src = [&](int c) {
-            return reinterpret_cast<const float4 *>(Ut + ((size_t)bh * NC + c0 + c) * D * 64) + (tk0 / 4) * D + r;
-        };
-        // The U row of the next chunk is only pulled into L2 ahead of time and loaded into registers
-        // right before it is used: a global load left in flight across TMEM loads makes their
-        // consumers wait for it as well.
-        auto prefetch_u = [&](int c) {
-            if (active && !zero_u) {
-                const float4 *src = u_src(c);
-#pragma unroll
-                for (int x = 0; x < 8; ++x) prefetch_l2(src + x * D);
+        // (c): output rows of chunk c (its QS / X buffers and decay slot are still intact), 16 of this thread's 32 tokens
+        auto emit = [&](int c, int part) -> bool {
+            const float *e1 = reinterpret_cast<const float *>(smem + SL::oG + (c % kDecaySlots) * SL::kG) + tk0 + 16 * part;
+            if (part == 0) {                               // (q S ran ahead of it)
+                if (!mbar_wait(&ms.barD3[c & 1], (c >> 1) & 1, abort_flag)) return false;
+                tc_fence_after_sync();
             }
-        };
-        // (c): output rows of chunk c (its QS / D3 buffers and decay slot are still intact)
-        auto emit = [&](int c) -> bool {
-            const float *e1 = reinterpret_cast<const float *>(smem + SL::oG + (c % kDecaySlots) * SL::kG);
-            if (!mbar_wait(&ms.barQS[c & 1], (c >> 1) & 1, abort_flag)) return false;
-            if (!mbar_wait(&ms.barD3[c & 1], (c >> 1) & 1, abort_flag)) return false;
-            tc_fence_after_sync();
-            const size_t off = (((size_t)b * L + (size_t)(c0 + c) * 64 + tk0) * H + h) * D + r;
-            uint32_t pk[16];                               // this thread's 32 tokens of row r, fp16 pairs
+            uint32_t x[16], y[16];
+            tmem_ld16(tmem + SL::cQS + 64 * (c & 1) + tk0 + 16 * part + lane_base, x);
+            tmem_ld16(tmem + SL::cX + 64 * (c & 1) + tk0 + 16 * part + lane_base, y);
+            tmem_wait_ld();
+            tc_fence_before_sync();
+            if (part == 1) {                               // this warp has read both buffers
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&ms.barE);
+            }
+            float o[16];
 #pragma unroll
-            for (int part = 0; part < 2; ++part) {        // 16 tokens at a time keeps registers low
-                uint32_t x[16], y[16];
-                tmem_ld16(tmem + SL::cQS + 64 * (c & 1) + tk0 + 16 * part + lane_base, x);
-                tmem_ld16(tmem + SL::cD3 + 64 * (c & 1) + tk0 + 16 * part + lane_base, y);
-                tmem_wait_ld();
-                float o[16];
+            for (int i = 0; i < 16; i += 4) {
+                const float4 f = *reinterpret_cast<const float4 *>(e1 + i);
+                o[i] = fmaf(scale_la * f.x, __uint_as_float(x[i]), __uint_as_float(y[i]));
+                o[i + 1] = fmaf(scale_la * f.y, __uint_as_float(x[i + 1]), __uint_as_float(y[i + 1]));
+                o[i + 2] = fmaf(scale_la * f.z, __uint_as_float(x[i + 2]), __uint_as_float(y[i + 2]));
+                o[i + 3] = fmaf(scale_la * f.w, __uint_as_float(x[i + 3]), __uint_as_float(y[i + 3]));
+            }
+            if (o_la32 && active) {                        // fp32 token-major copy (tests, backward)
+                const size_t off = (((size_t)b * L + (size_t)(c0 + c) * 64 + tk0 + 16 * part) * H + h) * D + r;
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    o[i] = fmaf(scale_la * e1[tk0 + 16 * part + i], __uint_as_float(x[i]), __uint_as_float(y[i]));
-#pragma unroll
-                for (int i = 0; i < 8; ++i) pk[8 * part + i] = pack_half2(o[2 * i], o[2 * i + 1]);
-                if (o_la32 && active) {                    // fp32 token-major copy (tests, backward)
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) o_la32[off + (size_t)(16 * part + i) * H * D] = o[i];
-                }
+                for (int i = 0; i < 16; ++i) o_la32[off + (size_t)i * H * D] = o[i];
             }
             if (active) {
                 uint4 *dst = reinterpret_cast<uint4 *>(o_la16 + ((size_t)bh * NC + c0 + c) * D * 64);
 #pragma unroll
-                for (int x4 = 0; x4 < 4; ++x4) {
-                    const int pc = tk0 / 8 + x4;
-                    dst[pc * D + (r ^ pc)] = make_uint4(pk[4 * x4], pk[4 * x4 + 1], pk[4 * x4 + 2], pk[4 * x4 + 3]);
+                for (int x4 = 0; x4 < 2; ++x4) {
+                    const int pc = tk0 / 8 + 2 * part + x4;
+                    dst[pc * D + (r ^ pc)] = make_uint4(pack_half2(o[8 * x4], o[8 * x4 + 1]), pack_half2(o[8 * x4 + 2], o[8 * x4 + 3]),
+                                                        pack_half2(o[8 * x4 + 4], o[8 * x4 + 5]), pack_half2(o[8 * x4 + 6], o[8 * x4 + 7]));
                 }
             }
-            tc_fence_before_sync();
             // this warp's rows of the chunk are stored: count it for the publisher
-            if (emit_flags) {
+            if (part == 1 && emit_flags) {
                 __syncwarp();
                 if (lane == 0) {
                     __threadfence_block();
@@ -808,51 +935,42 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
             }
             return true;
         };
-        prefetch_u(0);
         bool ok = true;
         for (int c = 0; c < ncs && ok; ++c) {
             const int s = c % kScanStages;
-            const float *e1 = reinterpret_cast<const float *>(smem + SL::oG + (c % kDecaySlots) * SL::kG);
-            const float *e2 = e1 + 64;
+            const float *e2 = reinterpret_cast<const float *>(smem + SL::oG + (c % kDecaySlots) * SL::kG) + 64 + tk0;
             // Block-level routing: the delta rule runs over every block, but a softmax block's
             // update is not committed -- its state increment is multiplied by zero, so that the
             // state only decays across it (Section 4.3, the decay-always equation).
             const float commit =
                 kBlock && block_route[((size_t)b * L + (size_t)(c0 + c) * 64) * H + h] ? 0.f : 1.f;
-            ok = mbar_wait(&ms.full[s], (c / kScanStages) & 1, abort_flag);
-            if (!ok) break;
-            if (c > 0) {                                   // S_c = gamma_C S_{c-1} + dS_{c-1}
+            // ---- (a) S_c = gamma_C S_{c-1} + dS_{c-1}, and as fp16 operand to TMEM: 32 columns at a time, so that their
+            // products start while the next ones are worked on ----
+            float gC = 1.f;
+            if (c > 0) {
+                gC = reinterpret_cast<const float *>(smem + SL::oG + ((c - 1) % kDecaySlots) * SL::kG)[63];
                 ok = mbar_wait(&ms.barSU, (c - 1) & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after_sync();
-                // decay across the previous chunk and its increment in one pass over the row
-                const float gC = reinterpret_cast<const float *>(smem + SL::oG + ((c - 1) % kDecaySlots) * SL::kG)[63];
+            }
+            uint32_t spk[kHalfCols / 2];
 #pragma unroll
-                for (int cb = 0; cb < kHalfCols / 32; ++cb) {
+            for (int pt = 0; pt < SL::kParts; ++pt) {
+                if (c > 0) {
                     uint32_t ds[32];
-                    tmem_ld32(tmem + SL::cS + col0 + cb * 32 + lane_base, ds);
+                    tmem_ld32(tmem + SL::cS + col0 + pt * 32 + lane_base, ds);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int x = 0; x < 32; ++x) S[cb * 32 + x] = fmaf(S[cb * 32 + x], gC, __uint_as_float(ds[x]));
+                    for (int x = 0; x < 32; ++x) S[pt * 32 + x] = fmaf(S[pt * 32 + x], gC, __uint_as_float(ds[x]));
                 }
-                tc_fence_before_sync();
-            }
-            // ---- (a) state row -> fp16 operand in TMEM; decay the register copy afterwards ----
-            uint32_t spk[kHalfCols / 2];
-            {
-                uint32_t (&pk)[kHalfCols / 2] = spk;
 #pragma unroll
-                for (int x = 0; x < kHalfCols / 2; ++x) pk[x] = pack_half2(S[2 * x], S[2 * x + 1]);
-                if (kHalfCols == 64)
-                    tmem_st32(tmem + SL::cA + half * (kHalfCols / 2) + lane_base,
-                              reinterpret_cast<const uint32_t (&)[32]>(pk));
-                else
-                    tmem_st16(tmem + SL::cA + half * (kHalfCols / 2) + lane_base,
-                              reinterpret_cast<const uint32_t (&)[16]>(pk));
+                for (int x = 0; x < 16; ++x) spk[pt * 16 + x] = pack_half2(S[pt * 32 + 2 * x], S[pt * 32 + 2 * x + 1]);
+                tmem_st16(tmem + SL::cA + half * (kHalfCols / 2) + pt * 16 + lane_base,
+                          reinterpret_cast<const uint32_t (&)[16]>(spk[pt * 16]));
                 tmem_wait_st();
+                tc_fence_before_sync();
+                mbar_arrive(&ms.barA[pt]);
             }
-            tc_fence_before_sync();
-            mbar_arrive(&ms.barA);
             // (exports for the backward go behind the arrivals, off the chain between the chunks)
             if (ex.S16 && active) {      // chunk-entry state: the operand itself, in pieces of keys
                 uint4 *sc = reinterpret_cast<uint4 *>(ex.S16) + (((size_t)bh * NC + c0 + c) * (D / 8) + col0 / 8) * D + r;
@@ -860,55 +978,45 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
                 for (int x = 0; x < kHalfCols / 8; ++x)
                     sc[(size_t)x * D] = make_uint4(spk[4 * x], spk[4 * x + 1], spk[4 * x + 2], spk[4 * x + 3]);
             }
-            float u[32];                                   // from L2; lands while W S is computed
-            if (active && !zero_u) {
-                const float4 *src = u_src(c);
-#pragma unroll
-                for (int x = 0; x < 8; ++x) {
-                    const float4 a = __ldg(src + x * D);
-                    u[4 * x] = a.x; u[4 * x + 1] = a.y; u[4 * x + 2] = a.z; u[4 * x + 3] = a.w;
-                }
-            } else {
-#pragma unroll
-                for (int x = 0; x < 32; ++x) u[x] = 0.f;
-            }
-            // ---- (b) U~ = U - W S for this thread's 32 tokens ----
+            // ---- behind the MMAs just released: the first half of the previous chunk's output ----
+            ok = mbar_wait(&ms.full[s], (c / kScanStages) & 1, abort_flag);
+            if (ok && c > 0 && emit_out) ok = emit(c - 1, 0);
+            if (!ok) break;
+            // ---- (b) U~ = U - W S for this thread's 32 tokens; the state update's operand first ----
             ok = mbar_wait(&ms.barWS, c & 1, abort_flag);
             if (!ok) break;
             tc_fence_after_sync();
-            {
-                uint32_t ws[32];
-                tmem_ld32(tmem + SL::cWS + tk0 + lane_base, ws);
-                tmem_wait_ld();
+            uint32_t ux[32];
+            tmem_ld32(tmem + SL::cX + 64 * (c & 1) + tk0 + lane_base, ux);
+            tmem_wait_ld();
+            uint32_t pk[16];
 #pragma unroll
-                for (int j = 0; j < 32; ++j) u[j] -= __uint_as_float(ws[j]);
+            for (int x = 0; x < 16; x += 2) {
+                float4 f = *reinterpret_cast<const float4 *>(e2 + 2 * x);
+                if (kBlock) { f.x *= commit; f.y *= commit; f.z *= commit; f.w *= commit; }
+                pk[x] = pack_half2(__uint_as_float(ux[2 * x]) * f.x, __uint_as_float(ux[2 * x + 1]) * f.y);
+                pk[x + 1] = pack_half2(__uint_as_float(ux[2 * x + 2]) * f.z, __uint_as_float(ux[2 * x + 3]) * f.w);
             }
-            uint32_t upk[32];
-            {
-                uint32_t (&pk)[32] = upk;     // [0,16): U~ of this thread's 32 tokens, [16,32): U~ gamma_C/gamma
-#pragma unroll
-                for (int x = 0; x < 16; ++x) {
-                    pk[x] = pack_half2(u[2 * x], u[2 * x + 1]);
-                    const float f0 = kBlock ? commit * e2[tk0 + 2 * x] : e2[tk0 + 2 * x];
-                    const float f1 = kBlock ? commit * e2[tk0 + 2 * x + 1] : e2[tk0 + 2 * x + 1];
-                    pk[16 + x] = pack_half2(u[2 * x] * f0, u[2 * x + 1] * f1);
-                }
-                tmem_st32(tmem + SL::cWS + tk0 + lane_base, pk);   // over this thread's own W S columns
-                tmem_wait_st();
-            }
+            tmem_st16(tmem + SL::cU + tk0 + 16 + lane_base, pk);
+            tmem_wait_st();
             tc_fence_before_sync();
             mbar_arrive(&ms.barB);
+#pragma unroll
+            for (int x = 0; x < 16; ++x) pk[x] = pack_half2(__uint_as_float(ux[2 * x]), __uint_as_float(ux[2 * x + 1]));
+            tmem_st16(tmem + SL::cU + tk0 + lane_base, pk);
+            tmem_wait_st();
+            tc_fence_before_sync();
+            mbar_arrive(&ms.barB2);
             if (ex.Ut16 && active) {     // U~: the operand itself, in pieces of tokens
                 uint4 *ut = reinterpret_cast<uint4 *>(ex.Ut16) + (((size_t)bh * NC + c0 + c) * 8 + tk0 / 8) * D + r;
 #pragma unroll
                 for (int x = 0; x < 4; ++x)
-                    ut[(size_t)x * D] = make_uint4(upk[4 * x], upk[4 * x + 1], upk[4 * x + 2], upk[4 * x + 3]);
+                    ut[(size_t)x * D] = make_uint4(pk[4 * x], pk[4 * x + 1], pk[4 * x + 2], pk[4 * x + 3]);
             }
-            // ---- behind the MMAs just released: next U row towards L2, previous chunk's output ----
-            if (c + 1 < ncs) prefetch_u(c + 1);
-            if (c > 0 && emit_out) ok = emit(c - 1);
+            // ---- behind the MMAs just released: the rest of the previous chunk's output ----
+            if (c > 0 && emit_out) ok = emit(c - 1, 1);
         }
-        if (ok && emit_out) ok = emit(ncs - 1);
+        if (ok && emit_out) ok = emit(ncs - 1, 0) && emit(ncs - 1, 1);
         // where the state after the segment's last chunk goes
         float *final_state = sg.mode == 1 ? (zero_u ? sg.trans : sg.incr) + (size_t)slot * D * D
                              : state_out && c0 + ncs == NC ? state_out + (size_t)bh * D * D
@@ -1054,42 +1162,49 @@ cudaError_t launch_scan_combine(const ScanSegments &sg, Shape s, cudaStream_t st
     return cudaGetLastError();
 }
 
-template <int D>
+template <int D, bool kTrain>
 static cudaError_t prepare_tc_impl(const void *q, const void *k, const void *v, const float *g,
                                    const float *beta, const uint8_t *route, float scale_la,
                                    const GdnTcWs &ws, const GdnTcExport &ex, int32_t *status,
                                    float norm_eps, int head_words, Shape s, cudaStream_t st) {
+    using PL = PrepLayout<D, kTrain>;
     const int NC = s.L / kC;
     const uint64_t BH = (uint64_t)s.B * s.H;
-    CUtensorMap mq, mk, mv, mqh, mkh;
+    CUtensorMap mq, mk, mwt, mtb, mph;
     if (!tch::make_map_blhd(&mq, q, s.B, s.L, s.H, D, 64) ||
         !tch::make_map_blhd(&mk, k, s.B, s.L, s.H, D, 64) ||
-        !tch::make_map_blhd(&mv, v, s.B, s.L, s.H, D, 64) ||
-        !tch::make_map_2d(&mqh, ws.Qh, BH * s.L, D, 64) ||
-        !tch::make_map_2d(&mkh, ws.Kh, BH * s.L, D, 64))
+        !tch::make_map_2d(&mwt, ws.Wt, BH * NC * D, 64, 64) ||
+        !tch::make_map_2d(&mtb, ws.Tb, BH * NC * 64, 64, 64) ||
+        !tch::make_map_2d(&mph, ws.Ph, BH * NC * 64, 64, 64))
         return cudaErrorInvalidValue;
-    cudaError_t e = allow_smem(gdn_prepare_tc_kernel<D>,
-                                         PrepLayout<D>::kTotal);
+    CUtensorMap mv = mq, mqh = mq, mkh = mq, mu = mq;          // (placeholders: only a training step's are used)
+    if (kTrain && (!tch::make_map_blhd(&mv, v, s.B, s.L, s.H, D, 64) || !tch::make_map_2d(&mqh, ws.Qh, BH * s.L, D, 64) ||
+                   !tch::make_map_2d(&mkh, ws.Kh, BH * s.L, D, 64) || !tch::make_map_2d(&mu, ex.U16, BH * NC * D, 64, 64)))
+        return cudaErrorInvalidValue;
+    auto kernel = gdn_prepare_tc_kernel<D, kTrain>;
+    cudaError_t e = allow_smem(kernel, PL::kTotal);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)NC * (unsigned)BH);
     count_launch();
-    return launch_kernel(gdn_prepare_tc_kernel<D>, grid, dim3(kPrepThreads), PrepLayout<D>::kTotal, st, false, mq, mk, mv, mqh,
-                         mkh, g, beta, route, scale_la, (__half *)ws.Wt, ws.Ut, (__half *)ws.Ph, ws.Gd, ex, status,
-                         head_words, s.L, s.H, norm_eps, debug_wait_kcycles());
+    return launch_kernel(kernel, grid, dim3(kPrepThreads), PL::kTotal, st, false, mq, mk, mv, mqh, mkh, mu, mwt, mtb, mph, g, beta,
+                         route, scale_la, (__half *)ws.Ph, ws.Gd, ws.Rn, ex, status, head_words, s.L, s.H, norm_eps,
+                         debug_wait_kcycles());
 }
 
 template <int D>
-static cudaError_t scan_tc_impl(const GdnTcWs &ws, float scale_la, const float *state_in,
+static cudaError_t scan_tc_impl(const void *q, const void *k, const void *v, const GdnTcWs &ws, float scale_la, const float *state_in,
                                 float *state_out, const ScanOut &out, const GdnTcExport &ex,
                                 const ScanSegments &sg, const uint8_t *block_route, int32_t *status,
-                                Shape s, cudaStream_t st, bool pdl) {
+                                Shape s, cudaStream_t st, bool pdl, bool normed) {
     const int NC = s.L / kC;
     const uint64_t BH = (uint64_t)s.B * s.H;
-    CUtensorMap mwt, mqh, mkh, mph;
+    CUtensorMap mwt, mq, mk, mv, mph, mtb;
     if (!tch::make_map_2d(&mwt, ws.Wt, BH * NC * D, 64, D) ||
-        !tch::make_map_2d(&mqh, ws.Qh, BH * s.L, D, 64) ||
-        !tch::make_map_2d(&mkh, ws.Kh, BH * s.L, D, 64) ||
-        !tch::make_map_2d(&mph, ws.Ph, BH * NC * 64, 64, 64))
+        !tch::make_map_blhd(&mq, q, s.B, s.L, s.H, D, 64) ||
+        !tch::make_map_blhd(&mk, k, s.B, s.L, s.H, D, 64) ||
+        !tch::make_map_blhd(&mv, v, s.B, s.L, s.H, D, 64) ||
+        !tch::make_map_2d(&mph, ws.Ph, BH * NC * 64, 64, 64) ||
+        !tch::make_map_2d(&mtb, ws.Tb, BH * NC * 64, 64, 64))
         return cudaErrorInvalidValue;
     auto kernel = block_route ? gdn_scan_tc_kernel<D, true> : gdn_scan_tc_kernel<D, false>;
     cudaError_t e = allow_smem(kernel,
@@ -1097,27 +1212,32 @@ static cudaError_t scan_tc_impl(const GdnTcWs &ws, float scale_la, const float *
     if (e != cudaSuccess) return e;
     const int ctas = s.B * s.H * (sg.mode == 0 ? 1 : sg.mode == 1 ? 2 * sg.nseg - 3 : sg.nseg);
     count_launch();
-    return launch_kernel(kernel, dim3(ctas), dim3(kScanThreads), ScanLayout<D>::kTotal, st, pdl, mwt, mqh, mkh, mph, ws.Ut,
-                         ws.Gd, scale_la, state_in, state_out, (__half *)out.o_la16, out.o_la32, out.emit_flags, ex, sg,
-                         block_route, status, s.L, s.H, debug_wait_kcycles());
+    return launch_kernel(kernel, dim3(ctas), dim3(kScanThreads), ScanLayout<D>::kTotal, st, pdl, mwt, mq, mk, mv, mph, mtb,
+                         ws.Gd, normed ? ws.Rn : nullptr, scale_la, state_in, state_out, (__half *)out.o_la16, out.o_la32,
+                         out.emit_flags, ex, sg, block_route, status, s.L, s.H, debug_wait_kcycles());
 }
 
 cudaError_t launch_gdn_prepare_tc(const void *q, const void *k, const void *v, const float *g,
                                   const float *beta, const uint8_t *route, float scale_la,
                                   const GdnTcWs &ws, const GdnTcExport &ex, int32_t *status, Shape s,
                                   cudaStream_t st, int head_words, float norm_eps) {
-    if (s.d == 128)
-        return prepare_tc_impl<128>(q, k, v, g, beta, route, scale_la, ws, ex, status, norm_eps, head_words, s, st);
-    return prepare_tc_impl<64>(q, k, v, g, beta, route, scale_la, ws, ex, status, norm_eps, head_words, s, st);
+#define RUN(D, TR) return prepare_tc_impl<D, TR>(q, k, v, g, beta, route, scale_la, ws, ex, status, norm_eps, head_words, s, st)
+    if (s.d == 128) {
+        if (ex.U16) RUN(128, true);
+        RUN(128, false);
+    }
+    if (ex.U16) RUN(64, true);
+    RUN(64, false);
+#undef RUN
 }
 
-cudaError_t launch_gdn_scan_tc(const GdnTcWs &ws, float scale_la, const float *state_in,
+cudaError_t launch_gdn_scan_tc(const void *q, const void *k, const void *v, const GdnTcWs &ws, float scale_la, const float *state_in,
                                float *state_out, const ScanOut &out, const GdnTcExport &ex,
                                const ScanSegments &sg, const uint8_t *block_route, int32_t *status,
-                               Shape s, cudaStream_t st, bool pdl) {
+                               Shape s, cudaStream_t st, bool pdl, bool normed) {
     if (s.d == 128)
-        return scan_tc_impl<128>(ws, scale_la, state_in, state_out, out, ex, sg, block_route, status, s, st, pdl);
-    return scan_tc_impl<64>(ws, scale_la, state_in, state_out, out, ex, sg, block_route, status, s, st, pdl);
+        return scan_tc_impl<128>(q, k, v, ws, scale_la, state_in, state_out, out, ex, sg, block_route, status, s, st, pdl, normed);
+    return scan_tc_impl<64>(q, k, v, ws, scale_la, state_in, state_out, out, ex, sg, block_route, status, s, st, pdl, normed);
 }
 
 }  // namespace natsl

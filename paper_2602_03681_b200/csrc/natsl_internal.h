@@ -162,13 +162,14 @@ cudaError_t launch_softmax_bwd_tc(const void *Qh, const void *dO16, const void *
 
 // gdn_tc.cu -- tensor-core chunkwise Gated DeltaNet (bf16 storage): intermediates in workspace
 struct GdnTcWs {
-    void *Qh, *Kh;   // fp16 copies of q, k              [B,H,L,d]
     void *Wt;        // W^T per chunk, fp16              [B,H,L/C,d,64]
-    float *Ut;       // U^T per chunk, fp32, in 4-token pieces   [B,H,L/C,16,d,4]
+    void *Tb;        // (I + A)^-1 diag(beta~) per chunk, fp16   [B,H,L/C,64,64]
     void *Ph;        // P per chunk, fp16                [B,H,L/C,64,64]
     float *Gd;       // per chunk: gamma_i (64), gamma_C / gamma_i (64), fp32   [B,H,L/C,128]
+    float *Rn;       // with the normalisation, per chunk: the factors of q's rows (64) and k's rows (64), fp32   [B,H,L/C,128]
+    void *Qh, *Kh;   // training step only: fp16 copies of q, k, as the products take them   [B,H,L,d]
 };
-// The chunkwise quantities the backward needs (all may be null), as fp16 -- what the forward's own MMA operands were
+// The chunkwise quantities the backward needs (all, or none: null), as fp16 -- what the forward's own MMA operands were
 // -- in the layout the backward's fragments are loaded from.  "Pieces": a transposed tile cut into 16-byte pieces
 // of 8 elements along the second index, all rows of a piece contiguous, [pieces][rows][8].
 struct GdnTcExport {
@@ -222,10 +223,11 @@ struct ScanOut {
     int32_t *emit_flags;
 };
 constexpr int kScanRowWarps = 8;
-cudaError_t launch_gdn_scan_tc(const GdnTcWs &ws, float scale_la, const float *state_in,
-                               float *state_out, const ScanOut &out, const GdnTcExport &ex,
+cudaError_t launch_gdn_scan_tc(const void *q, const void *k, const void *v, const GdnTcWs &ws, float scale_la,
+                               const float *state_in, float *state_out, const ScanOut &out, const GdnTcExport &ex,
                                const ScanSegments &sg, const uint8_t *block_route, int32_t *status,
-                               Shape s, cudaStream_t st, bool pdl = false);
+                               Shape s, cudaStream_t st, bool pdl, bool normed);
+// (normed: q's and k's rows are taken times ws.Rn)
 cudaError_t launch_scan_combine(const ScanSegments &sg, Shape s, cudaStream_t st, bool pdl = false);
 
 // bwd_simt.cu -- fp32 CUDA-core backward

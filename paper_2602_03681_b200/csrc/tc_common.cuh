@@ -266,6 +266,20 @@ __host__ __device__ constexpr uint32_t make_idesc(uint32_t fmt, int M, int N, bo
            ((uint32_t)(M >> 4) << 24);
 }
 
+// One thread issues tcgen05.mma and commit, but the warp around it must stay together: their operands are uniform
+// registers, and where one lane alone runs the loop that forms them (if (lane == 0) ...) every one of them is moved there
+// from vector registers, 80 to 100 cycles for each instruction issued.  So an issuing warp waits, counts and branches
+// as a warp (wait_all), takes its TMEM base through uniform() and wraps only the instructions in if (elect_one()).
+__device__ __forceinline__ bool elect_one() {       // always the same lane
+    uint32_t is;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(is));
+    return is != 0;
+}
+__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __reduce_or_sync(0xffffffffu, x); }
+__device__ __forceinline__ bool wait_all(uint64_t *bar, uint32_t parity, volatile int *abort_flag) {   // the whole warp
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
+}
+
 // D[tmem] (+)= A[smem] * B[smem]; one thread issues.
 __device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
                                        uint32_t idesc, bool accumulate) {

@@ -119,39 +119,44 @@ gdn_rscan_tc_kernel(const __grid_constant__ CUtensorMap map_do,    // dO (fp16) 
                 mbar_wait_drain(&ms.full[u % kRsStages], (u / kRsStages) & 1);
         }
     } else if (warp == 8) {
-        if (lane == 0) {
-            constexpr uint32_t id_x1 = make_idesc(kFmtF16, 128, 64, true, true);    // A = dO (MN), B = P (MN)
-            constexpr uint32_t id_x2 = make_idesc(kFmtF16, 128, 64, false, false);  // A = dS1 (TMEM), B = K
-            constexpr uint32_t id_y1 = make_idesc(kFmtF16, 128, D, true, true);     // A = dOg (MN), B = Q (MN)
-            constexpr uint32_t id_y2 = make_idesc(kFmtF16, 128, D, false, false, true);   // -dU~ (TMEM) x W^T
-            for (int n = 0; n < NC; ++n) {
-                const int s = n % kRsStages;
-                const uint32_t st = smem_u32(smem + s * SL::kStage);
-                if (!mbar_wait(&ms.full[s], (n / kRsStages) & 1, abort_flag)) break;
-                tc_fence_after_sync();
-                // X1 does not involve the gradient state and its columns are free (every row thread
-                // read them before its barB arrival of the previous chunk): issue it ahead.
+        constexpr uint32_t id_x1 = make_idesc(kFmtF16, 128, 64, true, true);    // A = dO (MN), B = P (MN)
+        constexpr uint32_t id_x2 = make_idesc(kFmtF16, 128, 64, false, false);  // A = dS1 (TMEM), B = K
+        constexpr uint32_t id_y1 = make_idesc(kFmtF16, 128, D, true, true);     // A = dOg (MN), B = Q (MN)
+        constexpr uint32_t id_y2 = make_idesc(kFmtF16, 128, D, false, false, true);   // -dU~ (TMEM) x W^T
+        const uint32_t tm = uniform(tmem), sm = smem_u32(smem);
+        for (int n = 0; n < NC; ++n) {
+            const int s = n % kRsStages;
+            const uint32_t st = sm + s * SL::kStage;
+            if (!wait_all(&ms.full[s], (n / kRsStages) & 1, abort_flag)) break;
+            tc_fence_after_sync();
+            // X1 does not involve the gradient state and its columns are free (every row thread
+            // read them before its barB arrival of the previous chunk): issue it ahead.
+            if (elect_one()) {
 #pragma unroll
                 for (int k16 = 0; k16 < 4; ++k16)
-                    mma_ss(tmem + SL::cX1, desc_mnmajor(st + SL::oDO + k16 * 2048, 8192),
+                    mma_ss(tm + SL::cX1, desc_mnmajor(st + SL::oDO + k16 * 2048, 8192),
                            desc_mnmajor(st + SL::oP + k16 * 2048, 0), id_x1, k16 != 0);
-                // barA: the row threads have consumed the previous chunk's Y and written dS1.
-                if (!mbar_wait(&ms.barA, n & 1, abort_flag)) break;
-                tc_fence_after_sync();
+            }
+            // barA: the row threads have consumed the previous chunk's Y and written dS1.
+            if (!wait_all(&ms.barA, n & 1, abort_flag)) break;
+            tc_fence_after_sync();
+            if (elect_one()) {
 #pragma unroll
                 for (int kk = 0; kk < D / 16; ++kk)
-                    mma_ts(tmem + SL::cX2, tmem + SL::cA + kk * 8,
+                    mma_ts(tm + SL::cX2, tm + SL::cA + kk * 8,
                            desc_kmajor(st + SL::oK + (kk >> 2) * 8192 + (kk & 3) * 32), id_x2, kk != 0);
                 mma_commit(&ms.barX);
 #pragma unroll
                 for (int k16 = 0; k16 < 4; ++k16)
-                    mma_ss(tmem + SL::cY, desc_mnmajor(st + SL::oDOg + k16 * 2048, 8192),
+                    mma_ss(tm + SL::cY, desc_mnmajor(st + SL::oDOg + k16 * 2048, 8192),
                            desc_mnmajor(st + SL::oQ + k16 * 2048, 8192), id_y1, k16 != 0);
-                if (!mbar_wait(&ms.barB, n & 1, abort_flag)) break;
-                tc_fence_after_sync();
+            }
+            if (!wait_all(&ms.barB, n & 1, abort_flag)) break;
+            tc_fence_after_sync();
+            if (elect_one()) {
 #pragma unroll
                 for (int k16 = 0; k16 < 4; ++k16)
-                    mma_ts(tmem + SL::cY, tmem + SL::cX2 + (k16 >> 1) * 32 + (k16 & 1) * 8,
+                    mma_ts(tm + SL::cY, tm + SL::cX2 + (k16 >> 1) * 32 + (k16 & 1) * 8,
                            desc_kmajor(st + SL::oW + k16 * 32), id_y2, true);
                 mma_commit(&ms.barY);
                 mma_commit(&ms.empty[s]);

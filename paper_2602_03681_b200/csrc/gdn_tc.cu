@@ -140,52 +140,55 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
     uint8_t *xHi = D == 128 ? sQK + 16384 : smem + PL::oX + 8192;
 
     if (warp == 4) {
-        if (lane == 0) {
+        const bool leader = elect_one();
+        const uint32_t tm = uniform(tmem), tWu = tm + (kTrain ? 64 : 0), sm = smem_u32(smem);
+        const uint32_t aV = sm + PL::oV, aQK = sm + PL::oQK, aK = aQK + 8192, aTb = D == 128 ? aQK : sm + PL::oX,
+                       aTg = aTb + (D == 128 ? 16384 : 8192);
+        if (leader) {
             mbar_arrive_expect_tx(&ms.barLoad, PL::kLoadBytes);
             for (int kb = 0; kb < KB; ++kb) {
                 tma_load_4d(sQK + kb * 16384 + 8192, &map_k, &ms.barLoad, kb * 64, h, tok0, b);
                 tma_load_4d(sQK + kb * 16384, &map_q, &ms.barLoad, kb * 64, h, tok0, b);
                 if (kTrain) tma_load_4d(sV + kb * 8192, &map_v, &ms.barLoad, kb * 64, h, tok0, b);
             }
-            bool ok = mbar_wait(&ms.barConv, 0, abort_flag);       // tiles converted to fp16
-            if (ok) {
-                // ---- fp16 copies of q and k for the backward; [Q ; K] K^T ----
-                if (kTrain) {
-                    for (int kb = 0; kb < KB; ++kb) {
-                        tma_store_2d(&map_qh, sQK + kb * 16384, kb * 64, bh * L + tok0);
-                        tma_store_2d(&map_kh, sQK + kb * 16384 + 8192, kb * 64, bh * L + tok0);
-                    }
-                    tma_store_commit();
+        }
+        bool ok = wait_all(&ms.barConv, 0, abort_flag);       // tiles converted to fp16
+        if (ok) {
+            // ---- fp16 copies of q and k for the backward; [Q ; K] K^T ----
+            if (kTrain && leader) {
+                for (int kb = 0; kb < KB; ++kb) {
+                    tma_store_2d(&map_qh, sQK + kb * 16384, kb * 64, bh * L + tok0);
+                    tma_store_2d(&map_kh, sQK + kb * 16384 + 8192, kb * 64, bh * L + tok0);
                 }
-                tc_fence_after_sync();
-                constexpr uint32_t idesc = make_idesc(kFmtF16, 128, 64, false, false);
-                const uint32_t aQK = smem_u32(sQK);
+                tma_store_commit();
+            }
+            tc_fence_after_sync();
+            constexpr uint32_t idesc = make_idesc(kFmtF16, 128, 64, false, false);
+            if (elect_one()) {
 #pragma unroll
                 for (int kb = 0; kb < KB; ++kb)
 #pragma unroll
                     for (int k16 = 0; k16 < 4; ++k16)
-                        mma_ss(tmem, desc_kmajor(aQK + kb * 16384 + k16 * 32),
+                        mma_ss(tm, desc_kmajor(aQK + kb * 16384 + k16 * 32),
                                desc_kmajor(aQK + kb * 16384 + 8192 + k16 * 32), idesc, (kb | k16) != 0);
                 mma_commit(&ms.barM);
-                if (kTrain) tma_store_wait_read();        // the q copy has left its blocks
-                ok = mbar_wait(&ms.barM, 0, abort_flag);  // and the MMAs have read them
-                mbar_arrive(&ms.barXfree);
             }
-            if (ok) ok = mbar_wait(&ms.barT, 0, abort_flag);
-            if (ok) {
-                // ---- T beta~ leaves; U^T = V^T (T beta~)^T,  W^T = K^T (T beta~ gamma)^T ----
-                tc_fence_after_sync();
-                tma_store_2d(&map_tb, xLo, 0, (int)chunk * 64);
-                tma_store_commit();
-                const uint32_t aV = smem_u32(sV), aK = smem_u32(sQK) + 8192, aTb = smem_u32(xLo),
-                               aTg = smem_u32(xHi);
+            if (kTrain && leader) tma_store_wait_read();      // the q copy has left its blocks
+            ok = wait_all(&ms.barM, 0, abort_flag);           // and the MMAs have read them
+            if (leader) mbar_arrive(&ms.barXfree);
+        }
+        if (ok) ok = wait_all(&ms.barT, 0, abort_flag);
+        if (ok) {
+            // ---- T beta~ leaves; U^T = V^T (T beta~)^T,  W^T = K^T (T beta~ gamma)^T ----
+            tc_fence_after_sync();
+            if (elect_one()) {
                 constexpr uint32_t idesc = make_idesc(kFmtF16, 128, 64, true, false);
                 if (D == 128 || !kTrain) {
 #pragma unroll
                     for (int k16 = 0; k16 < 4; ++k16) {
-                        if (kTrain) mma_ss(tmem, desc_mnmajor(aV + k16 * 2048, 8192), desc_kmajor(aTb + k16 * 32), idesc, k16 != 0);
+                        if (kTrain) mma_ss(tm, desc_mnmajor(aV + k16 * 2048, 8192), desc_kmajor(aTb + k16 * 32), idesc, k16 != 0);
                         // (d = 64: rows 64-127 of M are of no interest, K again)
-                        mma_ss(tW, desc_mnmajor(aK + k16 * 2048, D == 128 ? 16384 : 0), desc_kmajor(aTg + k16 * 32), idesc, k16 != 0);
+                        mma_ss(tWu, desc_mnmajor(aK + k16 * 2048, D == 128 ? 16384 : 0), desc_kmajor(aTg + k16 * 32), idesc, k16 != 0);
                     }
                 } else {
                     // d = 64: rows 0-63 of M are V^T, rows 64-127 are K^T (16 KB further on);
@@ -193,13 +196,16 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                     constexpr uint32_t idesc2 = make_idesc(kFmtF16, 128, 128, true, false);
 #pragma unroll
                     for (int k16 = 0; k16 < 4; ++k16)
-                        mma_ss(tmem, desc_mnmajor(aV + k16 * 2048, 16384), desc_kmajor(aTb + k16 * 32),
-                               idesc2, k16 != 0);
+                        mma_ss(tm, desc_mnmajor(aV + k16 * 2048, 16384), desc_kmajor(aTb + k16 * 32), idesc2, k16 != 0);
                 }
                 mma_commit(&ms.barUW);
             }
-            tma_store_wait_all();
+            if (leader) {
+                tma_store_2d(&map_tb, xLo, 0, (int)chunk * 64);
+                tma_store_commit();
+            }
         }
+        if (leader) tma_store_wait_all();
     } else {
         const int r = tid, i = r & 63;
         const bool solver = r >= 64;                       // rows 64-127: K K^T

@@ -126,50 +126,51 @@ softmax_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh  [B
             mbar_wait_drain(&ms.barQ, 0);
         }
     } else if (warp == kMmaWarpB) {
-        if (lane == 0 && T > 0) {
+        const int Tu = (int)uniform((uint32_t)T);
+        if (Tu > 0) {
             constexpr uint32_t id_s = make_idesc(kFmtF16, 128, 64, false, false);
             constexpr uint32_t id_dq = make_idesc(kFmtF16, 128, D, false, true);
-            const uint32_t aQ = smem_u32(smem + SL::oQ), aDO = smem_u32(smem + SL::oDO),
-                           aDS = smem_u32(smem + SL::oDS);
+            const uint32_t tm = uniform(tmem), sm = smem_u32(smem), aQ = sm + SL::oQ, aDO = sm + SL::oDO, aDS = sm + SL::oDS;
             auto issue_s = [&](int t) {
-                const uint32_t aK = smem_u32(smem + SL::oK + (t % SL::kStages) * SL::kKV);
-                const uint32_t aV = smem_u32(smem + SL::oV + (t % SL::kStages) * SL::kKV);
+                const uint32_t aK = sm + SL::oK + (t % SL::kStages) * SL::kKV, aV = sm + SL::oV + (t % SL::kStages) * SL::kKV;
+                if (!elect_one()) return;
 #pragma unroll
                 for (int kb = 0; kb < KB; ++kb)
 #pragma unroll
                     for (int k16 = 0; k16 < 4; ++k16) {
-                        mma_ss(tS, desc_kmajor(aQ + kb * 16384 + k16 * 32),
+                        mma_ss(tm, desc_kmajor(aQ + kb * 16384 + k16 * 32),
                                desc_kmajor(aK + kb * 8192 + k16 * 32), id_s, (kb | k16) != 0);
-                        mma_ss(tDP, desc_kmajor(aDO + kb * 16384 + k16 * 32),
+                        mma_ss(tm + 64, desc_kmajor(aDO + kb * 16384 + k16 * 32),
                                desc_kmajor(aV + kb * 8192 + k16 * 32), id_s, (kb | k16) != 0);
                     }
                 mma_commit(&ms.barS);
             };
-            bool ok = mbar_wait(&ms.barQ, 0, abort_flag) && mbar_wait(&ms.full[0], 0, abort_flag);
+            bool ok = wait_all(&ms.barQ, 0, abort_flag) && wait_all(&ms.full[0], 0, abort_flag);
             if (ok) {
                 tc_fence_after_sync();
                 issue_s(0);
             }
-            for (int t = 0; ok && t < T; ++t) {
+            for (int t = 0; ok && t < Tu; ++t) {
                 // S and dP of the next tile go into the same TMEM columns as soon as the row threads
                 // have read this tile's out of them (barSfree), i.e. while they still compute dS.
-                if (t + 1 < T) {
-                    ok = mbar_wait(&ms.full[(t + 1) % SL::kStages], ((t + 1) / SL::kStages) & 1, abort_flag) &&
-                         mbar_wait(&ms.barSfree, t & 1, abort_flag);
+                if (t + 1 < Tu) {
+                    ok = wait_all(&ms.full[(t + 1) % SL::kStages], ((t + 1) / SL::kStages) & 1, abort_flag) &&
+                         wait_all(&ms.barSfree, t & 1, abort_flag);
                     if (!ok) break;
                     tc_fence_after_sync();
                     issue_s(t + 1);
                 }
-                ok = mbar_wait(&ms.barP, t & 1, abort_flag);
+                ok = wait_all(&ms.barP, t & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after_sync();
-                const uint32_t aK = smem_u32(smem + SL::oK + (t % SL::kStages) * SL::kKV);
+                const uint32_t aK = sm + SL::oK + (t % SL::kStages) * SL::kKV;
+                if (elect_one()) {
 #pragma unroll
-                for (int k16 = 0; k16 < 4; ++k16)
-                    mma_ss(tDQ, desc_kmajor(aDS + k16 * 32), desc_mnmajor(aK + k16 * 2048, 8192), id_dq,
-                           (t | k16) != 0);
-                mma_commit(&ms.barAcc);
-                mma_commit(&ms.empty[t % SL::kStages]);     // K/V stage t is free after dQ(t)
+                    for (int k16 = 0; k16 < 4; ++k16)
+                        mma_ss(tm + 128, desc_kmajor(aDS + k16 * 32), desc_mnmajor(aK + k16 * 2048, 8192), id_dq, (t | k16) != 0);
+                    mma_commit(&ms.barAcc);
+                    mma_commit(&ms.empty[t % SL::kStages]);     // K/V stage t is free after dQ(t)
+                }
             }
         }
     } else {
@@ -356,50 +357,51 @@ softmax_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap map_q,    // Qh [B
             mbar_wait_drain(&ms.barQ, 0);
         }
     } else if (warp == kMmaWarpB) {
-        if (lane == 0) {
-            constexpr uint32_t id_s = make_idesc(kFmtF16, 128, 64, false, false);
-            constexpr uint32_t id_acc = make_idesc(kFmtF16, 128, D, false, true);
-            const uint32_t aK = smem_u32(smem + SL::oK), aV = smem_u32(smem + SL::oV), aP = smem_u32(smem + SL::oP);
-            auto stage = [&](int o, int t) { return smem_u32(smem + o + (t % SL::kStages) * SL::kQ); };
-            auto issue_logits = [&](uint32_t dst, uint32_t a, uint32_t b, uint64_t *bar) {
+        constexpr uint32_t id_s = make_idesc(kFmtF16, 128, 64, false, false);
+        constexpr uint32_t id_acc = make_idesc(kFmtF16, 128, D, false, true);
+        const int Tu = (int)uniform((uint32_t)T);
+        const uint32_t tm = uniform(tmem), sm = smem_u32(smem), aK = sm + SL::oK, aV = sm + SL::oV, aP = sm + SL::oP;
+        auto stage = [&](int o, int t) { return sm + o + (t % SL::kStages) * SL::kQ; };
+        auto issue_logits = [&](uint32_t dst, uint32_t a, uint32_t b, uint64_t *bar) {
+            if (!elect_one()) return;
 #pragma unroll
-                for (int kb = 0; kb < KB; ++kb)
+            for (int kb = 0; kb < KB; ++kb)
 #pragma unroll
-                    for (int k16 = 0; k16 < 4; ++k16)
-                        mma_ss(dst, desc_kmajor(a + kb * 16384 + k16 * 32), desc_kmajor(b + kb * 8192 + k16 * 32), id_s,
-                               (kb | k16) != 0);
-                mma_commit(bar);
-            };
-            bool ok = mbar_wait(&ms.barQ, 0, abort_flag) && mbar_wait(&ms.full[0], 0, abort_flag);
-            if (ok) {
-                tc_fence_after_sync();
-                issue_logits(tS, aK, stage(SL::oQ, 0), &ms.barS);
-                issue_logits(tDP, aV, stage(SL::oDO, 0), &ms.barDP);
-            }
-            for (int t = 0; ok && t < T; ++t) {
-                // S^T of the next query tile goes into the same TMEM columns as soon as the row threads have read
-                // this tile's out of them; dP^T of the next one behind this tile's products, which read dS^T there.
-                if (t + 1 < T) {
-                    ok = mbar_wait(&ms.full[(t + 1) % SL::kStages], ((t + 1) / SL::kStages) & 1, abort_flag) &&
-                         mbar_wait(&ms.barSfree, t & 1, abort_flag);
-                    if (!ok) break;
-                    tc_fence_after_sync();
-                    issue_logits(tS, aK, stage(SL::oQ, t + 1), &ms.barS);
-                }
-                ok = mbar_wait(&ms.barP, t & 1, abort_flag);
+                for (int k16 = 0; k16 < 4; ++k16)
+                    mma_ss(dst, desc_kmajor(a + kb * 16384 + k16 * 32), desc_kmajor(b + kb * 8192 + k16 * 32), id_s, (kb | k16) != 0);
+            mma_commit(bar);
+        };
+        bool ok = wait_all(&ms.barQ, 0, abort_flag) && wait_all(&ms.full[0], 0, abort_flag);
+        if (ok) {
+            tc_fence_after_sync();
+            issue_logits(tm, aK, stage(SL::oQ, 0), &ms.barS);
+            issue_logits(tm + 64, aV, stage(SL::oDO, 0), &ms.barDP);
+        }
+        for (int t = 0; ok && t < Tu; ++t) {
+            // S^T of the next query tile goes into the same TMEM columns as soon as the row threads have read
+            // this tile's out of them; dP^T of the next one behind this tile's products, which read dS^T there.
+            if (t + 1 < Tu) {
+                ok = wait_all(&ms.full[(t + 1) % SL::kStages], ((t + 1) / SL::kStages) & 1, abort_flag) &&
+                     wait_all(&ms.barSfree, t & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after_sync();
-                const uint32_t aQ = stage(SL::oQ, t), aDO = stage(SL::oDO, t);
+                issue_logits(tm, aK, stage(SL::oQ, t + 1), &ms.barS);
+            }
+            ok = wait_all(&ms.barP, t & 1, abort_flag);
+            if (!ok) break;
+            tc_fence_after_sync();
+            const uint32_t aQ = stage(SL::oQ, t), aDO = stage(SL::oDO, t);
+            if (elect_one()) {
 #pragma unroll
                 for (int k16 = 0; k16 < 4; ++k16) {
-                    mma_ss(tDV, desc_kmajor(aP + k16 * 32), desc_mnmajor(aDO + k16 * 2048, 8192), id_acc,
+                    mma_ss(tm + 128, desc_kmajor(aP + k16 * 32), desc_mnmajor(aDO + k16 * 2048, 8192), id_acc, (t | k16) != 0);
+                    mma_ts(tm + 128 + D, tm + 64 + (k16 >> 1) * 32 + (k16 & 1) * 8, desc_mnmajor(aQ + k16 * 2048, 8192), id_acc,
                            (t | k16) != 0);
-                    mma_ts(tDK, tDP + (k16 >> 1) * 32 + (k16 & 1) * 8, desc_mnmajor(aQ + k16 * 2048, 8192), id_acc, (t | k16) != 0);
                 }
                 mma_commit(&ms.barAcc);
                 mma_commit(&ms.empty[t % SL::kStages]);
-                if (t + 1 < T) issue_logits(tDP, aV, stage(SL::oDO, t + 1), &ms.barDP);
             }
+            if (t + 1 < Tu) issue_logits(tm + 64, aV, stage(SL::oDO, t + 1), &ms.barDP);
         }
     } else {
         const int wq = warp & 3, half = warp >> 2, r = wq * 32 + lane, j = kt * 128 + r;    // this thread's retained key

@@ -310,59 +310,61 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
         }
     } else if (warp == kMmaWarp) {
         // ------------------------------ MMA issuer ------------------------------
-        if (lane == 0 && T2 > 0) {
+        // (as a warp, with uniform operands: see elect_one)
+        const int Tu = (int)uniform((uint32_t)T), T2u = (int)uniform((uint32_t)T2);
+        if (T2u > 0) {
             // logits: q and k as given are bf16; normalised ones are fp16 (see the softmax threads)
             constexpr uint32_t idesc_qk = make_idesc(kNorm ? kFmtF16 : kFmtBF16, kBM, kBN, false, false);
             constexpr uint32_t idesc_pv = make_idesc(kFmtF16, kBM, D, false, true);
-            const uint32_t aQ = smem_u32(smem + SL::oQ);
-            auto issue_qk = [&](int t) {
-                const uint32_t aK = smem_u32(smem + SL::oK + (t % kStages) * SL::kKStage);
-#pragma unroll
-                for (int kb = 0; kb < KB; ++kb)
-#pragma unroll
-                    for (int k16 = 0; k16 < 4; ++k16)
-                        mma_ss(tS(t), desc_kmajor(aQ + kb * kBM * 128 + k16 * 32),
-                               desc_kmajor(aK + kb * kBN * 128 + k16 * 32), idesc_qk,
-                               (kb | k16) != 0);
-                mma_commit(&ms.emptyK[t % kStages]);
-                mma_commit(&ms.barS[t % kLogits]);
-            };
+            const uint32_t tm = uniform(tmem), tOu = tm + 64 * kLogits, sm = smem_u32(smem), aQ = sm + SL::oQ;
+            auto tSu = [&](int t) { return tm + 64 * (t % kLogits); };
             // (normalisation with block-level routing: an own-block tile's keys arrive raw and are
             // normalised in place by the softmax threads first.  One single-phase barrier per own-block
             // tile, of which a CTA has at most two: with one barrier and a phase per tile, nothing kept the
-            // softmax threads from completing the second phase before this thread had looked at the
+            // softmax threads from completing the second phase before this warp had looked at the
             // first -- a parity wait then never returns.)
             auto own_keys_ready = [&](int t) {
-                return !(kBlock && kNorm) || t < T || mbar_wait(&ms.barKn[t - T], 0, abort_flag);
+                return !(kBlock && kNorm) || t < Tu || wait_all(&ms.barKn[t - Tu], 0, abort_flag);
             };
             // logits of tile t, as soon as its keys are there (and its TMEM columns free: MMAs run in issue order)
             auto next_qk = [&](int t) {
-                if (t >= T2) return true;
-                if (!mbar_wait(&ms.fullK[t % kStages], (t / kStages) & 1, abort_flag) || !own_keys_ready(t)) return false;
+                if (t >= T2u) return true;
+                if (!wait_all(&ms.fullK[t % kStages], (t / kStages) & 1, abort_flag) || !own_keys_ready(t)) return false;
                 tc_fence_after_sync();
-                issue_qk(t);
+                const uint32_t aK = sm + SL::oK + (t % kStages) * SL::kKStage;
+                if (elect_one()) {
+#pragma unroll
+                    for (int kb = 0; kb < KB; ++kb)
+#pragma unroll
+                        for (int k16 = 0; k16 < 4; ++k16)
+                            mma_ss(tSu(t), desc_kmajor(aQ + kb * kBM * 128 + k16 * 32),
+                                   desc_kmajor(aK + kb * kBN * 128 + k16 * 32), idesc_qk, (kb | k16) != 0);
+                    mma_commit(&ms.emptyK[t % kStages]);
+                    mma_commit(&ms.barS[t % kLogits]);
+                }
                 return true;
             };
-            bool ok = mbar_wait(&ms.barQ, 0, abort_flag) && (!kNorm || mbar_wait(&ms.barQn, 0, abort_flag));
+            bool ok = wait_all(&ms.barQ, 0, abort_flag) && (!kNorm || wait_all(&ms.barQn, 0, abort_flag));
             for (int t = 0; t < kAhead && ok; ++t) ok = next_qk(t);
-            for (int t = 0; ok && t < T2; ++t) {
+            for (int t = 0; ok && t < T2u; ++t) {
                 // (keys that the softmax threads still have to normalise must not hold up this tile's product)
-                const bool late = kBlock && kNorm && t + kAhead >= T;
+                const bool late = kBlock && kNorm && t + kAhead >= Tu;
                 if (!late) ok = next_qk(t + kAhead);
-                ok = ok && mbar_wait(&ms.barP[t % kLogits], (t / kLogits) & 1, abort_flag) &&
-                     mbar_wait(&ms.fullV[t % kStages], (t / kStages) & 1, abort_flag);
+                ok = ok && wait_all(&ms.barP[t % kLogits], (t / kLogits) & 1, abort_flag) &&
+                     wait_all(&ms.fullV[t % kStages], (t / kStages) & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after_sync();
-                const uint32_t aV = smem_u32(smem + SL::oV + (t % kStages) * SL::kVStage);
+                const uint32_t aV = sm + SL::oV + (t % kStages) * SL::kVStage;
+                if (elect_one()) {
 #pragma unroll
-                for (int k16 = 0; k16 < 4; ++k16)      // A = P(t): fp16 pairs in the first 32 columns of S(t)
-                    mma_ts(tO, tS(t) + k16 * 8, desc_mnmajor(aV + k16 * 2048, kBN * 128),
-                           idesc_pv, (t | k16) != 0);
-                mma_commit(&ms.emptyV[t % kStages]);
-                mma_commit(&ms.barO[t & 1]);
+                    for (int k16 = 0; k16 < 4; ++k16)      // A = P(t): fp16 pairs in the first 32 columns of S(t)
+                        mma_ts(tOu, tSu(t) + k16 * 8, desc_mnmajor(aV + k16 * 2048, kBN * 128), idesc_pv, (t | k16) != 0);
+                    mma_commit(&ms.emptyV[t % kStages]);
+                    mma_commit(&ms.barO[t & 1]);
+                }
                 if (late) ok = next_qk(t + kAhead);
             }
-            if (ok) mma_commit(&ms.barF);              // every product has run
+            if (ok && elect_one()) mma_commit(&ms.barF);              // every product has run
         }
     } else {
         // ------------------------------ softmax + epilogue ------------------------------

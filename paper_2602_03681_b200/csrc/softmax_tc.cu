@@ -14,24 +14,20 @@
 // Epilogue: o_la arrives as the scan leaves it, fp16 and transposed per chunk (o_laT, one 16 KB tile
 // per chunk: [8 pieces][d][8 tokens], row r of piece p at slot r ^ p); the CTA's two tiles come in
 // by bulk copies (into the Q tile, free once the last Q K^T has run) while the last K/V tile is still
-// being processed, and each thread reads its query's column out of them (the slot permutation
-// spreads a warp's four pieces over the banks), normalises
-// its own row of both branches, combines them and writes its row of `out` into a swizzled
-// shared-memory tile that one bulk tensor store sends out, so that no global access of the
-// epilogue is issued per thread and row.
+// being processed, and each warp reads its 32 queries out of them transposed, in the layout it reads the accumulator in,
+// normalises the rows of both branches, combines them and writes them into a swizzled
+// shared-memory tile that one bulk tensor store sends out.
 // The kernel may run beside the scan that produces o_la (launched behind it as a programmatic
 // dependent): nothing before the epilogue needs o_la, and the epilogue's load waits, bounded, for
 // the per-chunk counters the scan raises (emit_flags); CTAs are then ordered by query tile first,
 // so that the tiles whose chunks the scan finishes first are also scheduled first.
-// Warp roles: one or two warpgroups of softmax/epilogue threads (thread r <-> query row r <-> TMEM lane r; two
-// take turns by tile and share the running maximum of a row, see SmLayout), then a warp that issues the
+// Warp roles: four softmax/epilogue warps (thread r <-> query row r <-> TMEM lane r), a warp that issues the
 // MMAs and one that issues the TMA loads.
-// What it costs (128 queries, measured by leaving parts out): about a third of the time of a short-context call is
-// the CTA's fixed part (Q, o_la and out through shared memory), a 64-key tile takes 690 cycles per SM at 64
-// columns and 1080 at 128, where the MMAs alone take 400 and 676; the exponentials do not show.  Packed fp32
-// operations, the rolled epilogue and one masking path keep the code small: waiting for instructions was the
-// second-largest stall.  Forward of ten sequences of 4096 tokens, six heads of two slices, block-routed and
-// normalised: 307 -> 258 us for this kernel alone; one sequence of 32768 tokens, d = 128: 344 -> 297 us.
+// What it costs: with two key tiles of 128 columns a CTA lives 15 thousand cycles, of which 3500 pass before the first
+// logits, 1100 a tile and, before its epilogue read o_laT and the accumulator in the matrix layout (ldmatrix, stmatrix,
+// 16x256b), 8 thousand behind the last; now 4500.  88 us before, 75 now for 4 x 4096 tokens and 16 heads by itself, 343 and 298
+// for one sequence of 32768.  With 64-column heads in the paper's mode an own-block tile takes twice as long as a retained one
+// (its keys are normalised and its values converted first), and waiting for instructions is a quarter of the stalls.
 // Block-level routing (template flag): after the retained tiles, one more tile per linear block of
 // the CTA's two, holding that block's own 64 tokens (Section 4.1, inner-chunk correlations).
 // Grouped softmax heads (template count kG; Section 4.3, several softmax heads under one linear head's
@@ -54,20 +50,21 @@ using namespace tc;
 
 constexpr int kBM = 128;        // queries per CTA
 constexpr int kBN = 64;         // retained tokens per K/V tile
-constexpr int kGroupThreads = 128;                 // a softmax warpgroup: one thread per query row
-constexpr int kMiscBytes = 5120;
+constexpr int kSoftmaxThreads = 128;                // one per query row
+constexpr int kThreadsS = kSoftmaxThreads + 64;
+constexpr int kMiscBytes = 1024;
 
 template <int D> struct SmLayout {
     static constexpr int KB = D / 64;                    // 64-column blocks of the head dimension
-    // TMEM decides how much of a CTA's tile loop can overlap (two CTAs per SM, 256 columns each).  64 columns: O
-    // and three logit tiles fit, and two warpgroups take turns, each with its next logits ready while the
-    // other's product runs.  128 columns: O leaves room for two logit tiles, i.e. for one group's next tile
-    // -- a second group would only wait (measured: same time).
-    static constexpr int kGroups = D == 64 ? 2 : 1;
-    static constexpr int kLogits = D == 64 ? 3 : 2;
-    static constexpr int kStages = kLogits;              // K/V tiles in flight
-    static constexpr int kSoftmaxThreads = kGroups * kGroupThreads;
-    static constexpr int kThreads = kSoftmaxThreads + 64;
+    // What overlaps: at 64 columns three CTAs per SM, each one tile at a time (128 TMEM columns: O and one logit tile); at
+    // 128 two CTAs, each with the next tile's logits ready (256 columns).  A CTA's tile is a chain, and a third of a CTA is
+    // its fixed part, another chain, so independent CTAs fill the SM better than more tiles in flight in each.  Forward of
+    // 96 pairs of 2048 tokens: 64.8 us with two warpgroups and three logit tiles in each of two CTAs, 53 now; with four
+    // CTAs 54 (their 80 registers mean reading half the logits twice).
+    static constexpr int kLogits = D == 64 ? 1 : 2;
+    static constexpr int kCtas = D == 64 ? 3 : 2;
+    static constexpr int kTmemCols = D == 64 ? 128 : 256;
+    static constexpr int kStages = 2;                    // K/V tiles in flight
     static constexpr int kQBytes = KB * kBM * 128;
     static constexpr int kKStage = KB * kBN * 128;
     static constexpr int kVStage = KB * kBN * 128;
@@ -76,19 +73,13 @@ template <int D> struct SmLayout {
     static constexpr int oV = oK + kStages * kKStage;
     static constexpr int oMisc = oV + kStages * kVStage;
     static constexpr int kTotal = oMisc + kMiscBytes;
-    // 4 KB per softmax warp through which o_nla leaves, when it is asked for: the K ring at 128 columns; at 64, where
-    // the ring holds o_laT tiles, behind everything else.
-    static constexpr int oRows = D == 128 ? oK : kTotal, kRows = D == 128 ? 0 : kSoftmaxThreads * 128;
-    static_assert(D == 64 || kStages * kKStage >= kSoftmaxThreads * 128, "rows do not fit the K ring");
 };
 
 struct Misc {                    // lives in the last kMiscBytes of the CTA's shared memory
-    uint64_t barQ, barQn, barKn[2], fullK[3], emptyK[3], fullV[3], emptyV[3], barS[3], barP[3], barO[2], barF, barE, barM[2][4];
+    uint64_t barQ, barQn, barKn[2], fullK[2], emptyK[2], fullV[2], emptyV[2], barS[2], barP[2], barO[2], barE;
     uint32_t tmem_base;
     int abort_flag, wait_kcycles;   // in this order: the waits read the limit as abort_flag[1]
     uint32_t kept[kBM / 32];        // which of the CTA's own tokens are retained
-    float m_row[kBM];               // running maximum of each row (base 2), handed from tile to tile
-    float2 xch[2][kBM], xch2[2][kBM];   // exchanges between the two warpgroups, per row
 };
 static_assert(sizeof(Misc) <= kMiscBytes, "misc page too small");
 
@@ -124,7 +115,7 @@ template <int N> __device__ __forceinline__ void row_to_fp16(uint8_t *rowp, int 
 // kBlock: block-level routing (own-block tiles after the retained ones); kG: softmax heads per linear
 // head; kNorm: RMS-normalised q and k (norm_eps is read only then)
 template <int D, bool kBlock, int kG, bool kNorm>
-__global__ void __launch_bounds__(SmLayout<D>::kThreads, 2)
+__global__ void __launch_bounds__(kThreadsS, SmLayout<D>::kCtas)
 softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                           const __grid_constant__ CUtensorMap map_k,
                           const __grid_constant__ CUtensorMap map_v,
@@ -139,8 +130,7 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                           float *__restrict__ lse, int32_t *sm_len, int len_cap, int32_t *status, int L, int H,
                           int wait_kcycles, int segs, int seg_tiles) {
     using SL = SmLayout<D>;
-    constexpr int KB = SL::KB, kStages = SL::kStages, kLogits = SL::kLogits, kGroups = SL::kGroups;
-    constexpr int kSoftmaxThreads = SL::kSoftmaxThreads, kAhead = kLogits - 1;
+    constexpr int KB = SL::KB, kStages = SL::kStages, kLogits = SL::kLogits, kAhead = kLogits - 1;
     constexpr int DL = D * kG;                            // columns of the linear head
     // the two o_laT tiles of the epilogue land in the Q tile and, for grouped heads, the K ring behind it
     static_assert(2 * DL * 128 <= SL::kQBytes + (kG > 1 ? kStages * SL::kKStage : 0), "o_laT tiles do not fit");
@@ -173,8 +163,8 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
         end_behind_scan();
         return;
     }
-    // The TMA warp sets the barriers up and requests the Q tile before anything else, so that the tile travels
-    // while the other warps look up which keys the CTA sees.
+    // The TMA warp sets the barriers up and requests the Q tile before anything else, and goes on to the key tiles as soon
+    // as it knows how many there are: it needs nothing of what the other warps set up.
     if (warp == kTmaWarp && lane == 0) {
         mbar_init(&ms.barQ, 1);
         mbar_init(&ms.barQn, kSoftmaxThreads);       // normalised queries written (NATSL_QK_NORM)
@@ -184,14 +174,8 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
             mbar_init(&ms.fullK[s], 1); mbar_init(&ms.emptyK[s], 1);
             mbar_init(&ms.fullV[s], 1); mbar_init(&ms.emptyV[s], 1);
         }
-        // (barP by logit tile, not by warpgroup: with the logits of tile t + 2 ready early, a fast warp's arrival for
-        // that tile would otherwise complete tile t's phase in place of a slow warp's)
-        for (int s = 0; s < kLogits; ++s) { mbar_init(&ms.barS[s], 1); mbar_init(&ms.barP[s], kGroupThreads); }
-        for (int s = 0; s < 2; ++s) {
-            mbar_init(&ms.barO[s], 1);
-            for (int q = 0; q < 4; ++q) mbar_init(&ms.barM[s][q], 1);
-        }
-        mbar_init(&ms.barF, 1);
+        for (int s = 0; s < kLogits; ++s) { mbar_init(&ms.barS[s], 1); mbar_init(&ms.barP[s], kSoftmaxThreads); }
+        for (int s = 0; s < 2; ++s) mbar_init(&ms.barO[s], 1);
         mbar_init(&ms.barE, 1);
         ms.abort_flag = 0;
         ms.wait_kcycles = wait_kcycles;
@@ -200,6 +184,10 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
         mbar_arrive_expect_tx(&ms.barQ, SL::kQBytes);
         for (int kb = 0; kb < KB; ++kb)
             tma_load_4d(smem + SL::oQ + kb * kBM * 128, &map_q, &ms.barQ, kb * 64, hq, p * kBM, b);
+    }
+    if (warp == kTmaWarp) {
+        __syncwarp();
+        named_barrier_arrive(4, kThreadsS);
     }
     const int c0 = 2 * p, c1 = min(2 * p + 2, NC);
     const int32_t *pre = sm_chunk_prefix + (size_t)bh * (NC + 1);
@@ -237,13 +225,12 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
         }
     }
     if (tid < kBM / 32) ms.kept[tid] = 0u;
-    if (tid < kBM) ms.m_row[tid] = -INFINITY;
-    if (warp == kMmaWarp) tmem_alloc(&ms.tmem_base, 256);
+    if (warp == kMmaWarp) tmem_alloc(&ms.tmem_base, SL::kTmemCols);
     tc_fence_before_sync();
-    __syncthreads();
+    if (warp != kTmaWarp) named_barrier_sync(4, kThreadsS);
     tc_fence_after_sync();
-    const uint32_t tmem = ms.tmem_base;
-    const uint32_t tO = tmem + 64 * kLogits;            // (128 columns: logits at 0, 64; 64 columns: at 0, 64, 128)
+    const uint32_t tmem = ms.tmem_base;                   // (not the TMA warp's business)
+    const uint32_t tO = tmem + 64 * kLogits;            // (logits at 0, and 64 at 128 columns)
     auto tS = [&](int t) { return tmem + 64 * (t % kLogits); };
     volatile int *abort_flag = &ms.abort_flag;
 
@@ -281,8 +268,6 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                         nv = t + 1;
                     }
                 }
-                // the Q tile and the K ring are free once the last Q K^T has run
-                if (ok) ok = mbar_wait(&ms.emptyK[(T2 - 1) % kStages], ((T2 - 1) / kStages) & 1, abort_flag);
             }
             mbar_wait_drain(&ms.barQ, 0);       // (the Q tile's copy, read or not, before its place is reused)
             // beside the scan: the tile's chunks of o_la are complete once all row warps of the scan
@@ -292,6 +277,8 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                     ok = wait_counter_ge(emit_flags + (size_t)bh * NC + c, kScanRowWarps, abort_flag);
                 fence_proxy_async_all();
             }
+            // the Q tile and the K ring are free once the last Q K^T has run
+            if (T2 > 0 && ok) ok = mbar_wait(&ms.emptyK[(T2 - 1) % kStages], ((T2 - 1) / kStages) & 1, abort_flag);
             bool e_issued = false;
             if (ok) {                           // the o_laT tiles of the CTA's one or two chunks
                 mbar_arrive_expect_tx(&ms.barE, (c1 - c0) * DL * 128);
@@ -348,7 +335,7 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
             for (int t = 0; t < kAhead && ok; ++t) ok = next_qk(t);
             for (int t = 0; ok && t < T2u; ++t) {
                 // (keys that the softmax threads still have to normalise must not hold up this tile's product)
-                const bool late = kBlock && kNorm && t + kAhead >= Tu;
+                const bool late = kAhead > 0 && kBlock && kNorm && t + kAhead >= Tu;
                 if (!late) ok = next_qk(t + kAhead);
                 ok = ok && wait_all(&ms.barP[t % kLogits], (t / kLogits) & 1, abort_flag) &&
                      wait_all(&ms.fullV[t % kStages], (t / kStages) & 1, abort_flag);
@@ -364,28 +351,25 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                 }
                 if (late) ok = next_qk(t + kAhead);
             }
-            if (ok && elect_one()) mma_commit(&ms.barF);              // every product has run
         }
     } else {
         // ------------------------------ softmax + epilogue ------------------------------
-        const int wg = warp >> 2, q = warp & 3;         // warpgroup; quarter of the rows
-        constexpr int kPq = 8 / kGroups;                // 16-byte pieces of a block of the query row per thread
-        const int tg = tid & (kGroupThreads - 1);
-        const int r = tg;                               // query row inside the tile, TMEM lane
+        const int q = warp;                             // quarter of the rows
+        const int r = tid;                              // query row inside the tile, TMEM lane
         const int i_abs = p * kBM + r;
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
         const float sl2 = scale_sm * 1.4426950408889634f;
-        float m_mine = -INFINITY, l = 0.f;              // maximum this thread's sum is relative to; the sum
+        float m = -INFINITY, l = 0.f;                   // maximum (base 2) the row's sum is relative to; the sum
         bool ok = true;
         // Which of the CTA's own tokens are retained (sm_idx lists this call's retained tokens; when the call
         // appends to a cache, pre[0] were there before): the keys a row sees are then a population count.
-        if (wg == 0 && n_full + tg < n_end) {
-            const int rel = sm_idx[(size_t)bh * L + n_full + tg - (appending ? pre[0] : 0)] - p * kBM;
+        if (n_full + r < n_end) {
+            const int rel = sm_idx[(size_t)bh * L + n_full + r - (appending ? pre[0] : 0)] - p * kBM;
             atomicOr(&ms.kept[(rel >> 5) & 3], 1u << (rel & 31));
         }
         if (kNorm && T2 > 0) {
-            // RMS-normalised queries (Section 4.3): the threads of row r rewrite their pieces of its
-            // blocks (bf16, as loaded) as fp16 of the normalised row, over the D columns of its softmax head;
+            // RMS-normalised queries (Section 4.3): thread r rewrites row r (bf16, as loaded) as fp16 of the normalised
+            // row, over the D columns of its softmax head;
             // the keys were normalised and stored as fp16 when they were gathered, so the logit product is
             // an fp16 MMA (bf16 keeps 8 bits: rounding the normalised keys to it alone costs 2.8e-2 of the
             // branch output's RMS).
@@ -394,16 +378,11 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
             float ss = 0.f;
             if (ok)
 #pragma unroll
-                for (int kb = 0; kb < KB; ++kb) ss += row_square_sum<kPq>(rowp + kb * kBM * 128, kPq * wg, r & 7);
-            if (kGroups > 1) {
-                ms.xch[wg][r].x = ss;
-                named_barrier_sync(1, kSoftmaxThreads);
-                ss = ms.xch[0][r].x + ms.xch[1][r].x;
-            }
+                for (int kb = 0; kb < KB; ++kb) ss += row_square_sum<8>(rowp + kb * kBM * 128, 0, r & 7);
             if (ok) {
                 const float rq = rsqrtf(ss / D + norm_eps);
 #pragma unroll
-                for (int kb = 0; kb < KB; ++kb) row_to_fp16<kPq>(rowp + kb * kBM * 128, kPq * wg, r & 7, rq);
+                for (int kb = 0; kb < KB; ++kb) row_to_fp16<8>(rowp + kb * kBM * 128, 0, r & 7, rq);
                 fence_proxy_async_smem();
                 mbar_arrive(&ms.barQn);
             }
@@ -416,84 +395,87 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
         int cnt = n_full + __popc(ms.kept[q] & ((2u << lane) - 1u));
 #pragma unroll
         for (int e = 0; e < kBM / 32 - 1; ++e) cnt += e < q ? __popc(ms.kept[e]) : 0;
-        for (int t = wg; ok && t < T2; t += kGroups) {
+        for (int t = 0; ok && t < T2; ++t) {
             if (kBlock && kNorm && t >= T) {
                 // Keys of an own-block tile (block-level routing with normalisation): raw bf16 rows from the
                 // layer's k; two threads per row rewrite it as fp16 of the RMS-normalised row.  One arrival per
                 // tile, after all rows are written.
                 ok = mbar_wait(&ms.fullK[t % kStages], (t / kStages) & 1, abort_flag);
-                uint8_t *rowp = smem + SL::oK + (t % kStages) * SL::kKStage + (tg >> 1) * 128;
+                uint8_t *rowp = smem + SL::oK + (t % kStages) * SL::kKStage + (r >> 1) * 128;
                 if (ok) {
                     float ss = 0.f;
 #pragma unroll
-                    for (int kb = 0; kb < KB; ++kb) ss += row_square_sum<4>(rowp + kb * kBN * 128, 4 * (tg & 1), (tg >> 1) & 7);
+                    for (int kb = 0; kb < KB; ++kb) ss += row_square_sum<4>(rowp + kb * kBN * 128, 4 * (r & 1), (r >> 1) & 7);
                     ss += __shfl_xor_sync(0xffffffffu, ss, 1);
                     const float rk = rsqrtf(ss / D + norm_eps);
 #pragma unroll
-                    for (int kb = 0; kb < KB; ++kb) row_to_fp16<4>(rowp + kb * kBN * 128, 4 * (tg & 1), (tg >> 1) & 7, rk);
+                    for (int kb = 0; kb < KB; ++kb) row_to_fp16<4>(rowp + kb * kBN * 128, 4 * (r & 1), (r >> 1) & 7, rk);
                 }
                 fence_proxy_async_smem();
-                named_barrier_sync(2 + wg, kGroupThreads);
-                if (tg == 0 && ok) mbar_arrive(&ms.barKn[t - T]);
+                named_barrier_sync(1, kSoftmaxThreads);
+                if (r == 0 && ok) mbar_arrive(&ms.barKn[t - T]);
                 if (!ok) break;
             }
             ok = mbar_wait(&ms.barS[t % kLogits], (t / kLogits) & 1, abort_flag);
             if (!ok) break;
             tc_fence_after_sync();
-            float x[kBN];                                // raw logits: the scale goes into the exponent's FMA
-            tmem_ld32(tS(t) + lane_base, reinterpret_cast<uint32_t (&)[32]>(x[0]));
-            tmem_ld32(tS(t) + lane_base + 32, reinterpret_cast<uint32_t (&)[32]>(x[32]));
-            tmem_wait_ld();
             // Keys of this tile the row sees: an own-block tile's 0 .. r % 64 if the row is in that block, else those
             // of the compacted order before `cnt`.
             const int vis = kBlock && t >= T ? ((r >> 6) == own_block(t) ? (r & 63) + 1 : 0) : cnt - t * kBN;
-            if (!__all_sync(0xffffffffu, vis >= kBN)) {   // some row of the warp is cut off here
+            const bool cut_off = !__all_sync(0xffffffffu, vis >= kBN);   // some row of the warp is cut off here
+            // 32 raw logits at a time (the scale goes into the exponent's FMA)
+            auto load_half = [&](int hf, float (&x)[32]) {
+                tmem_ld32(tS(t) + lane_base + 32 * hf, reinterpret_cast<uint32_t (&)[32]>(x));
+                tmem_wait_ld();
+                if (cut_off) {
 #pragma unroll
-                for (int c = 0; c < kBN; ++c) x[c] = c < vis ? x[c] : -INFINITY;
-            }
-            float mx4[4] = {x[0], x[1], x[2], x[3]};      // four independent chains
+                    for (int c = 0; c < 32; ++c) x[c] = c + 32 * hf < vis ? x[c] : -INFINITY;
+                }
+            };
+            auto max_half = [&](const float (&x)[32]) {      // four independent chains
+                float m4[4] = {x[0], x[1], x[2], x[3]};
 #pragma unroll
-            for (int c = 4; c < kBN - 4; c += 8)
+                for (int c = 4; c < 28; c += 8)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) mx4[e] = max3(mx4[e], x[c + e], x[c + 4 + e]);
+                    for (int e = 0; e < 4; ++e) m4[e] = max3(m4[e], x[c + e], x[c + 4 + e]);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) mx4[e] = fmaxf(mx4[e], x[kBN - 4 + e]);
+                for (int e = 0; e < 4; ++e) m4[e] = fmaxf(m4[e], x[28 + e]);
+                return fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+            };
+            float xa[32], xb[32];
+            load_half(0, xa);
+            float mx = max_half(xa);
+            load_half(1, xb);
             // (scale_sm > 0, checked on the host: the maximum of the raw logits is the maximum logit)
-            const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * sl2;
-            // The running maximum passes from tile to tile, i.e. between the warpgroups.  It only has to
+            mx = fmaxf(mx, max_half(xb)) * sl2;
+            // The running maximum only has to
             // bound the exponents, not equal the true maximum: it is raised (and O rescaled) only when a logit
             // exceeds it by more than 8 (base 2), so probabilities stay below 2^8 and, for inputs whose logits
             // vary little, the accumulator is never touched between the tiles.  lse = m + log2(l) holds for
             // any such m.
-            if (kGroups > 1 && t > 0) {
-                ok = mbar_wait(&ms.barM[(t - 1) & 1][q], ((t - 1) >> 1) & 1, abort_flag);
-                if (!ok) break;
-            }
-            const float m_old = kGroups > 1 ? ms.m_row[r] : m_mine;
-            const float m_new = (mx > m_old + 8.f || m_old == -INFINITY) ? fmaxf(m_old, mx) : m_old;
-            if (kGroups > 1) {
-                ms.m_row[r] = m_new;
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&ms.barM[t & 1][q]);
-            }
-            const float m_use = m_new == -INFINITY ? 0.f : m_new;
+            const float m_old = m;
+            m = (mx > m_old + 8.f || m_old == -INFINITY) ? fmaxf(m_old, mx) : m_old;
+            const float m_use = m == -INFINITY ? 0.f : m;
             uint64_t ps[2] = {0ull, 0ull};
             uint32_t pk[32];                            // P(t), over the logits this thread has consumed
             const uint64_t sl22 = pack2(sl2, sl2), nm2 = pack2(-m_use, -m_use);
+            auto exps = [&](int hf, const float (&x)[32]) {
 #pragma unroll
-            for (int c = 0; c < kBN; c += 2) {
-                const float2 e = unpack2(fma2(pack2(x[c], x[c + 1]), sl22, nm2));
-                const float p0 = ex2_ftz(e.x), p1 = ex2_ftz(e.y);
-                ps[(c >> 1) & 1] = add2(ps[(c >> 1) & 1], pack2(p0, p1));
-                pk[c >> 1] = pack_half2(p0, p1);
-            }
+                for (int c = 0; c < 32; c += 2) {
+                    const float2 e = unpack2(fma2(pack2(x[c], x[c + 1]), sl22, nm2));
+                    const float p0 = ex2_ftz(e.x), p1 = ex2_ftz(e.y);
+                    ps[(c >> 1) & 1] = add2(ps[(c >> 1) & 1], pack2(p0, p1));
+                    pk[16 * hf + (c >> 1)] = pack_half2(p0, p1);
+                }
+            };
+            exps(1, xb);
+            exps(0, xa);
             const float2 psf = unpack2(add2(ps[0], ps[1]));
-            l = l * ex2_ftz(m_mine - m_use) + (psf.x + psf.y);   // (m = -inf: l is 0)
-            m_mine = m_new;
+            l = l * ex2_ftz(m_old - m_use) + (psf.x + psf.y);    // (m = -inf: l is 0)
             tmem_st32(tS(t) + lane_base, pk);
-            if (t > 0 && __any_sync(0xffffffffu, m_new != m_old)) {
-                // (the logits of tile t were issued behind the product of tile t - 3, so the phase of this barrier
-                // before tile t - 1's has completed and the parity is unambiguous)
+            if (t > 0 && __any_sync(0xffffffffu, m != m_old)) {
+                // (the logits of tile t were issued behind the product of tile t - 2 at the latest, so the phase of this
+                // barrier before tile t - 1's has completed and the parity is unambiguous)
                 ok = mbar_wait(&ms.barO[(t - 1) & 1], ((t - 1) >> 1) & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after_sync();
@@ -513,7 +495,7 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                 ok = mbar_wait(&ms.fullV[t % kStages], (t / kStages) & 1, abort_flag);
                 if (!ok) break;
                 uint4 *vt = reinterpret_cast<uint4 *>(smem + SL::oV + (t % kStages) * SL::kVStage);
-                for (int i = tg; i < SL::kVStage / 16; i += kGroupThreads) {
+                for (int i = r; i < SL::kVStage / 16; i += kSoftmaxThreads) {
                     const uint4 a = vt[i];
                     auto cv = [](uint32_t wd) {
                         return pack_half2(__uint_as_float(wd << 16), __uint_as_float(wd & 0xffff0000u));
@@ -526,109 +508,121 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
             mbar_arrive(&ms.barP[t % kLogits]);
         }
         if (ok && T2 > 0) {
-            ok = mbar_wait(&ms.barF, 0, abort_flag);
+            ok = mbar_wait(&ms.barO[(T2 - 1) & 1], ((T2 - 1) >> 1) & 1, abort_flag);
             tc_fence_after_sync();
         }
-        // ---- epilogue: each warpgroup takes its share of the softmax head's columns of every row ----
-        constexpr int HC = D / kGroups;
-        float m = m_mine;
-        if (kGroups > 1) {
-            ms.xch[wg][r] = make_float2(l, m_mine);
-            named_barrier_sync(1, kSoftmaxThreads);
-            m = ms.m_row[r];
-            const float2 a0 = ms.xch[0][r], a1 = ms.xch[1][r];
-            l = (a0.x > 0.f ? a0.x * ex2_ftz(a0.y - m) : 0.f) + (a1.x > 0.f ? a1.x * ex2_ftz(a1.y - m) : 0.f);
-        }
+        // ---- epilogue ----
         if (ok) ok = mbar_wait(&ms.barE, 0, abort_flag);        // the tile's rows of o_la have landed
         // o_laT tiles (fp16): chunk e of the CTA at oQ + e * D * 128; piece pc (tokens 8 pc ..) of
-        // head-dimension row `row` at 16-byte slot pc * D + (row ^ pc).
+        // head-dimension row `row` at 16-byte slot pc * D + (row ^ pc): eight such rows are an 8 x 8 matrix, which ldmatrix
+        // transposes on the way.  The accumulator is read in the layout that gives (lane l: tokens l / 4, + 8 and the
+        // columns 2 (l % 4), + 1 of every 8), and `out` leaves that layout through stmatrix.
         // out tile (bf16): box kb (columns 64 kb ..) at oV + kb * 16 KB, row r, piece j at j ^ (r & 7).
+        // (A thread reading its own token's column out of these tiles took a two-byte load per value, twice: the epilogue
+        // was 8 of the 15 thousand cycles of a CTA with two key tiles.)
         const float inv = l > 0.f ? 1.f / l : 0.f;       // l = 0 (no visible key): o_nla = 0
-        const int tok = r & 63, tp = tok >> 3;
-        const uint8_t *la_col = smem + SL::oQ + (r >> 6) * (DL * 128) + tp * (DL * 16) + (tok & 7) * 2;
-        // Two passes over the row's columns, 32 at a time (rolled: the kernel is large enough for its warps to wait
-        // for instructions): mean squares of both branches, then the output.
-        auto la_pair = [&](int row) {        // o_la of this query, head-dimension rows row, row + 1
-            const __half a0 = *reinterpret_cast<const __half *>(la_col + ((row ^ tp) << 4));
-            const __half a1 = *reinterpret_cast<const __half *>(la_col + (((row + 1) ^ tp) << 4));
-            return __half22float2(__halves2half2(a0, a1));
-        };
-        auto load_o = [&](int cb, uint32_t (&ov)[32]) {
-            if (T2 > 0) {
-                tmem_ld32(tO + lane_base + wg * HC + cb * 32, ov);
-                tmem_wait_ld();
-            } else {
+        const uint32_t sm32 = smem_u32(smem);
+        const int l8 = lane & 7, mi = lane >> 3, g8 = lane >> 2;
+        constexpr int NB = D / 32;                       // 32-column blocks of the softmax head
+        // this lane's share of 16 tokens (from tok0 on) x 32 columns (from col on) of o_la, fp16 pairs: [8-column block][token half]
+        auto load_la = [&](int row0, int col, uint32_t (&la)[4][2]) {
+            const int pc = ((row0 & 63) >> 3) + (mi & 1);
+            const uint32_t tile = sm32 + SL::oQ + (row0 >> 6) * (DL * 128) + pc * (DL * 16);
 #pragma unroll
-                for (int e = 0; e < 32; ++e) ov[e] = 0u;
+            for (int c2 = 0; c2 < 2; ++c2) {
+                uint32_t v[4];
+                ldmatrix_x4_trans(tile + (((col + 16 * c2 + 8 * (mi >> 1) + l8) ^ pc) << 4), v);
+                la[2 * c2][0] = v[0]; la[2 * c2][1] = v[1]; la[2 * c2 + 1][0] = v[2]; la[2 * c2 + 1][1] = v[3];
             }
         };
-        float ssn4[4] = {0.f, 0.f, 0.f, 0.f}, ssl4[4] = {0.f, 0.f, 0.f, 0.f};
-        if (ok) {
-            if (kG > 1) {        // the other softmax heads' columns of the linear row: mean square only
-#pragma unroll 4
-                for (int e = 0; e < (kG - 1) * HC; e += 2) {
-                    const int gg = e / HC;
-                    const float2 a = la_pair((gg < sg ? gg : gg + 1) * D + wg * HC + e % HC);
-                    ssl4[(e >> 1) & 3] = fmaf(a.x, a.x, fmaf(a.y, a.y, ssl4[(e >> 1) & 3]));
-                }
-            }
+        auto quad_sum = [](float x) {
+            x += __shfl_xor_sync(0xffffffffu, x, 1);
+            return x + __shfl_xor_sync(0xffffffffu, x, 2);
+        };
 #pragma unroll 1
-            for (int cb = 0; cb < HC / 32; ++cb) {
-                uint32_t ov[32];
-                load_o(cb, ov);
+        for (int hh = 0; hh < 2; ++hh) {                 // 16 of the warp's 32 tokens at a time
+            const int row0 = 32 * q + 16 * hh;
+            uint32_t o[NB][16], la[NB][4][2];
+            float ssn[2] = {0.f, 0.f}, ssl[2] = {0.f, 0.f};        // squares: tokens row0 + g8, + 8
 #pragma unroll
-                for (int e = 0; e < 32; e += 2) {
-                    const float2 a = la_pair(sg * D + wg * HC + 32 * cb + e);
-                    ssl4[(e >> 1) & 3] = fmaf(a.x, a.x, fmaf(a.y, a.y, ssl4[(e >> 1) & 3]));
-                    const float o0 = __uint_as_float(ov[e]), o1 = __uint_as_float(ov[e + 1]);
-                    ssn4[(e >> 1) & 3] = fmaf(o0, o0, fmaf(o1, o1, ssn4[(e >> 1) & 3]));
+            for (int nb = 0; nb < NB; ++nb)
+                if (T2 > 0) tmem_ld_16x32(tO + lane_base + ((uint32_t)(16 * hh) << 16) + 32 * nb, o[nb]);
+                else {
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) o[nb][e] = 0u;
                 }
-            }
-        }
-        float ssn = (ssn4[0] + ssn4[1]) + (ssn4[2] + ssn4[3]), ssl = (ssl4[0] + ssl4[1]) + (ssl4[2] + ssl4[3]);
-        if (kGroups > 1) {
-            ms.xch2[wg][r] = make_float2(ssn, ssl);
-            named_barrier_sync(1, kSoftmaxThreads);
-            ssn = ms.xch2[0][r].x + ms.xch2[1][r].x;
-            ssl = ms.xch2[0][r].y + ms.xch2[1][r].y;
-        }
-        if (ok) {
-            // mean square of the normalised row = inv^2 * mean square of the accumulator row
-            const float wn = wv.x * rsqrtf(inv * inv * ssn / D + eps) * inv;          // applies to the raw accumulator
-            const float wl = wv.y * rsqrtf(ssl / DL + eps);
-#pragma unroll 1
-            for (int cb = 0; cb < HC / 32; ++cb) {
-                uint32_t ov[32];
-                load_o(cb, ov);
+            auto squares = [&](const uint32_t (&a)[4][2]) {
 #pragma unroll
-                for (int j2 = 0; j2 < 4; ++j2) {
-                    float y[8];
+                for (int j = 0; j < 4; ++j)
 #pragma unroll
-                    for (int e = 0; e < 8; e += 2) {
-                        const float2 a = la_pair(sg * D + wg * HC + 32 * cb + 8 * j2 + e);
-                        y[e] = fmaf(wn, __uint_as_float(ov[8 * j2 + e]), wl * a.x);
-                        y[e + 1] = fmaf(wn, __uint_as_float(ov[8 * j2 + e + 1]), wl * a.y);
+                    for (int t8 = 0; t8 < 2; ++t8) {
+                        const float2 y = __half22float2(*reinterpret_cast<const __half2 *>(&a[j][t8]));
+                        ssl[t8] = fmaf(y.x, y.x, fmaf(y.y, y.y, ssl[t8]));
                     }
-                    const int col = wg * HC + cb * 32 + j2 * 8;
-                    if (has_out)
-                        *reinterpret_cast<uint4 *>(smem + SL::oV + (col >> 6) * (kBM * 128) + sw128_offset(r, (col & 63) >> 3)) =
-                            make_uint4(pack_bf162(y[0], y[1]), pack_bf162(y[2], y[3]), pack_bf162(y[4], y[5]),
-                                       pack_bf162(y[6], y[7]));
-                }
-            }
-            if (o_nla) {                // the raw branch output (fp32); its own loop keeps the one above small
-                const int i_warp = p * kBM + 32 * (warp & 3);                           // the warp's first query
-                float *dst = o_nla + (((size_t)b * L + i_warp) * H + h) * DL + sg * D + wg * HC;
+            };
+            if (kG > 1) {        // the other softmax heads' columns of the linear row: mean square only
 #pragma unroll 1
-                for (int cb = 0; cb < HC / 32; ++cb) {
-                    uint32_t ov[32];
-                    load_o(cb, ov);
-                    store_rows32(smem + SL::oRows + warp * 4096, ov, inv, dst + cb * 32, (size_t)H * DL, L - i_warp, lane);
+                for (int e = 0; e < (kG - 1) * NB; ++e) {
+                    const int gg = e / NB;
+                    load_la(row0, (gg < sg ? gg : gg + 1) * D + e % NB * 32, la[0]);
+                    squares(la[0]);
                 }
             }
-            if (lse && wg == 0 && i_abs < L)
-                lse[(size_t)bhg * L + i_abs] = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
+#pragma unroll
+            for (int nb = 0; nb < NB; ++nb) {
+                load_la(row0, sg * D + 32 * nb, la[nb]);
+                squares(la[nb]);
+            }
+            if (T2 > 0) tmem_wait_ld();
+#pragma unroll
+            for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                for (int e = 0; e < 16; ++e)
+                    ssn[(e >> 1) & 1] = fmaf(__uint_as_float(o[nb][e]), __uint_as_float(o[nb][e]), ssn[(e >> 1) & 1]);
+            float iv[2], wn[2], wl[2];
+#pragma unroll
+            for (int t8 = 0; t8 < 2; ++t8) {
+                const int src = 16 * hh + g8 + 8 * t8;     // the lane that holds the token's row
+                iv[t8] = __shfl_sync(0xffffffffu, inv, src);
+                // mean square of the normalised row = inv^2 * mean square of the accumulator row
+                wn[t8] = __shfl_sync(0xffffffffu, wv.x, src) * rsqrtf(iv[t8] * iv[t8] * quad_sum(ssn[t8]) / D + eps) * iv[t8];   // applies to the raw accumulator
+                wl[t8] = __shfl_sync(0xffffffffu, wv.y, src) * rsqrtf(quad_sum(ssl[t8]) / DL + eps);
+            }
+            if (has_out && ok) {
+                const int r_st = row0 + 8 * (mi & 1) + l8;
+#pragma unroll
+                for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                    for (int c2 = 0; c2 < 2; ++c2) {
+                        uint32_t y[4];                     // [8-column block][token half]
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const int cb = 2 * c2 + (j >> 1), t8 = j & 1;
+                            const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&la[nb][cb][t8]));
+                            y[j] = pack_bf162(fmaf(wn[t8], __uint_as_float(o[nb][4 * cb + 2 * t8]), wl[t8] * a.x),
+                                              fmaf(wn[t8], __uint_as_float(o[nb][4 * cb + 2 * t8 + 1]), wl[t8] * a.y));
+                        }
+                        const int col = 32 * nb + 16 * c2 + 8 * (mi >> 1);
+                        stmatrix_x4(sm32 + SL::oV + (col >> 6) * (kBM * 128) + sw128_offset(r_st, (col & 63) >> 3), y[0], y[1], y[2], y[3]);
+                    }
+            }
+            if (o_nla && ok) {          // the raw branch output (fp32): a quad's pairs of columns are whole 32-byte sectors
+#pragma unroll
+                for (int t8 = 0; t8 < 2; ++t8) {
+                    const int i = p * kBM + row0 + g8 + 8 * t8;
+                    float *dst = o_nla + (((size_t)b * L + i) * H + h) * DL + sg * D + 2 * (lane & 3);
+                    if (i < L)
+#pragma unroll
+                        for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                            for (int cb = 0; cb < 4; ++cb)
+                                *reinterpret_cast<float2 *>(dst + 32 * nb + 8 * cb) =
+                                    make_float2(iv[t8] * __uint_as_float(o[nb][4 * cb + 2 * t8]), iv[t8] * __uint_as_float(o[nb][4 * cb + 2 * t8 + 1]));
+                }
+            }
         }
+        if (ok && lse && i_abs < L)
+            lse[(size_t)bhg * L + i_abs] = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
         fence_proxy_async_smem();
         named_barrier_sync(1, kSoftmaxThreads);
         if (tid == 0 && ok) {
@@ -644,7 +638,7 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
     __syncthreads();
     if (warp == kMmaWarp) {
         tc_fence_after_sync();
-        tmem_dealloc(tmem, 256);
+        tmem_dealloc(tmem, SL::kTmemCols);
     }
     if (tid == 0 && ms.abort_flag) atomicMin(status, (int)NATSL_ERR_TIMEOUT);
     end_behind_scan();
@@ -825,15 +819,15 @@ static cudaError_t softmax_tc_impl(const void *q, const void *k_sm, const void *
     if (norm_eps >= 0.f) kernel = softmax_combine_tc_kernel<D, false, G, true>;
     if (br.route) kernel = norm_eps >= 0.f ? softmax_combine_tc_kernel<D, true, G, true>
                                           : softmax_combine_tc_kernel<D, true, G, false>;
-    cudaError_t e = allow_smem(kernel, SL::kTotal + SL::kRows);
+    cudaError_t e = allow_smem(kernel, SL::kTotal);
     if (e != cudaSuccess) return e;
     // With emit_flags the kernel is launched as a programmatic dependent of the kernel before it in
     // the stream (the scan): it may start once all of the scan's CTAs are resident, and finds o_la
     // through the flags.  A launch the runtime serialises instead finds every flag already raised.
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(s.B * s.H * G, (s.L + kBM - 1) / kBM);
-    cfg.blockDim = dim3(SL::kThreads);
-    cfg.dynamicSmemBytes = SL::kTotal + (o_nla ? SL::kRows : 0);
+    cfg.blockDim = dim3(kThreadsS);
+    cfg.dynamicSmemBytes = SL::kTotal;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -331,7 +331,7 @@ static int bwd_forward_part(const void *q, const void *k, const void *v, const f
         // (the kernels of natsl_hybrid_fwd, overlapped like there)
         const bool pdl = !(p->flags & NATSL_SINGLE_STREAM);
         NATSL_TRY(launch_gdn_prepare_tc(q, k, v, g, beta, block ? nullptr : route, p->scale_la, f.tc, f.ex,
-                                        f.status, s, st, (int)(kStatusBytes / 4), hg.norm_eps));
+                                        f.status, s, st, (int)(kStatusBytes / 4), hg.norm_eps, pdl));
         NATSL_TRY(launch_route_gather_tc(k, v, route, f.sm_idx, f.prefix, nullptr, f.k_smb, nullptr, f.v16, f.k16, p->L,
                                          p->L, f.emit_flags, s, st, pdl, hg));
         NATSL_TRY(launch_gdn_scan_tc(q, k, v, f.tc, p->scale_la, p->state_in, state_out, ScanOut{f.o_la16, f.o_la, flags},
@@ -512,7 +512,7 @@ int natsl_hybrid_fwd(const void *q, const void *k, const void *v, const float *g
         const bool pdl = beside && scan_follows_closely(p);
         auto prepare = [&]() {   // block-level routing: every token takes part in the delta rule of its own block
             return launch_gdn_prepare_tc(q, k, v, g, beta, block ? nullptr : route, p->scale_la, f.tc, GdnTcExport{},
-                                         f.status, s, st, (int)(kStatusBytes / 4), hg.norm_eps);
+                                         f.status, s, st, (int)(kStatusBytes / 4), hg.norm_eps, beside);
         };
         auto gather = [&]() {
             return launch_route_gather_tc(k, v, route, f.sm_idx, f.prefix, append ? p->sm_len : nullptr, k_sm,

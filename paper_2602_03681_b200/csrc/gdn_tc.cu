@@ -122,12 +122,14 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
         ms.wait_kcycles = wait_kcycles;
         fence_mbar_init();
     }
+    if (warp == 4) tmem_alloc(&ms.tmem_base, PL::kTmemCols);
+    // (what is set up above needs nothing of the kernel ahead, whose last CTAs may still run)
+    grid_dependency_wait();
     // The forward's first kernel: clears the status page.  The compaction behind it needs nothing of this kernel and
     // may start as soon as the last CTAs have (it fills the multiprocessors as they drain); the scan waits for both.
     if (blockIdx.x == 0 && tid < head_words) status[tid] = 0;
     __threadfence();
     launch_dependents();
-    if (warp == 4) tmem_alloc(&ms.tmem_base, PL::kTmemCols);
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -1172,7 +1174,7 @@ template <int D, bool kTrain>
 static cudaError_t prepare_tc_impl(const void *q, const void *k, const void *v, const float *g,
                                    const float *beta, const uint8_t *route, float scale_la,
                                    const GdnTcWs &ws, const GdnTcExport &ex, int32_t *status,
-                                   float norm_eps, int head_words, Shape s, cudaStream_t st) {
+                                   float norm_eps, int head_words, Shape s, cudaStream_t st, bool pdl) {
     using PL = PrepLayout<D, kTrain>;
     const int NC = s.L / kC;
     const uint64_t BH = (uint64_t)s.B * s.H;
@@ -1192,7 +1194,7 @@ static cudaError_t prepare_tc_impl(const void *q, const void *k, const void *v, 
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)NC * (unsigned)BH);
     count_launch();
-    return launch_kernel(kernel, grid, dim3(kPrepThreads), PL::kTotal, st, false, mq, mk, mv, mqh, mkh, mu, mwt, mtb, mph, g, beta,
+    return launch_kernel(kernel, grid, dim3(kPrepThreads), PL::kTotal, st, pdl, mq, mk, mv, mqh, mkh, mu, mwt, mtb, mph, g, beta,
                          route, scale_la, (__half *)ws.Ph, ws.Gd, ws.Rn, ex, status, head_words, s.L, s.H, norm_eps,
                          debug_wait_kcycles());
 }
@@ -1226,8 +1228,8 @@ static cudaError_t scan_tc_impl(const void *q, const void *k, const void *v, con
 cudaError_t launch_gdn_prepare_tc(const void *q, const void *k, const void *v, const float *g,
                                   const float *beta, const uint8_t *route, float scale_la,
                                   const GdnTcWs &ws, const GdnTcExport &ex, int32_t *status, Shape s,
-                                  cudaStream_t st, int head_words, float norm_eps) {
-#define RUN(D, TR) return prepare_tc_impl<D, TR>(q, k, v, g, beta, route, scale_la, ws, ex, status, norm_eps, head_words, s, st)
+                                  cudaStream_t st, int head_words, float norm_eps, bool pdl) {
+#define RUN(D, TR) return prepare_tc_impl<D, TR>(q, k, v, g, beta, route, scale_la, ws, ex, status, norm_eps, head_words, s, st, pdl)
     if (s.d == 128) {
         if (ex.U16) RUN(128, true);
         RUN(128, false);

@@ -189,7 +189,7 @@ struct GdnTcGrads {
 cudaError_t launch_gdn_prepare_tc(const void *q, const void *k, const void *v, const float *g,
                                   const float *beta, const uint8_t *route, float scale_la,
                                   const GdnTcWs &ws, const GdnTcExport &ex, int32_t *status, Shape s,
-                                  cudaStream_t st, int head_words, float norm_eps = -1.f);
+                                  cudaStream_t st, int head_words, float norm_eps, bool pdl);
 // (the forward's first kernel: clears head_words words of the status page)
 // pdl (here and elsewhere): launched as a programmatic dependent of the kernel before it in the stream.  Every kernel
 // launched so waits for the one before it (grid_dependency_wait) before it ends, at its start or, where it needs nothing

@@ -12,6 +12,7 @@
 // bytes of the chunks' tokens go out as one contiguous run.
 #include "common.cuh"
 #include "natsl_internal.h"
+#include "tc_common.cuh"
 
 namespace natsl {
 
@@ -47,6 +48,9 @@ score_layer_kernel(const T *__restrict__ x, const float *__restrict__ w_score,
     const int g = tid / kHalfThreads, ht = tid % kHalfThreads;       // chunk of the pair, thread within it
     const bool live = c0 + g < NC;                                   // the last pair may be half empty
     const T *xc = x + ((size_t)b * L + (size_t)(c0 + g) * kC) * Dm;
+    // (a programmatic dependent of whatever is ahead of it: a launch's latency is a fifth of a call)
+    tc::grid_dependency_wait();
+    tc::launch_dependents();
 
     for (int col = ht * kE; col < Dm; col += kHalfThreads * kE) {
         float acc[kE];
@@ -115,10 +119,9 @@ cudaError_t score_layer_impl(const void *x, const float *w_score, float *scores,
     const size_t smem = (size_t)kScoreChunks * ((size_t)d_model + 2 * s.H) * sizeof(float);
     cudaError_t e = allow_smem(score_layer_kernel<T>, kScoreSmemMax);
     if (e != cudaSuccess) return e;
-    score_layer_kernel<T><<<grid, kScoreThreads, smem, st>>>((const T *)x, w_score, scores, route, s.L,
-                                                             d_model, s.H);
     count_launch();
-    return cudaGetLastError();
+    return launch_kernel(score_layer_kernel<T>, grid, dim3(kScoreThreads), smem, st, true, (const T *)x, w_score, scores, route,
+                         s.L, d_model, s.H);
 }
 
 }  // namespace

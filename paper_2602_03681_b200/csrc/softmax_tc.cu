@@ -158,6 +158,7 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
         if (tid == 0 && blockIdx.x == 0 && blockIdx.y == gridDim.y - 1) grid_dependency_wait();
     };
 
+    launch_dependents();
     if ((smem_u32(smem) & 1023u) != 0) {              // operand tiles need 1024-byte alignment
         if (tid == 0) atomicMin(status, (int)NATSL_ERR_CUDA);
         end_behind_scan();

@@ -44,6 +44,25 @@ __device__ __forceinline__ uint4 bf16x8_to_f16x8(uint4 u) {
     return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
+// ss + sum of the squares of 8 bf16 values; 8 bf16 values times f as fp16
+__device__ __forceinline__ float square_sum8(uint4 a, float ss) {
+    const uint32_t wd[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const float lo = __uint_as_float(wd[e] << 16), hi = __uint_as_float(wd[e] & 0xffff0000u);
+        ss = fmaf(lo, lo, fmaf(hi, hi, ss));
+    }
+    return ss;
+}
+__device__ __forceinline__ uint4 scale_f16x8(uint4 a, float f) {
+    const uint32_t wd[4] = {a.x, a.y, a.z, a.w};
+    uint32_t o[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        o[e] = pack_half2(__uint_as_float(wd[e] << 16) * f, __uint_as_float(wd[e] & 0xffff0000u) * f);
+    return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
 // ==========================================================================================
 // Prepare: one CTA per chunk of one (batch, head).  One MMA group with M = 128 stacks [Q ; K] on
 // the rows against K: TMEM rows 0-63 then hold Q K^T (-> P) and rows 64-127 K K^T (-> A).  Warps 0-1
@@ -53,7 +72,9 @@ __device__ __forceinline__ uint4 bf16x8_to_f16x8(uint4 u) {
 // 128 threads (one head-dimension row each) take W^T out of TMEM.  Warp 4 issues TMA and MMAs.
 // What bounds it is what it moves, so it hands on as little as the scan can work from: T beta~, W^T, P and the decay
 // factors (33 KB a chunk of 128 columns; the scan reads q, k, v itself and forms U on its tensor cores), and W^T, P, T beta~
-// leave through shared memory as whole tiles: five CTAs per SM, 124 us before, 83 now for 4096 chunks of 128 columns.
+// leave through shared memory as whole tiles: five CTAs per SM, 124 us before, 79 then for 4096 chunks of 128 columns.  What
+// it does per chunk is a chain, so nothing sits on it that need not: the tiles are multiplied as they come (bf16; the
+// normalisation's factors go on the results), k becomes the fp16 operand of W while the other warps invert: 70 us.
 // kTrain: the forward of a training step also writes the fp16 copies of q and k and U, T, the cumulative decays.
 // ==========================================================================================
 constexpr int kPrepThreads = 160;
@@ -77,7 +98,7 @@ struct PrepMisc {
     uint64_t barLoad, barConv, barM, barXfree, barT, barUW;
     uint32_t tmem_base;
     int abort_flag, wait_kcycles;   // in this order: the waits read the limit as abort_flag[1]
-    alignas(16) float G[64], bt[64], btg[64], wsum[2];   // cumulative log decay, beta~, beta~ gamma (read in pairs)
+    alignas(16) float G[64], bt[64], btg[64], rn[128], wsum[2];   // cumulative log decay, beta~, beta~ gamma (read in pairs)
 };
 static_assert(sizeof(PrepMisc) <= kPrepMisc, "misc page too small");
 
@@ -154,7 +175,8 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                 if (kTrain) tma_load_4d(sV + kb * 8192, &map_v, &ms.barLoad, kb * 64, h, tok0, b);
             }
         }
-        bool ok = wait_all(&ms.barConv, 0, abort_flag);       // tiles converted to fp16
+        // kTrain: the tiles as fp16; otherwise as they come (bf16, exactly; the normalisation's factors go on the results)
+        bool ok = wait_all(kTrain ? &ms.barConv : &ms.barLoad, 0, abort_flag);
         if (ok) {
             // ---- fp16 copies of q and k for the backward; [Q ; K] K^T ----
             if (kTrain && leader) {
@@ -165,7 +187,7 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                 tma_store_commit();
             }
             tc_fence_after_sync();
-            constexpr uint32_t idesc = make_idesc(kFmtF16, 128, 64, false, false);
+            constexpr uint32_t idesc = make_idesc(kTrain ? kFmtF16 : kFmtBF16, 128, 64, false, false);
             if (elect_one()) {
 #pragma unroll
                 for (int kb = 0; kb < KB; ++kb)
@@ -175,9 +197,11 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                                desc_kmajor(aQK + kb * 16384 + 8192 + k16 * 32), idesc, (kb | k16) != 0);
                 mma_commit(&ms.barM);
             }
-            if (kTrain && leader) tma_store_wait_read();      // the q copy has left its blocks
-            ok = wait_all(&ms.barM, 0, abort_flag);           // and the MMAs have read them
-            if (leader) mbar_arrive(&ms.barXfree);
+            if (kTrain) {
+                if (leader) tma_store_wait_read();            // the q copy has left its blocks
+                ok = wait_all(&ms.barM, 0, abort_flag);       // and the MMAs have read them
+                if (leader) mbar_arrive(&ms.barXfree);
+            }
         }
         if (ok) ok = wait_all(&ms.barT, 0, abort_flag);
         if (ok) {
@@ -229,8 +253,24 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
             ms.bt[i] = btv;
             ms.btg[i] = btv * exp_ftz(G);
         }
-        // ---- tiles to fp16, in place ----
         bool ok = mbar_wait(&ms.barLoad, 0, abort_flag);
+        if (!kTrain) {
+            // Factors of q's and k's rows (1 without the normalisation), while the products of the tiles run.
+            float rn = 1.f;
+            if (ok && norm_eps >= 0.f) {
+                const uint8_t *rowp = sQK + (solver ? 8192 : 0) + i * 128;
+                float ss = 0.f;
+#pragma unroll
+                for (int kb = 0; kb < KB; ++kb)
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) ss = square_sum8(*reinterpret_cast<const uint4 *>(rowp + kb * 16384 + ((c ^ (i & 7)) << 4)), ss);
+                rn = rsqrtf(ss + norm_eps);
+                Rn[chunk * 128 + r] = rn;                      // (the scan scales the rows likewise)
+            }
+            ms.rn[r] = rn;
+            named_barrier_sync(3, kRowThreads);
+        } else
+        // ---- training step: tiles to fp16, in place ----
         if (ok && norm_eps >= 0.f) {
             // L2-normalised q and k for the linear operation (Section 4.3): thread r owns row r of
             // [Q ; K] (all KB blocks of it), takes its 16-byte pieces in an order that spreads the warp
@@ -246,13 +286,7 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
             for (int kb = 0; kb < KB; ++kb)
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
-                    const uint4 a = *reinterpret_cast<const uint4 *>(rowp + kb * 16384 + ((c ^ (i & 7)) << 4));
-                    const uint32_t wd[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float lo = __uint_as_float(wd[e] << 16), hi = __uint_as_float(wd[e] & 0xffff0000u);
-                        ss = fmaf(lo, lo, fmaf(hi, hi, ss));
-                    }
+                    ss = square_sum8(*reinterpret_cast<const uint4 *>(rowp + kb * 16384 + ((c ^ (i & 7)) << 4)), ss);
                 }
             const float rn = rsqrtf(ss + norm_eps);
             Rn[chunk * 128 + r] = rn;                          // (q's rows, k's rows: the scan scales them likewise)
@@ -261,13 +295,7 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
                     uint4 *pp = reinterpret_cast<uint4 *>(rowp + kb * 16384 + ((c ^ (i & 7)) << 4));
-                    const uint4 a = *pp;
-                    const uint32_t wd[4] = {a.x, a.y, a.z, a.w};
-                    uint32_t o[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        o[e] = pack_half2(__uint_as_float(wd[e] << 16) * rn, __uint_as_float(wd[e] & 0xffff0000u) * rn);
-                    *pp = make_uint4(o[0], o[1], o[2], o[3]);
+                    *pp = scale_f16x8(*pp, rn);
                 }
         } else if (ok) {
             for (int idx = r; idx < PL::kLoadBytes / 16; idx += kRowThreads) {
@@ -276,9 +304,11 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
             }
         }
         if (ok) {
-            fence_proxy_async_smem();
-            mbar_arrive(&ms.barConv);
-            ok = mbar_wait(&ms.barXfree, 0, abort_flag);
+            if (kTrain) {
+                fence_proxy_async_smem();
+                mbar_arrive(&ms.barConv);
+            }
+            ok = mbar_wait(kTrain ? &ms.barXfree : &ms.barM, 0, abort_flag);
         }
         if (ok) {
             tc_fence_after_sync();
@@ -290,6 +320,7 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                 gd[i] = exp_ftz(G);
                 gd[64 + i] = exp_ftz(ms.G[63] - G);
                 if (ex.Gcum) ex.Gcum[(size_t)bh * L + tok0 + i] = G;
+                const float fq = kTrain ? scale_la : scale_la * ms.rn[i];
                 uint4 *prow = reinterpret_cast<uint4 *>(Ph + (chunk * 64 + i) * 64);
 #pragma unroll 1
                 for (int pc = 0; pc < 8; ++pc) {
@@ -302,7 +333,8 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                         const int j = 8 * pc + e;
                         // the mask goes on the exponent (exp(-inf) = 0): a conditional around the whole
                         // expression compiles to one divergent branch per element
-                        x[e] = scale_la * exp_ftz(j <= i ? G - ms.G[j] : -INFINITY) * __uint_as_float(d8[e]);
+                        x[e] = fq * exp_ftz(j <= i ? G - ms.G[j] : -INFINITY) * __uint_as_float(d8[e]);
+                        if (!kTrain) x[e] *= ms.rn[64 + j];
                     }
                     const uint4 pw = make_uint4(pack_half2(x[0], x[1]), pack_half2(x[2], x[3]),
                                                 pack_half2(x[4], x[5]), pack_half2(x[6], x[7]));
@@ -310,7 +342,6 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                     else *reinterpret_cast<uint4 *>(sP + sw128_offset(i, pc)) = pw;
                 }
                 tc_fence_before_sync();
-                mbar_arrive(&ms.barT);
                 if (!kTrain) {
                     fence_proxy_async_smem();
                     named_barrier_sync(1, 64);
@@ -318,32 +349,44 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                         tma_store_2d(&map_ph, sP, 0, (int)chunk * 64);
                         tma_store_commit();
                     }
+                    // k as the fp16 operand of W, while the other two warps invert
+#pragma unroll
+                    for (int kb = 0; kb < KB; ++kb)
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
+                            const int row = (i >> 3) + 8 * e;
+                            uint4 *pp = reinterpret_cast<uint4 *>(sQK + kb * 16384 + 8192) + row * 8 + (i & 7);
+                            *pp = scale_f16x8(*pp, ms.rn[64 + row]);
+                        }
+                    fence_proxy_async_smem();
                 }
+                mbar_arrive(&ms.barT);
             } else {
                 // ---- T = (I + A)^-1 with 16x16 blocks (T_bb = (I + A_bb)^-1 in fp32 registers; below the
                 // diagonal T_10 = -T_11 A_10 T_00, T_32 likewise, then the 32x32 block
                 // T_[23][01] = -T_[23][23] A_[23][01] T_[01][01], all as warp-level fp16 MMAs) ----
-                uint32_t dd[2][32];
-                tmem_ld32(tmem + lane_base, dd[0]);
-                tmem_ld32(tmem + lane_base + 32, dd[1]);
-                tmem_wait_ld();
-                tc_fence_before_sync();
                 const int sw = warp - 2;                   // solver warp: block rows 2 sw and 2 sw + 1
                 const int bk = i >> 4, il = i & 15;        // this thread's block row, its row inside it
                 const int g8 = lane >> 2, t4 = lane & 3;   // fragment coordinates
-                const float btv = ms.bt[i];
+                const float btv = kTrain ? ms.bt[i] : ms.bt[i] * ms.rn[r];
                 const uint32_t aA = smem_u32(xLo), aT = smem_u32(xHi);
                 // A_ij = beta~_i Gamma_ij (k_i.k_j), j < i: blocks left of the diagonal as fp16 rows of
                 // the A tile (xLo), the row of the diagonal block in registers.
                 float ablk[16];
 #pragma unroll
                 for (int jb = 0; jb < 4; ++jb) {
+                    uint32_t dd[16];                       // 16 columns at a time: all 64 would not fit the registers
+                    if (jb <= 2 * sw + 1) {                // (warp-uniform)
+                        tmem_ld16(tmem + lane_base + 16 * jb, dd);
+                        tmem_wait_ld();
+                    }
                     if (jb <= bk) {
                         float a[16];
 #pragma unroll
                         for (int jj = 0; jj < 16; ++jj) {
                             const int j = 16 * jb + jj;
-                            a[jj] = btv * exp_ftz(j < i ? G - ms.G[j] : -INFINITY) * __uint_as_float(dd[j >> 5][j & 31]);
+                            a[jj] = btv * exp_ftz(j < i ? G - ms.G[j] : -INFINITY) * __uint_as_float(dd[jj]);
+                            if (!kTrain) a[jj] *= ms.rn[64 + j];
                         }
                         if (jb < bk) {
 #pragma unroll
@@ -357,6 +400,7 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                         }
                     }
                 }
+                tc_fence_before_sync();
                 // Row il of the diagonal block's inverse: t_j = [j = il] - sum_{m > j} t_m A_mj, from the
                 // right; A_mj sits in the registers of the thread that owns row m of the block.
                 float td[16];
@@ -739,19 +783,8 @@ gdn_scan_tc_kernel(const __grid_constant__ CUtensorMap map_wt,
 #pragma unroll 4
                 for (int i = 0; i < KB * 8192 / 16 / kScanConvThreads; ++i) {
                     const int idx = t + i * kScanConvThreads;
-                    uint4 a = pp[idx];
-                    if (rn) {
-                        const float f = rn[(idx >> 3) & 63];
-                        const uint32_t wd[4] = {a.x, a.y, a.z, a.w};
-                        uint32_t o[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            o[e] = pack_half2(__uint_as_float(wd[e] << 16) * f, __uint_as_float(wd[e] & 0xffff0000u) * f);
-                        a = make_uint4(o[0], o[1], o[2], o[3]);
-                    } else {
-                        a = bf16x8_to_f16x8(a);
-                    }
-                    pp[idx] = a;
+                    const uint4 a = pp[idx];
+                    pp[idx] = rn ? scale_f16x8(a, rn[(idx >> 3) & 63]) : bf16x8_to_f16x8(a);
                 }
             };
             for (int c = 0; c < ncs; ++c) {

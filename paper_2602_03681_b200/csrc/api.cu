@@ -79,11 +79,16 @@ bool use_tensor_cores(const natsl_params *p) {
     return p->dtype == NATSL_BF16 && !(p->flags & NATSL_FORCE_SIMT);
 }
 
-// Whether the scan is a programmatic dependent of the kernels before it too, which saves the gap of a launch: only when
-// the prepare kernel is a single wave (four CTAs on each of 148 multiprocessors).  Behind several waves the scan's
-// CTAs, one to a multiprocessor, would be placed in the order these drain, i.e. crowded into a few GPCs, whose share of
-// the L2 bandwidth the scans then fight for: 60 of them took 310-370 us there instead of 128 us.
-bool scan_follows_closely(const natsl_params *p) { return (long long)p->B * p->H * (p->L / kC) <= 4 * 148; }
+// Whether the scan is a programmatic dependent of the kernels before it too, which saves the gap of a launch.  Its CTAs, one
+// to a multiprocessor, are then placed in the order in which the prepare kernel's drain, i.e. crowded into a few GPCs,
+// whose share of the L2 bandwidth the scans fight for (60 of them behind several waves: 310-370 us instead of 128).  So:
+// one CTA per pair only while most multiprocessors have no second prepare CTA; several segments, which take every
+// multiprocessor anyway, behind up to about one wave.  Without -> with, us a call: one CTA per pair, 128 chunks 34.5 -> 33.0,
+// 160 38.5 -> 36.3, 224 34.8 -> 34.4, 240 47.2 -> 48.2, 450 47.7 -> 55.1, 512 51.2 -> 63.0; segments, 256 chunks 53.1 -> 49.8,
+// 512 67.7 -> 69.1, 576 88.9 -> 85.9, 640 123.6 -> 117.6, 1024 108.9 -> 113.3 and 129.9 -> 137.1.
+bool scan_follows_closely(const natsl_params *p, bool segmented) {
+    return (long long)p->B * p->H * (p->L / kC) <= (segmented ? 4 * 148 : 160);
+}
 
 // Segments of the forward scan (tensor-core path).  A (batch, head) costs one CTA per SM for as long as its chain of
 // chunks, so with few of them most of the GPU waits.  Up to 32 pairs a first pass over the segments (1.6 us per chunk
@@ -336,7 +341,7 @@ static int bwd_forward_part(const void *q, const void *k, const void *v, const f
                                          p->L, f.emit_flags, s, st, pdl, hg));
         NATSL_TRY(launch_gdn_scan_tc(q, k, v, f.tc, p->scale_la, p->state_in, state_out, ScanOut{f.o_la16, f.o_la, flags},
                                      f.ex, ScanSegments{0, 1, 0, nullptr, nullptr, nullptr}, block_route,
-                                     f.status, s, st, pdl && scan_follows_closely(p), hg.norm_eps >= 0.f));
+                                     f.status, s, st, pdl && scan_follows_closely(p, false), hg.norm_eps >= 0.f));
         NATSL_TRY(launch_softmax_combine_tc(q, f.k_smb, f.v16, p->L, p->L, f.sm_idx, f.prefix, f.o_la16,
                                             flags, p->w, p->scale_sm, p->eps, out, f.o_nla, f.lse, nullptr, p->L,
                                             BlockRouting{block_route, k, v}, false, f.status, s, st, hg));
@@ -509,7 +514,7 @@ int natsl_hybrid_fwd(const void *q, const void *k, const void *v, const float *g
         const bool beside = !p->stage_events && !(p->flags & NATSL_SINGLE_STREAM);
         int seg_chunks = 0;
         const int nseg = scan_segments(p, &seg_chunks);
-        const bool pdl = beside && scan_follows_closely(p);
+        const bool pdl = beside && scan_follows_closely(p, nseg > 1);
         auto prepare = [&]() {   // block-level routing: every token takes part in the delta rule of its own block
             return launch_gdn_prepare_tc(q, k, v, g, beta, block ? nullptr : route, p->scale_la, f.tc, GdnTcExport{},
                                          f.status, s, st, (int)(kStatusBytes / 4), hg.norm_eps, beside);
@@ -573,7 +578,7 @@ int natsl_hybrid_fwd(const void *q, const void *k, const void *v, const float *g
     if (beside) NATSL_TRY(gather());
     NATSL_TRY(mark());
     NATSL_TRY(launch_gdn_scan_simt(q_la, k_la, g, f.W, f.U, f.P, p->scale_la, p->state_in,
-                                   p->state_out, nullptr, nullptr, o_la, br.route, s, st, scan_follows_closely(p)));
+                                   p->state_out, nullptr, nullptr, o_la, br.route, s, st, scan_follows_closely(p, true)));
     NATSL_TRY(mark());
     // (an own-block tile of block-level routing reads the layer's keys: the softmax operation's copy)
     NATSL_TRY(launch_softmax_combine_simt(q_sm, k_soft, v_soft, cap_soft, f.sm_idx, f.prefix, o_la, p->w,

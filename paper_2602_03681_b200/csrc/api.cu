@@ -91,23 +91,27 @@ bool scan_follows_closely(const natsl_params *p, bool segmented) {
 }
 
 // Segments of the forward scan (tensor-core path).  A (batch, head) costs one CTA per SM for as long as its chain of
-// chunks, so with few of them most of the GPU waits.  Up to 32 pairs a first pass over the segments (1.6 us per chunk
-// against 2.1 with outputs) gains more than it costs: there are as many segments as keep its 2 nseg - 3 runs per pair
+// chunks, so with few of them most of the GPU waits.  Up to a number of pairs a first pass over the segments (1.6 us per chunk
+// against 1.8 with outputs) gains more than it costs: there are as many segments as keep its 2 nseg - 3 runs per pair
 // in one wave, at least 4 chunks long (shorter ones gain less than their step of the chain), and at least three --
-// with two the two passes are as long as one over everything.  32 pairs: 3 segments, 16: 6, 4: 20.
-// Where 32 comes from: three segments would fit one wave up to 49 pairs, but the softmax kernel, which runs beside the pass
-// with outputs, then starts a pass later.  Time of one pass over everything against segments, 2048 to 16384 tokens: 16 pairs of 128 columns
-// 1.19 to 1.48 with 5 % softmax tokens and 1.08 to 1.17 with 20 %, 24 pairs 1.01 to 1.17 and 0.89 to 0.99, 32 pairs 0.95 to
-// 1.06 and 0.85 to 0.94, 36 pairs (10 %) 0.90 to 0.92, 48 pairs 0.80 to 0.86; 64 columns 32 pairs 1.04 to 1.09 and 0.91 to
-// 1.02, 36 pairs (10 %) 0.92 to 1.02, 48 pairs 0.86 to 0.90.  The share of softmax tokens is not known here: the line is
-// the last count at which segments still win for few of them.
+// with two the two passes are as long as one over everything.  22 pairs: 4 segments, 16: 6, 4: 20.
+// Where the line lies: three segments would fit one wave up to 49 pairs, but the softmax kernel, which runs beside the pass
+// with outputs, then starts a pass later, and the more it has to do the fewer pairs pay for that.  Time with segments
+// against one pass over everything, 2048 to 16384 tokens, 5 to 40 % softmax tokens: 128 columns 16 pairs 0.82 to 0.92, 18 pairs
+// 0.72 to 0.99, 22 pairs 0.85 to 1.07, 24 pairs 1.02 and 1.03, 32 pairs 1.12 to 1.15; 64 columns 24 pairs 0.86, 28 pairs 0.91 to
+// 1.06, 32 pairs 1.01, 36 pairs 1.08.  With own-block tiles 64 columns 16 pairs 0.93, 22 pairs 1.04; with two softmax heads as
+// well 10 pairs 0.75 to 0.99, 14 pairs 0.91 to 1.06, 16 pairs 1.06, 24 pairs 1.19.
+int segment_pairs(const natsl_params *p) {
+    const bool heavy = (p->flags & NATSL_BLOCK_ROUTING) || p->G > 1;
+    return p->d == 64 ? (heavy ? 18 : 30) : heavy ? 14 : 22;
+}
 // The two passes must save 8 chunks of the chain, which is what two more launches and the chaining take.
 // The last segment takes what remains, up to twice as much: the first pass does not run it, and in the second the
 // softmax kernel fills the other multiprocessors.  *chunks: of the others, even, so that they are whole query tiles.
 int scan_segments(const natsl_params *p, int *chunks = nullptr) {
     if (!use_tensor_cores(p) || (p->flags & NATSL_SINGLE_PASS_SCAN)) return 1;
     const int NC = p->L / kC, BH = p->B * p->H;
-    if (BH > 32 || NC < 16) return 1;
+    if (BH > segment_pairs(p) || NC < 16) return 1;
     const int most = std::min((148 / BH + 3) / 2, 32);
     const int n = std::max(4, ((NC + most) / (most + 1) + 1) & ~1);
     if (chunks) *chunks = n;

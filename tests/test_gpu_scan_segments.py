@@ -24,3 +24,21 @@ def test_segments(name, H, L, oracle):
         assert rel_err(seg[n], one[n]) <= TOL["bf16"], n
     if oracle:
         check_fwd(wl, seg, run_oracle(wl, x, state_in=S0), TOL["bf16"])
+
+
+# the last number of pairs that is cut into segments and the first that is not, 128 and 64 columns, the latter with block-level
+# routing too
+@pytest.mark.parametrize("name,H,block", [("cfg1_bf16_prefill", 22, False), ("cfg1_bf16_prefill", 23, False),
+                                          ("cfg4_bf16_train", 30, False), ("cfg4_bf16_train", 31, False),
+                                          ("cfg4_bf16_train", 18, True), ("cfg4_bf16_train", 19, True)])
+def test_segments_at_the_lines(name, H, block):
+    wl = inputs.WORKLOADS[name]
+    L = 1536
+    x = inputs.make_layer_inputs(wl, B=1, H=H, L=L)
+    if block:
+        x["route"] = np.repeat((np.random.default_rng(3).random((1, L // 64, H)) < 0.3).astype(np.uint8), 64, axis=1)
+    x["g"] = np.full((1, L, H), -1e-3, np.float32)
+    flags = binding.BLOCK_ROUTING if block else 0
+    seg, one = run_fwd(wl, x, flags=flags), run_fwd(wl, x, flags=flags | binding.SINGLE_PASS_SCAN)
+    for n in ("o_la", "state_out"):
+        assert rel_err(seg[n], one[n]) <= TOL["bf16"], n

@@ -7,9 +7,9 @@
 // are exact bf16 inputs), online softmax in registers (one thread per query row), probabilities
 // written as fp16 into the TMEM columns their logits came from and P V as an fp16 MMA with A in
 // TMEM (V is gathered as fp16: the bf16 inputs convert exactly, and an 11-bit probability keeps the
-// branch output within ~2e-3 of its RMS where an 8-bit one would not).  The logits are
-// double-buffered in TMEM, so the probabilities of tile t + 1 never wait for the product of tile
-// t; with P in a single shared-memory tile every tile paid that product's latency.  K and V
+// branch output within ~2e-3 of its RMS where an 8-bit one would not).  At 128 columns the logits are
+// double-buffered in TMEM, so that the probabilities of tile t + 1 never wait for the product of tile
+// t; at 64 a CTA has one logit tile and the SM a third CTA (see SmLayout).  K and V
 // tiles arrive by TMA into two-stage rings.
 // Epilogue: o_la arrives as the scan leaves it, fp16 and transposed per chunk (o_laT, one 16 KB tile
 // per chunk: [8 pieces][d][8 tokens], row r of piece p at slot r ^ p); the CTA's two tiles come in
@@ -27,7 +27,7 @@
 // logits, 1100 a tile and, before its epilogue read o_laT and the accumulator in the matrix layout (ldmatrix, stmatrix,
 // 16x256b), 8 thousand behind the last; now 4500.  88 us before, 75 now for 4 x 4096 tokens and 16 heads by itself, 343 and 298
 // for one sequence of 32768.  With 64-column heads in the paper's mode an own-block tile takes twice as long as a retained one
-// (its keys are normalised and its values converted first), and waiting for instructions is a quarter of the stalls.
+// (its keys are normalised and its values converted first), and waiting for instructions is a seventh of the stalls.
 // Block-level routing (template flag): after the retained tiles, one more tile per linear block of
 // the CTA's two, holding that block's own 64 tokens (Section 4.1, inner-chunk correlations).
 // Grouped softmax heads (template count kG; Section 4.3, several softmax heads under one linear head's

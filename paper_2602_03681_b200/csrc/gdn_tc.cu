@@ -161,6 +161,11 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
     // once K K^T / Q K^T and the q copy are done with them (d = 128), or in their own region (d = 64).
     uint8_t *xLo = D == 128 ? sQK : smem + PL::oX;
     uint8_t *xHi = D == 128 ? sQK + 16384 : smem + PL::oX + 8192;
+    // A wait that runs out is recorded and the chain goes on, on whatever the tiles then hold: the row threads meet at
+    // barriers, and a limit runs out for each thread by itself.  Every product is issued all the same, so the end can wait
+    // for the last one.
+    auto wait = [&](uint64_t *bar) { (void)mbar_wait(bar, 0, abort_flag); };
+    auto wait_warp = [&](uint64_t *bar) { (void)wait_all(bar, 0, abort_flag); };
 
     if (warp == 4) {
         const bool leader = elect_one();
@@ -176,62 +181,58 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
             }
         }
         // kTrain: the tiles as fp16; otherwise as they come (bf16, exactly; the normalisation's factors go on the results)
-        bool ok = wait_all(kTrain ? &ms.barConv : &ms.barLoad, 0, abort_flag);
-        if (ok) {
-            // ---- fp16 copies of q and k for the backward; [Q ; K] K^T ----
-            if (kTrain && leader) {
-                for (int kb = 0; kb < KB; ++kb) {
-                    tma_store_2d(&map_qh, sQK + kb * 16384, kb * 64, bh * L + tok0);
-                    tma_store_2d(&map_kh, sQK + kb * 16384 + 8192, kb * 64, bh * L + tok0);
-                }
-                tma_store_commit();
+        wait_warp(kTrain ? &ms.barConv : &ms.barLoad);
+        // ---- fp16 copies of q and k for the backward; [Q ; K] K^T ----
+        if (kTrain && leader) {
+            for (int kb = 0; kb < KB; ++kb) {
+                tma_store_2d(&map_qh, sQK + kb * 16384, kb * 64, bh * L + tok0);
+                tma_store_2d(&map_kh, sQK + kb * 16384 + 8192, kb * 64, bh * L + tok0);
             }
-            tc_fence_after_sync();
+            tma_store_commit();
+        }
+        tc_fence_after_sync();
+        if (elect_one()) {
             constexpr uint32_t idesc = make_idesc(kTrain ? kFmtF16 : kFmtBF16, 128, 64, false, false);
-            if (elect_one()) {
 #pragma unroll
-                for (int kb = 0; kb < KB; ++kb)
+            for (int kb = 0; kb < KB; ++kb)
 #pragma unroll
-                    for (int k16 = 0; k16 < 4; ++k16)
-                        mma_ss(tm, desc_kmajor(aQK + kb * 16384 + k16 * 32),
-                               desc_kmajor(aQK + kb * 16384 + 8192 + k16 * 32), idesc, (kb | k16) != 0);
-                mma_commit(&ms.barM);
-            }
-            if (kTrain) {
-                if (leader) tma_store_wait_read();            // the q copy has left its blocks
-                ok = wait_all(&ms.barM, 0, abort_flag);       // and the MMAs have read them
-                if (leader) mbar_arrive(&ms.barXfree);
-            }
+                for (int k16 = 0; k16 < 4; ++k16)
+                    mma_ss(tm, desc_kmajor(aQK + kb * 16384 + k16 * 32),
+                           desc_kmajor(aQK + kb * 16384 + 8192 + k16 * 32), idesc, (kb | k16) != 0);
+            mma_commit(&ms.barM);
         }
-        if (ok) ok = wait_all(&ms.barT, 0, abort_flag);
-        if (ok) {
-            // ---- T beta~ leaves; U^T = V^T (T beta~)^T,  W^T = K^T (T beta~ gamma)^T ----
-            tc_fence_after_sync();
-            if (elect_one()) {
-                constexpr uint32_t idesc = make_idesc(kFmtF16, 128, 64, true, false);
-                if (D == 128 || !kTrain) {
+        if (kTrain) {
+            if (leader) tma_store_wait_read();            // the q copy has left its blocks
+            wait_warp(&ms.barM);                          // and the MMAs have read them
+            if (leader) mbar_arrive(&ms.barXfree);
+        }
+        wait_warp(&ms.barT);
+        // ---- T beta~ leaves; U^T = V^T (T beta~)^T,  W^T = K^T (T beta~ gamma)^T ----
+        tc_fence_after_sync();
+        if (elect_one()) {
+            constexpr uint32_t idesc = make_idesc(kFmtF16, 128, 64, true, false);
+            if (D == 128 || !kTrain) {
 #pragma unroll
-                    for (int k16 = 0; k16 < 4; ++k16) {
-                        if (kTrain) mma_ss(tm, desc_mnmajor(aV + k16 * 2048, 8192), desc_kmajor(aTb + k16 * 32), idesc, k16 != 0);
-                        // (d = 64: rows 64-127 of M are of no interest, K again)
-                        mma_ss(tWu, desc_mnmajor(aK + k16 * 2048, D == 128 ? 16384 : 0), desc_kmajor(aTg + k16 * 32), idesc, k16 != 0);
-                    }
-                } else {
-                    // d = 64: rows 0-63 of M are V^T, rows 64-127 are K^T (16 KB further on);
-                    // N = 128 = [T beta~ ; T beta~ gamma] (adjacent).
-                    constexpr uint32_t idesc2 = make_idesc(kFmtF16, 128, 128, true, false);
-#pragma unroll
-                    for (int k16 = 0; k16 < 4; ++k16)
-                        mma_ss(tm, desc_mnmajor(aV + k16 * 2048, 16384), desc_kmajor(aTb + k16 * 32), idesc2, k16 != 0);
+                for (int k16 = 0; k16 < 4; ++k16) {
+                    if (kTrain) mma_ss(tm, desc_mnmajor(aV + k16 * 2048, 8192), desc_kmajor(aTb + k16 * 32), idesc, k16 != 0);
+                    // (d = 64: rows 64-127 of M are of no interest, K again)
+                    mma_ss(tWu, desc_mnmajor(aK + k16 * 2048, D == 128 ? 16384 : 0), desc_kmajor(aTg + k16 * 32), idesc, k16 != 0);
                 }
-                mma_commit(&ms.barUW);
+            } else {
+                // d = 64: rows 0-63 of M are V^T, rows 64-127 are K^T (16 KB further on);
+                // N = 128 = [T beta~ ; T beta~ gamma] (adjacent).
+                constexpr uint32_t idesc2 = make_idesc(kFmtF16, 128, 128, true, false);
+#pragma unroll
+                for (int k16 = 0; k16 < 4; ++k16)
+                    mma_ss(tm, desc_mnmajor(aV + k16 * 2048, 16384), desc_kmajor(aTb + k16 * 32), idesc2, k16 != 0);
             }
-            if (leader) {
-                tma_store_2d(&map_tb, xLo, 0, (int)chunk * 64);
-                tma_store_commit();
-            }
+            mma_commit(&ms.barUW);
         }
-        if (leader) tma_store_wait_all();
+        if (leader) {
+            tma_store_2d(&map_tb, xLo, 0, (int)chunk * 64);
+            tma_store_commit();
+            tma_store_wait_all();
+        }
     } else {
         const int r = tid, i = r & 63;
         const bool solver = r >= 64;                       // rows 64-127: K K^T
@@ -253,11 +254,11 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
             ms.bt[i] = btv;
             ms.btg[i] = btv * exp_ftz(G);
         }
-        bool ok = mbar_wait(&ms.barLoad, 0, abort_flag);
+        wait(&ms.barLoad);
         if (!kTrain) {
             // Factors of q's and k's rows (1 without the normalisation), while the products of the tiles run.
             float rn = 1.f;
-            if (ok && norm_eps >= 0.f) {
+            if (norm_eps >= 0.f) {
                 const uint8_t *rowp = sQK + (solver ? 8192 : 0) + i * 128;
                 float ss = 0.f;
 #pragma unroll
@@ -271,7 +272,7 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
             named_barrier_sync(3, kRowThreads);
         } else
         // ---- training step: tiles to fp16, in place ----
-        if (ok && norm_eps >= 0.f) {
+        if (norm_eps >= 0.f) {
             // L2-normalised q and k for the linear operation (Section 4.3): thread r owns row r of
             // [Q ; K] (all KB blocks of it), takes its 16-byte pieces in an order that spreads the warp
             // over the banks, and scales while it converts.  V is converted as below.
@@ -297,20 +298,18 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                     uint4 *pp = reinterpret_cast<uint4 *>(rowp + kb * 16384 + ((c ^ (i & 7)) << 4));
                     *pp = scale_f16x8(*pp, rn);
                 }
-        } else if (ok) {
+        } else {
             for (int idx = r; idx < PL::kLoadBytes / 16; idx += kRowThreads) {
                 uint4 *pp = reinterpret_cast<uint4 *>(smem) + idx;   // V and [Q ; K] are contiguous
                 *pp = bf16x8_to_f16x8(*pp);
             }
         }
-        if (ok) {
-            if (kTrain) {
-                fence_proxy_async_smem();
-                mbar_arrive(&ms.barConv);
-            }
-            ok = mbar_wait(kTrain ? &ms.barXfree : &ms.barM, 0, abort_flag);
+        if (kTrain) {
+            fence_proxy_async_smem();
+            mbar_arrive(&ms.barConv);
         }
-        if (ok) {
+        wait(kTrain ? &ms.barXfree : &ms.barM);
+        {   // ---- warps 0-1: P; warps 2-3: T ----
             tc_fence_after_sync();
             const float G = ms.G[i];
             if (!solver) {
@@ -532,10 +531,9 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                 fence_proxy_async_smem();
                 mbar_arrive(&ms.barT);
             }
-            ok = mbar_wait(&ms.barUW, 0, abort_flag);
+            wait(&ms.barUW);
         }
-        if (ok) {
-            // ---- (U^T and) W^T as fp16 tiles, over V and K; thread r <-> head-dimension row ----
+        {   // ---- (U^T and) W^T as fp16 tiles, over V and K; thread r <-> head-dimension row ----
             tc_fence_after_sync();
             auto stage = [&](uint32_t from, uint8_t *tile, int row) {
                 uint32_t x[2][32];
@@ -566,19 +564,21 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
         }
         named_barrier_sync(3, kRowThreads);
         if (tid == 0) {
-            if (ok) {
-                for (int kb = 0; kb < KB; ++kb) {
-                    if (kTrain) tma_store_2d(&map_u16, sV + kb * 8192, 0, (int)(chunk * D) + kb * 64);
-                    tma_store_2d(&map_wt, sQK + 8192 + kb * 16384, 0, (int)(chunk * D) + kb * 64);
-                }
-                tma_store_commit();
+            for (int kb = 0; kb < KB; ++kb) {
+                if (kTrain) tma_store_2d(&map_u16, sV + kb * 8192, 0, (int)(chunk * D) + kb * 64);
+                tma_store_2d(&map_wt, sQK + 8192 + kb * 16384, 0, (int)(chunk * D) + kb * 64);
             }
+            tma_store_commit();
             tma_store_wait_all();
         }
     }
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 4) {
+        if (*abort_flag) {          // no copy, no product in flight when the CTA gives its memories back
+            mbar_wait_drain(&ms.barLoad, 0);
+            mbar_wait_drain(&ms.barUW, 0);
+        }
         tc_fence_after_sync();
         tmem_dealloc(tmem, PL::kTmemCols);
     }

@@ -169,8 +169,8 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
     if (warp == kTmaWarp && lane == 0) {
         mbar_init(&ms.barQ, 1);
         mbar_init(&ms.barQn, kSoftmaxThreads);       // normalised queries written (NATSL_QK_NORM)
-        mbar_init(&ms.barKn[0], 1);                  // ... and the keys of an own-block tile: one barrier per tile,
-        mbar_init(&ms.barKn[1], 1);                  //     each completing once
+        mbar_init(&ms.barKn[0], kSoftmaxThreads);    // ... and the keys of an own-block tile: one barrier per tile,
+        mbar_init(&ms.barKn[1], kSoftmaxThreads);    //     each completing once
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&ms.fullK[s], 1); mbar_init(&ms.emptyK[s], 1);
             mbar_init(&ms.fullV[s], 1); mbar_init(&ms.emptyV[s], 1);
@@ -399,23 +399,20 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
         for (int t = 0; ok && t < T2; ++t) {
             if (kBlock && kNorm && t >= T) {
                 // Keys of an own-block tile (block-level routing with normalisation): raw bf16 rows from the
-                // layer's k; two threads per row rewrite it as fp16 of the RMS-normalised row.  One arrival per
-                // tile, after all rows are written.
+                // layer's k; two threads per row rewrite it as fp16 of the RMS-normalised row.  (Every thread arrives for
+                // itself: threads whose wait ran out leave the loop, so none may wait here for the others.)
                 ok = mbar_wait(&ms.fullK[t % kStages], (t / kStages) & 1, abort_flag);
-                uint8_t *rowp = smem + SL::oK + (t % kStages) * SL::kKStage + (r >> 1) * 128;
-                if (ok) {
-                    float ss = 0.f;
-#pragma unroll
-                    for (int kb = 0; kb < KB; ++kb) ss += row_square_sum<4>(rowp + kb * kBN * 128, 4 * (r & 1), (r >> 1) & 7);
-                    ss += __shfl_xor_sync(0xffffffffu, ss, 1);
-                    const float rk = rsqrtf(ss / D + norm_eps);
-#pragma unroll
-                    for (int kb = 0; kb < KB; ++kb) row_to_fp16<4>(rowp + kb * kBN * 128, 4 * (r & 1), (r >> 1) & 7, rk);
-                }
-                fence_proxy_async_smem();
-                named_barrier_sync(1, kSoftmaxThreads);
-                if (r == 0 && ok) mbar_arrive(&ms.barKn[t - T]);
                 if (!ok) break;
+                uint8_t *rowp = smem + SL::oK + (t % kStages) * SL::kKStage + (r >> 1) * 128;
+                float ss = 0.f;
+#pragma unroll
+                for (int kb = 0; kb < KB; ++kb) ss += row_square_sum<4>(rowp + kb * kBN * 128, 4 * (r & 1), (r >> 1) & 7);
+                ss += __shfl_xor_sync(0xffffffffu, ss, 1);
+                const float rk = rsqrtf(ss / D + norm_eps);
+#pragma unroll
+                for (int kb = 0; kb < KB; ++kb) row_to_fp16<4>(rowp + kb * kBN * 128, 4 * (r & 1), (r >> 1) & 7, rk);
+                fence_proxy_async_smem();
+                mbar_arrive(&ms.barKn[t - T]);
             }
             ok = mbar_wait(&ms.barS[t % kLogits], (t / kLogits) & 1, abort_flag);
             if (!ok) break;

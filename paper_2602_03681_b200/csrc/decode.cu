@@ -198,6 +198,7 @@ decode_step_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__
         s_abort[1] = 0;
         fence_mbar_init();
     }
+    if (kVaried && tid < kMaxItems / 32) s_empty[tid] = 0u;
     __syncthreads();
     volatile int *abort_flag = s_abort;
     grid_dependency_wait();
@@ -488,7 +489,8 @@ decode_step_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__
 #pragma unroll 1
     for (int i = 0, ord = 0; has(ord); ++i, ++ord) {
         if (kVaried && ord) {
-            if (ord == 1 && !mbar_wait(&looked, 0, abort_flag)) break;
+            // (after a time-out: go on, for the warps meet at the state items' barriers; what is not looked up gets a turn)
+            if (ord == 1) (void)mbar_wait(&looked, 0, abort_flag);
             if (__any_sync(0xffffffffu, empty_item(ord))) { --i; continue; }
         }
         int part, bh;

@@ -4,12 +4,14 @@ guard against cannot be provoked on a GPU without hanging it.
 A device-side wait on an mbarrier or a counter is bounded, and the bound runs out for each thread by itself: of two threads
 at the same wait one may give up while the other finds it complete.  A barrier of many threads has no bound.  So whether a
 thread arrives at one must not depend on how a bounded wait ended."""
+import glob
 import os
 import re
 
 import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(__file__)), "paper_2602_03681_b200", "csrc")
+SOURCES = sorted(os.path.basename(p) for p in glob.glob(os.path.join(CSRC, "*.cu")))
 BARRIER = re.compile(r"\b(named_barrier_sync|__syncthreads\w*)\s*\(")
 WAIT = r"\b(?:mbar_wait|wait_all|wait_counter_ge)\s*\("
 
@@ -82,7 +84,7 @@ def barriers_behind_a_wait(body):
     return missed
 
 
-@pytest.mark.parametrize("source", ["gdn_tc.cu", "softmax_tc.cu"])
+@pytest.mark.parametrize("source", SOURCES)
 def test_no_barrier_stands_behind_one_threads_wait(source):
     for name, body in kernels(os.path.join(CSRC, source)):
         assert not barriers_behind_a_wait(body), name

@@ -146,14 +146,15 @@ gdn_prepare_tc_kernel(const __grid_constant__ CUtensorMap map_q,
     if (warp == 4) tmem_alloc(&ms.tmem_base, PL::kTmemCols);
     // (what is set up above needs nothing of the kernel ahead, whose last CTAs may still run)
     grid_dependency_wait();
-    // The forward's first kernel: clears the status page.  The compaction behind it needs nothing of this kernel and
-    // may start as soon as the last CTAs have (it fills the multiprocessors as they drain); the scan waits for both.
+    // The forward's first kernel: clears the status page.
     if (blockIdx.x == 0 && tid < head_words) status[tid] = 0;
     __threadfence();
-    launch_dependents();
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
+    // The compaction behind this kernel needs nothing of it and may start as soon as the last CTAs have (it fills the
+    // multiprocessors as they drain); the scan waits for both.
+    launch_dependents();
     const uint32_t tmem = ms.tmem_base, tW = tmem + (kTrain ? 64 : 0);
     volatile int *abort_flag = &ms.abort_flag;
     uint8_t *sV = smem + PL::oV, *sQK = smem + PL::oQK, *sP = smem + PL::oP;

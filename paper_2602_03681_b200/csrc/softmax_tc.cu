@@ -158,11 +158,14 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
         if (tid == 0 && blockIdx.x == 0 && blockIdx.y == gridDim.y - 1) grid_dependency_wait();
     };
 
-    launch_dependents();
     if ((smem_u32(smem) & 1023u) != 0) {              // operand tiles need 1024-byte alignment
         if (tid == 0) atomicMin(status, (int)NATSL_ERR_CUDA);
         end_behind_scan();
         return;
+    }
+    if (warp == kMmaWarp) {
+        tmem_alloc(&ms.tmem_base, SL::kTmemCols);
+        launch_dependents();                          // (behind the allocation: see there)
     }
     // The TMA warp sets the barriers up and requests the Q tile before anything else, and goes on to the key tiles as soon
     // as it knows how many there are: it needs nothing of what the other warps set up.
@@ -226,7 +229,6 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
         }
     }
     if (tid < kBM / 32) ms.kept[tid] = 0u;
-    if (warp == kMmaWarp) tmem_alloc(&ms.tmem_base, SL::kTmemCols);
     tc_fence_before_sync();
     if (warp != kTmaWarp) named_barrier_sync(4, kThreadsS);
     tc_fence_after_sync();

@@ -90,6 +90,10 @@ __device__ __forceinline__ bool mbar_wait_drain(uint64_t *bar, uint32_t parity) 
 // Programmatic dependent launch: a kernel launched behind this one with the programmatic
 // stream-serialisation attribute may be scheduled once every CTA of this grid has executed this
 // (or exited).  Without such a dependent it does nothing.
+// A kernel that allocates tensor memory executes this behind its allocation.  An allocation waits for columns without a
+// limit, and a dependent holds its own while it waits for this kernel: were it there before a CTA of this kernel has its
+// columns, each could wait for the other.  This way whoever holds columns waits only for kernels that have all of theirs,
+// whatever shares a multiprocessor, and registers and shared memory per CTA need not keep them apart.
 __device__ __forceinline__ void launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

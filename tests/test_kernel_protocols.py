@@ -90,7 +90,30 @@ def test_no_barrier_stands_behind_one_threads_wait(source):
         assert not barriers_behind_a_wait(body), name
 
 
-def test_the_rule_finds_what_it_is_for():
+def lets_dependents_in_too_early(body):
+    """Whether a kernel that allocates tensor memory may let a programmatic dependent start before every CTA has its
+    columns: the dependent may hold columns while it waits for this kernel, and an allocation waits without a limit."""
+    alloc, release = body.find("tmem_alloc("), body.find("launch_dependents()")
+    if alloc < 0 or release < 0:
+        return False
+    if re.search(r"\{\s*tmem_alloc\([^;]*;\s*launch_dependents\(\)", body):       # (the allocating warp itself)
+        return body.count("launch_dependents()") != 1
+    barrier = BARRIER.search(body, alloc)
+    return barrier is None or release < barrier.end()
+
+
+@pytest.mark.parametrize("source", SOURCES)
+def test_dependents_start_behind_the_allocation_of_tensor_memory(source):
+    for name, body in kernels(os.path.join(CSRC, source)):
+        assert not lets_dependents_in_too_early(body), name
+
+
+def test_the_rules_find_what_they_are_for():
+    assert lets_dependents_in_too_early("launch_dependents(); if (w) tmem_alloc(&b, 64); __syncthreads();")
+    assert lets_dependents_in_too_early("if (w) tmem_alloc(&b, 64); launch_dependents(); __syncthreads();")
+    assert lets_dependents_in_too_early("launch_dependents(); if (w) { tmem_alloc(&b, 64); launch_dependents(); }")
+    assert not lets_dependents_in_too_early("if (w) tmem_alloc(&b, 64); __syncthreads(); launch_dependents();")
+    assert not lets_dependents_in_too_early("if (w) { tmem_alloc(&b, 64); launch_dependents(); } __syncthreads();")
     ok = "bool ok = mbar_wait(&a, 0, f); "
     assert barriers_behind_a_wait(ok + "if (ok) { x(); if (y) { named_barrier_sync(1, 64); } }")
     assert barriers_behind_a_wait(ok + "if (ok) __syncthreads();")

@@ -63,6 +63,11 @@ __device__ __forceinline__ void fma4(ulonglong2 a, ulonglong2 b, uint64_t &acc) 
     acc = tc::fma2(a.y, b.y, acc);
 }
 __device__ __forceinline__ ulonglong2 lds4(const float *p) { return *reinterpret_cast<const ulonglong2 *>(p); }
+// the first `n` (any number) of four values, zeros behind them
+__device__ __forceinline__ ulonglong2 first_of(ulonglong2 a, int n) {
+    const float2 lo = tc::unpack2(a.x), hi = tc::unpack2(a.y);
+    return make_ulonglong2(tc::pack2(n > 0 ? lo.x : 0.f, n > 1 ? lo.y : 0.f), tc::pack2(n > 2 ? hi.x : 0.f, n > 3 ? hi.y : 0.f));
+}
 __device__ __forceinline__ float both(uint64_t a) { const float2 x = tc::unpack2(a); return x.x + x.y; }
 
 // Sums of N values over W neighbouring lanes; lane w of them keeps values w N / W .. (the upper halves of the exchange
@@ -262,7 +267,7 @@ template <int D, int NV> struct SimtScan {
     static constexpr int oS = 0, oW = oS + NV * LD, oQ = oW + kTwice * kC * LD, oK = oQ + kTwice * kC * LD,
                          oP = oK + 2 * kC * LK, oU = oP + 2 * kC * LP, oUs = oU + 2 * kC * NV, oUt = oUs + kC * NV,
                          oG = oUt + NV * LU;
-    static constexpr int kBytes = (oG + 5 * kC) * 4;
+    static constexpr int kBytes = (oG + 5 * kC + 1) * 4;
     static_assert(kBytes <= 227 * 1024, "shared memory of a CTA");
 };
 
@@ -286,6 +291,7 @@ gdn_scan_simt_kernel(const T *__restrict__ q, const T *__restrict__ k, const flo
     float *raw = smem + SS::oG;                          // [2][64] log decay
     float *Gs = raw + 2 * kC;                            // [64] cumulative
     float *e1 = Gs + kC, *e2 = e1 + kC;                  // [64] scale_la gamma_i; [64] gamma_C / gamma_i
+    volatile int *outside = reinterpret_cast<int *>(e2 + kC);        // whether U~ has an infinity or a NaN
 
     const int slice = blockIdx.x, bh = blockIdx.y, b = bh / H, h = bh % H, tid = threadIdx.x;
     const int NC = L / kC;
@@ -312,6 +318,7 @@ gdn_scan_simt_kernel(const T *__restrict__ q, const T *__restrict__ k, const flo
     };
     fetch_wq(0);
     fetch_rest(0);
+    if (tid == 0) *outside = 0;
     for (int idx = tid; idx < D * NV; idx += kThreads) {
         const int a = idx / NV, cc = idx % NV;
         Ss[cc * LD + a] = state_in ? state_in[((size_t)bh * D + a) * D + c0 + cc] : 0.f;
@@ -349,6 +356,7 @@ gdn_scan_simt_kernel(const T *__restrict__ q, const T *__restrict__ k, const flo
         }
         // U~ = U - W S, and q S while the state's columns pass by
         float qs[kRw * kCl];
+        bool finite = true;                               // this thread's U~
         {
             uint64_t acc[2][4][2];                        // [row][column][W S, q S]
 #pragma unroll
@@ -377,15 +385,19 @@ gdn_scan_simt_kernel(const T *__restrict__ q, const T *__restrict__ k, const flo
                 for (int x = 0; x < kCl; ++x) {
                     const int r = r0 + 32 * e, cc = cg + kCg * (cc0 + x);
                     const float u = Uin[r * NV + cc] - sum[2 * (kCl * e + x)];
+                    finite &= fabsf(u) < INFINITY;
                     qs[kCl * e + x] = sum[2 * (kCl * e + x) + 1];
                     Us[r * NV + cc] = u;
                     Uts[cc * LU + r] = u;
                     if (Ut) Ut[(tok0 + (size_t)r * H) * D + c0 + cc] = u;
                 }
         }
+        if (!finite) *outside = 1;                        // (once and for all: the state takes it along)
         __syncthreads();
+        const bool again = *outside;
         if (SS::kTwice == 1 && c + 1 < NC) fetch_wq(c + 1);
-        // O = scale_la gamma_r q_r S + sum_{j<=r} P_rj U~_j   (P is zero above the diagonal)
+        // O = scale_la gamma_r q_r S + sum_{j<=r} P_rj U~_j.  P is zero above the diagonal, but zero times an infinity or a
+        // NaN is not: where there is one among U~, the sums are formed again, of the tokens up to each row's own only.
         {
             uint64_t acc[2][4];
 #pragma unroll
@@ -400,6 +412,22 @@ gdn_scan_simt_kernel(const T *__restrict__ q, const T *__restrict__ k, const flo
                     const ulonglong2 uv = lds4(Uts + (cg + kCg * x) * LU + j);
                     if (j < 32) fma4(p0, uv, acc[0][x]);
                     fma4(p1, uv, acc[1][x]);
+                }
+            }
+            if (again) {
+#pragma unroll
+                for (int e = 0; e < 2; ++e)
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) acc[e][x] = 0ull;
+#pragma unroll 1
+                for (int j = 4 * w1; j < kC; j += 4 * kW1) {
+                    const ulonglong2 p1 = lds4(Ps + (rp + 32) * LP + j), p0 = lds4(Ps + rp * LP + j);
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) {
+                        const ulonglong2 uv = lds4(Uts + (cg + kCg * x) * LU + j);
+                        if (j < 32) fma4(p0, first_of(uv, rp + 1 - j), acc[0][x]);
+                        fma4(p1, first_of(uv, rp + 33 - j), acc[1][x]);
+                    }
                 }
             }
             float sum[8];

@@ -99,8 +99,13 @@ bool scan_follows_closely(const natsl_params *p, bool segmented) {
 // with outputs, then starts a pass later, and the more it has to do the fewer pairs pay for that.  Time with segments
 // against one pass over everything, 2048 to 16384 tokens, 5 to 40 % softmax tokens: 128 columns 16 pairs 0.82 to 0.92, 18 pairs
 // 0.72 to 0.99, 22 pairs 0.85 to 1.07, 24 pairs 1.02 and 1.03, 32 pairs 1.12 to 1.15; 64 columns 24 pairs 0.86, 28 pairs 0.91 to
-// 1.06, 32 pairs 1.01, 36 pairs 1.08.  With own-block tiles 64 columns 16 pairs 0.93, 22 pairs 1.04; with two softmax heads as
-// well 10 pairs 0.75 to 0.99, 14 pairs 0.91 to 1.06, 16 pairs 1.06, 24 pairs 1.19.
+// 1.06, 32 pairs 1.01, 36 pairs 1.08.  With own-block tiles 64 columns 16 pairs 0.93, 22 pairs 1.04.  128 columns, in the
+// order (2048 tokens, 20 % softmax tokens), (8192, 5 %), (8192, 30 %), (16384, 10 %): own-block tiles 16 pairs 0.99, 0.75, 0.98,
+// 0.81, 18 pairs 0.99, 0.79, 1.00, 0.90, 20 pairs 1.14, 0.88, 1.08, 0.97, 22 pairs 1.10, 0.96, 1.10, 1.04; two softmax heads,
+// token routing 12 pairs 0.97, 0.65, 1.01, 0.78, 14 pairs 0.96, 0.70, 1.06, 0.86, 16 pairs 1.00, 0.75, 1.08, 0.92, 18 pairs 1.08,
+// 0.79, 1.06, 0.98 (normalised q, k: 0.02 to 0.06 less); both 10 pairs 0.75 to 0.99, 14 pairs 0.91 to 1.06, 16 pairs 1.06.
+// Own-block tiles with one softmax head of 128 columns would pay up to 18 pairs; they keep 14 because segments need scratch,
+// and calls of 15 to 18 pairs of 1024 tokens that fit natsl_hybrid_fwd_static's array (23 to 27 of 32 MiB) would not any more.
 int segment_pairs(const natsl_params *p) {
     const bool heavy = (p->flags & NATSL_BLOCK_ROUTING) || p->G > 1;
     return p->d == 64 ? (heavy ? 18 : 30) : heavy ? 14 : 22;

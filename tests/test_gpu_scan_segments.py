@@ -26,11 +26,12 @@ def test_segments(name, H, L, oracle):
         check_fwd(wl, seg, run_oracle(wl, x, state_in=S0), TOL["bf16"])
 
 
-# the last number of pairs that is cut into segments and the first that is not, 128 and 64 columns, the latter with block-level
-# routing too
+# the last number of pairs that is cut into segments and the first that is not, 128 and 64 columns, with block-level routing
+# too
 @pytest.mark.parametrize("name,H,block", [("cfg1_bf16_prefill", 22, False), ("cfg1_bf16_prefill", 23, False),
                                           ("cfg4_bf16_train", 30, False), ("cfg4_bf16_train", 31, False),
-                                          ("cfg4_bf16_train", 18, True), ("cfg4_bf16_train", 19, True)])
+                                          ("cfg4_bf16_train", 18, True), ("cfg4_bf16_train", 19, True),
+                                          ("cfg1_bf16_prefill", 14, True), ("cfg1_bf16_prefill", 15, True)])
 def test_segments_at_the_lines(name, H, block):
     wl = inputs.WORKLOADS[name]
     L = 1536

@@ -155,3 +155,69 @@ def test_a_programmatic_dependent_waits_for_its_predecessor(dtype, B, H, L, d):
         assert "grid_dependency_wait()" in sources[own[0]], f"{own[0]} does not wait for the kernel before it"
         seen.add(own[0])
     assert seen >= ({"softmax_combine_tc_kernel", "route_gather_kernel"} if dtype == "bf16" else {"softmax_combine_simt_kernel"})
+
+
+@pytest.mark.parametrize("d,G,norm,block", [(128, 2, True, True), (128, 1, False, False), (64, 1, False, False)])
+def test_a_training_step_starts_behind_the_one_before(d, G, norm, block):
+    """Two training steps in one graph.  The second one's first kernel is a programmatic dependent of what the first one ends
+    with, where two streams have been joined: every kernel of the first step lies ahead of it, and the graph gives the bits
+    of the same steps launched one by one."""
+    from paper_2602_03681_b200 import binding
+    B, H, L = 1, 2, 512
+    gen = torch.Generator(device="cuda").manual_seed(3)
+
+    def rand(*s):
+        return torch.randn(s, generator=gen, device="cuda")
+
+    t = {n: (torch.nn.functional.normalize(rand(B, L, H, d), dim=-1) if n in "qk" else rand(B, L, H, d)).bfloat16()
+         for n in ("q", "k", "v", "dout")}
+    g, beta = -torch.nn.functional.softplus(rand(B, L, H)), torch.sigmoid(rand(B, L, H))
+    w = torch.softmax(rand(B, L, H, 2), -1).contiguous()
+    route = (torch.rand((B, L // 64 if block else L, H), generator=gen, device="cuda") < 0.3).to(torch.uint8)
+    if block:
+        route = route.repeat_interleave(64, dim=1).contiguous()
+    dscore = torch.zeros((B, L // 64, H, 2), device="cuda")
+    # out and the gradients of each step; the second works on other values
+    results = [[torch.zeros_like(x) for x in (t["q"], t["q"], t["k"], t["v"], g, beta, w)] for _ in range(2)]
+    values = [t["v"], t["v"].flip(1).contiguous()]
+    flags = (binding.BLOCK_ROUTING if block else 0) | (binding.QK_NORM if norm else 0)
+    pf, pb = (binding.make_params(B, H, L, d, binding.NATSL_BF16, d ** -0.5, 1.0, w=w, G=G, norm_eps=1e-6, flags=flags | f)
+              for f in (binding.SAVE_FOR_BWD, binding.SAVED_FWD))
+    if block:
+        pf.dscore = pb.dscore = dscore.data_ptr()
+    ws = binding.alloc_workspace(pf, binding.OP_BWD)
+
+    def step(i):
+        out, *grads = results[i]
+        binding.natsl_hybrid_fwd(t["q"], t["k"], values[i], g, beta, route, out, pf, ws)
+        binding.natsl_hybrid_bwd(t["q"], t["k"], values[i], g, beta, route, t["dout"], *grads, pb, ws)
+
+    for i in range(2):
+        step(i)
+        torch.cuda.synchronize()
+        assert binding.natsl_device_status(ws) == 0
+    expected = [[x.clone() for x in r] for r in results]
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        step(0)
+        step(1)
+    names, reach, early = kernels_and_paths(graph)
+    first, second = sorted((n for n, name in names.items() if "gdn_prepare" in name), key=lambda n: -len(reach[n]))
+    assert second in early
+    ahead = [n for n in names if second in reach[n]]
+    assert len(ahead) == len(names) // 2 and first in ahead
+    assert all(n == second or n in reach[second] for n in names if n not in ahead)
+    sources = kernel_sources()
+    for x in early:
+        own = [k for k in sources if f"{len(k)}{k}" in names[x]]
+        assert len(own) == 1 and "grid_dependency_wait()" in sources[own[0]], names[x]
+    for r in results:
+        for x in r:
+            x.zero_()
+    graph.instantiate()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert binding.natsl_device_status(ws) == 0
+    for got, want in zip(results, expected):
+        for x, y in zip(got, want):
+            assert torch.equal(x, y)

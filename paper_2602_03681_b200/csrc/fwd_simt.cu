@@ -844,10 +844,14 @@ cudaError_t set_smem(K kernel, size_t bytes) {
 }  // namespace
 
 
-// Chunks up to which the prepare kernel cuts a chunk into four, i.e. up to two CTAs per SM: with more the four-fold A takes
-// more than the finer split of the rest gains.  Whole call with four parts against one: 8 chunks of 64 columns 21.8 / 26.4
-// us, 70 chunks 44.7 / 48.9 (128 columns 87.7 / 91.5), 80 chunks 44.7 / 48.9 (98.6 / 92.6), 128 chunks 104 / 102 (158 / 146).
-constexpr int kFewChunks = 74;
+// Chunks up to which the prepare kernel cuts a chunk into four, by head size: with more the four-fold A takes more than the
+// finer split of the rest gains.  128 columns: as many as are resident at once (78 KB, two CTAs per SM: 296 CTAs).  64
+// columns (49 KB, four per SM): three CTAs per SM, the fourth only shares their issue slots.  Whole call with four parts
+// against one, us: 8 chunks of 64 columns 21.9 / 26.5, 70 39.4 / 43.4, 74 (pairs of two chunks) 36.9 / 35.5, 80 43.2 / 55.1, 84
+// 60.0 / 60.2, 96 47.9 / 51.9 and 55.8 / 69.4, 98 62.0 / 77.1, 112 58.7 / 58.0 and 56.0 / 54.3, 128 65.7 / 65.4, 160 73.3 /
+// 67.1, 192 99.5 / 85.0; of 128 columns 8 chunks 30.6 / 40.1, 70 94.4 / 97.8, 72 86.7 / 90.0, 74 50.8 / 54.5, 80 117.0 /
+// 111.0, 96 98.8 / 92.2, 128 133.6 / 121.6.
+template <int D> constexpr int kFewChunks = D == 64 ? 3 * 148 / 4 : 2 * 148 / 4;
 
 #define NATSL_DISPATCH(FN, ...)                                                   \
     do {                                                                          \
@@ -864,7 +868,7 @@ static cudaError_t prepare_impl(const void *q, const void *k, const void *v, con
                                 const float *beta, const uint8_t *route, float scale_la, float *W,
                                 float *U, float *P, float *Abar, float *Gcum, Shape s,
                                 cudaStream_t st, int32_t *clear, int clear_words) {
-    const bool few = s.L / kC * s.B * s.H <= kFewChunks;     // (see the kernel)
+    const bool few = s.L / kC * s.B * s.H <= kFewChunks<D>;     // (see the kernel)
     const size_t smem = few ? SimtPrep<D, 4>::kBytes : SimtPrep<D, 1>::kBytes;
     auto kernel = few ? gdn_prepare_simt_kernel<T, D, 4> : gdn_prepare_simt_kernel<T, D, 1>;
     cudaError_t e = set_smem(kernel, smem);

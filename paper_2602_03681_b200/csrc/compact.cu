@@ -5,6 +5,7 @@
 // route may be checked to be one decision per chunk (block-level routing).
 #include "common.cuh"
 #include "natsl_internal.h"
+#include "route_slice.cuh"
 #include "tc_common.cuh"
 
 namespace natsl {
@@ -149,74 +150,29 @@ gather_kv_kernel(const T *__restrict__ k, const T *__restrict__ v, const int32_t
     reinterpret_cast<uint4 *>(v_sm + dst)[piece] = reinterpret_cast<const uint4 *>(v + src)[piece];
 }
 
-// Both in one kernel, for the forward of the CUDA-core path: grid = (slices of the chunks, B*H).  A CTA counts the
-// retained tokens before its slice itself (route bytes out of L2), lists its own chunks' and copies their rows -- from one
-// or two pairs of sources and destinations: a cache that keeps the keys as given beside the normalised keys the
-// softmax kernel reads.  It needs nothing of the prepare kernel ahead of it and, as its programmatic dependent, runs beside
-// it; what it reports goes out behind that kernel, which clears the status page.  (One CTA per (batch, head) for the lists
-// and a second kernel for the rows, both ahead of the prepare kernel: 8 us of a small call.)
-constexpr int kRowsThreads = 256, kRowsSlice = 32;          // threads, chunks of a CTA (at most)
+// Both in one kernel, for the forward of the CUDA-core path: a CTA lists its slice's retained tokens (see route_slice.cuh)
+// and copies their rows -- from one or two pairs of sources and destinations: a cache that keeps the keys as given beside
+// the normalised keys the softmax kernel reads.  It needs nothing of the prepare kernel ahead of it and, as its programmatic
+// dependent, runs beside it; what it reports goes out behind that kernel, which clears the status page.  (One CTA per (batch,
+// head) for the lists and a second kernel for the rows, both ahead of the prepare kernel: 8 us of a small call.)
 template <typename T, int D>
-__global__ void __launch_bounds__(kRowsThreads)
+__global__ void __launch_bounds__(kRouteThreads)
 route_gather_rows_kernel(const uint8_t *__restrict__ route, const T *__restrict__ v, const RowsJob j0, const RowsJob j1,
                          int32_t *__restrict__ sm_idx, int32_t *__restrict__ prefix, int32_t *sm_len, int len_cap,
                          int32_t *status, int check_blocks, int slice_chunks, int L, int H) {
-    constexpr int kVecPerRow = D * (int)sizeof(T) / 16, kRows = kRowsThreads / kVecPerRow;
-    __shared__ int list[kRowsSlice * kC];
-    __shared__ int counts[kRowsSlice], wsum[kRowsThreads / 32];
-    const int bh = blockIdx.y, b = bh / H, h = bh % H, NC = L / kC, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int c_lo = blockIdx.x * slice_chunks, nc = min(slice_chunks, NC - c_lo);
-    const uint8_t *rt = route + (size_t)b * L * H + h;
+    constexpr int kVecPerRow = D * (int)sizeof(T) / 16;
+    __shared__ RouteLists rl;
+    const int bh = blockIdx.y, b = bh / H, h = bh % H, NC = L / kC, piece = threadIdx.x % kVecPerRow;
     tc::launch_dependents();
-    int report = 0;
-    for (int c = warp; c < nc; c += kRowsThreads / 32) {
-        const size_t l0 = (size_t)(c_lo + c) * kC;
-        const uint8_t a0 = rt[(l0 + lane) * H], a1 = rt[(l0 + 32 + lane) * H];
-        const unsigned lo = __ballot_sync(0xffffffffu, a0 != 0), hi = __ballot_sync(0xffffffffu, a1 != 0);
-        const unsigned lt = (1u << lane) - 1u;
-        const int nlo = __popc(lo), n = nlo + __popc(hi);
-        if (a0) list[c * kC + __popc(lo & lt)] = (int)l0 + lane;
-        if (a1) list[c * kC + nlo + __popc(hi & lt)] = (int)l0 + 32 + lane;
-        if (check_blocks && n != 0 && n != kC) report = NATSL_ERR_ROUTE;      // one decision per chunk
-        if (lane == 0) counts[c] = n;
-    }
-    int before = 0;
-    const int n_before = c_lo * kC;
-    for (int l = tid; l < n_before; l += 8 * kRowsThreads) {                  // eight loads in flight
-        uint8_t x[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int ll = l + u * kRowsThreads;
-            x[u] = ll < n_before ? rt[(size_t)ll * H] : (uint8_t)0;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) before += x[u] != 0;
-    }
-    before = __reduce_add_sync(0xffffffffu, before);
-    if (lane == 0) wsum[warp] = before;
-    __syncthreads();
-    int base = 0, mine = 0;
-#pragma unroll
-    for (int wv = 0; wv < kRowsThreads / 32; ++wv) base += wsum[wv];
-    for (int c = 0; c < nc; ++c) mine += counts[c];
-    if (tid < nc) {
-        int pre = base;
-        for (int c = 0; c < tid; ++c) pre += counts[c];
-        prefix[(size_t)bh * (NC + 1) + c_lo + tid] = pre;
-    }
-    if (c_lo + nc == NC && tid == 0) {
-        prefix[(size_t)bh * (NC + 1) + NC] = base + mine;
+    const RouteSlice sl = list_slice(rl, route + (size_t)b * L * H + h, prefix + (size_t)bh * (NC + 1), 0, slice_chunks, NC, H);
+    int report = check_blocks && sl.mixed ? (int)NATSL_ERR_ROUTE : 0;         // one decision per chunk
+    const int n = sl.base + sl.mine;
+    if (sl.c_lo + sl.nc == NC && threadIdx.x == 0) {
         // The stored length never exceeds the rows the cache has, so a later decode step cannot be led past them.
-        if (sm_len) sm_len[bh] = min(base + mine, len_cap);
-        if (base + mine > len_cap) report = report ? min(report, (int)NATSL_ERR_CACHE_FULL) : (int)NATSL_ERR_CACHE_FULL;
+        if (sm_len) sm_len[bh] = min(n, len_cap);
+        if (n > len_cap) report = report ? min(report, (int)NATSL_ERR_CACHE_FULL) : (int)NATSL_ERR_CACHE_FULL;
     }
-    // the slice's rows, kRows at a time, chunk by chunk of the list
-    const int piece = tid % kVecPerRow;
-    int row0 = base, c = 0, in_c = tid / kVecPerRow;
-    while (true) {
-        while (c < nc && in_c >= counts[c]) { in_c -= counts[c]; row0 += counts[c]; ++c; }
-        if (c >= nc) break;
-        const int row = row0 + in_c, tok = list[c * kC + in_c];
+    for_each_row<kVecPerRow>(rl, sl, [&](int row, int tok) {
         const size_t src = (((size_t)b * L + tok) * H + h) * D;
         if (piece == 0) sm_idx[(size_t)bh * L + row] = tok;
         const uint4 vv = reinterpret_cast<const uint4 *>(v + src)[piece];
@@ -229,8 +185,7 @@ route_gather_rows_kernel(const uint8_t *__restrict__ route, const T *__restrict_
         };
         put(j0);
         put(j1);
-        in_c += kRows;
-    }
+    });
     tc::grid_dependency_wait();
     if (report) atomicMin(status, report);
 }
@@ -241,13 +196,9 @@ template <typename T, int D>
 static cudaError_t route_gather_rows_impl(const uint8_t *route, const void *v, const RowsJob &j0, const RowsJob &j1,
                                           int32_t *sm_idx, int32_t *prefix, int32_t *sm_len, int len_cap, int32_t *status,
                                           bool check_blocks, Shape s, cudaStream_t st, bool pdl) {
-    const int NC = s.L / kC, BH = s.B * s.H;             // about two CTAs per SM, at most 32 per pair
-    int slices = (2 * 148 + BH - 1) / BH;
-    slices = slices > 32 ? 32 : slices;
-    int cps = (NC + slices - 1) / slices;
-    cps = cps > kRowsSlice ? kRowsSlice : cps;
+    const int NC = s.L / kC, BH = s.B * s.H, cps = slice_chunks_of(NC, BH, 2);
     count_launch();
-    return launch_kernel(route_gather_rows_kernel<T, D>, dim3((NC + cps - 1) / cps, BH), dim3(kRowsThreads), 0, st, pdl, route,
+    return launch_kernel(route_gather_rows_kernel<T, D>, dim3((NC + cps - 1) / cps, BH), dim3(kRouteThreads), 0, st, pdl, route,
                          (const T *)v, j0, j1, sm_idx, prefix, sm_len, len_cap, status, check_blocks ? 1 : 0, cps, s.L, s.H);
 }
 

@@ -40,6 +40,7 @@
 // they were gathered, the softmax threads normalise the Q tile in place before the first product.
 #include "common.cuh"
 #include "natsl_internal.h"
+#include "route_slice.cuh"
 #include "tc_common.cuh"
 
 namespace natsl {
@@ -645,17 +646,13 @@ softmax_combine_tc_kernel(const __grid_constant__ CUtensorMap map_q,
 }
 
 // Route compaction and gather of the retained K/V in one kernel (the softmax branch's half of the forward's
-// set-up; grid = (slices of the chunks, B*H)).  A CTA counts the retained tokens before its slice itself -- route
-// bytes out of L2, a few microseconds however long the sequence, where one CTA per (batch, head) walking all chunks
-// took 28 us at 512 chunks --, lists its own chunks' retained tokens (one 64-bit ballot word per chunk) and copies
+// set-up; grid = (slices of the chunks, B*H)).  A CTA lists its slice's retained tokens (see route_slice.cuh) and copies
 // their K rows (bf16) and V rows (as fp16) into the compacted layouts [B,H,cap,d] / [B,H,capv,d] (optionally K as
 // fp16 too, for the backward).  The fp16 rows behind the last one are zeroed up to the next multiple of 128, so
 // that a K/V tile never multiplies a zero probability or a zero logit gradient with an uninitialised value.
 // It also clears the scan's per-chunk counters of the call.  It needs nothing of the prepare kernel before it in
 // the stream and is its programmatic dependent, so that it runs where that kernel's last wave leaves room; it only
 // must not end before it, since the scan waits for this kernel.
-constexpr int kRouteThreads = 256;
-constexpr int kMaxSlice = 32;                        // chunks per CTA
 struct RouteArgs {
     const uint8_t *route;
     int32_t *sm_idx, *prefix, *emit_flags;
@@ -671,53 +668,13 @@ route_gather_kernel(const __nv_bfloat16 *__restrict__ k, const __nv_bfloat16 *__
     // fp16 keys then go to k16 only
     constexpr int kVecPerRow = D * 2 / 16;
     constexpr int kRows = kRouteThreads / kVecPerRow;
-    __shared__ int list[kMaxSlice * kC];
-    __shared__ int counts[kMaxSlice], wsum[kRouteThreads / 32];
+    __shared__ RouteLists rl;
     const int bh = blockIdx.y, b = bh / H, h = bh % H, NC = L / kC;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int c_lo = blockIdx.x * slice_chunks, nc = min(slice_chunks, NC - c_lo);
-    const uint8_t *rt = ra.route + (size_t)b * L * H + h;
+    const int tid = threadIdx.x;
     launch_dependents();
-    for (int i = tid; i < nc; i += kRouteThreads) ra.emit_flags[(size_t)bh * NC + c_lo + i] = 0;
-    // ---- own chunks' ballots, and the count of everything before them ----
-    for (int c = warp; c < nc; c += kRouteThreads / 32) {
-        const size_t l0 = (size_t)(c_lo + c) * kC;
-        const uint8_t a0 = rt[(l0 + lane) * H], a1 = rt[(l0 + 32 + lane) * H];
-        const unsigned lo = __ballot_sync(0xffffffffu, a0 != 0), hi = __ballot_sync(0xffffffffu, a1 != 0);
-        const unsigned lt = (1u << lane) - 1u;
-        const int nlo = __popc(lo);
-        if (a0) list[c * kC + __popc(lo & lt)] = (int)l0 + lane;          // compacted within the chunk's 64 places
-        if (a1) list[c * kC + nlo + __popc(hi & lt)] = (int)l0 + 32 + lane;
-        if (lane == 0) counts[c] = nlo + __popc(hi);
-    }
-    int before = 0;
-    const int n_before = c_lo * kC;
-    for (int l = tid; l < n_before; l += 8 * kRouteThreads) {             // eight loads in flight
-        uint8_t x[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int ll = l + u * kRouteThreads;
-            x[u] = ll < n_before ? rt[(size_t)ll * H] : (uint8_t)0;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) before += x[u] != 0;
-    }
-    before = __reduce_add_sync(0xffffffffu, before);
-    if (lane == 0) wsum[warp] = before;
-    __syncthreads();
     const int base0 = ra.base_in ? ra.base_in[bh] : 0;
-    int base = base0;
-#pragma unroll
-    for (int wv = 0; wv < kRouteThreads / 32; ++wv) base += wsum[wv];
-    int mine = 0;                                                         // retained tokens of the slice
-    for (int c = 0; c < nc; ++c) mine += counts[c];
-    const bool last = c_lo + nc == NC;
-    if (tid < nc) {
-        int pre = base;
-        for (int c = 0; c < tid; ++c) pre += counts[c];
-        ra.prefix[(size_t)bh * (NC + 1) + c_lo + tid] = pre;
-    }
-    if (last && tid == 0) ra.prefix[(size_t)bh * (NC + 1) + NC] = base + mine;
+    const RouteSlice sl = list_slice(rl, ra.route + (size_t)b * L * H + h, ra.prefix + (size_t)bh * (NC + 1), base0, slice_chunks, NC, H);
+    for (int i = tid; i < sl.nc; i += kRouteThreads) ra.emit_flags[(size_t)bh * NC + sl.c_lo + i] = 0;
     // RMS-normalised keys of the softmax operation (Section 4.3), per softmax head = per slice of D / groups
     // columns, as fp16 (the softmax kernel's logit product is an fp16 MMA in this mode): the slice's pieces
     // sit in neighbouring lanes of the row's lanes.  bf16 pieces in, fp16 pieces out.
@@ -747,29 +704,21 @@ route_gather_kernel(const __nv_bfloat16 *__restrict__ k, const __nv_bfloat16 *__
         return make_uint4(o[0], o[1], o[2], o[3]);
     };
     // ---- the slice's rows: one row per group of kVecPerRow threads, chunk by chunk of the list ----
-    {
-        int row0 = base, c = 0, in_c = tid / kVecPerRow;   // in_c: index within chunk c's list
-        while (true) {
-            while (c < nc && in_c >= counts[c]) { in_c -= counts[c]; row0 += counts[c]; ++c; }
-            if (c >= nc) break;
-            const int row = row0 + in_c, tok = list[c * kC + in_c];
-            if (piece == 0) ra.sm_idx[(size_t)bh * L + row - base0] = tok;
-            if (row < cap) {
-                const size_t dst = ((size_t)bh * cap + row) * D, src = (((size_t)b * L + tok) * H + h) * D;
-                uint4 *dv16 = reinterpret_cast<uint4 *>(v16 + ((size_t)bh * capv + row) * D) + piece;
-                uint4 *dk16 = k16 ? reinterpret_cast<uint4 *>(k16 + ((size_t)bh * capv + row) * D) + piece : nullptr;
-                uint4 kk = reinterpret_cast<const uint4 *>(k + src)[piece];
-                const uint4 vv = reinterpret_cast<const uint4 *>(v + src)[piece];
-                if (norm_eps >= 0.f && raw_k_sm) reinterpret_cast<uint4 *>(k_sm + dst)[piece] = kk;
-                if (norm_eps >= 0.f) kk = rms_fp16(kk);
-                if (!(norm_eps >= 0.f && raw_k_sm)) reinterpret_cast<uint4 *>(k_sm + dst)[piece] = kk;
-                if (dk16) *dk16 = norm_eps >= 0.f ? kk : to_fp16(kk);      // (normalised: already fp16)
-                if (v_sm) reinterpret_cast<uint4 *>(v_sm + dst)[piece] = vv;
-                *dv16 = to_fp16(vv);
-            }
-            in_c += kRows;
-        }
-    }
+    for_each_row<kVecPerRow>(rl, sl, [&](int row, int tok) {
+        if (piece == 0) ra.sm_idx[(size_t)bh * L + row - base0] = tok;
+        if (row >= cap) return;
+        const size_t dst = ((size_t)bh * cap + row) * D, src = (((size_t)b * L + tok) * H + h) * D;
+        uint4 *dv16 = reinterpret_cast<uint4 *>(v16 + ((size_t)bh * capv + row) * D) + piece;
+        uint4 *dk16 = k16 ? reinterpret_cast<uint4 *>(k16 + ((size_t)bh * capv + row) * D) + piece : nullptr;
+        uint4 kk = reinterpret_cast<const uint4 *>(k + src)[piece];
+        const uint4 vv = reinterpret_cast<const uint4 *>(v + src)[piece];
+        if (norm_eps >= 0.f && raw_k_sm) reinterpret_cast<uint4 *>(k_sm + dst)[piece] = kk;
+        if (norm_eps >= 0.f) kk = rms_fp16(kk);
+        if (!(norm_eps >= 0.f && raw_k_sm)) reinterpret_cast<uint4 *>(k_sm + dst)[piece] = kk;
+        if (dk16) *dk16 = norm_eps >= 0.f ? kk : to_fp16(kk);      // (normalised: already fp16)
+        if (v_sm) reinterpret_cast<uint4 *>(v_sm + dst)[piece] = vv;
+        *dv16 = to_fp16(vv);
+    });
     // ---- rows of earlier calls: only the fp16 copy of their V rows is made (and, with the normalisation, the
     // normalised copy of their keys, which the cache keeps as given) ----
     if (ra.base_in) {
@@ -781,8 +730,8 @@ route_gather_kernel(const __nv_bfloat16 *__restrict__ k, const __nv_bfloat16 *__
                 reinterpret_cast<uint4 *>(k16 + d16)[piece] = rms_fp16(reinterpret_cast<const uint4 *>(k_sm + dst)[piece]);
         }
     }
-    if (last) {                                            // zero rows behind the last one
-        const int n = min(base + mine, cap), n_pad = min((n + 127) / 128 * 128, capv);
+    if (sl.c_lo + sl.nc == NC) {                           // zero rows behind the last one
+        const int n = min(sl.base + sl.mine, cap), n_pad = min((n + 127) / 128 * 128, capv);
         for (int row = n + tid / kVecPerRow; row < n_pad; row += kRows) {
             const size_t d16 = ((size_t)bh * capv + row) * D;
             reinterpret_cast<uint4 *>(v16 + d16)[piece] = make_uint4(0u, 0u, 0u, 0u);
@@ -865,13 +814,7 @@ cudaError_t launch_softmax_combine_tc(const void *q, const void *k_sm, const voi
 template <int D>
 static cudaError_t route_gather_impl(const void *k, const void *v, const RouteArgs &ra, void *k_sm, void *v_sm, void *v16,
                                      void *k16, int cap, int capv, Shape s, cudaStream_t st, bool pdl, HeadGroups hg, bool raw_k_sm) {
-    // slices of 1 to kMaxSlice chunks: about four CTAs per SM over all (batch, head) pairs, at most 32 per pair (each
-    // counts what lies before it)
-    const int NC = s.L / kC, BH = s.B * s.H;
-    int slices = (4 * 148 + BH - 1) / BH;
-    slices = slices < 1 ? 1 : (slices > 32 ? 32 : slices);
-    int cps = (NC + slices - 1) / slices;
-    if (cps > kMaxSlice) cps = kMaxSlice;
+    const int NC = s.L / kC, BH = s.B * s.H, cps = slice_chunks_of(NC, BH, 4);
     dim3 grid((NC + cps - 1) / cps, BH);
     count_launch();
     return launch_kernel(route_gather_kernel<D>, grid, dim3(kRouteThreads), 0, st, pdl, (const __nv_bfloat16 *)k,

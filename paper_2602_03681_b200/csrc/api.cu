@@ -96,19 +96,31 @@ bool scan_follows_closely(const natsl_params *p, bool segmented) {
 // in one wave, at least 4 chunks long (shorter ones gain less than their step of the chain), and at least three --
 // with two the two passes are as long as one over everything.  22 pairs: 4 segments, 16: 6, 4: 20.
 // Where the line lies: three segments would fit one wave up to 49 pairs, but the softmax kernel, which runs beside the pass
-// with outputs, then starts a pass later, and the more it has to do the fewer pairs pay for that.  Time with segments
-// against one pass over everything, 2048 to 16384 tokens, 5 to 40 % softmax tokens: 128 columns 16 pairs 0.82 to 0.92, 18 pairs
-// 0.72 to 0.99, 22 pairs 0.85 to 1.07, 24 pairs 1.02 and 1.03, 32 pairs 1.12 to 1.15; 64 columns 24 pairs 0.86, 28 pairs 0.91 to
-// 1.06, 32 pairs 1.01, 36 pairs 1.08.  With own-block tiles 64 columns 16 pairs 0.93, 22 pairs 1.04.  128 columns, in the
-// order (2048 tokens, 20 % softmax tokens), (8192, 5 %), (8192, 30 %), (16384, 10 %): own-block tiles 16 pairs 0.99, 0.75, 0.98,
-// 0.81, 18 pairs 0.99, 0.79, 1.00, 0.90, 20 pairs 1.14, 0.88, 1.08, 0.97, 22 pairs 1.10, 0.96, 1.10, 1.04; two softmax heads,
-// token routing 12 pairs 0.97, 0.65, 1.01, 0.78, 14 pairs 0.96, 0.70, 1.06, 0.86, 16 pairs 1.00, 0.75, 1.08, 0.92, 18 pairs 1.08,
-// 0.79, 1.06, 0.98 (normalised q, k: 0.02 to 0.06 less); both 10 pairs 0.75 to 0.99, 14 pairs 0.91 to 1.06, 16 pairs 1.06.
-// Own-block tiles with one softmax head of 128 columns would pay up to 18 pairs; they keep 14 because segments need scratch,
-// and calls of 15 to 18 pairs of 1024 tokens that fit natsl_hybrid_fwd_static's array (23 to 27 of 32 MiB) would not any more.
+// with outputs, then starts a pass later, and the more it has to do the fewer pairs pay for that: own-block tiles, two softmax
+// heads, many softmax tokens (whose share is not known here), and short sequences, whose passes do not hide the launches.  Time with
+// segments against one pass over everything, 2048 to 16384 tokens, 5 to 40 % softmax tokens: 128 columns 16 pairs 0.82 to 0.92, 18
+// pairs 0.72 to 0.99, 22 pairs 0.84 to 1.17, 24 pairs 0.85 to 1.14, 32 pairs 1.12 to 1.15; 64 columns 24 pairs 0.86, 28 pairs 0.91 to
+// 1.06, 32 pairs 0.96 to 1.18, 36 pairs 1.08.  From 4096 tokens on, at 5, 10, 20, 40 %, in the order 4096 | 8192 | 16384 tokens:
+//   128 columns          23 pairs 0.86 0.88 0.93 1.02 | 0.81 0.83 0.90 1.06 | 0.79 0.84 0.95 1.07
+//                        26 pairs 0.91 0.95 1.02 1.12 | 0.89 0.93 1.05 1.12 | 0.88 0.97 1.02 1.11
+//   own-block tiles      18 pairs 0.85 0.88 0.95 1.06 | 0.80 0.84 0.92 1.06 | 0.80 0.88 0.98 1.10
+//                        20 pairs 0.93 0.95 1.01 1.13 | 0.87 0.92 1.02 1.10 | 0.86 0.94 1.06 1.12
+//   two softmax heads    16 pairs 0.79 0.85 0.96 1.15 | 0.73 0.83 1.00 1.09 | 0.75 0.92 1.06 1.09
+//                        20 pairs 0.94 1.00 1.12 1.22 | 0.86 0.96 1.09 1.13 | 0.89 1.03 1.10 1.07
+//   both, normalised     15 pairs 0.86 0.91 0.99 1.14 | 0.79 0.86 1.01 1.08 | 0.80 0.92 1.04 1.07
+//                        18 pairs 0.92 0.97 1.08 1.13 | 0.92 0.98 1.06 1.11 | 0.95 1.03 1.07 1.06
+//   64 col., own-block   20 pairs 0.83 0.86 0.96 1.15 | 0.77 0.83 0.97 1.08 | 0.78 0.91 1.02 1.06
+//                        24 pairs 0.91 0.97 1.08 1.13 | 0.85 0.94 1.04 1.08 | 0.89 1.01 1.08 1.07
+// At 2048 tokens: own-block tiles 15 pairs 0.92 to 1.00, 18 pairs 0.98 to 1.06; two softmax heads 14 pairs 0.91 to 1.07, 16 pairs 0.94 to
+// 1.14; both 14 pairs 0.93 to 1.10, 16 pairs 0.98 to 1.18; 64 columns with own-block tiles 18 pairs 0.90 to 1.16, 20 pairs 0.91 to 1.14.
+// Shorter sequences keep the lower lines for another reason too: segments need scratch, and calls of 15 to 18 pairs of 1024
+// tokens that fit natsl_hybrid_fwd_static's array (23 to 27 of 32 MiB) would not any more; of 4096 tokens none fits it anyway.
 int segment_pairs(const natsl_params *p) {
-    const bool heavy = (p->flags & NATSL_BLOCK_ROUTING) || p->G > 1;
-    return p->d == 64 ? (heavy ? 18 : 30) : heavy ? 14 : 22;
+    const bool own = p->flags & NATSL_BLOCK_ROUTING, lng = p->L >= 4096;
+    if (p->d == 64) return !own && p->G <= 1 ? 30 : own && lng ? 20 : 18;
+    if (p->G > 1) return !lng ? 14 : own ? 15 : 16;
+    if (own) return lng ? 18 : 14;
+    return lng ? 23 : 22;
 }
 // The two passes must save 8 chunks of the chain, which is what two more launches and the chaining take.
 // The last segment takes what remains, up to twice as much: the first pass does not run it, and in the second the

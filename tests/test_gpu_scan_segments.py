@@ -47,19 +47,26 @@ def test_segments(name, H, L, oracle):
 
 
 # the last number of pairs that is cut into segments and the first that is not: 128 and 64 columns, with block-level routing too,
-# and 128 columns with two softmax heads.  What is not cut is the same call as with one pass and compared with the oracle.
+# and 128 columns with two softmax heads, below and from 4096 tokens on.  What is not cut is the same call as with one pass and compared with the oracle.
 @pytest.mark.parametrize("name,H,L,mode,cut", [("cfg1_bf16_prefill", 22, 1536, "token", True), ("cfg1_bf16_prefill", 23, 1536, "token", False),
                                                ("cfg4_bf16_train", 30, 2048, "token", True), ("cfg4_bf16_train", 31, 2048, "token", False),
                                                ("cfg4_bf16_train", 18, 1536, "block", True), ("cfg4_bf16_train", 19, 1536, "block", False),
                                                ("cfg1_bf16_prefill", 14, 1536, "block", True), ("cfg1_bf16_prefill", 15, 1536, "block", False),
-                                               ("cfg1_bf16_prefill", 14, 1536, "two heads", True), ("cfg1_bf16_prefill", 15, 1536, "two heads", False)])
+                                               ("cfg1_bf16_prefill", 14, 1536, "two heads", True), ("cfg1_bf16_prefill", 15, 1536, "two heads", False),
+                                               ("cfg1_bf16_prefill", 23, 4032, "token", False), ("cfg1_bf16_prefill", 23, 4096, "token", True),
+                                               ("cfg1_bf16_prefill", 24, 4096, "token", False),
+                                               ("cfg4_bf16_train", 20, 4096, "block", True), ("cfg4_bf16_train", 21, 4096, "block", False),
+                                               ("cfg1_bf16_prefill", 18, 4096, "block", True), ("cfg1_bf16_prefill", 19, 4096, "block", False),
+                                               ("cfg1_bf16_prefill", 16, 4096, "two heads", True), ("cfg1_bf16_prefill", 17, 4096, "two heads", False),
+                                               ("cfg1_bf16_prefill", 15, 4096, "both", True), ("cfg1_bf16_prefill", 16, 4096, "both", False)])
 def test_segments_at_the_lines(name, H, L, mode, cut):
     wl = inputs.WORKLOADS[name]
     x = inputs.make_layer_inputs(wl, B=1, H=H, L=L)
-    if mode == "block":
+    block, heads = mode in ("block", "both"), 2 if mode in ("two heads", "both") else 0
+    if block:
         x["route"] = np.repeat((np.random.default_rng(3).random((1, L // 64, H)) < 0.3).astype(np.uint8), 64, axis=1)
     x["g"] = np.full((1, L, H), -1e-3, np.float32)
-    seg, one, was_cut = both_ways(wl, x, binding.BLOCK_ROUTING if mode == "block" else 0, 2 if mode == "two heads" else 0)
+    seg, one, was_cut = both_ways(wl, x, binding.BLOCK_ROUTING if block else 0, heads)
     assert was_cut == cut
     if cut:
         for n in ("o_la", "state_out"):
@@ -67,8 +74,8 @@ def test_segments_at_the_lines(name, H, L, mode, cut):
         return
     for n in seg:
         assert np.array_equal(seg[n], one[n]), n
-    ref = run_oracle(wl, x, block=64 if mode == "block" else None)
-    if mode == "two heads":                       # (the linear branch does not see the softmax heads)
+    ref = run_oracle(wl, x, block=64 if block else None)
+    if heads:                       # (the linear branch does not see the softmax heads)
         for n in ("o_la", "state_out"):
             assert rel_err(seg[n], ref[n]) <= TOL["bf16"], n
     else:

@@ -111,6 +111,8 @@ bool scan_follows_closely(const natsl_params *p, bool segmented) {
 //                        18 pairs 0.92 0.97 1.08 1.13 | 0.92 0.98 1.06 1.11 | 0.95 1.03 1.07 1.06
 //   64 col., own-block   20 pairs 0.83 0.86 0.96 1.15 | 0.77 0.83 0.97 1.08 | 0.78 0.91 1.02 1.06
 //                        24 pairs 0.91 0.97 1.08 1.13 | 0.85 0.94 1.04 1.08 | 0.89 1.01 1.08 1.07
+// (One pass -> segments, us, 8192 tokens, 5 %: own-block tiles 15 pairs 265 -> 186, two softmax heads 15 pairs 255 -> 181, 64 columns
+// with own-block tiles 20 pairs 228 -> 175, 23 pairs 296 -> 237; own-block tiles 15 pairs of 16384 tokens 502 -> 344.)
 // At 2048 tokens: own-block tiles 15 pairs 0.92 to 1.00, 18 pairs 0.98 to 1.06; two softmax heads 14 pairs 0.91 to 1.07, 16 pairs 0.94 to
 // 1.14; both 14 pairs 0.93 to 1.10, 16 pairs 0.98 to 1.18; 64 columns with own-block tiles 18 pairs 0.90 to 1.16, 20 pairs 0.91 to 1.14.
 // Shorter sequences keep the lower lines for another reason too: segments need scratch, and calls of 15 to 18 pairs of 1024
